@@ -246,7 +246,7 @@ def prepare(case, seed):
     if kind == "score_layers":
         _, lse = _attention_of_window(case, inp)
         s.update(cfg=_config(case, L=1), lse=lse.transpose(0, 1).contiguous(),  # [L, B, Hq, w]
-                 psi=torch.zeros((L, B, Hkv, n), device="cuda"))
+                 psi=[torch.zeros((B, Hkv, n), device="cuda") for _ in range(L)])
         s["ws"] = mk.new_workspace(s["cfg"])
         return s
     psi, _ = _attention_of_window(case, inp)
@@ -256,10 +256,11 @@ def prepare(case, seed):
         s["buf"] = mk.EvictionBuffers(s["cfg"], B * L * Hkv * slack)
         s["buf"].psi.copy_(psi)
         return s
-    # layer by layer: every layer has its own ragged cache; the per-layer arrays lie behind one another
+    # layer by layer: every layer has its own ragged cache; the per-layer arrays lie behind one another, but for the
+    # scores, whose rows may have any length and whose base is aligned
     z = lambda *shape, dtype=torch.int32: torch.zeros(shape, dtype=dtype, device="cuda")  # noqa: E731
     cap = B * Hkv * min(slack * 2, n + s["cfg"].max_new_tokens)
-    s.update(one=_config(case, L=1), ws=mk.new_workspace(s["cfg"]), psi=psi.transpose(0, 1).contiguous(),
+    s.update(one=_config(case, L=1), ws=mk.new_workspace(s["cfg"]), psi=[psi[:, l].clone() for l in range(L)],
              mass=z(L, B, Hkv, 2, dtype=torch.float64), pref=z(L, B, Hkv, 2, dtype=torch.float64),
              demand=z(L, B, Hkv, 2), budgets=z(L, B, Hkv, 2), phi=z(B, L, dtype=torch.float64),
              kept_len=z(L, B * Hkv), seg_off=z(L, B * Hkv + 1, dtype=torch.int64), kept_idx=z(L, cap),
