@@ -2,21 +2,13 @@
 // (Eq. 10-11) and the integer per-head, per-modality budgets.
 //
 // All sums of psi are exact: psi is mapped to 2^-32 fixed point (psi_fix) and added as 64-bit integers, so the
-// results do not depend on the order of summation or on the launch shape. Eq. 9 is a "top-p" count: a three- or four-pass
-// radix descent over the order-preserving bit pattern of psi with per-bucket (count, mass) histograms in shared
-// memory finds the bucket in which the descending prefix mass reaches theta * W_m; ties inside the final bucket
-// share one value, so the remaining count is a division. The keys of a unit sit in registers between passes. The layer recurrence is a scalar fp64 scan per sequence
-// with explicitly rounded operations (no FMA contraction), so it is reproducible bit for bit.
-#include "common.cuh"
+// results do not depend on the order of summation or on the launch shape. Eq. 9 is a "top-p" count: the number of
+// largest keys whose mass reaches theta * W_m. The layer recurrence is a scalar fp64 scan per sequence with
+// explicitly rounded operations (no FMA contraction), so it is reproducible bit for bit.
+#include "rank_common.cuh"
 
 namespace madakv {
 namespace {
-
-typedef unsigned long long u64;
-constexpr int NT = 512;
-constexpr int KPT = 16;            // keys a thread holds in registers per round
-constexpr int ROUND = NT * KPT;    // keys a block takes per round
-constexpr unsigned int kFull = 0xffffffffu;
 
 struct AllocParams {
   const float* psi;
@@ -32,266 +24,356 @@ struct AllocParams {
   u64 theta_fix;  // floor(theta * 2^32)
 };
 
-// Shared histograms of one radix pass: per (modality, digit) a count and an exact 64-bit mass kept as two 32-bit
-// words (32-bit shared atomics are native; the carry of the low word is detected from the value the atomic returns).
-// A digit has DIG bits. Sequences of more than one round are re-read from L2 in every pass, and with 10-bit digits the
-// 30 bits in which importance values differ at most take three passes instead of four (long: allocation 0.26 -> 0.20
-// ms); a sequence that sits in registers gains nothing from that and pays for the larger histograms (llava 0.067 ->
-// 0.073 ms), so configs whose sequences fit one round keep 8-bit digits.
-// Bucket b sits at word b + b / kPerLane: the bucket walk has lane j read buckets kPerLane * j + i, which in a dense
-// array would be a many-way bank conflict on every load; with the skew the 32 lanes of a load hit 32 different banks.
-template <int DIG>
-struct Hist {
-  static constexpr int kBuckets = 1 << DIG;        // per modality
-  static constexpr int kPerLane = kBuckets / 32;   // buckets a lane of the walking warp owns
-  static constexpr int kWords = 2 * kBuckets + 2 * 32;
-  unsigned int cnt[kWords], mlo[kWords], mhi[kWords];
-  __device__ __forceinline__ static int slot(int bucket) { return bucket + bucket / kPerLane; }
-};
-#define hist_slot(b) (Hist<DIG>::slot(b))
-template <int DIG>
-__device__ __forceinline__ void hist_add(Hist<DIG>& h, int bucket, u64 m) {
-  const int s = hist_slot(bucket);
-  atomicAdd(&h.cnt[s], 1u);
-  const unsigned int add = (unsigned int)m;
-  const unsigned int old = atomicAdd(&h.mlo[s], add);
-  const unsigned int hi = (unsigned int)(m >> 32) + ((unsigned int)(old + add) < old ? 1u : 0u);
-  if (hi) atomicAdd(&h.mhi[s], hi);  // rare: importance values are mostly below 1, carries are few
-}
-template <int DIG>
-__device__ __forceinline__ u64 hist_mass(const Hist<DIG>& h, int bucket) {
-  const int s = hist_slot(bucket);
-  return ((u64)h.mhi[s] << 32) | h.mlo[s];
+// The low 32 bits of floor(x * 2^32), plus kLowBias, by fp32 additions, for keys below kSmallKey (512.0): adding 512
+// rounded towards zero leaves floor(x * 2^14) in the low bits of the significand, the remainder (exact) added to 2^-9 the
+// other 18 bits; the constants of the first sum are shifted out. (The conversion to a 64-bit integer runs at a small
+// fraction of the rate of additions.)
+constexpr uint32_t kSmallKey = 0x44000000u, kLowBias = 0x3b000000u;
+__device__ __forceinline__ uint32_t low_mass(uint32_t key) {
+  const float x = __uint_as_float(key);
+  const float t = __fadd_rz(x, 512.0f);
+  return (__float_as_uint(t) << 18) + __float_as_uint(__fadd_rz(__fsub_rn(x, __fsub_rn(t, 512.0f)), 0x1p-9f));
 }
 
-// One warp walks the buckets of modality m in ascending digit order (digits are taken from kmax - key, so this is
-// descending importance): the first bucket at which the running mass `above + mass[dig]` reaches need_c is the one
-// the threshold falls into (the last bucket if none does). Lane j owns buckets kPerLane * j ..; a warp prefix scan of
-// the lanes' totals tells which lane holds that bucket, and that lane alone walks its buckets. Returns the bucket,
-// and updates above / above_c to the mass / count strictly before it (identical in every lane).
-template <int DIG>
-__device__ __forceinline__ int descend(const Hist<DIG>& h, int m, u64 need_c, u64& above, unsigned int& above_c,
-                                       unsigned int& cnt_at) {
-  constexpr int kBuckets = Hist<DIG>::kBuckets, kPerLane = Hist<DIG>::kPerLane;
-  const int lane = threadIdx.x & 31;
-  const int first = m * kBuckets + lane * kPerLane;
-  u64 lm = 0;
-  unsigned int lc = 0;
-#pragma unroll 8
-  for (int i = 0; i < kPerLane; ++i) {
-    lm += hist_mass(h, first + i);
-    lc += h.cnt[hist_slot(first + i)];
-  }
-  u64 sm = lm;
-  unsigned int sc = lc;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const u64 tm = __shfl_up_sync(kFull, sm, off);
-    const unsigned int tc = __shfl_up_sync(kFull, sc, off);
-    if (lane >= off) {
-      sm += tm;
-      sc += tc;
-    }
-  }
-  // the lane whose buckets take the running mass to the threshold (lane 31 if none does)
-  u64 a = above + (sm - lm);
-  unsigned int ac = above_c + (sc - lc), c_at = 0;
-  const unsigned int hit = __ballot_sync(kFull, a + lm >= need_c || lane == 31);
-  const int win = __ffs(hit) - 1;
-  int found = kPerLane - 1;
-  if (lane == win) {
-    for (int i = 0; i < kPerLane; ++i) {
-      const u64 mi = hist_mass(h, first + i);
-      const unsigned int ci = h.cnt[hist_slot(first + i)];
-      if (a + mi >= need_c || i == kPerLane - 1) {
-        found = i;
-        c_at = ci;
-        break;
-      }
-      a += mi;
-      ac += ci;
-    }
-  }
-  above = __shfl_sync(kFull, a, win);
-  above_c = __shfl_sync(kFull, ac, win);
-  cnt_at = __shfl_sync(kFull, c_at, win);
-  return win * kPerLane + __shfl_sync(kFull, found, win);
-}
-
-// One block per unit. A thread keeps KPT keys in registers (loaded once when the sequence fits one round, else
-// re-read from L2 every pass), so a pass costs no dependent global loads.
-//
-// The radix digits are not taken from the key itself but from t = kmax - key, starting at the highest bit in which
-// the unit's keys differ (kmax, kmin: largest and smallest key of the unit). Importance values share their sign and
-// most exponent bits, so digits of the raw key would put nearly all keys into a handful of buckets and serialise
-// the shared atomics; the digits of t spread them over the whole histogram. Ascending t is descending importance.
-template <int DIG>
-__global__ void __launch_bounds__(NT, 2) alloc_unit_kernel(AllocParams p) {
-  constexpr int kDigitBits = DIG, kBuckets = Hist<DIG>::kBuckets, kPerLane = Hist<DIG>::kPerLane;
-  constexpr int kHistWords = Hist<DIG>::kWords;
-  __shared__ Hist<DIG> hist;
-  __shared__ uint32_t s_prefix[2];
-  __shared__ int s_done[2];
-  __shared__ u64 s_W[2];
-  __shared__ uint32_t s_red[2][NT / 32];
-
-  const int u = blockIdx.x;
+// Masses, preference and Eq. 9's counts of one unit, by a team of blocks (see rank_common.cuh). A bucket holds a count and
+// the sum of its keys' masses modulo 2^32, two shared atomics without a result per key. That is enough for the exact mass:
+// all keys of a bucket lie between its two edges, so the mass is count * (mass of the lower edge) plus a remainder below
+// count * (distance of the edges), and the remainder is known exactly where that bound is below 2^32 (it is by a wide
+// margin for importance values: buckets are narrow where the keys are). A unit for which the bound fails anywhere, or with
+// scores of 512 and more, goes the slow way: exact sweeps that halve the range.
+// (Exact 64-bit masses by atomics that return the old word, to detect carries: alloc 52 us on llava.)
+template <int KPT, int TEAM>
+__global__ void __launch_bounds__(kRankThreads, 2) alloc_unit_kernel(AllocParams p) {
+  using SH = RankShared<TEAM, 2>;
+  constexpr int kPer = SH::kPer;
+  __shared__ SH sh;
+  pdl_wait();
+  pdl_go();
+  const uint32_t rank = TEAM > 1 ? team_rank() : 0u;
+  const int u = blockIdx.x / TEAM;
   const int b = u / (p.Hkv * p.L);
-  const int n = clamped_len(p.seq_len, b, p.n_max);
   const float* psi = p.psi + (int64_t)u * p.n_max;
+  const int mis = (int)(((int64_t)u * p.n_max) & 3);
   const uint8_t* mask = p.mask + (int64_t)b * p.n_max;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rounds = (n + ROUND - 1) / ROUND;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int kRound = kRankThreads * KPT;
+  const int rounds = (p.n_max + kRound * TEAM - 1) / (kRound * TEAM);
+  const int pos_first = (int)rank * rounds * kRound + tid * KPT;  // a block owns consecutive positions
+  const int n = clamped_len(p.seq_len, b, p.n_max);
 
-  uint32_t key[KPT];
-  uint32_t flags = 0;  // bit j: key j exists; bit 16 + j: key j is a visual token
-  // a thread takes KPT consecutive keys of a round (which keys a thread holds does not matter: all sums are exact);
-  // a full, aligned stretch comes in four 16-byte loads of scores and one of mask bytes
-  const bool vec = (p.n_max & 3) == 0 && (reinterpret_cast<uintptr_t>(mask) & 15) == 0;
+  uint32_t key[KPT], vis = 0;
   auto load_round = [&](int r) {
-    flags = 0;
-    const int i0 = r * ROUND + (int)threadIdx.x * KPT;
-    if (vec && i0 + KPT <= n) {
+    const int pos0 = pos_first + r * kRound;
+    load_scores<KPT>(psi, mis, p.n_max, pos0, key);
+    vis = load_mask<KPT>(mask, p.n_max, pos0);
+    const uint32_t valid = valid_bits<KPT>(n, pos0);
+    if (valid != valid_bits<KPT>(KPT, 0)) {
 #pragma unroll
-      for (int j = 0; j < KPT; j += 4) {
-        const float4 v = __ldg(reinterpret_cast<const float4*>(psi + i0 + j));
-        key[j] = psi_key(v.x);
-        key[j + 1] = psi_key(v.y);
-        key[j + 2] = psi_key(v.z);
-        key[j + 3] = psi_key(v.w);
-      }
-      const uint4 mv = __ldg(reinterpret_cast<const uint4*>(mask + i0));
-      flags = 0xffffu | ((nonzero_bytes(mv.x) | (nonzero_bytes(mv.y) << 4) | (nonzero_bytes(mv.z) << 8) |
-                          (nonzero_bytes(mv.w) << 12)) << 16);
-    } else {
-#pragma unroll
-      for (int j = 0; j < KPT; ++j) {
-        const int i = i0 + j;
-        key[j] = 0;
-        if (i < n) {
-          key[j] = psi_key(__ldg(psi + i));
-          flags |= (1u << j) | (__ldg(mask + i) ? (0x10000u << j) : 0u);
-        }
-      }
+      for (int j = 0; j < KPT; ++j)
+        if (!((valid >> j) & 1u)) key[j] = kNoKey;
     }
   };
 
-  // range of the unit's keys
+  // ---- range of the keys
   uint32_t kmax = 0, kmin = 0xffffffffu;
   for (int r = 0; r < rounds; ++r) {
     load_round(r);
 #pragma unroll
-    for (int j = 0; j < KPT; ++j)
-      if ((flags >> j) & 1u) {
-        kmax = max(kmax, key[j]);
-        kmin = min(kmin, key[j]);
-      }
+    for (int j = 0; j < KPT; ++j) {
+      kmax = (uint32_t)max((int)kmax, (int)key[j]);  // (kNoKey is negative)
+      kmin = min(kmin, key[j]);
+    }
   }
-  kmax = __reduce_max_sync(kFull, kmax);
-  kmin = __reduce_min_sync(kFull, kmin);
-  if (lane == 0) {
-    s_red[0][warp] = kmax;
-    s_red[1][warp] = kmin;
-  }
-  __syncthreads();
+  team_range<TEAM, 2>(sh, rank, kmax, kmin);
+  auto to_t = [&]() {
 #pragma unroll
-  for (int i = 0; i < NT / 32; ++i) {
-    kmax = max(kmax, s_red[0][i]);
-    kmin = min(kmin, s_red[1][i]);
-  }
-  if (kmin > kmax) kmin = kmax;  // no keys at all
-  // significant bits of t = kmax - key; at least one pass always runs (it also yields the masses of Eq. 6)
-  const int top = max(32 - __clz(kmax - kmin), 1);
-  if (rounds == 1) {
-#pragma unroll
-    for (int j = 0; j < KPT; ++j) key[j] = (flags >> j) & 1u ? kmax - key[j] : 0xffffffffu;  // (see the passes)
-  }
-
-  // state of the descent, kept by warp m (all lanes alike) for modality m
-  u64 need_c = 0, above = 0;
-  unsigned int above_c = 0;
-
-  // Eq. 9: radix descent, both modalities at once. The first pass sees every key, so its histogram also yields the
-  // modality masses W_v, W_t of Eq. 6. `rem` counts the bits of t not yet resolved.
-  for (int rem = top, pass = 0; rem > 0; ++pass) {
-    const int bits = min(rem, kDigitBits), shift = rem - bits;
-    const uint32_t dmask = (1u << bits) - 1u;
-    for (int x = threadIdx.x; x < kHistWords; x += NT) {
-      hist.cnt[x] = 0;
-      hist.mlo[x] = 0;
-      hist.mhi[x] = 0;
+    for (int j = 0; j < KPT; ++j) key[j] = key[j] == kNoKey ? kNoKey : kmax - key[j];
+  };
+  if (rounds == 1) to_t();
+  auto reload = [&](int r) {
+    if (rounds > 1) {
+      load_round(r);
+      to_t();
+    }
+  };
+  // the mass to reach, Eq. 9: theta_fix * W has 96 bits; the prefix test  prefix * 2^32 >= theta_fix * W  is
+  // prefix >= ceil(theta_fix * W / 2^32)
+  auto target = [&](u64 W) {
+    const u64 hi = __umul64hi(p.theta_fix, W), lo = p.theta_fix * W;
+    return (hi << 32) + (lo >> 32) + ((lo & 0xffffffffull) ? 1ull : 0ull);
+  };
+  // sums over the team, into every thread (of values that are already summed up over the warp)
+  auto team_sums = [&](u64& a0, u64& a1) {
+    __syncthreads();
+    if (lane == 0) {
+      sh.wsum[0][warp] = a0;
+      sh.wsum[1][warp] = a1;
     }
     __syncthreads();
-    const uint32_t pre0 = pass ? s_prefix[0] : 0u, pre1 = pass ? s_prefix[1] : 0u;
-    const bool act0 = pass == 0 || !s_done[0], act1 = pass == 0 || !s_done[1];
-    if (act0 || act1) {
+    if (warp == 0) {
+      const u64 t0 = warp_sum64(lane < kRankWarps ? sh.wsum[0][lane] : 0ull);
+      const u64 t1 = warp_sum64(lane < kRankWarps ? sh.wsum[1][lane] : 0ull);
+      if (lane < TEAM) {
+        peer_store<TEAM>(&sh.slice_q[0][rank], lane, t0);
+        peer_store<TEAM>(&sh.slice_q[1][rank], lane, t1);
+      }
+    }
+    team_sync<TEAM>();
+    a0 = warp_sum64(lane < TEAM ? sh.slice_q[0][lane] : 0ull);
+    a1 = warp_sum64(lane < TEAM ? sh.slice_q[1][lane] : 0ull);
+    team_sync<TEAM>();
+  };
+
+  const uint32_t all_span = kmax - kmin;
+  RankRange r0{0u, all_span, kNoKey, 0u}, r1 = r0;
+  u64 above0 = 0, above1 = 0;  // exact mass before r0.lo, r1.lo
+  u64 need0 = 0, need1 = 0, W0 = 0, W1 = 0;
+  bool exact = kmax < kSmallKey;
+
+  for (int pass = 0; pass < 2 && exact; ++pass) {
+    // ---- buckets
+    const int shift0 = range_shift(r0.span, SH::kDig), shift1 = range_shift(r1.span, SH::kDig);
+    if (pass == 0) {  // all keys take part, both modalities over the same range
       for (int r = 0; r < rounds; ++r) {
-        if (rounds > 1) {
-          load_round(r);
-#pragma unroll
-          for (int j = 0; j < KPT; ++j) key[j] = (flags >> j) & 1u ? kmax - key[j] : 0xffffffffu;
-        }
-        // One comparison per key: t of an existing key is below 2^top <= 2^31, a slot without a key holds all ones,
-        // and a modality that is done gets a prefix no shifted t can equal (rem >= 1).
-        const uint32_t want0 = act0 ? pre0 : 0xffffffffu, want1 = act1 ? pre1 : 0xffffffffu;
+        reload(r);
 #pragma unroll
         for (int j = 0; j < KPT; ++j) {
-          const bool vis = (flags >> (16 + j)) & 1u;
-          if ((key[j] >> rem) == (vis ? want0 : want1))
-            hist_add(hist, (vis ? 0 : kBuckets) + (int)((key[j] >> shift) & dmask), psi_fix(kmax - key[j]));
+          uint32_t* at = sh.cnt + ((vis >> j) & 1u ? 0 : SH::kStride) + min(key[j] >> shift0, (uint32_t)SH::kBuckets);
+          atomicAdd(at, 1u);
+          atomicAdd(at + 2 * SH::kStride, low_mass(kmax - key[j]));
         }
       }
-    }
-    __syncthreads();
-    if (warp < 2) {
-      const int m = warp;
-      if (pass == 0) {
-        u64 wsum = 0;
-#pragma unroll 8
-        for (int j = 0; j < kPerLane; ++j) wsum += hist_mass(hist, m * kBuckets + lane * kPerLane + j);
+    } else {
+      for (int x = tid; x < 4 * SH::kStride / 4; x += kRankThreads) reinterpret_cast<uint4*>(sh.cnt)[x] = make_uint4(0, 0, 0, 0);
+      __syncthreads();
+      for (int r = 0; r < rounds; ++r) {
+        reload(r);
 #pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) wsum += __shfl_xor_sync(kFull, wsum, off);
-        const u64 W = wsum;
-        // need = theta_fix * W (96 bits); the prefix test  prefix * 2^32 >= need  is  prefix >= ceil(need / 2^32)
-        const u64 hi = __umul64hi(p.theta_fix, W), lo = p.theta_fix * W;
-        need_c = (hi << 32) + (lo >> 32) + ((lo & 0xffffffffull) ? 1ull : 0ull);
-        if (lane == 0) {
-          s_prefix[m] = 0;
-          s_done[m] = (need_c == 0);
-          s_W[m] = W;
-          p.mass[(int64_t)u * 2 + m] = __ull2double_rn(W) / 4294967296.0;
-          if (need_c == 0) p.demand[(int64_t)u * 2 + m] = 0;
-        }
-      }
-      __syncwarp();
-      if (need_c != 0) {
-        unsigned int c_at = 0;
-        const int dig = min(descend(hist, m, need_c, above, above_c, c_at), (int)dmask);
-        if (lane == 0) {
-          const uint32_t prefix = (s_prefix[m] << bits) | (uint32_t)dig;
-          s_prefix[m] = prefix;
-          if (shift == 0) {
-            // t is resolved: every key in the final bucket has the value kmax - prefix; take as few of them as
-            // reach the threshold
-            const u64 each = psi_fix(kmax - prefix);
-            unsigned int take = c_at;
-            if (each > 0) {
-              const u64 t = (need_c - above + each - 1) / each;
-              if (t < (u64)take) take = (unsigned int)t;
-            }
-            p.demand[(int64_t)u * 2 + m] = (int32_t)(above_c + take);
+        for (int j = 0; j < KPT; ++j) {
+          const bool v = (vis >> j) & 1u;
+          const uint32_t x = key[j] - (v ? r0.lo : r1.lo);
+          if (x <= (v ? r0.span : r1.span)) {
+            uint32_t* at = sh.cnt + (v ? 0 : SH::kStride) + (x >> (v ? shift0 : shift1));
+            atomicAdd(at, 1u);
+            atomicAdd(at + 2 * SH::kStride, low_mass(kmax - key[j]));
           }
         }
       }
     }
-    __syncthreads();
-    if (pass == 0 && threadIdx.x == 0) {
-      const u64 W0 = s_W[0], W1 = s_W[1], tot = W0 + W1;
-      p.pref[(int64_t)u * 2 + 0] = tot ? __ddiv_rn(__ull2double_rn(W0), __ull2double_rn(tot)) : 0.0;
-      p.pref[(int64_t)u * 2 + 1] = tot ? __ddiv_rn(__ull2double_rn(W1), __ull2double_rn(tot)) : 0.0;
+    // ---- walk: block r of the team adds up its share of the buckets over all blocks; half of the threads per modality
+    const int m = tid / kHalf, i = tid % kHalf;
+    const uint32_t b0 = (rank * kHalf + i) * kPer;
+    const RankRange my = m ? r1 : r0;
+    const int shift = m ? shift1 : shift0;
+    if (tid == 0) sh.inexact = 0;
+    team_sync<TEAM>();
+    uint32_t c[kPer], s[kPer], lc = 0;
+    u64 q[kPer], lq = 0;
+    bucket_counts<TEAM, 2>(sh, m * SH::kStride + b0, c);
+    bucket_counts<TEAM, 2>(sh, (2 + m) * SH::kStride + b0, s);
+    {
+      auto edge = [&](uint32_t bk) {  // mass of the largest value of bucket bk
+        const u64 t = (u64)my.lo + ((u64)bk << shift);
+        return t <= kmax ? __float2ull_rz(__uint_as_float(kmax - (uint32_t)t) * 4294967296.0f) : 0ull;
+      };
+      u64 e = edge(b0);
+      bool bad = false;
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) {
+        const u64 e1 = edge(b0 + k + 1);
+        q[k] = c[k] * e1 + (u64)(s[k] - c[k] * (kLowBias + (uint32_t)e1));
+        bad = bad || c[k] * (e - e1) >> 32;
+        e = e1;
+        lc += c[k];
+        lq += q[k];
+      }
+      if (bad) {
+#pragma unroll
+        for (int r = 0; r < TEAM; ++r) peer_store<TEAM>(&sh.inexact, r, 1u);
+      }
     }
-    rem = shift;
+    uint32_t ic = warp_scan32(lc);
+    u64 iq = warp_scan64(lq);
+    if (lane == 31) {
+      sh.wscan_c[warp] = ic;
+      sh.wscan_q[warp] = iq;
+    }
+    __syncthreads();
+    {
+      const bool lower = lane >= m * (kRankWarps / 2) && lane < warp;
+      ic += __reduce_add_sync(kFull, lower ? sh.wscan_c[lane] : 0u);
+      iq += warp_sum64(lower ? sh.wscan_q[lane] : 0ull);
+    }
+    if (i >= kHalf - 32) {  // the last warp of the modality has the block's totals (in its last lane): to every block
+      const uint32_t tc = __shfl_sync(kFull, ic, 31);
+      const u64 tq = __shfl_sync(kFull, iq, 31);
+      if (lane < TEAM) {
+        peer_store<TEAM>(&sh.slice_c[m][rank], lane, tc);
+        peer_store<TEAM>(&sh.slice_q[m][rank], lane, tq);
+      }
+    }
+    team_sync<TEAM>();
+    if (TEAM > 1) {
+      const bool lower = lane < (int)rank;
+      ic += __reduce_add_sync(kFull, lower ? sh.slice_c[m][lane] : 0u);
+      iq += warp_sum64(lower ? sh.slice_q[m][lane] : 0ull);
+    }
+    exact = sh.inexact == 0;
+    if (pass == 0) {
+      W0 = warp_sum64(lane < TEAM ? sh.slice_q[0][lane] : 0ull);
+      W1 = warp_sum64(lane < TEAM ? sh.slice_q[1][lane] : 0ull);
+      need0 = target(W0);
+      need1 = target(W1);
+    }
+    const u64 need = m ? need1 : need0;
+    ic += my.above;
+    iq += m ? above1 : above0;
+    if (need && iq - lq < need && iq >= need) {  // the threshold lies in one of this thread's buckets
+      u64 run = iq - lq, at_q = 0;
+      uint32_t run_c = ic - lc, at = 0, at_c = 0, at_in = 0;
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) {
+        if (run < need) {
+          at = b0 + k;
+          at_c = run_c;
+          at_in = c[k];
+          at_q = run;
+        }
+        run += q[k];
+        run_c += c[k];
+      }
+#pragma unroll
+      for (int r = 0; r < TEAM; ++r) {
+        peer_store<TEAM>(&sh.first[m], r, ((u64)at_c << 32) | at);
+        peer_store<TEAM>(&sh.last[m], r, (u64)at_in);
+        peer_store<TEAM>(&sh.first_q[m], r, at_q);
+      }
+    }
+    team_sync<TEAM>();
+    auto narrow = [&](RankRange& g, u64& above, u64 need, int q2, int sft) {
+      if (!need) {  // nothing to reach
+        g = RankRange{kNowhere, 0u, 0u, 0u};
+        return;
+      }
+      const uint32_t cut = (uint32_t)sh.first[q2] << sft;
+      g.span = min(g.span - cut, (1u << sft) - 1u);
+      g.lo += cut;
+      g.above = (uint32_t)(sh.first[q2] >> 32);
+      g.in = (uint32_t)sh.last[q2];
+      above = sh.first_q[q2];
+    };
+    if (exact) {
+      narrow(r0, above0, need0, 0, shift0);
+      narrow(r1, above1, need1, 1, shift1);
+      if (r0.in <= kListCap && r1.in <= kListCap) break;
+    }
   }
+
+  // ---- (rare) too many keys in a range, or sums that were not exact: halve it with exact sweeps until its keys fit the
+  // list or are all alike
+  auto crowded = [](const RankRange& g) { return g.in > kListCap && g.span > 0; };
+  if (!exact) {
+    W0 = W1 = 0;
+    uint32_t c0 = 0, c1 = 0;
+    for (int r = 0; r < rounds; ++r) {
+      reload(r);
+#pragma unroll
+      for (int j = 0; j < KPT; ++j)
+        if (key[j] != kNoKey) {
+          const u64 q = psi_fix(kmax - key[j]);
+          if ((vis >> j) & 1u) { W0 += q; ++c0; } else { W1 += q; ++c1; }
+        }
+    }
+    W0 = warp_sum64(W0);
+    W1 = warp_sum64(W1);
+    team_sums(W0, W1);
+    u64 n0 = __reduce_add_sync(kFull, c0), n1 = __reduce_add_sync(kFull, c1);
+    team_sums(n0, n1);
+    need0 = target(W0);
+    need1 = target(W1);
+    r0 = need0 ? RankRange{0u, all_span, (uint32_t)n0, 0u} : RankRange{kNowhere, 0u, 0u, 0u};
+    r1 = need1 ? RankRange{0u, all_span, (uint32_t)n1, 0u} : RankRange{kNowhere, 0u, 0u, 0u};
+    above0 = above1 = 0;
+  }
+  while (crowded(r0) || crowded(r1)) {
+    const bool on0 = crowded(r0), on1 = crowded(r1);
+    const uint32_t mid0 = r0.lo + (r0.span >> 1), mid1 = r1.lo + (r1.span >> 1);
+    u64 a0 = 0, a1 = 0;
+    uint32_t c0 = 0, c1 = 0;
+    for (int r = 0; r < rounds; ++r) {
+      reload(r);
+#pragma unroll
+      for (int j = 0; j < KPT; ++j) {
+        const bool v = (vis >> j) & 1u;
+        if ((v ? on0 : on1) && key[j] >= (v ? r0.lo : r1.lo) && key[j] <= (v ? mid0 : mid1)) {
+          const u64 q = psi_fix(kmax - key[j]);
+          if (v) { a0 += q; ++c0; } else { a1 += q; ++c1; }
+        }
+      }
+    }
+    a0 = warp_sum64(a0);
+    a1 = warp_sum64(a1);
+    team_sums(a0, a1);
+    u64 n0 = __reduce_add_sync(kFull, c0), n1 = __reduce_add_sync(kFull, c1);
+    team_sums(n0, n1);
+    auto halve = [](RankRange& g, u64& above, u64 need, u64 a, uint32_t c) {
+      const uint32_t half = g.span >> 1;
+      if (above + a >= need) {
+        g.span = half;
+        g.in = c;
+      } else {
+        above += a;
+        g.above += c;
+        g.in -= c;
+        g.lo += half + 1;
+        g.span -= half + 1;
+      }
+    };
+    if (on0) halve(r0, above0, need0, a0, (uint32_t)n0);
+    if (on1) halve(r1, above1, need1, a1, (uint32_t)n1);
+  }
+  if (rank == 0 && tid < 2) {
+    const u64 W = tid ? W1 : W0, tot = W0 + W1;
+    p.mass[(int64_t)u * 2 + tid] = __ull2double_rn(W) / 4294967296.0;
+    p.pref[(int64_t)u * 2 + tid] = tot ? __ddiv_rn(__ull2double_rn(W), __ull2double_rn(tot)) : 0.0;
+    if ((tid ? need1 : need0) == 0) p.demand[(int64_t)u * 2 + tid] = 0;
+  }
+
+  // ---- the keys inside the ranges
+  for (int r = 0; r < rounds; ++r) {
+    reload(r);
+    uint32_t in = 0;
+#pragma unroll
+    for (int j = 0; j < KPT; ++j) {
+      const bool v = (vis >> j) & 1u;
+      if (key[j] - (v ? r0.lo : r1.lo) <= (v ? r0.span : r1.span)) in |= 1u << j;
+    }
+    append<TEAM, 2, KPT>(sh, r0.in <= kListCap ? in & vis : 0u, r1.in <= kListCap ? in & ~vis : 0u, key, r0.lo, r1.lo);
+  }
+  team_sync<TEAM>();
+
+  // ---- finish: block 0
+  if (rank == 0) {
+    const uint32_t got = gather_lists<TEAM, 2>(sh);
+    const bool on0 = need0 && r0.in <= kListCap, on1 = need1 && r1.in <= kListCap;
+    finish_lists<TEAM, 2, true>(sh, r0, r1, got, on0, on1, need0, need1, above0, above1, kmax);
+    if (tid < 2 && (tid ? need1 : need0)) {
+      // every key left has the value kmax - t: as few of them as reach the threshold
+      const RankRange my = tid ? r1 : r0;
+      const bool listed = tid ? on1 : on0;
+      uint32_t take = listed ? sh.fin_in[tid] : my.in;
+      if (take > 1) {
+        const u64 need = tid ? need1 : need0, above = listed ? sh.fin_m[tid] : (tid ? above1 : above0);
+        const u64 each = psi_fix(kmax - (listed ? sh.fin_lo[tid] : my.lo));
+        if (each > 0) {
+          const u64 k = (need - above + each - 1) / each;
+          if (k < (u64)take) take = (uint32_t)k;
+        }
+      }
+      p.demand[(int64_t)u * 2 + tid] = (int32_t)((listed ? sh.fin_c[tid] : my.above) + take);
+    }
+  }
+  if (TEAM > 1) team_sync<TEAM>();  // no block leaves while block 0 still reads its shared memory
 }
 
 // Visual tokens among the first n of a sequence, counted by the whole block into *s_nv (which the caller has zeroed
@@ -328,14 +410,21 @@ __device__ __forceinline__ long long layer_demand(const int32_t* demand_layer, i
 __device__ __forceinline__ double rounded_budget(double ph, double lo, double hi) {
   return fmin(fmax(floor(__dadd_rn(ph, 0.5)), lo), hi);
 }
-__device__ __forceinline__ double next_phi(double ph, long long dem, int Hkv, int L, int l, int hcc_mode, double lo,
-                                           double hi) {
+// The divisor of Eq. 11 for the step from layer l (0 for a mode without one) and its correctly rounded reciprocal: both
+// are known before the recurrence starts.
+__device__ __forceinline__ double phi_divisor(int Hkv, int L, int l, int hcc_mode) {
+  if (hcc_mode == MADAKV_HCC_PAPER || hcc_mode == MADAKV_HCC_DEMAND) return (double)((long long)Hkv * (L - l));  // per-head units
+  return hcc_mode == MADAKV_HCC_LITERAL ? (double)(L - l) : 0.0;  // Eq. 11 as printed
+}
+// K / div rounded to nearest, with the reciprocal at hand: the quotient of the product is within one unit in the last
+// place, and one correction by the exact remainder makes it the correctly rounded one (Markstein, "Computation of
+// elementary functions on the IBM RISC System/6000 processor", 1990). Three dependent operations instead of a division in
+// a chain that is one layer after the other (llava: 11.8 us for the 32 layers with divisions).
+__device__ __forceinline__ double next_phi(double ph, long long dem, int Hkv, double div, double rcp, double lo, double hi) {
   const double K = __dsub_rn((double)dem, __dmul_rn((double)Hkv, ph));  // Eq. 10
-  double next = ph;
-  if (hcc_mode == MADAKV_HCC_PAPER || hcc_mode == MADAKV_HCC_DEMAND)
-    next = __dsub_rn(ph, __ddiv_rn(K, (double)((long long)Hkv * (L - l))));  // Eq. 11, per-head units
-  else if (hcc_mode == MADAKV_HCC_LITERAL)
-    next = __dsub_rn(ph, __ddiv_rn(K, (double)(L - l)));  // Eq. 11 as printed
+  const double q = __dmul_rn(K, rcp);
+  const double quot = __fma_rn(__fma_rn(-q, div, K), rcp, q);
+  const double next = div > 0.0 ? __dsub_rn(ph, quot) : ph;  // Eq. 11
   return fmin(fmax(next, lo), hi);
 }
 // Eq. 8 integerised for one head: the visual share rounded half up, the rest to text, surplus of a modality with too
@@ -366,10 +455,12 @@ __device__ __forceinline__ void split_budget(const AllocParams& p, int64_t u, do
   p.budgets[u * 2 + 1] = bt;
 }
 
-// One block per sequence: Eq. 10-11 as a scalar scan over layers, then Eq. 8 integerised for every (layer, head).
-__global__ void alloc_seq_kernel(AllocParams p) {
-  extern __shared__ double s_Phi[];  // [L] rounded budgets, then [L] demand sums (as long long)
-  long long* s_dem = reinterpret_cast<long long*>(s_Phi + p.L);
+// One block per sequence: Eq. 10-11 as a scalar scan over layers, then Eq. 8 integerised for every (layer, head). The
+// tokens are counted before the wait for the kernel that computes the demands (it has waited for all kernels before
+// it, so mask and lengths are final).
+__global__ void __launch_bounds__(1024) alloc_seq_kernel(AllocParams p) {
+  extern __shared__ double s_phi[];  // [L] reciprocals of Eq. 11's divisors, replaced by phi; then [L] demand sums (as long long)
+  long long* s_dem = reinterpret_cast<long long*>(s_phi + p.L);
   __shared__ int s_nv, s_wv;
   const int b = blockIdx.x;
   const int n = clamped_len(p.seq_len, b, p.n_max);
@@ -378,6 +469,12 @@ __global__ void alloc_seq_kernel(AllocParams p) {
   __syncthreads();
   count_visual(p.mask + (int64_t)b * p.n_max, n, &s_nv);
   if (wlen > 0) count_visual(p.mask + (int64_t)b * p.n_max + (n - wlen), wlen, &s_wv);
+  for (int l = threadIdx.x; l < p.L; l += blockDim.x) {
+    const double div = l + 1 < p.L ? phi_divisor(p.Hkv, p.L, l + 1, p.hcc_mode) : 0.0;
+    s_phi[l] = div > 0.0 ? __drcp_rn(div) : 0.0;
+  }
+  pdl_wait();
+  pdl_go();
   // Eq. 10's sum over heads, one warp per layer (integers: any order gives the same sum)
   for (int l = threadIdx.x >> 5; l < p.L; l += blockDim.x >> 5) {
     const long long dem = layer_demand(p.demand + ((int64_t)b * p.L + l) * p.Hkv * 2, p.Hkv);
@@ -386,34 +483,41 @@ __global__ void alloc_seq_kernel(AllocParams p) {
   __syncthreads();
   const int n_v = s_nv, n_t = n - n_v;
   const int lo_v = p.mpa ? s_wv : 0, lo_t = wlen - lo_v;
+  const double lo = n >= 1 ? 1.0 : 0.0, hi = (double)n;
   if (threadIdx.x == 0) {
-    const double lo = n >= 1 ? 1.0 : 0.0, hi = (double)n;
     double ph = (double)p.budget[b];
-    for (int l = 1; l <= p.L; ++l) {
-      p.phi[(int64_t)b * p.L + (l - 1)] = ph;
-      s_Phi[l - 1] = rounded_budget(ph, lo, hi);
-      if (l < p.L) ph = next_phi(ph, s_dem[l - 1], p.Hkv, p.L, l, p.hcc_mode, lo, hi);
+#pragma unroll 4
+    for (int l = 0; l < p.L; ++l) {
+      const double rcp = s_phi[l];
+      s_phi[l] = ph;
+      if (l + 1 < p.L) ph = next_phi(ph, s_dem[l], p.Hkv, phi_divisor(p.Hkv, p.L, l + 1, p.hcc_mode), rcp, lo, hi);
     }
   }
   __syncthreads();
+  for (int l = threadIdx.x; l < p.L; l += blockDim.x) p.phi[(int64_t)b * p.L + l] = s_phi[l];
   for (int x = threadIdx.x; x < p.L * p.Hkv; x += blockDim.x)
-    split_budget(p, (int64_t)b * p.L * p.Hkv + x, s_Phi[x / p.Hkv], n, n_v, n_t, lo_v, lo_t,
+    split_budget(p, (int64_t)b * p.L * p.Hkv + x, rounded_budget(s_phi[x / p.Hkv], lo, hi), n, n_v, n_t, lo_v, lo_t,
                  p.hcc_mode == MADAKV_HCC_DEMAND && x / p.Hkv + 1 < p.L);
 }
 
 // One block per sequence, one layer of a layer-by-layer pass: the same arithmetic as one trip of the scan above. The
 // per-layer arrays (pref, demand, budgets) hold this layer only; phi [B, depth] is the state carried between calls.
-__global__ void alloc_layer_kernel(AllocParams p, int depth, int layer) {
+// `after_demand`: the kernel before this one in the stream is alloc_unit_kernel, which has waited for all kernels before it,
+// so the tokens can be counted before the wait for its results.
+__global__ void __launch_bounds__(1024) alloc_layer_kernel(AllocParams p, int depth, int layer, int after_demand) {
   __shared__ int s_nv, s_wv;
   __shared__ double s_Phi;
   __shared__ long long s_dem;
   const int b = blockIdx.x;
+  if (!after_demand) pdl_wait();
   const int n = clamped_len(p.seq_len, b, p.n_max);
   const int wlen = p.keep_window ? min(p.window, n) : 0;
   if (threadIdx.x == 0) s_nv = s_wv = 0;
   __syncthreads();
   count_visual(p.mask + (int64_t)b * p.n_max, n, &s_nv);
   if (wlen > 0) count_visual(p.mask + (int64_t)b * p.n_max + (n - wlen), wlen, &s_wv);
+  if (after_demand) pdl_wait();
+  pdl_go();
   if (threadIdx.x < 32) {
     const long long dem = layer_demand(p.demand + (int64_t)b * p.Hkv * 2, p.Hkv);
     if (threadIdx.x == 0) s_dem = dem;
@@ -432,7 +536,10 @@ __global__ void alloc_layer_kernel(AllocParams p, int depth, int layer) {
       ph = p.phi[(int64_t)b * depth + layer];
     }
     s_Phi = rounded_budget(ph, lo, hi);
-    if (l < depth) p.phi[(int64_t)b * depth + l] = next_phi(ph, s_dem, p.Hkv, depth, l, p.hcc_mode, lo, hi);
+    if (l < depth) {
+      const double div = phi_divisor(p.Hkv, depth, l, p.hcc_mode);
+      p.phi[(int64_t)b * depth + l] = next_phi(ph, s_dem, p.Hkv, div, div > 0.0 ? __drcp_rn(div) : 0.0, lo, hi);
+    }
   }
   __syncthreads();
   for (int x = threadIdx.x; x < p.Hkv; x += blockDim.x)
@@ -440,10 +547,18 @@ __global__ void alloc_layer_kernel(AllocParams p, int depth, int layer) {
                  p.hcc_mode == MADAKV_HCC_DEMAND && layer + 1 < depth);
 }
 
-// 8-bit digits while every sequence fits one round of the kernel, 10-bit digits beyond
 void launch_alloc_unit(const madakv_config& c, const AllocParams& p, int units, cudaStream_t st) {
-  if (c.max_seq_len <= ROUND) alloc_unit_kernel<8><<<units, NT, 0, st>>>(p);
-  else alloc_unit_kernel<10><<<units, NT, 0, st>>>(p);
+  const RankShape s = rank_shape(units, c.max_seq_len);
+  switch (s.kpt + s.team) {
+    case 8 + 1: launch_team(alloc_unit_kernel<8, 1>, units, 1, st, p); break;
+    case 8 + 2: launch_team(alloc_unit_kernel<8, 2>, units, 2, st, p); break;
+    case 8 + 4: launch_team(alloc_unit_kernel<8, 4>, units, 4, st, p); break;
+    case 8 + 8: launch_team(alloc_unit_kernel<8, 8>, units, 8, st, p); break;
+    case 16 + 1: launch_team(alloc_unit_kernel<16, 1>, units, 1, st, p); break;
+    case 16 + 2: launch_team(alloc_unit_kernel<16, 2>, units, 2, st, p); break;
+    case 16 + 4: launch_team(alloc_unit_kernel<16, 4>, units, 4, st, p); break;
+    default: launch_team(alloc_unit_kernel<16, 8>, units, 8, st, p); break;
+  }
 }
 
 }  // namespace
@@ -472,7 +587,7 @@ int launch_allocate(const madakv_config& c, const float* psi, const uint8_t* mas
   p.theta_fix = (u64)((double)c.theta * 4294967296.0);
   const int units = c.batch * c.n_layers * c.n_kv_heads;
   launch_alloc_unit(c, p, units, st);
-  alloc_seq_kernel<<<c.batch, 1024, c.n_layers * (sizeof(double) + sizeof(long long)), st>>>(p);
+  launch_pdl(alloc_seq_kernel, dim3(c.batch), dim3(1024), c.n_layers * (sizeof(double) + sizeof(long long)), st, p);
   return launch_status();
 }
 
@@ -499,7 +614,7 @@ int launch_allocate_layer(const madakv_config& c, int layer, const float* psi, c
   p.window = c.window;
   p.theta_fix = (u64)((double)c.theta * 4294967296.0);
   if (psi) launch_alloc_unit(c, p, c.batch * c.n_kv_heads, st);  // else: done by launch_demand_layer
-  alloc_layer_kernel<<<c.batch, 1024, 0, st>>>(p, c.n_layers, layer);
+  launch_pdl(alloc_layer_kernel, dim3(c.batch), dim3(1024), 0, st, p, c.n_layers, layer, psi ? 1 : 0);
   return launch_status();
 }
 

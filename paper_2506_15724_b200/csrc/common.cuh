@@ -142,24 +142,35 @@ inline int launch_status() {
 // still running, which hides its launch latency. A kernel launched this way calls pdl_wait() before it touches global
 // memory (the call returns once the kernels before it have completed and their writes are visible; it is a no-op in a
 // kernel launched the ordinary way) and pdl_go() to let the kernel after it be scheduled.
+// `team` > 1 launches thread-block clusters of that many blocks.
 template <typename... KArgs, typename... Args>
-inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+inline void launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int team, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
+  cfg.attrs = attr;
+  if (team > 1) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = (unsigned)team;
+    attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
+    ++cfg.numAttrs;
+  }
   // a stream that is being captured gets the ordinary launch (full serialisation: the waits in the kernels are no-ops)
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusActive;
   if (cap == cudaStreamCaptureStatusNone) {
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+    ++cfg.numAttrs;
   }
-  cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+  cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);  // (a failure is what launch_status() reports)
+}
+template <typename... KArgs, typename... Args>
+inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+  launch_ex(kernel, grid, block, smem, st, 1, args...);
 }
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -188,9 +199,13 @@ __device__ __forceinline__ uint32_t nonzero_bytes(uint32_t w) {
   const uint32_t x = ((((w & 0x7f7f7f7fu) + 0x7f7f7f7fu) | w) & 0x80808080u) >> 7;  // bits 0, 8, 16, 24
   return (x & 1u) | ((x >> 7) & 2u) | ((x >> 14) & 4u) | ((x >> 21) & 8u);
 }
-// floor(x * 2^32) of a key produced by psi_key.
+// floor(x * 2^32) of a key produced by psi_key, by shifting the 24-bit significand into place (the conversion instruction
+// gives the same number but runs at a small fraction of the rate of integer instructions): exponent field e stands for
+// significand * 2^(e - 150), so the product is (significand << 40) >> (158 - e). Values of 2^32 and more saturate.
 __device__ __forceinline__ unsigned long long psi_fix(uint32_t key) {
-  return key ? __float2ull_rz(__uint_as_float(key) * 4294967296.0f) : 0ull;
+  const uint32_t top = key >= (95u << 23) ? (key << 8) | 0x80000000u : 0u;  // below 2^-32: 0
+  const unsigned long long q = ((unsigned long long)top << 32) >> ((158u - (key >> 23)) & 63u);
+  return key >= (159u << 23) ? ~0ull : q;
 }
 
 __device__ __forceinline__ void set_status(void* ws, int code) { atomicCAS((int*)ws, 0, code); }

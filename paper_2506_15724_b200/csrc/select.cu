@@ -2,30 +2,19 @@
 //
 //   seg_scan     one block: visual-token count of every sequence, kept_len[u] = b_v + b_t and the exclusive scan
 //                seg_off (rows, with headroom)
-//   select_unit  one block per unit: a three- or four-pass shared-memory radix select over the order-preserving bit pattern of
-//                psi finds, for both modalities at once, the budget-th largest value and how many of its ties are
-//                still needed; an ordered sweep then emits the kept positions in ascending order, giving ties to
-//                the lowest positions (block-wide prefix scans provide the tie ranks and the output slots).
-//                A thread owns KPT consecutive positions and keeps their keys in registers from the first pass to
-//                the sweep (sequences longer than one chunk are re-read from L2 chunk by chunk).
+//   select_unit  a team of blocks per unit (rank_common.cuh) finds, for both modalities at once, the budget-th largest
+//                value and how many of its ties are still needed; an ordered sweep then emits the kept positions in
+//                ascending order, giving ties to the lowest positions (prefix sums over the team provide the tie ranks
+//                and the output slots). It runs beside seg_scan and waits for the segment offsets only before it emits.
 // Two options outside the paper: with pooling the ranking key of a position is the maximum of the keys of the
 // positions around it (a maximum of fp32 values is exact, so nothing changes for the integer results); with
 // forced retention the proxy tokens are emitted by the sweep without taking part in the ranking, and the wanted
 // counts shrink by their number.
 // Integer work only: results are bit-exact functions of (psi bits, mask, budgets).
-#include "common.cuh"
+#include "rank_common.cuh"
 
 namespace madakv {
 namespace {
-
-constexpr int NT = 256;
-constexpr int KPT = 32;                // consecutive positions per thread
-constexpr int CHUNK = NT * KPT;        // 8192 positions per chunk
-constexpr unsigned int kFull = 0xffffffffu;
-// A radix digit has DIG bits: 10 for configs whose sequences are longer than one chunk (they are re-read from L2 in
-// every pass, and the 30 bits in which importance values differ at most then take three passes instead of four),
-// 8 for those that sit in registers (the larger histograms only cost there). Bucket b of a modality sits at word
-// b + b / kPerLane, so that the lanes of the walking warp (lane j owns buckets kPerLane * j ..) read 32 different banks.
 
 struct SelParams {
   const float* psi;
@@ -42,42 +31,50 @@ struct SelParams {
   int units, B, L, Hkv, n_max, mpa, headroom, keep_window, window, pool_r;  // pool_r: (pool_kernel - 1) / 2
 };
 
+// One block. The visual tokens are counted by warps that share the sequences (several warps per sequence when there are
+// fewer sequences than warps), then the segments are scanned, 1024 units at a time.
 __global__ void __launch_bounds__(1024) seg_scan_kernel(SelParams p) {
   __shared__ long long warp_tot[32];
   __shared__ long long carry;
-  __shared__ int s_cnt, s_wcnt;
+  __shared__ int s_cnt[32], s_wcnt[32];
+  pdl_wait();
+  pdl_go();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // visual tokens among the first seq_len[b] positions of every sequence
-  for (int b = 0; b < p.B; ++b) {
-    const int n = clamped_len(p.seq_len, b, p.n_max);
-    const uint8_t* mask = p.mask + (int64_t)b * p.n_max;
-    const int wfrom = p.keep_window ? max(n - p.window, 0) : n;  // first proxy token retained unconditionally
-    if (threadIdx.x == 0) s_cnt = s_wcnt = 0;
+  const int share = p.B >= 32 ? 1 : 32 / p.B;  // warps per sequence
+  for (int b0 = 0; b0 < p.B; b0 += 32 / share) {
+    if (warp == 0) s_cnt[lane] = s_wcnt[lane] = 0;
     __syncthreads();
-    int c = 0, cw = 0;  // visual tokens, visual proxy tokens
-    if (p.mpa) {
-      int done = 0;
-      if ((reinterpret_cast<uintptr_t>(mask) & 15) == 0) {  // 16 mask bytes per load
-        const int n16 = n >> 4;
-        for (int i = threadIdx.x; i < n16; i += 1024) {
-          const uint4 v = __ldg(reinterpret_cast<const uint4*>(mask) + i);
+    const int slot = warp / share, b = b0 + slot, part = warp % share;
+    if (slot < 32 / share && b < p.B) {
+      const int n = clamped_len(p.seq_len, b, p.n_max);
+      const uint8_t* mask = p.mask + (int64_t)b * p.n_max;
+      const int wfrom = p.keep_window ? max(n - p.window, 0) : n;  // first proxy token retained unconditionally
+      int c = 0, cw = 0;                                           // visual tokens, visual proxy tokens
+      if (p.mpa) {
+        // whole 16-byte pieces of the row by vector loads, its ends by bytes
+        const int lead = min(n, (int)((16 - (reinterpret_cast<uintptr_t>(mask) & 15)) & 15));
+        const int n16 = (n - lead) >> 4;
+        for (int i = part * 32 + lane; i < n16; i += share * 32) {
+          const uint4 v = __ldg(reinterpret_cast<const uint4*>(mask + lead) + i);
           c += __popc(nonzero_bytes(v.x) | (nonzero_bytes(v.y) << 4) | (nonzero_bytes(v.z) << 8) | (nonzero_bytes(v.w) << 12));
         }
-        done = n16 << 4;
+        if (part == 0) {
+          if (lane < lead) c += mask[lane] ? 1 : 0;
+          const int i = lead + (n16 << 4) + lane;
+          if (i < n) c += mask[i] ? 1 : 0;
+        }
+        for (int i = wfrom + part * 32 + lane; i < n; i += share * 32) cw += mask[i] ? 1 : 0;  // (no proxy tokens: wfrom = n)
       }
-      for (int i = done + threadIdx.x; i < n; i += 1024) c += mask[i] ? 1 : 0;
-      for (int i = wfrom + threadIdx.x; i < n; i += 1024) cw += mask[i] ? 1 : 0;  // (no proxy tokens: wfrom = n)
+      c = __reduce_add_sync(kFull, c);
+      cw = __reduce_add_sync(kFull, cw);
+      if (lane == 0 && c) atomicAdd(&s_cnt[slot], c);
+      if (lane == 0 && cw) atomicAdd(&s_wcnt[slot], cw);
     }
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) {
-      c += __shfl_xor_sync(kFull, c, off);
-      cw += __shfl_xor_sync(kFull, cw, off);
-    }
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&s_cnt, c);
-    if ((threadIdx.x & 31) == 0 && cw) atomicAdd(&s_wcnt, cw);
     __syncthreads();
-    if (threadIdx.x == 0) {
-      p.seq_nv[b] = s_cnt;
-      p.seq_wv[b] = s_wcnt;
+    if (warp == 0 && lane < 32 / share && b0 + lane < p.B) {
+      p.seq_nv[b0 + lane] = s_cnt[lane];
+      p.seq_wv[b0 + lane] = s_wcnt[lane];
     }
     __syncthreads();
   }
@@ -117,271 +114,351 @@ __global__ void __launch_bounds__(1024) seg_scan_kernel(SelParams p) {
   }
 }
 
-// Exclusive block scan of a packed pair of 16-bit counters (each total <= CHUNK < 65536).
-__device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* warp_tot, uint32_t* total) {
-  uint32_t incl = v;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const uint32_t t = __shfl_up_sync(kFull, incl, off);
-    if ((threadIdx.x & 31) >= off) incl += t;
-  }
-  __syncthreads();
-  if ((threadIdx.x & 31) == 31) warp_tot[threadIdx.x >> 5] = incl;
-  __syncthreads();
-  uint32_t wbase = 0, tot = 0;
-#pragma unroll
-  for (int i = 0; i < NT / 32; ++i) {
-    const uint32_t t = warp_tot[i];
-    if (i < (int)(threadIdx.x >> 5)) wbase += t;
-    tot += t;
-  }
-  *total = tot;
-  return wbase + incl - v;
-}
-
+// Keys of the two options: the maximum over the 2 * pool_r + 1 positions around each of KPT consecutive ones (pool_r may
+// be 0; positions outside the sequence do not count).
 constexpr int kMaxPoolR = 7;  // pool_kernel <= 15
-
-// Keys of KPT consecutive positions from pos0. valid: positions that take part in the ranking (inside the sequence
-// and not retained unconditionally); forced: proxy tokens retained unconditionally (positions wfrom .. n-1);
-// vis: visual tokens. kPool is the variant for the two options outside the paper: the key of a position is the maximum
-// over the 2 * pool_r + 1 positions around it (pool_r may be 0), and the proxy tokens from wfrom on are forced; without
-// kPool neither exists and the code is the plain paper-literal selection.
-template <bool kVec, bool kPool>
-__device__ __forceinline__ void load_chunk(const float* psi, const uint8_t* mask, int n, int pos0, int mpa, int wfrom,
-                                           int pool_r, uint32_t (&key)[KPT], uint32_t& valid, uint32_t& vis,
-                                           uint32_t& forced) {
-  valid = 0;
-  vis = 0;
-  forced = 0;
-  if (kPool) {
-    uint32_t e[KPT + 2 * kMaxPoolR];  // keys of positions pos0 - 7 .. pos0 + KPT + 6 (0 outside the sequence)
+template <int KPT>
+__device__ __forceinline__ void load_pooled(const float* row, int mis, int n, int pos0, int pool_r, uint32_t (&key)[KPT]) {
+  uint32_t e[KPT + 16];  // keys of positions pos0 - 8 .. pos0 + KPT + 7
+  if (mis == 0 && pos0 >= 8 && pos0 + KPT + 8 <= n) {
 #pragma unroll
-    for (int x = 0; x < KPT + 2 * kMaxPoolR; ++x) {
-      const int pos = pos0 - kMaxPoolR + x;
-      e[x] = (pos >= 0 && pos < n) ? psi_key(__ldg(psi + pos)) : 0u;
+    for (int x = 0; x < KPT + 16; x += 4) {
+      const float4 v = __ldg(reinterpret_cast<const float4*>(row + pos0 - 8 + x));
+      e[x] = score_key(v.x);
+      e[x + 1] = score_key(v.y);
+      e[x + 2] = score_key(v.z);
+      e[x + 3] = score_key(v.w);
     }
-#pragma unroll
-    for (int j = 0; j < KPT; ++j) {
-      uint32_t m = e[j + kMaxPoolR];
-#pragma unroll
-      for (int d = 1; d <= kMaxPoolR; ++d)
-        if (d <= pool_r) m = max(m, max(e[j + kMaxPoolR - d], e[j + kMaxPoolR + d]));
-      key[j] = pos0 + j < n ? m : 0u;
-      if (pos0 + j < n) valid |= 1u << j;
-    }
-  } else if (kVec && pos0 + KPT <= n) {
-#pragma unroll
-    for (int j = 0; j < KPT; j += 4) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(psi + pos0 + j));
-      key[j] = psi_key(v.x);
-      key[j + 1] = psi_key(v.y);
-      key[j + 2] = psi_key(v.z);
-      key[j + 3] = psi_key(v.w);
-    }
-    valid = 0xffffffffu;
   } else {
 #pragma unroll
-    for (int j = 0; j < KPT; ++j) {
-      key[j] = 0;
-      if (pos0 + j < n) {
-        key[j] = psi_key(__ldg(psi + pos0 + j));
-        valid |= 1u << j;
-      }
+    for (int x = 0; x < KPT + 16; ++x) {
+      const int pos = pos0 - 8 + x;
+      e[x] = (pos >= 0 && pos < n) ? score_key(__ldg(row + pos)) : 0u;
     }
   }
-  if (mpa) {
-    if (kVec && pos0 + KPT <= n && (reinterpret_cast<uintptr_t>(mask + pos0) & 15) == 0) {  // 16 mask bytes per load
 #pragma unroll
-      for (int j = 0; j < KPT; j += 16) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(mask + pos0 + j));
-        vis |= (nonzero_bytes(v.x) | (nonzero_bytes(v.y) << 4) | (nonzero_bytes(v.z) << 8) | (nonzero_bytes(v.w) << 12)) << j;
-      }
-    } else {
+  for (int j = 0; j < KPT; ++j) {
+    uint32_t m = e[j + 8];
 #pragma unroll
-      for (int j = 0; j < KPT; ++j)
-        if (pos0 + j < n && __ldg(mask + pos0 + j)) vis |= 1u << j;
-    }
-  }
-  if (kPool && pos0 + KPT > wfrom) {  // proxy tokens retained unconditionally: out of the ranking, into the output
-#pragma unroll
-    for (int j = 0; j < KPT; ++j)
-      if (pos0 + j >= wfrom && pos0 + j < n) forced |= 1u << j;
-    valid &= ~forced;
+    for (int d = 1; d <= kMaxPoolR; ++d)
+      if (d <= pool_r) m = max(m, max(e[j + 8 - d], e[j + 8 + d]));
+    key[j] = m;
   }
 }
 
-// The radix digits are taken from t = kmax - key, starting at the highest bit in which the unit's keys differ
-// (kmax, kmin: largest and smallest key of the unit): importance values share their sign and most exponent bits,
-// so digits of the raw key would put nearly all keys into a handful of buckets and serialise the shared atomics.
-// Ascending t is descending importance.
-template <bool kVec, bool kPool, int DIG>
-__global__ void __launch_bounds__(NT) select_unit_kernel(SelParams p) {
-  constexpr int kDigitBits = DIG, kBuckets = 1 << DIG, kPerLane = kBuckets / 32, kCntWords = kBuckets + 32;
-  auto cnt_slot = [](uint32_t digit) { return (int)(digit + digit / kPerLane); };
-  __shared__ unsigned int cnt[2][kCntWords];
-  __shared__ uint32_t s_prefix[2];
-  __shared__ unsigned int s_above[2];
-  __shared__ uint32_t warp_tot[NT / 32];
-  __shared__ uint32_t s_red[2][NT / 32];
-
-  const int u = blockIdx.x;
+template <int KPT, int TEAM, bool kPool>
+__global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(SelParams p) {
+  using SH = RankShared<TEAM, 1>;
+  constexpr int kPer = SH::kPer;
+  __shared__ SH sh;
+  // (no wait here: seg_scan, the kernel before, has waited for everything before it, so the scores, the mask and the
+  // budgets are final; what seg_scan itself writes is read after the wait below)
+  const uint32_t rank = TEAM > 1 ? team_rank() : 0u;
+  const int u = blockIdx.x / TEAM;
   const int b = u / (p.Hkv * p.L);
-  const int n = clamped_len(p.seq_len, b, p.n_max);
   const float* psi = p.psi + (int64_t)u * p.n_max;
+  const int mis = (int)(((int64_t)u * p.n_max) & 3);
   const uint8_t* mask = p.mask + (int64_t)b * p.n_max;
-  const int64_t off0 = p.seg_off[u];
-  if (off0 + p.kept_len[u] + p.headroom > p.capacity) return;  // seg_scan has raised MADAKV_ECAPACITY
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int kRound = kRankThreads * KPT;
+  const int rounds = (p.n_max + kRound * TEAM - 1) / (kRound * TEAM);
+  const int pos_first = (int)rank * rounds * kRound + tid * KPT;  // a block owns consecutive positions
+  const int n = clamped_len(p.seq_len, b, p.n_max);
   // proxy tokens retained unconditionally (none without cfg->keep_window): they are emitted by the sweep and the
   // ranking only has to find the rest of each modality's budget
   const int wfrom = kPool && p.keep_window ? max(n - p.window, 0) : n;
+  if (kPool) pdl_wait();  // (the forced tokens' counts are seg_scan's)
   const int lo_v = kPool ? p.seq_wv[b] : 0, lo_t = (n - wfrom) - lo_v;
-  const int want0 = p.mpa ? max(p.budgets[2 * u] - lo_v, 0) : 0, want1 = max(p.budgets[2 * u + 1] - lo_t, 0);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int chunks = (n + CHUNK - 1) / CHUNK;
+  const uint32_t want0 = (uint32_t)(p.mpa ? max(p.budgets[2 * u] - lo_v, 0) : 0),
+                 want1 = (uint32_t)max(p.budgets[2 * u + 1] - lo_t, 0);
 
-  // range of the unit's keys (the chunk stays in registers when there is only one)
-  uint32_t key[KPT], valid = 0, vis = 0, forced = 0;
+  uint32_t key[KPT], vis = 0, forced = 0;
+  auto load_round = [&](int r) {
+    const int pos0 = pos_first + r * kRound;
+    if (kPool) load_pooled<KPT>(psi, mis, n, pos0, p.pool_r, key);
+    else load_scores<KPT>(psi, mis, p.n_max, pos0, key);
+    vis = p.mpa ? load_mask<KPT>(mask, p.n_max, pos0) : 0u;
+    uint32_t valid = valid_bits<KPT>(n, pos0);
+    if (kPool) {  // proxy tokens retained unconditionally: not ranked, always emitted
+      forced = valid & ~valid_bits<KPT>(wfrom, pos0);
+      valid &= ~forced;
+    }
+    if (valid != valid_bits<KPT>(KPT, 0)) {
+#pragma unroll
+      for (int j = 0; j < KPT; ++j)
+        if (!((valid >> j) & 1u)) key[j] = kNoKey;
+    }
+  };
+
+  // ---- range of the keys
   uint32_t kmax = 0, kmin = 0xffffffffu;
-  for (int c = 0; c < chunks; ++c) {
-    load_chunk<kVec, kPool>(psi, mask, n, c * CHUNK + (int)threadIdx.x * KPT, p.mpa, wfrom, p.pool_r, key, valid, vis, forced);
+  for (int r = 0; r < rounds; ++r) {
+    load_round(r);
 #pragma unroll
-    for (int j = 0; j < KPT; ++j)
-      if ((valid >> j) & 1u) {
-        kmax = max(kmax, key[j]);
-        kmin = min(kmin, key[j]);
-      }
-  }
-  kmax = __reduce_max_sync(kFull, kmax);
-  kmin = __reduce_min_sync(kFull, kmin);
-  if (lane == 0) {
-    s_red[0][warp] = kmax;
-    s_red[1][warp] = kmin;
-  }
-  if (threadIdx.x < 2) {
-    s_prefix[threadIdx.x] = 0;
-    s_above[threadIdx.x] = 0;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < NT / 32; ++i) {
-    kmax = max(kmax, s_red[0][i]);
-    kmin = min(kmin, s_red[1][i]);
-  }
-  if (kmin > kmax) kmin = kmax;  // no keys at all
-  const int top = 32 - __clz(kmax - kmin);  // significant bits of t; 0 when all keys are equal
-  if (chunks == 1) {
-#pragma unroll
-    for (int j = 0; j < KPT; ++j) key[j] = (valid >> j) & 1u ? kmax - key[j] : 0xffffffffu;
-  }
-
-  // radix select: when all bits of t are resolved, s_prefix[m] is the t of the want[m]-th largest key of modality m
-  // (if that many exist) and s_above[m] counts the keys strictly above it. `rem` counts the bits not yet resolved.
-  for (int rem = top; rem > 0;) {
-    const int bits = min(rem, kDigitBits), shift = rem - bits;
-    const uint32_t dmask = (1u << bits) - 1u;
-    for (int x = threadIdx.x; x < 2 * kCntWords; x += NT) (&cnt[0][0])[x] = 0;
-    __syncthreads();
-    const uint32_t pre0 = s_prefix[0], pre1 = s_prefix[1];
-    for (int c = 0; c < chunks; ++c) {
-      if (chunks > 1) {
-        load_chunk<kVec, kPool>(psi, mask, n, c * CHUNK + (int)threadIdx.x * KPT, p.mpa, wfrom, p.pool_r, key, valid, vis, forced);
-#pragma unroll
-        for (int j = 0; j < KPT; ++j) key[j] = (valid >> j) & 1u ? kmax - key[j] : 0xffffffffu;
-      }
-#pragma unroll
-      for (int j = 0; j < KPT; ++j) {  // (a position outside the ranking holds all ones: no prefix equals its shifted t)
-        const int m = (vis >> j) & 1u ? 0 : 1;
-        if ((key[j] >> rem) == (m == 0 ? pre0 : pre1)) atomicAdd(&cnt[m][cnt_slot((key[j] >> shift) & dmask)], 1u);
-      }
+    for (int j = 0; j < KPT; ++j) {
+      kmax = (uint32_t)max((int)kmax, (int)key[j]);  // (kNoKey is negative)
+      kmin = min(kmin, key[j]);
     }
-    __syncthreads();
-    if (warp < 2) {
-      // warp m walks modality m's buckets in ascending digit order: a prefix scan of the lanes' totals tells which
-      // lane holds the bucket that takes the running count to `want` (lane 31 if none does), and that lane alone
-      // walks its buckets
-      const int m = warp;
-      const unsigned int want = (unsigned int)(m == 0 ? want0 : want1);
-      unsigned int lc = 0;
-#pragma unroll 8
-      for (int i = 0; i < kPerLane; ++i) lc += cnt[m][cnt_slot(lane * kPerLane + i)];
-      unsigned int sc = lc;
+  }
+  team_range<TEAM, 1>(sh, rank, kmax, kmin);
+  auto to_t = [&]() {
 #pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const unsigned int t = __shfl_up_sync(kFull, sc, off);
-        if (lane >= off) sc += t;
+    for (int j = 0; j < KPT; ++j) key[j] = key[j] == kNoKey ? kNoKey : kmax - key[j];
+  };
+  if (rounds == 1) to_t();
+  auto reload = [&](int r) {
+    if (rounds > 1) {
+      load_round(r);
+      to_t();
+    }
+  };
+
+  RankRange r0 = want0 ? RankRange{0u, kmax - kmin, kNoKey, 0u} : RankRange{kNowhere, 0u, 0u, 0u};
+  RankRange r1 = want1 ? RankRange{0u, kmax - kmin, kNoKey, 0u} : RankRange{kNowhere, 0u, 0u, 0u};
+  bool short0 = false, short1 = false;  // the modality has no more keys than are wanted: all of them are kept
+  auto crowded = [](const RankRange& g) { return g.in > kListCap && g.span > 0; };
+
+  for (int pass = 0; pass < 2; ++pass) {
+    // ---- buckets
+    const int shift0 = range_shift(pass ? r0.span : kmax - kmin, SH::kDig), shift1 = range_shift(pass ? r1.span : kmax - kmin, SH::kDig);
+    if (pass == 0) {  // all keys take part, both modalities over the same range (one of which nothing is wanted is not walked)
+      for (int r = 0; r < rounds; ++r) {
+        reload(r);
+#pragma unroll
+        for (int j = 0; j < KPT; ++j)
+          atomicAdd(sh.cnt + ((vis >> j) & 1u ? 0 : SH::kStride) + min(key[j] >> shift0, (uint32_t)SH::kBuckets), 1u);
       }
-      unsigned int above = s_above[m] + (sc - lc);
-      const unsigned int hit = __ballot_sync(kFull, above + lc >= want || lane == 31);
-      if (lane == __ffs(hit) - 1) {
-        int found = kPerLane - 1;
-        for (int i = 0; i < kPerLane; ++i) {
-          const unsigned int ci = cnt[m][cnt_slot(lane * kPerLane + i)];
-          if (above + ci >= want || i == kPerLane - 1) {
-            found = i;
-            break;
-          }
-          above += ci;
+    } else {
+      for (int x = tid; x < 2 * SH::kStride / 4; x += kRankThreads) reinterpret_cast<uint4*>(sh.cnt)[x] = make_uint4(0, 0, 0, 0);
+      __syncthreads();
+      for (int r = 0; r < rounds; ++r) {
+        reload(r);
+#pragma unroll
+        for (int j = 0; j < KPT; ++j) {
+          const bool v = (vis >> j) & 1u;
+          const uint32_t x = key[j] - (v ? r0.lo : r1.lo);
+          if (x <= (v ? r0.span : r1.span)) atomicAdd(sh.cnt + (v ? 0 : SH::kStride) + (x >> (v ? shift0 : shift1)), 1u);
         }
-        // buckets beyond the pass's digit range are empty; landing there means "fewer keys than wanted"
-        s_above[m] = above;
-        s_prefix[m] = (s_prefix[m] << bits) | min((uint32_t)(lane * kPerLane + found), dmask);
       }
     }
-    __syncthreads();
-    rem = shift;
-  }
-  const uint32_t thr0 = s_prefix[0], thr1 = s_prefix[1];
-  // ties at the threshold value that are still needed (all of them if the modality has fewer tokens than wanted)
-  const int ties0 = max(want0 - (int)s_above[0], 0), ties1 = max(want1 - (int)s_above[1], 0);
-
-  // ordered sweep: a thread's positions are consecutive, threads and chunks follow in position order
-  int tie_run0 = 0, tie_run1 = 0;  // threshold-valued keys met in earlier chunks, per modality
-  int out_run = 0;                 // kept positions emitted by earlier chunks
-  for (int c = 0; c < chunks; ++c) {
-    const int pos0 = c * CHUNK + (int)threadIdx.x * KPT;
-    if (chunks > 1) {
-      load_chunk<kVec, kPool>(psi, mask, n, pos0, p.mpa, wfrom, p.pool_r, key, valid, vis, forced);
+    // ---- walk: block r of the team adds up its share of the buckets over all blocks; half of the threads per modality
+    const int m = tid / kHalf, i = tid % kHalf;
+    const uint32_t b0 = (rank * kHalf + i) * kPer;
+    const uint32_t want = m ? want1 : want0;
+    if (i == 0) sh.first[m] = ~0ull;  // (stays if the modality has fewer keys than wanted)
+    team_sync<TEAM>();
+    uint32_t c[kPer], lc = 0;
+    bucket_counts<TEAM, 1>(sh, m * SH::kStride + b0, c);
 #pragma unroll
-      for (int j = 0; j < KPT; ++j) key[j] = (valid >> j) & 1u ? kmax - key[j] : 0xffffffffu;
+    for (int k = 0; k < kPer; ++k) lc += c[k];
+    uint32_t ic = warp_scan32(lc);
+    if (lane == 31) sh.wscan_c[warp] = ic;
+    __syncthreads();
+    ic += __reduce_add_sync(kFull, lane >= m * (kRankWarps / 2) && lane < warp ? sh.wscan_c[lane] : 0u);
+    if (TEAM > 1) {
+      if (i >= kHalf - 32) {  // the last warp of the modality has the block's total (in its last lane): to every block
+        const uint32_t tc = __shfl_sync(kFull, ic, 31);
+        if (lane < TEAM) peer_store<TEAM>(&sh.slice_c[m][rank], lane, tc);
+      }
+      team_sync<TEAM>();
+      ic += __reduce_add_sync(kFull, lane < (int)rank ? sh.slice_c[m][lane] : 0u);
     }
-    uint32_t eq_bits = 0, gt_bits = 0;
+    ic += m ? r1.above : r0.above;
+    if (want && ic - lc < want && ic >= want) {
+      uint32_t run = ic - lc, at = 0, at_c = 0, at_in = 0;
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) {
+        if (run < want) {
+          at = b0 + k;
+          at_c = run;
+          at_in = c[k];
+        }
+        run += c[k];
+      }
+#pragma unroll
+      for (int r = 0; r < TEAM; ++r) {
+        peer_store<TEAM>(&sh.first[m], r, ((u64)at_c << 32) | at);
+        peer_store<TEAM>(&sh.last[m], r, (u64)at_in);
+      }
+    }
+    team_sync<TEAM>();
+    {
+      auto narrow = [&](RankRange& g, bool& is_short, int q, int s) {
+        if (sh.first[q] == ~0ull) {
+          is_short = true;
+          g = RankRange{kNowhere, 0u, 0u, 0u};
+          return;
+        }
+        const uint32_t cut = (uint32_t)sh.first[q] << s;
+        g.span = min(g.span - cut, (1u << s) - 1u);
+        g.lo += cut;
+        g.above = (uint32_t)(sh.first[q] >> 32);
+        g.in = (uint32_t)sh.last[q];
+      };
+      if (want0 && !short0) narrow(r0, short0, 0, shift0);
+      if (want1 && !short1) narrow(r1, short1, 1, shift1);
+    }
+    if (!crowded(r0) && !crowded(r1)) break;
+  }
+
+  // ---- (rare) too many keys in a range: halve it with exact sweeps until they fit the list or are all alike
+  while (crowded(r0) || crowded(r1)) {
+    const bool on0 = crowded(r0), on1 = crowded(r1);
+    const uint32_t mid0 = r0.lo + (r0.span >> 1), mid1 = r1.lo + (r1.span >> 1);
+    uint32_t c0 = 0, c1 = 0;
+    for (int r = 0; r < rounds; ++r) {
+      reload(r);
+#pragma unroll
+      for (int j = 0; j < KPT; ++j) {
+        const bool v = (vis >> j) & 1u;
+        if ((v ? on0 : on1) && key[j] >= (v ? r0.lo : r1.lo) && key[j] <= (v ? mid0 : mid1)) {
+          if (v) ++c0; else ++c1;
+        }
+      }
+    }
+    c0 = __reduce_add_sync(kFull, c0);
+    c1 = __reduce_add_sync(kFull, c1);
+    if (lane == 0) {
+      sh.wcnt[0][warp] = c0;
+      sh.wcnt[1][warp] = c1;
+    }
+    team_sync<TEAM>();
+    c0 = c1 = 0;
+#pragma unroll 1
+    for (uint32_t r = 0; r < TEAM; ++r)
+#pragma unroll 1
+      for (int w = 0; w < kRankWarps; ++w) {
+        c0 += peer_load<TEAM>(&sh.wcnt[0][w], r);
+        c1 += peer_load<TEAM>(&sh.wcnt[1][w], r);
+      }
+    auto halve = [](RankRange& g, uint32_t want, uint32_t c) {
+      const uint32_t half = g.span >> 1;
+      if (g.above + c >= want) {
+        g.span = half;
+        g.in = c;
+      } else {
+        g.above += c;
+        g.in -= c;
+        g.lo += half + 1;
+        g.span -= half + 1;
+      }
+    };
+    if (on0) halve(r0, want0, c0);
+    if (on1) halve(r1, want1, c1);
+    team_sync<TEAM>();
+  }
+
+  // ---- candidates of this block
+  for (int r = 0; r < rounds; ++r) {
+    reload(r);
+    uint32_t in = 0;
 #pragma unroll
     for (int j = 0; j < KPT; ++j) {
       const bool v = (vis >> j) & 1u;
-      const uint32_t thr = v ? thr0 : thr1;
-      // (thresholds are below 2^31; a position outside the ranking holds all ones and is neither equal nor smaller)
-      if (key[j] == thr) eq_bits |= 1u << j;
-      if (key[j] < thr && (v ? want0 : want1) > 0) gt_bits |= 1u << j;  // smaller t: larger importance
+      if (key[j] - (v ? r0.lo : r1.lo) <= (v ? r0.span : r1.span)) in |= 1u << j;
     }
-    const uint32_t eq_pack = (uint32_t)__popc(eq_bits & vis) | ((uint32_t)__popc(eq_bits & ~vis) << 16);
-    uint32_t eq_total;
-    const uint32_t eq_before = block_excl_scan(eq_pack, warp_tot, &eq_total);
-    // a threshold-valued key is kept while its rank among the modality's ties (in position order) is below ties[m]
-    const int room0 = ties0 - (tie_run0 + (int)(eq_before & 0xffffu));
-    const int room1 = ties1 - (tie_run1 + (int)(eq_before >> 16));
-    uint32_t keep_bits = kPool ? (gt_bits | forced) : gt_bits;
-    {
-      uint32_t ev = eq_bits & vis, et = eq_bits & ~vis;
-      for (int k = 0; k < room0 && ev && want0 > 0; ++k) {  // lowest positions first
-        keep_bits |= ev & (0u - ev);
-        ev &= ev - 1;
-      }
-      for (int k = 0; k < room1 && et && want1 > 0; ++k) {
-        keep_bits |= et & (0u - et);
-        et &= et - 1;
-      }
+    append<TEAM, 1, KPT>(sh, r0.in <= kListCap ? in & vis : 0u, r1.in <= kListCap ? in & ~vis : 0u, key, r0.lo, r1.lo);
+  }
+  team_sync<TEAM>();
+  // ---- every block gathers the team's candidates and finds the thresholds: the smallest t up to which the wanted number of
+  // keys lies, and how many keys of exactly that t are still wanted
+  const uint32_t got = gather_lists<TEAM, 1>(sh);
+  const bool on0 = want0 && !short0 && r0.in <= kListCap, on1 = want1 && !short1 && r1.in <= kListCap;
+  finish_lists<TEAM, 1, false>(sh, r0, r1, got, on0, on1, want0, want1, 0ull, 0ull, kmax);
+  // (nothing wanted: nothing lies before 0 and no tie is kept; all wanted: everything lies before kNowhere)
+  const uint32_t thr0 = !want0 ? 0u : (short0 ? kNowhere : (on0 ? sh.fin_lo[0] : r0.lo));
+  const uint32_t thr1 = !want1 ? 0u : (short1 ? kNowhere : (on1 ? sh.fin_lo[1] : r1.lo));
+  const uint32_t ties0 = !want0 || short0 ? 0u : want0 - (on0 ? sh.fin_c[0] : r0.above);
+  const uint32_t ties1 = !want1 || short1 ? 0u : want1 - (on1 ? sh.fin_c[1] : r1.above);
+
+  // ---- ordered sweep: positions are consecutive within a thread, threads and blocks follow in position order. A key
+  // before its modality's threshold is kept, one at the threshold while its rank among these ties (in position order) is
+  // below the number still wanted. The counts of (ties v, ties t, kept outright) travel as one 3 x 21-bit word.
+  uint32_t eq, gt;
+  auto classify = [&]() {
+    eq = gt = 0;
+#pragma unroll
+    for (int j = 0; j < KPT; ++j) {
+      const uint32_t thr = (vis >> j) & 1u ? thr0 : thr1;
+      if (key[j] == thr) eq |= 1u << j;
+      if (key[j] < thr) gt |= 1u << j;
     }
-    uint32_t keep_total;
-    const uint32_t slot = block_excl_scan((uint32_t)__popc(keep_bits), warp_tot, &keep_total);
-    int o = out_run + (int)slot;
-    while (keep_bits) {
-      const int j = __ffs(keep_bits) - 1;
-      keep_bits &= keep_bits - 1;
-      p.kept_idx[off0 + o++] = pos0 + j;
+    if (kPool) gt |= forced;
+    return (u64)__popc(eq & vis) | ((u64)__popc(eq & ~vis) << 21) | ((u64)__popc(gt) << 42);
+  };
+  u64 before = 0;  // counts before this block (a block on its own needs no totals before it emits)
+  u64 mine = 0;
+  if (rounds == 1) {
+    mine = classify();
+  } else if (TEAM > 1) {
+    for (int r = 0; r < rounds; ++r) {
+      reload(r);
+      mine += classify();
     }
-    tie_run0 += (int)(eq_total & 0xffffu);
-    tie_run1 += (int)(eq_total >> 16);
-    out_run += (int)keep_total;
+  }
+  u64 incl = warp_scan64(mine);
+  if (lane == 31) sh.wscan_q[warp] = incl;
+  __syncthreads();
+  if (TEAM > 1) {
+    if (warp == 0) {
+      const u64 tot = warp_sum64(lane < kRankWarps ? sh.wscan_q[lane] : 0ull);
+      if (lane < TEAM) peer_store<TEAM>(&sh.slice_q[0][rank], lane, tot);
+    }
+    team_sync<TEAM>();  // (also the last access to a peer's shared memory)
+    before = warp_sum64(lane < (int)rank ? sh.slice_q[0][lane] : 0ull);
+  }
+  if (!kPool) pdl_wait();
+  pdl_go();
+  const int64_t off0 = p.seg_off[u];
+  if (off0 + p.kept_len[u] + p.headroom > p.capacity) return;  // seg_scan has raised MADAKV_ECAPACITY
+  auto emit = [&](int pos0, u64 ahead) {  // ahead: counts before this thread's positions
+    const uint32_t e0 = (uint32_t)ahead & 0x1fffffu, e1 = (uint32_t)(ahead >> 21) & 0x1fffffu, g = (uint32_t)(ahead >> 42);
+    int32_t* out = p.kept_idx + off0 + g + min(e0, ties0) + min(e1, ties1);
+    uint32_t keep = gt;
+    uint32_t ev = eq & vis, et = eq & ~vis;
+    for (uint32_t k = e0; k < ties0 && ev; ++k) {  // lowest positions first
+      keep |= ev & (0u - ev);
+      ev &= ev - 1;
+    }
+    for (uint32_t k = e1; k < ties1 && et; ++k) {
+      keep |= et & (0u - et);
+      et &= et - 1;
+    }
+    while (keep) {
+      const int j = __ffs(keep) - 1;
+      keep &= keep - 1;
+      *out++ = pos0 + j;
+    }
+  };
+  if (rounds == 1) {
+    emit(pos_first, before + incl - mine + warp_sum64(lane < warp ? sh.wscan_q[lane] : 0ull));
+  } else {
+    for (int r = 0; r < rounds; ++r) {
+      reload(r);
+      mine = classify();
+      incl = warp_scan64(mine);
+      __syncthreads();
+      if (lane == 31) sh.wscan_r[warp] = incl;
+      __syncthreads();
+      const u64 ahead = before + incl - mine + warp_sum64(lane < warp ? sh.wscan_r[lane] : 0ull);
+      before += warp_sum64(lane < kRankWarps ? sh.wscan_r[lane] : 0ull);
+      emit(pos_first + r * kRound, ahead);
+    }
+  }
+}
+
+template <bool kPool>
+void launch_select_unit(const madakv_config& c, const SelParams& p, cudaStream_t st) {
+  const RankShape s = rank_shape(p.units, c.max_seq_len);
+  switch (s.kpt + s.team) {
+    case 8 + 1: launch_team(select_unit_kernel<8, 1, kPool>, p.units, 1, st, p); break;
+    case 8 + 2: launch_team(select_unit_kernel<8, 2, kPool>, p.units, 2, st, p); break;
+    case 8 + 4: launch_team(select_unit_kernel<8, 4, kPool>, p.units, 4, st, p); break;
+    case 8 + 8: launch_team(select_unit_kernel<8, 8, kPool>, p.units, 8, st, p); break;
+    case 16 + 1: launch_team(select_unit_kernel<16, 1, kPool>, p.units, 1, st, p); break;
+    case 16 + 2: launch_team(select_unit_kernel<16, 2, kPool>, p.units, 2, st, p); break;
+    case 16 + 4: launch_team(select_unit_kernel<16, 4, kPool>, p.units, 4, st, p); break;
+    default: launch_team(select_unit_kernel<16, 8, kPool>, p.units, 8, st, p); break;
   }
 }
 
@@ -412,19 +489,9 @@ int launch_select(const madakv_config& c, const float* psi, const uint8_t* mask,
   p.keep_window = c.keep_window;
   p.window = c.window;
   p.pool_r = (c.pool_kernel - 1) / 2;
-  seg_scan_kernel<<<1, 1024, 0, st>>>(p);
-  // 16-byte loads of psi need every unit's row (n_max floats apart) to start on a 16-byte boundary
-  const bool wide = c.max_seq_len > CHUNK;  // 10-bit digits when sequences can be longer than one chunk
-  if (c.pool_kernel > 1 || c.keep_window) {
-    if (wide) select_unit_kernel<false, true, 10><<<p.units, NT, 0, st>>>(p);
-    else select_unit_kernel<false, true, 8><<<p.units, NT, 0, st>>>(p);
-  } else if (c.max_seq_len % 4 == 0) {
-    if (wide) select_unit_kernel<true, false, 10><<<p.units, NT, 0, st>>>(p);
-    else select_unit_kernel<true, false, 8><<<p.units, NT, 0, st>>>(p);
-  } else {
-    if (wide) select_unit_kernel<false, false, 10><<<p.units, NT, 0, st>>>(p);
-    else select_unit_kernel<false, false, 8><<<p.units, NT, 0, st>>>(p);
-  }
+  launch_pdl(seg_scan_kernel, dim3(1), dim3(1024), 0, st, p);
+  if (c.pool_kernel > 1 || c.keep_window) launch_select_unit<true>(c, p, st);
+  else launch_select_unit<false>(c, p, st);
   return launch_status();
 }
 
