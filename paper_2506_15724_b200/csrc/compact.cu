@@ -1,15 +1,15 @@
 // Stage 4b: gather the kept K/V rows of every unit into the ragged per-head cache (bit copies).
 //
 // A row is d * elem_bytes = 128..512 bytes = LPR lanes of 16 bytes; a warp moves 32 / LPR rows of K and of V per
-// instruction. Reads are whole 128-byte lines at random rows, writes are contiguous.
+// instruction. Reads are whole 128-byte lines at random rows, writes are contiguous. A thread has U rows of K and of V in
+// flight: all positions are read before the first row, all rows before the first store.
 #include "common.cuh"
 
 namespace madakv {
 namespace {
 
 constexpr int NT = 256;
-constexpr int ROWS_PER_BLOCK = 128;
-constexpr int kMaxBlocksX = 64;  // blocks per unit at most
+constexpr int kMaxBlocksX = 64;  // blocks per unit at most in calls with many units
 
 struct CompactParams {
   const char* k;
@@ -25,34 +25,60 @@ struct CompactParams {
   int L, Hkv, n_max, row_bytes, headroom;
 };
 
-template <int LPR>  // 16-byte lanes per row
+template <int LPR, int U>  // 16-byte lanes per row, rows per thread and iteration
 __global__ void __launch_bounds__(NT) compact_kernel(CompactParams p) {
+  constexpr int RPI = NT / LPR;  // rows the block's threads cover once
+  pdl_wait();
+  pdl_go();
   const int u = blockIdx.y;
   const int len = p.kept_len[u];
-  if ((int)blockIdx.x * ROWS_PER_BLOCK >= len) return;
+  if ((int)blockIdx.x * RPI * U >= len) return;
   const int64_t off = p.seg_off[u];
   // a segment that selection refused (MADAKV_ECAPACITY: it would end beyond the cache) has no index list: skip it
   if (off + len + p.headroom > p.capacity) return;
   const int h = u % p.Hkv, l = (u / p.Hkv) % p.L, b = u / (p.Hkv * p.L);
-  const int64_t src_base = b * p.stride_b + l * p.stride_l + h * p.stride_h;
   const int lane = threadIdx.x % LPR, sub = threadIdx.x / LPR;
-  constexpr int RPI = NT / LPR;  // rows per block iteration
-  // a block takes every gridDim.x-th stretch of ROWS_PER_BLOCK rows (the grid has at most kMaxBlocksX blocks per
-  // unit: with one block per stretch of the longest possible segment nearly all blocks of a long-context call were
-  // launched only to return)
-  for (int row0 = blockIdx.x * ROWS_PER_BLOCK; row0 < len; row0 += gridDim.x * ROWS_PER_BLOCK) {
-  const int row_end = min(len, row0 + ROWS_PER_BLOCK);
-#pragma unroll 2
-  for (int r = row0 + sub; r < row_end; r += RPI) {
-    const int idx = p.kept_idx[off + r];
-    if (idx < 0 || idx >= p.n_max) continue;
-    const int64_t src = src_base + (int64_t)idx * p.stride_t + lane * 16;
-    const int64_t dst = (off + r) * (int64_t)p.row_bytes + lane * 16;
-    const uint4 kv = __ldg(reinterpret_cast<const uint4*>(p.k + src));
-    const uint4 vv = __ldg(reinterpret_cast<const uint4*>(p.v + src));
-    *reinterpret_cast<uint4*>(p.k_c + dst) = kv;
-    *reinterpret_cast<uint4*>(p.v_c + dst) = vv;
+  const int64_t src_base = b * p.stride_b + l * p.stride_l + h * p.stride_h + lane * 16;
+  // a block takes every gridDim.x-th stretch of RPI * U rows
+  for (int row0 = blockIdx.x * RPI * U; row0 < len; row0 += gridDim.x * RPI * U) {
+    int idx[U];
+    uint4 kv[U], vv[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const int r = row0 + j * RPI + sub;
+      idx[j] = r < len ? __ldg(p.kept_idx + off + r) : -1;
+      if (idx[j] >= p.n_max) idx[j] = -1;
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j)
+      if (idx[j] >= 0) {
+        const int64_t src = src_base + (int64_t)idx[j] * p.stride_t;
+        kv[j] = __ldg(reinterpret_cast<const uint4*>(p.k + src));
+        vv[j] = __ldg(reinterpret_cast<const uint4*>(p.v + src));
+      }
+#pragma unroll
+    for (int j = 0; j < U; ++j)
+      if (idx[j] >= 0) {
+        const int64_t dst = (off + row0 + j * RPI + sub) * (int64_t)p.row_bytes + lane * 16;
+        *reinterpret_cast<uint4*>(p.k_c + dst) = kv[j];
+        *reinterpret_cast<uint4*>(p.v_c + dst) = vv[j];
+      }
   }
+}
+
+// Calls with many units are bound by HBM: four rows of K and V per thread keep enough loads on the wire. A call with few
+// units (one layer) is bound by the latency of its blocks: one row per thread and as many blocks as the longest possible
+// segment can use, so that every row's chain of three loads and a store runs once (one layer of 4 heads with 128-row
+// blocks that looped eight times: 13.5 us).
+template <int LPR>
+void launch_rows(const CompactParams& p, int units, cudaStream_t st) {
+  constexpr int RPI = NT / LPR;
+  if (units >= 64) {
+    const int stretches = (p.n_max + RPI * 4 - 1) / (RPI * 4);
+    launch_pdl(compact_kernel<LPR, 4>, dim3(stretches < kMaxBlocksX ? stretches : kMaxBlocksX, units), dim3(NT), 0, st, p);
+  } else {
+    const int stretches = (p.n_max + RPI - 1) / RPI, most = 4096 / units;
+    launch_pdl(compact_kernel<LPR, 1>, dim3(stretches < most ? stretches : most, units), dim3(NT), 0, st, p);
   }
 }
 
@@ -84,12 +110,10 @@ int launch_compact(const madakv_config& c, const void* k, const void* v, madakv_
   p.headroom = c.max_new_tokens;
   const int units = c.batch * c.n_layers * c.n_kv_heads;
   if (units > 65535) return MADAKV_EUNSUPPORTED;
-  const int stretches = (c.max_seq_len + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK;
-  const dim3 grid(stretches < kMaxBlocksX ? stretches : kMaxBlocksX, units);
   switch (p.row_bytes / 16) {
-    case 8: compact_kernel<8><<<grid, NT, 0, st>>>(p); break;
-    case 16: compact_kernel<16><<<grid, NT, 0, st>>>(p); break;
-    case 32: compact_kernel<32><<<grid, NT, 0, st>>>(p); break;
+    case 8: launch_rows<8>(p, units, st); break;
+    case 16: launch_rows<16>(p, units, st); break;
+    case 32: launch_rows<32>(p, units, st); break;
     default: return MADAKV_EUNSUPPORTED;
   }
   return launch_status();
