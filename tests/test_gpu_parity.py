@@ -363,6 +363,42 @@ def test_allocate_and_select_on_crafted_scores(kind, n):
         assert_segments_equal(kept_len, seg_off, buf.kept_idx.cpu().numpy(), kept_idx, "kept_idx")
 
 
+# (units, positions): one block of 8 and of 16 keys per thread, in one round and in several; teams of 2, 4 and 8 blocks with
+# 8 and with 16 keys per thread; rows that start on every 4-byte boundary
+@pytest.mark.parametrize("units,n", [(3, 4096), (150, 4097), (148, 16391), (74, 8190), (74, 9001), (40, 16384), (38, 20003),
+                                     (4, 32768), (6, 33333), (1, 131073)])
+@pytest.mark.parametrize("kind", ["importance", "crowded", "extremes"])
+def test_allocate_and_select_over_blocks_and_lengths(kind, units, n):
+    """Every way the ranking kernels spread a unit's keys, bit-exact against the oracle: importance-like scores, ties and
+    clusters that overflow the candidate list, and scores from denormals to far above 512 (masses that do not fit the
+    bucket sums)."""
+    wl = synth.scaled(TINY, B=1, L=units, Hq=1, Hkv=1, n=n, w=8, budget=n // 7, theta=0.4)
+    rng = np.random.RandomState(units + n)
+    shape = (1, units, 1, n)
+    if kind == "importance":
+        psi = np.exp(rng.normal(-9.0, 1.0, size=shape))
+    elif kind == "crowded":
+        psi = np.where(rng.rand(*shape) < 0.5, 1e-4, rng.choice([1e-4, 1.00001e-4, 3e-5, 0.0, 0.5], size=shape))
+    else:
+        psi = np.exp(rng.uniform(-95.0, 14.0, size=shape)) * (rng.rand(*shape) < 0.8)
+    psi = np.ascontiguousarray(psi, np.float32)
+    mask = (rng.rand(1, n) < 0.7).astype(np.uint8)
+    sl, bud = np.array([n - 3], np.int32), np.array([wl.budget], np.int32)
+    cfg = config_of(wl)
+    buf = mk.EvictionBuffers(cfg, capacity_of(wl))
+    d_psi, d_mask, d_sl, d_bud = (torch.from_numpy(x).cuda() for x in (psi, mask, sl, bud))
+    mk.madakv_allocate(cfg, d_psi, d_mask, d_sl, d_bud, buf.mass, buf.pref, buf.demand, buf.phi, buf.budgets, buf.ws)
+    mk.madakv_select(cfg, d_psi, d_mask, d_sl, buf.budgets, buf.kept_len, buf.seg_off, buf.kept_idx, buf.ws)
+    assert mk.madakv_poll_status(buf.ws) == 0
+    al = oracle.allocate(psi, mask, sl, bud, float(np.float32(wl.theta)))
+    for key in ("mass", "pref", "demand", "phi", "budgets"):
+        assert np.array_equal(getattr(buf, key).cpu().numpy(), al[key]), key
+    rc, kept_len, seg_off, kept_idx = oracle.select(psi, mask, sl, al["budgets"], headroom=wl.max_new_tokens,
+                                                    capacity=capacity_of(wl))
+    assert rc == 0 and np.array_equal(buf.kept_len.cpu().numpy(), kept_len)
+    assert_segments_equal(kept_len, seg_off, buf.kept_idx.cpu().numpy(), kept_idx, "kept_idx")
+
+
 @pytest.mark.parametrize("name", ["tiny_gqa_ragged", "bf16_d128", "bf16_gqa7", "tc_short_seqs"])
 @pytest.mark.parametrize("hcc", [mk.HCC_PAPER, mk.HCC_LITERAL, mk.HCC_DEMAND])
 @pytest.mark.parametrize("split", [False, True])
