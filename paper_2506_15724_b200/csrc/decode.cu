@@ -1,14 +1,15 @@
-// Stage 5: cache append (Eq. 4) and decode attention over the ragged per-head cache (Eq. 5).
+// Stage 5: cache append (Eq. 4) and decode attention over the ragged per-head cache (Eq. 5), one launch per call.
 //
-//   append   (Eq. 4) has no kernel of its own: the partial block whose share holds the new row copies it from
-//            k_new / v_new behind the segment and attends over it; the merge kernel bumps kept_len
-//   partial  up to 8, 16 or 32 blocks per segment (blocks_per_segment), each taking an equal share of the segment's rows (the share is a
-//            function of the segment's length alone: short segments use fewer blocks, never fewer than kDecodeMinRows
-//            rows each): a group of LPR lanes owns a cache row (16 bytes per lane), the g query heads of the KV group
-//            share every K/V row read; online softmax in the log2 domain, fp32 accumulation; the block's row groups
-//            are merged in shared memory. For bf16 caches with 3 <= g <= 16 the same share is computed by
-//            decode_partial_mma_kernel on the tensor cores instead.
-//   merge    one block per query head: fixed-order combination of the blocks' partials, rounding to dtype once
+//   append   (Eq. 4) has no kernel of its own: the block whose share holds the new row copies it from k_new / v_new
+//            behind the segment and attends over it; the block that merges the segment bumps kept_len
+//   attend   a segment's rows are shared out over up to `slots` blocks (decode_shape). Scalar kernel: a group of LPR lanes owns
+//            a cache row (16 bytes per lane), the g query heads of the KV group share every K/V row read; online
+//            softmax in the log2 domain, fp32 accumulation; the block's row groups are merged in shared memory. For bf16
+//            caches with 3 <= g <= 16 the same share is computed by decode_mma_kernel on the tensor cores instead.
+//   merge    the block that arrives last at the segment's counter combines the blocks' results in block order and rounds
+//            to dtype once. (A second kernel for it cost a launch on the host, 2.2 us, and 3-9 us on the GPU per call; a
+//            thread-block cluster per segment that merges through distributed shared memory left too few blocks
+//            resident: 248 us instead of 148 on 1024 segments of 1638 rows.)
 #include <mutex>
 
 #include "common.cuh"
@@ -17,9 +18,8 @@ namespace madakv {
 namespace {
 
 constexpr int NT = 128;
-constexpr int kDecodeSlots = 32;    // blocks (and partials) per segment at most
-constexpr int kDecodeMinRows = 512; // a block's share of a segment is at least this many rows: shorter shares leave
-                                    // the block's load pipeline no time to fill (measured: 256 rows cost 5-8 %)
+constexpr int kDecodeSlots = 32;    // blocks per segment at most
+
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
@@ -34,10 +34,11 @@ struct DecodeParams {
   int64_t capacity;
   void* out;
   float* lse_out;
-  float* part;  // ws: [B*L*Hq, slots, D + 2]
-  int32_t* eff_len;  // ws: [units] rows each segment's attention covered (appending calls; else null)
+  float* part;        // slots > 1: [B*L*Hq, slots, D] partial outputs, then [B*L*Hq, slots, 2] their (max, sum)
+  float2* part_ml;
+  unsigned* counter;  // slots > 1: one per segment of the call, zero between calls
   void* ws;
-  int L, Hq, Hkv, g, layer, slots, n_sel, min_rows, slot_fast;
+  int L, Hq, Hkv, g, layer, slots, n_sel, min_rows;
   float scale2;
 };
 
@@ -72,8 +73,7 @@ __device__ __forceinline__ int segment_rows(const DecodeParams& p, int u) {
 __device__ __forceinline__ int segment_blocks(const DecodeParams& p, int len) {
   return max(1, min(p.slots, (len + p.min_rows - 1) / p.min_rows));
 }
-__device__ __forceinline__ void block_rows(const DecodeParams& p, int len, int x, int& row_begin, int& row_end) {
-  const int nb = segment_blocks(p, len);
+__device__ __forceinline__ void block_rows(int nb, int len, int x, int& row_begin, int& row_end) {
   const int share = ((len + nb - 1) / nb + 15) / 16 * 16;
   row_begin = min(len, x * share);
   row_end = min(len, row_begin + share);
@@ -81,9 +81,8 @@ __device__ __forceinline__ void block_rows(const DecodeParams& p, int len, int x
 
 // What a block of unit u works on. When the call appends (Eq. 4), the new row is part of the attention: the one block
 // whose share holds it copies it from k_new / v_new into the cache and reads it from there, all others see the old
-// rows only. kept_len itself is bumped by the merge kernel, after every block of both kernels has read the old value
-// (merge blocks read the length the partial kernel recorded in the workspace instead). A segment without room for the
-// row (or one that selection refused) is left as it is and MADAKV_ECAPACITY is recorded.
+// rows only. kept_len itself is bumped by the block that merges, after every block of the segment has read the old value.
+// A segment without room for the row (or one that selection refused) is left as it is and MADAKV_ECAPACITY is recorded.
 struct SegView {
   int len;      // rows attention covers, the appended one included
   int new_row;  // its index in the segment, or -1
@@ -143,140 +142,333 @@ struct Vec16<__nv_bfloat16> {
   }
 };
 
-template <typename T, int D, int G>
-__global__ void __launch_bounds__(NT) decode_partial_kernel(DecodeParams p) {
-  constexpr int EPL = Vec16<T>::N;          // elements per lane
-  constexpr int LPR = D / EPL;              // lanes per row
-  constexpr int GROUPS = NT / LPR;          // rows in flight per block
-  constexpr int ROW_BYTES = D * (int)sizeof(T);
-  __shared__ float s_o[GROUPS][G][D];
-  __shared__ float s_m[GROUPS][G], s_l[GROUPS][G];
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// The weight of a partial with maximum m against the overall maximum M.
+__device__ __forceinline__ float part_weight(float m, float M) { return m == -INFINITY ? 0.f : exp2f(m - M); }
 
-  pdl_wait();
-  pdl_go();
-  const int y = p.slot_fast ? blockIdx.x / p.slots : blockIdx.x % p.n_sel;
-  const int u = unit_of(p, y);
-  const int slot = p.slot_fast ? blockIdx.x % p.slots : blockIdx.x / p.n_sel;
-  const SegView view = segment_view(p, u, slot == 0 && threadIdx.x == 0);
-  const int len = view.len;
-  if (slot == 0 && threadIdx.x == 0 && p.eff_len) p.eff_len[u] = len;
-  if (slot >= segment_blocks(p, len)) return;
-  int row_begin, row_end;
-  block_rows(p, len, slot, row_begin, row_end);
-  const int64_t off = p.seg_off[u];
-  store_new_row<ROW_BYTES>(p, u, off, view, row_begin, row_end);
-  const int h = u % p.Hkv, bl = u / p.Hkv;
-  const int lane = threadIdx.x % LPR, grp = threadIdx.x / LPR;
+// Four results of one query head: `o` unnormalised, l their sum of weights.
+template <typename T, int D>
+__device__ __forceinline__ void store4(const DecodeParams& p, int64_t row, int c, float4 o, float l) {
+  const float r0 = l > 0.f ? o.x / l : 0.f, r1 = l > 0.f ? o.y / l : 0.f, r2 = l > 0.f ? o.z / l : 0.f, r3 = l > 0.f ? o.w / l : 0.f;
+  if constexpr (sizeof(T) == 4) {
+    *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + row * D + c) = make_float4(r0, r1, r2, r3);
+  } else {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(r0, r1), b = __floats2bfloat162_rn(r2, r3);
+    *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + row * D + c) =
+        make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+  }
+}
+__device__ __forceinline__ void store_lse(const DecodeParams& p, int64_t row, float M, float l) {
+  if (p.lse_out) p.lse_out[row] = l > 0.f ? (M + log2f(l)) * kLn2 : -INFINITY;
+}
 
-  float qr[G][EPL];
+// The end of a block: its results lie in shared memory (bo [g][D] unnormalised, bm and bl [g], complete behind a barrier of
+// the block); they are combined with those of the segment's other blocks, in block order. fac: kDecodeSlots * g floats of
+// shared memory. `nb` blocks of the segment have results; the others arrive at the counter all the same, so that the last
+// one knows that all have read the segment's length.
+template <typename T, int D, int NTHR>
+__device__ __forceinline__ void finish_segment(const DecodeParams& p, const float* bo, const float* bm, const float* bl, float* fac,
+                                               int u, int y, int slot, int nb, SegView view) {
+  constexpr int C4 = D / 4;
+  const int h = u % p.Hkv, blr = u / p.Hkv;
+  const int64_t row0 = (int64_t)blr * p.Hq + h * p.g;
+  if (p.slots == 1) {
+    for (int x = threadIdx.x; x < p.g * C4; x += NTHR) {
+      const int i = x / C4, c = x % C4 * 4;
+      store4<T, D>(p, row0 + i, c, *reinterpret_cast<const float4*>(bo + i * D + c), bl[i]);
+      if (c == 0) store_lse(p, row0 + i, bm[i], bl[i]);
+    }
+    if (threadIdx.x == 0 && view.new_row >= 0) p.kept_len[u] = view.len;
+    return;
+  }
+  if (slot < nb) {
+    for (int x = threadIdx.x; x < p.g * C4; x += NTHR) {
+      const int i = x / C4, c = x % C4 * 4;
+      __stcg(reinterpret_cast<float4*>(p.part + ((row0 + i) * p.slots + slot) * D + c),
+             *reinterpret_cast<const float4*>(bo + i * D + c));
+    }
+    if ((int)threadIdx.x < p.g) __stcg(p.part_ml + (row0 + threadIdx.x) * p.slots + slot, make_float2(bm[threadIdx.x], bl[threadIdx.x]));
+  }
+  __shared__ unsigned s_last;
+  __syncthreads();
+  if (threadIdx.x == 0) {  // (one thread's fences order what the whole block wrote before the barrier, and will read)
+    __threadfence();
+    s_last = atomicInc(p.counter + y, (unsigned)p.slots - 1u);  // (wraps to 0: ready for the next call)
+    __threadfence();
+  }
+  __syncthreads();
+  if (s_last != (unsigned)p.slots - 1u) return;
+  if (threadIdx.x == 0 && view.new_row >= 0) p.kept_len[u] = view.len;
+  // weights of the partials, and every head's maximum and sum
+  __shared__ float s_l[16];
+  for (int i = threadIdx.x / 32; i < p.g; i += NTHR / 32) {
+    const int s = threadIdx.x % 32;
+    const float2 v = s < nb ? __ldcg(p.part_ml + (row0 + i) * p.slots + s) : make_float2(-INFINITY, 0.f);
+    const float m = v.x;
+    float M = m;
 #pragma unroll
-  for (int i = 0; i < G; ++i) {
-    if (i < p.g) {
-      const T* qp = reinterpret_cast<const T*>(p.q) + ((int64_t)bl * p.Hq + h * p.g + i) * D + lane * EPL;
-      Vec16<T>::load(qp, qr[i]);
-    } else {
+    for (int off = 16; off >= 1; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
+    const float f = part_weight(m, M);
+    float l = v.y * f;
+    if (s < nb) fac[i * kDecodeSlots + s] = f;
 #pragma unroll
-      for (int c = 0; c < EPL; ++c) qr[i][c] = 0.f;
+    for (int off = 16; off >= 1; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+    if (s == 0) {
+      s_l[i] = l;
+      store_lse(p, row0 + i, M, l);
     }
   }
-  float m[G], l[G], o[G][EPL];
+  __syncthreads();
+  for (int x = threadIdx.x; x < p.g * C4; x += NTHR) {
+    const int i = x / C4, c = x % C4 * 4;
+    const float4* src = reinterpret_cast<const float4*>(p.part + (row0 + i) * p.slots * D + c);
+    float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < nb; s0 += 8) {
+      float4 v[8];
 #pragma unroll
-  for (int i = 0; i < G; ++i) {
-    m[i] = -INFINITY;
-    l[i] = 0.f;
+      for (int s = 0; s < 8; ++s) v[s] = s0 + s < nb ? __ldcg(src + (s0 + s) * C4) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int c = 0; c < EPL; ++c) o[i][c] = 0.f;
-  }
-  const char* kc = (const char*)p.k_c + off * ROW_BYTES + lane * 16;
-  const char* vc = (const char*)p.v_c + off * ROW_BYTES + lane * 16;
-  // the appended row is read from where it comes from, not from the cache row this block is writing
-  const char* kn = view.new_row >= 0 ? (const char*)p.k_new + (int64_t)u * ROW_BYTES + lane * 16 : nullptr;
-  const char* vn = view.new_row >= 0 ? (const char*)p.v_new + (int64_t)u * ROW_BYTES + lane * 16 : nullptr;
-  // U rows per thread are in flight at a time: all their 16-byte K and V loads are issued before the first use, so a
-  // block keeps GROUPS * U * 2 * ROW_BYTES bytes on the wire (the online-softmax chain below is short next to the
-  // memory latency). Uniform trip count: the shuffles need full warps.
-  constexpr int U = G <= 2 ? 4 : 2;
-  for (int r0 = row_begin; r0 < row_end; r0 += GROUPS * U) {
-    uint4 kraw[U], vraw[U];
-#pragma unroll
-    for (int j = 0; j < U; ++j) {
-      const int r = r0 + grp + GROUPS * j;
-      kraw[j] = vraw[j] = make_uint4(0u, 0u, 0u, 0u);
-      if (r < row_end) {
-        const bool fresh = r == view.new_row;
-        kraw[j] = __ldcs(reinterpret_cast<const uint4*>(fresh ? kn : kc + (int64_t)r * ROW_BYTES));
-        vraw[j] = __ldcs(reinterpret_cast<const uint4*>(fresh ? vn : vc + (int64_t)r * ROW_BYTES));
+      for (int s = 0; s < 8; ++s) {
+        const float f = s0 + s < nb ? fac[i * kDecodeSlots + s0 + s] : 0.f;
+        O.x += v[s].x * f;
+        O.y += v[s].y * f;
+        O.z += v[s].z * f;
+        O.w += v[s].w * f;
       }
     }
+    store4<T, D>(p, row0 + i, c, O, s_l[i]);
+  }
+}
+
+// ---- scalar kernel (fp32, or bf16 with g <= 2) -------------------------------------------------------------------------
+// HBM-bound. The rows of a share lie one behind the other in the cache, so one thread streams them into a ring of
+// shared-memory stages with bulk copies (8 KB of K and 8 KB of V each) that count their bytes on the stage's barrier, and
+// four warps work on whole stages: 32 KB are on the wire per block whatever the compiler does with the loop (with 16-byte
+// loads to registers the kernel took 139 or 241 us on 1024 segments of 1638 rows depending on the code around them; this
+// one takes 135, merge included: 0.98 of the measured copy bandwidth. 12 segments of 53038 rows: 118 -> 72 us).
+constexpr int kRingStages = 2;      // a small ring keeps seven blocks resident per SM, so that a block's start and end are
+                                    // covered by the others (four stages: 163 us instead of 135)
+constexpr int kStageBytes = 16384;  // K, then V
+constexpr long long kCopyWait = 4000000000ll;  // ~2 s: bound of a wait for a copy
+
+__device__ __forceinline__ void bar_init(uint64_t* bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count));
+}
+__device__ __forceinline__ void bar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void bar_expect(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool bar_try(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+      : "=r"(ok)
+      : "r"(smem_addr(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// Bounded wait; a wait that runs out is reported (where there is a workspace) and the caller goes on with what is there.
+__device__ __forceinline__ void bar_wait(const DecodeParams& p, uint64_t* bar, uint32_t parity) {
+  if (bar_try(bar, parity)) return;
+  const long long t0 = clock64();
+  while (!bar_try(bar, parity))
+    if (clock64() - t0 > kCopyWait) {
+      if (p.ws) set_status(p.ws, MADAKV_ETIMEOUT);
+      return;
+    }
+}
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(smem_addr(bar))
+               : "memory");
+}
+
+template <typename T, int D, int G>
+__global__ void __launch_bounds__(NT) decode_kernel(const __grid_constant__ DecodeParams p) {
+  constexpr int EPL = Vec16<T>::N;          // elements per lane
+  constexpr int LPR = D / EPL;              // lanes per row
+  constexpr int GROUPS = NT / LPR;          // rows the block reads per instruction
+  constexpr int U = 4;                      // rows per thread and stage
+  constexpr int ROW_BYTES = D * (int)sizeof(T);
+  constexpr int ROWS = GROUPS * U;          // rows per stage
+  static_assert(2 * ROWS * ROW_BYTES == kStageBytes, "stage size");
+  static_assert(GROUPS * G * (D + 2) * 4 + G * (D + 2) * 4 <= kRingStages * kStageBytes, "the merge reuses the ring");
+  extern __shared__ __align__(128) unsigned char dsmem[];
+  __shared__ uint64_t full[kRingStages], empty[kRingStages];
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kRingStages; ++i) {
+      bar_init(&full[i], 1);
+      bar_init(&empty[i], NT / 32);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  pdl_wait();
+  pdl_go();
+  const int y = blockIdx.x / p.slots, slot = blockIdx.x % p.slots;
+  const int u = unit_of(p, y);
+  const SegView view = segment_view(p, u, slot == 0 && threadIdx.x == 0);
+  const int len = view.len, nb = segment_blocks(p, len);
+  int row_begin, row_end;
+  block_rows(nb, len, slot, row_begin, row_end);  // (empty beyond the nb-th block)
+  const int h = u % p.Hkv, bl = u / p.Hkv;
+  const int lane = threadIdx.x % LPR, grp = threadIdx.x / LPR;
+  __syncthreads();
+
+  float* s_o = reinterpret_cast<float*>(dsmem);  // [GROUPS][G][D], once the ring is done with
+  float* s_m = s_o + GROUPS * G * D;             // [GROUPS][G]
+  float* s_l = s_m + GROUPS * G;
+  float* b_o = s_l + GROUPS * G;                 // the block's result: [G][D], [G], [G]
+  float* b_m = b_o + G * D;
+  float* b_l = b_m + G;
+  static_assert((GROUPS * G * (D + 2)) % 4 == 0, "b_o is read in 16-byte pieces");
+  if (slot < nb) {
+    const int64_t off = p.seg_off[u];
+    store_new_row<ROW_BYTES>(p, u, off, view, row_begin, row_end);
+    const int steps = (row_end - row_begin + ROWS - 1) / ROWS;
+    // one thread: the rows of a step into their stage. The appended row, always the last one of the segment, is read from
+    // where it comes from, not from the cache row this block is writing.
+    auto issue = [&](int it) {
+      const int r = row_begin + it * ROWS, rows = min(ROWS, row_end - r), st = it % kRingStages;
+      const bool fresh = view.new_row >= r && view.new_row < r + rows;
+      const uint32_t bytes = (uint32_t)(rows - (fresh ? 1 : 0)) * ROW_BYTES;
+      const uint32_t kd = smem_addr(dsmem) + st * kStageBytes, vd = kd + kStageBytes / 2;
+      bar_expect(&full[st], (uint32_t)(2 * rows * ROW_BYTES));
+      if (bytes) {
+        bulk_load(kd, (const char*)p.k_c + (off + r) * ROW_BYTES, bytes, &full[st]);
+        bulk_load(vd, (const char*)p.v_c + (off + r) * ROW_BYTES, bytes, &full[st]);
+      }
+      if (fresh) {
+        bulk_load(kd + bytes, (const char*)p.k_new + (int64_t)u * ROW_BYTES, ROW_BYTES, &full[st]);
+        bulk_load(vd + bytes, (const char*)p.v_new + (int64_t)u * ROW_BYTES, ROW_BYTES, &full[st]);
+      }
+    };
+    if (threadIdx.x == 0)
+      for (int it = 0; it < min(kRingStages, steps); ++it) issue(it);
+
+    float qr[G][EPL];
 #pragma unroll
-    for (int j = 0; j < U; ++j) {
-      const bool valid = r0 + grp + GROUPS * j < row_end;
-      float kf[EPL], vf[EPL];
-      Vec16<T>::cvt(kraw[j], kf);
-      Vec16<T>::cvt(vraw[j], vf);
-      // all heads of the group at once (heads beyond g have zero queries): the dot products, then the lane
-      // reductions of all heads interleaved, then the softmax updates, so that independent chains overlap
-      float sc[G];
+    for (int i = 0; i < G; ++i) {
+      if (i < p.g) {
+        const T* qp = reinterpret_cast<const T*>(p.q) + ((int64_t)bl * p.Hq + h * p.g + i) * D + lane * EPL;
+        Vec16<T>::load(qp, qr[i]);
 #pragma unroll
-      for (int i = 0; i < G; ++i) {
-        float s = 0.f;
+        for (int c = 0; c < EPL; ++c) qr[i][c] *= p.scale2;
+      } else {
 #pragma unroll
-        for (int c = 0; c < EPL; ++c) s = fmaf(qr[i][c], kf[c], s);
-        sc[i] = s;
+        for (int c = 0; c < EPL; ++c) qr[i][c] = 0.f;
+      }
+    }
+    float m[G], l[G], o[G][EPL];
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+      m[i] = -INFINITY;
+      l[i] = 0.f;
+#pragma unroll
+      for (int c = 0; c < EPL; ++c) o[i][c] = 0.f;
+    }
+    for (int it = 0; it < steps; ++it) {
+      const int st = it % kRingStages;
+      const uint32_t use = (uint32_t)(it / kRingStages) & 1u;
+      bar_wait(p, &full[st], use);
+      const uint4* ks = reinterpret_cast<const uint4*>(dsmem + st * kStageBytes) + grp * LPR + lane;
+      const uint4* vs = ks + kStageBytes / 32;
+      const int left = row_end - row_begin - it * ROWS - grp;  // row j of this thread exists while GROUPS * j < left
+      // scores of the U rows for all heads (heads beyond g have zero queries), then one softmax step for the U rows
+      float sc[G][U];
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        float kf[EPL];
+        Vec16<T>::cvt(ks[GROUPS * LPR * j], kf);
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+          float x = 0.f;
+#pragma unroll
+          for (int c = 0; c < EPL; ++c) x = fmaf(qr[i][c], kf[c], x);
+          sc[i][j] = x;
+        }
       }
 #pragma unroll
       for (int sh = LPR / 2; sh >= 1; sh >>= 1) {
 #pragma unroll
-        for (int i = 0; i < G; ++i) sc[i] += __shfl_xor_sync(0xffffffffu, sc[i], sh);
+        for (int i = 0; i < G; ++i)
+#pragma unroll
+          for (int j = 0; j < U; ++j) sc[i][j] += __shfl_xor_sync(0xffffffffu, sc[i][j], sh);
       }
-      if (valid) {
 #pragma unroll
-        for (int i = 0; i < G; ++i) {
-          const float s = sc[i] * p.scale2;
-          if (s > m[i]) {
-            const float f = fast_ex2(m[i] - s);  // exp2(-inf) = 0 on the first row
-            l[i] *= f;
+      for (int i = 0; i < G; ++i) {
+        float mn = m[i];
 #pragma unroll
-            for (int c = 0; c < EPL; ++c) o[i][c] *= f;
-            m[i] = s;
-          }
-          const float pw = fast_ex2(s - m[i]);
-          l[i] += pw;
+        for (int j = 0; j < U; ++j) {
+          if (GROUPS * j >= left) sc[i][j] = -INFINITY;
+          mn = fmaxf(mn, sc[i][j]);
+        }
+        const float base = mn == -INFINITY ? 0.f : mn;  // (no row yet: all weights exp2(-inf) = 0)
+        const float f = fast_ex2(m[i] - base);
+        l[i] *= f;
 #pragma unroll
-          for (int c = 0; c < EPL; ++c) o[i][c] = fmaf(pw, vf[c], o[i][c]);
+        for (int c = 0; c < EPL; ++c) o[i][c] *= f;
+        m[i] = mn;
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+          sc[i][j] = fast_ex2(sc[i][j] - base);
+          l[i] += sc[i][j];
         }
       }
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        // (what a stage holds beyond the share's last row is undefined: not to be multiplied, not even by 0)
+        const uint4 raw = vs[GROUPS * LPR * j];
+        float vf[EPL];
+        Vec16<T>::cvt(GROUPS * j < left ? raw : make_uint4(0u, 0u, 0u, 0u), vf);
+#pragma unroll
+        for (int i = 0; i < G; ++i)
+#pragma unroll
+          for (int c = 0; c < EPL; ++c) o[i][c] = fmaf(sc[i][j], vf[c], o[i][c]);
+      }
+      __syncwarp();
+      if (threadIdx.x % 32 == 0) bar_arrive(&empty[st]);
+      if (threadIdx.x == 0 && it + kRingStages < steps) {  // refill the stage once all warps are done with it
+        bar_wait(p, &empty[st], use);
+        issue(it + kRingStages);
+      }
     }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+      if (lane == 0) {
+        s_m[grp * G + i] = m[i];
+        s_l[grp * G + i] = l[i];
+      }
+#pragma unroll
+      for (int c = 0; c < EPL; c += 4)
+        *reinterpret_cast<float4*>(s_o + (grp * G + i) * D + lane * EPL + c) =
+            make_float4(o[i][c], o[i][c + 1], o[i][c + 2], o[i][c + 3]);
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < p.g * D; x += NT) {
+      const int i = x / D, c = x % D;
+      float M = -INFINITY;
+#pragma unroll
+      for (int gq = 0; gq < GROUPS; ++gq) M = fmaxf(M, s_m[gq * G + i]);
+      float Lsum = 0.f, O = 0.f;
+#pragma unroll
+      for (int gq = 0; gq < GROUPS; ++gq) {
+        const float f = part_weight(s_m[gq * G + i], M);
+        Lsum += s_l[gq * G + i] * f;
+        O += s_o[(gq * G + i) * D + c] * f;
+      }
+      b_o[i * D + c] = O;
+      if (c == 0) {
+        b_m[i] = M;
+        b_l[i] = Lsum;
+      }
+    }
+    __syncthreads();
   }
-#pragma unroll
-  for (int i = 0; i < G; ++i) {
-    if (lane == 0) {
-      s_m[grp][i] = m[i];
-      s_l[grp][i] = l[i];
-    }
-#pragma unroll
-    for (int c = 0; c < EPL; ++c) s_o[grp][i][lane * EPL + c] = o[i][c];
-  }
-  __syncthreads();
-  for (int x = threadIdx.x; x < p.g * D; x += NT) {
-    const int i = x / D, c = x % D;
-    float M = -INFINITY;
-#pragma unroll
-    for (int gq = 0; gq < GROUPS; ++gq) M = fmaxf(M, s_m[gq][i]);
-    float Lsum = 0.f, O = 0.f;
-#pragma unroll
-    for (int gq = 0; gq < GROUPS; ++gq) {
-      const float f = (s_m[gq][i] == -INFINITY) ? 0.f : exp2f(s_m[gq][i] - M);
-      Lsum += s_l[gq][i] * f;
-      O += s_o[gq][i][c] * f;
-    }
-    float* dst = p.part + (((int64_t)bl * p.Hq + h * p.g + i) * p.slots + slot) * (D + 2);
-    dst[c] = O;
-    if (c == 0) {
-      dst[D] = M;
-      dst[D + 1] = Lsum;
-    }
-  }
+  finish_segment<T, D, NT>(p, b_o, b_m, b_l, s_o, u, y, slot, nb, view);
 }
 
 // ---- grouped-query partial on the warp-level tensor-core path (bf16, 3 <= g <= 16) ----------------------------------
@@ -289,7 +481,6 @@ __global__ void __launch_bounds__(NT) decode_partial_kernel(DecodeParams p) {
 // 16-row chunks of the split and are merged in shared memory at its end.
 constexpr int kMmaWarps = 4;
 
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
   const int bytes = valid ? 16 : 0;  // zero bytes read: the 16 destination bytes are filled with zeros
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
@@ -331,11 +522,14 @@ struct MmaTile {
   static constexpr int WARP = 4 * TILE;               // two buffers of (K, V)
   static constexpr int OPITCH = D + 8;                // floats from one head's merged row to the next
   static constexpr int BYTES = kMmaWarps * WARP;
-  static_assert(16 * OPITCH * 4 + 2 * 16 * 4 <= WARP, "the merge staging reuses a warp's K/V buffers");
+  static constexpr int BLOCK_OFF = 16 * OPITCH * 4 + 2 * 16 * 4;  // the block's result in warp 0's area: o [16][D], m [16], l [16]
+  static_assert(BLOCK_OFF % 16 == 0 && BLOCK_OFF + 16 * D * 4 + 2 * 16 * 4 <= WARP,
+                "the merge staging reuses a warp's K/V buffers");
+  static_assert(16 * kDecodeSlots * 4 <= 16 * OPITCH * 4, "the weights of a split call's partials take warp 0's place");
 };
 
 template <int D>
-__global__ void __launch_bounds__(kMmaWarps * 32, 3) decode_partial_mma_kernel(DecodeParams p) {
+__global__ void __launch_bounds__(kMmaWarps * 32, 3) decode_mma_kernel(const __grid_constant__ DecodeParams p) {
   using MT = MmaTile<D>;
   constexpr int ROW_BYTES = D * 2;
   constexpr int LPR = ROW_BYTES / 16;  // 16-byte pieces per row
@@ -345,14 +539,14 @@ __global__ void __launch_bounds__(kMmaWarps * 32, 3) decode_partial_mma_kernel(D
 
   pdl_wait();
   pdl_go();
-  const int u = unit_of(p, p.slot_fast ? blockIdx.x / p.slots : blockIdx.x % p.n_sel);
-  const int slot = p.slot_fast ? blockIdx.x % p.slots : blockIdx.x / p.n_sel;
+  const int y = blockIdx.x / p.slots, slot = blockIdx.x % p.slots;
+  const int u = unit_of(p, y);
   const SegView view = segment_view(p, u, slot == 0 && threadIdx.x == 0);
-  const int len = view.len;
-  if (slot == 0 && threadIdx.x == 0 && p.eff_len) p.eff_len[u] = len;
-  if (slot >= segment_blocks(p, len)) return;
+  const int len = view.len, nb = segment_blocks(p, len);
   int row_begin, row_end;
-  block_rows(p, len, slot, row_begin, row_end);
+  block_rows(nb, len, slot, row_begin, row_end);  // (empty beyond the nb-th block)
+  float* bo = reinterpret_cast<float*>(dsmem + MT::BLOCK_OFF);
+  if (slot < nb) {
   const int64_t off = p.seg_off[u];
   store_new_row<D * 2>(p, u, off, view, row_begin, row_end);
   const int h = u % p.Hkv, bl = u / p.Hkv;
@@ -499,110 +693,81 @@ __global__ void __launch_bounds__(kMmaWarps * 32, 3) decode_partial_mma_kernel(D
 #pragma unroll
       for (int w = 0; w < kMmaWarps; ++w) {
         const float* wo = reinterpret_cast<const float*>(dsmem + w * MT::WARP);
-        const float fw = (mw[w] == -INFINITY) ? 0.f : exp2f(mw[w] - M);
+        const float fw = part_weight(mw[w], M);
         Lsum += wo[16 * MT::OPITCH + 16 + i] * fw;
         O += wo[i * MT::OPITCH + c] * fw;
       }
-      float* dst = p.part + (((int64_t)bl * p.Hq + h * p.g + i) * p.slots + slot) * (D + 2);
-      dst[c] = O;
+      bo[x] = O;
       if (c == 0) {
-        dst[D] = M;
-        dst[D + 1] = Lsum;
+        bo[16 * D + i] = M;
+        bo[16 * D + 16 + i] = Lsum;
       }
     }
   }
+  __syncthreads();
+  }
+  finish_segment<__nv_bfloat16, D, kMmaWarps * 32>(p, bo, bo + 16 * D, bo + 16 * D + 16, reinterpret_cast<float*>(dsmem), u, y,
+                                                          slot, nb, view);
 }
 
-template <typename T, int D>
-__global__ void __launch_bounds__(D) decode_merge_kernel(DecodeParams p) {
-  // blockIdx.x enumerates the query heads of the selected layer(s)
-  pdl_wait();
-  pdl_go();
-  int row;
-  if (p.layer < 0) {
-    row = blockIdx.x;
+// Blocks per segment and the rows a block takes at least. The segments' lengths are device data; the rows of the cache per
+// segment stand in for them, so that short segments do not launch blocks only to arrive at the counter.
+//   fewer than 64 segments (one layer of a model): bound by the latency of the blocks, so shares of at least 128 rows
+//     (tensor-core kernel: 256, four iterations of its warps), as many blocks as are resident at once, at most 32 (16
+//     segments of 8725 rows, g = 4: 46 us with 16 blocks each, 56 with 32, which no longer fit; 12 of 53038, g = 1: 72
+//     with 32, 111 with 16)
+//   more: shares of 1024 rows where that gives two full waves of blocks, else 512 (896 segments of 2512 rows, g = 7:
+//     190 us at 1024, 197 at 512, 247 at 256; 10240 of 410, g = 1: 311 with one block each, 335 with two; 1024 of 1638,
+//     g = 1: 137 at 1024, 135 at 512; 112 of 3000, g = 1: 44 at 1024, 38 at 512)
+//   more than there are counters: one block each
+struct DecodeShape {
+  int slots, min_rows;
+};
+DecodeShape decode_shape(const madakv_config& c, int n_sel, int64_t capacity, bool tensor_core_kernel, int splits) {
+  if (n_sel > kDecodeCounters) return {1, 1};
+  const int64_t units = (int64_t)c.batch * c.n_layers * c.n_kv_heads, longest = c.max_seq_len + c.max_new_tokens;
+  const int64_t rows = capacity / units < longest ? capacity / units : longest;
+  const int resident = 148 * (tensor_core_kernel ? 3 : 7);
+  int share, most;
+  if (n_sel < 64) {
+    share = tensor_core_kernel ? 256 : 128;
+    most = resident / n_sel < kDecodeSlots ? resident / n_sel : kDecodeSlots;
   } else {
-    const int b = blockIdx.x / p.Hq, hq = blockIdx.x % p.Hq;
-    row = (b * p.L + p.layer) * p.Hq + hq;
+    share = n_sel * (rows / 1024 + 1) >= 2 * resident ? 1024 : 512;
+    most = 8;
   }
-  const int bl = row / p.Hq, hq = row % p.Hq;
-  const int u = bl * p.Hkv + hq / p.g;
-  // an appending call: the length the partial kernel worked with; the first head of the group makes it the segment's
-  const int len = p.eff_len ? p.eff_len[u] : segment_rows(p, u);
-  if (p.eff_len && hq % p.g == 0 && threadIdx.x == 0 && len > p.kept_len[u]) p.kept_len[u] = len;
-  const int used = segment_blocks(p, len);
-  const float* part = p.part + (int64_t)row * p.slots * (D + 2);
-  const int c = threadIdx.x;
-  float M = -INFINITY;
-  for (int s = 0; s < used; ++s) M = fmaxf(M, part[s * (D + 2) + D]);
-  float Lsum = 0.f, O = 0.f;
-  for (int s = 0; s < used; ++s) {
-    const float ms = part[s * (D + 2) + D];
-    const float f = (ms == -INFINITY) ? 0.f : exp2f(ms - M);
-    Lsum += part[s * (D + 2) + D + 1] * f;
-    O += part[s * (D + 2) + c] * f;
-  }
-  const float res = Lsum > 0.f ? O / Lsum : 0.f;
-  if constexpr (sizeof(T) == 4)
-    reinterpret_cast<float*>(p.out)[(int64_t)row * D + c] = res;
-  else
-    reinterpret_cast<__nv_bfloat16*>(p.out)[(int64_t)row * D + c] = __float2bfloat16_rn(res);
-  if (p.lse_out && c == 0) p.lse_out[row] = Lsum > 0.f ? (M + log2f(Lsum)) * kLn2 : -INFINITY;
-}
-
-// Smallest share of a segment that a block takes. 512 rows when there are segments enough to fill the GPU (shorter
-// shares leave a block's load pipeline no time to fill and cost more merge work: measured 5-8 % at 256 rows); a call
-// with few segments (one layer of a long-context model: 8 segments) is bound by the latency of its longest block,
-// and there shorter shares spread a segment over more blocks: 128 rows for the scalar kernel (one layer of the llava
-// workload: 747 -> 488 us for the 32 layers of a step), 256 for the tensor-core kernel, whose four warps take 64
-// rows per iteration (at 128 rows it lost more in merge work than it gained: long 429 -> 471 us, at 256: 426).
-int min_share_rows(int n_sel, bool tensor_core_kernel) {
-  return n_sel >= 64 ? kDecodeMinRows : (tensor_core_kernel ? 256 : 128);
-}
-
-// Blocks launched per segment (the grid is segments x this number, and a block whose share of its segment is empty
-// returns at once). With segments enough to fill the GPU 8 is plenty, and the thousands of blocks that 32 per segment
-// launched only to return cost a tenth of the call (batched 246 -> 219 us, qwen 26.6 -> 23.8); a long segment then
-// simply gets longer shares. A call with few segments keeps 32 (scalar kernel) or 16 (tensor-core kernel).
-int blocks_per_segment(int n_sel, bool tensor_core_kernel, int splits) {
-  const int want = n_sel >= 64 ? 8 : (tensor_core_kernel ? 16 : kDecodeSlots);
-  return splits < want ? splits : want;
-}
-
-// Block order of the grid. With many segments a segment's blocks follow one another (neighbouring blocks stream
-// neighbouring rows); with fewer segments than SMs the grid is a wave or two, and then the blocks are ordered by slot so
-// that every segment's last and shortest block is scheduled last.
-int slot_order(int n_sel) {
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return 1;
-  return n_sel >= sms ? 1 : 0;
+  const int64_t want = 3 * rows / (2 * share) + 1;  // (segments may be longer than the mean)
+  const int slots = splits < most ? splits : most;
+  return {(int)(want < slots ? want : slots), share};
 }
 
 template <typename T, int D>
-int run(const DecodeParams& p, const madakv_config&, cudaStream_t st) {
-  const int n_sel = p.n_sel;
-  // every host-side refusal comes before the first launch (an appending call changes the cache)
+int run(DecodeParams p, const madakv_config& c, int splits, cudaStream_t st) {
+  // every host-side refusal comes before the launch (an appending call changes the cache)
   const bool mma = sizeof(T) == 2 && p.g >= 3 && p.g <= 16;
   if (!mma && p.g > 8) return MADAKV_EUNSUPPORTED;
+  const DecodeShape s = decode_shape(c, p.n_sel, p.capacity, mma, splits);
+  p.slots = s.slots;
+  p.min_rows = s.min_rows;
+  p.part_ml = reinterpret_cast<float2*>(p.part + (int64_t)c.batch * c.n_layers * c.n_q_heads * s.slots * D);
+  const dim3 grid((unsigned)p.n_sel * p.slots);  // one dimension: no 65535 limit on the number of segments
   if constexpr (sizeof(T) == 2) {
-    if (mma && cudaFuncSetAttribute(decode_partial_mma_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    MmaTile<D>::BYTES) != cudaSuccess)
-      return MADAKV_ECUDA;
+    if (mma) {
+      if (cudaFuncSetAttribute(decode_mma_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, MmaTile<D>::BYTES) !=
+          cudaSuccess)
+        return MADAKV_ECUDA;
+      launch_pdl(decode_mma_kernel<D>, grid, dim3(kMmaWarps * 32), MmaTile<D>::BYTES, st, p);
+      return launch_status();
+    }
   }
-  const dim3 grid((unsigned)n_sel * p.slots);  // one dimension: no 65535 limit on the number of segments
-  if constexpr (sizeof(T) == 2) {
-    if (mma) launch_pdl(decode_partial_mma_kernel<D>, grid, dim3(kMmaWarps * 32), MmaTile<D>::BYTES, st, p);
-  }
-  if (mma) {
-  } else if (p.g == 1) launch_pdl(decode_partial_kernel<T, D, 1>, grid, dim3(NT), 0, st, p);
-  else if (p.g == 2) launch_pdl(decode_partial_kernel<T, D, 2>, grid, dim3(NT), 0, st, p);
-  else if (p.g <= 4) launch_pdl(decode_partial_kernel<T, D, 4>, grid, dim3(NT), 0, st, p);
-  else launch_pdl(decode_partial_kernel<T, D, 8>, grid, dim3(NT), 0, st, p);
-  // (the merge may be scheduled while the partial kernel runs; it waits for its completion before reading anything)
-  launch_pdl(decode_merge_kernel<T, D>, dim3(n_sel * p.g), dim3(D), 0, st, p);
-  return launch_status();
+  auto go = [&](auto kernel) {
+    launch_pdl(kernel, grid, dim3(NT), kRingStages * kStageBytes, st, p);
+    return launch_status();
+  };
+  if (p.g == 1) return go(decode_kernel<T, D, 1>);
+  if (p.g == 2) return go(decode_kernel<T, D, 2>);
+  if constexpr (sizeof(T) == 4) return p.g <= 4 ? go(decode_kernel<T, D, 4>) : go(decode_kernel<T, D, 8>);
+  return MADAKV_EUNSUPPORTED;
 }
 
 }  // namespace
@@ -623,7 +788,7 @@ int launch_decode(const madakv_config& c, int layer, const void* q, const void* 
   p.out = out;
   p.lse_out = lse_out;
   p.part = reinterpret_cast<float*>((char*)ws + wl.decode_off);
-  p.eff_len = k_new ? reinterpret_cast<int32_t*>((char*)ws + wl.decode_len_off) : nullptr;
+  p.counter = reinterpret_cast<unsigned*>((char*)ws + kHeaderBytes);
   p.ws = ws;
   p.L = c.n_layers;
   p.Hq = c.n_q_heads;
@@ -631,13 +796,10 @@ int launch_decode(const madakv_config& c, int layer, const void* q, const void* 
   p.g = c.n_q_heads / c.n_kv_heads;
   p.layer = layer;
   p.n_sel = (layer < 0 ? c.batch * c.n_layers : c.batch) * c.n_kv_heads;
-  const bool tc = c.dtype == MADAKV_BF16 && p.g >= 3 && p.g <= 16;
-  p.slots = blocks_per_segment(p.n_sel, tc, wl.decode_splits);
-  p.min_rows = min_share_rows(p.n_sel, tc);
-  p.slot_fast = slot_order(p.n_sel);
+  const int splits = wl.decode_splits;
   p.scale2 = scale_of(c) * kLog2e;
-  if (c.dtype == MADAKV_F32) return c.head_dim == 64 ? run<float, 64>(p, c, st) : run<float, 128>(p, c, st);
-  return c.head_dim == 64 ? run<__nv_bfloat16, 64>(p, c, st) : run<__nv_bfloat16, 128>(p, c, st);
+  if (c.dtype == MADAKV_F32) return c.head_dim == 64 ? run<float, 64>(p, c, splits, st) : run<float, 128>(p, c, splits, st);
+  return c.head_dim == 64 ? run<__nv_bfloat16, 64>(p, c, splits, st) : run<__nv_bfloat16, 128>(p, c, splits, st);
 }
 
 }  // namespace madakv
@@ -647,8 +809,13 @@ int launch_decode(const madakv_config& c, int layer, const void* q, const void* 
 // image, for callers that have no way to provide (or allocate) a workspace.
 // ---------------------------------------------------------------------------------------------------------------
 
-// Split partials of the no-allocation entry point. One copy per GPU that loads the library, shared by all calls.
-static __device__ __align__(256) unsigned char g_static_scratch[MADAKV_STATIC_SCRATCH_BYTES];
+// Split partials of the no-allocation entry point. One copy per GPU that loads the library, shared by all calls. The segment
+// counters of a split call lie behind them; they start at zero and every call leaves them at zero.
+struct StaticScratch {
+  unsigned char part[MADAKV_STATIC_SCRATCH_BYTES];
+  unsigned counter[madakv::kDecodeCounters];
+};
+static __device__ __align__(256) StaticScratch g_static_scratch;
 
 namespace madakv {
 namespace {
@@ -696,6 +863,7 @@ extern "C" int madakv_decode_attn_static(const madakv_config* cfg, int32_t layer
   if (need > (size_t)MADAKV_STATIC_SCRATCH_BYTES) return MADAKV_ESTATIC;
   void* scratch = nullptr;
   if ((rc = static_scratch(&scratch))) return rc;
+  unsigned* counters = reinterpret_cast<unsigned*>((char*)scratch + offsetof(StaticScratch, counter));
 
   DecodeParams p;
   p.q = q;
@@ -709,7 +877,7 @@ extern "C" int madakv_decode_attn_static(const madakv_config* cfg, int32_t layer
   p.out = out;
   p.lse_out = lse_out;
   p.part = reinterpret_cast<float*>(scratch);
-  p.eff_len = nullptr;
+  p.counter = counters;
   p.ws = nullptr;  // only an appending call reports through the workspace
   p.L = c.n_layers;
   p.Hq = c.n_q_heads;
@@ -717,12 +885,8 @@ extern "C" int madakv_decode_attn_static(const madakv_config* cfg, int32_t layer
   p.g = c.n_q_heads / c.n_kv_heads;
   p.layer = layer;
   p.n_sel = (layer < 0 ? c.batch * c.n_layers : c.batch) * c.n_kv_heads;
-  const bool tc = c.dtype == MADAKV_BF16 && p.g >= 3 && p.g <= 16;
-  p.slots = blocks_per_segment(p.n_sel, tc, splits);  // what the kernels use of the (larger) documented bound
-  p.min_rows = min_share_rows(p.n_sel, tc);
-  p.slot_fast = slot_order(p.n_sel);
   p.scale2 = scale_of(c) * kLog2e;
   cudaStream_t st = (cudaStream_t)stream;
-  if (c.dtype == MADAKV_F32) return c.head_dim == 64 ? run<float, 64>(p, c, st) : run<float, 128>(p, c, st);
-  return c.head_dim == 64 ? run<__nv_bfloat16, 64>(p, c, st) : run<__nv_bfloat16, 128>(p, c, st);
+  if (c.dtype == MADAKV_F32) return c.head_dim == 64 ? run<float, 64>(p, c, splits, st) : run<float, 128>(p, c, splits, st);
+  return c.head_dim == 64 ? run<__nv_bfloat16, 64>(p, c, splits, st) : run<__nv_bfloat16, 128>(p, c, splits, st);
 }

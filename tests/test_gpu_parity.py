@@ -639,6 +639,51 @@ def test_decode_with_more_than_65535_segments():
     assert np.abs(out.cpu().numpy() - want).max() <= 2e-5
 
 
+# one segment over 32 blocks, a wave of few segments, more segments at shares of 512 rows and at one block each; stages of
+# the ring that end inside and at the last row, segments without rows, group sizes of both kernels
+@pytest.mark.parametrize("dtype,d,g,units,rows", [
+    ("bf16", 128, 1, 1, 6000), ("bf16", 64, 2, 9, 513), ("bf16", 128, 5, 3, 4100), ("bf16", 64, 16, 20, 257),
+    ("bf16", 128, 1, 70, 1500), ("bf16", 128, 3, 70, 1025), ("bf16", 128, 2, 1100, 63), ("f32", 128, 1, 5, 1000),
+    ("f32", 64, 3, 66, 700), ("f32", 128, 7, 2, 300), ("f32", 64, 8, 64, 33)])
+def test_decode_over_blocks_per_segment(dtype, d, g, units, rows):
+    """Every way the decode kernels share a segment out, against the oracle: two appending steps in a row on a workspace
+    that a call of another shape has used, then a step without append. Tolerances as for the other decode tests."""
+    wl = synth.scaled(TINY, dtype=dtype, B=1, L=units, Hq=g, Hkv=1, d=d, n=rows, w=4, max_new_tokens=3)
+    cfg = config_of(wl)
+    rng = np.random.RandomState(units + rows)
+    lens = rng.randint(rows // 2, rows + 1, size=units).astype(np.int32)
+    lens[rng.randint(units)] = rows
+    if units > 1:
+        lens[0], lens[-1] = 0, rows // 32 * 32
+    seg_off = np.concatenate([[0], np.cumsum(lens.astype(np.int64) + wl.max_new_tokens)])
+    total = int(seg_off[-1])
+    k_c, v_c = (synth.hash_normal(1, t, 0, total * d).view(total, d).to(wl.torch_dtype) for t in (91, 92))
+    d_kc, d_vc, d_len, d_off = k_c.cuda(), v_c.cuda(), torch.from_numpy(lens).cuda(), torch.from_numpy(seg_off).cuda()
+    kc_np, vc_np, lens_np = to_np(k_c).copy(), to_np(v_c).copy(), lens.copy()
+    ws = mk.new_workspace(cfg)
+    if units > 1:  # another shape on the same workspace: one layer alone
+        one = config_of(wl)
+        q = synth.make_decode_step(wl, 9)[0].cuda()
+        mk.madakv_decode_attn(one, units - 1, q, None, None, d_kc, d_vc, d_off, d_len, torch.zeros_like(q), None, ws)
+    for step in range(3):
+        q, kn, vn = synth.make_decode_step(wl, step)
+        if step == 2:
+            kn = vn = None
+        out = torch.zeros((1, units, g, d), dtype=wl.torch_dtype, device="cuda")
+        lse = torch.zeros((1, units, g), device="cuda")
+        mk.madakv_decode_attn(cfg, -1, q.cuda(), None if kn is None else kn.cuda(), None if vn is None else vn.cuda(),
+                              d_kc, d_vc, d_off, d_len, out, lse, ws)
+        assert mk.madakv_poll_status(ws) == 0
+        rc, want, want_lse = oracle.decode(dcode(wl), to_np(q), None if kn is None else to_np(kn),
+                                           None if vn is None else to_np(vn), kc_np, vc_np, seg_off, lens_np, Hkv=1)
+        assert rc == 0 and np.array_equal(d_len.cpu().numpy(), lens_np)
+        assert np.abs(out.float().cpu().numpy() - want).max() <= DEC_ATOL[dtype]
+        some = np.isfinite(want_lse)
+        assert np.array_equal(some, np.isfinite(lse.cpu().numpy()))
+        assert np.abs(lse.cpu().numpy()[some] - want_lse[some]).max() <= 1e-5 * max(1.0, np.abs(want_lse[some]).max())
+    assert np.array_equal(to_np(d_kc), kc_np) and np.array_equal(to_np(d_vc), vc_np)
+
+
 def test_bounded_wait_runs_out_and_the_library_recovers(monkeypatch):
     """Failure detection without a GPU fault: the two-phase scoring kernel's phase-2 items wait (bounded) for row flags
     that phase 1 publishes. With the flags withheld and the bound shortened to ~1 ms the wait runs out: the kernel
