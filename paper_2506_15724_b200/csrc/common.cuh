@@ -38,7 +38,7 @@ struct WsHeader {
 static_assert(sizeof(WsHeader) == kHeaderBytes, "header size");
 
 struct WsLayout {
-  size_t seq_nv_off, score_done_off, score_lse_off, score_part_off, decode_off, total;
+  size_t seq_nv_off, score_done_off, score_lse_off, score_part_off, score_split_off, decode_off, total;
   int score_chunks, score_tc_chunks, decode_splits;
 };
 
@@ -49,13 +49,29 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // tiles meets at most ceil(t / floor(T / G)) + 1 of the G ranges (T tiles in all), and T >= L * Hkv * t, which
 // gives the bound below whatever the lengths in the batch are.
 constexpr int kWideMaxGrid = 160;
-inline int wide_max_runs(const madakv_config& c) {
-  const long long lh = (long long)c.n_layers * c.n_kv_heads;
+inline int wide_max_runs(int units_per_seq, int n_max) {
+  const long long lh = units_per_seq;
   long long runs = (2ll * kWideMaxGrid + lh - 1) / lh + 1;
-  const long long tiles = (c.max_seq_len + 127) / 128;
+  const long long tiles = (n_max + 127) / 128;
   if (runs > kWideMaxGrid) runs = kWideMaxGrid;
   if (runs > tiles) runs = tiles;
   return (int)(runs < 1 ? 1 : runs);
+}
+// fp32 scoring on the tensor cores: keys and queries split into three bf16 terms each, 6 bytes per element, for as many units
+// at a time as kSplitBytes hold (at least one). 96 MB stay in the L2 for the most part between the two passes over them and
+// give the GPU's SMs several tiles each.
+constexpr size_t kSplitBytes = 96u << 20;
+inline size_t split_unit_bytes(const madakv_config& c) {
+  return ((size_t)c.max_seq_len + (size_t)(c.n_q_heads / c.n_kv_heads) * c.window) * c.head_dim * 6;
+}
+inline int split_units(const madakv_config& c) {
+  const long long lh = (long long)c.n_layers * c.n_kv_heads, total = lh * c.batch;
+  long long fit = (long long)(kSplitBytes / split_unit_bytes(c));
+  if (fit < 1) fit = 1;
+  if (fit >= total) return (int)total;
+  if (fit >= lh) return (int)(fit / lh * lh);
+  const long long parts = (lh + fit - 1) / fit;  // parts of a sequence, as even as possible
+  return (int)((lh + parts - 1) / parts);
 }
 
 inline WsLayout ws_layout(const madakv_config& c) {
@@ -74,17 +90,20 @@ inline WsLayout ws_layout(const madakv_config& c) {
   off = align_up(off + units * rows_pad * sizeof(float), 256);
   w.score_part_off = off;
   w.score_tc_chunks = (c.max_seq_len + kScoreTcChunk - 1) / kScoreTcChunk;
-  // partials: the generic path keeps one (max, sum) per (chunk, row); the tensor-core path (rows <= 64 only) one
-  // per (work item, TMEM lane quarter, padded row)
+  // partials: the generic path keeps one (max, sum) per (chunk, row); the two-phase tensor-core path (rows <= 64 only) one
+  // per (work item, TMEM lane quarter, padded row); the wide-window path, which takes up to 256 rows per launch, one per
+  // run of a unit, padded row and column share: a sequence of x units has at most 320 + 2 x runs (wide_max_runs)
   size_t part = units * (size_t)w.score_chunks * rows * sizeof(float2);
   if (rows <= 64) {
     const size_t tc = units * rows_pad * (size_t)w.score_tc_chunks * 4 * sizeof(float2);
     part = tc > part ? tc : part;
-  } else if (rows <= 256) {  // wide-window path: per run of a unit and padded row one pair for each column share
-    const size_t wide = units * (size_t)wide_max_runs(c) * (rows <= 128 ? 4 : 2) * rows_pad * sizeof(float2);
-    part = wide > part ? wide : part;
   }
+  const size_t share_rows = rows_pad <= 128 ? 4 * rows_pad : 512;  // column shares x rows of a launch
+  const size_t wide = (2 * kWideMaxGrid * (size_t)c.batch + 2 * units) * share_rows * sizeof(float2);
+  part = wide > part ? wide : part;
   off = align_up(off + part, 256);
+  w.score_split_off = off;
+  if (c.dtype == MADAKV_F32) off = align_up(off + split_unit_bytes(c) * (size_t)split_units(c), 256);
   w.decode_off = off;
   off = align_up(off + (size_t)c.batch * c.n_layers * c.n_q_heads * (size_t)w.decode_splits * (c.head_dim + 2) *
                            sizeof(float), 256);

@@ -334,15 +334,14 @@ int launch_score_lse(const madakv_config& c, const void* q, madakv_strides sq, c
 int launch_score(const madakv_config& c, const void* q, madakv_strides sq, const void* k, madakv_strides sk,
                  const int32_t* seq_len, float* lse, float* psi, void* ws, cudaStream_t st) {
   if (score_tc_supported(c, sq, sk)) {
-    // tensor-core paths: logits resident in a cluster's TMEM when a unit fits, else the two-phase kernel; shapes
-    // they decline go the generic way
+    // logits resident in a cluster's TMEM when a unit fits
     int rc = launch_score_cluster(c, q, sq, k, sk, seq_len, lse, psi, ws, st);
     if (rc != MADAKV_EUNSUPPORTED) return rc;
+    // else the two-phase kernel; sequences too long for its lead of work items go on
     rc = launch_score_tc(c, q, sq, k, sk, seq_len, lse, psi, ws, st);
     if (rc != MADAKV_EUNSUPPORTED) return rc;
   }
   if (tc_device_ok()) {
-    // wide windows (64 < g * w <= 256): window rows on M, one row per epilogue thread
     const int rc = launch_score_rows(c, q, sq, k, sk, seq_len, lse, psi, ws, st);
     if (rc != MADAKV_EUNSUPPORTED) return rc;
   }

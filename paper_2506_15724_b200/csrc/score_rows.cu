@@ -1,6 +1,13 @@
-// Stage 1, tensor-core path for wide windows (Eq. 7 with the softmax of Eq. 5): bf16 inputs with 64 < g * w <= 256
-// window rows per KV head (grouped-query attention with many query heads per KV head), and the single-pass form of
-// stage 1 (log-sum-exps supplied by the caller) for every bf16 shape with g * w <= 256.
+// Stage 1, tensor-core path for wide windows (Eq. 7 with the softmax of Eq. 5): bf16 inputs whose logits do not fit a
+// cluster's TMEM, fp32 inputs, and the single-pass form of stage 1 (log-sum-exps supplied by the caller).
+//
+// A launch takes up to 256 window rows per KV head (fp32: 128); shapes with more go in chunks of query heads (or, for
+// windows beyond that, of window rows) one launch after the other, each adding its part to psi.
+//
+// fp32 inputs are split exactly into three bf16 numbers of 8 significand bits each (split_kernel writes them to the
+// workspace, a slice of the units at a time), and a product q * k is taken as the six partial products that are not below
+// 2^-24 of it: hi hi, hi mid, mid hi, mid mid, hi lo, lo hi, all accumulated in fp32. An SM's fp32 pipes do 256 FLOP per
+// clock, its tensor cores 8192 / 6.
 //
 // With that many rows the work per key byte is dominated by the exponentials (g * w of them per key and pass), not
 // by HBM: the special-function unit delivers 16 exp2 per clock and SM, which for 256 rows is 2048 clocks per 128-key
@@ -40,26 +47,34 @@ struct RowParams {
   const int32_t* seq_len;
   float* psi;        // [units, n_max]
   float2* part;      // ws: [units, smax, cparts, rs] (max, sum) of every row over a column share of one CTA's run
+  const float* given_lse;  // pass 2: natural-log sum-exps [B, L, Hq, w] supplied by the caller (lse2 is not used then)
   const float* lse2; // ws: [units, rs] NEGATED log2-domain log-sum-exp, padding rows hold kEmptyMax (pass 2)
   int32_t* status;   // ws header
   int B, units, L, Hq, Hkv, g, w, R, n_max, causal, rs, mblocks, cparts, n16;  // n16: R rounded up to 16
+  int lh;            // units per sequence (of this launch)
+  int u0;            // fp32: first unit of the slice; unit u of the launch is unit u0 + u of the call
+  int h0, r0, wc;    // the launch's window rows: rows [r0, r0 + wc) of query heads h0 .. of the group, R = heads * wc
+  int accumulate;    // psi += instead of =
   int smax;          // runs (CTAs) a unit's tiles can be spread over at most: wide_max_runs()
   int grid;          // CTAs of the two passes (the merge kernel needs the partition)
   float scale2;
 };
 
-template <int D, int PASS>
+template <int D, int PASS, int NS>  // NS: bf16 terms per operand (1, or 3 for fp32)
 struct RowSmem {
-  // pass 2 gives up one K stage for the operands of its extra contraction step (see the MMA issuer)
-  static constexpr int kStages = (D == 128 ? 4 : 8) - (PASS == 2 ? (D == 128 ? 1 : 2) : 0);
+  // NS = 1: a stage is a whole K tile. NS = 3: a stage is one 64-wide piece of one term of it, 16 KB.
+  // pass 2 gives up K stages for the operands of its extra contraction step (see the MMA issuer)
+  static constexpr int kStages = NS == 3 ? (PASS == 2 ? 5 : 6) : (D == 128 ? 4 : 8) - (PASS == 2 ? (D == 128 ? 1 : 2) : 0);
   static constexpr int kKBlocks = D / 64;
-  static constexpr int kStageBytes = kTileKeys * D * 2;
-  static constexpr int kQBytes = 256 * D * 2;  // up to two blocks of 128 rows
+  static constexpr int kPieces = NS == 3 ? 3 * kKBlocks : 1;  // stages per tile
+  static constexpr int kStageBytes = NS == 3 ? kTileKeys * 128 : kTileKeys * D * 2;
+  static constexpr int kQRows = NS == 3 ? 128 : 256;  // up to two blocks of 128 rows
+  static constexpr int kQBytes = kQRows * D * 2 * NS;
   static constexpr int kKOff = 0;
   static constexpr int kQOff = kStages * kStageBytes;
   static constexpr int kOnesOff = kQOff + kQBytes;                          // pass 2: [128 keys][64] bf16, 1 in columns 0-2
-  static constexpr int kShiftOff = kOnesOff + (PASS == 2 ? 128 * 128 : 0);  // pass 2: [256 rows][64] bf16, columns 0-2
-  static constexpr int kBarOff = kShiftOff + (PASS == 2 ? 256 * 128 : 0);
+  static constexpr int kShiftOff = kOnesOff + (PASS == 2 ? 128 * 128 : 0);  // pass 2: [rows][64] bf16, columns 0-2
+  static constexpr int kBarOff = kShiftOff + (PASS == 2 ? kQRows * 128 : 0);
   // full[kStages], empty[kStages], qfull, qempty, tfull[2], tempty[2], drain, xfull[8], xempty[8]
   static constexpr int kNumBars = 2 * kStages + 2 + 4 + 1 + 16;
   static constexpr int kMiscOff = (kBarOff + kNumBars * 8 + 15) / 16 * 16;
@@ -239,7 +254,7 @@ __device__ __forceinline__ void cursor_settle(const RowParams& p, TileCursor& c,
       break;
     }
     c.tb = tiles_of(p, c.b, exact);
-    c.per_b = p.L * p.Hkv * c.tb;
+    c.per_b = p.lh * c.tb;
   }
 }
 __device__ __forceinline__ Run cursor_run(const RowParams& p, const TileCursor& c) {
@@ -248,7 +263,7 @@ __device__ __forceinline__ Run cursor_run(const RowParams& p, const TileCursor& 
   r.t0 = c.r - ub * c.tb;
   r.cnt = min(c.tb - r.t0, c.left);
   r.b = c.b;
-  r.u = c.b * p.L * p.Hkv + ub;
+  r.u = c.b * p.lh + ub;
   r.n = clamped_len(p.seq_len, c.b, p.n_max);
   const int real = (r.n + kTileKeys - 1) / kTileKeys;  // tiles of the unit that hold keys
   r.tiles = max(0, min(r.t0 + r.cnt, real) - r.t0);
@@ -268,10 +283,10 @@ __device__ __forceinline__ int cta_of(long long total, int grid, long long x) {
   return c;
 }
 
-template <int D, int PASS>
+template <int D, int PASS, int NS>
 __global__ void __launch_bounds__(kRowThreads, 1)  // 96 registers: warps are allocated four at a time (18 -> 20)
 score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_q, RowParams p) {
-  using SL = RowSmem<D, PASS>;
+  using SL = RowSmem<D, PASS, NS>;
   constexpr int kStages = SL::kStages;
   constexpr int kKBlocks = SL::kKBlocks;
   extern __shared__ uint8_t smem_raw[];
@@ -316,11 +331,22 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  // rows R..255 of the Q buffer are never written by TMA: keep them zero so their logits are 0. Pass 2: the operands
+  // of the extra contraction step start out as zeros, the key side gets its three ones per row (128-byte rows with
+  // the 128-byte swizzle: the 16-byte piece that holds columns 0-7 of row r sits at position r % 8).
+  for (int x = threadIdx.x; x < (SL::kBarOff - SL::kQOff) / 16; x += kRowThreads)
+    reinterpret_cast<uint4*>(q_s)[x] = make_uint4(0, 0, 0, 0);
+  for (int x = threadIdx.x; x < 256; x += kRowThreads) rowpos[x] = p.r0 + x % p.wc;
+  // (everything above touches only this CTA's shared memory: it overlaps the kernel before this one)
+  pdl_wait();
+  pdl_go();
+  if (threadIdx.x == 0) {
     // this CTA's range of tiles
     const bool exact = p.B <= kMaxSeqScan;
     long long total = 0;
     if (exact) {
-      for (int b = 0; b < p.B; ++b) total += (long long)p.L * p.Hkv * tiles_of(p, b, true);
+      for (int b = 0; b < p.B; ++b) total += (long long)p.lh * tiles_of(p, b, true);
     } else {
       total = (long long)p.units * tiles_of(p, 0, false);
     }
@@ -333,13 +359,13 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
     long long r0 = lo;
     if (exact) {
       while (b0 < p.B) {
-        const long long per = (long long)p.L * p.Hkv * tiles_of(p, b0, true);
+        const long long per = (long long)p.lh * tiles_of(p, b0, true);
         if (r0 < per) break;
         r0 -= per;
         ++b0;
       }
     } else {
-      const long long per = (long long)p.L * p.Hkv * tiles_of(p, 0, false);
+      const long long per = (long long)p.lh * tiles_of(p, 0, false);
       b0 = (int)(lo / per);
       r0 = lo - (long long)b0 * per;
     }
@@ -351,12 +377,6 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
     range_s[5] = (int)total;
     range_s[6] = (int)ctas;
   }
-  // rows R..255 of the Q buffer are never written by TMA: keep them zero so their logits are 0. Pass 2: the operands
-  // of the extra contraction step start out as zeros, the key side gets its three ones per row (128-byte rows with
-  // the 128-byte swizzle: the 16-byte piece that holds columns 0-7 of row r sits at position r % 8).
-  for (int x = threadIdx.x; x < (SL::kBarOff - SL::kQOff) / 16; x += kRowThreads)
-    reinterpret_cast<uint4*>(q_s)[x] = make_uint4(0, 0, 0, 0);
-  for (int x = threadIdx.x; x < 256; x += kRowThreads) rowpos[x] = x % p.w;
   __syncthreads();
   if (PASS == 2 && threadIdx.x < kTileKeys) {
     const int r = threadIdx.x;
@@ -382,7 +402,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
     c.left = c.b < p.B ? range_s[2] : 0;
     c.done = 0;
     c.tb = c.left > 0 ? tiles_of(p, c.b, exact) : 1;
-    c.per_b = p.L * p.Hkv * c.tb;
+    c.per_b = p.lh * c.tb;
     cursor_settle(p, c, exact);
     return c;
   };
@@ -390,7 +410,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
   if (warp == 0) {
     // ================================================================ TMA producer: lane 0 waits and issues the
     // copies; the whole warp walks the items with it, because in pass 2 all 32 lanes write the unit's shift rows
-    const uint64_t pol_k = l2_policy_evict_first();
+    const uint64_t pol_k = NS == 3 ? l2_policy_evict_last() : l2_policy_evict_first();  // (split keys are read again)
     const uint64_t pol_q = l2_policy_evict_last();
     int stage = 0, cur_u = -1;
     uint32_t stage_par = 0, q_par = 0;
@@ -400,7 +420,8 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
       cursor_advance(p, c, run, exact);
       const int u = run.u, tiles = run.tiles, key_begin = run.t0 * kTileKeys;
       if (tiles == 0) continue;
-      const int h = u % p.Hkv, l = (u / p.Hkv) % p.L, b = u / (p.Hkv * p.L);
+      // fp32: the slice's split operands are [units][n_max][3 D] and [units * g][w][3 D]
+      const int h = NS == 3 ? u : u % p.Hkv, l = NS == 3 ? 0 : (u / p.Hkv) % p.L, b = NS == 3 ? 0 : u / p.lh;
       if (u != cur_u) {  // a new run: the unit's queries (and, in pass 2, its shift rows)
         cur_u = u;
         if (lane == 0) ok = mbar_wait(qempty, q_par ^ 1, abort_flag, p.status, kSiteQEmpty);
@@ -413,8 +434,19 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
           // and the epilogue needs no per-row operand at all.
           const float inv = 1.0f / p.scale2;
           const float* src = p.lse2 + (int64_t)u * p.rs;
+          const int gh = (p.u0 + u) % p.Hkv, gbl = (p.u0 + u) / p.Hkv;
           for (int r = lane; r < p.n16; r += 32) {
-            const float v = src[r] * inv;
+            float nl;  // a row that sees no key (-inf) and the padding rows get a shift that turns every weight into 0
+            if (p.given_lse) {
+              nl = kEmptyMax;
+              if (r < p.R) {
+                const float gl = p.given_lse[((int64_t)gbl * p.Hq + gh * p.g + p.h0 + r / p.wc) * p.w + p.r0 + r % p.wc];
+                if (gl > -INFINITY) nl = -gl * kLog2e;
+              }
+            } else {
+              nl = src[r];
+            }
+            const float v = nl * inv;
             const float hi = __bfloat162float(__float2bfloat16_rn(v));
             const float mid = __bfloat162float(__float2bfloat16_rn(v - hi));
             const float low = __bfloat162float(__float2bfloat16_rn((v - hi) - mid));
@@ -425,19 +457,26 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
           __syncwarp();  // every lane's rows are written (and fenced) before lane 0 signals the unit ready
         }
         if (lane == 0) {
-          mbar_expect_tx(qfull, (uint32_t)(p.R * 128 * kKBlocks));
-          for (int kb = 0; kb < kKBlocks; ++kb)
-            tma_load_5d(q_s + kb * 256 * 128, &tmap_q, qfull, kb * 64, 0, h * p.g, l, b, pol_q);
+          mbar_expect_tx(qfull, (uint32_t)(p.R * 128 * kKBlocks * NS));
+          for (int kb = 0; kb < kKBlocks * NS; ++kb)
+            tma_load_5d(q_s + kb * SL::kQRows * 128, &tmap_q, qfull, kb * 64, p.r0, h * p.g + p.h0, l, b, pol_q);
         }
       }
       if (lane == 0) {
-        for (int t = 0; t < tiles; ++t) {
+        for (int x = 0; x < tiles * SL::kPieces; ++x) {
+          const int t = x / SL::kPieces, piece = x % SL::kPieces;
           ok = mbar_wait(&empty[stage], stage_par ^ 1, abort_flag, p.status, kSiteStage);
           if (!ok) break;
           mbar_expect_tx(&full[stage], (uint32_t)SL::kStageBytes);
-          for (int kb = 0; kb < kKBlocks; ++kb)
-            tma_load_5d(k_s + stage * SL::kStageBytes + kb * kTileKeys * 128, &tmap_k, &full[stage], kb * 64,
-                        key_begin + t * kTileKeys, h, l, b, pol_k);
+          if (NS == 3) {
+            tma_load_5d(k_s + stage * SL::kStageBytes, &tmap_k, &full[stage],
+                        ((2 - piece / kKBlocks) * kKBlocks + piece % kKBlocks) * 64, key_begin + t * kTileKeys, h, l,
+                        b, pol_k);
+          } else {
+            for (int kb = 0; kb < kKBlocks; ++kb)
+              tma_load_5d(k_s + stage * SL::kStageBytes + kb * kTileKeys * 128, &tmap_k, &full[stage], kb * 64,
+                          key_begin + t * kTileKeys, h, l, b, pol_k);
+          }
           if (++stage == kStages) {
             stage = 0;
             stage_par ^= 1;
@@ -474,9 +513,59 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
         for (int t = 0; t < tiles; ++t, ++n_tile) {
           const int buf = n_tile & 1;
           const uint32_t use_par = (uint32_t)(n_tile >> 1) & 1u;
+          ok = mbar_wait(&tempty[buf], use_par ^ 1, abort_flag, p.status, kSiteTEmpty);
+          if (!ok) break;
+          if (NS == 3) {
+            // A stage is 64 contraction steps of one term of the keys, in the order lo, mid, hi. The accumulation
+            // truncates, so the small products come first (lo hi, mid hi, mid mid, hi lo, hi mid) and the 8 or 4 steps of
+            // hi hi last, for which the stages of hi are held: the result is as exact as that of a plain bf16 contraction.
+            // (hi hi first: log-sum-exps off by 7e-7 instead of 6e-8, relative.)
+            auto product = [&](uint32_t k_lo, int qt, int kb, uint32_t first) {
+#pragma unroll
+              for (int kk = 0; kk < 4; ++kk) {
+                const uint32_t q_op = q_lo0 + (((qt * kKBlocks + kb) * SL::kQRows * 128 + kk * 32) >> 4);
+                const uint32_t k_op = k_lo + ((kk * 32) >> 4), add = first && kk == 0 ? 0u : 1u;
+                if (PASS == 1) umma_bf16(tmem_base + buf * 256, q_op, k_op, kIdescRows, add);
+                else umma_bf16(tmem_base + buf * 256, k_op, q_op, idesc2, add);
+              }
+            };
+            uint32_t hi_lo[kKBlocks];
+            int hi_stage[kKBlocks];
+#pragma unroll
+            for (int piece = 0; piece < SL::kPieces; ++piece) {
+              const int term = 2 - piece / kKBlocks, kb = piece % kKBlocks;
+              ok = ok && mbar_wait(&full[stage], stage_par, abort_flag, p.status, kSiteFull);
+              if (ok) {
+                tc_fence_after();
+                const uint32_t k_lo = k_lo0 + (uint32_t)stage * (SL::kStageBytes >> 4);
+                if (term == 2) {
+                  product(k_lo, 0, kb, piece == 0);
+                } else {
+                  product(k_lo, term == 1 ? 0 : 2, kb, 0);
+                  product(k_lo, 1, kb, 0);
+                }
+                if (term == 0) {
+                  hi_lo[kb] = k_lo;
+                  hi_stage[kb] = stage;
+                } else {
+                  umma_commit(&empty[stage]);  // the K stage may be refilled
+                }
+                if (++stage == kStages) {
+                  stage = 0;
+                  stage_par ^= 1;
+                }
+              }
+            }
+            if (!ok) break;
+#pragma unroll
+            for (int kb = 0; kb < kKBlocks; ++kb) {
+              product(hi_lo[kb], 0, kb, 0);
+              umma_commit(&empty[hi_stage[kb]]);
+            }
+            if (PASS == 2) umma_bf16(tmem_base + buf * 256, ones_lo, shift_lo, idesc2, 1u);
+          } else {
           const uint32_t k_lo = k_lo0 + (uint32_t)stage * (SL::kStageBytes >> 4);
-          ok = mbar_wait(&tempty[buf], use_par ^ 1, abort_flag, p.status, kSiteTEmpty) &&
-               mbar_wait(&full[stage], stage_par, abort_flag, p.status, kSiteFull);
+          ok = mbar_wait(&full[stage], stage_par, abort_flag, p.status, kSiteFull);
           if (!ok) break;
           tc_fence_after();
           if (PASS == 1) {  // D[row, key]: a row block of the queries is operand A, the K tile operand B
@@ -499,11 +588,12 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
             umma_bf16(tmem_base + buf * 256, ones_lo, shift_lo, idesc2, 1u);
           }
           umma_commit(&empty[stage]);  // the K stage may be refilled
-          umma_commit(&tfull[buf]);    // the accumulators are ready
           if (++stage == kStages) {
             stage = 0;
             stage_par ^= 1;
           }
+          }
+          umma_commit(&tfull[buf]);    // the accumulators are ready
         }
       }
       if (!ok) {  // abandoned: TMEM may only be freed once this thread's MMAs have completed
@@ -542,6 +632,12 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
     float m = 4.f * kEmptyMax, z_run = 0.f;
     uint64_t zacc[4] = {0ull, 0ull, 0ull, 0ull};  // pass 1: the item's sum, as four packed partial sums
     float* xslot = xch + quarter * 32 + lane;  // pass 2: [buffer][share - 1][128 keys]
+    if (PASS == 2 && exact && !p.accumulate) {  // sequences without keys have no tiles
+      for (int b = 0; b < p.B; ++b)
+        if (clamped_len(p.seq_len, b, p.n_max) == 0)
+          for (int64_t x = (int64_t)blockIdx.x * 512 + ew * 32 + lane; x < (int64_t)p.lh * p.n_max; x += (int64_t)gridDim.x * 512)
+            p.psi[(int64_t)b * p.lh * p.n_max + x] = 0.f;
+    }
 
     for (TileCursor c = cursor_begin(); ok && c.left > 0;) {
       const Run run = cursor_run(p, c);
@@ -554,7 +650,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
       zacc[0] = zacc[1] = zacc[2] = zacc[3] = 0ull;
       int vis = 0;  // pass 1: keys the row may see: [0, vis)
       if (PASS == 1 && row < p.R) {
-        const int pos = n - p.w + row % p.w;
+        const int pos = n - p.w + p.r0 + row % p.wc;
         if (pos >= 0) vis = p.causal ? pos + 1 : n;
       }
       for (int t = 0; t < tiles; ++t, ++n_tile) {
@@ -654,9 +750,13 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
             if (!ok) break;
             total = ((total + xslot[(buf * 3 + 0) * 128]) + xslot[(buf * 3 + 1) * 128]) + xslot[(buf * 3 + 2) * 128];
             mbar_arrive(&xempty[buf * 4 + quarter]);
-            if (key < p.n_max) psi[key] = key < n ? total : 0.f;
+            if (key < p.n_max) psi[key] = key < n ? (p.accumulate ? psi[key] + total : total) : 0.f;
           }
         }
+      }
+      if (PASS == 2 && ok && !p.accumulate && run.t0 + run.cnt >= (n + kTileKeys - 1) / kTileKeys) {
+        // the keys no tile covers, by the CTA that has the unit's last tile
+        for (int key = (n + kTileKeys - 1) / kTileKeys * kTileKeys + ew * 32 + lane; key < p.n_max; key += 512) psi[key] = 0.f;
       }
       if (!ok) break;
       if (PASS == 1) {
@@ -687,174 +787,251 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
   }
 }
 
-// psi of the keys no tile covers: everything from the end of the sequence's last tile
-__device__ __forceinline__ void clear_tail(const RowParams& p, int u, int row) {
-  const int b = u / (p.Hkv * p.L);
-  const int n = clamped_len(p.seq_len, b, p.n_max);
-  const int from = (n + kTileKeys - 1) / kTileKeys * kTileKeys;
-  float* psi = p.psi + (int64_t)u * p.n_max;
-  for (int key = from + row; key < p.n_max; key += p.rs) psi[key] = 0.f;
-}
-
-// merge: per (unit, row) the (max, sum) pairs of all runs and column shares, in a fixed order -> log2-domain
-// log-sum-exp, stored negated (pass 2 adds it inside a fused multiply-add); padding rows get a shift that turns
-// every weight into 0
-__global__ void score_rows_merge_kernel(RowParams p, float* nlse2, float* lse_out, int total) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= total) return;
-  const int u = x / p.rs, row = x % p.rs;
-  clear_tail(p, u, row);
+// merge: per (unit, row) the (max, sum) pairs of all runs and column shares, in a fixed order -> log2-domain log-sum-exp,
+// stored negated (pass 2 adds it inside the contraction); padding rows get a shift that turns every weight into 0. A block
+// takes 32 rows of one unit, eight threads per row: a unit of an fp32 slice can be spread over half of the CTAs (one thread
+// per row took 53 us for 300 pairs).
+__global__ void __launch_bounds__(256) score_rows_merge_kernel(RowParams p, float* nlse2, float* lse_out) {
+  __shared__ float s_m[8][32], s_z[8][32];
+  __shared__ int s_entries;
+  const int blocks = p.rs / 32, u = blockIdx.x / blocks, lane = threadIdx.x & 31, part_i = threadIdx.x >> 5;
+  const int row = blockIdx.x % blocks * 32 + lane;
+  pdl_wait();
+  pdl_go();
+  if (threadIdx.x == 0) {
+    // the CTAs of pass 1 that the unit's tiles were spread over: the same partition as in the kernel
+    const int b = u / p.lh;
+    const bool exact = p.B <= kMaxSeqScan;
+    long long all_tiles = 0, first = 0;  // tiles of the batch; the unit's first tile in the global order
+    const int tb = tiles_of(p, b, exact);
+    if (exact) {
+      for (int b2 = 0; b2 < p.B; ++b2) {
+        const long long per = (long long)p.lh * tiles_of(p, b2, true);
+        if (b2 < b) first += per;
+        all_tiles += per;
+      }
+    } else {
+      all_tiles = (long long)p.units * tb;
+      first = (long long)b * p.lh * tb;
+    }
+    first += (long long)(u - b * p.lh) * tb;
+    s_entries = 0;
+    if (tb > 0) {
+      const int ctas = (int)(all_tiles < p.grid ? all_tiles : p.grid);
+      s_entries = p.cparts * min(p.smax, cta_of(all_tiles, ctas, first + tb - 1) - cta_of(all_tiles, ctas, first) + 1);
+    }
+  }
+  __syncthreads();
+  const int entries = s_entries;
+  const float2* part = p.part + (int64_t)u * p.cparts * p.smax * p.rs + row;
+  float M = kEmptyMax, Z = 0.f;
+  for (int s0 = part_i; s0 < entries; s0 += 32) {
+    float2 v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = s0 + 8 * j < entries ? part[(int64_t)(s0 + 8 * j) * p.rs] : make_float2(kEmptyMax, 0.f);
+    const float mn = fmaxf(fmaxf(fmaxf(v[0].x, v[1].x), fmaxf(v[2].x, v[3].x)), M);
+    Z *= exp2f(M - mn);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) Z += v[j].y * exp2f(v[j].x - mn);  // an empty pair has sum 0
+    M = mn;
+  }
+  s_m[part_i][lane] = M;
+  s_z[part_i][lane] = Z;
+  __syncthreads();
+  if (part_i) return;
+  const int64_t x = (int64_t)u * p.rs + row;
   if (row >= p.R) {
     nlse2[x] = kEmptyMax;
     return;
   }
-  const int b = u / (p.Hkv * p.L);
-  // the CTAs of pass 1 that the unit's tiles were spread over: the same partition as in the kernel
-  const bool exact = p.B <= kMaxSeqScan;
-  long long all_tiles = 0, first = 0;  // tiles of the batch; the unit's first tile in the global order
-  const int tb = tiles_of(p, b, exact);
-  if (exact) {
-    for (int b2 = 0; b2 < p.B; ++b2) {
-      const long long per = (long long)p.L * p.Hkv * tiles_of(p, b2, true);
-      if (b2 < b) first += per;
-      all_tiles += per;
-    }
-  } else {
-    all_tiles = (long long)p.units * tb;
-    first = (long long)b * p.L * p.Hkv * tb;
-  }
-  first += (long long)(u - b * p.L * p.Hkv) * tb;
-  int entries = 0;
-  if (tb > 0) {
-    const int ctas = (int)(all_tiles < p.grid ? all_tiles : p.grid);
-    entries = p.cparts * min(p.smax, cta_of(all_tiles, ctas, first + tb - 1) - cta_of(all_tiles, ctas, first) + 1);
-  }
-  const float2* part = p.part + (int64_t)u * p.cparts * p.smax * p.rs + row;
-  float M = kEmptyMax;
-  for (int s = 0; s < entries; ++s) M = fmaxf(M, part[(int64_t)s * p.rs].x);
-  float Z = 0.f;
-  for (int s = 0; s < entries; ++s) {
-    const float2 v = part[(int64_t)s * p.rs];
-    Z += v.y * exp2f(v.x - M);  // an empty pair has sum 0
-  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) M = fmaxf(M, s_m[j][lane]);
+  Z = 0.f;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) Z += s_z[j][lane] * exp2f(s_m[j][lane] - M);
   const float l2 = Z > 0.f ? M + log2f(Z) : 0.f;
   nlse2[x] = -l2;
   if (lse_out) {
-    const int h = u % p.Hkv, bl = u / p.Hkv;
-    const int hq = h * p.g + row / p.w, wr = row % p.w;
+    const int h = (p.u0 + u) % p.Hkv, bl = (p.u0 + u) / p.Hkv;
+    const int hq = h * p.g + p.h0 + row / p.wc, wr = p.r0 + row % p.wc;
     lse_out[((int64_t)bl * p.Hq + hq) * p.w + wr] = Z > 0.f ? l2 * 0.6931471805599453f : -INFINITY;
   }
 }
 
-// caller-supplied natural-log sum-exps [B, L, H_q, w] -> negated log2-domain values in the (unit, row) layout of pass 2;
-// a row that saw no key (-inf) and the padding rows get the shift that turns every weight into 0
-__global__ void score_rows_given_lse_kernel(RowParams p, const float* lse, float* nlse2, int total) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= total) return;
-  const int u = x / p.rs, row = x % p.rs;
-  clear_tail(p, u, row);
-  float v = kEmptyMax;
-  if (row < p.R) {
-    const int h = u % p.Hkv, bl = u / p.Hkv;
-    const int hq = h * p.g + row / p.w, wr = row % p.w;
-    const float l = lse[((int64_t)bl * p.Hq + hq) * p.w + wr];
-    if (l > -INFINITY) v = -l * kLog2e;
-  }
-  nlse2[x] = v;
-}
-
-template <int D, int PASS>
+template <int D, int PASS, int NS>
 int launch_pass(const CUtensorMap& mk, const CUtensorMap& mq, const RowParams& p, int grid, cudaStream_t st) {
-  using SL = RowSmem<D, PASS>;
-  if (cudaFuncSetAttribute(score_rows_kernel<D, PASS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SL::kAlloc) !=
+  using SL = RowSmem<D, PASS, NS>;
+  if (cudaFuncSetAttribute(score_rows_kernel<D, PASS, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SL::kAlloc) !=
       cudaSuccess)
     return MADAKV_ECUDA;
-  score_rows_kernel<D, PASS><<<grid, kRowThreads, SL::kAlloc, st>>>(mk, mq, p);
+  launch_pdl(score_rows_kernel<D, PASS, NS>, dim3(grid), dim3(kRowThreads), (size_t)SL::kAlloc, st, mk, mq, p);
   return MADAKV_OK;
 }
+template <int PASS>
+int launch_pass(const madakv_config& c, const CUtensorMap& mk, const CUtensorMap& mq, const RowParams& p, int grid, cudaStream_t st) {
+  if (c.dtype == MADAKV_F32)
+    return c.head_dim == 128 ? launch_pass<128, PASS, 3>(mk, mq, p, grid, st) : launch_pass<64, PASS, 3>(mk, mq, p, grid, st);
+  return c.head_dim == 128 ? launch_pass<128, PASS, 1>(mk, mq, p, grid, st) : launch_pass<64, PASS, 1>(mk, mq, p, grid, st);
+}
 
-}  // namespace
+// ---- fp32 operands -> three bf16 terms each, whose sum is the operand exactly (8 significand bits per term)
+struct SplitParams {
+  const float* src;
+  __nv_bfloat16* dst;  // [rows of the slice][3][D]
+  const int32_t* seq_len;
+  madakv_strides s;    // of src, in elements
+  int L, H, D, tokens, head0;  // head0: first head of the slice; seq_len: nullptr = all tokens
+};
+// (blocks: first the keys' heads, k_blocks each, then the queries')
+__global__ void __launch_bounds__(256) split_kernel(SplitParams pk, SplitParams pq, int k_heads, int k_blocks, int q_blocks) {
+  pdl_wait();
+  pdl_go();
+  int bx = (int)blockIdx.x;
+  const bool is_q = bx >= k_heads * k_blocks;
+  if (is_q) bx -= k_heads * k_blocks;
+  const SplitParams& p = is_q ? pq : pk;
+  const int per = is_q ? q_blocks : k_blocks, y = bx / per;
+  const int lg = p.D == 128 ? 5 : 4;  // 16-byte pieces per row: 32 or 16
+  const int x = (bx - y * per) * 256 + threadIdx.x, tok = x >> lg, c = (x & ((1 << lg) - 1)) * 4;
+  const int hh = y + p.head0;  // head of the call, counted over (sequence, layer, head)
+  const int h = hh % p.H, l = hh / p.H % p.L, b = hh / (p.H * p.L);
+  if (tok >= (p.seq_len ? clamped_len(p.seq_len, b, p.tokens) : p.tokens)) return;  // (keys beyond the sequence are masked)
+  const int64_t row = (int64_t)y * p.tokens + tok;
+  const float4 v = __ldg(reinterpret_cast<const float4*>(p.src + b * p.s.batch + l * p.s.layer + h * p.s.head + tok * p.s.token + c));
+  const float f[4] = {v.x, v.y, v.z, v.w};
+  uint32_t t[3][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float r = f[i];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      uint32_t hi = __float_as_uint(__bfloat162float(__float2bfloat16_rn(r)));
+      if ((hi & 0x7fffffffu) == 0x7f800000u) hi = __float_as_uint(r) & 0xffff0000u;  // (rounded up to infinity: cut off instead)
+      t[k][i] = hi >> 16;
+      r = __fsub_rn(r, __uint_as_float(hi));
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    *reinterpret_cast<uint2*>(p.dst + (row * 3 + k) * p.D + c) = make_uint2(t[k][0] | (t[k][1] << 16), t[k][2] | (t[k][3] << 16));
+}
 
-// parameters shared by the two-pass and the single-pass launch; false if the shape is outside this file's range
-static bool rows_setup(const madakv_config& c, const void* q, madakv_strides sq, const void* k, madakv_strides sk,
-                       const int32_t* seq_len, float* psi, void* ws, RowParams& p, float*& lse2, CUtensorMap& mk,
-                       CUtensorMap& mq, int& grid, int& rc) {
-  const int g = c.n_q_heads / c.n_kv_heads;
-  const int R = g * c.window;
-  rc = MADAKV_EUNSUPPORTED;
-  if (c.dtype != MADAKV_BF16 || R > 256 || c.window > 256 || g > 256) return false;
+// One slice of the units (bf16: all of them), window rows chunk by chunk. given_lse: single pass with supplied log-sum-exps.
+struct Slice {
+  int b0, B, u0, lh;  // first sequence, sequences, first unit, units per sequence
+};
+int score_slice(const madakv_config& c, const Slice& sl, const void* q, madakv_strides sq, const void* k, madakv_strides sk,
+                const int32_t* seq_len, const float* given_lse, float* lse, float* psi, void* ws, cudaStream_t st) {
   const WsLayout wl = ws_layout(c);
-  p.seq_len = seq_len;
-  p.psi = psi;
+  const bool f32 = c.dtype == MADAKV_F32;
+  const int g = c.n_q_heads / c.n_kv_heads, d = c.head_dim;
+  RowParams p;
+  p.seq_len = seq_len + sl.b0;
+  p.psi = psi + (int64_t)sl.u0 * c.max_seq_len;
   p.part = reinterpret_cast<float2*>((char*)ws + wl.score_part_off);
-  lse2 = reinterpret_cast<float*>((char*)ws + wl.score_lse_off);
+  float* lse2 = reinterpret_cast<float*>((char*)ws + wl.score_lse_off);
   p.lse2 = lse2;
   p.status = reinterpret_cast<int32_t*>(ws);
-  p.B = c.batch;
-  p.units = c.batch * c.n_layers * c.n_kv_heads;
+  p.B = sl.B;
+  p.units = sl.B * sl.lh;
+  p.lh = sl.lh;
+  p.u0 = sl.u0;
   p.L = c.n_layers;
   p.Hq = c.n_q_heads;
   p.Hkv = c.n_kv_heads;
   p.g = g;
   p.w = c.window;
-  p.R = R;
   p.n_max = c.max_seq_len;
   p.causal = c.causal;
-  p.smax = wide_max_runs(c);
-  p.rs = (R + 31) / 32 * 32;  // row stride of the workspace arrays
-  p.mblocks = R <= 128 ? 1 : 2;
-  p.cparts = R <= 128 ? 4 : 2;
-  p.n16 = (R + 15) / 16 * 16;
+  p.smax = wide_max_runs(sl.lh, c.max_seq_len);
   p.scale2 = scale_of(c) * kLog2e;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    rc = MADAKV_ECUDA;
-    return false;
-  }
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return MADAKV_ECUDA;
   const long long tiles = (long long)p.units * ((c.max_seq_len + kTileKeys - 1) / kTileKeys);
-  if (tiles > 0x3fffffff) return false;
+  if (tiles > 0x3fffffff) return MADAKV_EUNSUPPORTED;
   if (sms > kWideMaxGrid) sms = kWideMaxGrid;
-  grid = (int)(tiles < sms ? tiles : sms);
+  const int grid = (int)(tiles < sms ? tiles : sms);
   p.grid = grid;
-  if (!make_map(&mk, k, c.head_dim, c.max_seq_len, c.n_kv_heads, c.n_layers, c.batch, sk, kTileKeys, 1) ||
-      !make_map(&mq, q, c.head_dim, c.window, c.n_q_heads, c.n_layers, c.batch, sq, c.window, g))
-    return false;
-  return true;
+  CUtensorMap mk, mq;
+  const madakv_strides split_k{0, 0, (int64_t)c.max_seq_len * 3 * d, 3 * d}, split_q{0, 0, (int64_t)c.window * 3 * d, 3 * d};
+  if (f32) {
+    __nv_bfloat16* ks = reinterpret_cast<__nv_bfloat16*>((char*)ws + wl.score_split_off);
+    __nv_bfloat16* qs = ks + (int64_t)p.units * c.max_seq_len * 3 * d;
+    if (!make_map(&mk, ks, 3 * d, c.max_seq_len, p.units, 1, 1, split_k, kTileKeys, 1)) return MADAKV_EUNSUPPORTED;
+    SplitParams x{(const float*)k, ks, seq_len, sk, c.n_layers, c.n_kv_heads, d, c.max_seq_len, sl.u0};
+    SplitParams y{(const float*)q, qs, nullptr, sq, c.n_layers, c.n_q_heads, d, c.window, sl.u0 * g};
+    const int kb = (c.max_seq_len * (d / 4) + 255) / 256, qb = (c.window * (d / 4) + 255) / 256;
+    launch_pdl(split_kernel, dim3((unsigned)(p.units * (kb + g * qb))), dim3(256), 0, st, x, y, p.units, kb, qb);
+    q = qs;
+  } else if (!make_map(&mk, k, d, c.max_seq_len, c.n_kv_heads, c.n_layers, c.batch, sk, kTileKeys, 1)) {
+    return MADAKV_EUNSUPPORTED;
+  }
+  const int rows_max = f32 ? 128 : 256;
+  // chunks of equal size as far as possible (7 heads of 64 rows: 4 + 3)
+  const int heads_max = c.window < rows_max ? rows_max / c.window : 1, head_chunks = (g + heads_max - 1) / heads_max;
+  const int row_chunks = (c.window + rows_max - 1) / rows_max;
+  const int hc = (g + head_chunks - 1) / head_chunks, rc = (c.window + row_chunks - 1) / row_chunks;
+  p.accumulate = 0;
+  for (p.h0 = 0; p.h0 < g; p.h0 += hc)
+    for (p.r0 = 0; p.r0 < c.window; p.r0 += rc) {
+      const int heads = g - p.h0 < hc ? g - p.h0 : hc;
+      p.wc = c.window - p.r0 < rc ? c.window - p.r0 : rc;
+      p.R = heads * p.wc;
+      p.rs = (p.R + 31) / 32 * 32;  // row stride of the workspace arrays
+      p.mblocks = p.R <= 128 ? 1 : 2;
+      p.cparts = p.R <= 128 ? 4 : 2;
+      p.n16 = (p.R + 15) / 16 * 16;
+      if (!(f32 ? make_map(&mq, q, 3 * d, c.window, p.units * g, 1, 1, split_q, p.wc, heads)
+                : make_map(&mq, q, d, c.window, c.n_q_heads, c.n_layers, c.batch, sq, p.wc, heads)))
+        return MADAKV_EUNSUPPORTED;
+      p.given_lse = given_lse;
+      int rc2;
+      if (!given_lse) {
+        if ((rc2 = launch_pass<1>(c, mk, mq, p, grid, st))) return rc2;
+        launch_pdl(score_rows_merge_kernel, dim3(p.units * (p.rs / 32)), dim3(256), 0, st, p, lse2, lse);
+      }
+      if ((rc2 = launch_pass<2>(c, mk, mq, p, grid, st))) return rc2;
+      p.accumulate = 1;
+    }
+  return launch_status();
 }
+
+// fp32: slices whose split operands fit the workspace's area, whole sequences or a part of one
+int score_slices(const madakv_config& c, const void* q, madakv_strides sq, const void* k, madakv_strides sk, const int32_t* seq_len,
+                 const float* given_lse, float* lse, float* psi, void* ws, cudaStream_t st) {
+  const int lh = c.n_layers * c.n_kv_heads;
+  if (c.dtype != MADAKV_F32)
+    return score_slice(c, Slice{0, c.batch, 0, lh}, q, sq, k, sk, seq_len, given_lse, lse, psi, ws, st);
+  const int most = split_units(c);  // units per slice
+  if (most >= lh) {
+    for (int b = 0; b < c.batch; b += most / lh) {
+      const int nb = c.batch - b < most / lh ? c.batch - b : most / lh;
+      const int rc = score_slice(c, Slice{b, nb, b * lh, lh}, q, sq, k, sk, seq_len, given_lse, lse, psi, ws, st);
+      if (rc) return rc;
+    }
+    return MADAKV_OK;
+  }
+  for (int b = 0; b < c.batch; ++b)
+    for (int u = 0; u < lh; u += most) {
+      const int rc = score_slice(c, Slice{b, 1, b * lh + u, lh - u < most ? lh - u : most}, q, sq, k, sk, seq_len, given_lse, lse, psi, ws, st);
+      if (rc) return rc;
+    }
+  return MADAKV_OK;
+}
+
+}  // namespace
 
 int launch_score_rows(const madakv_config& c, const void* q, madakv_strides sq, const void* k, madakv_strides sk,
                       const int32_t* seq_len, float* lse, float* psi, void* ws, cudaStream_t st) {
-  if ((c.n_q_heads / c.n_kv_heads) * c.window <= 64) return MADAKV_EUNSUPPORTED;  // the TMEM-resident kernels' range
-  RowParams p;
-  float* lse2;
-  CUtensorMap mk, mq;
-  int grid, rc;
-  // the workspace layout reserves (max, sum) pairs for [units, splits, column shares, rs]
-  if (!rows_setup(c, q, sq, k, sk, seq_len, psi, ws, p, lse2, mk, mq, grid, rc)) return rc;
-  const int total = p.units * p.rs;
-  rc = c.head_dim == 128 ? launch_pass<128, 1>(mk, mq, p, grid, st) : launch_pass<64, 1>(mk, mq, p, grid, st);
-  if (rc) return rc;
-  score_rows_merge_kernel<<<(total + 255) / 256, 256, 0, st>>>(p, lse2, lse, total);
-  rc = c.head_dim == 128 ? launch_pass<128, 2>(mk, mq, p, grid, st) : launch_pass<64, 2>(mk, mq, p, grid, st);
-  if (rc) return rc;
-  return launch_status();
+  return score_slices(c, q, sq, k, sk, seq_len, nullptr, lse, psi, ws, st);
 }
 
 // Single-pass scoring with the rows' log-sum-exps supplied by the caller: a conversion kernel, then pass 2 alone.
-// Any bf16 shape with g * w <= 256.
 int launch_score_lse_rows(const madakv_config& c, const void* q, madakv_strides sq, const void* k, madakv_strides sk,
                           const int32_t* seq_len, const float* lse, float* psi, void* ws, cudaStream_t st) {
-  RowParams p;
-  float* lse2;
-  CUtensorMap mk, mq;
-  int grid, rc;
-  if (!rows_setup(c, q, sq, k, sk, seq_len, psi, ws, p, lse2, mk, mq, grid, rc)) return rc;
-  const int total = p.units * p.rs;
-  score_rows_given_lse_kernel<<<(total + 255) / 256, 256, 0, st>>>(p, lse, lse2, total);
-  rc = c.head_dim == 128 ? launch_pass<128, 2>(mk, mq, p, grid, st) : launch_pass<64, 2>(mk, mq, p, grid, st);
-  if (rc) return rc;
-  return launch_status();
+  return score_slices(c, q, sq, k, sk, seq_len, lse, nullptr, psi, ws, st);
 }
 
 }  // namespace madakv

@@ -126,6 +126,34 @@ def test_single_pass_score_with_given_lse(name, causal, path, monkeypatch):
     assert psi_close(buf.psi.cpu().numpy(), two.psi.cpu().numpy().astype(np.float64), 1e-4) < 1e-4
 
 
+# chunks of query heads and of window rows (more than 256 rows per KV head, fp32: 128), and fp32 calls whose split operands come
+# in slices: parts of a sequence, whole sequences, one unit that is larger than a slice would be
+@pytest.mark.parametrize("dtype,B,L,Hq,Hkv,d,n,w", [
+    ("bf16", 1, 2, 7, 1, 128, 300, 48), ("bf16", 2, 1, 10, 2, 64, 777, 64), ("bf16", 1, 1, 2, 1, 128, 700, 300),
+    ("f32", 2, 1, 6, 2, 64, 389, 50), ("f32", 1, 1, 2, 1, 128, 400, 131), ("f32", 1, 70, 1, 1, 128, 2000, 8),
+    ("f32", 3, 8, 10, 5, 128, 2001, 5), ("f32", 1, 2, 1, 1, 64, 129, 128)])
+@pytest.mark.parametrize("causal", [1, 0])
+def test_score_in_chunks_and_slices(dtype, B, L, Hq, Hkv, d, n, w, causal):
+    wl = synth.scaled(TINY, dtype=dtype, B=B, L=L, Hq=Hq, Hkv=Hkv, d=d, n=n, w=w, layout="blocks70", budget=n // 5)
+    q = synth.make_q_win(wl)
+    k = synth.hash_normal(3, 5, 0, B * L * Hkv * n * d).view(B, L, Hkv, n, d).to(wl.torch_dtype)
+    sl = np.array([n - 61 * b for b in range(B)], np.int32)
+    cfg = config_of(wl, causal=causal)
+    lse = torch.zeros((B, L, Hq, w), device="cuda")
+    psi = torch.full((B, L, Hkv, n), -1.0, device="cuda")
+    ws = mk.new_workspace(cfg)
+    d_q, d_k, d_sl = q.cuda(), k.cuda(), torch.from_numpy(sl).cuda()
+    mk.madakv_score(cfg, d_q, d_k, d_sl, lse, psi, ws)
+    assert mk.madakv_poll_status(ws) == 0
+    want, want_lse = oracle.score(dcode(wl), to_np(q), to_np(k), sl, causal=causal, want_lse=True)
+    assert psi_close(psi.cpu().numpy(), want, PSI_RTOL) < PSI_RTOL_SEEN
+    assert np.abs(lse.cpu().numpy() - want_lse).max() <= 1e-5 * np.abs(want_lse).max()
+    psi.fill_(-1.0)
+    mk.madakv_score_lse(cfg, d_q, d_k, d_sl, lse, psi, ws)
+    assert mk.madakv_poll_status(ws) == 0
+    assert psi_close(psi.cpu().numpy(), want, PSI_RTOL) < PSI_RTOL_SEEN
+
+
 @pytest.mark.parametrize("lag", ["8", "9", "40", "1000"])
 def test_tensor_core_score_item_interleaving(lag, monkeypatch):
     # many more work items than the phase-1 lead: exercises the interleaved phase-2 / phase-1 item order and the
