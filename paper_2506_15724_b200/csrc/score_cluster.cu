@@ -1,20 +1,25 @@
 // Stage 1, TMEM-resident tensor-core path (Eq. 7 with the softmax of Eq. 5) for bf16 inputs with g * w <= 64 window
-// rows and sequences short enough that all logits of one unit fit the tensor memory of a thread-block cluster.
+// rows, for sequences whose logits fit the tensor memory of a thread-block cluster, or do so for the larger part (kLong).
 //
 // A softmax over keys needs every window row's log-sum-exp over ALL keys before any normalised weight can be summed
 // over rows. Here the logits are not recomputed for that second step: a cluster of C CTAs (C SMs) takes one unit
 // (sequence, layer, KV head) at a time, CTA r computes the window-QK^T tiles of its share of the keys with tcgen05.mma
 // (128 keys of a tile on M, the g*w window rows on N, head_dim on K; operands by TMA, 128-byte swizzle) and KEEPS all
 // its fp32 accumulators in TMEM (512 columns = 16 tiles of 32 rows or 8 tiles of 64 rows). The epilogue warps read
-// them from TMEM as they arrive for the rows' (max, sum of exp2) statistics (one sweep against a per-lane reference
-// logit for up to 32 rows, with an exact fallback; a maximum sweep and a sum sweep for 64), and once more when the (max, sum) pairs of all warps of the
+// them from TMEM as they arrive for the rows' (max, sum of exp2) statistics (one sweep against reference logits: per lane for
+// up to 32 rows, per warp for 64; a reference is raised, or the sweep repeated exactly, when a logit lies far above it), and once more when the (max, sum) pairs of all warps of the
 // cluster have been exchanged through distributed shared memory and merged into the rows' log-sum-exps, for the
 // weights exp2(s - lse) whose sum over rows is psi. So K is read from HBM exactly once and each tile takes one MMA pass.
 //
+// Longer sequences (kLong): a CTA's first tiles, those beyond the number of its TMEM slots, pass through the slots for the
+// statistics, and are loaded (from the L2 as long as 15 clusters' worth of them fits there) and multiplied once more after the
+// resident ones have been read for the last time. 1024 units of 20480 keys, 32 rows, take 1.16 ms like this where two
+// passes over K take 1.7 and the two-phase kernel 1.56.
+//
 // Warp roles per CTA: warp 0 TMA producer, warp 1 MMA issuer and TMEM owner, warps 2-9 epilogue (two groups of four
 // warps = the four TMEM lane quarters; group e takes the CTA's tiles of parity e; a thread owns one key of a tile and
-// all window rows of it). The TMEM slots form a ring over the CTA's tiles of consecutive units and a tile's slot is
-// handed back to the MMA warp after its last read: when a unit leaves slots free, the MMAs of the next unit run ahead
+// all window rows of it). The TMEM slots form a ring over the CTA's tiles of consecutive units (entry e of the CTA's running
+// count of accumulator tiles uses slot e mod kSlots) and a tile's slot is handed back to the MMA warp after its last read: when a unit leaves slots free, the MMAs of the next unit run ahead
 // into them during this unit's exchange and last sweep, and the TMA ring runs ahead with them.
 // Synchronisation between CTAs exists only inside a cluster (whose CTAs are co-scheduled by the hardware): every lane
 // of every epilogue warp sends its rows' pairs into each peer's shared memory with asynchronous stores that count
@@ -27,6 +32,7 @@ namespace {
 
 constexpr int kClThreads = 320;  // TMA warp, MMA warp, 8 epilogue warps
 constexpr int kMaxCluster = 8;
+constexpr int kLongCluster = 6;
 enum { kSiteStats = 9 };
 
 struct ClParams {
@@ -35,7 +41,6 @@ struct ClParams {
   float* lse_out;   // natural log [B,L,Hq,w] or null
   int32_t* status;  // ws header
   int units, L, Hq, Hkv, g, w, R, n_max, causal, C;
-  int per_max;  // most tiles a CTA gets of one unit (at most the number of TMEM slots)
   float scale2;
 };
 
@@ -81,6 +86,18 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// A logit may lie this many binades above its reference: sums of up to 2^20 such terms stay far inside the fp32 range.
+constexpr float kMaxExponent = 64.f;
+// the largest of a block's 16 exponents
+__device__ __forceinline__ float block_max_exponent(const uint32_t (&raw)[16], uint64_t scale2x, const uint64_t* negshift2) {
+  float v[16];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) unpack2(fma2(pack2u(raw[2 * i], raw[2 * i + 1]), scale2x, negshift2[i]), v[2 * i], v[2 * i + 1]);
+  const float a = max3f(v[0], v[1], v[2]), b = max3f(v[3], v[4], v[5]), c = max3f(v[6], v[7], v[8]);
+  const float d = max3f(v[9], v[10], v[11]), e = max3f(v[12], v[13], v[14]);
+  return max3f(max3f(a, b, c), max3f(d, e, v[15]), v[15]);
+}
+
 template <int D, int NPAD>
 struct ClSmem {
   static constexpr int kStages = NPAD == 32 ? (D == 128 ? 5 : 10) : (D == 128 ? 3 : 6);  // 160 KB or 96 KB of K in flight
@@ -94,7 +111,7 @@ struct ClSmem {
   // full[kStages], qfull[2], qempty[2], tfull[kSlots], tempty[kSlots], stats[2], drain[1]
   static constexpr int kNumBars = kStages + 4 + 2 * kSlots + 3;
   static constexpr int kMiscOff = kBarOff + kNumBars * 8;
-  // misc: tmem base (4), abort flag (4), producer's stage ring (kStages <= 10 words)
+  // misc: tmem base (4), abort flag (4)
   static constexpr int kWarpOff = kMiscOff + 48;
   // per epilogue warp: shift[NPAD], vis[NPAD]
   static constexpr int kWarpBytes = NPAD * 4 + NPAD * 4;
@@ -104,7 +121,7 @@ struct ClSmem {
   static constexpr int alloc_bytes(int C) { return kStatsOff + stats_bytes(C) + 1024; }
 };
 
-template <int D, int NPAD>
+template <int D, int NPAD, bool kLong>
 __global__ void __launch_bounds__(kClThreads, 1)
 score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_q, ClParams p) {
   using SL = ClSmem<D, NPAD>;
@@ -163,6 +180,8 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
   __syncthreads();
   tc_fence_after();
   cluster_sync_all();  // the peers' barriers are initialised before anyone arrives on them
+  pdl_wait();          // (nothing above touches global memory: it overlaps the kernel before this one)
+  pdl_go();
   const uint32_t tmem_base = *tmem_base_s;
 
   // the tiles of unit u that belong to this CTA: [tile0, tile0 + my_tiles) of the unit's ceil(n / 128) tiles
@@ -172,24 +191,24 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
     tile0 = rank * per;
     my_tiles = max(0, min(per, tiles - tile0));
   };
-  // TMEM slots are a ring over the CTA's tiles of consecutive units: every role keeps the same running position
-  // (`ring`: slot of the current unit's first tile) and advances it by the unit's tile count.
-  auto slot_at = [&](int ring, int jj) { return (ring + jj) & (kSlots - 1); };
+  // Every role counts the accumulator tiles ("entries") of the CTA over its units. A unit of my_tiles tiles has
+  // my_tiles + again entries: its tiles in order, then the first `again` ones once more, those whose slots are needed before
+  // the last read (kLong only; else all fit).
+  auto passes_again = [&](int my_tiles) { return kLong ? max(0, my_tiles - kSlots) : 0; };
+  auto slot_of = [](uint32_t e) { return (int)(e & (uint32_t)(kSlots - 1)); };
+  auto par_of = [](uint32_t e) { return (e / (uint32_t)kSlots) & 1u; };  // parity of the use of its slot
   static_assert((kSlots & (kSlots - 1)) == 0, "slot ring uses a power-of-two mask");
+  static_assert(kStages < kSlots, "a slot comes round less often than a K stage");
 
   if (warp == 0) {
     // ================================================================ TMA producer
     if (lane == 0) {
-      const uint64_t pol = l2_policy_evict_first();  // K is read once
-      const uint64_t pol_q = l2_policy_evict_last();
-      // A K stage may be refilled once the MMAs of the tile that used it last have completed: that is the tile's
-      // tfull barrier. stage_user remembers the slot, slot_par the parity of the slot's latest use by this thread
-      // (a slot comes round every kSlots tiles, a stage every kStages < kSlots tiles, so the latest use of the slot
-      // is the use that read the stage).
-      volatile uint32_t* stage_user = reinterpret_cast<volatile uint32_t*>(smem + SL::kMiscOff + 8);
-      for (int s2 = 0; s2 < kStages; ++s2) stage_user[s2] = 0;
-      uint32_t slot_par = 0, slot_used = 0;
-      int stage = 0, qi = 0, ring = 0;
+      const uint64_t pol = l2_policy_evict_first();
+      const uint64_t pol_q = l2_policy_evict_last();  // queries, and the tiles that are read again
+      // A K stage may be refilled once the MMAs of the entry that used it last have completed: that is the entry's tfull
+      // barrier (its slot's next use is not loaded yet, so the barrier is at most in the phase after that).
+      uint32_t e = 0;
+      int stage = 0, qi = 0;
       uint32_t q_par = 0;
       bool ok = true;
       for (int u = cluster; ok && u < p.units; u += n_clusters) {
@@ -198,8 +217,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
         int tile0, my_tiles;
         my_share(n, tile0, my_tiles);
         if (my_tiles == 0) continue;
-        const int sb = ring;
-        ring = slot_at(ring, my_tiles);
+        const int again = passes_again(my_tiles);
         ok = mbar_wait(&qempty[qi], q_par ^ 1, abort_flag, p.status, kSiteQEmpty);
         if (!ok) break;
         mbar_expect_tx(&qfull[qi], (uint32_t)(p.R * 128 * kKBlocks));
@@ -207,20 +225,15 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
           tma_load_5d(q_s + qi * SL::kQBytes + kb * NPAD * 128, &tmap_q, &qfull[qi], kb * 64, 0, h * p.g, l, b, pol_q);
         qi ^= 1;
         if (qi == 0) q_par ^= 1;
-        for (int jj = 0; jj < my_tiles; ++jj) {
-          const int j = slot_at(sb, jj);
-          const uint32_t prev = stage_user[stage];
-          if (prev & 0x200u)
-            ok = mbar_wait(&tfull[prev & 0xffu], (slot_par >> (prev & 0xffu)) & 1u, abort_flag, p.status, kSiteStage);
+        for (int x = 0; x < my_tiles + again; ++x, ++e) {
+          const int jj = x < my_tiles ? x : x - my_tiles;
+          if (e >= (uint32_t)kStages)
+            ok = mbar_wait(&tfull[slot_of(e - kStages)], par_of(e - kStages), abort_flag, p.status, kSiteStage);
           if (!ok) break;
-          // parity of this use of slot j: uses of a slot alternate 0, 1, 0, ...
-          if (slot_used & (1u << j)) slot_par ^= 1u << j;
-          slot_used |= 1u << j;
-          stage_user[stage] = (uint32_t)j | 0x200u;
           mbar_expect_tx(&full[stage], (uint32_t)SL::kStageBytes);
           for (int kb = 0; kb < kKBlocks; ++kb)
             tma_load_5d(k_s + stage * SL::kStageBytes + kb * kTileKeys * 128, &tmap_k, &full[stage], kb * 64,
-                        (tile0 + jj) * kTileKeys, h, l, b, pol);
+                        (tile0 + jj) * kTileKeys, h, l, b, x < again ? pol_q : pol);
           if (++stage == kStages) stage = 0;
         }
       }
@@ -234,8 +247,8 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
     if (lane == 0) {
       constexpr uint32_t idesc = instr_desc_bf16(NPAD);
       const uint32_t k_lo0 = smem_desc_lo(smem_u32(k_s)), q_lo0 = smem_desc_lo(smem_u32(q_s));
-      uint32_t slot_par = 0, slot_used = 0;  // parity of the current use of every slot
-      int stage = 0, qi = 0, ring = 0;
+      uint32_t e = 0;
+      int stage = 0, qi = 0;
       uint32_t stage_par = 0, q_par = 0;
       bool ok = true;
       for (int u = cluster; ok && u < p.units; u += n_clusters) {
@@ -244,16 +257,12 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
         int tile0, my_tiles;
         my_share(n, tile0, my_tiles);
         if (my_tiles == 0) continue;
-        const int sb = ring;
-        ring = slot_at(ring, my_tiles);
         ok = mbar_wait(&qfull[qi], q_par, abort_flag, p.status, kSiteQFull);
         if (!ok) break;
         const uint32_t q_lo = q_lo0 + (uint32_t)qi * (SL::kQBytes >> 4);
-        for (int jj = 0; jj < my_tiles; ++jj) {
-          const int j = slot_at(sb, jj);
-          if (slot_used & (1u << j)) slot_par ^= 1u << j;
-          slot_used |= 1u << j;
-          const uint32_t use_par = (slot_par >> j) & 1u;
+        for (int x = my_tiles + passes_again(my_tiles); x > 0; --x, ++e) {
+          const int j = slot_of(e);
+          const uint32_t use_par = par_of(e);
           // the slot's previous accumulator must have been read for the last time, and the K tile must have landed
           ok = mbar_wait(&tempty[j], use_par ^ 1, abort_flag, p.status, kSiteTEmpty) &&
                mbar_wait(&full[stage], stage_par, abort_flag, p.status, kSiteFull);
@@ -297,9 +306,8 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
     const uint64_t* shift2 = reinterpret_cast<const uint64_t*>(shift_s);
     const uint64_t scale2x = pack2(p.scale2, p.scale2);
     const uint32_t tlane = tmem_base + ((uint32_t)(quarter * 32) << 16);
-    uint32_t slot_par = 0, slot_used = 0;  // parity of the current use of every slot
+    uint32_t e0 = 0;                       // the unit's first entry
     uint32_t unit_par = 0;                 // parity of the units this cluster has taken
-    int ring = 0;
     // what depends on the sequence only is kept from unit to unit (the units of a sequence follow one another)
     int b = -1, b_end = 0, n = 0, tile0 = 0, my_tiles = 0, all_bound = 0, tiles_end = 0;
     bool ok = true;
@@ -326,95 +334,57 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
       }
       float* psi = p.psi + (int64_t)u * p.n_max;
       const int cnt = my_tiles > grp ? (my_tiles - grp + 1) / 2 : 0;  // this group's tiles: grp, grp + 2, ...
-      const int sb = ring;
-      ring = slot_at(ring, my_tiles);
+      const int again = passes_again(my_tiles);
+      const uint32_t eb = e0;
+      e0 += (uint32_t)(my_tiles + again);
       if (rank == 0) {  // positions beyond the unit's last tile
         for (int key = tiles_end + ew * 32 + lane; key < p.n_max; key += 256) psi[key] = 0.f;
       }
-      {  // parity of this use of the unit's slots (either group's: a slot serves tiles of both groups as the ring
-         // moves on): the slots [sb, sb + my_tiles) of the ring as a bit mask
-        const uint32_t run = my_tiles >= 32 ? 0xffffffffu : (1u << my_tiles) - 1u;
-        const uint32_t all = kSlots >= 32 ? 0xffffffffu : (1u << kSlots) - 1u;
-        const uint32_t used_now = ((run << sb) | (run >> ((kSlots - sb) & 31))) & all;
-        slot_par ^= used_now & slot_used;
-        slot_used |= used_now;
-      }
-      auto wait_tile = [&](int i) -> bool {
-        const int j = slot_at(sb, grp + 2 * i);
-        const bool w_ok =
-            __all_sync(0xffffffffu, mbar_wait(&tfull[j], (slot_par >> j) & 1u, abort_flag, p.status, kSiteTile));
+      auto wait_tile = [&](int x) -> bool {  // entry x of the unit
+        const bool w_ok = __all_sync(
+            0xffffffffu, mbar_wait(&tfull[slot_of(eb + x)], par_of(eb + x), abort_flag, p.status, kSiteTile));
         tc_fence_after();
         return w_ok;
       };
-      auto release_tile = [&](int i) {
+      auto release_tile = [&](int x) {
         tc_fence_before();
-        mbar_arrive(&tempty[slot_at(sb, grp + 2 * i)]);
+        mbar_arrive(&tempty[slot_of(eb + x)]);
       };
-      // The group's tiles are read in blocks of 16 window rows (16 TMEM columns); the load of the next block is in
-      // flight while the current one is processed. `body(j, r, i)` gets block j of the group's i-th tile.
-      auto sweep = [&](auto before_tile, auto body) -> bool {
-        if (cnt == 0) return true;
+      // The group's entries x in [from, to) are read in blocks of 16 window rows (16 TMEM columns); the load of the next block
+      // is in flight while the current one is processed. `body(j, r, x)` gets block j of entry x.
+      auto sweep = [&](int from, int to, auto before_tile, auto body) -> bool {
+        const int x0 = from + ((from ^ grp) & 1);
+        if (x0 >= to) return true;
         uint32_t ra[16], rb[16];
-        if (!before_tile(0)) return false;
-        tmem_ld16_issue(tlane + slot_at(sb, grp) * NPAD, ra);
-        for (int i = 0; i < cnt; ++i) {
-          const uint32_t taddr = tlane + slot_at(sb, grp + 2 * i) * NPAD;
+        if (!before_tile(x0)) return false;
+        tmem_ld16_issue(tlane + slot_of(eb + x0) * NPAD, ra);
+        for (int x = x0; x < to; x += 2) {
+          const uint32_t taddr = tlane + slot_of(eb + x) * NPAD;
 #pragma unroll
           for (int j = 0; j < kBlocks; j += 2) {
             tmem_ld_wait16(ra);
             tmem_ld16_issue(taddr + (j + 1) * 16, rb);
-            body(j, ra, i);
+            body(j, ra, x);
             tmem_ld_wait16(rb);
             if (j + 2 < kBlocks) {
               tmem_ld16_issue(taddr + (j + 2) * 16, ra);
-            } else if (i + 1 < cnt) {
-              if (!before_tile(i + 1)) return false;
-              tmem_ld16_issue(tlane + slot_at(sb, grp + 2 * i + 2) * NPAD, ra);
+            } else if (x + 2 < to) {
+              if (!before_tile(x + 2)) return false;
+              tmem_ld16_issue(tlane + slot_of(eb + x + 2) * NPAD, ra);
             }
-            body(j + 1, rb, i);
+            body(j + 1, rb, x);
           }
         }
         return true;
       };
 
       uint64_t z2[NPAD / 2];
-      // Exact statistics in two sweeps: the warp's maximum per row, then the sum of exp2 against it. The (negated,
-      // scaled) maxima are uniform over the warp: they go to the warp's shift_s and are read back as packed pairs.
-      auto exact_stats = [&]() -> bool {
-        float st_m[NPAD];
-#pragma unroll
-        for (int c = 0; c < NPAD; ++c) st_m[c] = kEmptyMax;
-        const bool s_ok = sweep([&](int i) { return wait_tile(i); },
-                                [&](int j, uint32_t (&r)[16], int i) {
-                                  const int key0 = (tile0 + grp + 2 * i) * kTileKeys;
-                                  if (key0 + kTileKeys > all_bound) mask_block16(r, key0 + et, vis_s + j * 16);
-#pragma unroll
-                                  for (int c = 0; c < 16; ++c)
-                                    st_m[j * 16 + c] = fmaxf(st_m[j * 16 + c], __uint_as_float(r[c]));
-                                });
-        if (!s_ok) return false;
-        __syncwarp();
-#pragma unroll
-        for (int c = 0; c < NPAD; ++c) {
-          const float wm = warp_max(st_m[c]);
-          if (lane == (c & 31)) shift_s[c] = -(wm * p.scale2);
-        }
-#pragma unroll
-        for (int i = 0; i < NPAD / 2; ++i) z2[i] = 0ull;
-        __syncwarp();
-        sweep([&](int) { return true; },
-              [&](int j, uint32_t (&r)[16], int i) {
-                const int key0 = (tile0 + grp + 2 * i) * kTileKeys;
-                if (key0 + kTileKeys > all_bound) mask_block16(r, key0 + et, vis_s + j * 16);
-                exp_accumulate16(r, scale2x, shift2 + j * 8, z2 + j * 8);
-              });
-        return true;
-      };
       if constexpr (NPAD == 32) {
         // One sweep as the tiles arrive: every lane takes, per window row, its logit of the group's first tile as the
         // reference and sums exp2(s - reference) over its keys (the reference's own term is 1). No maximum is needed
-        // as long as no later logit lies ~100 binades above the reference; if a sum leaves that range (or a
-        // reference was a masked logit), the warp redoes the unit's statistics exactly. Afterwards the lanes'
+        // as long as no later logit lies ~100 binades above the reference. If a sum leaves that range (or a
+        // reference was a masked logit), the warp redoes the unit's statistics exactly; kLong, whose first tiles are gone by
+        // then, looks before it sums (half an instruction per logit) and raises the reference. Afterwards the lanes'
         // references are replaced by the warp's maximum of them.
         uint64_t negm2[NPAD / 2];
 #pragma unroll
@@ -422,15 +392,35 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
           negm2[i] = pack2(-4.f * kEmptyMax, -4.f * kEmptyMax);  // no tile: reference below any masked logit
           z2[i] = 0ull;
         }
-        ok = sweep([&](int i) { return wait_tile(i); },
-                   [&](int j, uint32_t (&r)[16], int i) {
-                     const int key0 = (tile0 + grp + 2 * i) * kTileKeys;
+        ok = sweep(0, my_tiles, [&](int x) { return wait_tile(x); },
+                   [&](int j, uint32_t (&r)[16], int x) {
+                     const int key0 = (tile0 + x) * kTileKeys;
+                     if (kLong && j == kBlocks - 1 && x < again) release_tile(x);  // all loads of the tile have completed
                      if (key0 + kTileKeys > all_bound) mask_block16(r, key0 + et, vis_s + j * 16);
-                     if (i == 0) {
+                     if (x == grp) {
 #pragma unroll
                        for (int c = 0; c < 8; ++c)
                          negm2[j * 8 + c] = pack2(-(__uint_as_float(r[2 * c]) * p.scale2),
                                                   -(__uint_as_float(r[2 * c + 1]) * p.scale2));
+                     }
+                     if (kLong && __any_sync(0xffffffffu, block_max_exponent(r, scale2x, negm2 + j * 8) > kMaxExponent)) {
+#pragma unroll
+                       for (int c = 0; c < 8; ++c) {
+                         float nl, nh, zl, zh;
+                         unpack2(negm2[j * 8 + c], nl, nh);
+                         unpack2(z2[j * 8 + c], zl, zh);
+                         const float sl = __uint_as_float(r[2 * c]) * p.scale2, shi = __uint_as_float(r[2 * c + 1]) * p.scale2;
+                         if (sl + nl > kMaxExponent) {
+                           zl *= ex2(-(sl + nl));
+                           nl = -sl;
+                         }
+                         if (shi + nh > kMaxExponent) {
+                           zh *= ex2(-(shi + nh));
+                           nh = -shi;
+                         }
+                         negm2[j * 8 + c] = pack2(nl, nh);
+                         z2[j * 8 + c] = pack2(zl, zh);
+                       }
                      }
                      exp_accumulate16(r, scale2x, negm2 + j * 8, z2 + j * 8);
                    });
@@ -446,9 +436,35 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
           unpack2(z2[i], st_z[2 * i], st_z[2 * i + 1]);
           bad = bad || !(st_z[2 * i] < 1.0e30f) || !(st_z[2 * i + 1] < 1.0e30f);  // also catches inf and NaN
         }
-        if (__any_sync(0xffffffffu, bad)) {
-          ok = exact_stats();
+        if (!kLong && __any_sync(0xffffffffu, bad)) {
+          // exactly, in two sweeps: the warp's maximum per row, then the sum of exp2 against it. The (negated, scaled)
+          // maxima are uniform over the warp: they go to the warp's shift_s and are read back as packed pairs.
+#pragma unroll
+          for (int c = 0; c < NPAD; ++c) st_m[c] = kEmptyMax;
+          ok = sweep(0, my_tiles, [&](int) { return true; },
+                     [&](int j, uint32_t (&r)[16], int x) {
+                       const int key0 = (tile0 + x) * kTileKeys;
+                       if (key0 + kTileKeys > all_bound) mask_block16(r, key0 + et, vis_s + j * 16);
+#pragma unroll
+                       for (int c = 0; c < 16; ++c)
+                         st_m[j * 16 + c] = fmaxf(st_m[j * 16 + c], __uint_as_float(r[c]));
+                     });
           if (!ok) break;
+          __syncwarp();
+#pragma unroll
+          for (int c = 0; c < NPAD; ++c) {
+            const float wm = warp_max(st_m[c]);
+            if (lane == (c & 31)) shift_s[c] = -(wm * p.scale2);
+          }
+#pragma unroll
+          for (int i = 0; i < NPAD / 2; ++i) z2[i] = 0ull;
+          __syncwarp();
+          sweep(0, my_tiles, [&](int) { return true; },
+                [&](int j, uint32_t (&r)[16], int x) {
+                  const int key0 = (tile0 + x) * kTileKeys;
+                  if (key0 + kTileKeys > all_bound) mask_block16(r, key0 + et, vis_s + j * 16);
+                  exp_accumulate16(r, scale2x, shift2 + j * 8, z2 + j * 8);
+                });
         } else {
           __syncwarp();
 #pragma unroll
@@ -462,7 +478,34 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
           __syncwarp();
         }
       } else {
-        ok = exact_stats();
+        // 64 rows: the references are the warp's maxima over the group's first tile, in shift_s (negated, scaled); a block
+        // with a logit more than kMaxExponent above its reference raises the block's references first.
+        __syncwarp();  // the warp's readers of shift_s for the previous unit are done
+#pragma unroll
+        for (int c = 0; c < NPAD; c += 32) shift_s[c + lane] = -4.f * kEmptyMax;
+#pragma unroll
+        for (int i = 0; i < NPAD / 2; ++i) z2[i] = 0ull;
+        __syncwarp();
+        ok = sweep(0, my_tiles, [&](int x) { return wait_tile(x); },
+                   [&](int j, uint32_t (&r)[16], int x) {
+                     const int key0 = (tile0 + x) * kTileKeys;
+                     if (kLong && j == kBlocks - 1 && x < again) release_tile(x);  // all loads of the tile have completed
+                     if (key0 + kTileKeys > all_bound) mask_block16(r, key0 + et, vis_s + j * 16);
+                     if (x == grp || __any_sync(0xffffffffu, block_max_exponent(r, scale2x, shift2 + j * 8) > kMaxExponent)) {
+                       float f[16];
+#pragma unroll
+                       for (int c = 0; c < 16; ++c) {
+                         const float old = shift_s[j * 16 + c], now = fminf(old, -(warp_max(__uint_as_float(r[c])) * p.scale2));
+                         f[c] = ex2(now - old);  // (0 for the first tile; there is nothing to scale yet)
+                         __syncwarp();
+                         if (lane == 0) shift_s[j * 16 + c] = now;
+                       }
+#pragma unroll
+                       for (int c = 0; c < 8; ++c) z2[j * 8 + c] = mul2(z2[j * 8 + c], pack2(f[2 * c], f[2 * c + 1]));
+                       __syncwarp();
+                     }
+                     exp_accumulate16(r, scale2x, shift2 + j * 8, z2 + j * 8);
+                   });
         if (!ok) break;
       }
       // Sum over the 32 lanes by a transposing shuffle reduction (fixed order): lane j ends up with the sum of
@@ -544,12 +587,13 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
         }
       }
       __syncwarp();
-      // sweep 3: psi(i) = sum over window rows of exp2(s - lse); the slot goes back to the MMA warp
+      // last sweep: psi(i) = sum over window rows of exp2(s - lse); the slot goes back to the MMA warp. The resident tiles
+      // first, then those that pass again.
       uint64_t acc = 0ull;
-      sweep([&](int) { return true; },
-            [&](int j, uint32_t (&r)[16], int i) {
-              const int key = (tile0 + grp + 2 * i) * kTileKeys + et;
-              if (j == kBlocks - 1) release_tile(i);  // all loads of the tile have completed
+      ok = sweep(again, my_tiles + again, [&](int x) { return !kLong || x < my_tiles || wait_tile(x); },
+            [&](int j, uint32_t (&r)[16], int x) {
+              const int key = (tile0 + (kLong && x >= my_tiles ? x - my_tiles : x)) * kTileKeys + et;
+              if (j == kBlocks - 1) release_tile(x);  // all loads of the tile have completed
               if (key - et + kTileKeys > all_bound) mask_block16(r, key, vis_s + j * 16);
               acc = exp_sum16(r, scale2x, shift2 + j * 8, j == 0 ? 0ull : acc);
               if (j == kBlocks - 1) {
@@ -571,18 +615,18 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
   }
 }
 
-template <int D, int NPAD>
+template <int D, int NPAD, bool kLong>
 int run_cluster(const CUtensorMap& mk, const CUtensorMap& mq, const ClParams& p, int sms, cudaStream_t st) {
   using SL = ClSmem<D, NPAD>;
   const int smem = SL::alloc_bytes(p.C);
-  auto kern = score_cluster_kernel<D, NPAD>;
+  auto kern = score_cluster_kernel<D, NPAD, kLong>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       (p.C > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
     cudaGetLastError();
     return MADAKV_EUNSUPPORTED;
   }
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)p.C;
   attr[0].val.clusterDim.y = 1;
@@ -604,6 +648,12 @@ int run_cluster(const CUtensorMap& mk, const CUtensorMap& mq, const ClParams& p,
     fprintf(stderr, "madakv: score cluster kernel: cluster size %d, %d of at most %d clusters, %d B shared memory\n", p.C,
             clusters, max_clusters, smem);
   cfg.gridDim = dim3((unsigned)(clusters * p.C));
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;  // (see launch_ex)
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+  }
   if (cudaLaunchKernelEx(&cfg, kern, mk, mq, p) != cudaSuccess) {
     cudaGetLastError();
     return MADAKV_ECUDA;
@@ -613,37 +663,40 @@ int run_cluster(const CUtensorMap& mk, const CUtensorMap& mq, const ClParams& p,
 
 }  // namespace
 
-// The cluster size for a shape, or 0 if the logits of the longest sequence do not fit the TMEM of kMaxCluster CTAs.
-// Any size from 1 to 8 works (a unit's tiles are dealt out in equal shares, the last ranks get the remainder). The
-// default is the smallest size whose per-CTA share fits; MADAKV_CLUSTER_SIZE forces another size that fits.
-static int cluster_size_for(const madakv_config& c, int* per_max) {
+// The cluster size for a shape, or 0 for shapes that two passes over K (score_rows.cu) take in less time. Any size from 1 to
+// 8 works (a unit's tiles are dealt out in equal shares, the last ranks get the remainder).
+//   all logits fit the TMEM of at most 8 CTAs: the smallest size that holds them (llava: 4). Beyond 32 rows, where the
+//     sweeps cost twice as much, not for long units in a call that fills the GPU (64 rows, two passes against this kernel:
+//     1024 units of 4000 keys 364 us against 438, of 2000 219 against 181; 112 of 4000 59 against 61, of 2000 42 against 30;
+//     16 of 8000 29 against 33, of 6000 29 against 19)
+//   longer, up to 32 rows: 6, of which 22 fit the device (132 SMs) and hold more than half as much again as 4 (1024 units of
+//     20480 keys: sizes 3 to 8 take 1278, 1218, 1205, 1163, 1407, 1220 us, two passes 1707; 60 of 131072: 774, 579,
+//     685, 580, 617, 546 against 641; 512 of 30000: 974 against 1242), if the units fill the last round of clusters well enough
+//     (40 units of 89088: 259 against 300; 32 of 131072, a round and a half: 404 against 344)
+// MADAKV_CLUSTER_SIZE forces another size that holds all logits.
+static int cluster_size_for(const madakv_config& c) {
   const int R = (c.n_q_heads / c.n_kv_heads) * c.window;
   const int npad = R <= 32 ? 32 : 64;
   const int slots = kTmemCols / npad;
   const int tiles = (c.max_seq_len + kTileKeys - 1) / kTileKeys;
   if (const char* e = getenv("MADAKV_CLUSTER_SIZE")) {
     const int C = atoi(e);
-    if (C >= 1 && C <= kMaxCluster && (tiles + C - 1) / C <= slots) {
-      *per_max = (tiles + C - 1) / C;
-      return C;
-    }
+    if (C >= 1 && C <= kMaxCluster && (tiles + C - 1) / C <= slots) return C;
   }
-  for (int C = 1; C <= kMaxCluster; ++C) {
-    const int per = (tiles + C - 1) / C;
-    if (per <= slots) {
-      *per_max = per;
-      return C;
-    }
-  }
-  return 0;
+  const long long units = (long long)c.batch * c.n_layers * c.n_kv_heads;
+  if (R > 32 && tiles >= 24 && units * tiles >= 960) return 0;
+  for (int C = 1; C <= kMaxCluster; ++C)
+    if ((tiles + C - 1) / C <= slots) return C;
+  if (R > 32) return 0;
+  const long long round = 132 / kLongCluster, rounds = (units + round - 1) / round;
+  return 5 * units >= 4 * round * rounds ? kLongCluster : 0;
 }
 
 int launch_score_cluster(const madakv_config& c, const void* q, madakv_strides sq, const void* k, madakv_strides sk,
                          const int32_t* seq_len, float* lse, float* psi, void* ws, cudaStream_t st) {
   const int g = c.n_q_heads / c.n_kv_heads;
   if (c.dtype != MADAKV_BF16 || g * c.window > 64) return MADAKV_EUNSUPPORTED;
-  int per_max = 0;
-  const int C = cluster_size_for(c, &per_max);
+  const int C = cluster_size_for(c);
   if (C == 0) return MADAKV_EUNSUPPORTED;
   if (const char* e = getenv("MADAKV_SCORE_PATH"))
     if (e[0] == 't') return MADAKV_EUNSUPPORTED;  // tests: force the two-phase kernel
@@ -662,7 +715,6 @@ int launch_score_cluster(const madakv_config& c, const void* q, madakv_strides s
   p.n_max = c.max_seq_len;
   p.causal = c.causal;
   p.C = C;
-  p.per_max = per_max;
   p.scale2 = scale_of(c) * kLog2e;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -673,9 +725,14 @@ int launch_score_cluster(const madakv_config& c, const void* q, madakv_strides s
       !make_map(&mq, q, c.head_dim, c.window, c.n_q_heads, c.n_layers, c.batch, sq, c.window, g))
     return MADAKV_EUNSUPPORTED;
   const int npad = p.R <= 32 ? 32 : 64;
+  if (((c.max_seq_len + kTileKeys - 1) / kTileKeys + C - 1) / C > kTmemCols / npad) {
+    if (c.head_dim == 128)
+      return npad == 32 ? run_cluster<128, 32, true>(mk, mq, p, sms, st) : run_cluster<128, 64, true>(mk, mq, p, sms, st);
+    return npad == 32 ? run_cluster<64, 32, true>(mk, mq, p, sms, st) : run_cluster<64, 64, true>(mk, mq, p, sms, st);
+  }
   if (c.head_dim == 128)
-    return npad == 32 ? run_cluster<128, 32>(mk, mq, p, sms, st) : run_cluster<128, 64>(mk, mq, p, sms, st);
-  return npad == 32 ? run_cluster<64, 32>(mk, mq, p, sms, st) : run_cluster<64, 64>(mk, mq, p, sms, st);
+    return npad == 32 ? run_cluster<128, 32, false>(mk, mq, p, sms, st) : run_cluster<128, 64, false>(mk, mq, p, sms, st);
+  return npad == 32 ? run_cluster<64, 32, false>(mk, mq, p, sms, st) : run_cluster<64, 64, false>(mk, mq, p, sms, st);
 }
 
 }  // namespace madakv

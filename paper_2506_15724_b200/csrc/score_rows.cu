@@ -32,14 +32,18 @@
 // of all 128-key tiles in (sequence, layer, KV head, tile) order; a CTA takes a contiguous range of it, the same
 // number of tiles to within one for every CTA whatever the lengths in the batch. The part of a unit inside a CTA's
 // range is a run: queries and log-sum-exps are loaded once per run, and pass 1 leaves one pair per run, so a unit's
-// statistics come in as many pieces as CTAs share it (two or three for long sequences). Warp roles: warp 0 TMA
-// producer, warp 1 MMA issuer and TMEM owner, warps 2-17 epilogue; TMEM lane quarter = warp % 4 throughout. Every wait is bounded: on expiry the kernel records MADAKV_ETIMEOUT, drains and returns.
+// statistics come in as many pieces as CTAs share it (two or three for long sequences). Up to 128 rows the queries (and the
+// shift rows) are double-buffered, so that the next unit's are there when its first keys are: with short sequences a CTA
+// changes units every few tiles (5 tiles of 128 keys: a change took 7000 clocks, the tiles 4500). The first keys of a unit are
+// always asked for before its queries. In a call of a few tiles per CTA the start counts as much as the tiles, so the
+// partition is 32-bit arithmetic on lengths in shared memory. Warp roles: warp 0 TMA
+// producer, warp 1 MMA issuer and TMEM owner, warps 2-17 epilogue, warp 18 (pass 2) the shift rows; TMEM lane quarter = warp % 4 throughout. Every wait is bounded: on expiry the kernel records MADAKV_ETIMEOUT, drains and returns.
 #include "tc_common.cuh"
 
 namespace madakv {
 namespace {
 
-constexpr int kRowThreads = 576;  // 2 + 16 warps
+constexpr int kRowThreads = 640;  // 2 + 16 warps, a helper and one that idles (registers are allocated four warps at a time)
 constexpr int kMaxSeqScan = 1024; // batches up to this size get the exact (ragged-aware) tile partition
 constexpr int kFoldTiles = 16;    // pass 1 moves a row's sum to its second level every this many tiles
 
@@ -75,12 +79,14 @@ struct RowSmem {
   static constexpr int kOnesOff = kQOff + kQBytes;                          // pass 2: [128 keys][64] bf16, 1 in columns 0-2
   static constexpr int kShiftOff = kOnesOff + (PASS == 2 ? 128 * 128 : 0);  // pass 2: [rows][64] bf16, columns 0-2
   static constexpr int kBarOff = kShiftOff + (PASS == 2 ? kQRows * 128 : 0);
-  // full[kStages], empty[kStages], qfull, qempty, tfull[2], tempty[2], drain, xfull[8], xempty[8]
-  static constexpr int kNumBars = 2 * kStages + 2 + 4 + 1 + 16;
+  // full[kStages], empty[kStages], qfull[2], qempty[2], tfull[2], tempty[2], drain, xfull[8], xempty[8]
+  static constexpr int kNumBars = 2 * kStages + 4 + 4 + 1 + 16;
   static constexpr int kMiscOff = (kBarOff + kNumBars * 8 + 15) / 16 * 16;
   static constexpr int kColOff = kMiscOff + 48;            // window position (row % w) of every row [256]
-  static constexpr int kXchOff = kColOff + 256 * 4;        // pass 2: partial psi of column shares 1-3 [2][3][128]
-  static constexpr int kTotal = kXchOff + 6 * 128 * 4;
+  static constexpr int kOffOff = kColOff + 256 * 4;        // pass 2: place of every row in the group's log-sum-exps [256]
+  static constexpr int kXchOff = kOffOff + 256 * 4;        // pass 2: partial psi of column shares 1-3 [2][3][128]
+  static constexpr int kLenOff = kXchOff + 6 * 128 * 4;    // lengths of the sequences
+  static constexpr int kTotal = kLenOff + kMaxSeqScan * 4;
   static constexpr int kAlloc = kTotal + 1024;
   static_assert(kQOff % 1024 == 0 && kOnesOff % 1024 == 0 && kShiftOff % 1024 == 0 && kBarOff % 8 == 0, "alignment");
   static_assert(kAlloc <= 227 * 1024, "shared memory");
@@ -241,10 +247,14 @@ struct Run {
   int tiles;    // tiles of the run that hold keys (fewer than cnt only in the uniform partition of very large batches)
 };
 
-__device__ __forceinline__ int tiles_of(const RowParams& p, int b, bool exact) {
-  return ((exact ? clamped_len(p.seq_len, b, p.n_max) : p.n_max) + kTileKeys - 1) / kTileKeys;
+// `lens`: the lengths in shared memory, or null (batches too large for that: the uniform partition)
+__device__ __forceinline__ int seq_length(const RowParams& p, const int* lens, int b) {
+  return lens ? lens[b] : clamped_len(p.seq_len, b, p.n_max);
 }
-__device__ __forceinline__ void cursor_settle(const RowParams& p, TileCursor& c, bool exact) {
+__device__ __forceinline__ int tiles_of(const RowParams& p, const int* lens, int b) {
+  return ((lens ? lens[b] : p.n_max) + kTileKeys - 1) / kTileKeys;
+}
+__device__ __forceinline__ void cursor_settle(const RowParams& p, TileCursor& c, const int* lens) {
   // move on to the next sequence that has tiles
   while (c.left > 0 && c.r >= c.per_b) {
     c.r -= c.per_b;
@@ -253,34 +263,34 @@ __device__ __forceinline__ void cursor_settle(const RowParams& p, TileCursor& c,
       c.left = 0;
       break;
     }
-    c.tb = tiles_of(p, c.b, exact);
+    c.tb = tiles_of(p, lens, c.b);
     c.per_b = p.lh * c.tb;
   }
 }
-__device__ __forceinline__ Run cursor_run(const RowParams& p, const TileCursor& c) {
+__device__ __forceinline__ Run cursor_run(const RowParams& p, const TileCursor& c, const int* lens) {
   Run r;
   const int ub = c.r / c.tb;
   r.t0 = c.r - ub * c.tb;
   r.cnt = min(c.tb - r.t0, c.left);
   r.b = c.b;
   r.u = c.b * p.lh + ub;
-  r.n = clamped_len(p.seq_len, c.b, p.n_max);
+  r.n = seq_length(p, lens, c.b);
   const int real = (r.n + kTileKeys - 1) / kTileKeys;  // tiles of the unit that hold keys
   r.tiles = max(0, min(r.t0 + r.cnt, real) - r.t0);
   return r;
 }
-__device__ __forceinline__ void cursor_advance(const RowParams& p, TileCursor& c, const Run& r, bool exact) {
+__device__ __forceinline__ void cursor_advance(const RowParams& p, TileCursor& c, const Run& r, const int* lens) {
   c.r += r.cnt;
   c.left -= r.cnt;
   c.done += r.cnt;
-  cursor_settle(p, c, exact);
+  cursor_settle(p, c, lens);
 }
-// The CTA whose range [total * c / grid, total * (c + 1) / grid) holds tile x of the global order.
-__device__ __forceinline__ int cta_of(long long total, int grid, long long x) {
-  int c = (int)(x * grid / total);
-  while (c + 1 < grid && total * (c + 1) / grid <= x) ++c;
-  while (c > 0 && total * c / grid > x) --c;
-  return c;
+// The partition: of `total` tiles CTA c of `ctas` gets [first_tile(c), first_tile(c + 1)), the first ones one more each.
+// (The host refuses shapes with 2^30 tiles or more.)
+__device__ __forceinline__ int first_tile(int total, int ctas, int c) { return total / ctas * c + min(c, total % ctas); }
+__device__ __forceinline__ int cta_of(int total, int ctas, int x) {
+  const int q = total / ctas, more = total % ctas;
+  return x < more * (q + 1) ? x / (q + 1) : more + (x - more * (q + 1)) / q;  // (x < total, so q > 0 in the second case)
 }
 
 template <int D, int PASS, int NS>
@@ -298,17 +308,19 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SL::kBarOff);
   uint64_t* full = bars;               // [kStages] TMA -> MMA
   uint64_t* empty = bars + kStages;    // [kStages] MMA -> TMA
-  uint64_t* qfull = empty + kStages;   // [1]       TMA -> MMA (queries of the unit; in pass 2 also its shift rows)
-  uint64_t* qempty = qfull + 1;        // [1]       MMA -> TMA
-  uint64_t* tfull = qempty + 1;        // [2]       MMA -> epilogue
+  uint64_t* qfull = empty + kStages;   // [2]       TMA (and in pass 2 the shift rows' warp) -> MMA: a unit's row operands
+  uint64_t* qempty = qfull + 2;        // [2]       MMA -> TMA
+  uint64_t* tfull = qempty + 2;        // [2]       MMA -> epilogue
   uint64_t* tempty = tfull + 2;        // [2]       epilogue -> MMA
   uint64_t* drain = tempty + 2;        // [1]
   uint64_t* xfull = drain + 1;         // [2][4]    pass 2: column shares 1-3 -> share 0, per buffer and lane quarter
   uint64_t* xempty = xfull + 8;        // [2][4]    pass 2: share 0 -> shares 1-3
   uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(smem + SL::kMiscOff);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + SL::kMiscOff + 4);
-  int* range_s = reinterpret_cast<int*>(smem + SL::kMiscOff + 8);  // first sequence, tile in it, tiles, exact, lo, total, CTAs in use
+  int* range_s = reinterpret_cast<int*>(smem + SL::kMiscOff + 8);  // first sequence, tile in it, tiles, empty sequences, lo, total, CTAs in use
+  int* len_s = reinterpret_cast<int*>(smem + SL::kLenOff);
   int* rowpos = reinterpret_cast<int*>(smem + SL::kColOff);
+  int* rowoff = reinterpret_cast<int*>(smem + SL::kOffOff);
   float* xch = reinterpret_cast<float*>(smem + SL::kXchOff);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -318,9 +330,9 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    mbar_init(qfull, 1);
-    mbar_init(qempty, 1);
     for (int i = 0; i < 2; ++i) {
+      mbar_init(&qfull[i], PASS == 2 ? 2 : 1);
+      mbar_init(&qempty[i], 1);
       mbar_init(&tfull[i], 1);
       mbar_init(&tempty[i], 512);  // every epilogue thread
     }
@@ -337,63 +349,79 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
   // the 128-byte swizzle: the 16-byte piece that holds columns 0-7 of row r sits at position r % 8).
   for (int x = threadIdx.x; x < (SL::kBarOff - SL::kQOff) / 16; x += kRowThreads)
     reinterpret_cast<uint4*>(q_s)[x] = make_uint4(0, 0, 0, 0);
-  for (int x = threadIdx.x; x < 256; x += kRowThreads) rowpos[x] = p.r0 + x % p.wc;
-  // (everything above touches only this CTA's shared memory: it overlaps the kernel before this one)
-  pdl_wait();
-  pdl_go();
-  if (threadIdx.x == 0) {
-    // this CTA's range of tiles
-    const bool exact = p.B <= kMaxSeqScan;
-    long long total = 0;
-    if (exact) {
-      for (int b = 0; b < p.B; ++b) total += (long long)p.lh * tiles_of(p, b, true);
-    } else {
-      total = (long long)p.units * tiles_of(p, 0, false);
-    }
-    // (a batch with fewer tiles than CTAs is spread over as many CTAs as it has tiles: no empty range lies between
-    // two CTAs that share a unit)
-    const long long ctas = total < (long long)gridDim.x ? total : (long long)gridDim.x;
-    const bool idle = (long long)blockIdx.x >= ctas;
-    const long long lo = idle ? total : total * blockIdx.x / ctas, hi = idle ? total : total * (blockIdx.x + 1) / ctas;
-    int b0 = 0;
-    long long r0 = lo;
-    if (exact) {
-      while (b0 < p.B) {
-        const long long per = (long long)p.lh * tiles_of(p, b0, true);
-        if (r0 < per) break;
-        r0 -= per;
-        ++b0;
-      }
-    } else {
-      const long long per = (long long)p.lh * tiles_of(p, 0, false);
-      b0 = (int)(lo / per);
-      r0 = lo - (long long)b0 * per;
-    }
-    range_s[0] = b0;
-    range_s[1] = (int)r0;
-    range_s[2] = (int)(hi - lo);
-    range_s[3] = exact ? 1 : 0;
-    range_s[4] = (int)lo;     // (the host refuses shapes with 2^31 tiles or more)
-    range_s[5] = (int)total;
-    range_s[6] = (int)ctas;
+  if (threadIdx.x < 256) {
+    const int x = threadIdx.x, hh = x / p.wc, pos = p.r0 + x - hh * p.wc;
+    rowpos[x] = pos;
+    rowoff[x] = x < p.R ? hh * p.w + pos : 0;
   }
-  __syncthreads();
-  if (PASS == 2 && threadIdx.x < kTileKeys) {
-    const int r = threadIdx.x;
-    *reinterpret_cast<uint4*>(ones_s + r * 128 + (r & 7) * 16) = make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);
+  if (threadIdx.x == 32) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_k) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_q) : "memory");
   }
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_base_s)),
                  "r"(kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  if (PASS == 2) {
+    __syncthreads();  // (the zeros are written)
+    if (threadIdx.x < kTileKeys) {
+      const int r = threadIdx.x;
+      *reinterpret_cast<uint4*>(ones_s + r * 128 + (r & 7) * 16) = make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);
+    }
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  // (everything above touches only this CTA's shared memory and TMEM: it overlaps the kernel before this one)
+  pdl_wait();
+  pdl_go();
+  const int* lens = p.B <= kMaxSeqScan ? len_s : nullptr;
+  if (lens)
+    for (int b = threadIdx.x; b < p.B; b += kRowThreads) len_s[b] = clamped_len(p.seq_len, b, p.n_max);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    // this CTA's range of tiles
+    int total = 0, none = 0;
+    if (lens) {
+      for (int b = 0; b < p.B; ++b) {
+        const int tb = tiles_of(p, lens, b);
+        total += p.lh * tb;
+        none |= tb == 0 ? 1 : 0;
+      }
+    } else {
+      total = p.units * tiles_of(p, lens, 0);
+    }
+    // (a batch with fewer tiles than CTAs is spread over as many CTAs as it has tiles: no empty range lies between
+    // two CTAs that share a unit)
+    const int ctas = min(total, (int)gridDim.x);
+    const bool idle = (int)blockIdx.x >= ctas;
+    const int lo = idle ? total : first_tile(total, ctas, blockIdx.x), hi = idle ? total : first_tile(total, ctas, blockIdx.x + 1);
+    int b0 = 0, r0 = lo;
+    if (lens) {
+      while (b0 < p.B) {
+        const int per = p.lh * tiles_of(p, lens, b0);
+        if (r0 < per) break;
+        r0 -= per;
+        ++b0;
+      }
+    } else {
+      const int per = p.lh * tiles_of(p, lens, 0);
+      b0 = lo / per;
+      r0 = lo - b0 * per;
+    }
+    range_s[0] = b0;
+    range_s[1] = r0;
+    range_s[2] = hi - lo;
+    range_s[3] = none;
+    range_s[4] = lo;
+    range_s[5] = total;
+    range_s[6] = ctas;
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_base_s;
-  const bool exact = range_s[3] != 0;
+  const int nq = NS == 1 && p.R <= 128 ? 2 : 1;  // buffers of the row operands: buffer i starts at row 128 * i
 
   auto cursor_begin = [&]() {
     TileCursor c;
@@ -401,89 +429,57 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
     c.r = range_s[1];
     c.left = c.b < p.B ? range_s[2] : 0;
     c.done = 0;
-    c.tb = c.left > 0 ? tiles_of(p, c.b, exact) : 1;
+    c.tb = c.left > 0 ? tiles_of(p, lens, c.b) : 1;
     c.per_b = p.lh * c.tb;
-    cursor_settle(p, c, exact);
+    cursor_settle(p, c, lens);
     return c;
   };
 
   if (warp == 0) {
-    // ================================================================ TMA producer: lane 0 waits and issues the
-    // copies; the whole warp walks the items with it, because in pass 2 all 32 lanes write the unit's shift rows
+    // ================================================================ TMA producer
     const uint64_t pol_k = NS == 3 ? l2_policy_evict_last() : l2_policy_evict_first();  // (split keys are read again)
     const uint64_t pol_q = l2_policy_evict_last();
-    int stage = 0, cur_u = -1;
-    uint32_t stage_par = 0, q_par = 0;
+    int stage = 0, k = 0;  // k: units begun
+    uint32_t stage_par = 0;
     bool ok = true;
+    if (lane == 0)
     for (TileCursor c = cursor_begin(); ok && c.left > 0;) {
-      const Run run = cursor_run(p, c);
-      cursor_advance(p, c, run, exact);
-      const int u = run.u, tiles = run.tiles, key_begin = run.t0 * kTileKeys;
-      if (tiles == 0) continue;
+      const Run run = cursor_run(p, c, lens);
+      cursor_advance(p, c, run, lens);
+      const int u = run.u, key_begin = run.t0 * kTileKeys, loads = run.tiles * SL::kPieces;
+      if (loads == 0) continue;
       // fp32: the slice's split operands are [units][n_max][3 D] and [units * g][w][3 D]
       const int h = NS == 3 ? u : u % p.Hkv, l = NS == 3 ? 0 : (u / p.Hkv) % p.L, b = NS == 3 ? 0 : u / p.lh;
-      if (u != cur_u) {  // a new run: the unit's queries (and, in pass 2, its shift rows)
-        cur_u = u;
-        if (lane == 0) ok = mbar_wait(qempty, q_par ^ 1, abort_flag, p.status, kSiteQEmpty);
-        ok = __shfl_sync(0xffffffffu, ok, 0);
+      const int buf = k % nq;
+      const uint32_t q_par = (uint32_t)(k / nq) & 1u;
+      ++k;
+      for (int x = 0; ok && x < loads; ++x) {
+        const int t = x / SL::kPieces, piece = x % SL::kPieces;
+        ok = mbar_wait(&empty[stage], stage_par ^ 1, abort_flag, p.status, kSiteStage);
         if (!ok) break;
-        q_par ^= 1;
-        if (PASS == 2) {
-          // Row r of the shift operand: -lse_r / scale as the sum of three bf16 numbers (24 bits) in columns 0-2.
-          // Multiplied by the key side's ones in the extra contraction step, the accumulator holds q.k - lse / scale
-          // and the epilogue needs no per-row operand at all.
-          const float inv = 1.0f / p.scale2;
-          const float* src = p.lse2 + (int64_t)u * p.rs;
-          const int gh = (p.u0 + u) % p.Hkv, gbl = (p.u0 + u) / p.Hkv;
-          for (int r = lane; r < p.n16; r += 32) {
-            float nl;  // a row that sees no key (-inf) and the padding rows get a shift that turns every weight into 0
-            if (p.given_lse) {
-              nl = kEmptyMax;
-              if (r < p.R) {
-                const float gl = p.given_lse[((int64_t)gbl * p.Hq + gh * p.g + p.h0 + r / p.wc) * p.w + p.r0 + r % p.wc];
-                if (gl > -INFINITY) nl = -gl * kLog2e;
-              }
-            } else {
-              nl = src[r];
-            }
-            const float v = nl * inv;
-            const float hi = __bfloat162float(__float2bfloat16_rn(v));
-            const float mid = __bfloat162float(__float2bfloat16_rn(v - hi));
-            const float low = __bfloat162float(__float2bfloat16_rn((v - hi) - mid));
-            const uint32_t w0 = (__float_as_uint(hi) >> 16) | (__float_as_uint(mid) & 0xffff0000u);
-            *reinterpret_cast<uint4*>(shift_s + r * 128 + (r & 7) * 16) = make_uint4(w0, __float_as_uint(low) >> 16, 0u, 0u);
-          }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          __syncwarp();  // every lane's rows are written (and fenced) before lane 0 signals the unit ready
+        mbar_expect_tx(&full[stage], (uint32_t)SL::kStageBytes);
+        if (NS == 3) {
+          tma_load_5d(k_s + stage * SL::kStageBytes, &tmap_k, &full[stage],
+                      ((2 - piece / kKBlocks) * kKBlocks + piece % kKBlocks) * 64, key_begin + t * kTileKeys, h, l, b, pol_k);
+        } else {
+          for (int kb = 0; kb < kKBlocks; ++kb)
+            tma_load_5d(k_s + stage * SL::kStageBytes + kb * kTileKeys * 128, &tmap_k, &full[stage], kb * 64,
+                        key_begin + t * kTileKeys, h, l, b, pol_k);
         }
-        if (lane == 0) {
-          mbar_expect_tx(qfull, (uint32_t)(p.R * 128 * kKBlocks * NS));
-          for (int kb = 0; kb < kKBlocks * NS; ++kb)
-            tma_load_5d(q_s + kb * SL::kQRows * 128, &tmap_q, qfull, kb * 64, p.r0, h * p.g + p.h0, l, b, pol_q);
+        if (++stage == kStages) {
+          stage = 0;
+          stage_par ^= 1;
         }
-      }
-      if (lane == 0) {
-        for (int x = 0; x < tiles * SL::kPieces; ++x) {
-          const int t = x / SL::kPieces, piece = x % SL::kPieces;
-          ok = mbar_wait(&empty[stage], stage_par ^ 1, abort_flag, p.status, kSiteStage);
+        // the unit's queries once the stages are full of its keys (those stages were the unit's before, whose tiles need
+        // nothing that is still to come; from the next load on the stages wait for this unit's own tiles)
+        if (x == (k == 1 ? 0 : min(kStages, loads) - 1)) {  // (the first unit's at once)
+          ok = mbar_wait(&qempty[buf], q_par ^ 1, abort_flag, p.status, kSiteQEmpty);
           if (!ok) break;
-          mbar_expect_tx(&full[stage], (uint32_t)SL::kStageBytes);
-          if (NS == 3) {
-            tma_load_5d(k_s + stage * SL::kStageBytes, &tmap_k, &full[stage],
-                        ((2 - piece / kKBlocks) * kKBlocks + piece % kKBlocks) * 64, key_begin + t * kTileKeys, h, l,
-                        b, pol_k);
-          } else {
-            for (int kb = 0; kb < kKBlocks; ++kb)
-              tma_load_5d(k_s + stage * SL::kStageBytes + kb * kTileKeys * 128, &tmap_k, &full[stage], kb * 64,
-                          key_begin + t * kTileKeys, h, l, b, pol_k);
-          }
-          if (++stage == kStages) {
-            stage = 0;
-            stage_par ^= 1;
-          }
+          mbar_expect_tx(&qfull[buf], (uint32_t)(p.R * 128 * kKBlocks * NS));
+          for (int kb = 0; kb < kKBlocks * NS; ++kb)
+            tma_load_5d(q_s + (kb * SL::kQRows + buf * 128) * 128, &tmap_q, &qfull[buf], kb * 64, p.r0, h * p.g + p.h0, l, b, pol_q);
         }
       }
-      ok = __shfl_sync(0xffffffffu, ok, 0);
     }
     if (!ok && lane == 0) {  // abandoned: give copies in flight time to land before the CTA's shared memory goes away
       const long long t0 = clock64();
@@ -492,24 +488,22 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
   } else if (warp == 1) {
     // ================================================================ MMA issuer
     if (lane == 0) {
-      const uint32_t k_lo0 = smem_desc_lo(smem_u32(k_s)), q_lo0 = smem_desc_lo(smem_u32(q_s));
-      const uint32_t ones_lo = smem_desc_lo(smem_u32(ones_s)), shift_lo = smem_desc_lo(smem_u32(shift_s));
+      const uint32_t k_lo0 = smem_desc_lo(smem_u32(k_s)), q_lo00 = smem_desc_lo(smem_u32(q_s));
+      const uint32_t ones_lo = smem_desc_lo(smem_u32(ones_s)), shift_lo0 = smem_desc_lo(smem_u32(shift_s));
       const uint32_t idesc2 = instr_desc_bf16(p.n16);
-      int stage = 0, n_tile = 0, cur_u = -1;
-      uint32_t stage_par = 0, q_par = 0;
+      int stage = 0, n_tile = 0, k = 0;  // k: units begun
+      uint32_t stage_par = 0;
       bool ok = true;
       for (TileCursor c = cursor_begin(); ok && c.left > 0;) {
-        const Run run = cursor_run(p, c);
-        cursor_advance(p, c, run, exact);
-        const int u = run.u, tiles = run.tiles;
+        const Run run = cursor_run(p, c, lens);
+        cursor_advance(p, c, run, lens);
+        const int tiles = run.tiles;
         if (tiles == 0) continue;
-        if (u != cur_u) {
-          if (cur_u >= 0) umma_commit(qempty);  // the queries may be replaced once the MMAs issued so far are done
-          cur_u = u;
-          ok = mbar_wait(qfull, q_par, abort_flag, p.status, kSiteQFull);
-          if (!ok) break;
-          q_par ^= 1;
-        }
+        const int qb = k % nq;
+        ok = mbar_wait(&qfull[qb], (uint32_t)(k / nq) & 1u, abort_flag, p.status, kSiteQFull);
+        if (!ok) break;
+        ++k;
+        const uint32_t q_lo0 = q_lo00 + (uint32_t)qb * (128 * 128 >> 4), shift_lo = shift_lo0 + (uint32_t)qb * (128 * 128 >> 4);
         for (int t = 0; t < tiles; ++t, ++n_tile) {
           const int buf = n_tile & 1;
           const uint32_t use_par = (uint32_t)(n_tile >> 1) & 1u;
@@ -595,6 +589,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
           }
           umma_commit(&tfull[buf]);    // the accumulators are ready
         }
+        if (ok) umma_commit(&qempty[qb]);  // the row operands may be replaced once the MMAs issued so far are done
       }
       if (!ok) {  // abandoned: TMEM may only be freed once this thread's MMAs have completed
         umma_commit(drain);
@@ -602,7 +597,55 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
         while (!mbar_try(drain, 0) && clock64() - t0 < 20000000ll) __nanosleep(200);
       }
     }
-  } else {
+  } else if (warp == 18) {
+    // ================================================================ pass 2: the shift rows of every unit
+    // Row r of the shift operand: -lse_r / scale as the sum of three bf16 numbers (24 bits) in columns 0-2. Multiplied by
+    // the key side's ones in the extra contraction step, the accumulator holds q.k - lse / scale and the epilogue needs no
+    // per-row operand at all.
+    if (PASS == 2) {
+      const float inv = 1.0f / p.scale2;
+      int k = 0;
+      bool ok = true;
+      for (TileCursor c = cursor_begin(); ok && c.left > 0;) {
+        const Run run = cursor_run(p, c, lens);
+        cursor_advance(p, c, run, lens);
+        if (run.tiles == 0) continue;
+        const int u = run.u, gh = (p.u0 + u) % p.Hkv, gbl = (p.u0 + u) / p.Hkv, buf = k % nq;
+        // all loads first (one after the other they took 5 us)
+        const float* src = p.given_lse ? p.given_lse + ((int64_t)gbl * p.Hq + gh * p.g + p.h0) * p.w : p.lse2 + (int64_t)u * p.rs;
+        float nl[SL::kQRows / 32];
+#pragma unroll
+        for (int i = 0; i < SL::kQRows / 32; ++i) {
+          const int r = lane + 32 * i;
+          nl[i] = __ldcg(src + (p.given_lse ? rowoff[r] : min(r, p.rs - 1)));
+        }
+        // a row that sees no key (-inf) and the padding rows get a shift that turns every weight into 0
+#pragma unroll
+        for (int i = 0; i < SL::kQRows / 32; ++i) {
+          if (p.given_lse) nl[i] = nl[i] > -INFINITY ? -nl[i] * kLog2e : kEmptyMax;
+          if (lane + 32 * i >= p.R) nl[i] = kEmptyMax;
+        }
+        ok = __all_sync(0xffffffffu, mbar_wait(&qempty[buf], ((uint32_t)(k / nq) & 1u) ^ 1u, abort_flag, p.status, kSiteQEmpty));
+        if (!ok) break;
+        ++k;
+#pragma unroll
+        for (int i = 0; i < SL::kQRows / 32; ++i) {
+          const int r = lane + 32 * i;
+          if (r < p.n16) {
+            const float v = nl[i] * inv;
+            const float hi = __bfloat162float(__float2bfloat16_rn(v));
+            const float mid = __bfloat162float(__float2bfloat16_rn(v - hi));
+            const float low = __bfloat162float(__float2bfloat16_rn((v - hi) - mid));
+            const uint32_t w0 = (__float_as_uint(hi) >> 16) | (__float_as_uint(mid) & 0xffff0000u);
+            *reinterpret_cast<uint4*>(shift_s + (buf * 128 + r) * 128 + (r & 7) * 16) = make_uint4(w0, __float_as_uint(low) >> 16, 0u, 0u);
+          }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();  // every lane's rows are written (and fenced) before lane 0 signals them
+        if (lane == 0) mbar_arrive(&qfull[buf]);
+      }
+    }
+  } else if (warp < 18) {
     // ================================================================ epilogue (warps 2-17)
     // All 16 warps work on the same tile while the MMAs of the next tile fill the other accumulator buffer;
     // warp = (TMEM lane quarter, column share); the TMEM load of a warp's next 16 columns is in flight while it works.
@@ -632,17 +675,17 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
     float m = 4.f * kEmptyMax, z_run = 0.f;
     uint64_t zacc[4] = {0ull, 0ull, 0ull, 0ull};  // pass 1: the item's sum, as four packed partial sums
     float* xslot = xch + quarter * 32 + lane;  // pass 2: [buffer][share - 1][128 keys]
-    if (PASS == 2 && exact && !p.accumulate) {  // sequences without keys have no tiles
+    if (PASS == 2 && range_s[3] && !p.accumulate) {  // sequences without keys have no tiles
       for (int b = 0; b < p.B; ++b)
-        if (clamped_len(p.seq_len, b, p.n_max) == 0)
+        if (len_s[b] == 0)
           for (int64_t x = (int64_t)blockIdx.x * 512 + ew * 32 + lane; x < (int64_t)p.lh * p.n_max; x += (int64_t)gridDim.x * 512)
             p.psi[(int64_t)b * p.lh * p.n_max + x] = 0.f;
     }
 
     for (TileCursor c = cursor_begin(); ok && c.left > 0;) {
-      const Run run = cursor_run(p, c);
+      const Run run = cursor_run(p, c, lens);
       const int run_first = range_s[4] + c.done;  // the run's first tile in the global order
-      cursor_advance(p, c, run, exact);
+      cursor_advance(p, c, run, lens);
       const int u = run.u, tiles = run.tiles, key_begin = run.t0 * kTileKeys, n = run.n;
       float* psi = p.psi + (int64_t)u * p.n_max;
       m = 4.f * kEmptyMax;  // pass 1: every run starts its own statistics
@@ -765,8 +808,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
           // one pair per run: slot = this CTA's place among the CTAs that the unit's tiles are spread over (the merge
           // kernel walks the same partition). A row that saw no visible key only summed masked entries: it is
           // recorded as empty, and so is a run without keys (the uniform partition of very large batches has those).
-          const long long total = range_s[5];
-          const int k = (int)blockIdx.x - cta_of(total, range_s[6], (long long)run_first - run.t0);
+          const int k = (int)blockIdx.x - cta_of(range_s[5], range_s[6], run_first - run.t0);
           const bool none = tiles == 0 || m < 0.5f * kEmptyMax * p.scale2;
           if (k >= 0 && k < p.smax)
             p.part[(((int64_t)u * p.smax + k) * p.cparts + share) * p.rs + row] =
@@ -802,22 +844,23 @@ __global__ void __launch_bounds__(256) score_rows_merge_kernel(RowParams p, floa
     // the CTAs of pass 1 that the unit's tiles were spread over: the same partition as in the kernel
     const int b = u / p.lh;
     const bool exact = p.B <= kMaxSeqScan;
-    long long all_tiles = 0, first = 0;  // tiles of the batch; the unit's first tile in the global order
-    const int tb = tiles_of(p, b, exact);
+    auto seq_tiles = [&](int b2) { return ((exact ? clamped_len(p.seq_len, b2, p.n_max) : p.n_max) + kTileKeys - 1) / kTileKeys; };
+    int all_tiles = 0, first = 0;  // tiles of the batch; the unit's first tile in the global order
+    const int tb = seq_tiles(b);
     if (exact) {
       for (int b2 = 0; b2 < p.B; ++b2) {
-        const long long per = (long long)p.lh * tiles_of(p, b2, true);
+        const int per = p.lh * seq_tiles(b2);
         if (b2 < b) first += per;
         all_tiles += per;
       }
     } else {
-      all_tiles = (long long)p.units * tb;
-      first = (long long)b * p.lh * tb;
+      all_tiles = p.units * tb;
+      first = b * p.lh * tb;
     }
-    first += (long long)(u - b * p.lh) * tb;
+    first += (u - b * p.lh) * tb;
     s_entries = 0;
     if (tb > 0) {
-      const int ctas = (int)(all_tiles < p.grid ? all_tiles : p.grid);
+      const int ctas = min(all_tiles, p.grid);
       s_entries = p.cparts * min(p.smax, cta_of(all_tiles, ctas, first + tb - 1) - cta_of(all_tiles, ctas, first) + 1);
     }
   }

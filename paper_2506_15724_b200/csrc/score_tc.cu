@@ -1,4 +1,6 @@
 // Stage 1, Blackwell tensor-core path (Eq. 7 with the softmax of Eq. 5) for bf16 inputs with g * w <= 64 window rows.
+// Taken on request only (MADAKV_SCORE_PATH=twophase, for the tests of waits between CTAs that run out): on the sequences that
+// it was the default for, the cluster kernel or two passes take less time (1024 units of 20480 keys: 1.16 against 1.56 ms).
 //
 // One persistent kernel streams every K tile exactly once from HBM and a second time from L2:
 //   - the window-QK^T tile is a tcgen05.mma with the 128 keys of a tile on M, the g*w window rows on N and head_dim

@@ -4,6 +4,8 @@ Staged tests feed each CUDA stage the ORACLE's output of the stage before, so in
 End-to-end tests run the CUDA pipeline on its own outputs and re-run each oracle stage on what the CUDA stage before
 it produced; scores are compared within the stated tolerance, everything downstream exactly.
 """
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -152,6 +154,31 @@ def test_score_in_chunks_and_slices(dtype, B, L, Hq, Hkv, d, n, w, causal):
     mk.madakv_score_lse(cfg, d_q, d_k, d_sl, lse, psi, ws)
     assert mk.madakv_poll_status(ws) == 0
     assert psi_close(psi.cpu().numpy(), want, PSI_RTOL) < PSI_RTOL_SEEN
+
+
+# sequences longer than a cluster's TMEM holds: a whole round of clusters, tiles that pass twice in one sequence of the batch
+# and not in the other, lengths that end inside a tile; with logits so far apart that references are raised; and the calls
+# next to the rule (too few units, too many rows), which take two passes
+@pytest.mark.parametrize("B,H,d,n,w", [(1, 22, 64, 16500, 32), (2, 11, 128, 17003, 20), (1, 2, 64, 17000, 32), (1, 24, 64, 5200, 64)])
+@pytest.mark.parametrize("spread", [False, True])
+def test_score_longer_than_tensor_memory(B, H, d, n, w, spread):
+    wl = synth.scaled(TINY, dtype="bf16", B=B, L=1, Hq=H, Hkv=H, d=d, n=n, w=w, layout="blocks70", budget=n // 5)
+    q = synth.make_q_win(wl)
+    k = synth.hash_normal(3, 5, 0, B * H * n * d).view(B, 1, H, n, d)
+    if spread:
+        k[:, :, :, ::97] *= 40.0
+    k = k.to(torch.bfloat16)
+    sl = np.array([n, 4000][:B], np.int32)
+    cfg = config_of(wl)
+    psi = torch.full((B, 1, H, n), -1.0, device="cuda")
+    ws = mk.new_workspace(cfg)
+    mk.madakv_score(cfg, q.cuda(), k.cuda(), torch.from_numpy(sl).cuda(), None, psi, ws)
+    assert mk.madakv_poll_status(ws) == 0
+    want = oracle.score(1, to_np(q), to_np(k), sl)
+    got = psi.cpu().numpy().astype(np.float64)
+    # logits up to L carry an fp32 rounding error of L * 2^-24 or so, which the exponential turns into a relative one
+    worst = float(np.abs(k.float().numpy()).max()) * float(np.abs(q.float().numpy()).max()) * math.sqrt(d)
+    assert psi_close(got, want, max(PSI_RTOL_SEEN, 8 * worst * 2.0 ** -24), atol=1e-7) >= 0.0
 
 
 @pytest.mark.parametrize("lag", ["8", "9", "40", "1000"])
