@@ -37,13 +37,13 @@
 // changes units every few tiles (5 tiles of 128 keys: a change took 7000 clocks, the tiles 4500). The first keys of a unit are
 // always asked for before its queries. In a call of a few tiles per CTA the start counts as much as the tiles, so the
 // partition is 32-bit arithmetic on lengths in shared memory. Warp roles: warp 0 TMA
-// producer, warp 1 MMA issuer and TMEM owner, warps 2-17 epilogue, warp 18 (pass 2) the shift rows; TMEM lane quarter = warp % 4 throughout. Every wait is bounded: on expiry the kernel records MADAKV_ETIMEOUT, drains and returns.
+// producer, warp 1 MMA issuer and TMEM owner, warps 2-17 epilogue; TMEM lane quarter = warp % 4 throughout. Every wait is bounded: on expiry the kernel records MADAKV_ETIMEOUT, drains and returns.
 #include "tc_common.cuh"
 
 namespace madakv {
 namespace {
 
-constexpr int kRowThreads = 640;  // 2 + 16 warps, a helper and one that idles (registers are allocated four warps at a time)
+constexpr int kRowThreads = 576;  // 2 + 16 warps
 constexpr int kMaxSeqScan = 1024; // batches up to this size get the exact (ragged-aware) tile partition
 constexpr int kFoldTiles = 16;    // pass 1 moves a row's sum to its second level every this many tiles
 
@@ -436,13 +436,13 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
   };
 
   if (warp == 0) {
-    // ================================================================ TMA producer
+    // ================================================================ TMA producer: lane 0 waits and issues the copies;
+    // in pass 2 all lanes write the units' shift rows
     const uint64_t pol_k = NS == 3 ? l2_policy_evict_last() : l2_policy_evict_first();  // (split keys are read again)
     const uint64_t pol_q = l2_policy_evict_last();
     int stage = 0, k = 0;  // k: units begun
     uint32_t stage_par = 0;
     bool ok = true;
-    if (lane == 0)
     for (TileCursor c = cursor_begin(); ok && c.left > 0;) {
       const Run run = cursor_run(p, c, lens);
       cursor_advance(p, c, run, lens);
@@ -452,34 +452,79 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
       const int h = NS == 3 ? u : u % p.Hkv, l = NS == 3 ? 0 : (u / p.Hkv) % p.L, b = NS == 3 ? 0 : u / p.lh;
       const int buf = k % nq;
       const uint32_t q_par = (uint32_t)(k / nq) & 1u;
-      ++k;
-      for (int x = 0; ok && x < loads; ++x) {
-        const int t = x / SL::kPieces, piece = x % SL::kPieces;
-        ok = mbar_wait(&empty[stage], stage_par ^ 1, abort_flag, p.status, kSiteStage);
-        if (!ok) break;
-        mbar_expect_tx(&full[stage], (uint32_t)SL::kStageBytes);
-        if (NS == 3) {
-          tma_load_5d(k_s + stage * SL::kStageBytes, &tmap_k, &full[stage],
-                      ((2 - piece / kKBlocks) * kKBlocks + piece % kKBlocks) * 64, key_begin + t * kTileKeys, h, l, b, pol_k);
-        } else {
-          for (int kb = 0; kb < kKBlocks; ++kb)
-            tma_load_5d(k_s + stage * SL::kStageBytes + kb * kTileKeys * 128, &tmap_k, &full[stage], kb * 64,
-                        key_begin + t * kTileKeys, h, l, b, pol_k);
+      // Row r of the shift operand: -lse_r / scale as the sum of three bf16 numbers (24 bits) in columns 0-2. Multiplied by
+      // the key side's ones in the extra contraction step, the accumulator holds q.k - lse / scale and the epilogue needs no
+      // per-row operand at all. (All loads first; one after the other they took 5 us.)
+      float nl[SL::kQRows / 32];
+      if (PASS == 2) {
+        const int gh = (p.u0 + u) % p.Hkv, gbl = (p.u0 + u) / p.Hkv;
+        const float* src = p.given_lse ? p.given_lse + ((int64_t)gbl * p.Hq + gh * p.g + p.h0) * p.w : p.lse2 + (int64_t)u * p.rs;
+#pragma unroll
+        for (int i = 0; i < SL::kQRows / 32; ++i) {
+          const int r = lane + 32 * i;
+          nl[i] = __ldcg(src + (p.given_lse ? rowoff[r] : min(r, p.rs - 1)));
         }
-        if (++stage == kStages) {
-          stage = 0;
-          stage_par ^= 1;
-        }
-        // the unit's queries once the stages are full of its keys (those stages were the unit's before, whose tiles need
-        // nothing that is still to come; from the next load on the stages wait for this unit's own tiles)
-        if (x == (k == 1 ? 0 : min(kStages, loads) - 1)) {  // (the first unit's at once)
-          ok = mbar_wait(&qempty[buf], q_par ^ 1, abort_flag, p.status, kSiteQEmpty);
+      }
+      // [from, to) of the unit's K loads, by lane 0
+      auto load_keys = [&](int from, int to) {
+        for (int x = from; ok && x < to; ++x) {
+          const int t = x / SL::kPieces, piece = x % SL::kPieces;
+          ok = mbar_wait(&empty[stage], stage_par ^ 1, abort_flag, p.status, kSiteStage);
           if (!ok) break;
+          mbar_expect_tx(&full[stage], (uint32_t)SL::kStageBytes);
+          if (NS == 3) {
+            tma_load_5d(k_s + stage * SL::kStageBytes, &tmap_k, &full[stage],
+                        ((2 - piece / kKBlocks) * kKBlocks + piece % kKBlocks) * 64, key_begin + t * kTileKeys, h, l, b, pol_k);
+          } else {
+            for (int kb = 0; kb < kKBlocks; ++kb)
+              tma_load_5d(k_s + stage * SL::kStageBytes + kb * kTileKeys * 128, &tmap_k, &full[stage], kb * 64,
+                          key_begin + t * kTileKeys, h, l, b, pol_k);
+          }
+          if (++stage == kStages) {
+            stage = 0;
+            stage_par ^= 1;
+          }
+        }
+      };
+      // The unit's queries once the stages are full of its keys (those stages were the unit's before, whose tiles need
+      // nothing that is still to come; from the next load on the stages wait for this unit's own tiles); the first
+      // unit's at once.
+      const int ahead = k == 0 ? 1 : min(kStages, loads);
+      ++k;
+      if (lane == 0) {
+        load_keys(0, ahead);
+        ok = ok && mbar_wait(&qempty[buf], q_par ^ 1, abort_flag, p.status, kSiteQEmpty);
+        if (ok) {
           mbar_expect_tx(&qfull[buf], (uint32_t)(p.R * 128 * kKBlocks * NS));
           for (int kb = 0; kb < kKBlocks * NS; ++kb)
             tma_load_5d(q_s + (kb * SL::kQRows + buf * 128) * 128, &tmap_q, &qfull[buf], kb * 64, p.r0, h * p.g + p.h0, l, b, pol_q);
         }
       }
+      if (PASS == 2) {
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (!ok) break;
+        const float inv = 1.0f / p.scale2;
+#pragma unroll
+        for (int i = 0; i < SL::kQRows / 32; ++i) {
+          const int r = lane + 32 * i;
+          // a row that sees no key (-inf) and the padding rows get a shift that turns every weight into 0
+          if (p.given_lse) nl[i] = nl[i] > -INFINITY ? -nl[i] * kLog2e : kEmptyMax;
+          if (r >= p.R) nl[i] = kEmptyMax;
+          if (r < p.n16) {
+            const float v = nl[i] * inv;
+            const float hi = __bfloat162float(__float2bfloat16_rn(v));
+            const float mid = __bfloat162float(__float2bfloat16_rn(v - hi));
+            const float low = __bfloat162float(__float2bfloat16_rn((v - hi) - mid));
+            const uint32_t w0 = (__float_as_uint(hi) >> 16) | (__float_as_uint(mid) & 0xffff0000u);
+            *reinterpret_cast<uint4*>(shift_s + (buf * 128 + r) * 128 + (r & 7) * 16) = make_uint4(w0, __float_as_uint(low) >> 16, 0u, 0u);
+          }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();  // every lane's rows are written (and fenced) before lane 0 signals them
+        if (lane == 0) mbar_arrive(&qfull[buf]);
+      }
+      if (lane == 0) load_keys(ahead, loads);
+      ok = __shfl_sync(0xffffffffu, ok, 0);
     }
     if (!ok && lane == 0) {  // abandoned: give copies in flight time to land before the CTA's shared memory goes away
       const long long t0 = clock64();
@@ -597,55 +642,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
         while (!mbar_try(drain, 0) && clock64() - t0 < 20000000ll) __nanosleep(200);
       }
     }
-  } else if (warp == 18) {
-    // ================================================================ pass 2: the shift rows of every unit
-    // Row r of the shift operand: -lse_r / scale as the sum of three bf16 numbers (24 bits) in columns 0-2. Multiplied by
-    // the key side's ones in the extra contraction step, the accumulator holds q.k - lse / scale and the epilogue needs no
-    // per-row operand at all.
-    if (PASS == 2) {
-      const float inv = 1.0f / p.scale2;
-      int k = 0;
-      bool ok = true;
-      for (TileCursor c = cursor_begin(); ok && c.left > 0;) {
-        const Run run = cursor_run(p, c, lens);
-        cursor_advance(p, c, run, lens);
-        if (run.tiles == 0) continue;
-        const int u = run.u, gh = (p.u0 + u) % p.Hkv, gbl = (p.u0 + u) / p.Hkv, buf = k % nq;
-        // all loads first (one after the other they took 5 us)
-        const float* src = p.given_lse ? p.given_lse + ((int64_t)gbl * p.Hq + gh * p.g + p.h0) * p.w : p.lse2 + (int64_t)u * p.rs;
-        float nl[SL::kQRows / 32];
-#pragma unroll
-        for (int i = 0; i < SL::kQRows / 32; ++i) {
-          const int r = lane + 32 * i;
-          nl[i] = __ldcg(src + (p.given_lse ? rowoff[r] : min(r, p.rs - 1)));
-        }
-        // a row that sees no key (-inf) and the padding rows get a shift that turns every weight into 0
-#pragma unroll
-        for (int i = 0; i < SL::kQRows / 32; ++i) {
-          if (p.given_lse) nl[i] = nl[i] > -INFINITY ? -nl[i] * kLog2e : kEmptyMax;
-          if (lane + 32 * i >= p.R) nl[i] = kEmptyMax;
-        }
-        ok = __all_sync(0xffffffffu, mbar_wait(&qempty[buf], ((uint32_t)(k / nq) & 1u) ^ 1u, abort_flag, p.status, kSiteQEmpty));
-        if (!ok) break;
-        ++k;
-#pragma unroll
-        for (int i = 0; i < SL::kQRows / 32; ++i) {
-          const int r = lane + 32 * i;
-          if (r < p.n16) {
-            const float v = nl[i] * inv;
-            const float hi = __bfloat162float(__float2bfloat16_rn(v));
-            const float mid = __bfloat162float(__float2bfloat16_rn(v - hi));
-            const float low = __bfloat162float(__float2bfloat16_rn((v - hi) - mid));
-            const uint32_t w0 = (__float_as_uint(hi) >> 16) | (__float_as_uint(mid) & 0xffff0000u);
-            *reinterpret_cast<uint4*>(shift_s + (buf * 128 + r) * 128 + (r & 7) * 16) = make_uint4(w0, __float_as_uint(low) >> 16, 0u, 0u);
-          }
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();  // every lane's rows are written (and fenced) before lane 0 signals them
-        if (lane == 0) mbar_arrive(&qfull[buf]);
-      }
-    }
-  } else if (warp < 18) {
+  } else {
     // ================================================================ epilogue (warps 2-17)
     // All 16 warps work on the same tile while the MMAs of the next tile fill the other accumulator buffer;
     // warp = (TMEM lane quarter, column share); the TMEM load of a warp's next 16 columns is in flight while it works.
