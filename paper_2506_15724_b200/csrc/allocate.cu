@@ -22,7 +22,141 @@ struct AllocParams {
   int32_t* budgets;
   int L, Hkv, n_max, mpa, hcc_mode, keep_window, window;
   u64 theta_fix;  // floor(theta * 2^32)
+  unsigned* counter;  // one per sequence, zero between calls: the units that are done; null: masses and demands only
+  int depth, layer;   // one layer of a pass over `depth` layers (the arrays hold that layer, L = 1), or layer = -1: all layers
 };
+
+// Visual tokens among the first n of a sequence, counted by the whole block into *s_nv (which the caller has zeroed
+// behind a barrier); the caller synchronises before reading it.
+__device__ __forceinline__ void count_visual(const uint8_t* mask, int n, int* s_nv) {
+  int c = 0;
+  if ((reinterpret_cast<uintptr_t>(mask) & 15) == 0) {  // 16 tokens per load
+    const int n16 = n >> 4;
+    for (int i = threadIdx.x; i < n16; i += blockDim.x) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(mask) + i);
+      const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k)  // a byte counts if it is not zero
+        c += __popc(((w4[k] | (w4[k] >> 1) | (w4[k] >> 2) | (w4[k] >> 3) | (w4[k] >> 4) | (w4[k] >> 5) | (w4[k] >> 6) |
+                      (w4[k] >> 7)) & 0x01010101u));
+    }
+    for (int i = (n16 << 4) + threadIdx.x; i < n; i += blockDim.x) c += mask[i] ? 1 : 0;
+  } else {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) c += mask[i] ? 1 : 0;
+  }
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
+  if ((threadIdx.x & 31) == 0 && c) atomicAdd(s_nv, c);
+}
+// Eq. 10's sum over the heads of one layer (both modalities), by one warp; every lane returns it.
+__device__ __forceinline__ long long layer_demand(const int32_t* demand_layer, int Hkv) {
+  long long dem = 0;
+  for (int x = threadIdx.x & 31; x < 2 * Hkv; x += 32) dem += (long long)__ldcg(demand_layer + x);
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) dem += __shfl_xor_sync(0xffffffffu, dem, off);
+  return dem;
+}
+// The layer's integer budget Phi^l from phi^l, and phi^{l+1} (Eq. 10-11); l counts from 1, the update exists for l < L.
+__device__ __forceinline__ double rounded_budget(double ph, double lo, double hi) {
+  return fmin(fmax(floor(__dadd_rn(ph, 0.5)), lo), hi);
+}
+// The divisor of Eq. 11 for the step from layer l (0 for a mode without one) and its correctly rounded reciprocal: both
+// are known before the recurrence starts.
+__device__ __forceinline__ double phi_divisor(int Hkv, int L, int l, int hcc_mode) {
+  if (hcc_mode == MADAKV_HCC_PAPER || hcc_mode == MADAKV_HCC_DEMAND) return (double)((long long)Hkv * (L - l));  // per-head units
+  return hcc_mode == MADAKV_HCC_LITERAL ? (double)(L - l) : 0.0;  // Eq. 11 as printed
+}
+// K / div rounded to nearest, with the reciprocal at hand: the quotient of the product is within one unit in the last
+// place, and one correction by the exact remainder makes it the correctly rounded one (Markstein, "Computation of
+// elementary functions on the IBM RISC System/6000 processor", 1990). Three dependent operations instead of a division in
+// a chain that is one layer after the other (llava: 11.8 us for the 32 layers with divisions).
+__device__ __forceinline__ double next_phi(double ph, long long dem, int Hkv, double div, double rcp, double lo, double hi) {
+  const double K = __dsub_rn((double)dem, __dmul_rn((double)Hkv, ph));  // Eq. 10
+  const double q = __dmul_rn(K, rcp);
+  const double quot = __fma_rn(__fma_rn(-q, div, K), rcp, q);
+  const double next = div > 0.0 ? __dsub_rn(ph, quot) : ph;  // Eq. 11
+  return next < lo ? lo : (next > hi ? hi : next);  // (never NaN; both comparisons at once)
+}
+// Eq. 8 integerised for one head: the visual share rounded half up, the rest to text, surplus of a modality with too
+// few tokens passed to the other. With `keep_demand` (mode DEMAND, every layer but the last) the head keeps what
+// Eq. 9 asked for instead. lo_v, lo_t: the proxy tokens of each modality when they are retained unconditionally
+// (cfg->keep_window), else 0: budgets are floored at them, the head's total at their sum.
+__device__ __forceinline__ void split_budget(const AllocParams& p, int64_t u, double Phi, int n, int n_v, int n_t,
+                                             int lo_v, int lo_t, bool keep_demand) {
+  if (keep_demand) {
+    const int dv = __ldcg(p.demand + u * 2), dt = __ldcg(p.demand + u * 2 + 1);
+    p.budgets[u * 2] = p.mpa ? max(dv, lo_v) : 0;
+    p.budgets[u * 2 + 1] = p.mpa ? max(dt, lo_t) : min(max(dv + dt, lo_v + lo_t), n);
+    return;
+  }
+  const int P = max((int)Phi, lo_v + lo_t);
+  int bv, bt;
+  if (p.mpa) {
+    bv = (int)floor(__dadd_rn(__dmul_rn(__ldcg(p.pref + u * 2), Phi), 0.5));  // Eq. 8, rounded half up
+    bv = min(max(bv, lo_v), P - lo_t);
+    bt = P - bv;
+    if (bv > n_v) { bt += bv - n_v; bv = n_v; }
+    if (bt > n_t) { bv = min(n_v, bv + (bt - n_t)); bt = n_t; }
+  } else {
+    bv = 0;
+    bt = min(P, n);
+  }
+  p.budgets[u * 2] = bv;
+  p.budgets[u * 2 + 1] = bt;
+}
+
+// What is left once all units of sequence b have their masses and demands, by one block: Eq. 10-11 as a scalar scan over the
+// layers (or one step of it), then Eq. 8 integerised for every (layer, head). n_v: the sequence's visual tokens.
+// s_phi, s_dem: kLayerChunk values each in shared memory.
+constexpr int kLayerChunk = 1024;
+__device__ __noinline__ void sequence_budgets(const AllocParams& p, int b, int n, int n_v, double* s_phi, long long* s_dem) {
+  __shared__ int s_wv;
+  const int wlen = p.keep_window ? min(p.window, n) : 0;  // proxy tokens retained unconditionally
+  if (threadIdx.x == 0) s_wv = 0;
+  __syncthreads();
+  if (wlen > 0) {
+    count_visual(p.mask + (int64_t)b * p.n_max + (n - wlen), wlen, &s_wv);
+    __syncthreads();
+  }
+  const int n_t = n - n_v;
+  const int lo_v = p.mpa ? s_wv : 0, lo_t = wlen - lo_v;
+  const double lo = n >= 1 ? 1.0 : 0.0, hi = (double)n;
+  const int depth = p.depth, first = max(p.layer, 0);  // the layers of the arrays: first .. first + L - 1 of depth
+  double ph = 0.0;
+  for (int l0 = 0; l0 < p.L; l0 += kLayerChunk) {
+    const int ln = min(kLayerChunk, p.L - l0);
+    for (int l = threadIdx.x; l < ln; l += blockDim.x) {
+      const double div = first + l0 + l + 1 < depth ? phi_divisor(p.Hkv, depth, first + l0 + l + 1, p.hcc_mode) : 0.0;
+      s_phi[l] = div > 0.0 ? __drcp_rn(div) : 0.0;
+    }
+    // Eq. 10's sum over heads, one warp per layer (integers: any order gives the same sum)
+    for (int l = threadIdx.x >> 5; l < ln; l += blockDim.x >> 5) {
+      const long long dem = layer_demand(p.demand + ((int64_t)b * p.L + l0 + l) * p.Hkv * 2, p.Hkv);
+      if ((threadIdx.x & 31) == 0) s_dem[l] = dem;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      if (l0 == 0) ph = first == 0 ? (double)p.budget[b] : p.phi[(int64_t)b * depth + first];
+#pragma unroll 4
+      for (int l = 0; l < ln; ++l) {
+        const double rcp = s_phi[l];
+        s_phi[l] = ph;
+        const int at = first + l0 + l + 1;  // the paper counts layers from 1
+        if (at < depth) ph = next_phi(ph, s_dem[l], p.Hkv, phi_divisor(p.Hkv, depth, at, p.hcc_mode), rcp, lo, hi);
+      }
+      if (p.layer >= 0 && first + 1 < depth) p.phi[(int64_t)b * depth + first + 1] = ph;
+    }
+    __syncthreads();
+    for (int l = threadIdx.x; l < ln; l += blockDim.x)
+      if (p.layer <= 0) p.phi[(int64_t)b * depth + l0 + l] = s_phi[l];
+    for (int x = threadIdx.x; x < ln * p.Hkv; x += blockDim.x) {
+      const int l = x / p.Hkv;
+      split_budget(p, ((int64_t)b * p.L + l0) * p.Hkv + x, rounded_budget(s_phi[l], lo, hi), n, n_v, n_t, lo_v, lo_t,
+                   p.hcc_mode == MADAKV_HCC_DEMAND && first + l0 + l + 1 < depth);
+    }
+    __syncthreads();
+  }
+}
 
 // The low 32 bits of floor(x * 2^32), plus kLowBias, by fp32 additions, for keys below kSmallKey (512.0): adding 512
 // rounded towards zero leaves floor(x * 2^14) in the low bits of the significand, the remainder (exact) added to 2^-9 the
@@ -43,7 +177,7 @@ __device__ __forceinline__ uint32_t low_mass(uint32_t key) {
 // scores of 512 and more, goes the slow way: exact sweeps that halve the range.
 // (Exact 64-bit masses by atomics that return the old word, to detect carries: alloc 52 us on llava.)
 template <int KPT, int TEAM>
-__global__ void __launch_bounds__(kRankThreads, 2) alloc_unit_kernel(AllocParams p) {
+__global__ void __launch_bounds__(kRankThreads, 2) alloc_unit_kernel(const __grid_constant__ AllocParams p) {
   using SH = RankShared<TEAM, 2>;
   constexpr int kPer = SH::kPer;
   __shared__ SH sh;
@@ -129,6 +263,7 @@ __global__ void __launch_bounds__(kRankThreads, 2) alloc_unit_kernel(AllocParams
   u64 above0 = 0, above1 = 0;  // exact mass before r0.lo, r1.lo
   u64 need0 = 0, need1 = 0, W0 = 0, W1 = 0;
   bool exact = kmax < kSmallKey;
+  uint32_t n_vis = 0;  // visual tokens
 
   for (int pass = 0; pass < 2 && exact; ++pass) {
     // ---- buckets
@@ -220,6 +355,7 @@ __global__ void __launch_bounds__(kRankThreads, 2) alloc_unit_kernel(AllocParams
     }
     exact = sh.inexact == 0;
     if (pass == 0) {
+      n_vis = __reduce_add_sync(kFull, lane < TEAM ? sh.slice_c[0][lane] : 0u);
       W0 = warp_sum64(lane < TEAM ? sh.slice_q[0][lane] : 0ull);
       W1 = warp_sum64(lane < TEAM ? sh.slice_q[1][lane] : 0ull);
       need0 = target(W0);
@@ -289,6 +425,7 @@ __global__ void __launch_bounds__(kRankThreads, 2) alloc_unit_kernel(AllocParams
     team_sums(W0, W1);
     u64 n0 = __reduce_add_sync(kFull, c0), n1 = __reduce_add_sync(kFull, c1);
     team_sums(n0, n1);
+    n_vis = (uint32_t)n0;
     need0 = target(W0);
     need1 = target(W1);
     r0 = need0 ? RankRange{0u, all_span, (uint32_t)n0, 0u} : RankRange{kNowhere, 0u, 0u, 0u};
@@ -374,180 +511,41 @@ __global__ void __launch_bounds__(kRankThreads, 2) alloc_unit_kernel(AllocParams
     }
   }
   if (TEAM > 1) team_sync<TEAM>();  // no block leaves while block 0 still reads its shared memory
+  // ---- the unit that is done last goes on with its sequence
+  if (rank != 0 || !p.counter) return;
+  __shared__ unsigned s_last;
+  __syncthreads();
+  if (tid == 0) {  // (one thread's fences order what the block wrote before the barrier, and will read)
+    __threadfence();
+    s_last = atomicInc(p.counter + b, (unsigned)(p.L * p.Hkv) - 1u);  // (wraps to 0: ready for the next call)
+    __threadfence();
+  }
+  __syncthreads();
+  if (s_last != (unsigned)(p.L * p.Hkv) - 1u) return;
+  static_assert(sizeof(sh.cnt) >= kLayerChunk * 16, "the scan reuses the buckets");
+  sequence_budgets(p, b, n, (int)n_vis, reinterpret_cast<double*>(sh.cnt), reinterpret_cast<long long*>(sh.cnt) + kLayerChunk);
 }
 
-// Visual tokens among the first n of a sequence, counted by the whole block into *s_nv (which the caller has zeroed
-// behind a barrier); the caller synchronises before reading it.
-__device__ __forceinline__ void count_visual(const uint8_t* mask, int n, int* s_nv) {
-  int c = 0;
-  if ((reinterpret_cast<uintptr_t>(mask) & 15) == 0) {  // 16 tokens per load
-    const int n16 = n >> 4;
-    for (int i = threadIdx.x; i < n16; i += blockDim.x) {
-      const uint4 v = __ldg(reinterpret_cast<const uint4*>(mask) + i);
-      const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k)  // a byte counts if it is not zero
-        c += __popc(((w4[k] | (w4[k] >> 1) | (w4[k] >> 2) | (w4[k] >> 3) | (w4[k] >> 4) | (w4[k] >> 5) | (w4[k] >> 6) |
-                      (w4[k] >> 7)) & 0x01010101u));
-    }
-    for (int i = (n16 << 4) + threadIdx.x; i < n; i += blockDim.x) c += mask[i] ? 1 : 0;
-  } else {
-    for (int i = threadIdx.x; i < n; i += blockDim.x) c += mask[i] ? 1 : 0;
-  }
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
-  if ((threadIdx.x & 31) == 0 && c) atomicAdd(s_nv, c);
-}
-// Eq. 10's sum over the heads of one layer (both modalities), by one warp; every lane returns it.
-__device__ __forceinline__ long long layer_demand(const int32_t* demand_layer, int Hkv) {
-  long long dem = 0;
-  for (int x = threadIdx.x & 31; x < 2 * Hkv; x += 32) dem += (long long)demand_layer[x];
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) dem += __shfl_xor_sync(0xffffffffu, dem, off);
-  return dem;
-}
-// The layer's integer budget Phi^l from phi^l, and phi^{l+1} (Eq. 10-11); l counts from 1, the update exists for l < L.
-__device__ __forceinline__ double rounded_budget(double ph, double lo, double hi) {
-  return fmin(fmax(floor(__dadd_rn(ph, 0.5)), lo), hi);
-}
-// The divisor of Eq. 11 for the step from layer l (0 for a mode without one) and its correctly rounded reciprocal: both
-// are known before the recurrence starts.
-__device__ __forceinline__ double phi_divisor(int Hkv, int L, int l, int hcc_mode) {
-  if (hcc_mode == MADAKV_HCC_PAPER || hcc_mode == MADAKV_HCC_DEMAND) return (double)((long long)Hkv * (L - l));  // per-head units
-  return hcc_mode == MADAKV_HCC_LITERAL ? (double)(L - l) : 0.0;  // Eq. 11 as printed
-}
-// K / div rounded to nearest, with the reciprocal at hand: the quotient of the product is within one unit in the last
-// place, and one correction by the exact remainder makes it the correctly rounded one (Markstein, "Computation of
-// elementary functions on the IBM RISC System/6000 processor", 1990). Three dependent operations instead of a division in
-// a chain that is one layer after the other (llava: 11.8 us for the 32 layers with divisions).
-__device__ __forceinline__ double next_phi(double ph, long long dem, int Hkv, double div, double rcp, double lo, double hi) {
-  const double K = __dsub_rn((double)dem, __dmul_rn((double)Hkv, ph));  // Eq. 10
-  const double q = __dmul_rn(K, rcp);
-  const double quot = __fma_rn(__fma_rn(-q, div, K), rcp, q);
-  const double next = div > 0.0 ? __dsub_rn(ph, quot) : ph;  // Eq. 11
-  return fmin(fmax(next, lo), hi);
-}
-// Eq. 8 integerised for one head: the visual share rounded half up, the rest to text, surplus of a modality with too
-// few tokens passed to the other. With `keep_demand` (mode DEMAND, every layer but the last) the head keeps what
-// Eq. 9 asked for instead. lo_v, lo_t: the proxy tokens of each modality when they are retained unconditionally
-// (cfg->keep_window), else 0: budgets are floored at them, the head's total at their sum.
-__device__ __forceinline__ void split_budget(const AllocParams& p, int64_t u, double Phi, int n, int n_v, int n_t,
-                                             int lo_v, int lo_t, bool keep_demand) {
-  if (keep_demand) {
-    const int dv = p.demand[u * 2], dt = p.demand[u * 2 + 1];
-    p.budgets[u * 2] = p.mpa ? max(dv, lo_v) : 0;
-    p.budgets[u * 2 + 1] = p.mpa ? max(dt, lo_t) : min(max(dv + dt, lo_v + lo_t), n);
-    return;
-  }
-  const int P = max((int)Phi, lo_v + lo_t);
-  int bv, bt;
-  if (p.mpa) {
-    bv = (int)floor(__dadd_rn(__dmul_rn(p.pref[u * 2], Phi), 0.5));  // Eq. 8, rounded half up
-    bv = min(max(bv, lo_v), P - lo_t);
-    bt = P - bv;
-    if (bv > n_v) { bt += bv - n_v; bv = n_v; }
-    if (bt > n_t) { bv = min(n_v, bv + (bt - n_t)); bt = n_t; }
-  } else {
-    bv = 0;
-    bt = min(P, n);
-  }
-  p.budgets[u * 2] = bv;
-  p.budgets[u * 2 + 1] = bt;
-}
-
-// One block per sequence: Eq. 10-11 as a scalar scan over layers, then Eq. 8 integerised for every (layer, head). The
-// tokens are counted before the wait for the kernel that computes the demands (it has waited for all kernels before
-// it, so mask and lengths are final).
-__global__ void __launch_bounds__(1024) alloc_seq_kernel(AllocParams p) {
-  extern __shared__ double s_phi[];  // [L] reciprocals of Eq. 11's divisors, replaced by phi; then [L] demand sums (as long long)
-  long long* s_dem = reinterpret_cast<long long*>(s_phi + p.L);
-  __shared__ int s_nv, s_wv;
+// The same as a kernel of its own, one block per sequence: for the budgets of one layer whose masses and demands are given
+// (madakv_demand_layer), and after alloc_unit_kernel in calls of many units. `after_units`: the kernel before this one is that
+// one, which has waited for all kernels before it, so the tokens can be counted before the wait for its results.
+__global__ void __launch_bounds__(1024) alloc_seq_kernel(const __grid_constant__ AllocParams p, int after_units) {
+  __shared__ int s_nv;
+  __shared__ double s_phi[kLayerChunk];
+  __shared__ long long s_dem[kLayerChunk];
+  if (!after_units) pdl_wait();
   const int b = blockIdx.x;
   const int n = clamped_len(p.seq_len, b, p.n_max);
-  const int wlen = p.keep_window ? min(p.window, n) : 0;  // proxy tokens retained unconditionally
-  if (threadIdx.x == 0) s_nv = s_wv = 0;
+  if (threadIdx.x == 0) s_nv = 0;
   __syncthreads();
   count_visual(p.mask + (int64_t)b * p.n_max, n, &s_nv);
-  if (wlen > 0) count_visual(p.mask + (int64_t)b * p.n_max + (n - wlen), wlen, &s_wv);
-  for (int l = threadIdx.x; l < p.L; l += blockDim.x) {
-    const double div = l + 1 < p.L ? phi_divisor(p.Hkv, p.L, l + 1, p.hcc_mode) : 0.0;
-    s_phi[l] = div > 0.0 ? __drcp_rn(div) : 0.0;
-  }
-  pdl_wait();
+  __syncthreads();
+  if (after_units) pdl_wait();
   pdl_go();
-  // Eq. 10's sum over heads, one warp per layer (integers: any order gives the same sum)
-  for (int l = threadIdx.x >> 5; l < p.L; l += blockDim.x >> 5) {
-    const long long dem = layer_demand(p.demand + ((int64_t)b * p.L + l) * p.Hkv * 2, p.Hkv);
-    if ((threadIdx.x & 31) == 0) s_dem[l] = dem;
-  }
-  __syncthreads();
-  const int n_v = s_nv, n_t = n - n_v;
-  const int lo_v = p.mpa ? s_wv : 0, lo_t = wlen - lo_v;
-  const double lo = n >= 1 ? 1.0 : 0.0, hi = (double)n;
-  if (threadIdx.x == 0) {
-    double ph = (double)p.budget[b];
-#pragma unroll 4
-    for (int l = 0; l < p.L; ++l) {
-      const double rcp = s_phi[l];
-      s_phi[l] = ph;
-      if (l + 1 < p.L) ph = next_phi(ph, s_dem[l], p.Hkv, phi_divisor(p.Hkv, p.L, l + 1, p.hcc_mode), rcp, lo, hi);
-    }
-  }
-  __syncthreads();
-  for (int l = threadIdx.x; l < p.L; l += blockDim.x) p.phi[(int64_t)b * p.L + l] = s_phi[l];
-  for (int x = threadIdx.x; x < p.L * p.Hkv; x += blockDim.x)
-    split_budget(p, (int64_t)b * p.L * p.Hkv + x, rounded_budget(s_phi[x / p.Hkv], lo, hi), n, n_v, n_t, lo_v, lo_t,
-                 p.hcc_mode == MADAKV_HCC_DEMAND && x / p.Hkv + 1 < p.L);
+  sequence_budgets(p, b, n, s_nv, s_phi, s_dem);
 }
 
-// One block per sequence, one layer of a layer-by-layer pass: the same arithmetic as one trip of the scan above. The
-// per-layer arrays (pref, demand, budgets) hold this layer only; phi [B, depth] is the state carried between calls.
-// `after_demand`: the kernel before this one in the stream is alloc_unit_kernel, which has waited for all kernels before it,
-// so the tokens can be counted before the wait for its results.
-__global__ void __launch_bounds__(1024) alloc_layer_kernel(AllocParams p, int depth, int layer, int after_demand) {
-  __shared__ int s_nv, s_wv;
-  __shared__ double s_Phi;
-  __shared__ long long s_dem;
-  const int b = blockIdx.x;
-  if (!after_demand) pdl_wait();
-  const int n = clamped_len(p.seq_len, b, p.n_max);
-  const int wlen = p.keep_window ? min(p.window, n) : 0;
-  if (threadIdx.x == 0) s_nv = s_wv = 0;
-  __syncthreads();
-  count_visual(p.mask + (int64_t)b * p.n_max, n, &s_nv);
-  if (wlen > 0) count_visual(p.mask + (int64_t)b * p.n_max + (n - wlen), wlen, &s_wv);
-  if (after_demand) pdl_wait();
-  pdl_go();
-  if (threadIdx.x < 32) {
-    const long long dem = layer_demand(p.demand + (int64_t)b * p.Hkv * 2, p.Hkv);
-    if (threadIdx.x == 0) s_dem = dem;
-  }
-  __syncthreads();
-  const int n_v = s_nv, n_t = n - n_v;
-  const int lo_v = p.mpa ? s_wv : 0, lo_t = wlen - lo_v;
-  if (threadIdx.x == 0) {
-    const double lo = n >= 1 ? 1.0 : 0.0, hi = (double)n;
-    const int l = layer + 1;  // the paper counts layers from 1
-    double ph;
-    if (layer == 0) {
-      ph = (double)p.budget[b];
-      p.phi[(int64_t)b * depth] = ph;
-    } else {
-      ph = p.phi[(int64_t)b * depth + layer];
-    }
-    s_Phi = rounded_budget(ph, lo, hi);
-    if (l < depth) {
-      const double div = phi_divisor(p.Hkv, depth, l, p.hcc_mode);
-      p.phi[(int64_t)b * depth + l] = next_phi(ph, s_dem, p.Hkv, div, div > 0.0 ? __drcp_rn(div) : 0.0, lo, hi);
-    }
-  }
-  __syncthreads();
-  for (int x = threadIdx.x; x < p.Hkv; x += blockDim.x)
-    split_budget(p, (int64_t)b * p.Hkv + x, s_Phi, n, n_v, n_t, lo_v, lo_t,
-                 p.hcc_mode == MADAKV_HCC_DEMAND && layer + 1 < depth);
-}
-
-void launch_alloc_unit(const madakv_config& c, const AllocParams& p, int units, cudaStream_t st) {
+void launch_alloc_units(const madakv_config& c, const AllocParams& p, int units, cudaStream_t st) {
   const RankShape s = rank_shape(units, c.max_seq_len);
   switch (s.kpt + s.team) {
     case 8 + 1: launch_team(alloc_unit_kernel<8, 1>, units, 1, st, p); break;
@@ -561,23 +559,27 @@ void launch_alloc_unit(const madakv_config& c, const AllocParams& p, int units, 
   }
 }
 
-}  // namespace
+// Masses, demands and, with p.budgets, what follows from them. In a call of fewer units than SMs the last unit of a
+// sequence goes on with it (a kernel for that cost 2 us on the host and 4-6 on the GPU); in a larger one the fences and
+// counters of all units cost more than the kernel (256 units of 131072 keys: 606 us with them for the three steps after scoring,
+// 597 without).
+void launch_alloc(const madakv_config& c, AllocParams p, void* ws, cudaStream_t st) {
+  const int units = c.batch * p.L * p.Hkv;
+  p.counter = p.budgets && units < 148 ? reinterpret_cast<unsigned*>((char*)ws + kHeaderBytes) : nullptr;
+  launch_alloc_units(c, p, units, st);
+  if (p.budgets && !p.counter) launch_pdl(alloc_seq_kernel, dim3(c.batch), dim3(1024), 0, st, p, 1);
+}
 
-int launch_allocate(const madakv_config& c, const float* psi, const uint8_t* mask, const int32_t* seq_len,
-                    const int32_t* budget, double* mass, double* pref, int32_t* demand, double* phi, int32_t* budgets,
-                    void* ws, cudaStream_t st) {
-  (void)ws;
-  AllocParams p;
+AllocParams alloc_params(const madakv_config& c, int layers, const float* psi, const uint8_t* mask, const int32_t* seq_len,
+                         double* mass, double* pref, int32_t* demand) {
+  AllocParams p = {};
   p.psi = psi;
   p.mask = mask;
   p.seq_len = seq_len;
-  p.budget = budget;
   p.mass = mass;
   p.pref = pref;
   p.demand = demand;
-  p.phi = phi;
-  p.budgets = budgets;
-  p.L = c.n_layers;
+  p.L = layers;
   p.Hkv = c.n_kv_heads;
   p.n_max = c.max_seq_len;
   p.mpa = c.mpa;
@@ -585,61 +587,40 @@ int launch_allocate(const madakv_config& c, const float* psi, const uint8_t* mas
   p.keep_window = c.keep_window;
   p.window = c.window;
   p.theta_fix = (u64)((double)c.theta * 4294967296.0);
-  const int units = c.batch * c.n_layers * c.n_kv_heads;
-  launch_alloc_unit(c, p, units, st);
-  launch_pdl(alloc_seq_kernel, dim3(c.batch), dim3(1024), c.n_layers * (sizeof(double) + sizeof(long long)), st, p);
+  p.depth = c.n_layers;
+  p.layer = -1;
+  return p;
+}
+
+}  // namespace
+
+int launch_allocate(const madakv_config& c, const float* psi, const uint8_t* mask, const int32_t* seq_len,
+                    const int32_t* budget, double* mass, double* pref, int32_t* demand, double* phi, int32_t* budgets,
+                    void* ws, cudaStream_t st) {
+  AllocParams p = alloc_params(c, c.n_layers, psi, mask, seq_len, mass, pref, demand);
+  p.budget = budget;
+  p.phi = phi;
+  p.budgets = budgets;
+  launch_alloc(c, p, ws, st);
   return launch_status();
 }
 
 int launch_allocate_layer(const madakv_config& c, int layer, const float* psi, const uint8_t* mask,
                           const int32_t* seq_len, const int32_t* budget, double* mass, double* pref, int32_t* demand,
                           double* phi, int32_t* budgets, void* ws, cudaStream_t st) {
-  (void)ws;
-  AllocParams p;
-  p.psi = psi;
-  p.mask = mask;
-  p.seq_len = seq_len;
+  AllocParams p = alloc_params(c, 1, psi, mask, seq_len, mass, pref, demand);  // the per-layer arrays hold one layer
   p.budget = budget;
-  p.mass = mass;
-  p.pref = pref;
-  p.demand = demand;
   p.phi = phi;
   p.budgets = budgets;
-  p.L = 1;  // the per-layer arrays hold one layer
-  p.Hkv = c.n_kv_heads;
-  p.n_max = c.max_seq_len;
-  p.mpa = c.mpa;
-  p.hcc_mode = c.hcc_mode;
-  p.keep_window = c.keep_window;
-  p.window = c.window;
-  p.theta_fix = (u64)((double)c.theta * 4294967296.0);
-  if (psi) launch_alloc_unit(c, p, c.batch * c.n_kv_heads, st);  // else: done by launch_demand_layer
-  launch_pdl(alloc_layer_kernel, dim3(c.batch), dim3(1024), 0, st, p, c.n_layers, layer, psi ? 1 : 0);
+  p.layer = layer;
+  if (psi) launch_alloc(c, p, ws, st);
+  else launch_pdl(alloc_seq_kernel, dim3(c.batch), dim3(1024), 0, st, p, 0);  // masses and demands come from launch_demand_layer
   return launch_status();
 }
 
 int launch_demand_layer(const madakv_config& c, const float* psi, const uint8_t* mask, const int32_t* seq_len,
                         double* mass, double* pref, int32_t* demand, void* ws, cudaStream_t st) {
-  (void)ws;
-  AllocParams p;
-  p.psi = psi;
-  p.mask = mask;
-  p.seq_len = seq_len;
-  p.budget = nullptr;
-  p.mass = mass;
-  p.pref = pref;
-  p.demand = demand;
-  p.phi = nullptr;
-  p.budgets = nullptr;
-  p.L = 1;  // the per-layer arrays hold one layer
-  p.Hkv = c.n_kv_heads;
-  p.n_max = c.max_seq_len;
-  p.mpa = c.mpa;
-  p.hcc_mode = c.hcc_mode;
-  p.keep_window = c.keep_window;
-  p.window = c.window;
-  p.theta_fix = (u64)((double)c.theta * 4294967296.0);
-  launch_alloc_unit(c, p, c.batch * c.n_kv_heads, st);
+  launch_alloc(c, alloc_params(c, 1, psi, mask, seq_len, mass, pref, demand), ws, st);
   return launch_status();
 }
 

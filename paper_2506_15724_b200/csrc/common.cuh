@@ -14,8 +14,9 @@ namespace madakv {
 // ---------------------------------------------------------------------------------------------------------------
 // Workspace layout (device memory owned by the caller)
 //   [0, 256)                 header: int32 status, then counters used by persistent kernels
-//   [256, 256 + 64 K)        decode attention: blocks that have arrived, per segment of the call. At the same place for
-//                            every config (a workspace may serve several), zero to begin with and after every call
+//   [256, 256 + 64 K)        blocks that have arrived, per segment of a decode call or per sequence of an allocation. At the
+//                            same place for every config (a workspace may serve several), zero to begin with and after
+//                            every call
 //   [.., ..)                 stage 4 scratch: visual-token count per sequence [B] int32, visual tokens among the
 //                            proxy tokens per sequence [B] int32
 //   [.., .. + score)         stage 1 scratch: finished-item counters [units * rows] int32, log2-domain row
@@ -27,7 +28,7 @@ namespace madakv {
 constexpr size_t kHeaderBytes = 256;
 constexpr int kScoreChunk = 1024;   // keys per (max, sum) partial of the generic scoring path
 constexpr int kScoreTcChunk = 512;  // keys per work item (and per partial) of the tensor-core scoring path
-constexpr int kDecodeCounters = 16384;
+constexpr int kCounters = 16384;
 constexpr int kDecodeChunk = 256;   // cache rows per split of decode attention
 
 struct WsHeader {
@@ -80,7 +81,7 @@ inline WsLayout ws_layout(const madakv_config& c) {
   const size_t rows = (size_t)(c.n_q_heads / c.n_kv_heads) * c.window;
   w.score_chunks = (c.max_seq_len + kScoreChunk - 1) / kScoreChunk;
   w.decode_splits = (c.max_seq_len + c.max_new_tokens + kDecodeChunk - 1) / kDecodeChunk;
-  size_t off = kHeaderBytes + kDecodeCounters * sizeof(uint32_t);
+  size_t off = kHeaderBytes + kCounters * sizeof(uint32_t);
   w.seq_nv_off = off;
   off = align_up(off + 2 * (size_t)c.batch * sizeof(int32_t), 256);  // per sequence: visual tokens, visual proxy tokens
   const size_t rows_pad = (rows + 31) / 32 * 32;  // the tensor-core path pads the row count

@@ -724,7 +724,7 @@ struct DecodeShape {
   int slots, min_rows;
 };
 DecodeShape decode_shape(const madakv_config& c, int n_sel, int64_t capacity, bool tensor_core_kernel, int splits) {
-  if (n_sel > kDecodeCounters) return {1, 1};
+  if (n_sel > kCounters) return {1, 1};
   const int64_t units = (int64_t)c.batch * c.n_layers * c.n_kv_heads, longest = c.max_seq_len + c.max_new_tokens;
   const int64_t rows = capacity / units < longest ? capacity / units : longest;
   const int resident = 148 * (tensor_core_kernel ? 3 : 7);
@@ -813,7 +813,7 @@ int launch_decode(const madakv_config& c, int layer, const void* q, const void* 
 // counters of a split call lie behind them; they start at zero and every call leaves them at zero.
 struct StaticScratch {
   unsigned char part[MADAKV_STATIC_SCRATCH_BYTES];
-  unsigned counter[madakv::kDecodeCounters];
+  unsigned counter[madakv::kCounters];
 };
 static __device__ __align__(256) StaticScratch g_static_scratch;
 

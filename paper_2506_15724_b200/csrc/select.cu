@@ -1,7 +1,7 @@
 // Stage 4a: per-head, per-modality top-budget selection (Section 3.3, the eviction step after Eq. 8).
 //
-//   seg_scan     one block: visual-token count of every sequence, kept_len[u] = b_v + b_t and the exclusive scan
-//                seg_off (rows, with headroom)
+//   seg_scan     (batches only) one block: visual-token count of every sequence, kept_len[u] = b_v + b_t and the exclusive
+//                scan seg_off (rows, with headroom)
 //   select_unit  a team of blocks per unit (rank_common.cuh) finds, for both modalities at once, the budget-th largest
 //                value and how many of its ties are still needed; an ordered sweep then emits the kept positions in
 //                ascending order, giving ties to the lowest positions (prefix sums over the team provide the tie ranks
@@ -29,6 +29,7 @@ struct SelParams {
   int32_t* seq_nv;  // ws: visual-token count of every sequence
   int32_t* seq_wv;  // ws: visual tokens among the proxy tokens of every sequence (forced retention)
   int units, B, L, Hkv, n_max, mpa, headroom, keep_window, window, pool_r;  // pool_r: (pool_kernel - 1) / 2
+  int alone;  // no seg_scan before: every unit adds up the segments before its own
 };
 
 // One block. The visual tokens are counted by warps that share the sequences (several warps per sequence when there are
@@ -151,8 +152,9 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(SelParams 
   using SH = RankShared<TEAM, 1>;
   constexpr int kPer = SH::kPer;
   __shared__ SH sh;
-  // (no wait here: seg_scan, the kernel before, has waited for everything before it, so the scores, the mask and the
-  // budgets are final; what seg_scan itself writes is read after the wait below)
+  // (no wait here after seg_scan: it has waited for everything before it, so the scores, the mask and the budgets are final;
+  // what seg_scan itself writes is read after the wait below)
+  if (p.alone) pdl_wait();
   const uint32_t rank = TEAM > 1 ? team_rank() : 0u;
   const int u = blockIdx.x / TEAM;
   const int b = u / (p.Hkv * p.L);
@@ -168,7 +170,11 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(SelParams 
   // ranking only has to find the rest of each modality's budget
   const int wfrom = kPool && p.keep_window ? max(n - p.window, 0) : n;
   if (kPool) pdl_wait();  // (the forced tokens' counts are seg_scan's)
-  const int lo_v = kPool ? p.seq_wv[b] : 0, lo_t = (n - wfrom) - lo_v;
+  int lo_v = 0;
+  if (kPool && !p.alone) lo_v = p.seq_wv[b];
+  if (kPool && p.alone && p.mpa)  // (a window has at most 1024 tokens)
+    for (int x = wfrom; x < n; x += kRankThreads) lo_v += __syncthreads_count(x + tid < n && mask[x + tid] != 0);
+  const int lo_t = (n - wfrom) - lo_v;
   const uint32_t want0 = (uint32_t)(p.mpa ? max(p.budgets[2 * u] - lo_v, 0) : 0),
                  want1 = (uint32_t)max(p.budgets[2 * u + 1] - lo_t, 0);
 
@@ -217,6 +223,7 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(SelParams 
   RankRange r1 = want1 ? RankRange{0u, kmax - kmin, kNoKey, 0u} : RankRange{kNowhere, 0u, 0u, 0u};
   bool short0 = false, short1 = false;  // the modality has no more keys than are wanted: all of them are kept
   auto crowded = [](const RankRange& g) { return g.in > kListCap && g.span > 0; };
+  uint32_t n_vis = 0;  // visual tokens in the ranking
 
   for (int pass = 0; pass < 2; ++pass) {
     // ---- buckets
@@ -255,11 +262,11 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(SelParams 
     if (lane == 31) sh.wscan_c[warp] = ic;
     __syncthreads();
     ic += __reduce_add_sync(kFull, lane >= m * (kRankWarps / 2) && lane < warp ? sh.wscan_c[lane] : 0u);
+    if (i >= kHalf - 32) {  // the last warp of the modality has the block's total (in its last lane): to every block
+      const uint32_t tc = __shfl_sync(kFull, ic, 31);
+      if (lane < TEAM) peer_store<TEAM>(&sh.slice_c[m][rank], lane, tc);
+    }
     if (TEAM > 1) {
-      if (i >= kHalf - 32) {  // the last warp of the modality has the block's total (in its last lane): to every block
-        const uint32_t tc = __shfl_sync(kFull, ic, 31);
-        if (lane < TEAM) peer_store<TEAM>(&sh.slice_c[m][rank], lane, tc);
-      }
       team_sync<TEAM>();
       ic += __reduce_add_sync(kFull, lane < (int)rank ? sh.slice_c[m][lane] : 0u);
     }
@@ -282,6 +289,7 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(SelParams 
       }
     }
     team_sync<TEAM>();
+    if (pass == 0) n_vis = __reduce_add_sync(kFull, lane < TEAM ? sh.slice_c[0][lane] : 0u);
     {
       auto narrow = [&](RankRange& g, bool& is_short, int q, int s) {
         if (sh.first[q] == ~0ull) {
@@ -407,10 +415,39 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(SelParams 
     team_sync<TEAM>();  // (also the last access to a peer's shared memory)
     before = warp_sum64(lane < (int)rank ? sh.slice_q[0][lane] : 0ull);
   }
-  if (!kPool) pdl_wait();
-  pdl_go();
-  const int64_t off0 = p.seg_off[u];
-  if (off0 + p.kept_len[u] + p.headroom > p.capacity) return;  // seg_scan has raised MADAKV_ECAPACITY
+  int64_t off0;
+  if (p.alone) {
+    // one sequence: the segments' lengths follow from the budgets and the modalities' token counts, which are at hand
+    pdl_go();
+    const int n_v = (int)n_vis + lo_v;
+    auto length = [&](int x) {
+      const int2 bud = __ldg(reinterpret_cast<const int2*>(p.budgets) + x);
+      return (p.mpa ? min(max(bud.x, lo_v), n_v) : 0) + min(max(bud.y, lo_t), n - n_v);
+    };
+    u64 sum = 0;
+    for (int x = tid; x < u; x += kRankThreads) sum += (u64)(length(x) + p.headroom);
+    sum = warp_sum64(sum);
+    __syncthreads();
+    if (lane == 0) sh.wsum[0][warp] = sum;
+    __syncthreads();
+    off0 = (int64_t)warp_sum64(lane < kRankWarps ? sh.wsum[0][lane] : 0ull);
+    const int len = length(u);
+    const int64_t end = off0 + len + p.headroom;
+    if (rank == 0 && tid == 0) {
+      p.kept_len[u] = len;
+      p.seg_off[u] = off0;
+      if (u + 1 == p.units) {
+        p.seg_off[p.units] = end;
+        if (end > p.capacity) set_status(p.ws, MADAKV_ECAPACITY);
+      }
+    }
+    if (end > p.capacity) return;
+  } else {
+    if (!kPool) pdl_wait();
+    pdl_go();
+    off0 = p.seg_off[u];
+    if (off0 + p.kept_len[u] + p.headroom > p.capacity) return;  // seg_scan has raised MADAKV_ECAPACITY
+  }
   auto emit = [&](int pos0, u64 ahead) {  // ahead: counts before this thread's positions
     const uint32_t e0 = (uint32_t)ahead & 0x1fffffu, e1 = (uint32_t)(ahead >> 21) & 0x1fffffu, g = (uint32_t)(ahead >> 42);
     int32_t* out = p.kept_idx + off0 + g + min(e0, ties0) + min(e1, ties1);
@@ -489,7 +526,11 @@ int launch_select(const madakv_config& c, const float* psi, const uint8_t* mask,
   p.keep_window = c.keep_window;
   p.window = c.window;
   p.pool_r = (c.pool_kernel - 1) / 2;
-  launch_pdl(seg_scan_kernel, dim3(1), dim3(1024), 0, st, p);
+  // One sequence, few units: no kernel of its own for the scan of the segments (2 us on the host, 3-5 on the GPU). Units of
+  // other sequences would need those sequences' visual-token counts, and a larger call is better off with a scan that runs
+  // beside the ranking.
+  p.alone = c.batch == 1 && p.units < 148;
+  if (!p.alone) launch_pdl(seg_scan_kernel, dim3(1), dim3(1024), 0, st, p);
   if (c.pool_kernel > 1 || c.keep_window) launch_select_unit<true>(c, p, st);
   else launch_select_unit<false>(c, p, st);
   return launch_status();
