@@ -492,16 +492,21 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
                      if (kLong && j == kBlocks - 1 && x < again) release_tile(x);  // all loads of the tile have completed
                      if (key0 + kTileKeys > all_bound) mask_block16(r, key0 + et, vis_s + j * 16);
                      if (x == grp || __any_sync(0xffffffffu, block_max_exponent(r, scale2x, shift2 + j * 8) > kMaxExponent)) {
-                       float f[16];
+                       float mine = kEmptyMax;  // lane c < 16: the warp's maximum of row c
 #pragma unroll
                        for (int c = 0; c < 16; ++c) {
-                         const float old = shift_s[j * 16 + c], now = fminf(old, -(warp_max(__uint_as_float(r[c])) * p.scale2));
-                         f[c] = ex2(now - old);  // (0 for the first tile; there is nothing to scale yet)
-                         __syncwarp();
-                         if (lane == 0) shift_s[j * 16 + c] = now;
+                         const float wm = warp_max(__uint_as_float(r[c]));
+                         mine = lane == c ? wm : mine;
                        }
+                       const float old = shift_s[j * 16 + (lane & 15)], now = fminf(old, -(mine * p.scale2));
+                       __syncwarp();
+                       if (lane < 16) shift_s[j * 16 + lane] = now;
+                       if (x != grp) {  // (there is nothing to scale yet in the first tile)
+                         const float f = ex2(now - old);
 #pragma unroll
-                       for (int c = 0; c < 8; ++c) z2[j * 8 + c] = mul2(z2[j * 8 + c], pack2(f[2 * c], f[2 * c + 1]));
+                         for (int c = 0; c < 8; ++c)
+                           z2[j * 8 + c] = mul2(z2[j * 8 + c], pack2(__shfl_sync(0xffffffffu, f, 2 * c), __shfl_sync(0xffffffffu, f, 2 * c + 1)));
+                       }
                        __syncwarp();
                      }
                      exp_accumulate16(r, scale2x, shift2 + j * 8, z2 + j * 8);
@@ -663,12 +668,18 @@ int run_cluster(const CUtensorMap& mk, const CUtensorMap& mq, const ClParams& p,
 
 }  // namespace
 
+// Clusters of each size that the device holds at once, one CTA per SM (cudaOccupancyMaxActiveClusters on a B200; the GPCs are
+// not multiples of every size). Only the choice of a size rests on them.
+constexpr int kClustersAtOnce[kMaxCluster + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
+
 // The cluster size for a shape, or 0 for shapes that two passes over K (score_rows.cu) take in less time. Any size from 1 to
 // 8 works (a unit's tiles are dealt out in equal shares, the last ranks get the remainder).
-//   all logits fit the TMEM of at most 8 CTAs: the smallest size that holds them (llava: 4). Beyond 32 rows, where the
-//     sweeps cost twice as much, not for long units in a call that fills the GPU (64 rows, two passes against this kernel:
-//     1024 units of 4000 keys 364 us against 438, of 2000 219 against 181; 112 of 4000 59 against 61, of 2000 42 against 30;
-//     16 of 8000 29 against 33, of 6000 29 against 19)
+//   all logits fit the TMEM of at most 8 CTAs: the smallest size that holds them (llava: 4), but in a call whose clusters are
+//     all there at once, which lasts as long as one CTA's share, the largest for which they still are and that leaves two tiles
+//     per CTA (4 units of 2000 keys, 32 rows: sizes 1 to 8 take 16.8, 11.4, 9.9, 9.0, 9.2, 8.4, 8.6, 8.3 us; 32 units: 16.9,
+//     11.7, 10.6, 9.8, then 14.0). Beyond 32 rows, where the sweeps cost twice as much, not for long units in several rounds
+//     (64 rows, two passes against this kernel: 1024 units of 4000 keys 364 us against 438, of 2000 219 against 181; 112 of
+//     4000 57 against 58; 56 of 4000 38 against 31, of 8000 55 against 60; 16 of 8000 28 against 31)
 //   longer, up to 32 rows: 6, of which 22 fit the device (132 SMs) and hold more than half as much again as 4 (1024 units of
 //     20480 keys: sizes 3 to 8 take 1278, 1218, 1205, 1163, 1407, 1220 us, two passes 1707; 60 of 131072: 774, 579,
 //     685, 580, 617, 546 against 641; 512 of 30000: 974 against 1242), if the units fill the last round of clusters well enough
@@ -684,11 +695,17 @@ static int cluster_size_for(const madakv_config& c) {
     if (C >= 1 && C <= kMaxCluster && (tiles + C - 1) / C <= slots) return C;
   }
   const long long units = (long long)c.batch * c.n_layers * c.n_kv_heads;
-  if (R > 32 && tiles >= 24 && units * tiles >= 960) return 0;
-  for (int C = 1; C <= kMaxCluster; ++C)
-    if ((tiles + C - 1) / C <= slots) return C;
+  int fit = 1;
+  while (fit <= kMaxCluster && (tiles + fit - 1) / fit > slots) ++fit;
+  if (fit <= kMaxCluster) {
+    const long long rounds = (units + kClustersAtOnce[fit] - 1) / kClustersAtOnce[fit];
+    if (R > 32 && tiles >= 24 && rounds > (fit <= 4 ? 3 : 1)) return 0;
+    for (int C = kMaxCluster; C > fit; --C)
+      if (C != 7 && 2 * (C - 1) < tiles && units <= kClustersAtOnce[C]) return C;
+    return fit;
+  }
   if (R > 32) return 0;
-  const long long round = 132 / kLongCluster, rounds = (units + round - 1) / round;
+  const long long round = kClustersAtOnce[kLongCluster], rounds = (units + round - 1) / round;
   return 5 * units >= 4 * round * rounds ? kLongCluster : 0;
 }
 
