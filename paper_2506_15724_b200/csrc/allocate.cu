@@ -169,73 +169,174 @@ __device__ __forceinline__ uint32_t low_mass(uint32_t key) {
   return (__float_as_uint(t) << 18) + __float_as_uint(__fadd_rz(__fsub_rn(x, __fsub_rn(t, 512.0f)), 0x1p-9f));
 }
 
-// Masses, preference and Eq. 9's counts of one unit, by a team of blocks (see rank_common.cuh). A bucket holds a count and
-// the sum of its keys' masses modulo 2^32, two shared atomics without a result per key. That is enough for the exact mass:
-// all keys of a bucket lie between its two edges, so the mass is count * (mass of the lower edge) plus a remainder below
-// count * (distance of the edges), and the remainder is known exactly where that bound is below 2^32 (it is by a wide
-// margin for importance values: buckets are narrow where the keys are). A unit for which the bound fails anywhere, or with
-// scores of 512 and more, goes the slow way: exact sweeps that halve the range.
+// The ranges Eq. 9's two thresholds can lie in, with the exact masses before them, the masses to reach and the modalities' own.
+struct MassRanges {
+  RankRange r0, r1;
+  u64 above0, above1, need0, need1, W0, W1;
+  bool exact;
+  uint32_t n_vis;  // visual tokens
+  __device__ __forceinline__ bool listed() const { return r0.in <= kListCap && r1.in <= kListCap; }
+  __device__ __forceinline__ bool crowded0() const { return r0.in > kListCap && r0.span > 0; }
+  __device__ __forceinline__ bool crowded1() const { return r1.in > kListCap && r1.span > 0; }
+};
+// The mass to reach, Eq. 9: theta_fix * W has 96 bits; the prefix test  prefix * 2^32 >= theta_fix * W  is
+// prefix >= ceil(theta_fix * W / 2^32)
+__device__ __forceinline__ u64 mass_target(u64 theta_fix, u64 W) {
+  const u64 hi = __umul64hi(theta_fix, W), lo = theta_fix * W;
+  return (hi << 32) + (lo >> 32) + ((lo & 0xffffffffull) ? 1ull : 0ull);
+}
+
+// A bucket holds a count and the sum of its keys' masses modulo 2^32, two shared atomics without a result per key. That is
+// enough for the exact mass: all keys of a bucket lie between its two edges, so the mass is count * (mass of the lower
+// edge) plus a remainder below count * (distance of the edges), and the remainder is known exactly where that bound is
+// below 2^32 (it is by a wide margin for importance values: buckets are narrow where the keys are). A unit for which the
+// bound fails anywhere, or with scores of 512 and more, goes the slow way: exact sweeps that halve the range.
 // (Exact 64-bit masses by atomics that return the old word, to detect carries: alloc 52 us on llava.)
+template <int TEAM>
+__device__ __forceinline__ void add_key(uint32_t* at, uint32_t t) {
+  atomicAdd(at, 1u);
+  atomicAdd(at + 2 * RankShared<TEAM, 2>::kStride, low_mass(kTopKey - t));
+}
 template <int KPT, int TEAM>
-__global__ void __launch_bounds__(kRankThreads, 2) alloc_unit_kernel(const __grid_constant__ AllocParams p) {
+__device__ __forceinline__ void add_first(RankShared<TEAM, 2>& sh, const uint32_t (&t)[KPT], uint32_t vis, uint32_t valid) {
+  constexpr int kStride = RankShared<TEAM, 2>::kStride;
+  if (valid == valid_bits<KPT>(KPT, 0)) {
+#pragma unroll
+    for (int j = 0; j < KPT; ++j) add_key<TEAM>(sh.cnt + ((vis >> j) & 1u ? 0 : kStride) + map_bucket(t[j]), t[j]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < KPT; ++j)
+      if ((valid >> j) & 1u) add_key<TEAM>(sh.cnt + ((vis >> j) & 1u ? 0 : kStride) + map_bucket(t[j]), t[j]);
+  }
+}
+template <int KPT, int TEAM>
+__device__ __forceinline__ void add_again(RankShared<TEAM, 2>& sh, const MassRanges& g, const uint32_t (&t)[KPT], uint32_t vis, int shift0,
+                                          int shift1) {
+#pragma unroll
+  for (int j = 0; j < KPT; ++j) {
+    const bool v = (vis >> j) & 1u;
+    const uint32_t x = t[j] - (v ? g.r0.lo : g.r1.lo);
+    if (x <= (v ? g.r0.span : g.r1.span)) add_key<TEAM>(sh.cnt + (v ? 0 : RankShared<TEAM, 2>::kStride) + (x >> (v ? shift0 : shift1)), t[j]);
+  }
+}
+
+// Walk of the buckets: block r of the team adds up its share of the buckets over all blocks, half of the threads per modality;
+// the ranges shrink to the buckets in which the masses are reached (if all sums are exact).
+template <int TEAM>
+__device__ __forceinline__ void mass_walk(RankShared<TEAM, 2>& sh, uint32_t rank, bool first, u64 theta_fix, MassRanges& g, int shift0, int shift1) {
   using SH = RankShared<TEAM, 2>;
   constexpr int kPer = SH::kPer;
-  __shared__ SH sh;
-  pdl_wait();
-  pdl_go();
-  const uint32_t rank = TEAM > 1 ? team_rank() : 0u;
-  const int u = blockIdx.x / TEAM;
-  const int b = u / (p.Hkv * p.L);
-  const float* psi = p.psi + (int64_t)u * p.n_max;
-  const int mis = (int)(((int64_t)u * p.n_max) & 3);
-  const uint8_t* mask = p.mask + (int64_t)b * p.n_max;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  constexpr int kRound = kRankThreads * KPT;
-  const int rounds = (p.n_max + kRound * TEAM - 1) / (kRound * TEAM);
-  const int pos_first = (int)rank * rounds * kRound + tid * KPT;  // a block owns consecutive positions
-  const int n = clamped_len(p.seq_len, b, p.n_max);
-
-  uint32_t key[KPT], vis = 0;
-  auto load_round = [&](int r) {
-    const int pos0 = pos_first + r * kRound;
-    load_scores<KPT>(psi, mis, p.n_max, pos0, key);
-    vis = load_mask<KPT>(mask, p.n_max, pos0);
-    const uint32_t valid = valid_bits<KPT>(n, pos0);
-    if (valid != valid_bits<KPT>(KPT, 0)) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, m = tid / kHalf, i = tid % kHalf;
+  const uint32_t b0 = (rank * kHalf + i) * kPer;
+  const uint32_t lo = first ? (uint32_t)kMapFirst << kMapShift : (m ? g.r1.lo : g.r0.lo);
+  const int shift = first ? kMapShift : (m ? shift1 : shift0);
+  if (tid == 0) sh.inexact = 0;
+  team_sync<TEAM>();
+  uint32_t c[kPer], s[kPer], lc = 0;
+  u64 q[kPer], lq = 0;
+  bucket_counts<TEAM, 2>(sh, m * SH::kStride + b0, c);
+  bucket_counts<TEAM, 2>(sh, (2 + m) * SH::kStride + b0, s);
+  {
+    auto edge = [&](uint32_t bk) {  // mass of the largest value of bucket bk (the bucket of 512 and more counts as inexact)
+      const u64 t = (u64)lo + ((u64)bk << shift);
+      return t <= kTopKey && !(first && bk >= kBuckets) ? __float2ull_rz(__uint_as_float(kTopKey - (uint32_t)t) * 4294967296.0f) : 0ull;
+    };
+    u64 e = edge(b0);
+    bool bad = false;
 #pragma unroll
-      for (int j = 0; j < KPT; ++j)
-        if (!((valid >> j) & 1u)) key[j] = kNoKey;
+    for (int k = 0; k < kPer; ++k) {
+      const u64 e1 = edge(b0 + k + 1);
+      q[k] = c[k] * e1 + (u64)(s[k] - c[k] * (kLowBias + (uint32_t)e1));
+      bad = bad || c[k] * (e - e1) >> 32;
+      e = e1;
+      lc += c[k];
+      lq += q[k];
     }
-  };
-
-  // ---- range of the keys
-  uint32_t kmax = 0, kmin = 0xffffffffu;
-  for (int r = 0; r < rounds; ++r) {
-    load_round(r);
+    if (bad) {
 #pragma unroll
-    for (int j = 0; j < KPT; ++j) {
-      kmax = (uint32_t)max((int)kmax, (int)key[j]);  // (kNoKey is negative)
-      kmin = min(kmin, key[j]);
+      for (int r = 0; r < TEAM; ++r) peer_store<TEAM>(&sh.inexact, r, 1u);
     }
   }
-  team_range<TEAM, 2>(sh, rank, kmax, kmin);
-  auto to_t = [&]() {
-#pragma unroll
-    for (int j = 0; j < KPT; ++j) key[j] = key[j] == kNoKey ? kNoKey : kmax - key[j];
-  };
-  if (rounds == 1) to_t();
-  auto reload = [&](int r) {
-    if (rounds > 1) {
-      load_round(r);
-      to_t();
+  uint32_t ic = warp_scan32(lc);
+  u64 iq = warp_scan64(lq);
+  if (lane == 31) {
+    sh.wscan_c[warp] = ic;
+    sh.wscan_q[warp] = iq;
+  }
+  __syncthreads();
+  {
+    const bool lower = lane >= m * (kRankWarps / 2) && lane < warp;
+    ic += __reduce_add_sync(kFull, lower ? sh.wscan_c[lane] : 0u);
+    iq += warp_sum64(lower ? sh.wscan_q[lane] : 0ull);
+  }
+  if (i >= kHalf - 32) {  // the last warp of the modality has the block's totals (in its last lane): to every block
+    const uint32_t tc = __shfl_sync(kFull, ic, 31);
+    const u64 tq = __shfl_sync(kFull, iq, 31);
+    if (lane < TEAM) {
+      peer_store<TEAM>(&sh.slice_c[m][rank], lane, tc);
+      peer_store<TEAM>(&sh.slice_q[m][rank], lane, tq);
     }
+  }
+  team_sync<TEAM>();
+  if (TEAM > 1) {
+    const bool lower = lane < (int)rank;
+    ic += __reduce_add_sync(kFull, lower ? sh.slice_c[m][lane] : 0u);
+    iq += warp_sum64(lower ? sh.slice_q[m][lane] : 0ull);
+  }
+  g.exact = sh.inexact == 0;
+  if (first) {
+    g.n_vis = __reduce_add_sync(kFull, lane < TEAM ? sh.slice_c[0][lane] : 0u);
+    g.W0 = warp_sum64(lane < TEAM ? sh.slice_q[0][lane] : 0ull);
+    g.W1 = warp_sum64(lane < TEAM ? sh.slice_q[1][lane] : 0ull);
+    g.need0 = mass_target(theta_fix, g.W0);
+    g.need1 = mass_target(theta_fix, g.W1);
+  }
+  const u64 need = m ? g.need1 : g.need0;
+  ic += m ? g.r1.above : g.r0.above;
+  iq += m ? g.above1 : g.above0;
+  if (need && iq - lq < need && iq >= need) {  // the threshold lies in one of this thread's buckets
+    u64 run = iq - lq, at_q = 0;
+    uint32_t run_c = ic - lc, at = 0, at_c = 0, at_in = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      if (run < need) {
+        at = b0 + k;
+        at_c = run_c;
+        at_in = c[k];
+        at_q = run;
+      }
+      run += q[k];
+      run_c += c[k];
+    }
+#pragma unroll
+    for (int r = 0; r < TEAM; ++r) {
+      peer_store<TEAM>(&sh.first[m], r, ((u64)at_c << 32) | at);
+      peer_store<TEAM>(&sh.last[m], r, (u64)at_in);
+      peer_store<TEAM>(&sh.first_q[m], r, at_q);
+    }
+  }
+  team_sync<TEAM>();
+  auto narrow = [&](RankRange& r, u64& above, u64 need, int q2, int sft) {
+    if (!need) {  // nothing to reach
+      r = RankRange{kNowhere, 0u, 0u, 0u};
+      return;
+    }
+    bucket_range(r, first, (uint32_t)sh.first[q2], sft);
+    r.above = (uint32_t)(sh.first[q2] >> 32);
+    r.in = (uint32_t)sh.last[q2];
+    above = sh.first_q[q2];
   };
-  // the mass to reach, Eq. 9: theta_fix * W has 96 bits; the prefix test  prefix * 2^32 >= theta_fix * W  is
-  // prefix >= ceil(theta_fix * W / 2^32)
-  auto target = [&](u64 W) {
-    const u64 hi = __umul64hi(p.theta_fix, W), lo = p.theta_fix * W;
-    return (hi << 32) + (lo >> 32) + ((lo & 0xffffffffull) ? 1ull : 0ull);
-  };
+  if (g.exact) {
+    narrow(g.r0, g.above0, g.need0, 0, shift0);
+    narrow(g.r1, g.above1, g.need1, 1, shift1);
+  }
+}
+
+// (Rare) too many keys in a range, or sums that were not exact: halve it with exact sweeps until its keys fit the list or
+// are all alike. `sweep` calls its argument with the keys of the thread, some at a time.
+template <int TEAM, typename Sweep>
+__device__ __forceinline__ void mass_bisect(RankShared<TEAM, 2>& sh, uint32_t rank, u64 theta_fix, MassRanges& g, Sweep sweep) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // sums over the team, into every thread (of values that are already summed up over the warp)
   auto team_sums = [&](u64& a0, u64& a1) {
     __syncthreads();
@@ -257,251 +358,87 @@ __global__ void __launch_bounds__(kRankThreads, 2) alloc_unit_kernel(const __gri
     a1 = warp_sum64(lane < TEAM ? sh.slice_q[1][lane] : 0ull);
     team_sync<TEAM>();
   };
-
-  const uint32_t all_span = kmax - kmin;
-  RankRange r0{0u, all_span, kNoKey, 0u}, r1 = r0;
-  u64 above0 = 0, above1 = 0;  // exact mass before r0.lo, r1.lo
-  u64 need0 = 0, need1 = 0, W0 = 0, W1 = 0;
-  bool exact = kmax < kSmallKey;
-  uint32_t n_vis = 0;  // visual tokens
-
-  for (int pass = 0; pass < 2 && exact; ++pass) {
-    // ---- buckets
-    const int shift0 = range_shift(r0.span, SH::kDig), shift1 = range_shift(r1.span, SH::kDig);
-    if (pass == 0) {  // all keys take part, both modalities over the same range
-      for (int r = 0; r < rounds; ++r) {
-        reload(r);
-#pragma unroll
-        for (int j = 0; j < KPT; ++j) {
-          uint32_t* at = sh.cnt + ((vis >> j) & 1u ? 0 : SH::kStride) + min(key[j] >> shift0, (uint32_t)SH::kBuckets);
-          atomicAdd(at, 1u);
-          atomicAdd(at + 2 * SH::kStride, low_mass(kmax - key[j]));
-        }
-      }
-    } else {
-      for (int x = tid; x < 4 * SH::kStride / 4; x += kRankThreads) reinterpret_cast<uint4*>(sh.cnt)[x] = make_uint4(0, 0, 0, 0);
-      __syncthreads();
-      for (int r = 0; r < rounds; ++r) {
-        reload(r);
-#pragma unroll
-        for (int j = 0; j < KPT; ++j) {
-          const bool v = (vis >> j) & 1u;
-          const uint32_t x = key[j] - (v ? r0.lo : r1.lo);
-          if (x <= (v ? r0.span : r1.span)) {
-            uint32_t* at = sh.cnt + (v ? 0 : SH::kStride) + (x >> (v ? shift0 : shift1));
-            atomicAdd(at, 1u);
-            atomicAdd(at + 2 * SH::kStride, low_mass(kmax - key[j]));
-          }
-        }
-      }
-    }
-    // ---- walk: block r of the team adds up its share of the buckets over all blocks; half of the threads per modality
-    const int m = tid / kHalf, i = tid % kHalf;
-    const uint32_t b0 = (rank * kHalf + i) * kPer;
-    const RankRange my = m ? r1 : r0;
-    const int shift = m ? shift1 : shift0;
-    if (tid == 0) sh.inexact = 0;
-    team_sync<TEAM>();
-    uint32_t c[kPer], s[kPer], lc = 0;
-    u64 q[kPer], lq = 0;
-    bucket_counts<TEAM, 2>(sh, m * SH::kStride + b0, c);
-    bucket_counts<TEAM, 2>(sh, (2 + m) * SH::kStride + b0, s);
-    {
-      auto edge = [&](uint32_t bk) {  // mass of the largest value of bucket bk
-        const u64 t = (u64)my.lo + ((u64)bk << shift);
-        return t <= kmax ? __float2ull_rz(__uint_as_float(kmax - (uint32_t)t) * 4294967296.0f) : 0ull;
-      };
-      u64 e = edge(b0);
-      bool bad = false;
-#pragma unroll
-      for (int k = 0; k < kPer; ++k) {
-        const u64 e1 = edge(b0 + k + 1);
-        q[k] = c[k] * e1 + (u64)(s[k] - c[k] * (kLowBias + (uint32_t)e1));
-        bad = bad || c[k] * (e - e1) >> 32;
-        e = e1;
-        lc += c[k];
-        lq += q[k];
-      }
-      if (bad) {
-#pragma unroll
-        for (int r = 0; r < TEAM; ++r) peer_store<TEAM>(&sh.inexact, r, 1u);
-      }
-    }
-    uint32_t ic = warp_scan32(lc);
-    u64 iq = warp_scan64(lq);
-    if (lane == 31) {
-      sh.wscan_c[warp] = ic;
-      sh.wscan_q[warp] = iq;
-    }
-    __syncthreads();
-    {
-      const bool lower = lane >= m * (kRankWarps / 2) && lane < warp;
-      ic += __reduce_add_sync(kFull, lower ? sh.wscan_c[lane] : 0u);
-      iq += warp_sum64(lower ? sh.wscan_q[lane] : 0ull);
-    }
-    if (i >= kHalf - 32) {  // the last warp of the modality has the block's totals (in its last lane): to every block
-      const uint32_t tc = __shfl_sync(kFull, ic, 31);
-      const u64 tq = __shfl_sync(kFull, iq, 31);
-      if (lane < TEAM) {
-        peer_store<TEAM>(&sh.slice_c[m][rank], lane, tc);
-        peer_store<TEAM>(&sh.slice_q[m][rank], lane, tq);
-      }
-    }
-    team_sync<TEAM>();
-    if (TEAM > 1) {
-      const bool lower = lane < (int)rank;
-      ic += __reduce_add_sync(kFull, lower ? sh.slice_c[m][lane] : 0u);
-      iq += warp_sum64(lower ? sh.slice_q[m][lane] : 0ull);
-    }
-    exact = sh.inexact == 0;
-    if (pass == 0) {
-      n_vis = __reduce_add_sync(kFull, lane < TEAM ? sh.slice_c[0][lane] : 0u);
-      W0 = warp_sum64(lane < TEAM ? sh.slice_q[0][lane] : 0ull);
-      W1 = warp_sum64(lane < TEAM ? sh.slice_q[1][lane] : 0ull);
-      need0 = target(W0);
-      need1 = target(W1);
-    }
-    const u64 need = m ? need1 : need0;
-    ic += my.above;
-    iq += m ? above1 : above0;
-    if (need && iq - lq < need && iq >= need) {  // the threshold lies in one of this thread's buckets
-      u64 run = iq - lq, at_q = 0;
-      uint32_t run_c = ic - lc, at = 0, at_c = 0, at_in = 0;
-#pragma unroll
-      for (int k = 0; k < kPer; ++k) {
-        if (run < need) {
-          at = b0 + k;
-          at_c = run_c;
-          at_in = c[k];
-          at_q = run;
-        }
-        run += q[k];
-        run_c += c[k];
-      }
-#pragma unroll
-      for (int r = 0; r < TEAM; ++r) {
-        peer_store<TEAM>(&sh.first[m], r, ((u64)at_c << 32) | at);
-        peer_store<TEAM>(&sh.last[m], r, (u64)at_in);
-        peer_store<TEAM>(&sh.first_q[m], r, at_q);
-      }
-    }
-    team_sync<TEAM>();
-    auto narrow = [&](RankRange& g, u64& above, u64 need, int q2, int sft) {
-      if (!need) {  // nothing to reach
-        g = RankRange{kNowhere, 0u, 0u, 0u};
-        return;
-      }
-      const uint32_t cut = (uint32_t)sh.first[q2] << sft;
-      g.span = min(g.span - cut, (1u << sft) - 1u);
-      g.lo += cut;
-      g.above = (uint32_t)(sh.first[q2] >> 32);
-      g.in = (uint32_t)sh.last[q2];
-      above = sh.first_q[q2];
-    };
-    if (exact) {
-      narrow(r0, above0, need0, 0, shift0);
-      narrow(r1, above1, need1, 1, shift1);
-      if (r0.in <= kListCap && r1.in <= kListCap) break;
-    }
-  }
-
-  // ---- (rare) too many keys in a range, or sums that were not exact: halve it with exact sweeps until its keys fit the
-  // list or are all alike
-  auto crowded = [](const RankRange& g) { return g.in > kListCap && g.span > 0; };
-  if (!exact) {
-    W0 = W1 = 0;
+  if (!g.exact) {
+    u64 W0 = 0, W1 = 0;
     uint32_t c0 = 0, c1 = 0;
-    for (int r = 0; r < rounds; ++r) {
-      reload(r);
-#pragma unroll
-      for (int j = 0; j < KPT; ++j)
-        if (key[j] != kNoKey) {
-          const u64 q = psi_fix(kmax - key[j]);
-          if ((vis >> j) & 1u) { W0 += q; ++c0; } else { W1 += q; ++c1; }
-        }
-    }
+    sweep([&](uint32_t t, bool v) {
+      if (t != kNoKey) {
+        const u64 q = psi_fix(kTopKey - t);
+        if (v) { W0 += q; ++c0; } else { W1 += q; ++c1; }
+      }
+    });
     W0 = warp_sum64(W0);
     W1 = warp_sum64(W1);
     team_sums(W0, W1);
     u64 n0 = __reduce_add_sync(kFull, c0), n1 = __reduce_add_sync(kFull, c1);
     team_sums(n0, n1);
-    n_vis = (uint32_t)n0;
-    need0 = target(W0);
-    need1 = target(W1);
-    r0 = need0 ? RankRange{0u, all_span, (uint32_t)n0, 0u} : RankRange{kNowhere, 0u, 0u, 0u};
-    r1 = need1 ? RankRange{0u, all_span, (uint32_t)n1, 0u} : RankRange{kNowhere, 0u, 0u, 0u};
-    above0 = above1 = 0;
+    g.n_vis = (uint32_t)n0;
+    g.W0 = W0;
+    g.W1 = W1;
+    g.need0 = mass_target(theta_fix, W0);
+    g.need1 = mass_target(theta_fix, W1);
+    g.r0 = g.need0 ? RankRange{0u, kTopKey, (uint32_t)n0, 0u} : RankRange{kNowhere, 0u, 0u, 0u};
+    g.r1 = g.need1 ? RankRange{0u, kTopKey, (uint32_t)n1, 0u} : RankRange{kNowhere, 0u, 0u, 0u};
+    g.above0 = g.above1 = 0;
   }
-  while (crowded(r0) || crowded(r1)) {
-    const bool on0 = crowded(r0), on1 = crowded(r1);
-    const uint32_t mid0 = r0.lo + (r0.span >> 1), mid1 = r1.lo + (r1.span >> 1);
+  while (g.crowded0() || g.crowded1()) {
+    const bool on0 = g.crowded0(), on1 = g.crowded1();
+    const uint32_t mid0 = g.r0.lo + (g.r0.span >> 1), mid1 = g.r1.lo + (g.r1.span >> 1);
     u64 a0 = 0, a1 = 0;
     uint32_t c0 = 0, c1 = 0;
-    for (int r = 0; r < rounds; ++r) {
-      reload(r);
-#pragma unroll
-      for (int j = 0; j < KPT; ++j) {
-        const bool v = (vis >> j) & 1u;
-        if ((v ? on0 : on1) && key[j] >= (v ? r0.lo : r1.lo) && key[j] <= (v ? mid0 : mid1)) {
-          const u64 q = psi_fix(kmax - key[j]);
-          if (v) { a0 += q; ++c0; } else { a1 += q; ++c1; }
-        }
+    sweep([&](uint32_t t, bool v) {
+      if ((v ? on0 : on1) && t >= (v ? g.r0.lo : g.r1.lo) && t <= (v ? mid0 : mid1)) {
+        const u64 q = psi_fix(kTopKey - t);
+        if (v) { a0 += q; ++c0; } else { a1 += q; ++c1; }
       }
-    }
+    });
     a0 = warp_sum64(a0);
     a1 = warp_sum64(a1);
     team_sums(a0, a1);
     u64 n0 = __reduce_add_sync(kFull, c0), n1 = __reduce_add_sync(kFull, c1);
     team_sums(n0, n1);
-    auto halve = [](RankRange& g, u64& above, u64 need, u64 a, uint32_t c) {
-      const uint32_t half = g.span >> 1;
+    auto halve = [](RankRange& r, u64& above, u64 need, u64 a, uint32_t c) {
+      const uint32_t half = r.span >> 1;
       if (above + a >= need) {
-        g.span = half;
-        g.in = c;
+        r.span = half;
+        r.in = c;
       } else {
         above += a;
-        g.above += c;
-        g.in -= c;
-        g.lo += half + 1;
-        g.span -= half + 1;
+        r.above += c;
+        r.in -= c;
+        r.lo += half + 1;
+        r.span -= half + 1;
       }
     };
-    if (on0) halve(r0, above0, need0, a0, (uint32_t)n0);
-    if (on1) halve(r1, above1, need1, a1, (uint32_t)n1);
+    if (on0) halve(g.r0, g.above0, g.need0, a0, (uint32_t)n0);
+    if (on1) halve(g.r1, g.above1, g.need1, a1, (uint32_t)n1);
   }
+}
+
+// With the candidates of all blocks in their lists: block 0 finds the counts and writes the unit's results; the unit that is
+// done last goes on with its sequence.
+template <int TEAM>
+__device__ __forceinline__ void mass_finish(RankShared<TEAM, 2>& sh, const AllocParams& p, uint32_t rank, int u, int b, int n, const MassRanges& g) {
+  const int tid = threadIdx.x;
   if (rank == 0 && tid < 2) {
-    const u64 W = tid ? W1 : W0, tot = W0 + W1;
+    const u64 W = tid ? g.W1 : g.W0, tot = g.W0 + g.W1;
     p.mass[(int64_t)u * 2 + tid] = __ull2double_rn(W) / 4294967296.0;
     p.pref[(int64_t)u * 2 + tid] = tot ? __ddiv_rn(__ull2double_rn(W), __ull2double_rn(tot)) : 0.0;
-    if ((tid ? need1 : need0) == 0) p.demand[(int64_t)u * 2 + tid] = 0;
-  }
-
-  // ---- the keys inside the ranges
-  for (int r = 0; r < rounds; ++r) {
-    reload(r);
-    uint32_t in = 0;
-#pragma unroll
-    for (int j = 0; j < KPT; ++j) {
-      const bool v = (vis >> j) & 1u;
-      if (key[j] - (v ? r0.lo : r1.lo) <= (v ? r0.span : r1.span)) in |= 1u << j;
-    }
-    append<TEAM, 2, KPT>(sh, r0.in <= kListCap ? in & vis : 0u, r1.in <= kListCap ? in & ~vis : 0u, key, r0.lo, r1.lo);
+    if ((tid ? g.need1 : g.need0) == 0) p.demand[(int64_t)u * 2 + tid] = 0;
   }
   team_sync<TEAM>();
-
-  // ---- finish: block 0
   if (rank == 0) {
     const uint32_t got = gather_lists<TEAM, 2>(sh);
-    const bool on0 = need0 && r0.in <= kListCap, on1 = need1 && r1.in <= kListCap;
-    finish_lists<TEAM, 2, true>(sh, r0, r1, got, on0, on1, need0, need1, above0, above1, kmax);
-    if (tid < 2 && (tid ? need1 : need0)) {
-      // every key left has the value kmax - t: as few of them as reach the threshold
-      const RankRange my = tid ? r1 : r0;
+    const bool on0 = g.need0 && g.r0.in <= kListCap, on1 = g.need1 && g.r1.in <= kListCap;
+    finish_lists<TEAM, 2, true>(sh, g.r0, g.r1, got, on0, on1, g.need0, g.need1, g.above0, g.above1);
+    if (tid < 2 && (tid ? g.need1 : g.need0)) {
+      // every key left has the value kTopKey - t: as few of them as reach the threshold
+      const RankRange my = tid ? g.r1 : g.r0;
       const bool listed = tid ? on1 : on0;
       uint32_t take = listed ? sh.fin_in[tid] : my.in;
       if (take > 1) {
-        const u64 need = tid ? need1 : need0, above = listed ? sh.fin_m[tid] : (tid ? above1 : above0);
-        const u64 each = psi_fix(kmax - (listed ? sh.fin_lo[tid] : my.lo));
+        const u64 need = tid ? g.need1 : g.need0, above = listed ? sh.fin_m[tid] : (tid ? g.above1 : g.above0);
+        const u64 each = psi_fix(kTopKey - (listed ? sh.fin_lo[tid] : my.lo));
         if (each > 0) {
           const u64 k = (need - above + each - 1) / each;
           if (k < (u64)take) take = (uint32_t)k;
@@ -511,7 +448,6 @@ __global__ void __launch_bounds__(kRankThreads, 2) alloc_unit_kernel(const __gri
     }
   }
   if (TEAM > 1) team_sync<TEAM>();  // no block leaves while block 0 still reads its shared memory
-  // ---- the unit that is done last goes on with its sequence
   if (rank != 0 || !p.counter) return;
   __shared__ unsigned s_last;
   __syncthreads();
@@ -523,7 +459,134 @@ __global__ void __launch_bounds__(kRankThreads, 2) alloc_unit_kernel(const __gri
   __syncthreads();
   if (s_last != (unsigned)(p.L * p.Hkv) - 1u) return;
   static_assert(sizeof(sh.cnt) >= kLayerChunk * 16, "the scan reuses the buckets");
-  sequence_budgets(p, b, n, (int)n_vis, reinterpret_cast<double*>(sh.cnt), reinterpret_cast<long long*>(sh.cnt) + kLayerChunk);
+  sequence_budgets(p, b, n, (int)g.n_vis, reinterpret_cast<double*>(sh.cnt), reinterpret_cast<long long*>(sh.cnt) + kLayerChunk);
+}
+
+// t of KPT consecutive positions (kNoKey outside the sequence); returns those that are inside.
+template <int KPT>
+__device__ __forceinline__ uint32_t load_valid(const float* psi, int mis, int n_max, int n, int pos0, uint32_t (&t)[KPT]) {
+  load_scores<KPT>(psi, mis, n_max, pos0, t);
+  const uint32_t valid = valid_bits<KPT>(n, pos0);
+  if (valid != valid_bits<KPT>(KPT, 0)) {
+#pragma unroll
+    for (int j = 0; j < KPT; ++j)
+      if (!((valid >> j) & 1u)) t[j] = kNoKey;
+  }
+  return valid;
+}
+
+// Masses, preference and Eq. 9's counts of one unit whose keys fit the registers of its team (see rank_common.cuh).
+template <int KPT, int TEAM>
+__global__ void __launch_bounds__(kRankThreads, 2) alloc_unit_kernel(const __grid_constant__ AllocParams p) {
+  __shared__ RankShared<TEAM, 2> sh;
+  pdl_wait();
+  pdl_go();
+  const uint32_t rank = TEAM > 1 ? team_rank() : 0u;
+  const int u = blockIdx.x / TEAM, b = u / (p.Hkv * p.L);
+  const int n = clamped_len(p.seq_len, b, p.n_max);
+  const int pos0 = (int)rank * kRankThreads * KPT + threadIdx.x * KPT;  // a block owns consecutive positions
+  uint32_t t[KPT];
+  const uint32_t valid = load_valid<KPT>(p.psi + (int64_t)u * p.n_max, (int)(((int64_t)u * p.n_max) & 3), p.n_max, n, pos0, t);
+  const uint32_t vis = load_mask<KPT>(p.mask + (int64_t)b * p.n_max, p.n_max, pos0);
+  zero_buckets<TEAM, 2>(sh);
+  add_first<KPT, TEAM>(sh, t, vis, valid);
+  MassRanges g = {};
+  mass_walk<TEAM>(sh, rank, true, p.theta_fix, g, 0, 0);
+  if (!g.exact || !g.listed()) {
+    if (g.exact) {
+      const int shift0 = range_shift(g.r0.span, kDig), shift1 = range_shift(g.r1.span, kDig);
+      zero_buckets<TEAM, 2>(sh);
+      add_again<KPT, TEAM>(sh, g, t, vis, shift0, shift1);
+      mass_walk<TEAM>(sh, rank, false, p.theta_fix, g, shift0, shift1);
+    }
+    mass_bisect<TEAM>(sh, rank, p.theta_fix, g, [&](auto each) {
+#pragma unroll
+      for (int j = 0; j < KPT; ++j) each(t[j], (vis >> j) & 1u);
+    });
+  }
+  uint32_t in = 0;
+#pragma unroll
+  for (int j = 0; j < KPT; ++j) {
+    const bool v = (vis >> j) & 1u;
+    if (t[j] - (v ? g.r0.lo : g.r1.lo) <= (v ? g.r0.span : g.r1.span)) in |= 1u << j;
+  }
+  append<TEAM, 2, KPT>(sh, g.r0.in <= kListCap ? in & vis : 0u, g.r1.in <= kListCap ? in & ~vis : 0u, t, g.r0.lo, g.r1.lo);
+  mass_finish<TEAM>(sh, p, rank, u, b, n, g);
+}
+
+// The same for a longer unit, which is read twice, for the buckets and for the candidates (listed as positions); the mask is
+// kept as bits in shared memory. (256 units of 131072 keys: 111 us; 153 with three sweeps over keys and mask.)
+template <int TEAM>
+__global__ void __launch_bounds__(kRankThreads, 2) alloc_long_kernel(const __grid_constant__ AllocParams p) {
+  constexpr int KPT = 16, kRound = kRankThreads * KPT;
+  __shared__ RankShared<TEAM, 2> sh;
+  extern __shared__ __align__(16) uint32_t bits[];
+  pdl_wait();
+  pdl_go();
+  const uint32_t rank = TEAM > 1 ? team_rank() : 0u;
+  const int tid = threadIdx.x, u = blockIdx.x / TEAM, b = u / (p.Hkv * p.L);
+  const int n = clamped_len(p.seq_len, b, p.n_max);
+  const float* psi = p.psi + (int64_t)u * p.n_max;
+  const int mis = (int)(((int64_t)u * p.n_max) & 3);
+  const uint8_t* mask = p.mask + (int64_t)b * p.n_max;
+  uint32_t *pos0 = bits, *pos1 = bits + kListCap, *vis_w = bits + 2 * kListCap;
+  const int rounds = (n + kRound * TEAM - 1) / (kRound * TEAM);
+  const int start = (int)rank * rounds * kRound;  // a block owns consecutive positions
+  zero_buckets<TEAM, 2>(sh);
+#pragma unroll 1
+  for (int r = 0; r < rounds; ++r) {
+    const int at = start + r * kRound + tid * KPT;
+    uint32_t t[KPT];
+    const uint32_t valid = load_valid<KPT>(psi, mis, p.n_max, n, at, t);
+    const uint32_t vis = load_mask<KPT>(mask, p.n_max, at);
+    bits_of_thread(vis_w, r) = (uint16_t)vis;
+    add_first<KPT, TEAM>(sh, t, vis, valid);
+  }
+  MassRanges g = {};
+  mass_walk<TEAM>(sh, rank, true, p.theta_fix, g, 0, 0);
+  if (!g.exact || !g.listed()) {
+    if (g.exact) {
+      const int shift0 = range_shift(g.r0.span, kDig), shift1 = range_shift(g.r1.span, kDig);
+      zero_buckets<TEAM, 2>(sh);
+#pragma unroll 1
+      for (int r = 0; r < rounds; ++r) {
+        uint32_t t[KPT];
+        load_valid<KPT>(psi, mis, p.n_max, n, start + r * kRound + tid * KPT, t);
+        add_again<KPT, TEAM>(sh, g, t, bits_of_thread(vis_w, r), shift0, shift1);
+      }
+      mass_walk<TEAM>(sh, rank, false, p.theta_fix, g, shift0, shift1);
+    }
+    mass_bisect<TEAM>(sh, rank, p.theta_fix, g, [&](auto each) {
+#pragma unroll 1
+      for (int r = 0; r < rounds; ++r) {
+        uint32_t t[KPT];
+        load_valid<KPT>(psi, mis, p.n_max, n, start + r * kRound + tid * KPT, t);
+        const uint32_t vis = bits_of_thread(vis_w, r);
+#pragma unroll
+        for (int j = 0; j < KPT; ++j) each(t[j], (vis >> j) & 1u);
+      }
+    });
+  }
+  const bool on0 = g.r0.in <= kListCap, on1 = g.r1.in <= kListCap;
+#pragma unroll 1
+  for (int r = 0; r < rounds; ++r) {
+    const int at = r * kRound + tid * KPT;
+    uint32_t t[KPT];
+    load_valid<KPT>(psi, mis, p.n_max, n, start + at, t);
+    const uint32_t vis = bits_of_thread(vis_w, r);
+    uint32_t in = 0;
+#pragma unroll
+    for (int j = 0; j < KPT; ++j) {
+      const bool v = (vis >> j) & 1u;
+      if (t[j] - (v ? g.r0.lo : g.r1.lo) <= (v ? g.r0.span : g.r1.span)) in |= 1u << j;
+    }
+    append_positions<TEAM, 2>(sh, pos0, pos1, on0 ? in & vis : 0u, on1 ? in & ~vis : 0u, at);
+  }
+  __syncthreads();
+  const int m = tid / kHalf, mine_n = m ? sh.list_n >> 16 : sh.list_n & 0xffffu;
+  for (int i = tid % kHalf; i < mine_n; i += kHalf)
+    sh.list[m][i] = score_t(__ldg(psi + start + (m ? pos1 : pos0)[i])) - (m ? g.r1.lo : g.r0.lo);
+  mass_finish<TEAM>(sh, p, rank, u, b, n, g);
 }
 
 // The same as a kernel of its own, one block per sequence: for the budgets of one layer whose masses and demands are given
@@ -545,17 +608,29 @@ __global__ void __launch_bounds__(1024) alloc_seq_kernel(const __grid_constant__
   sequence_budgets(p, b, n, s_nv, s_phi, s_dem);
 }
 
+template <int TEAM>
+void launch_alloc_long(const AllocParams& p, int units, cudaStream_t st) {
+  auto kern = alloc_long_kernel<TEAM>;
+  // (the largest of any call, so that threads with calls of different sizes do not take the room from one another; a failure
+  // shows at the launch)
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (2 * kListCap + long_words(kLongKeys, 1)) * 4);
+  launch_team(kern, units, TEAM, (size_t)(2 * kListCap + long_words(p.n_max, TEAM)) * 4, st, p);
+}
 void launch_alloc_units(const madakv_config& c, const AllocParams& p, int units, cudaStream_t st) {
   const RankShape s = rank_shape(units, c.max_seq_len);
-  switch (s.kpt + s.team) {
-    case 8 + 1: launch_team(alloc_unit_kernel<8, 1>, units, 1, st, p); break;
-    case 8 + 2: launch_team(alloc_unit_kernel<8, 2>, units, 2, st, p); break;
-    case 8 + 4: launch_team(alloc_unit_kernel<8, 4>, units, 4, st, p); break;
-    case 8 + 8: launch_team(alloc_unit_kernel<8, 8>, units, 8, st, p); break;
-    case 16 + 1: launch_team(alloc_unit_kernel<16, 1>, units, 1, st, p); break;
-    case 16 + 2: launch_team(alloc_unit_kernel<16, 2>, units, 2, st, p); break;
-    case 16 + 4: launch_team(alloc_unit_kernel<16, 4>, units, 4, st, p); break;
-    default: launch_team(alloc_unit_kernel<16, 8>, units, 8, st, p); break;
+  switch (s.kpt * 16 + s.team) {
+    case 8 * 16 + 1: launch_team(alloc_unit_kernel<8, 1>, units, 1, 0, st, p); break;
+    case 8 * 16 + 2: launch_team(alloc_unit_kernel<8, 2>, units, 2, 0, st, p); break;
+    case 8 * 16 + 4: launch_team(alloc_unit_kernel<8, 4>, units, 4, 0, st, p); break;
+    case 8 * 16 + 8: launch_team(alloc_unit_kernel<8, 8>, units, 8, 0, st, p); break;
+    case 16 * 16 + 1: launch_team(alloc_unit_kernel<16, 1>, units, 1, 0, st, p); break;
+    case 16 * 16 + 2: launch_team(alloc_unit_kernel<16, 2>, units, 2, 0, st, p); break;
+    case 16 * 16 + 4: launch_team(alloc_unit_kernel<16, 4>, units, 4, 0, st, p); break;
+    case 16 * 16 + 8: launch_team(alloc_unit_kernel<16, 8>, units, 8, 0, st, p); break;
+    case 1: launch_alloc_long<1>(p, units, st); break;
+    case 2: launch_alloc_long<2>(p, units, st); break;
+    case 4: launch_alloc_long<4>(p, units, st); break;
+    default: launch_alloc_long<8>(p, units, st); break;
   }
 }
 

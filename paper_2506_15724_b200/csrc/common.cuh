@@ -215,10 +215,10 @@ __device__ __forceinline__ int clamped_len(const int32_t* seq_len, int b, int n_
   return max(0, min(seq_len[b], n_max));
 }
 __device__ __forceinline__ uint32_t psi_key(float x) { return x > 0.0f ? __float_as_uint(x) : 0u; }
-// Bit i of the result: byte i of the word is not zero (four mask bytes at a time).
+// Bit i of the result: byte i of the word is not zero (four mask bytes at a time). The product brings bits 7, 15, 23 and 31
+// to the top, its other partial products fall on different bits below.
 __device__ __forceinline__ uint32_t nonzero_bytes(uint32_t w) {
-  const uint32_t x = ((((w & 0x7f7f7f7fu) + 0x7f7f7f7fu) | w) & 0x80808080u) >> 7;  // bits 0, 8, 16, 24
-  return (x & 1u) | ((x >> 7) & 2u) | ((x >> 14) & 4u) | ((x >> 21) & 8u);
+  return (((((w & 0x7f7f7f7fu) + 0x7f7f7f7fu) | w) & 0x80808080u) * 0x00204081u) >> 28;
 }
 // floor(x * 2^32) of a key produced by psi_key, by shifting the 24-bit significand into place (the conversion instruction
 // gives the same number but runs at a small fraction of the rate of integer instructions): exponent field e stands for

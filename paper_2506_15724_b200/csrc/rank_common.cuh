@@ -3,19 +3,19 @@
 //
 // A unit's keys sit in registers (KPT consecutive positions per thread); a long unit in a call with few units is spread over
 // a thread-block cluster, whose blocks exchange their partial results through distributed shared memory, and a unit
-// longer than its blocks' registers is read again from L2 in every sweep (see rank_shape). The threshold (the budget-th
+// longer than its blocks' registers is read twice by a kernel of its own (see rank_shape). The threshold (the budget-th
 // largest key, or the key at which a mass is reached) is found in few steps. Two things bound these kernels: the integer
 // instructions per key in calls with many units (an SM has some 230 000 keys of 256 units of 131072 keys to handle), and the
-// fixed latency of a step (barriers, walking the buckets) in calls with few. Three sweeps over the keys instead of the four
-// or five passes of a plain radix descent, and no shared atomic that returns a value, took allocation + selection from
-// 162 + 295 to 153 + 185 us on 256 units of 131072 keys, from 52 + 48 to 50 + 37 on 1024 units of 8192 and from 30 + 54 to 13 + 11
-// on 4 units of 32768.
-//   range    largest and smallest key; digits are taken from t = kmax - key (ascending t is descending importance),
-//            because importance values share their sign and most exponent bits
-//   buckets  a count (and for Eq. 9 a mass, see allocate.cu) per key into 2048 buckets over the range; a walk of the
-//            buckets narrows the range of t that the threshold can lie in to one bucket, usually some tens of keys
+// fixed latency of a step (barriers, walking the buckets) in calls with few.
+//   buckets  a count (and for Eq. 9 a mass, see allocate.cu) per key into 2048 buckets that are the same for all units, by
+//            shared atomics without a result; a walk of the buckets narrows the range that the threshold can lie in to one
+//            bucket, usually some tens of keys
 //   list     the keys of the narrowed range are collected in shared memory, where half of a block's threads per modality
 //            lay buckets over them once more; the few keys left are compared with one another
+// Buckets over the range of each unit's keys needed a sweep for that range before; without it, and with long units read
+// twice instead of three (allocation) or four times (selection), allocation + selection + compaction went from 602 to 483 us
+// on 256 units of 131072 keys, from 618 to 523 on 1600 of 13411, from 213 to 161 on 3360 of 471, from 31 to 26 on 200 of 772.
+// (The same in four or five passes of a plain radix descent: 750 us on the first of these.)
 // Keys that crowd (many ties, a few values far away from all others) make the list overflow; then the buckets are laid
 // over the narrowed range once more, and after that the range is bisected with exact sweeps over all keys, which ends
 // for any input, at the latest when the range holds one value.
@@ -33,6 +33,7 @@ constexpr int kHalf = kRankThreads / 2;        // threads per modality in the wa
 constexpr int kListCap = 1024;                 // candidates per modality
 constexpr int kFewCap = 32;                    // candidates compared with one another
 constexpr int kMaxTeam = 8;
+constexpr uint32_t kTopKey = 0x7f81ffffu;      // t = kTopKey - key: ascending t is descending importance
 constexpr uint32_t kNoKey = 0xffffffffu;       // t of a slot without a key
 constexpr uint32_t kNowhere = 0xfffffffeu;     // start of a range that holds no t at all (t < 2^31)
 typedef unsigned long long u64;
@@ -111,18 +112,18 @@ __device__ __forceinline__ u64 warp_scan64(u64 v) {
 // Rows of odd lengths start anywhere: scores are read in aligned 16-byte pieces and moved down by `mis` elements
 // (the same for the whole unit), mask bytes in aligned words and funnel shifts; only threads at the ends of a row go
 // element by element.
-// A score becomes an order-preserving key: its bits where it is positive, else (NaN too) 0.
-__device__ __forceinline__ uint32_t score_key(float x) { return __float_as_uint(fmaxf(x, 0.0f)); }
+// A score's order-preserving key is its bits where it is positive, else (NaN too) 0; kept is t, its distance from kTopKey.
+__device__ __forceinline__ uint32_t score_t(float x) { return kTopKey - __float_as_uint(fmaxf(x, 0.0f)); }
 template <int KPT>
-__device__ __forceinline__ void load_scores(const float* row, int mis, int n_max, int pos0, uint32_t (&key)[KPT]) {
+__device__ __forceinline__ void load_scores(const float* row, int mis, int n_max, int pos0, uint32_t (&t)[KPT]) {
   if (mis == 0 && pos0 + KPT <= n_max) {
 #pragma unroll
     for (int j = 0; j < KPT; j += 4) {
       const float4 v = __ldg(reinterpret_cast<const float4*>(row + pos0 + j));
-      key[j] = score_key(v.x);
-      key[j + 1] = score_key(v.y);
-      key[j + 2] = score_key(v.z);
-      key[j + 3] = score_key(v.w);
+      t[j] = score_t(v.x);
+      t[j + 1] = score_t(v.y);
+      t[j + 2] = score_t(v.z);
+      t[j + 3] = score_t(v.w);
     }
   } else if (mis != 0 && pos0 + KPT + 4 <= n_max) {
     // (a misaligned row has a unit before it: the pieces start inside the array; they end inside the row)
@@ -139,10 +140,10 @@ __device__ __forceinline__ void load_scores(const float* row, int mis, int n_max
 #pragma unroll
     for (int j = 0; j < KPT + 3; ++j) f[j] = (mis & 1) ? f[j + 1] : f[j];
 #pragma unroll
-    for (int j = 0; j < KPT; ++j) key[j] = score_key((mis & 2) ? f[j + 2] : f[j]);
+    for (int j = 0; j < KPT; ++j) t[j] = score_t((mis & 2) ? f[j + 2] : f[j]);
   } else {
 #pragma unroll
-    for (int j = 0; j < KPT; ++j) key[j] = pos0 + j < n_max ? score_key(__ldg(row + pos0 + j)) : 0u;
+    for (int j = 0; j < KPT; ++j) t[j] = pos0 + j < n_max ? score_t(__ldg(row + pos0 + j)) : kTopKey;
   }
 }
 template <int KPT>
@@ -184,19 +185,30 @@ __device__ __forceinline__ uint32_t load_mask(const uint8_t* row, int n_max, int
   }
   return vis;
 }
+// Bits of a long unit in shared memory, one per position of the block: word w sits at w + w / 32, so that threads that walk
+// several consecutive words each hit different banks. A thread's 16 positions of round r are half a word.
+__device__ __forceinline__ int bits_slot(int w) { return w + (w >> 5); }
+__device__ __forceinline__ uint16_t& bits_of_thread(uint32_t* words, int r) {
+  const int half = r * kRankThreads + threadIdx.x;
+  return reinterpret_cast<uint16_t*>(words)[2 * bits_slot(half >> 1) + (half & 1)];
+}
 template <int KPT>
 __device__ __forceinline__ uint32_t valid_bits(int n, int pos0) {  // bit j: position pos0 + j lies inside the sequence
   const int k = min(max(n - pos0, 0), KPT);
   return k == 32 ? 0xffffffffu : (1u << k) - 1u;
 }
 
+// The first layout of the buckets is the same for all units, so that no sweep has to find the range of the keys before: 64
+// buckets per octave from 512 down to 2^-23, the first and the last one take what lies outside. It is as fine as a
+// layout over the range of importance values is (they spread over some twenty octaves).
+constexpr int kMapShift = 17, kMapFirst = 7616;  // t >> 17 of the values from 512 up
+constexpr int kDig = 11, kBuckets = 1 << kDig;
+
 // ---- shared memory of a block
 template <int TEAM, int WORDS>  // WORDS: count, or count and mass, per bucket
 struct RankShared {
-  static constexpr int kDig = 11;
-  static constexpr int kBuckets = 1 << kDig;
   static constexpr int kPer = kBuckets / (kHalf * TEAM);  // buckets per thread of the walk: 8, 4, 2, 1
-  static constexpr int kStride = kBuckets + 4;            // a place for slots without a key behind the buckets
+  static constexpr int kStride = kBuckets;
   // the buckets' counts; once they are walked, the candidates of the whole team and the buckets of the finish (count,
   // mass low, mass high; one per thread and modality) take their place
   static constexpr int kFinish = 2 * kListCap + 6 * kHalf;
@@ -210,8 +222,7 @@ struct RankShared {
   u64 first[2], last[2], first_q[2];            // walk: (count before << 32) | bucket, its count, mass before
   u64 fin_m[2];                                 // finish: mass before the range
   uint32_t slice_c[2][kMaxTeam];
-  uint32_t team_max[kMaxTeam], team_min[kMaxTeam];
-  uint32_t wmax[kRankWarps], wmin[kRankWarps], wscan_c[kRankWarps], wcnt[2][kRankWarps], inexact;
+  uint32_t wscan_c[kRankWarps], wcnt[2][kRankWarps], inexact;
   uint32_t few[2][kFewCap], few_n[2];
   uint32_t fin_c[2], fin_lo[2], fin_in[2], fin_more[2];
   uint32_t list_n;                              // candidates of this block: visual | text << 16
@@ -228,35 +239,26 @@ struct RankRange {
 };
 __device__ __forceinline__ int range_shift(uint32_t span, int dig) { return max(32 - __clz((int)span) - dig, 0); }
 
-// The unit's largest and smallest key into every thread (from the thread's own). Ends with a barrier of the team; zeroes the
-// buckets on the way.
+__device__ __forceinline__ uint32_t map_bucket(uint32_t t) {
+  return (uint32_t)max(min((int)(t >> kMapShift) - kMapFirst, kBuckets - 1), 0);
+}
+// The range of t of bucket `at`, of the first layout or of one over g with 2^shift values of t per bucket.
+__device__ __forceinline__ void bucket_range(RankRange& g, bool first, uint32_t at, int shift) {
+  if (first) {
+    g.lo = at ? (kMapFirst + at) << kMapShift : 0u;
+    g.span = (at < kBuckets - 1 ? ((kMapFirst + at + 1) << kMapShift) - 1u : kTopKey) - g.lo;
+  } else {
+    const uint32_t cut = at << shift;
+    g.span = min(g.span - cut, (1u << shift) - 1u);
+    g.lo += cut;
+  }
+}
 template <int TEAM, int WORDS>
-__device__ __forceinline__ void team_range(RankShared<TEAM, WORDS>& sh, uint32_t rank, uint32_t& kmax, uint32_t& kmin) {
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  for (int x = tid; x < 2 * WORDS * RankShared<TEAM, WORDS>::kStride / 4; x += kRankThreads)
+__device__ __forceinline__ void zero_buckets(RankShared<TEAM, WORDS>& sh) {
+  for (int x = threadIdx.x; x < 2 * WORDS * RankShared<TEAM, WORDS>::kStride / 4; x += kRankThreads)
     reinterpret_cast<uint4*>(sh.cnt)[x] = make_uint4(0, 0, 0, 0);
-  if (tid == 0) sh.list_n = 0;
-  kmax = __reduce_max_sync(kFull, kmax);
-  kmin = __reduce_min_sync(kFull, kmin);
-  if (lane == 0) {
-    sh.wmax[warp] = kmax;
-    sh.wmin[warp] = kmin;
-  }
+  if (threadIdx.x == 0) sh.list_n = 0;
   __syncthreads();
-  if (TEAM == 1 || warp == 0) {
-    kmax = __reduce_max_sync(kFull, sh.wmax[lane & (kRankWarps - 1)]);
-    kmin = __reduce_min_sync(kFull, sh.wmin[lane & (kRankWarps - 1)]);
-  }
-  if (TEAM > 1) {  // every block's figures go to every block: lane r of warp 0 writes them to block r
-    if (warp == 0 && lane < TEAM) {
-      peer_store<TEAM>(&sh.team_max[rank], lane, kmax);
-      peer_store<TEAM>(&sh.team_min[rank], lane, kmin);
-    }
-    team_sync<TEAM>();
-    kmax = __reduce_max_sync(kFull, lane < TEAM ? sh.team_max[lane] : 0u);
-    kmin = __reduce_min_sync(kFull, lane < TEAM ? sh.team_min[lane] : 0xffffffffu);
-  }
-  if (kmin > kmax) kmin = kmax;  // no keys at all
 }
 
 // This thread's words of the buckets, from word `at` on, added up over all blocks (the loads from distributed shared memory are
@@ -322,6 +324,20 @@ __device__ __forceinline__ void append(RankShared<TEAM, WORDS>& sh, uint32_t in0
   }
 }
 
+// The same for a unit that is not in registers: positions instead of keys (the keys are read again when the list is complete).
+template <int TEAM, int WORDS>
+__device__ __forceinline__ void append_positions(RankShared<TEAM, WORDS>& sh, uint32_t* pos0, uint32_t* pos1, uint32_t in0, uint32_t in1, int at) {
+  if (!__any_sync(kFull, (in0 | in1) != 0)) return;
+  const int lane = threadIdx.x & 31;
+  const uint32_t mine = __popc(in0) | (__popc(in1) << 16), incl = warp_scan32(mine);
+  uint32_t base = 0;
+  if (lane == 31) base = atomicAdd(&sh.list_n, incl);
+  base = __shfl_sync(kFull, base, 31) + incl - mine;
+  uint32_t o0 = base & 0xffffu, o1 = base >> 16;
+  for (; in0; in0 &= in0 - 1) pos0[o0++] = (uint32_t)(at + __ffs(in0) - 1);
+  for (; in1; in1 &= in1 - 1) pos1[o1++] = (uint32_t)(at + __ffs(in1) - 1);
+}
+
 // All blocks' candidates into this block (warp r copies block r's); returns their number, visual | text << 16. A block on
 // its own has them already. Ends with a barrier of the block.
 template <int TEAM, int WORDS>
@@ -348,7 +364,7 @@ __device__ __forceinline__ uint32_t gather_lists(RankShared<TEAM, WORDS>& sh) {
 // that equal it). A modality that is not `on` is left out. Ends with a barrier of the block.
 template <int TEAM, int WORDS, bool kMass>
 __device__ __forceinline__ void finish_lists(RankShared<TEAM, WORDS>& sh, const RankRange& r0, const RankRange& r1, uint32_t got, bool on0,
-                                             bool on1, u64 need0, u64 need1, u64 before0, u64 before1, uint32_t kmax) {
+                                             bool on1, u64 need0, u64 need1, u64 before0, u64 before1) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, m = tid / kHalf, i = tid % kHalf;
   const uint32_t n = m ? got >> 16 : got & 0xffffu, base = m ? r1.lo : r0.lo;
   const bool on = m ? on1 : on0;
@@ -357,7 +373,7 @@ __device__ __forceinline__ void finish_lists(RankShared<TEAM, WORDS>& sh, const 
   uint32_t lo = 0, span = m ? r1.span : r0.span, in = n, above_c = m ? r1.above : r0.above;
   u64 above = m ? before1 : before0;
   uint32_t *fc = sh.fin_bucket(m, 0), *flo = sh.fin_bucket(m, 1), *fhi = sh.fin_bucket(m, 2);
-  auto mass = [&](uint32_t x) { return psi_fix(kmax - (base + x)); };
+  auto mass = [&](uint32_t x) { return psi_fix(kTopKey - (base + x)); };
   for (;;) {
     const bool more = on && in > kFewCap && span > 0;
     if (i == 0) {
@@ -467,12 +483,13 @@ __device__ __forceinline__ void finish_lists(RankShared<TEAM, WORDS>& sh, const 
 struct RankShape {
   int kpt, team;  // keys per thread, blocks per unit
 };
-// A call with a unit or more per SM gets one block per unit, which reads the keys of a long unit again in every sweep:
-// spread over 2, 4 and 8 blocks such a call was slower the more blocks there were (256 units of 131072 keys: allocation
-// 156, 167, 174, 228 us, selection 219, 223, 240, 297 us), because every block pays for the fixed steps. With fewer units a
-// team of up to 8 blocks per unit brings the call to about a block per SM, and a call with a few units (one layer), which is
-// bound by the latency of its blocks, takes 8 keys per thread instead of 16 (4 units of 32768 keys: 12.8 + 10.9 us with 8
-// blocks of 8 keys, 15.5 + 13.7 with 4 blocks of 16, 30 + 54 with one block per unit).
+// A call with a unit or more per SM gets one block per unit, which reads the keys of a long unit in every sweep (kpt = 0, the
+// "long" kernels): spread over 2, 4 and 8 blocks such a call was slower the more blocks there were (256 units of 131072 keys:
+// allocation 156, 167, 174, 228 us, selection 219, 223, 240, 297 us), because every block pays for the fixed steps. With
+// fewer units a team of up to 8 blocks per unit brings the call to about a block per SM, and a call with a few units (one
+// layer), which is bound by the latency of its blocks, takes 8 keys per thread instead of 16 (4 units of 32768 keys: 12.8 +
+// 10.9 us with 8 blocks of 8 keys, 15.5 + 13.7 with 4 blocks of 16, 30 + 54 with one block per unit).
+constexpr int kLongKeys = 262144;  // keys per block that a long kernel has bits for in shared memory
 inline RankShape rank_shape(long long units, int n_max) {
   const int cap16 = kRankThreads * 16, cap8 = kRankThreads * 8;
   if (n_max <= cap8) return {8, 1};
@@ -481,13 +498,20 @@ inline RankShape rank_shape(long long units, int n_max) {
   while (fit16 < kMaxTeam && (long long)fit16 * cap16 < n_max) fit16 *= 2;
   while (team < kMaxTeam && units * team < 148) team *= 2;
   if (team >= fit8 && (long long)fit8 * cap8 >= n_max) return {8, fit8};
-  return {16, team < fit16 ? team : fit16};
+  if (team >= fit16 && (long long)fit16 * cap16 >= n_max) return {16, fit16};
+  while (team < kMaxTeam && (long long)team * kLongKeys < n_max) team *= 2;
+  return {0, team < fit16 ? team : fit16};
+}
+// Words of shared memory that a block of a long kernel needs per kind of bit.
+inline int long_words(int n_max, int team) {
+  const int round = kRankThreads * 16 * team;
+  return (n_max + round - 1) / round * (kRankThreads * 16 / 32 + kRankThreads * 16 / 1024);
 }
 
 // Launch of `units` teams, with programmatic stream serialisation (see launch_pdl).
 template <typename... KArgs, typename... Args>
-inline void launch_team(void (*kernel)(KArgs...), int units, int team, cudaStream_t st, Args... args) {
-  launch_ex(kernel, dim3((unsigned)units * (unsigned)team), dim3(kRankThreads), 0, st, team, KArgs(args)...);
+inline void launch_team(void (*kernel)(KArgs...), int units, int team, size_t smem, cudaStream_t st, Args... args) {
+  launch_ex(kernel, dim3((unsigned)units * (unsigned)team), dim3(kRankThreads), smem, st, team, KArgs(args)...);
 }
 
 }  // namespace

@@ -29,6 +29,7 @@ struct SelParams {
   int32_t* seq_nv;  // ws: visual-token count of every sequence
   int32_t* seq_wv;  // ws: visual tokens among the proxy tokens of every sequence (forced retention)
   int units, B, L, Hkv, n_max, mpa, headroom, keep_window, window, pool_r;  // pool_r: (pool_kernel - 1) / 2
+  int words;  // of bits, per kind of bit and block (long kernels)
   int alone;  // no seg_scan before: every unit adds up the segments before its own
 };
 
@@ -116,25 +117,25 @@ __global__ void __launch_bounds__(1024) seg_scan_kernel(SelParams p) {
 }
 
 // Keys of the two options: the maximum over the 2 * pool_r + 1 positions around each of KPT consecutive ones (pool_r may
-// be 0; positions outside the sequence do not count).
+// be 0; positions outside the sequence do not count). The largest score is the smallest t.
 constexpr int kMaxPoolR = 7;  // pool_kernel <= 15
 template <int KPT>
-__device__ __forceinline__ void load_pooled(const float* row, int mis, int n, int pos0, int pool_r, uint32_t (&key)[KPT]) {
-  uint32_t e[KPT + 16];  // keys of positions pos0 - 8 .. pos0 + KPT + 7
+__device__ __forceinline__ void load_pooled(const float* row, int mis, int n, int pos0, int pool_r, uint32_t (&t)[KPT]) {
+  uint32_t e[KPT + 16];  // t of positions pos0 - 8 .. pos0 + KPT + 7
   if (mis == 0 && pos0 >= 8 && pos0 + KPT + 8 <= n) {
 #pragma unroll
     for (int x = 0; x < KPT + 16; x += 4) {
       const float4 v = __ldg(reinterpret_cast<const float4*>(row + pos0 - 8 + x));
-      e[x] = score_key(v.x);
-      e[x + 1] = score_key(v.y);
-      e[x + 2] = score_key(v.z);
-      e[x + 3] = score_key(v.w);
+      e[x] = score_t(v.x);
+      e[x + 1] = score_t(v.y);
+      e[x + 2] = score_t(v.z);
+      e[x + 3] = score_t(v.w);
     }
   } else {
 #pragma unroll
     for (int x = 0; x < KPT + 16; ++x) {
       const int pos = pos0 - 8 + x;
-      e[x] = (pos >= 0 && pos < n) ? score_key(__ldg(row + pos)) : 0u;
+      e[x] = (pos >= 0 && pos < n) ? score_t(__ldg(row + pos)) : kTopKey;
     }
   }
 #pragma unroll
@@ -142,188 +143,171 @@ __device__ __forceinline__ void load_pooled(const float* row, int mis, int n, in
     uint32_t m = e[j + 8];
 #pragma unroll
     for (int d = 1; d <= kMaxPoolR; ++d)
-      if (d <= pool_r) m = max(m, max(e[j + 8 - d], e[j + 8 + d]));
-    key[j] = m;
+      if (d <= pool_r) m = min(m, min(e[j + 8 - d], e[j + 8 + d]));
+    t[j] = m;
   }
 }
 
-template <int KPT, int TEAM, bool kPool>
-__global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(SelParams p) {
-  using SH = RankShared<TEAM, 1>;
-  constexpr int kPer = SH::kPer;
-  __shared__ SH sh;
-  // (no wait here after seg_scan: it has waited for everything before it, so the scores, the mask and the budgets are final;
-  // what seg_scan itself writes is read after the wait below)
-  if (p.alone) pdl_wait();
-  const uint32_t rank = TEAM > 1 ? team_rank() : 0u;
-  const int u = blockIdx.x / TEAM;
-  const int b = u / (p.Hkv * p.L);
-  const float* psi = p.psi + (int64_t)u * p.n_max;
-  const int mis = (int)(((int64_t)u * p.n_max) & 3);
-  const uint8_t* mask = p.mask + (int64_t)b * p.n_max;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  constexpr int kRound = kRankThreads * KPT;
-  const int rounds = (p.n_max + kRound * TEAM - 1) / (kRound * TEAM);
-  const int pos_first = (int)rank * rounds * kRound + tid * KPT;  // a block owns consecutive positions
-  const int n = clamped_len(p.seq_len, b, p.n_max);
-  // proxy tokens retained unconditionally (none without cfg->keep_window): they are emitted by the sweep and the
-  // ranking only has to find the rest of each modality's budget
-  const int wfrom = kPool && p.keep_window ? max(n - p.window, 0) : n;
-  if (kPool) pdl_wait();  // (the forced tokens' counts are seg_scan's)
-  int lo_v = 0;
-  if (kPool && !p.alone) lo_v = p.seq_wv[b];
-  if (kPool && p.alone && p.mpa)  // (a window has at most 1024 tokens)
-    for (int x = wfrom; x < n; x += kRankThreads) lo_v += __syncthreads_count(x + tid < n && mask[x + tid] != 0);
-  const int lo_t = (n - wfrom) - lo_v;
-  const uint32_t want0 = (uint32_t)(p.mpa ? max(p.budgets[2 * u] - lo_v, 0) : 0),
-                 want1 = (uint32_t)max(p.budgets[2 * u + 1] - lo_t, 0);
-
-  uint32_t key[KPT], vis = 0, forced = 0;
-  auto load_round = [&](int r) {
-    const int pos0 = pos_first + r * kRound;
-    if (kPool) load_pooled<KPT>(psi, mis, n, pos0, p.pool_r, key);
-    else load_scores<KPT>(psi, mis, p.n_max, pos0, key);
-    vis = p.mpa ? load_mask<KPT>(mask, p.n_max, pos0) : 0u;
+// A unit of a block, and what is wanted of it.
+template <bool kPool>
+struct SelUnit {
+  const float* psi;
+  const uint8_t* mask;
+  int u, b, mis, n, wfrom, lo_v, lo_t;
+  uint32_t want0, want1;
+  __device__ __forceinline__ SelUnit(const SelParams& p, int unit) {
+    u = unit;
+    b = u / (p.Hkv * p.L);
+    psi = p.psi + (int64_t)u * p.n_max;
+    mis = (int)(((int64_t)u * p.n_max) & 3);
+    mask = p.mask + (int64_t)b * p.n_max;
+    n = clamped_len(p.seq_len, b, p.n_max);
+    // proxy tokens retained unconditionally (none without cfg->keep_window): they are emitted by the sweep and the
+    // ranking only has to find the rest of each modality's budget
+    wfrom = kPool && p.keep_window ? max(n - p.window, 0) : n;
+    if (kPool) pdl_wait();  // (the forced tokens' counts are seg_scan's)
+    lo_v = 0;
+    if (kPool && !p.alone) lo_v = p.seq_wv[b];
+    if (kPool && p.alone && p.mpa)  // (a window has at most 1024 tokens)
+      for (int x = wfrom; x < n; x += kRankThreads)
+        lo_v += __syncthreads_count(x + (int)threadIdx.x < n && mask[x + threadIdx.x] != 0);
+    lo_t = (n - wfrom) - lo_v;
+    want0 = (uint32_t)(p.mpa ? max(p.budgets[2 * u] - lo_v, 0) : 0);
+    want1 = (uint32_t)max(p.budgets[2 * u + 1] - lo_t, 0);
+  }
+  // t of KPT consecutive positions; returns those that are ranked, `forced`: those that are kept without
+  template <int KPT>
+  __device__ __forceinline__ uint32_t load(const SelParams& p, int pos0, uint32_t (&t)[KPT], uint32_t& forced) const {
+    if (kPool) load_pooled<KPT>(psi, mis, n, pos0, p.pool_r, t);
+    else load_scores<KPT>(psi, mis, p.n_max, pos0, t);
     uint32_t valid = valid_bits<KPT>(n, pos0);
-    if (kPool) {  // proxy tokens retained unconditionally: not ranked, always emitted
+    forced = 0;
+    if (kPool) {
       forced = valid & ~valid_bits<KPT>(wfrom, pos0);
       valid &= ~forced;
     }
     if (valid != valid_bits<KPT>(KPT, 0)) {
 #pragma unroll
       for (int j = 0; j < KPT; ++j)
-        if (!((valid >> j) & 1u)) key[j] = kNoKey;
+        if (!((valid >> j) & 1u)) t[j] = kNoKey;
     }
-  };
+    return valid;
+  }
+  __device__ __forceinline__ uint32_t load_one(const SelParams& p, int pos) const {  // the same of one ranked position
+    if (!kPool) return score_t(__ldg(psi + pos));
+    uint32_t m = kTopKey;
+    for (int x = max(pos - p.pool_r, 0); x <= min(pos + p.pool_r, n - 1); ++x) m = min(m, score_t(__ldg(psi + x)));
+    return m;
+  }
+};
 
-  // ---- range of the keys
-  uint32_t kmax = 0, kmin = 0xffffffffu;
-  for (int r = 0; r < rounds; ++r) {
-    load_round(r);
+// The ranges the two thresholds can lie in. short: the modality has no more keys than are wanted, all of them are kept.
+struct SelRanges {
+  RankRange r0, r1;
+  bool short0, short1;
+  uint32_t n_vis;  // visual tokens in the ranking
+  __device__ __forceinline__ bool crowded0() const { return r0.in > kListCap && r0.span > 0; }
+  __device__ __forceinline__ bool crowded1() const { return r1.in > kListCap && r1.span > 0; }
+};
+
+template <int KPT, int TEAM>
+__device__ __forceinline__ void count_first(RankShared<TEAM, 1>& sh, const uint32_t (&t)[KPT], uint32_t vis, uint32_t valid) {
+  constexpr int kStride = RankShared<TEAM, 1>::kStride;
+  if (valid == valid_bits<KPT>(KPT, 0)) {
 #pragma unroll
-    for (int j = 0; j < KPT; ++j) {
-      kmax = (uint32_t)max((int)kmax, (int)key[j]);  // (kNoKey is negative)
-      kmin = min(kmin, key[j]);
+    for (int j = 0; j < KPT; ++j) atomicAdd(sh.cnt + ((vis >> j) & 1u ? 0 : kStride) + map_bucket(t[j]), 1u);
+  } else {
+#pragma unroll
+    for (int j = 0; j < KPT; ++j)
+      if ((valid >> j) & 1u) atomicAdd(sh.cnt + ((vis >> j) & 1u ? 0 : kStride) + map_bucket(t[j]), 1u);
+  }
+}
+template <int KPT, int TEAM>
+__device__ __forceinline__ void count_again(RankShared<TEAM, 1>& sh, const SelRanges& g, const uint32_t (&t)[KPT], uint32_t vis, int shift0, int shift1) {
+#pragma unroll
+  for (int j = 0; j < KPT; ++j) {
+    const bool v = (vis >> j) & 1u;
+    const uint32_t x = t[j] - (v ? g.r0.lo : g.r1.lo);
+    if (x <= (v ? g.r0.span : g.r1.span)) atomicAdd(sh.cnt + (v ? 0 : RankShared<TEAM, 1>::kStride) + (x >> (v ? shift0 : shift1)), 1u);
+  }
+}
+
+// Walk of the buckets: block r of the team adds up its share of the buckets over all blocks, half of the threads per modality;
+// the ranges shrink to the buckets with the wanted keys.
+template <int TEAM>
+__device__ __forceinline__ void select_walk(RankShared<TEAM, 1>& sh, uint32_t rank, bool first, uint32_t want0, uint32_t want1, SelRanges& g,
+                                            int shift0, int shift1) {
+  using SH = RankShared<TEAM, 1>;
+  constexpr int kPer = SH::kPer;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, m = tid / kHalf, i = tid % kHalf;
+  const uint32_t b0 = (rank * kHalf + i) * kPer;
+  const uint32_t want = m ? want1 : want0;
+  if (i == 0) sh.first[m] = ~0ull;  // (stays if the modality has fewer keys than wanted)
+  team_sync<TEAM>();
+  uint32_t c[kPer], lc = 0;
+  bucket_counts<TEAM, 1>(sh, m * SH::kStride + b0, c);
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) lc += c[k];
+  uint32_t ic = warp_scan32(lc);
+  if (lane == 31) sh.wscan_c[warp] = ic;
+  __syncthreads();
+  ic += __reduce_add_sync(kFull, lane >= m * (kRankWarps / 2) && lane < warp ? sh.wscan_c[lane] : 0u);
+  if (i >= kHalf - 32) {  // the last warp of the modality has the block's total (in its last lane): to every block
+    const uint32_t tc = __shfl_sync(kFull, ic, 31);
+    if (lane < TEAM) peer_store<TEAM>(&sh.slice_c[m][rank], lane, tc);
+  }
+  if (TEAM > 1) {
+    team_sync<TEAM>();
+    ic += __reduce_add_sync(kFull, lane < (int)rank ? sh.slice_c[m][lane] : 0u);
+  }
+  ic += m ? g.r1.above : g.r0.above;
+  if (want && ic - lc < want && ic >= want) {
+    uint32_t run = ic - lc, at = 0, at_c = 0, at_in = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      if (run < want) {
+        at = b0 + k;
+        at_c = run;
+        at_in = c[k];
+      }
+      run += c[k];
+    }
+#pragma unroll
+    for (int r = 0; r < TEAM; ++r) {
+      peer_store<TEAM>(&sh.first[m], r, ((u64)at_c << 32) | at);
+      peer_store<TEAM>(&sh.last[m], r, (u64)at_in);
     }
   }
-  team_range<TEAM, 1>(sh, rank, kmax, kmin);
-  auto to_t = [&]() {
-#pragma unroll
-    for (int j = 0; j < KPT; ++j) key[j] = key[j] == kNoKey ? kNoKey : kmax - key[j];
+  team_sync<TEAM>();
+  if (first) g.n_vis = __reduce_add_sync(kFull, lane < TEAM ? sh.slice_c[0][lane] : 0u);
+  auto narrow = [&](RankRange& r, bool& is_short, int q, int s) {
+    if (sh.first[q] == ~0ull) {
+      is_short = true;
+      r = RankRange{kNowhere, 0u, 0u, 0u};
+      return;
+    }
+    bucket_range(r, first, (uint32_t)sh.first[q], s);
+    r.above = (uint32_t)(sh.first[q] >> 32);
+    r.in = (uint32_t)sh.last[q];
   };
-  if (rounds == 1) to_t();
-  auto reload = [&](int r) {
-    if (rounds > 1) {
-      load_round(r);
-      to_t();
-    }
-  };
+  if (want0 && !g.short0) narrow(g.r0, g.short0, 0, shift0);
+  if (want1 && !g.short1) narrow(g.r1, g.short1, 1, shift1);
+}
 
-  RankRange r0 = want0 ? RankRange{0u, kmax - kmin, kNoKey, 0u} : RankRange{kNowhere, 0u, 0u, 0u};
-  RankRange r1 = want1 ? RankRange{0u, kmax - kmin, kNoKey, 0u} : RankRange{kNowhere, 0u, 0u, 0u};
-  bool short0 = false, short1 = false;  // the modality has no more keys than are wanted: all of them are kept
-  auto crowded = [](const RankRange& g) { return g.in > kListCap && g.span > 0; };
-  uint32_t n_vis = 0;  // visual tokens in the ranking
-
-  for (int pass = 0; pass < 2; ++pass) {
-    // ---- buckets
-    const int shift0 = range_shift(pass ? r0.span : kmax - kmin, SH::kDig), shift1 = range_shift(pass ? r1.span : kmax - kmin, SH::kDig);
-    if (pass == 0) {  // all keys take part, both modalities over the same range (one of which nothing is wanted is not walked)
-      for (int r = 0; r < rounds; ++r) {
-        reload(r);
-#pragma unroll
-        for (int j = 0; j < KPT; ++j)
-          atomicAdd(sh.cnt + ((vis >> j) & 1u ? 0 : SH::kStride) + min(key[j] >> shift0, (uint32_t)SH::kBuckets), 1u);
-      }
-    } else {
-      for (int x = tid; x < 2 * SH::kStride / 4; x += kRankThreads) reinterpret_cast<uint4*>(sh.cnt)[x] = make_uint4(0, 0, 0, 0);
-      __syncthreads();
-      for (int r = 0; r < rounds; ++r) {
-        reload(r);
-#pragma unroll
-        for (int j = 0; j < KPT; ++j) {
-          const bool v = (vis >> j) & 1u;
-          const uint32_t x = key[j] - (v ? r0.lo : r1.lo);
-          if (x <= (v ? r0.span : r1.span)) atomicAdd(sh.cnt + (v ? 0 : SH::kStride) + (x >> (v ? shift0 : shift1)), 1u);
-        }
-      }
-    }
-    // ---- walk: block r of the team adds up its share of the buckets over all blocks; half of the threads per modality
-    const int m = tid / kHalf, i = tid % kHalf;
-    const uint32_t b0 = (rank * kHalf + i) * kPer;
-    const uint32_t want = m ? want1 : want0;
-    if (i == 0) sh.first[m] = ~0ull;  // (stays if the modality has fewer keys than wanted)
-    team_sync<TEAM>();
-    uint32_t c[kPer], lc = 0;
-    bucket_counts<TEAM, 1>(sh, m * SH::kStride + b0, c);
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) lc += c[k];
-    uint32_t ic = warp_scan32(lc);
-    if (lane == 31) sh.wscan_c[warp] = ic;
-    __syncthreads();
-    ic += __reduce_add_sync(kFull, lane >= m * (kRankWarps / 2) && lane < warp ? sh.wscan_c[lane] : 0u);
-    if (i >= kHalf - 32) {  // the last warp of the modality has the block's total (in its last lane): to every block
-      const uint32_t tc = __shfl_sync(kFull, ic, 31);
-      if (lane < TEAM) peer_store<TEAM>(&sh.slice_c[m][rank], lane, tc);
-    }
-    if (TEAM > 1) {
-      team_sync<TEAM>();
-      ic += __reduce_add_sync(kFull, lane < (int)rank ? sh.slice_c[m][lane] : 0u);
-    }
-    ic += m ? r1.above : r0.above;
-    if (want && ic - lc < want && ic >= want) {
-      uint32_t run = ic - lc, at = 0, at_c = 0, at_in = 0;
-#pragma unroll
-      for (int k = 0; k < kPer; ++k) {
-        if (run < want) {
-          at = b0 + k;
-          at_c = run;
-          at_in = c[k];
-        }
-        run += c[k];
-      }
-#pragma unroll
-      for (int r = 0; r < TEAM; ++r) {
-        peer_store<TEAM>(&sh.first[m], r, ((u64)at_c << 32) | at);
-        peer_store<TEAM>(&sh.last[m], r, (u64)at_in);
-      }
-    }
-    team_sync<TEAM>();
-    if (pass == 0) n_vis = __reduce_add_sync(kFull, lane < TEAM ? sh.slice_c[0][lane] : 0u);
-    {
-      auto narrow = [&](RankRange& g, bool& is_short, int q, int s) {
-        if (sh.first[q] == ~0ull) {
-          is_short = true;
-          g = RankRange{kNowhere, 0u, 0u, 0u};
-          return;
-        }
-        const uint32_t cut = (uint32_t)sh.first[q] << s;
-        g.span = min(g.span - cut, (1u << s) - 1u);
-        g.lo += cut;
-        g.above = (uint32_t)(sh.first[q] >> 32);
-        g.in = (uint32_t)sh.last[q];
-      };
-      if (want0 && !short0) narrow(r0, short0, 0, shift0);
-      if (want1 && !short1) narrow(r1, short1, 1, shift1);
-    }
-    if (!crowded(r0) && !crowded(r1)) break;
-  }
-
-  // ---- (rare) too many keys in a range: halve it with exact sweeps until they fit the list or are all alike
-  while (crowded(r0) || crowded(r1)) {
-    const bool on0 = crowded(r0), on1 = crowded(r1);
-    const uint32_t mid0 = r0.lo + (r0.span >> 1), mid1 = r1.lo + (r1.span >> 1);
+// (Rare) too many keys in a range: halve it with exact sweeps until they fit the list or are all alike. `sweep` calls its
+// argument with the keys of the thread, some at a time.
+template <int TEAM, typename Sweep>
+__device__ __forceinline__ void select_bisect(RankShared<TEAM, 1>& sh, uint32_t want0, uint32_t want1, SelRanges& g, Sweep sweep) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  while (g.crowded0() || g.crowded1()) {
+    const bool on0 = g.crowded0(), on1 = g.crowded1();
+    const uint32_t mid0 = g.r0.lo + (g.r0.span >> 1), mid1 = g.r1.lo + (g.r1.span >> 1);
     uint32_t c0 = 0, c1 = 0;
-    for (int r = 0; r < rounds; ++r) {
-      reload(r);
-#pragma unroll
-      for (int j = 0; j < KPT; ++j) {
-        const bool v = (vis >> j) & 1u;
-        if ((v ? on0 : on1) && key[j] >= (v ? r0.lo : r1.lo) && key[j] <= (v ? mid0 : mid1)) {
-          if (v) ++c0; else ++c1;
-        }
+    sweep([&](uint32_t t, bool v) {
+      if ((v ? on0 : on1) && t >= (v ? g.r0.lo : g.r1.lo) && t <= (v ? mid0 : mid1)) {
+        if (v) ++c0; else ++c1;
       }
-    }
+    });
     c0 = __reduce_add_sync(kFull, c0);
     c1 = __reduce_add_sync(kFull, c1);
     if (lane == 0) {
@@ -339,74 +323,56 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(SelParams 
         c0 += peer_load<TEAM>(&sh.wcnt[0][w], r);
         c1 += peer_load<TEAM>(&sh.wcnt[1][w], r);
       }
-    auto halve = [](RankRange& g, uint32_t want, uint32_t c) {
-      const uint32_t half = g.span >> 1;
-      if (g.above + c >= want) {
-        g.span = half;
-        g.in = c;
+    auto halve = [](RankRange& r, uint32_t want, uint32_t c) {
+      const uint32_t half = r.span >> 1;
+      if (r.above + c >= want) {
+        r.span = half;
+        r.in = c;
       } else {
-        g.above += c;
-        g.in -= c;
-        g.lo += half + 1;
-        g.span -= half + 1;
+        r.above += c;
+        r.in -= c;
+        r.lo += half + 1;
+        r.span -= half + 1;
       }
     };
-    if (on0) halve(r0, want0, c0);
-    if (on1) halve(r1, want1, c1);
+    if (on0) halve(g.r0, want0, c0);
+    if (on1) halve(g.r1, want1, c1);
     team_sync<TEAM>();
   }
+}
 
-  // ---- candidates of this block
-  for (int r = 0; r < rounds; ++r) {
-    reload(r);
-    uint32_t in = 0;
-#pragma unroll
-    for (int j = 0; j < KPT; ++j) {
-      const bool v = (vis >> j) & 1u;
-      if (key[j] - (v ? r0.lo : r1.lo) <= (v ? r0.span : r1.span)) in |= 1u << j;
-    }
-    append<TEAM, 1, KPT>(sh, r0.in <= kListCap ? in & vis : 0u, r1.in <= kListCap ? in & ~vis : 0u, key, r0.lo, r1.lo);
-  }
+// With the candidates of all blocks in their lists: the smallest t up to which the wanted number of keys lies, and how many keys
+// of exactly that t are still wanted, found by every block for itself. (Nothing wanted: nothing lies before 0 and no tie is
+// kept; all wanted: everything lies before kNowhere.)
+struct Thresholds {
+  uint32_t thr0, thr1, ties0, ties1;
+};
+template <int TEAM>
+__device__ __forceinline__ Thresholds select_thresholds(RankShared<TEAM, 1>& sh, uint32_t want0, uint32_t want1, const SelRanges& g) {
   team_sync<TEAM>();
-  // ---- every block gathers the team's candidates and finds the thresholds: the smallest t up to which the wanted number of
-  // keys lies, and how many keys of exactly that t are still wanted
   const uint32_t got = gather_lists<TEAM, 1>(sh);
-  const bool on0 = want0 && !short0 && r0.in <= kListCap, on1 = want1 && !short1 && r1.in <= kListCap;
-  finish_lists<TEAM, 1, false>(sh, r0, r1, got, on0, on1, want0, want1, 0ull, 0ull, kmax);
-  // (nothing wanted: nothing lies before 0 and no tie is kept; all wanted: everything lies before kNowhere)
-  const uint32_t thr0 = !want0 ? 0u : (short0 ? kNowhere : (on0 ? sh.fin_lo[0] : r0.lo));
-  const uint32_t thr1 = !want1 ? 0u : (short1 ? kNowhere : (on1 ? sh.fin_lo[1] : r1.lo));
-  const uint32_t ties0 = !want0 || short0 ? 0u : want0 - (on0 ? sh.fin_c[0] : r0.above);
-  const uint32_t ties1 = !want1 || short1 ? 0u : want1 - (on1 ? sh.fin_c[1] : r1.above);
+  const bool on0 = want0 && !g.short0 && g.r0.in <= kListCap, on1 = want1 && !g.short1 && g.r1.in <= kListCap;
+  finish_lists<TEAM, 1, false>(sh, g.r0, g.r1, got, on0, on1, want0, want1, 0ull, 0ull);
+  Thresholds h;
+  h.thr0 = !want0 ? 0u : (g.short0 ? kNowhere : (on0 ? sh.fin_lo[0] : g.r0.lo));
+  h.thr1 = !want1 ? 0u : (g.short1 ? kNowhere : (on1 ? sh.fin_lo[1] : g.r1.lo));
+  h.ties0 = !want0 || g.short0 ? 0u : want0 - (on0 ? sh.fin_c[0] : g.r0.above);
+  h.ties1 = !want1 || g.short1 ? 0u : want1 - (on1 ? sh.fin_c[1] : g.r1.above);
+  return h;
+}
 
-  // ---- ordered sweep: positions are consecutive within a thread, threads and blocks follow in position order. A key
-  // before its modality's threshold is kept, one at the threshold while its rank among these ties (in position order) is
-  // below the number still wanted. The counts of (ties v, ties t, kept outright) travel as one 3 x 21-bit word.
-  uint32_t eq, gt;
-  auto classify = [&]() {
-    eq = gt = 0;
-#pragma unroll
-    for (int j = 0; j < KPT; ++j) {
-      const uint32_t thr = (vis >> j) & 1u ? thr0 : thr1;
-      if (key[j] == thr) eq |= 1u << j;
-      if (key[j] < thr) gt |= 1u << j;
-    }
-    if (kPool) gt |= forced;
-    return (u64)__popc(eq & vis) | ((u64)__popc(eq & ~vis) << 21) | ((u64)__popc(gt) << 42);
-  };
-  u64 before = 0;  // counts before this block (a block on its own needs no totals before it emits)
-  u64 mine = 0;
-  if (rounds == 1) {
-    mine = classify();
-  } else if (TEAM > 1) {
-    for (int r = 0; r < rounds; ++r) {
-      reload(r);
-      mine += classify();
-    }
-  }
-  u64 incl = warp_scan64(mine);
+// Counts of (ties v, ties t, kept outright) travel as one 3 x 21-bit word. What lies before this thread's positions, from its
+// own counts.
+__device__ __forceinline__ u64 emit_counts(uint32_t gt, uint32_t eq, uint32_t vis) {
+  return (u64)__popc(eq & vis) | ((u64)__popc(eq & ~vis) << 21) | ((u64)__popc(gt) << 42);
+}
+template <int TEAM>
+__device__ __forceinline__ u64 counts_before(RankShared<TEAM, 1>& sh, uint32_t rank, u64 mine) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const u64 incl = warp_scan64(mine);
   if (lane == 31) sh.wscan_q[warp] = incl;
   __syncthreads();
+  u64 before = 0;
   if (TEAM > 1) {
     if (warp == 0) {
       const u64 tot = warp_sum64(lane < kRankWarps ? sh.wscan_q[lane] : 0ull);
@@ -415,87 +381,243 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(SelParams 
     team_sync<TEAM>();  // (also the last access to a peer's shared memory)
     before = warp_sum64(lane < (int)rank ? sh.slice_q[0][lane] : 0ull);
   }
-  int64_t off0;
+  return before + incl - mine + warp_sum64(lane < warp ? sh.wscan_q[lane] : 0ull);
+}
+
+// Where the unit's segment starts; -1: the cache is too small.
+template <int TEAM, bool kPool>
+__device__ __forceinline__ int64_t segment_start(RankShared<TEAM, 1>& sh, const SelParams& p, const SelUnit<kPool>& x, uint32_t rank, uint32_t n_vis) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (p.alone) {
     // one sequence: the segments' lengths follow from the budgets and the modalities' token counts, which are at hand
     pdl_go();
-    const int n_v = (int)n_vis + lo_v;
-    auto length = [&](int x) {
-      const int2 bud = __ldg(reinterpret_cast<const int2*>(p.budgets) + x);
-      return (p.mpa ? min(max(bud.x, lo_v), n_v) : 0) + min(max(bud.y, lo_t), n - n_v);
+    const int n_v = (int)n_vis + x.lo_v;
+    auto length = [&](int i) {
+      const int2 bud = __ldg(reinterpret_cast<const int2*>(p.budgets) + i);
+      return (p.mpa ? min(max(bud.x, x.lo_v), n_v) : 0) + min(max(bud.y, x.lo_t), x.n - n_v);
     };
     u64 sum = 0;
-    for (int x = tid; x < u; x += kRankThreads) sum += (u64)(length(x) + p.headroom);
+    for (int i = tid; i < x.u; i += kRankThreads) sum += (u64)(length(i) + p.headroom);
     sum = warp_sum64(sum);
     __syncthreads();
     if (lane == 0) sh.wsum[0][warp] = sum;
     __syncthreads();
-    off0 = (int64_t)warp_sum64(lane < kRankWarps ? sh.wsum[0][lane] : 0ull);
-    const int len = length(u);
-    const int64_t end = off0 + len + p.headroom;
+    const int64_t off = (int64_t)warp_sum64(lane < kRankWarps ? sh.wsum[0][lane] : 0ull);
+    const int len = length(x.u);
+    const int64_t end = off + len + p.headroom;
     if (rank == 0 && tid == 0) {
-      p.kept_len[u] = len;
-      p.seg_off[u] = off0;
-      if (u + 1 == p.units) {
+      p.kept_len[x.u] = len;
+      p.seg_off[x.u] = off;
+      if (x.u + 1 == p.units) {
         p.seg_off[p.units] = end;
         if (end > p.capacity) set_status(p.ws, MADAKV_ECAPACITY);
       }
     }
-    if (end > p.capacity) return;
-  } else {
-    if (!kPool) pdl_wait();
-    pdl_go();
-    off0 = p.seg_off[u];
-    if (off0 + p.kept_len[u] + p.headroom > p.capacity) return;  // seg_scan has raised MADAKV_ECAPACITY
+    return end > p.capacity ? -1 : off;
   }
-  auto emit = [&](int pos0, u64 ahead) {  // ahead: counts before this thread's positions
-    const uint32_t e0 = (uint32_t)ahead & 0x1fffffu, e1 = (uint32_t)(ahead >> 21) & 0x1fffffu, g = (uint32_t)(ahead >> 42);
-    int32_t* out = p.kept_idx + off0 + g + min(e0, ties0) + min(e1, ties1);
-    uint32_t keep = gt;
-    uint32_t ev = eq & vis, et = eq & ~vis;
-    for (uint32_t k = e0; k < ties0 && ev; ++k) {  // lowest positions first
-      keep |= ev & (0u - ev);
-      ev &= ev - 1;
-    }
-    for (uint32_t k = e1; k < ties1 && et; ++k) {
-      keep |= et & (0u - et);
-      et &= et - 1;
-    }
-    while (keep) {
-      const int j = __ffs(keep) - 1;
-      keep &= keep - 1;
-      *out++ = pos0 + j;
-    }
-  };
-  if (rounds == 1) {
-    emit(pos_first, before + incl - mine + warp_sum64(lane < warp ? sh.wscan_q[lane] : 0ull));
-  } else {
-    for (int r = 0; r < rounds; ++r) {
-      reload(r);
-      mine = classify();
-      incl = warp_scan64(mine);
-      __syncthreads();
-      if (lane == 31) sh.wscan_r[warp] = incl;
-      __syncthreads();
-      const u64 ahead = before + incl - mine + warp_sum64(lane < warp ? sh.wscan_r[lane] : 0ull);
-      before += warp_sum64(lane < kRankWarps ? sh.wscan_r[lane] : 0ull);
-      emit(pos_first + r * kRound, ahead);
-    }
+  if (!kPool) pdl_wait();
+  pdl_go();
+  const int64_t off = p.seg_off[x.u];
+  return off + p.kept_len[x.u] + p.headroom > p.capacity ? -1 : off;  // (seg_scan has raised MADAKV_ECAPACITY)
+}
+
+// Up to 32 consecutive positions: a key before its modality's threshold (gt) is kept, one at the threshold (eq) while its rank
+// among these ties, in position order, is below the number still wanted. `ahead`: counts before these positions.
+__device__ __forceinline__ void emit(int32_t* seg, const Thresholds& h, int pos0, u64 ahead, uint32_t gt, uint32_t eq, uint32_t vis) {
+  const uint32_t e0 = (uint32_t)ahead & 0x1fffffu, e1 = (uint32_t)(ahead >> 21) & 0x1fffffu, g = (uint32_t)(ahead >> 42);
+  int32_t* out = seg + g + min(e0, h.ties0) + min(e1, h.ties1);
+  uint32_t keep = gt;
+  uint32_t ev = eq & vis, et = eq & ~vis;
+  for (uint32_t k = e0; k < h.ties0 && ev; ++k) {  // lowest positions first
+    keep |= ev & (0u - ev);
+    ev &= ev - 1;
+  }
+  for (uint32_t k = e1; k < h.ties1 && et; ++k) {
+    keep |= et & (0u - et);
+    et &= et - 1;
+  }
+  while (keep) {
+    const int j = __ffs(keep) - 1;
+    keep &= keep - 1;
+    *out++ = pos0 + j;
   }
 }
 
+// A unit whose keys fit the registers of its team.
+template <int KPT, int TEAM, bool kPool>
+__global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(SelParams p) {
+  __shared__ RankShared<TEAM, 1> sh;
+  // (no wait here after seg_scan: it has waited for everything before it, so the scores, the mask and the budgets are final;
+  // what seg_scan itself writes is read after the wait of segment_start)
+  if (p.alone) pdl_wait();
+  const uint32_t rank = TEAM > 1 ? team_rank() : 0u;
+  const SelUnit<kPool> x(p, blockIdx.x / TEAM);
+  const int pos0 = (int)rank * kRankThreads * KPT + threadIdx.x * KPT;  // a block owns consecutive positions
+  uint32_t t[KPT], forced;
+  const uint32_t valid = x.template load<KPT>(p, pos0, t, forced);
+  const uint32_t vis = p.mpa ? load_mask<KPT>(x.mask, p.n_max, pos0) : 0u;
+  zero_buckets<TEAM, 1>(sh);
+  count_first<KPT, TEAM>(sh, t, vis, valid);
+  SelRanges g{{kNowhere, 0u, 0u, 0u}, {kNowhere, 0u, 0u, 0u}, false, false, 0u};
+  select_walk<TEAM>(sh, rank, true, x.want0, x.want1, g, 0, 0);
+  if (g.crowded0() || g.crowded1()) {
+    const int shift0 = range_shift(g.r0.span, kDig), shift1 = range_shift(g.r1.span, kDig);
+    zero_buckets<TEAM, 1>(sh);
+    count_again<KPT, TEAM>(sh, g, t, vis, shift0, shift1);
+    select_walk<TEAM>(sh, rank, false, x.want0, x.want1, g, shift0, shift1);
+    select_bisect<TEAM>(sh, x.want0, x.want1, g, [&](auto each) {
+#pragma unroll
+      for (int j = 0; j < KPT; ++j) each(t[j], (vis >> j) & 1u);
+    });
+  }
+  uint32_t in = 0;
+#pragma unroll
+  for (int j = 0; j < KPT; ++j) {
+    const bool v = (vis >> j) & 1u;
+    if (t[j] - (v ? g.r0.lo : g.r1.lo) <= (v ? g.r0.span : g.r1.span)) in |= 1u << j;
+  }
+  append<TEAM, 1, KPT>(sh, g.r0.in <= kListCap ? in & vis : 0u, g.r1.in <= kListCap ? in & ~vis : 0u, t, g.r0.lo, g.r1.lo);
+  const Thresholds h = select_thresholds<TEAM>(sh, x.want0, x.want1, g);
+  uint32_t eq = 0, gt = 0;
+#pragma unroll
+  for (int j = 0; j < KPT; ++j) {
+    const uint32_t thr = (vis >> j) & 1u ? h.thr0 : h.thr1;
+    if (t[j] == thr) eq |= 1u << j;
+    if (t[j] < thr) gt |= 1u << j;
+  }
+  if (kPool) gt |= forced;
+  const u64 ahead = counts_before<TEAM>(sh, rank, emit_counts(gt, eq, vis));
+  const int64_t off = segment_start<TEAM, kPool>(sh, p, x, rank, g.n_vis);
+  if (off >= 0) emit(p.kept_idx + off, h, pos0, ahead, gt, eq, vis);
+}
+
+// A longer unit is read twice: once for the buckets, once to sort its keys into kept, dropped and candidates. The first two are
+// three bits per key (visual, kept, candidate) in shared memory; candidates go to the list as positions, and when the
+// thresholds are known their bits are put right, so that the positions are emitted from the bits. (With every sweep over the
+// keys themselves, range, buckets, candidates and emission, 256 units of 131072 keys took 187 us instead of 110.)
+template <int TEAM, bool kPool>
+__global__ void __launch_bounds__(kRankThreads, 2) select_long_kernel(SelParams p) {
+  constexpr int KPT = 16, kRound = kRankThreads * KPT;
+  __shared__ RankShared<TEAM, 1> sh;
+  extern __shared__ __align__(16) uint32_t bits[];
+  if (p.alone) pdl_wait();
+  const uint32_t rank = TEAM > 1 ? team_rank() : 0u;
+  const int tid = threadIdx.x;
+  const SelUnit<kPool> x(p, blockIdx.x / TEAM);
+  uint32_t* cand_pos[2] = {bits, bits + kListCap};
+  uint32_t* vis_w = bits + 2 * kListCap;
+  uint32_t* keep_w = vis_w + p.words;
+  uint32_t* cand_w = keep_w + p.words;
+  const int rounds = (x.n + kRound * TEAM - 1) / (kRound * TEAM);
+  const int start = (int)rank * rounds * kRound;  // a block owns consecutive positions
+
+  zero_buckets<TEAM, 1>(sh);
+#pragma unroll 1
+  for (int r = 0; r < rounds; ++r) {
+    const int pos0 = start + r * kRound + tid * KPT;
+    uint32_t t[KPT], forced;
+    const uint32_t valid = x.template load<KPT>(p, pos0, t, forced);
+    const uint32_t vis = p.mpa ? load_mask<KPT>(x.mask, p.n_max, pos0) : 0u;
+    bits_of_thread(vis_w, r) = (uint16_t)vis;
+    count_first<KPT, TEAM>(sh, t, vis, valid);
+  }
+  SelRanges g{{kNowhere, 0u, 0u, 0u}, {kNowhere, 0u, 0u, 0u}, false, false, 0u};
+  select_walk<TEAM>(sh, rank, true, x.want0, x.want1, g, 0, 0);
+  if (g.crowded0() || g.crowded1()) {
+    const int shift0 = range_shift(g.r0.span, kDig), shift1 = range_shift(g.r1.span, kDig);
+    zero_buckets<TEAM, 1>(sh);
+#pragma unroll 1
+    for (int r = 0; r < rounds; ++r) {
+      uint32_t t[KPT], forced;
+      x.template load<KPT>(p, start + r * kRound + tid * KPT, t, forced);
+      count_again<KPT, TEAM>(sh, g, t, bits_of_thread(vis_w, r), shift0, shift1);
+    }
+    select_walk<TEAM>(sh, rank, false, x.want0, x.want1, g, shift0, shift1);
+    select_bisect<TEAM>(sh, x.want0, x.want1, g, [&](auto each) {
+#pragma unroll 1
+      for (int r = 0; r < rounds; ++r) {
+        uint32_t t[KPT], forced;
+        x.template load<KPT>(p, start + r * kRound + tid * KPT, t, forced);
+        const uint32_t vis = bits_of_thread(vis_w, r);
+#pragma unroll
+        for (int j = 0; j < KPT; ++j) each(t[j], (vis >> j) & 1u);
+      }
+    });
+  }
+
+  // ---- kept and candidates. Nothing wanted: nothing lies before 0; all wanted: everything lies before kNowhere.
+  const uint32_t lo0 = x.want0 ? g.r0.lo : 0u, lo1 = x.want1 ? g.r1.lo : 0u;
+  const uint32_t wide0 = x.want0 && !g.short0 ? g.r0.span + 1u : 0u, wide1 = x.want1 && !g.short1 ? g.r1.span + 1u : 0u;
+  const bool on0 = g.r0.in <= kListCap, on1 = g.r1.in <= kListCap;
+#pragma unroll 1
+  for (int r = 0; r < rounds; ++r) {
+    const int at = r * kRound + tid * KPT;
+    uint32_t t[KPT], forced;
+    x.template load<KPT>(p, start + at, t, forced);
+    const uint32_t vis = bits_of_thread(vis_w, r);
+    uint32_t in = 0, keep = forced;
+#pragma unroll
+    for (int j = 0; j < KPT; ++j) {
+      const bool v = (vis >> j) & 1u;
+      const uint32_t lo = v ? lo0 : lo1;
+      if (t[j] < lo) keep |= 1u << j;
+      if (t[j] - lo < (v ? wide0 : wide1)) in |= 1u << j;
+    }
+    bits_of_thread(keep_w, r) = (uint16_t)keep;
+    bits_of_thread(cand_w, r) = (uint16_t)in;
+    append_positions<TEAM, 1>(sh, cand_pos[0], cand_pos[1], on0 ? in & vis : 0u, on1 ? in & ~vis : 0u, at);
+  }
+  __syncthreads();
+  const int m = tid / kHalf, mine_n = m ? sh.list_n >> 16 : sh.list_n & 0xffffu;
+  for (int i = tid % kHalf; i < mine_n; i += kHalf)
+    sh.list[m][i] = x.load_one(p, start + (int)cand_pos[m][i]) - (m ? lo1 : lo0);
+  const Thresholds h = select_thresholds<TEAM>(sh, x.want0, x.want1, g);
+  // ---- of the candidates, those before the threshold are kept and those at it stay candidates (ties)
+  for (int i = tid % kHalf; i < mine_n; i += kHalf) {
+    const uint32_t t = sh.list[m][i] + (m ? lo1 : lo0), thr = m ? h.thr1 : h.thr0, at = cand_pos[m][i];
+    if (t < thr) atomicOr(keep_w + bits_slot(at >> 5), 1u << (at & 31));
+    if (t != thr) atomicAnd(cand_w + bits_slot(at >> 5), ~(1u << (at & 31)));
+  }
+  __syncthreads();
+  const int words = rounds * (kRound / 32), share = (words + kRankThreads - 1) / kRankThreads;  // consecutive words per thread
+  const int w0 = min(tid * share, words), w1 = min(w0 + share, words);
+  u64 mine = 0;
+  for (int w = w0; w < w1; ++w) mine += emit_counts(keep_w[bits_slot(w)], cand_w[bits_slot(w)], vis_w[bits_slot(w)]);
+  u64 ahead = counts_before<TEAM>(sh, rank, mine);
+  const int64_t off = segment_start<TEAM, kPool>(sh, p, x, rank, g.n_vis);
+  if (off < 0) return;
+  for (int w = w0; w < w1; ++w) {
+    const uint32_t gt = keep_w[bits_slot(w)], eq = cand_w[bits_slot(w)], vis = vis_w[bits_slot(w)];
+    emit(p.kept_idx + off, h, start + w * 32, ahead, gt, eq, vis);
+    ahead += emit_counts(gt, eq, vis);
+  }
+}
+
+template <int TEAM, bool kPool>
+void launch_long(SelParams p, cudaStream_t st) {
+  auto kern = select_long_kernel<TEAM, kPool>;
+  p.words = long_words(p.n_max, TEAM);
+  // (the largest of any call, so that threads with calls of different sizes do not take the room from one another; a failure
+  // shows at the launch)
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (2 * kListCap + 3 * long_words(kLongKeys, 1)) * 4);
+  launch_team(kern, p.units, TEAM, (size_t)(2 * kListCap + 3 * p.words) * 4, st, p);
+}
 template <bool kPool>
 void launch_select_unit(const madakv_config& c, const SelParams& p, cudaStream_t st) {
   const RankShape s = rank_shape(p.units, c.max_seq_len);
-  switch (s.kpt + s.team) {
-    case 8 + 1: launch_team(select_unit_kernel<8, 1, kPool>, p.units, 1, st, p); break;
-    case 8 + 2: launch_team(select_unit_kernel<8, 2, kPool>, p.units, 2, st, p); break;
-    case 8 + 4: launch_team(select_unit_kernel<8, 4, kPool>, p.units, 4, st, p); break;
-    case 8 + 8: launch_team(select_unit_kernel<8, 8, kPool>, p.units, 8, st, p); break;
-    case 16 + 1: launch_team(select_unit_kernel<16, 1, kPool>, p.units, 1, st, p); break;
-    case 16 + 2: launch_team(select_unit_kernel<16, 2, kPool>, p.units, 2, st, p); break;
-    case 16 + 4: launch_team(select_unit_kernel<16, 4, kPool>, p.units, 4, st, p); break;
-    default: launch_team(select_unit_kernel<16, 8, kPool>, p.units, 8, st, p); break;
+  switch (s.kpt * 16 + s.team) {
+    case 8 * 16 + 1: launch_team(select_unit_kernel<8, 1, kPool>, p.units, 1, 0, st, p); break;
+    case 8 * 16 + 2: launch_team(select_unit_kernel<8, 2, kPool>, p.units, 2, 0, st, p); break;
+    case 8 * 16 + 4: launch_team(select_unit_kernel<8, 4, kPool>, p.units, 4, 0, st, p); break;
+    case 8 * 16 + 8: launch_team(select_unit_kernel<8, 8, kPool>, p.units, 8, 0, st, p); break;
+    case 16 * 16 + 1: launch_team(select_unit_kernel<16, 1, kPool>, p.units, 1, 0, st, p); break;
+    case 16 * 16 + 2: launch_team(select_unit_kernel<16, 2, kPool>, p.units, 2, 0, st, p); break;
+    case 16 * 16 + 4: launch_team(select_unit_kernel<16, 4, kPool>, p.units, 4, 0, st, p); break;
+    case 16 * 16 + 8: launch_team(select_unit_kernel<16, 8, kPool>, p.units, 8, 0, st, p); break;
+    case 1: launch_long<1, kPool>(p, st); break;
+    case 2: launch_long<2, kPool>(p, st); break;
+    case 4: launch_long<4, kPool>(p, st); break;
+    default: launch_long<8, kPool>(p, st); break;
   }
 }
 

@@ -418,10 +418,10 @@ def test_allocate_and_select_on_crafted_scores(kind, n):
         assert_segments_equal(kept_len, seg_off, buf.kept_idx.cpu().numpy(), kept_idx, "kept_idx")
 
 
-# (units, positions): one block of 8 and of 16 keys per thread, in one round and in several; teams of 2, 4 and 8 blocks with
-# 8 and with 16 keys per thread; rows that start on every 4-byte boundary
+# (units, positions): one block of 8 and of 16 keys per thread; teams of 2, 4 and 8 blocks with 8 and with 16 keys per thread;
+# units longer than their team's registers, on 1 to 8 blocks; rows that start on every 4-byte boundary
 @pytest.mark.parametrize("units,n", [(3, 4096), (150, 4097), (148, 16391), (74, 8190), (74, 9001), (40, 16384), (38, 20003),
-                                     (4, 32768), (6, 33333), (1, 131073)])
+                                     (4, 32768), (6, 33333), (1, 131073), (2, 65536), (148, 8193), (40, 40961), (160, 24576), (1, 600001)])
 @pytest.mark.parametrize("kind", ["importance", "crowded", "extremes"])
 def test_allocate_and_select_over_blocks_and_lengths(kind, units, n):
     """Every way the ranking kernels spread a unit's keys, bit-exact against the oracle: importance-like scores, ties and
