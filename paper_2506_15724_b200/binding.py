@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libmadakv.so: the same names as include/madakv.h, argument marshalling only.
+"""Thin binding of libmadakv.so: the same names as include/madakv.h, argument marshalling only. The asynchronous calls go
+through a small C++ extension (_native.so) that reads the tensors itself, the rest through ctypes.
 
 Every step of the eviction pass runs in the library's CUDA kernels; PyTorch is used for device memory and streams.
 There is no CPU fallback: importing this module without the built library, or calling it without a CUDA device,
@@ -90,17 +91,27 @@ def make_config(dtype, batch, n_layers, n_q_heads, n_kv_heads, head_dim, max_seq
                         pool_kernel)
 
 
-# What a call costs on the host is mostly this file (a decode call on one layer: 12.3 us, 6.4 of them in the library), so
-# arguments are passed as plain integers (the declared argument types convert them) and the stream handle is fetched
-# without building a torch.cuda.Stream object (3.2 us).
+class _Unbuilt:
+    """Stands for the extension where it has not been built: any call raises."""
+
+    def __init__(self, why):
+        self.why = why
+
+    def __getattr__(self, name):
+        raise ImportError(f"{self.why}: run `python -m paper_2506_15724_b200.build` (needs nvcc and g++)")
+
+
+# What a call on one layer costs is mostly the host's part. With the tensors' pointers gathered in Python and passed through
+# ctypes it was 5.4 us for decode, 5.2-6.4 for allocate_layer, select and compact, 6.8 for score_lse; with the extension, which
+# takes the tensors, it is 3.1, 2.5-2.9 and 5.1, most of that the launch.
+try:
+    from . import _native
+except ImportError as e:
+    _native = _Unbuilt(e)
+
+
 def _ptr(t):
     return None if t is None else t.data_ptr()
-
-
-def _strides5(t):
-    st = t.stride()
-    assert len(st) == 5 and st[4] == 1, "expected [B, L, H, tokens, d] with contiguous d"
-    return MadakvStrides(st[0], st[1], st[2], st[3])
 
 
 def _stream():
@@ -124,54 +135,52 @@ def new_workspace(cfg, device="cuda"):
 
 
 def madakv_score(cfg, q_win, k, seq_len, lse, psi, ws):
-    _check("madakv_score", lib().madakv_score(cfg, _ptr(q_win), _strides5(q_win), _ptr(k), _strides5(k),
-                                              _ptr(seq_len), _ptr(lse), _ptr(psi), _ptr(ws), ws.numel(), _stream()))
+    rc = _native.score(cfg, q_win, k, seq_len, lse, psi, ws)
+    if rc:
+        raise MadakvError("madakv_score", rc)
 
 
 def madakv_score_lse(cfg, q_win, k, seq_len, lse, psi, ws):
-    _check("madakv_score_lse", lib().madakv_score_lse(cfg, _ptr(q_win), _strides5(q_win), _ptr(k),
-                                                      _strides5(k), _ptr(seq_len), _ptr(lse), _ptr(psi), _ptr(ws),
-                                                      ws.numel(), _stream()))
+    rc = _native.score_lse(cfg, q_win, k, seq_len, lse, psi, ws)
+    if rc:
+        raise MadakvError("madakv_score_lse", rc)
 
 
 def madakv_allocate(cfg, psi, mask, seq_len, budget, mass, pref, demand, phi, budgets, ws):
-    _check("madakv_allocate", lib().madakv_allocate(cfg, _ptr(psi), _ptr(mask), _ptr(seq_len),
-                                                    _ptr(budget), _ptr(mass), _ptr(pref), _ptr(demand), _ptr(phi),
-                                                    _ptr(budgets), _ptr(ws), ws.numel(), _stream()))
+    rc = _native.allocate(cfg, psi, mask, seq_len, budget, mass, pref, demand, phi, budgets, ws)
+    if rc:
+        raise MadakvError("madakv_allocate", rc)
 
 
 def madakv_demand_layer(cfg, psi, mask, seq_len, mass, pref, demand, ws):
-    _check("madakv_demand_layer", lib().madakv_demand_layer(cfg, _ptr(psi), _ptr(mask), _ptr(seq_len),
-                                                            _ptr(mass), _ptr(pref), _ptr(demand), _ptr(ws), ws.numel(),
-                                                            _stream()))
+    rc = _native.demand_layer(cfg, psi, mask, seq_len, mass, pref, demand, ws)
+    if rc:
+        raise MadakvError("madakv_demand_layer", rc)
 
 
 def madakv_allocate_layer(cfg, layer, psi, mask, seq_len, budget, mass, pref, demand, phi, budgets, ws):
     """psi may be None: mass, pref and demand then come from madakv_demand_layer."""
-    _check("madakv_allocate_layer", lib().madakv_allocate_layer(cfg, int(layer), _ptr(psi), _ptr(mask),
-                                                                _ptr(seq_len), _ptr(budget), _ptr(mass), _ptr(pref),
-                                                                _ptr(demand), _ptr(phi), _ptr(budgets), _ptr(ws),
-                                                                ws.numel(), _stream()))
+    rc = _native.allocate_layer(cfg, int(layer), psi, mask, seq_len, budget, mass, pref, demand, phi, budgets, ws)
+    if rc:
+        raise MadakvError("madakv_allocate_layer", rc)
 
 
 def madakv_select(cfg, psi, mask, seq_len, budgets, kept_len, seg_off, kept_idx, ws):
-    _check("madakv_select", lib().madakv_select(cfg, _ptr(psi), _ptr(mask), _ptr(seq_len), _ptr(budgets),
-                                                _ptr(kept_len), _ptr(seg_off), _ptr(kept_idx), kept_idx.numel(),
-                                                _ptr(ws), ws.numel(), _stream()))
+    rc = _native.select(cfg, psi, mask, seq_len, budgets, kept_len, seg_off, kept_idx, ws)
+    if rc:
+        raise MadakvError("madakv_select", rc)
 
 
 def madakv_compact(cfg, k, v, kept_idx, seg_off, kept_len, k_c, v_c, ws):
-    assert k.stride() == v.stride()
-    _check("madakv_compact", lib().madakv_compact(cfg, _ptr(k), _ptr(v), _strides5(k), _ptr(kept_idx),
-                                                  _ptr(seg_off), _ptr(kept_len), _ptr(k_c), _ptr(v_c), k_c.shape[0],
-                                                  _ptr(ws), ws.numel(), _stream()))
+    rc = _native.compact(cfg, k, v, kept_idx, seg_off, kept_len, k_c, v_c, ws)
+    if rc:
+        raise MadakvError("madakv_compact", rc)
 
 
 def madakv_decode_attn(cfg, layer, q, k_new, v_new, k_c, v_c, seg_off, kept_len, out, lse_out, ws):
-    _check("madakv_decode_attn", lib().madakv_decode_attn(cfg, layer, _ptr(q), _ptr(k_new), _ptr(v_new),
-                                                          _ptr(k_c), _ptr(v_c), _ptr(seg_off), _ptr(kept_len),
-                                                          k_c.shape[0], _ptr(out), _ptr(lse_out), _ptr(ws),
-                                                          ws.numel(), _stream()))
+    rc = _native.decode_attn(cfg, layer, q, k_new, v_new, k_c, v_c, seg_off, kept_len, out, lse_out, ws)
+    if rc:
+        raise MadakvError("madakv_decode_attn", rc)
 
 
 def madakv_decode_attn_static(cfg, layer, q, k_c, v_c, seg_off, kept_len, out, lse_out):

@@ -1,12 +1,15 @@
-"""Builds libmadakv.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libmadakv.so (the C-ABI CUDA library, nvcc for sm_100a) and _native.so (its Python entry points, g++) in-tree."""
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libmadakv.so")
+NATIVE_SRC = os.path.join(HERE, "csrc", "py_binding.cpp")
+NATIVE = os.path.join(HERE, "_native.so")
 PROBE_SRC = os.path.join(HERE, "csrc", "probe", "exp2_roof.cu")
 PROBE = os.path.join(HERE, "exp2_roof.bin")  # measures the exp2 roof (see the source); used by bench.py
 
@@ -31,9 +34,27 @@ def build_probe(force=False):
     return PROBE
 
 
+def build_native(force=False):
+    """The Python entry points: a C++ extension against torch's headers that links to libmadakv.so beside it."""
+    header = os.path.join(ROOT, "include", "madakv.h")
+    newest = max(os.path.getmtime(NATIVE_SRC), os.path.getmtime(header))
+    if force or not os.path.exists(NATIVE) or os.path.getmtime(NATIVE) < newest:
+        import torch
+        from torch.utils import cpp_extension
+
+        inc = cpp_extension.include_paths("cuda") + [sysconfig.get_paths()["include"], os.path.join(ROOT, "include")]
+        subprocess.check_call(
+            ["g++", "-std=c++17", "-O2", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+            + [x for d in inc for x in ("-isystem", d)] + ["-o", NATIVE, NATIVE_SRC, "-L", HERE]
+            + [x for d in cpp_extension.library_paths("cuda") for x in ("-L", d)]
+            + ["-lmadakv", "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-Wl,-rpath,$ORIGIN"])
+    return NATIVE
+
+
 def build(force=False, verbose=False):
     build_probe(force)
     if not force and not needs_build():
+        build_native()
         return LIB
     cmd = [
         "nvcc", "-std=c++17", "-O3", "-lineinfo", "-gencode", "arch=compute_100a,code=sm_100a",
@@ -41,6 +62,7 @@ def build(force=False, verbose=False):
         "-o", LIB,
     ] + (["-Xptxas", "-v"] if verbose else []) + sources()
     subprocess.check_call(cmd)
+    build_native(force)
     return LIB
 
 
