@@ -58,21 +58,19 @@ inline int wide_max_runs(int units_per_seq, int n_max) {
   if (runs > tiles) runs = tiles;
   return (int)(runs < 1 ? 1 : runs);
 }
-// fp32 scoring on the tensor cores: keys and queries split into three bf16 terms each, 6 bytes per element, for as many units
-// at a time as kSplitBytes hold (at least one). 96 MB stay in the L2 for the most part between the two passes over them and
-// give the GPU's SMs several tiles each.
-constexpr size_t kSplitBytes = 96u << 20;
-inline size_t split_unit_bytes(const madakv_config& c) {
-  return ((size_t)c.max_seq_len + (size_t)(c.n_q_heads / c.n_kv_heads) * c.window) * c.head_dim * 6;
+// fp32 scoring on the tensor cores takes keys and queries as three bf16 terms each. A two-pass call with less than a tile per
+// SM has them written to the workspace first (6 bytes per element): its CTAs start 3-6 us earlier with TMA loads of the
+// terms than with loads and conversions of their own. From there on the kernels split the values as they load them (us, terms
+// first / on loading: 16 tiles 18.0 / 21.5 with head_dim 64, 20.9 / 27.3 with 128; 64: 20.3 / 21.1, 24.0 / 27.3; 148: 23.6 / 23.3,
+// 29.3 / 30.2; 296: 28.7 / 26.4, 38.8 / 34.4), and so does the single pass over K (16 tiles 10.5 / 8.6, 296 22.4 / 12.3).
+constexpr int kSplitTiles = 148;
+inline bool split_first(const madakv_config& c) {
+  return c.dtype == MADAKV_F32 &&
+         (long long)c.batch * c.n_layers * c.n_kv_heads * ((c.max_seq_len + 127) / 128) < kSplitTiles;
 }
-inline int split_units(const madakv_config& c) {
-  const long long lh = (long long)c.n_layers * c.n_kv_heads, total = lh * c.batch;
-  long long fit = (long long)(kSplitBytes / split_unit_bytes(c));
-  if (fit < 1) fit = 1;
-  if (fit >= total) return (int)total;
-  if (fit >= lh) return (int)(fit / lh * lh);
-  const long long parts = (lh + fit - 1) / fit;  // parts of a sequence, as even as possible
-  return (int)((lh + parts - 1) / parts);
+inline size_t split_bytes(const madakv_config& c) {
+  return (size_t)c.batch * c.n_layers * c.n_kv_heads *
+         ((size_t)c.max_seq_len + (size_t)(c.n_q_heads / c.n_kv_heads) * c.window) * c.head_dim * 6;
 }
 
 inline WsLayout ws_layout(const madakv_config& c) {
@@ -104,7 +102,7 @@ inline WsLayout ws_layout(const madakv_config& c) {
   part = wide > part ? wide : part;
   off = align_up(off + part, 256);
   w.score_split_off = off;
-  if (c.dtype == MADAKV_F32) off = align_up(off + split_unit_bytes(c) * (size_t)split_units(c), 256);
+  if (split_first(c)) off = align_up(off + split_bytes(c), 256);
   w.decode_off = off;
   off = align_up(off + (size_t)c.batch * c.n_layers * c.n_q_heads * (size_t)w.decode_splits * (c.head_dim + 2) *
                            sizeof(float), 256);

@@ -4,10 +4,17 @@
 // A launch takes up to 256 window rows per KV head (fp32: 128); shapes with more go in chunks of query heads (or, for
 // windows beyond that, of window rows) one launch after the other, each adding its part to psi.
 //
-// fp32 inputs are split exactly into three bf16 numbers of 8 significand bits each (split_kernel writes them to the
-// workspace, a slice of the units at a time), and a product q * k is taken as the six partial products that are not below
-// 2^-24 of it: hi hi, hi mid, mid hi, mid mid, hi lo, lo hi, all accumulated in fp32. An SM's fp32 pipes do 256 FLOP per
-// clock, its tensor cores 8192 / 6.
+// fp32 inputs are split exactly into three bf16 numbers of 8 significand bits each, and a product q * k is taken as the six
+// partial products that are not below 2^-24 of it: hi hi, hi mid, mid hi, mid mid, hi lo, lo hi, all accumulated in fp32.
+// An SM's fp32 pipes do 256 FLOP per clock, its tensor cores 8192 / 6. In all but the smallest calls (split_first()) 16 warps of a
+// CTA, in the place of the TMA producer and of most of the epilogue, load the fp32 rows and write the terms into the operands'
+// shared memory, so that both passes read K as it is (CV). What bounds them is that conversion, 2700-3500 clocks per 64 columns of
+// 128 keys and lately the operands' shared-memory traffic, 3072 + 768 clocks per tile of six products; the exponentials of 128 rows
+// need 1024, so four epilogue warps do. (us with the terms of all keys written to the workspace by a kernel before, in slices of
+// 96 MB -> now: 16 units of 73557 keys at most, 56 rows 1072 -> 329; 1024 of 1263, 64 rows 1064 -> 466; 8 of 82828, 224 rows 964 ->
+// 450; 1280 of 2357, head_dim 64, 64 rows 1236 -> 600. Eight converting warps and eight or four for the epilogue: 379 and 359 on
+// the first. An issuer chosen by elect.sync, which spares a move to a uniform register per operand, took the MMA issue from 5000 to
+// 2900 clocks per tile.)
 //
 // With that many rows the work per key byte is dominated by the exponentials (g * w of them per key and pass), not
 // by HBM: the special-function unit delivers 16 exp2 per clock and SM, which for 256 rows is 2048 clocks per 128-key
@@ -43,9 +50,20 @@
 namespace madakv {
 namespace {
 
-constexpr int kRowThreads = 576;  // 2 + 16 warps
+constexpr int kConvertWarps = 16;  // CV: the last 16 warps
 constexpr int kMaxSeqScan = 1024; // batches up to this size get the exact (ragged-aware) tile partition
 constexpr int kFoldTiles = 16;    // pass 1 moves a row's sum to its second level every this many tiles
+
+// Division of numbers below 2^31 by a number known on the host: a multiplication instead of some forty instructions, of which
+// every warp of a CTA did several before its first tile.
+struct FastDiv {
+  uint32_t d, mul, shift;
+  explicit FastDiv(int by = 1) : d((uint32_t)by), shift(0) {
+    while ((1ull << shift) < d) ++shift;
+    mul = (uint32_t)((((1ull << shift) - d) << 32) / d + 1);
+  }
+  __device__ __forceinline__ int div(int x) const { return (int)((__umulhi((uint32_t)x, mul) + (uint32_t)x) >> shift); }
+};
 
 struct RowParams {
   const int32_t* seq_len;
@@ -55,8 +73,10 @@ struct RowParams {
   const float* lse2; // ws: [units, rs] NEGATED log2-domain log-sum-exp, padding rows hold kEmptyMax (pass 2)
   int32_t* status;   // ws header
   int B, units, L, Hq, Hkv, g, w, R, n_max, causal, rs, mblocks, cparts, n16;  // n16: R rounded up to 16
-  int lh;            // units per sequence (of this launch)
-  int u0;            // fp32: first unit of the slice; unit u of the launch is unit u0 + u of the call
+  int lh;            // units per sequence
+  FastDiv by_hkv, by_wc;
+  const float *qf, *kf;  // fp32 inputs
+  madakv_strides sq, sk; // of fp32 inputs, in elements
   int h0, r0, wc;    // the launch's window rows: rows [r0, r0 + wc) of query heads h0 .. of the group, R = heads * wc
   int accumulate;    // psi += instead of =
   int smax;          // runs (CTAs) a unit's tiles can be spread over at most: wide_max_runs()
@@ -64,13 +84,16 @@ struct RowParams {
   float scale2;
 };
 
-template <int D, int PASS, int NS>  // NS: bf16 terms per operand (1, or 3 for fp32)
+template <int D, int PASS, int NS, bool CV>  // NS: bf16 terms per operand (1, or 3 for fp32); CV: fp32 inputs are split here
 struct RowSmem {
   // NS = 1: a stage is a whole K tile. NS = 3: a stage is one 64-wide piece of one term of it, 16 KB.
   // pass 2 gives up K stages for the operands of its extra contraction step (see the MMA issuer)
-  static constexpr int kStages = NS == 3 ? (PASS == 2 ? 5 : 6) : (D == 128 ? 4 : 8) - (PASS == 2 ? (D == 128 ? 1 : 2) : 0);
+  static constexpr int kStages = NS == 3 ? (PASS == 2 ? 5 : 6 + CV) : (D == 128 ? 4 : 8) - (PASS == 2 ? (D == 128 ? 1 : 2) : 0);
   static constexpr int kKBlocks = D / 64;
   static constexpr int kPieces = NS == 3 ? 3 * kKBlocks : 1;  // stages per tile
+  static constexpr int kEpiWarps = CV ? 4 : 16;
+  static constexpr int kThreads = 32 * (2 + kEpiWarps + (CV ? kConvertWarps : 0));
+  static constexpr int kShares = kEpiWarps / 4;       // column shares of a row block (pass 1), of a tile's rows (pass 2)
   static constexpr int kStageBytes = NS == 3 ? kTileKeys * 128 : kTileKeys * D * 2;
   static constexpr int kQRows = NS == 3 ? 128 : 256;  // up to two blocks of 128 rows
   static constexpr int kQBytes = kQRows * D * 2 * NS;
@@ -243,6 +266,7 @@ struct TileCursor {
 };
 struct Run {
   int u, b, n;  // unit, its sequence and that sequence's length
+  int l, h;     // layer and KV head
   int t0, cnt;  // first tile of the run within the unit, tiles in the run (what the partition counts)
   int tiles;    // tiles of the run that hold keys (fewer than cnt only in the uniform partition of very large batches)
 };
@@ -269,8 +293,16 @@ __device__ __forceinline__ void cursor_settle(const RowParams& p, TileCursor& c,
 }
 __device__ __forceinline__ Run cursor_run(const RowParams& p, const TileCursor& c, const int* lens) {
   Run r;
-  const int ub = c.r / c.tb;
-  r.t0 = c.r - ub * c.tb;
+  int ub = 0;  // c.r / c.tb: by the reciprocal, then put right (it is off by one at most, there are few units per sequence)
+  r.t0 = c.r;
+  if (c.r >= c.tb) {
+    ub = (int)((float)c.r * __frcp_rn((float)c.tb));
+    r.t0 = c.r - ub * c.tb;
+    while (r.t0 < 0) --ub, r.t0 += c.tb;
+    while (r.t0 >= c.tb) ++ub, r.t0 -= c.tb;
+  }
+  r.l = p.by_hkv.div(ub);
+  r.h = ub - r.l * p.Hkv;
   r.cnt = min(c.tb - r.t0, c.left);
   r.b = c.b;
   r.u = c.b * p.lh + ub;
@@ -293,10 +325,45 @@ __device__ __forceinline__ int cta_of(int total, int ctas, int x) {
   return x < more * (q + 1) ? x / (q + 1) : more + (x - more * (q + 1)) / q;  // (x < total, so q > 0 in the second case)
 }
 
-template <int D, int PASS, int NS>
-__global__ void __launch_bounds__(kRowThreads, 1)  // 96 registers: warps are allocated four at a time (18 -> 20)
+// Four fp32 values as three bf16 terms each, whose sum is the value exactly (8 significand bits per term): lo goes to `store`,
+// hi (x, y) and mid (z, w) are returned, packed.
+template <typename Store>
+__device__ __forceinline__ uint4 split4(float4 v, Store store) {
+  auto pack = [](float a, float b) {
+    const __nv_bfloat162 x = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&x);
+  };
+  auto low = [](uint32_t x) { return __uint_as_float(x << 16); };
+  auto high = [](uint32_t x) { return __uint_as_float(x & 0xffff0000u); };
+  uint4 t;
+  t.x = pack(v.x, v.y);
+  t.y = pack(v.z, v.w);
+  // (values that would round up to infinity are cut off instead)
+  if (max3f(fabsf(v.x), fabsf(v.y), fmaxf(fabsf(v.z), fabsf(v.w))) >= __uint_as_float(0x7f7f8000u)) {
+    t.x = (__float_as_uint(v.x) >> 16) | (__float_as_uint(v.y) & 0xffff0000u);
+    t.y = (__float_as_uint(v.z) >> 16) | (__float_as_uint(v.w) & 0xffff0000u);
+  }
+  v.x = __fsub_rn(v.x, low(t.x));
+  v.y = __fsub_rn(v.y, high(t.x));
+  v.z = __fsub_rn(v.z, low(t.y));
+  v.w = __fsub_rn(v.w, high(t.y));
+  t.z = pack(v.x, v.y);
+  t.w = pack(v.z, v.w);
+  store(make_uint2(pack(__fsub_rn(v.x, low(t.z)), __fsub_rn(v.y, high(t.z))), pack(__fsub_rn(v.z, low(t.w)), __fsub_rn(v.w, high(t.w)))));
+  return t;
+}
+
+// A load that stays where it is written (the compiler may move a plain one down to its use, which is a step later).
+__device__ __forceinline__ float4 load4(const float* p) {
+  float4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+
+template <int D, int PASS, int NS, bool CV>
+__global__ void __launch_bounds__((RowSmem<D, PASS, NS, CV>::kThreads), 1)  // 96 registers: warps are allocated four at a time (18 -> 20)
 score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_q, RowParams p) {
-  using SL = RowSmem<D, PASS, NS>;
+  using SL = RowSmem<D, PASS, NS, CV>;
   constexpr int kStages = SL::kStages;
   constexpr int kKBlocks = SL::kKBlocks;
   extern __shared__ uint8_t smem_raw[];
@@ -322,23 +389,24 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
   int* rowpos = reinterpret_cast<int*>(smem + SL::kColOff);
   int* rowoff = reinterpret_cast<int*>(smem + SL::kOffOff);
   float* xch = reinterpret_cast<float*>(smem + SL::kXchOff);
+  int* rowhead = reinterpret_cast<int*>(xch);  // fp32, whose tiles are not shared out: query head of every row within the launch's
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
-      mbar_init(&full[s], 1);
+      mbar_init(&full[s], CV ? kConvertWarps : 1);
       mbar_init(&empty[s], 1);
     }
     for (int i = 0; i < 2; ++i) {
-      mbar_init(&qfull[i], PASS == 2 ? 2 : 1);
+      mbar_init(&qfull[i], (CV ? kConvertWarps : 1) + (PASS == 2 ? 1 : 0));
       mbar_init(&qempty[i], 1);
       mbar_init(&tfull[i], 1);
-      mbar_init(&tempty[i], 512);  // every epilogue thread
+      mbar_init(&tempty[i], 32 * SL::kEpiWarps);  // every epilogue thread
     }
     mbar_init(drain, 1);
     for (int i = 0; i < 8; ++i) {
-      mbar_init(&xfull[i], 96);
+      mbar_init(&xfull[i], SL::kShares > 1 ? 32 * (SL::kShares - 1) : 1);
       mbar_init(&xempty[i], 32);
     }
     *abort_flag = 0;
@@ -347,14 +415,15 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
   // rows R..255 of the Q buffer are never written by TMA: keep them zero so their logits are 0. Pass 2: the operands
   // of the extra contraction step start out as zeros, the key side gets its three ones per row (128-byte rows with
   // the 128-byte swizzle: the 16-byte piece that holds columns 0-7 of row r sits at position r % 8).
-  for (int x = threadIdx.x; x < (SL::kBarOff - SL::kQOff) / 16; x += kRowThreads)
+  for (int x = threadIdx.x; x < (SL::kBarOff - SL::kQOff) / 16; x += SL::kThreads)
     reinterpret_cast<uint4*>(q_s)[x] = make_uint4(0, 0, 0, 0);
   if (threadIdx.x < 256) {
-    const int x = threadIdx.x, hh = x / p.wc, pos = p.r0 + x - hh * p.wc;
+    const int x = threadIdx.x, hh = p.by_wc.div(x), pos = p.r0 + x - hh * p.wc;
     rowpos[x] = pos;
+    if (CV && x < 128) rowhead[x] = hh;
     rowoff[x] = x < p.R ? hh * p.w + pos : 0;
   }
-  if (threadIdx.x == 32) {
+  if (!CV && threadIdx.x == 32) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_k) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmap_q) : "memory");
   }
@@ -377,7 +446,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
   pdl_go();
   const int* lens = p.B <= kMaxSeqScan ? len_s : nullptr;
   if (lens)
-    for (int b = threadIdx.x; b < p.B; b += kRowThreads) len_s[b] = clamped_len(p.seq_len, b, p.n_max);
+    for (int b = threadIdx.x; b < p.B; b += SL::kThreads) len_s[b] = clamped_len(p.seq_len, b, p.n_max);
   __syncthreads();
   if (threadIdx.x == 0) {
     // this CTA's range of tiles
@@ -437,7 +506,8 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
 
   if (warp == 0) {
     // ================================================================ TMA producer: lane 0 waits and issues the copies;
-    // in pass 2 all lanes write the units' shift rows
+    // in pass 2 all lanes write the units' shift rows (with
+    // CV all that this warp does)
     const uint64_t pol_k = NS == 3 ? l2_policy_evict_last() : l2_policy_evict_first();  // (split keys are read again)
     const uint64_t pol_q = l2_policy_evict_last();
     int stage = 0, k = 0;  // k: units begun
@@ -448,8 +518,9 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
       cursor_advance(p, c, run, lens);
       const int u = run.u, key_begin = run.t0 * kTileKeys, loads = run.tiles * SL::kPieces;
       if (loads == 0) continue;
-      // fp32: the slice's split operands are [units][n_max][3 D] and [units * g][w][3 D]
-      const int h = NS == 3 ? u : u % p.Hkv, l = NS == 3 ? 0 : (u / p.Hkv) % p.L, b = NS == 3 ? 0 : u / p.lh;
+      const int h = run.h, l = run.l, b = run.b;
+      // split operands are [units][n_max][3 D] and [units * g][w][3 D]
+      const int th = NS == 3 ? u : h, tl = NS == 3 ? 0 : l, tb = NS == 3 ? 0 : b;
       const int buf = k % nq;
       const uint32_t q_par = (uint32_t)(k / nq) & 1u;
       // Row r of the shift operand: -lse_r / scale as the sum of three bf16 numbers (24 bits) in columns 0-2. Multiplied by
@@ -457,8 +528,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
       // per-row operand at all. (All loads first; one after the other they took 5 us.)
       float nl[SL::kQRows / 32];
       if (PASS == 2) {
-        const int gh = (p.u0 + u) % p.Hkv, gbl = (p.u0 + u) / p.Hkv;
-        const float* src = p.given_lse ? p.given_lse + ((int64_t)gbl * p.Hq + gh * p.g + p.h0) * p.w : p.lse2 + (int64_t)u * p.rs;
+        const float* src = p.given_lse ? p.given_lse + (((int64_t)b * p.L + l) * p.Hq + h * p.g + p.h0) * p.w : p.lse2 + (int64_t)u * p.rs;
 #pragma unroll
         for (int i = 0; i < SL::kQRows / 32; ++i) {
           const int r = lane + 32 * i;
@@ -472,13 +542,13 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
           ok = mbar_wait(&empty[stage], stage_par ^ 1, abort_flag, p.status, kSiteStage);
           if (!ok) break;
           mbar_expect_tx(&full[stage], (uint32_t)SL::kStageBytes);
-          if (NS == 3) {
-            tma_load_5d(k_s + stage * SL::kStageBytes, &tmap_k, &full[stage],
-                        ((2 - piece / kKBlocks) * kKBlocks + piece % kKBlocks) * 64, key_begin + t * kTileKeys, h, l, b, pol_k);
+          if (NS == 3) {  // (the order of the MMA issuer: lo, mid, hi of 64 columns, then of the others)
+            tma_load_5d(k_s + stage * SL::kStageBytes, &tmap_k, &full[stage], ((2 - piece % 3) * kKBlocks + piece / 3) * 64,
+                        key_begin + t * kTileKeys, th, tl, tb, pol_k);
           } else {
             for (int kb = 0; kb < kKBlocks; ++kb)
               tma_load_5d(k_s + stage * SL::kStageBytes + kb * kTileKeys * 128, &tmap_k, &full[stage], kb * 64,
-                          key_begin + t * kTileKeys, h, l, b, pol_k);
+                          key_begin + t * kTileKeys, th, tl, tb, pol_k);
           }
           if (++stage == kStages) {
             stage = 0;
@@ -492,12 +562,12 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
       const int ahead = k == 0 ? 1 : min(kStages, loads);
       ++k;
       if (lane == 0) {
-        load_keys(0, ahead);
+        if (!CV) load_keys(0, ahead);
         ok = ok && mbar_wait(&qempty[buf], q_par ^ 1, abort_flag, p.status, kSiteQEmpty);
-        if (ok) {
+        if (ok && !CV) {
           mbar_expect_tx(&qfull[buf], (uint32_t)(p.R * 128 * kKBlocks * NS));
           for (int kb = 0; kb < kKBlocks * NS; ++kb)
-            tma_load_5d(q_s + (kb * SL::kQRows + buf * 128) * 128, &tmap_q, &qfull[buf], kb * 64, p.r0, h * p.g + p.h0, l, b, pol_q);
+            tma_load_5d(q_s + (kb * SL::kQRows + buf * 128) * 128, &tmap_q, &qfull[buf], kb * 64, p.r0, th * p.g + p.h0, tl, tb, pol_q);
         }
       }
       if (PASS == 2) {
@@ -523,16 +593,16 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
         __syncwarp();  // every lane's rows are written (and fenced) before lane 0 signals them
         if (lane == 0) mbar_arrive(&qfull[buf]);
       }
-      if (lane == 0) load_keys(ahead, loads);
+      if (!CV && lane == 0) load_keys(ahead, loads);
       ok = __shfl_sync(0xffffffffu, ok, 0);
     }
-    if (!ok && lane == 0) {  // abandoned: give copies in flight time to land before the CTA's shared memory goes away
+    if (!CV && !ok && lane == 0) {  // abandoned: give copies in flight time to land before the CTA's shared memory goes away
       const long long t0 = clock64();
       while (clock64() - t0 < 2000000ll) __nanosleep(1000);
     }
   } else if (warp == 1) {
     // ================================================================ MMA issuer
-    if (lane == 0) {
+    if (CV ? elect_one() : lane == 0) {
       const uint32_t k_lo0 = smem_desc_lo(smem_u32(k_s)), q_lo00 = smem_desc_lo(smem_u32(q_s));
       const uint32_t ones_lo = smem_desc_lo(smem_u32(ones_s)), shift_lo0 = smem_desc_lo(smem_u32(shift_s));
       const uint32_t idesc2 = instr_desc_bf16(p.n16);
@@ -555,10 +625,10 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
           ok = mbar_wait(&tempty[buf], use_par ^ 1, abort_flag, p.status, kSiteTEmpty);
           if (!ok) break;
           if (NS == 3) {
-            // A stage is 64 contraction steps of one term of the keys, in the order lo, mid, hi. The accumulation
-            // truncates, so the small products come first (lo hi, mid hi, mid mid, hi lo, hi mid) and the 8 or 4 steps of
-            // hi hi last, for which the stages of hi are held: the result is as exact as that of a plain bf16 contraction.
-            // (hi hi first: log-sum-exps off by 7e-7 instead of 6e-8, relative.)
+            // A stage is one term of 64 columns of the keys, in the order lo, mid, hi of the first 64, then of the others. The
+            // accumulation truncates, so the small products come first (lo hi, mid hi, mid mid, hi lo, hi mid) and the 8 or 4
+            // steps of hi hi last, for which the stages of hi are held: the result is as exact as that of a plain bf16
+            // contraction. (hi hi first: log-sum-exps off by 7e-7 instead of 6e-8, relative.)
             auto product = [&](uint32_t k_lo, int qt, int kb, uint32_t first) {
 #pragma unroll
               for (int kk = 0; kk < 4; ++kk) {
@@ -571,8 +641,8 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
             uint32_t hi_lo[kKBlocks];
             int hi_stage[kKBlocks];
 #pragma unroll
-            for (int piece = 0; piece < SL::kPieces; ++piece) {
-              const int term = 2 - piece / kKBlocks, kb = piece % kKBlocks;
+            for (int piece = 0; piece < 3 * kKBlocks; ++piece) {
+              const int term = 2 - piece % 3, kb = piece / 3;
               ok = ok && mbar_wait(&full[stage], stage_par, abort_flag, p.status, kSiteFull);
               if (ok) {
                 tc_fence_after();
@@ -642,14 +712,15 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
         while (!mbar_try(drain, 0) && clock64() - t0 < 20000000ll) __nanosleep(200);
       }
     }
-  } else {
-    // ================================================================ epilogue (warps 2-17)
-    // All 16 warps work on the same tile while the MMAs of the next tile fill the other accumulator buffer;
+  } else if (warp < 2 + SL::kEpiWarps) {
+    // ================================================================ epilogue (warps 2-17, with CV 2-5)
+    // All of its warps work on the same tile while the MMAs of the next tile fill the other accumulator buffer;
     // warp = (TMEM lane quarter, column share); the TMEM load of a warp's next 16 columns is in flight while it works.
     const int ew = warp - 2;
     const int quarter = warp & 3;  // TMEM lanes [32 * quarter, 32 * quarter + 32)
-    // pass 1: (row block mb, column share): two row blocks x 2 shares of 64 keys, or one row block x 4 shares of 32
-    // pass 2: column share = a quarter of the n16 / 16 blocks of window rows (as even as possible)
+    // pass 1: (row block mb, column share): two row blocks x 2 shares of 64 keys, or one row block x 4 shares of 32 (CV:
+    // one of 128)
+    // pass 2: column share = a quarter (CV: all) of the n16 / 16 blocks of window rows (as even as possible)
     const int mb = PASS == 1 && p.mblocks == 2 ? (ew >> 2) & 1 : 0;
     const int share = PASS == 1 ? (p.mblocks == 2 ? ew >> 3 : ew >> 2) : ew >> 2;
     int blk0, nblk;  // this warp's 16-column blocks of a tile's accumulator: blk0 .. blk0 + nblk - 1
@@ -657,7 +728,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
       nblk = 8 / p.cparts;
       blk0 = nblk * share;
     } else {
-      const int total = p.n16 >> 4, base = total >> 2, rem = total & 3;
+      const int total = p.n16 >> 4, base = total / SL::kShares, rem = total % SL::kShares;
       nblk = base + (share < rem ? 1 : 0);
       blk0 = share * base + min(share, rem);
     }
@@ -675,7 +746,8 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
     if (PASS == 2 && range_s[3] && !p.accumulate) {  // sequences without keys have no tiles
       for (int b = 0; b < p.B; ++b)
         if (len_s[b] == 0)
-          for (int64_t x = (int64_t)blockIdx.x * 512 + ew * 32 + lane; x < (int64_t)p.lh * p.n_max; x += (int64_t)gridDim.x * 512)
+          for (int64_t x = ((int64_t)blockIdx.x * SL::kEpiWarps + ew) * 32 + lane; x < (int64_t)p.lh * p.n_max;
+               x += (int64_t)gridDim.x * SL::kEpiWarps * 32)
             p.psi[(int64_t)b * p.lh * p.n_max + x] = 0.f;
     }
 
@@ -690,7 +762,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
       zacc[0] = zacc[1] = zacc[2] = zacc[3] = 0ull;
       int vis = 0;  // pass 1: keys the row may see: [0, vis)
       if (PASS == 1 && row < p.R) {
-        const int pos = n - p.w + p.r0 + row % p.wc;
+        const int pos = n - p.w + rowpos[row];
         if (pos >= 0) vis = p.causal ? pos + 1 : n;
       }
       for (int t = 0; t < tiles; ++t, ++n_tile) {
@@ -744,10 +816,15 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
         };
         if (plain) {  // all but the tiles at the window
           if (PASS == 1) {
-            if (nblk == 4) stat_tile<4>(taddr, p.scale2, sc2, m, zacc, z_run);
+            if (SL::kShares == 1) stat_tile<8>(taddr, p.scale2, sc2, m, zacc, z_run);
+            else if (nblk == 4) stat_tile<4>(taddr, p.scale2, sc2, m, zacc, z_run);
             else stat_tile<2>(taddr, p.scale2, sc2, m, zacc, z_run);
           } else {
             switch (nblk) {
+              case 8: if (SL::kShares == 1) psi_tile<8>(taddr, sc2, acc); break;
+              case 7: if (SL::kShares == 1) psi_tile<7>(taddr, sc2, acc); break;
+              case 6: if (SL::kShares == 1) psi_tile<6>(taddr, sc2, acc); break;
+              case 5: if (SL::kShares == 1) psi_tile<5>(taddr, sc2, acc); break;
               case 4: psi_tile<4>(taddr, sc2, acc); break;
               case 3: psi_tile<3>(taddr, sc2, acc); break;
               case 2: psi_tile<2>(taddr, sc2, acc); break;
@@ -776,19 +853,22 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
           zacc[0] = zacc[1] = zacc[2] = zacc[3] = 0ull;
         }
         if (PASS == 2) {
-          // the four warps that share the key add up in a fixed order: shares 1-3 hand their sums to share 0 (a
+          // the warps that share the key add up in a fixed order: shares 1-3 hand their sums to share 0 (a
           // slot is free once share 0 has taken the tile before last)
           float total = sum4(acc);
           const uint32_t xp = (uint32_t)(n_tile >> 1) & 1u;
-          if (share) {
+          if (SL::kShares == 1) {
+            if (key < p.n_max) psi[key] = key < n ? (p.accumulate ? psi[key] + total : total) : 0.f;
+          } else if (share) {
             ok = __all_sync(0xffffffffu, mbar_wait(&xempty[buf * 4 + quarter], xp ^ 1, abort_flag, p.status, kSiteFlag));
             if (!ok) break;
-            xslot[(buf * 3 + share - 1) * 128] = total;
+            xslot[(buf * (SL::kShares - 1) + share - 1) * 128] = total;
             mbar_arrive(&xfull[buf * 4 + quarter]);
           } else {
             ok = __all_sync(0xffffffffu, mbar_wait(&xfull[buf * 4 + quarter], xp, abort_flag, p.status, kSiteFlag));
             if (!ok) break;
-            total = ((total + xslot[(buf * 3 + 0) * 128]) + xslot[(buf * 3 + 1) * 128]) + xslot[(buf * 3 + 2) * 128];
+#pragma unroll
+            for (int x = 0; x < SL::kShares - 1; ++x) total += xslot[(buf * (SL::kShares - 1) + x) * 128];
             mbar_arrive(&xempty[buf * 4 + quarter]);
             if (key < p.n_max) psi[key] = key < n ? (p.accumulate ? psi[key] + total : total) : 0.f;
           }
@@ -796,7 +876,8 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
       }
       if (PASS == 2 && ok && !p.accumulate && run.t0 + run.cnt >= (n + kTileKeys - 1) / kTileKeys) {
         // the keys no tile covers, by the CTA that has the unit's last tile
-        for (int key = (n + kTileKeys - 1) / kTileKeys * kTileKeys + ew * 32 + lane; key < p.n_max; key += 512) psi[key] = 0.f;
+        for (int key = (n + kTileKeys - 1) / kTileKeys * kTileKeys + ew * 32 + lane; key < p.n_max; key += SL::kEpiWarps * 32)
+          psi[key] = 0.f;
       }
       if (!ok) break;
       if (PASS == 1) {
@@ -805,13 +886,121 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
           // one pair per run: slot = this CTA's place among the CTAs that the unit's tiles are spread over (the merge
           // kernel walks the same partition). A row that saw no visible key only summed masked entries: it is
           // recorded as empty, and so is a run without keys (the uniform partition of very large batches has those).
-          const int k = (int)blockIdx.x - cta_of(range_s[5], range_s[6], run_first - run.t0);
+          const int k = run.t0 ? (int)blockIdx.x - cta_of(range_s[5], range_s[6], run_first - run.t0) : 0;
           const bool none = tiles == 0 || m < 0.5f * kEmptyMax * p.scale2;
           if (k >= 0 && k < p.smax)
             p.part[(((int64_t)u * p.smax + k) * p.cparts + share) * p.rs + row] =
                 none ? make_float2(kEmptyMax, 0.f) : make_float2(m, z_run);
           else
             set_status(p.status, MADAKV_ESHAPE);  // cannot happen: smax bounds the runs of a unit
+        }
+      }
+    }
+  }
+  if constexpr (CV) {
+    if (warp >= 2 + SL::kEpiWarps) {
+      // ============================================================== converters (CV): a step is 64 columns of the 128 keys of
+      // a tile; half a warp reads the 256 bytes of a row, and each thread turns 8 x 4 values into three terms each, written as
+      // three stages. The next step's values are on their way to registers meanwhile, those of two steps later to the L2.
+      const int cw = warp - 2 - SL::kEpiWarps, sub = lane >> 4, c4 = (lane & 15) * 4;  // rows kStep * i + 2 * cw + sub, columns c4 .. c4 + 3
+      const int r0 = 2 * cw + sub;
+      constexpr int kStep = 2 * kConvertWarps, kRep = kTileKeys / kStep;  // rows per load of all warps, loads per thread and step
+      auto place = [&](int r) { return r * 128 + (((lane & 15) >> 1) ^ (r & 7)) * 16 + (lane & 1) * 8; };  // in a piece
+      int stage = 0, k = 0;
+      uint32_t stage_par = 0;
+      bool ok = true;
+      for (TileCursor c = cursor_begin(); ok && c.left > 0;) {
+        const Run run = cursor_run(p, c, lens);
+        cursor_advance(p, c, run, lens);
+        if (run.tiles == 0) continue;
+        const int h = run.h, l = run.l, b = run.b, n = run.n;
+        const float* kf = p.kf + b * p.sk.batch + l * p.sk.layer + h * p.sk.head;
+        const float* qf = p.qf + b * p.sq.batch + l * p.sq.layer + (int64_t)(h * p.g + p.h0) * p.sq.head;
+        const int steps = run.tiles * kKBlocks;
+        float4 next[kRep];
+        auto load = [&](int step) {
+          const int key0 = (run.t0 + step / kKBlocks) * kTileKeys + r0;
+          const float* src = kf + (step % kKBlocks) * 64 + c4;
+#pragma unroll
+          for (int i = 0; i < kRep; ++i)
+            next[i] = key0 + kStep * i < n ? load4(src + (int64_t)(key0 + kStep * i) * p.sk.token)
+                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+        };
+        auto prefetch = [&](int step) {  // 2 x 128 bytes of each of the 128 rows, one per thread
+          const int x = cw * 32 + lane, key = (run.t0 + step / kKBlocks) * kTileKeys + (x >> 1);
+          if (x < 256 && step < steps && key < n)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(kf + (int64_t)key * p.sk.token + (step % kKBlocks) * 64 + (x & 1) * 32));
+        };
+        load(0);
+        // the unit's queries
+        float4 qv[kKBlocks][kRep];
+#pragma unroll
+        for (int kb = 0; kb < kKBlocks; ++kb)
+#pragma unroll
+          for (int i = 0; i < kRep; ++i) {
+            const int r = r0 + kStep * i;
+            qv[kb][i] = r < p.R ? load4(qf + rowhead[r] * p.sq.head + rowpos[r] * p.sq.token + kb * 64 + c4) : make_float4(0.f, 0.f, 0.f, 0.f);
+          }
+        prefetch(1);
+        prefetch(2);
+        ok = __all_sync(0xffffffffu, mbar_wait(&qempty[0], ((uint32_t)k & 1u) ^ 1u, abort_flag, p.status, kSiteQEmpty));
+        if (!ok) break;
+        ++k;
+#pragma unroll
+        for (int kb = 0; kb < kKBlocks; ++kb)
+#pragma unroll
+          for (int i = 0; i < kRep; ++i) {
+            uint8_t* to = q_s + kb * SL::kQRows * 128 + place(r0 + kStep * i);
+            constexpr int kTerm = kKBlocks * SL::kQRows * 128;
+            const uint4 t = split4(qv[kb][i], [&](uint2 lo) { *reinterpret_cast<uint2*>(to + 2 * kTerm) = lo; });
+            *reinterpret_cast<uint2*>(to + kTerm) = make_uint2(t.z, t.w);
+            *reinterpret_cast<uint2*>(to) = make_uint2(t.x, t.y);
+          }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&qfull[0]);
+        // its keys
+        auto take_stage = [&]() {
+          ok = __all_sync(0xffffffffu, mbar_wait(&empty[stage], stage_par ^ 1u, abort_flag, p.status, kSiteStage));
+          return k_s + stage * SL::kStageBytes;
+        };
+        auto give_stage = [&]() {
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&full[stage]);
+          if (++stage == kStages) {
+            stage = 0;
+            stage_par ^= 1;
+          }
+        };
+#pragma unroll 1
+        for (int step = 0; step < steps; ++step) {
+          uint4 t[kRep];  // hi and mid of four values each, packed
+          uint8_t* to = take_stage();
+          if (!ok) break;
+#pragma unroll
+          for (int i = 0; i < kRep; ++i)
+            t[i] = split4(next[i], [&](uint2 lo) { *reinterpret_cast<uint2*>(to + place(r0 + kStep * i)) = lo; });
+          give_stage();
+          if (step + 1 < steps) load(step + 1);
+          prefetch(step + 3);
+          const int s1 = stage, s2 = stage + 1 == kStages ? 0 : stage + 1;
+          const uint32_t par2 = s2 ? stage_par : stage_par ^ 1u;
+          const bool free = mbar_wait(&empty[s1], stage_par ^ 1u, abort_flag, p.status, kSiteStage) &&
+                            mbar_wait(&empty[s2], par2 ^ 1u, abort_flag, p.status, kSiteStage);
+          ok = __all_sync(0xffffffffu, free);
+          if (!ok) break;
+#pragma unroll
+          for (int i = 0; i < kRep; ++i) {
+            const int at = place(r0 + kStep * i);
+            *reinterpret_cast<uint2*>(k_s + s1 * SL::kStageBytes + at) = make_uint2(t[i].z, t[i].w);
+            *reinterpret_cast<uint2*>(k_s + s2 * SL::kStageBytes + at) = make_uint2(t[i].x, t[i].y);
+          }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane < 2) mbar_arrive(&full[lane ? s2 : s1]);
+          stage = s2 + 1 == kStages ? 0 : s2 + 1;
+          stage_par = s2 + 1 == kStages ? par2 ^ 1u : par2;
         }
       }
     }
@@ -828,8 +1017,8 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
 
 // merge: per (unit, row) the (max, sum) pairs of all runs and column shares, in a fixed order -> log2-domain log-sum-exp,
 // stored negated (pass 2 adds it inside the contraction); padding rows get a shift that turns every weight into 0. A block
-// takes 32 rows of one unit, eight threads per row: a unit of an fp32 slice can be spread over half of the CTAs (one thread
-// per row took 53 us for 300 pairs).
+// takes 32 rows of one unit, eight threads per row: a call's only unit can be spread over all CTAs (one thread per row took 53 us
+// for 300 pairs).
 __global__ void __launch_bounds__(256) score_rows_merge_kernel(RowParams p, float* nlse2, float* lse_out) {
   __shared__ float s_m[8][32], s_z[8][32];
   __shared__ int s_entries;
@@ -892,35 +1081,38 @@ __global__ void __launch_bounds__(256) score_rows_merge_kernel(RowParams p, floa
   const float l2 = Z > 0.f ? M + log2f(Z) : 0.f;
   nlse2[x] = -l2;
   if (lse_out) {
-    const int h = (p.u0 + u) % p.Hkv, bl = (p.u0 + u) / p.Hkv;
+    const int h = u % p.Hkv, bl = u / p.Hkv;
     const int hq = h * p.g + p.h0 + row / p.wc, wr = p.r0 + row % p.wc;
     lse_out[((int64_t)bl * p.Hq + hq) * p.w + wr] = Z > 0.f ? l2 * 0.6931471805599453f : -INFINITY;
   }
 }
 
-template <int D, int PASS, int NS>
+template <int D, int PASS, int NS, bool CV>
 int launch_pass(const CUtensorMap& mk, const CUtensorMap& mq, const RowParams& p, int grid, cudaStream_t st) {
-  using SL = RowSmem<D, PASS, NS>;
-  if (cudaFuncSetAttribute(score_rows_kernel<D, PASS, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SL::kAlloc) !=
+  using SL = RowSmem<D, PASS, NS, CV>;
+  if (cudaFuncSetAttribute(score_rows_kernel<D, PASS, NS, CV>, cudaFuncAttributeMaxDynamicSharedMemorySize, SL::kAlloc) !=
       cudaSuccess)
     return MADAKV_ECUDA;
-  launch_pdl(score_rows_kernel<D, PASS, NS>, dim3(grid), dim3(kRowThreads), (size_t)SL::kAlloc, st, mk, mq, p);
+  launch_pdl(score_rows_kernel<D, PASS, NS, CV>, dim3(grid), dim3(SL::kThreads), (size_t)SL::kAlloc, st, mk, mq, p);
   return MADAKV_OK;
 }
 template <int PASS>
-int launch_pass(const madakv_config& c, const CUtensorMap& mk, const CUtensorMap& mq, const RowParams& p, int grid, cudaStream_t st) {
-  if (c.dtype == MADAKV_F32)
-    return c.head_dim == 128 ? launch_pass<128, PASS, 3>(mk, mq, p, grid, st) : launch_pass<64, PASS, 3>(mk, mq, p, grid, st);
-  return c.head_dim == 128 ? launch_pass<128, PASS, 1>(mk, mq, p, grid, st) : launch_pass<64, PASS, 1>(mk, mq, p, grid, st);
+int launch_pass(const madakv_config& c, bool convert, const CUtensorMap& mk, const CUtensorMap& mq, const RowParams& p, int grid, cudaStream_t st) {
+  const bool wide = c.head_dim == 128;
+  if (c.dtype != MADAKV_F32)
+    return wide ? launch_pass<128, PASS, 1, false>(mk, mq, p, grid, st) : launch_pass<64, PASS, 1, false>(mk, mq, p, grid, st);
+  if (convert)
+    return wide ? launch_pass<128, PASS, 3, true>(mk, mq, p, grid, st) : launch_pass<64, PASS, 3, true>(mk, mq, p, grid, st);
+  return wide ? launch_pass<128, PASS, 3, false>(mk, mq, p, grid, st) : launch_pass<64, PASS, 3, false>(mk, mq, p, grid, st);
 }
 
 // ---- fp32 operands -> three bf16 terms each, whose sum is the operand exactly (8 significand bits per term)
 struct SplitParams {
   const float* src;
-  __nv_bfloat16* dst;  // [rows of the slice][3][D]
+  __nv_bfloat16* dst;  // [rows][3][D]
   const int32_t* seq_len;
   madakv_strides s;    // of src, in elements
-  int L, H, D, tokens, head0;  // head0: first head of the slice; seq_len: nullptr = all tokens
+  int L, H, D, tokens;  // seq_len: nullptr = all tokens
 };
 // (blocks: first the keys' heads, k_blocks each, then the queries')
 __global__ void __launch_bounds__(256) split_kernel(SplitParams pk, SplitParams pq, int k_heads, int k_blocks, int q_blocks) {
@@ -933,49 +1125,36 @@ __global__ void __launch_bounds__(256) split_kernel(SplitParams pk, SplitParams 
   const int per = is_q ? q_blocks : k_blocks, y = bx / per;
   const int lg = p.D == 128 ? 5 : 4;  // 16-byte pieces per row: 32 or 16
   const int x = (bx - y * per) * 256 + threadIdx.x, tok = x >> lg, c = (x & ((1 << lg) - 1)) * 4;
-  const int hh = y + p.head0;  // head of the call, counted over (sequence, layer, head)
-  const int h = hh % p.H, l = hh / p.H % p.L, b = hh / (p.H * p.L);
+  const int h = y % p.H, l = y / p.H % p.L, b = y / (p.H * p.L);
   if (tok >= (p.seq_len ? clamped_len(p.seq_len, b, p.tokens) : p.tokens)) return;  // (keys beyond the sequence are masked)
   const int64_t row = (int64_t)y * p.tokens + tok;
   const float4 v = __ldg(reinterpret_cast<const float4*>(p.src + b * p.s.batch + l * p.s.layer + h * p.s.head + tok * p.s.token + c));
-  const float f[4] = {v.x, v.y, v.z, v.w};
-  uint32_t t[3][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float r = f[i];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      uint32_t hi = __float_as_uint(__bfloat162float(__float2bfloat16_rn(r)));
-      if ((hi & 0x7fffffffu) == 0x7f800000u) hi = __float_as_uint(r) & 0xffff0000u;  // (rounded up to infinity: cut off instead)
-      t[k][i] = hi >> 16;
-      r = __fsub_rn(r, __uint_as_float(hi));
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-    *reinterpret_cast<uint2*>(p.dst + (row * 3 + k) * p.D + c) = make_uint2(t[k][0] | (t[k][1] << 16), t[k][2] | (t[k][3] << 16));
+  __nv_bfloat16* dst = p.dst + row * 3 * p.D + c;
+  const uint4 t = split4(v, [&](uint2 lo) { *reinterpret_cast<uint2*>(dst + 2 * p.D) = lo; });
+  *reinterpret_cast<uint2*>(dst + p.D) = make_uint2(t.z, t.w);
+  *reinterpret_cast<uint2*>(dst) = make_uint2(t.x, t.y);
 }
 
-// One slice of the units (bf16: all of them), window rows chunk by chunk. given_lse: single pass with supplied log-sum-exps.
-struct Slice {
-  int b0, B, u0, lh;  // first sequence, sequences, first unit, units per sequence
-};
-int score_slice(const madakv_config& c, const Slice& sl, const void* q, madakv_strides sq, const void* k, madakv_strides sk,
-                const int32_t* seq_len, const float* given_lse, float* lse, float* psi, void* ws, cudaStream_t st) {
+// Window rows chunk by chunk. given_lse: single pass with supplied log-sum-exps.
+int score_rows(const madakv_config& c, const void* q, madakv_strides sq, const void* k, madakv_strides sk, const int32_t* seq_len,
+               const float* given_lse, float* lse, float* psi, void* ws, cudaStream_t st) {
   const WsLayout wl = ws_layout(c);
   const bool f32 = c.dtype == MADAKV_F32;
   const int g = c.n_q_heads / c.n_kv_heads, d = c.head_dim;
   RowParams p;
-  p.seq_len = seq_len + sl.b0;
-  p.psi = psi + (int64_t)sl.u0 * c.max_seq_len;
+  p.seq_len = seq_len;
+  p.psi = psi;
   p.part = reinterpret_cast<float2*>((char*)ws + wl.score_part_off);
   float* lse2 = reinterpret_cast<float*>((char*)ws + wl.score_lse_off);
   p.lse2 = lse2;
   p.status = reinterpret_cast<int32_t*>(ws);
-  p.B = sl.B;
-  p.units = sl.B * sl.lh;
-  p.lh = sl.lh;
-  p.u0 = sl.u0;
+  p.B = c.batch;
+  p.lh = c.n_layers * c.n_kv_heads;
+  p.units = c.batch * p.lh;
+  p.qf = static_cast<const float*>(q);
+  p.kf = static_cast<const float*>(k);
+  p.sq = sq;
+  p.sk = sk;
   p.L = c.n_layers;
   p.Hq = c.n_q_heads;
   p.Hkv = c.n_kv_heads;
@@ -983,8 +1162,9 @@ int score_slice(const madakv_config& c, const Slice& sl, const void* q, madakv_s
   p.w = c.window;
   p.n_max = c.max_seq_len;
   p.causal = c.causal;
-  p.smax = wide_max_runs(sl.lh, c.max_seq_len);
+  p.smax = wide_max_runs(p.lh, c.max_seq_len);
   p.scale2 = scale_of(c) * kLog2e;
+  p.by_hkv = FastDiv(c.n_kv_heads);
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -994,18 +1174,19 @@ int score_slice(const madakv_config& c, const Slice& sl, const void* q, madakv_s
   if (sms > kWideMaxGrid) sms = kWideMaxGrid;
   const int grid = (int)(tiles < sms ? tiles : sms);
   p.grid = grid;
-  CUtensorMap mk, mq;
+  const bool convert = f32 && (given_lse || !split_first(c));
+  CUtensorMap mk = {}, mq = {};  // (convert: not used)
   const madakv_strides split_k{0, 0, (int64_t)c.max_seq_len * 3 * d, 3 * d}, split_q{0, 0, (int64_t)c.window * 3 * d, 3 * d};
-  if (f32) {
+  if (f32 && !convert) {
     __nv_bfloat16* ks = reinterpret_cast<__nv_bfloat16*>((char*)ws + wl.score_split_off);
     __nv_bfloat16* qs = ks + (int64_t)p.units * c.max_seq_len * 3 * d;
     if (!make_map(&mk, ks, 3 * d, c.max_seq_len, p.units, 1, 1, split_k, kTileKeys, 1)) return MADAKV_EUNSUPPORTED;
-    SplitParams x{(const float*)k, ks, seq_len, sk, c.n_layers, c.n_kv_heads, d, c.max_seq_len, sl.u0};
-    SplitParams y{(const float*)q, qs, nullptr, sq, c.n_layers, c.n_q_heads, d, c.window, sl.u0 * g};
+    SplitParams x{(const float*)k, ks, seq_len, sk, c.n_layers, c.n_kv_heads, d, c.max_seq_len};
+    SplitParams y{(const float*)q, qs, nullptr, sq, c.n_layers, c.n_q_heads, d, c.window};
     const int kb = (c.max_seq_len * (d / 4) + 255) / 256, qb = (c.window * (d / 4) + 255) / 256;
     launch_pdl(split_kernel, dim3((unsigned)(p.units * (kb + g * qb))), dim3(256), 0, st, x, y, p.units, kb, qb);
     q = qs;
-  } else if (!make_map(&mk, k, d, c.max_seq_len, c.n_kv_heads, c.n_layers, c.batch, sk, kTileKeys, 1)) {
+  } else if (!f32 && !make_map(&mk, k, d, c.max_seq_len, c.n_kv_heads, c.n_layers, c.batch, sk, kTileKeys, 1)) {
     return MADAKV_EUNSUPPORTED;
   }
   const int rows_max = f32 ? 128 : 256;
@@ -1019,59 +1200,37 @@ int score_slice(const madakv_config& c, const Slice& sl, const void* q, madakv_s
       const int heads = g - p.h0 < hc ? g - p.h0 : hc;
       p.wc = c.window - p.r0 < rc ? c.window - p.r0 : rc;
       p.R = heads * p.wc;
+      p.by_wc = FastDiv(p.wc);
       p.rs = (p.R + 31) / 32 * 32;  // row stride of the workspace arrays
       p.mblocks = p.R <= 128 ? 1 : 2;
-      p.cparts = p.R <= 128 ? 4 : 2;
+      p.cparts = convert ? 1 : (p.R <= 128 ? 4 : 2);
       p.n16 = (p.R + 15) / 16 * 16;
-      if (!(f32 ? make_map(&mq, q, 3 * d, c.window, p.units * g, 1, 1, split_q, p.wc, heads)
-                : make_map(&mq, q, d, c.window, c.n_q_heads, c.n_layers, c.batch, sq, p.wc, heads)))
+      if (!convert && !(f32 ? make_map(&mq, q, 3 * d, c.window, p.units * g, 1, 1, split_q, p.wc, heads)
+                            : make_map(&mq, q, d, c.window, c.n_q_heads, c.n_layers, c.batch, sq, p.wc, heads)))
         return MADAKV_EUNSUPPORTED;
       p.given_lse = given_lse;
       int rc2;
       if (!given_lse) {
-        if ((rc2 = launch_pass<1>(c, mk, mq, p, grid, st))) return rc2;
+        if ((rc2 = launch_pass<1>(c, convert, mk, mq, p, grid, st))) return rc2;
         launch_pdl(score_rows_merge_kernel, dim3(p.units * (p.rs / 32)), dim3(256), 0, st, p, lse2, lse);
       }
-      if ((rc2 = launch_pass<2>(c, mk, mq, p, grid, st))) return rc2;
+      if ((rc2 = launch_pass<2>(c, convert, mk, mq, p, grid, st))) return rc2;
       p.accumulate = 1;
     }
   return launch_status();
-}
-
-// fp32: slices whose split operands fit the workspace's area, whole sequences or a part of one
-int score_slices(const madakv_config& c, const void* q, madakv_strides sq, const void* k, madakv_strides sk, const int32_t* seq_len,
-                 const float* given_lse, float* lse, float* psi, void* ws, cudaStream_t st) {
-  const int lh = c.n_layers * c.n_kv_heads;
-  if (c.dtype != MADAKV_F32)
-    return score_slice(c, Slice{0, c.batch, 0, lh}, q, sq, k, sk, seq_len, given_lse, lse, psi, ws, st);
-  const int most = split_units(c);  // units per slice
-  if (most >= lh) {
-    for (int b = 0; b < c.batch; b += most / lh) {
-      const int nb = c.batch - b < most / lh ? c.batch - b : most / lh;
-      const int rc = score_slice(c, Slice{b, nb, b * lh, lh}, q, sq, k, sk, seq_len, given_lse, lse, psi, ws, st);
-      if (rc) return rc;
-    }
-    return MADAKV_OK;
-  }
-  for (int b = 0; b < c.batch; ++b)
-    for (int u = 0; u < lh; u += most) {
-      const int rc = score_slice(c, Slice{b, 1, b * lh + u, lh - u < most ? lh - u : most}, q, sq, k, sk, seq_len, given_lse, lse, psi, ws, st);
-      if (rc) return rc;
-    }
-  return MADAKV_OK;
 }
 
 }  // namespace
 
 int launch_score_rows(const madakv_config& c, const void* q, madakv_strides sq, const void* k, madakv_strides sk,
                       const int32_t* seq_len, float* lse, float* psi, void* ws, cudaStream_t st) {
-  return score_slices(c, q, sq, k, sk, seq_len, nullptr, lse, psi, ws, st);
+  return score_rows(c, q, sq, k, sk, seq_len, nullptr, lse, psi, ws, st);
 }
 
 // Single-pass scoring with the rows' log-sum-exps supplied by the caller: a conversion kernel, then pass 2 alone.
 int launch_score_lse_rows(const madakv_config& c, const void* q, madakv_strides sq, const void* k, madakv_strides sk,
                           const int32_t* seq_len, const float* lse, float* psi, void* ws, cudaStream_t st) {
-  return score_slices(c, q, sq, k, sk, seq_len, lse, nullptr, psi, ws, st);
+  return score_rows(c, q, sq, k, sk, seq_len, lse, nullptr, psi, ws, st);
 }
 
 }  // namespace madakv

@@ -128,14 +128,15 @@ def test_single_pass_score_with_given_lse(name, causal, path, monkeypatch):
     assert psi_close(buf.psi.cpu().numpy(), two.psi.cpu().numpy().astype(np.float64), 1e-4) < 1e-4
 
 
-# chunks of query heads and of window rows (more than 256 rows per KV head, fp32: 128), and fp32 calls whose split operands come
-# in slices: parts of a sequence, whole sequences, one unit that is larger than a slice would be
+# chunks of query heads and of window rows (more than 256 rows per KV head, fp32: 128), and fp32 calls on both sides of the rule
+# that has their operands split by a kernel before or as they are loaded
 @pytest.mark.parametrize("dtype,B,L,Hq,Hkv,d,n,w", [
     ("bf16", 1, 2, 7, 1, 128, 300, 48), ("bf16", 2, 1, 10, 2, 64, 777, 64), ("bf16", 1, 1, 2, 1, 128, 700, 300),
     ("f32", 2, 1, 6, 2, 64, 389, 50), ("f32", 1, 1, 2, 1, 128, 400, 131), ("f32", 1, 70, 1, 1, 128, 2000, 8),
-    ("f32", 3, 8, 10, 5, 128, 2001, 5), ("f32", 1, 2, 1, 1, 64, 129, 128)])
+    ("f32", 3, 8, 10, 5, 128, 2001, 5), ("f32", 1, 2, 1, 1, 64, 129, 128), ("f32", 2, 40, 3, 1, 64, 389, 50),
+    ("f32", 1, 147, 1, 1, 64, 77, 9), ("f32", 1, 74, 2, 1, 128, 129, 64)])
 @pytest.mark.parametrize("causal", [1, 0])
-def test_score_in_chunks_and_slices(dtype, B, L, Hq, Hkv, d, n, w, causal):
+def test_score_in_chunks(dtype, B, L, Hq, Hkv, d, n, w, causal):
     wl = synth.scaled(TINY, dtype=dtype, B=B, L=L, Hq=Hq, Hkv=Hkv, d=d, n=n, w=w, layout="blocks70", budget=n // 5)
     q = synth.make_q_win(wl)
     k = synth.hash_normal(3, 5, 0, B * L * Hkv * n * d).view(B, L, Hkv, n, d).to(wl.torch_dtype)
