@@ -451,11 +451,7 @@ __device__ __forceinline__ void mass_finish(RankShared<TEAM, 2>& sh, const Alloc
   if (rank != 0 || !p.counter) return;
   __shared__ unsigned s_last;
   __syncthreads();
-  if (tid == 0) {  // (one thread's fences order what the block wrote before the barrier, and will read)
-    __threadfence();
-    s_last = atomicInc(p.counter + b, (unsigned)(p.L * p.Hkv) - 1u);  // (wraps to 0: ready for the next call)
-    __threadfence();
-  }
+  if (tid == 0) s_last = arrive_inc(p.counter + b, (unsigned)(p.L * p.Hkv) - 1u);  // (wraps to 0: ready for the next call)
   __syncthreads();
   if (s_last != (unsigned)(p.L * p.Hkv) - 1u) return;
   static_assert(sizeof(sh.cnt) >= kLayerChunk * 16, "the scan reuses the buckets");

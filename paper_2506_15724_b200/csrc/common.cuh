@@ -227,6 +227,15 @@ __device__ __forceinline__ unsigned long long psi_fix(uint32_t key) {
   return key >= (159u << 23) ? ~0ull : q;
 }
 
+// One arrival at a counter that wraps to 0 behind `last`; the returned number of arrivals before tells the last one. What the
+// caller's block wrote before a barrier before the call is visible to whoever arrives later, and the other way round. (As an atomic
+// between two full fences it took 2300 clocks.)
+__device__ __forceinline__ unsigned arrive_inc(unsigned* counter, unsigned last) {
+  unsigned before;
+  asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;" : "=r"(before) : "l"(counter), "r"(last) : "memory");
+  return before;
+}
+
 __device__ __forceinline__ void set_status(void* ws, int code) { atomicCAS((int*)ws, 0, code); }
 #endif
 

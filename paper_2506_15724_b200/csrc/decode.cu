@@ -191,25 +191,36 @@ __device__ __forceinline__ void finish_segment(const DecodeParams& p, const floa
   }
   __shared__ unsigned s_last;
   __syncthreads();
-  if (threadIdx.x == 0) {  // (one thread's fences order what the whole block wrote before the barrier, and will read)
-    __threadfence();
-    s_last = atomicInc(p.counter + y, (unsigned)p.slots - 1u);  // (wraps to 0: ready for the next call)
-    __threadfence();
-  }
+  if (threadIdx.x == 0) s_last = arrive_inc(p.counter + y, (unsigned)p.slots - 1u);  // (wraps to 0: ready for the next call)
   __syncthreads();
   if (s_last != (unsigned)p.slots - 1u) return;
   if (threadIdx.x == 0 && view.new_row >= 0) p.kept_len[u] = view.len;
-  // weights of the partials, and every head's maximum and sum
+  // weights of the partials, and every head's maximum and sum; the first partials are on their way meanwhile
   __shared__ float s_l[16];
-  for (int i = threadIdx.x / 32; i < p.g; i += NTHR / 32) {
-    const int s = threadIdx.x % 32;
-    const float2 v = s < nb ? __ldcg(p.part_ml + (row0 + i) * p.slots + s) : make_float2(-INFINITY, 0.f);
-    const float m = v.x;
+  constexpr int kFirst = 8, kHeads = 16 * 32 / NTHR;  // heads per warp at most
+  float2 ml[kHeads];
+#pragma unroll
+  for (int j = 0; j < kHeads; ++j) {
+    const int i = (int)threadIdx.x / 32 + j * (NTHR / 32), s = threadIdx.x % 32;
+    ml[j] = i < p.g && s < nb ? __ldcg(p.part_ml + (row0 + i) * p.slots + s) : make_float2(-INFINITY, 0.f);
+  }
+  float4 v[kFirst];
+  auto load_parts = [&](int x, int s0) {
+    const float4* src = reinterpret_cast<const float4*>(p.part + (row0 + x / C4) * p.slots * D + x % C4 * 4);
+#pragma unroll
+    for (int s = 0; s < kFirst; ++s) v[s] = s0 + s < nb ? __ldcg(src + (s0 + s) * C4) : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  if ((int)threadIdx.x < p.g * C4) load_parts(threadIdx.x, 0);
+#pragma unroll
+  for (int j = 0; j < kHeads; ++j) {
+    const int i = (int)threadIdx.x / 32 + j * (NTHR / 32), s = threadIdx.x % 32;
+    if (i >= p.g) break;
+    const float m = ml[j].x;
     float M = m;
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
     const float f = part_weight(m, M);
-    float l = v.y * f;
+    float l = ml[j].y * f;
     if (s < nb) fac[i * kDecodeSlots + s] = f;
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
@@ -221,14 +232,11 @@ __device__ __forceinline__ void finish_segment(const DecodeParams& p, const floa
   __syncthreads();
   for (int x = threadIdx.x; x < p.g * C4; x += NTHR) {
     const int i = x / C4, c = x % C4 * 4;
-    const float4* src = reinterpret_cast<const float4*>(p.part + (row0 + i) * p.slots * D + c);
     float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s0 = 0; s0 < nb; s0 += 8) {
-      float4 v[8];
+    for (int s0 = 0; s0 < nb; s0 += kFirst) {
+      if (s0 || x != (int)threadIdx.x) load_parts(x, s0);
 #pragma unroll
-      for (int s = 0; s < 8; ++s) v[s] = s0 + s < nb ? __ldcg(src + (s0 + s) * C4) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int s = 0; s < 8; ++s) {
+      for (int s = 0; s < kFirst; ++s) {
         const float f = s0 + s < nb ? fac[i * kDecodeSlots + s0 + s] : 0.f;
         O.x += v[s].x * f;
         O.y += v[s].y * f;
@@ -535,7 +543,7 @@ __global__ void __launch_bounds__(kMmaWarps * 32, 3) decode_mma_kernel(const __g
   constexpr int LPR = ROW_BYTES / 16;  // 16-byte pieces per row
   constexpr int KC = D / 16;           // contraction chunks of Q K^T
   constexpr int NB = D / 8;            // 8-column blocks of the output
-  extern __shared__ __align__(16) unsigned char dsmem[];
+  extern __shared__ __align__(128) unsigned char dsmem[];
 
   pdl_wait();
   pdl_go();
@@ -713,9 +721,10 @@ __global__ void __launch_bounds__(kMmaWarps * 32, 3) decode_mma_kernel(const __g
 // Blocks per segment and the rows a block takes at least. The segments' lengths are device data; the rows of the cache per
 // segment stand in for them, so that short segments do not launch blocks only to arrive at the counter.
 //   fewer than 64 segments (one layer of a model): bound by the latency of the blocks, so shares of at least 128 rows
-//     (tensor-core kernel: 256, four iterations of its warps), as many blocks as are resident at once, at most 32 (16
-//     segments of 8725 rows, g = 4: 46 us with 16 blocks each, 56 with 32, which no longer fit; 12 of 53038, g = 1: 72
-//     with 32, 111 with 16)
+//     (tensor-core kernel, two iterations of its warps; 256 where that would be more than a block per SM, because every
+//     block more makes the merge longer: 4 segments of 771 rows, g = 7, 9.7 us at 128, 10.8 at 256; 8 of 1777 8.6 and
+//     9.0; 8 of 2952 11.9 and 10.9; 20 of 2000 15.8 and 15.5), as many blocks as are resident at once, at most 32 (16 segments of 8725 rows, g = 4: 46 us with 16 blocks each, 56 with
+//     32, which no longer fit; 12 of 53038, g = 1: 72 with 32, 111 with 16)
 //   more: shares of 1024 rows where that gives two full waves of blocks, else 512 (896 segments of 2512 rows, g = 7:
 //     190 us at 1024, 197 at 512, 247 at 256; 10240 of 410, g = 1: 311 with one block each, 335 with two; 1024 of 1638,
 //     g = 1: 137 at 1024, 135 at 512; 112 of 3000, g = 1: 44 at 1024, 38 at 512)
@@ -730,7 +739,7 @@ DecodeShape decode_shape(const madakv_config& c, int n_sel, int64_t capacity, bo
   const int resident = 148 * (tensor_core_kernel ? 3 : 7);
   int share, most;
   if (n_sel < 64) {
-    share = tensor_core_kernel ? 256 : 128;
+    share = tensor_core_kernel && n_sel * ((rows + 127) / 128) > 148 ? 256 : 128;
     most = resident / n_sel < kDecodeSlots ? resident / n_sel : kDecodeSlots;
   } else {
     share = n_sel * (rows / 1024 + 1) >= 2 * resident ? 1024 : 512;
