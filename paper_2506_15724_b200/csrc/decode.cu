@@ -11,6 +11,7 @@
 //            thread-block cluster per segment that merges through distributed shared memory left too few blocks
 //            resident: 248 us instead of 148 on 1024 segments of 1638 rows.)
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -254,8 +255,11 @@ __device__ __forceinline__ void finish_segment(const DecodeParams& p, const floa
 // four warps work on whole stages: 32 KB are on the wire per block whatever the compiler does with the loop (with 16-byte
 // loads to registers the kernel took 139 or 241 us on 1024 segments of 1638 rows depending on the code around them; this
 // one takes 135, merge included: 0.98 of the measured copy bandwidth. 12 segments of 53038 rows: 118 -> 72 us).
-constexpr int kRingStages = 2;      // a small ring keeps seven blocks resident per SM, so that a block's start and end are
-                                    // covered by the others (four stages: 163 us instead of 135)
+// Stages: two keep seven blocks resident per SM, so that a block's start and end are covered by the others (four stages: 163 us
+// instead of 135); in a call of at most two blocks per SM six hold most of a share (8 segments of 3020 fp32 rows, us with 2 / 3
+// / 4 / 6 stages: g = 1 14.1 / 13.6 / 13.6 / 13.5, g = 4 23.0 / 20.6 / 22.9 / 20.4; 4 of 11329 bf16 rows 15.9 / 15.6 / 15.8 / 15.2).
+// (The tensor-core kernel gains nothing by deeper buffers, 10.5 -> 10.9 us for 8 segments of 2952 rows, g = 4: with them the next
+// call's blocks find no room beside these.)
 constexpr int kStageBytes = 16384;  // K, then V
 constexpr long long kCopyWait = 4000000000ll;  // ~2 s: bound of a wait for a copy
 
@@ -293,7 +297,7 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                : "memory");
 }
 
-template <typename T, int D, int G>
+template <typename T, int D, int G, int kRingStages>
 __global__ void __launch_bounds__(NT) decode_kernel(const __grid_constant__ DecodeParams p) {
   constexpr int EPL = Vec16<T>::N;          // elements per lane
   constexpr int LPR = D / EPL;              // lanes per row
@@ -769,13 +773,20 @@ int run(DecodeParams p, const madakv_config& c, int splits, cudaStream_t st) {
       return launch_status();
     }
   }
-  auto go = [&](auto kernel) {
-    launch_pdl(kernel, grid, dim3(NT), kRingStages * kStageBytes, st, p);
+  auto go = [&](auto heads) {
+    constexpr int G = decltype(heads)::value;
+    if (p.n_sel * p.slots <= 2 * 148) {
+      auto kernel = decode_kernel<T, D, G, 6>;
+      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 6 * kStageBytes) != cudaSuccess) return (int)MADAKV_ECUDA;
+      launch_pdl(kernel, grid, dim3(NT), 6 * kStageBytes, st, p);
+    } else {
+      launch_pdl(decode_kernel<T, D, G, 2>, grid, dim3(NT), 2 * kStageBytes, st, p);
+    }
     return launch_status();
   };
-  if (p.g == 1) return go(decode_kernel<T, D, 1>);
-  if (p.g == 2) return go(decode_kernel<T, D, 2>);
-  if constexpr (sizeof(T) == 4) return p.g <= 4 ? go(decode_kernel<T, D, 4>) : go(decode_kernel<T, D, 8>);
+  if (p.g == 1) return go(std::integral_constant<int, 1>());
+  if (p.g == 2) return go(std::integral_constant<int, 2>());
+  if constexpr (sizeof(T) == 4) return p.g <= 4 ? go(std::integral_constant<int, 4>()) : go(std::integral_constant<int, 8>());
   return MADAKV_EUNSUPPORTED;
 }
 
