@@ -310,11 +310,14 @@ def run_reference(args, wl):
 
 # ----------------------------------------------------------------------------------------------- the CUDA arm
 def launches_per_step(wl):
-    """Kernels of this library launched by one step: score 1 (bf16 with g * w <= 64: one tensor-core kernel) or 3
-    (bf16 with g * w <= 256: pass 1, merge, pass 2; otherwise the three fp32 kernels), allocate 2, select 2,
-    compact 1, decode 2 (partial with the append of Eq. 4 inside, merge)."""
-    one_kernel = wl.dtype == "bf16" and wl.g * wl.w <= 64
-    return (1 if one_kernel else 3) + 2 + 2 + 1 + 2
+    """Kernels of this library launched by one step: score 1 (bf16 with g * w <= 64: the cluster kernel) or 3 (pass 1,
+    merge, pass 2; one more, which splits the operands, in fp32 calls of less than 148 tiles of 128 keys), allocate 1
+    below 148 units, else 2, select the same (a batch always 2), compact 1, decode 1."""
+    score = 1 if wl.dtype == "bf16" and wl.g * wl.w <= 64 else 3
+    if wl.dtype == "f32" and wl.units * ((wl.n + 127) // 128) < 148:
+        score += 1
+    few = wl.units < 148
+    return score + (1 if few else 2) + (1 if few and wl.B == 1 else 2) + 1 + 1
 
 
 class Bench:

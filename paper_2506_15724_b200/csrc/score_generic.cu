@@ -314,8 +314,8 @@ int launch_score_generic(const madakv_config& c, const void* q, madakv_strides s
   return c.head_dim == 64 ? run<__nv_bfloat16, 64>(p, units, st) : run<__nv_bfloat16, 128>(p, units, st);
 }
 
-// Single-pass scoring (Eq. 7) with the softmax normalisers supplied: tensor-core kernel for bf16 with g * w <= 256,
-// the fp32 psi kernel otherwise.
+// Single-pass scoring (Eq. 7) with the softmax normalisers supplied: the tensor-core kernel, or the fp32 psi kernel where it is
+// asked for or a tensor map cannot describe the operands.
 int launch_score_lse(const madakv_config& c, const void* q, madakv_strides sq, const void* k, madakv_strides sk,
                      const int32_t* seq_len, const float* lse, float* psi, void* ws, cudaStream_t st) {
   if (tc_device_ok()) {  // false also when MADAKV_SCORE_PATH asks for the fp32 kernels
