@@ -64,13 +64,18 @@ inline int wide_max_runs(int units_per_seq, int n_max) {
 // first / on loading: 16 tiles 18.0 / 21.5 with head_dim 64, 20.9 / 27.3 with 128; 64: 20.3 / 21.1, 24.0 / 27.3; 148: 23.6 / 23.3,
 // 29.3 / 30.2; 296: 28.7 / 26.4, 38.8 / 34.4), and so does the single pass over K (16 tiles 10.5 / 8.6, 296 22.4 / 12.3).
 constexpr int kSplitTiles = 148;
-inline bool split_first(const madakv_config& c) {
-  return c.dtype == MADAKV_F32 &&
-         (long long)c.batch * c.n_layers * c.n_kv_heads * ((c.max_seq_len + 127) / 128) < kSplitTiles;
+constexpr size_t kSplitBytes = 96u << 20;
+inline size_t split_unit_bytes(const madakv_config& c) {
+  return ((size_t)c.max_seq_len + (size_t)(c.n_q_heads / c.n_kv_heads) * c.window) * c.head_dim * 6;
 }
-inline size_t split_bytes(const madakv_config& c) {
-  return (size_t)c.batch * c.n_layers * c.n_kv_heads *
-         ((size_t)c.max_seq_len + (size_t)(c.n_q_heads / c.n_kv_heads) * c.window) * c.head_dim * 6;
+// The most units that such a call may have. The workspace of any fp32 config holds that many (or all of its own), so that it
+// serves calls on one of its layers too.
+inline size_t split_units_max(const madakv_config& c) {
+  const size_t tiles = ((size_t)c.max_seq_len + 127) / 128, by_tiles = (kSplitTiles - 1) / tiles, by_bytes = kSplitBytes / split_unit_bytes(c);
+  return by_tiles < by_bytes ? by_tiles : by_bytes;
+}
+inline bool split_first(const madakv_config& c) {
+  return c.dtype == MADAKV_F32 && (size_t)c.batch * c.n_layers * c.n_kv_heads <= split_units_max(c);
 }
 
 inline WsLayout ws_layout(const madakv_config& c) {
@@ -102,7 +107,7 @@ inline WsLayout ws_layout(const madakv_config& c) {
   part = wide > part ? wide : part;
   off = align_up(off + part, 256);
   w.score_split_off = off;
-  if (split_first(c)) off = align_up(off + split_bytes(c), 256);
+  if (c.dtype == MADAKV_F32) off = align_up(off + (units < split_units_max(c) ? units : split_units_max(c)) * split_unit_bytes(c), 256);
   w.decode_off = off;
   off = align_up(off + (size_t)c.batch * c.n_layers * c.n_q_heads * (size_t)w.decode_splits * (c.head_dim + 2) *
                            sizeof(float), 256);

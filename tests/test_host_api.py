@@ -113,3 +113,12 @@ def test_entry_points_reject_bad_arguments_before_launch(lib):
     assert lib.madakv_compact(ctypes.byref(b), FAKE, FAKE, good, FAKE, FAKE, FAKE, FAKE, FAKE, 10, FAKE, need,
                               None) == mk.EUNSUPPORTED
     assert lib.madakv_poll_status(None, None, None) == mk.EINVAL
+
+
+@pytest.mark.parametrize("dtype", [mk.MADAKV_F32, mk.MADAKV_BF16])
+@pytest.mark.parametrize("n,w,Hq", [(1, 1, 2), (77, 9, 8), (1719, 8, 8), (20000, 64, 4), (128, 1024, 8)])
+def test_workspace_of_a_config_serves_its_layers(dtype, n, w, Hq):
+    """A layer-by-layer pass uses the whole config's workspace with configs of fewer layers (or sequences)."""
+    sizes = [mk.madakv_workspace_bytes(mk.make_config(dtype, B, L, Hq, 2, 128, n, w))
+             for B, L in ((1, 1), (1, 2), (2, 5), (3, 32), (8, 64))]
+    assert sizes == sorted(sizes)
