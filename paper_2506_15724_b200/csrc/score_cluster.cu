@@ -382,10 +382,13 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
       if constexpr (NPAD == 32) {
         // One sweep as the tiles arrive: every lane takes, per window row, its logit of the group's first tile as the
         // reference and sums exp2(s - reference) over its keys (the reference's own term is 1). No maximum is needed
-        // as long as no later logit lies ~100 binades above the reference. If a sum leaves that range (or a
-        // reference was a masked logit), the warp redoes the unit's statistics exactly; kLong, whose first tiles are gone by
-        // then, looks before it sums (half an instruction per logit) and raises the reference. Afterwards the lanes'
-        // references are replaced by the warp's maximum of them.
+        // as long as no later logit lies ~100 binades above the reference. If a sum leaves that range, the warp redoes the
+        // unit's statistics exactly; kLong, whose first tiles are gone by then, looks before it sums (half an instruction
+        // per logit) and raises the reference. Afterwards the lanes' references are replaced by the warp's maximum of them.
+        // A masked logit, or one of -inf, is no reference: the lane takes one between it and every real logit, against
+        // which its terms are 0. (Against itself it would be off by the rounding of its product with the scale, some 2^69:
+        // exp2 of that is 0 or infinite, as the scale has it.)
+        const float neg_lowest = -0.75f * kEmptyMax * p.scale2;
         uint64_t negm2[NPAD / 2];
 #pragma unroll
         for (int i = 0; i < NPAD / 2; ++i) {
@@ -400,8 +403,8 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
                      if (x == grp) {
 #pragma unroll
                        for (int c = 0; c < 8; ++c)
-                         negm2[j * 8 + c] = pack2(-(__uint_as_float(r[2 * c]) * p.scale2),
-                                                  -(__uint_as_float(r[2 * c + 1]) * p.scale2));
+                         negm2[j * 8 + c] = pack2(fminf(-(__uint_as_float(r[2 * c]) * p.scale2), neg_lowest),
+                                                  fminf(-(__uint_as_float(r[2 * c + 1]) * p.scale2), neg_lowest));
                      }
                      if (kLong && __any_sync(0xffffffffu, block_max_exponent(r, scale2x, negm2 + j * 8) > kMaxExponent)) {
 #pragma unroll

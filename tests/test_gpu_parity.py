@@ -182,6 +182,66 @@ def test_score_longer_than_tensor_memory(B, H, d, n, w, spread):
     assert psi_close(got, want, max(PSI_RTOL_SEEN, 8 * worst * 2.0 ** -24), atol=1e-7) >= 0.0
 
 
+# short sequences beside one that a cluster's TMEM does not hold: CTAs whose first tile (or two) is the last of the sequence, so
+# that lanes begin with keys their rows may not see, at scales for which the product of mask and scale is rounded up and down
+@pytest.mark.parametrize("d,scale", [(64, 0.0), (64, 0.05), (64, 1.0), (128, 0.0), (128, 0.08), (128, 0.25)])
+@pytest.mark.parametrize("causal", [1, 0])
+def test_score_of_short_sequences_beside_long_ones(d, scale, causal):
+    sl = np.array([17003, 100, 2 * 128, 31 * 128 - 5, 32 * 128, 36 * 128 + 1], np.int32)
+    B, H, n, w = len(sl), 7, int(sl[0]), 20
+    wl = synth.scaled(TINY, dtype="bf16", B=B, L=1, Hq=H, Hkv=H, d=d, n=n, w=w, layout="blocks70", budget=n // 5)
+    q = synth.make_q_win(wl)
+    k = synth.hash_normal(3, 5, 0, B * H * n * d).view(B, 1, H, n, d).to(torch.bfloat16)
+    cfg = config_of(wl, causal=causal, softmax_scale=scale)
+    psi = torch.full((B, 1, H, n), -1.0, device="cuda")
+    lse = torch.zeros((B, 1, H, w), device="cuda")
+    ws = mk.new_workspace(cfg)
+    mk.madakv_score(cfg, q.cuda(), k.cuda(), torch.from_numpy(sl).cuda(), lse, psi, ws)
+    assert mk.madakv_poll_status(ws) == 0
+    want, want_lse = oracle.score(1, to_np(q), to_np(k), sl, causal=causal, scale=scale or None, want_lse=True)
+    # a logit's fp32 rounding error, at most d + 1 roundings of values up to the largest one, becomes a relative one of the weight
+    worst = float((q.float() @ k.float().mT).abs().max()) * (scale or d ** -0.5)
+    bound = max(PSI_RTOL_SEEN, 8 * worst * 2.0 ** -24)
+    psi_close(psi.cpu().numpy(), want, bound)
+    np.testing.assert_allclose(lse.cpu().numpy(), want_lse, rtol=0, atol=max(2e-5, bound))
+
+
+# a key whose logit is -inf for every row weighs nothing, wherever it stands: resident logits (32 and 64 rows), a sequence longer
+# than the TMEM, two passes over K, the fp32 forms
+INF_KEYS = {
+    "resident_r32": ("bf16", 1, 3, 3, 128, 2500, 32), "resident_r64": ("bf16", 1, 4, 2, 64, 1500, 32),
+    "longer": ("bf16", 22, 1, 1, 64, 17003, 32), "two_passes": ("bf16", 1, 8, 2, 128, 900, 32),
+}
+
+
+@pytest.mark.parametrize("name", list(INF_KEYS))
+def test_score_with_infinite_keys(name):
+    dtype, L, Hq, Hkv, d, n, w = INF_KEYS[name]
+    wl = synth.scaled(TINY, dtype=dtype, B=1, L=L, Hq=Hq, Hkv=Hkv, d=d, n=n, w=w, layout="blocks70", budget=n // 5)
+    q = synth.make_q_win(wl).float()
+    q[..., 0] = q[..., 0].abs() + 0.01  # (of one sign, else the same key's logit is +inf for another row)
+    q = q.to(wl.torch_dtype)
+    k = synth.hash_normal(3, 5, 0, L * Hkv * n * d).view(1, L, Hkv, n, d)
+    dead = torch.zeros(n, dtype=torch.bool)
+    dead[0:200:3] = dead[n // 2] = dead[n - w - 5] = True
+    k[:, :, :, dead, 0] = -math.inf
+    k = k.to(wl.torch_dtype)
+    sl = np.array([n], np.int32)
+    cfg = config_of(wl)
+    psi = torch.full((1, L, Hkv, n), -1.0, device="cuda")
+    lse = torch.zeros((1, L, Hq, w), device="cuda")
+    ws = mk.new_workspace(cfg)
+    args = q.cuda(), k.cuda(), torch.from_numpy(sl).cuda(), lse, psi, ws
+    want, want_lse = oracle.score(dcode(wl), to_np(q), to_np(k), sl, want_lse=True)
+    assert np.isfinite(want).all() and (want[..., dead.numpy()] == 0).all()
+    mk.madakv_score(cfg, *args)
+    assert psi_close(psi.cpu().numpy(), want, PSI_RTOL) < PSI_RTOL_SEEN
+    np.testing.assert_allclose(lse.cpu().numpy(), want_lse, rtol=0, atol=2e-5)
+    mk.madakv_score_lse(cfg, *args)
+    assert psi_close(psi.cpu().numpy(), want, PSI_RTOL) < PSI_RTOL_SEEN
+    assert mk.madakv_poll_status(ws) == 0
+
+
 @pytest.mark.parametrize("lag", ["8", "9", "40", "1000"])
 def test_tensor_core_score_item_interleaving(lag, monkeypatch):
     # many more work items than the phase-1 lead: exercises the interleaved phase-2 / phase-1 item order and the
