@@ -108,7 +108,8 @@ int madakv_workspace_bytes(const madakv_config* cfg, size_t* bytes_out);
  *   lse     [B, L, H_q, w] fp32, natural-log sum-exp of every window row's scaled logits. The call computes
  *           these values and stores them here when `lse` is non-null (may be null).
  *   psi     [B, L, H_kv, n_max] fp32, contiguous, written in full
- * Deterministic: a fixed reduction order, no floating-point atomics.
+ * Deterministic: a fixed reduction order, no floating-point atomics. A key whose logit is -inf has weight 0 (fp32: where
+ * an infinite element meets finite ones below 2^9 in magnitude; above that the logit may be NaN).
  * The scoring kernels are persistent grids sized to the whole device. No CTA waits for one outside its thread-block
  * cluster, except in a kernel that only the environment variable MADAKV_SCORE_PATH=twophase selects: there, if kernels of
  * another stream keep part of the grid from being scheduled, a bounded wait runs out and the call reports MADAKV_ETIMEOUT

@@ -326,23 +326,21 @@ __device__ __forceinline__ int cta_of(int total, int ctas, int x) {
 }
 
 // Four fp32 values as three bf16 terms each, whose sum is the value exactly (8 significand bits per term): lo goes to `store`,
-// hi (x, y) and mid (z, w) are returned, packed.
+// hi (x, y) and mid (z, w) are returned, packed. The conversion stops at the largest finite number, which is exact for values that
+// would round up to infinity; of an infinity all three terms are that number, so that its products have the sign of an
+// infinity's (and none is infinite that should not be, for partners below 2^9), not NaN.
 template <typename Store>
 __device__ __forceinline__ uint4 split4(float4 v, Store store) {
   auto pack = [](float a, float b) {
-    const __nv_bfloat162 x = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<const uint32_t*>(&x);
+    uint32_t x;
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(x) : "f"(b), "f"(a));
+    return x;
   };
   auto low = [](uint32_t x) { return __uint_as_float(x << 16); };
   auto high = [](uint32_t x) { return __uint_as_float(x & 0xffff0000u); };
   uint4 t;
   t.x = pack(v.x, v.y);
   t.y = pack(v.z, v.w);
-  // (values that would round up to infinity are cut off instead)
-  if (max3f(fabsf(v.x), fabsf(v.y), fmaxf(fabsf(v.z), fabsf(v.w))) >= __uint_as_float(0x7f7f8000u)) {
-    t.x = (__float_as_uint(v.x) >> 16) | (__float_as_uint(v.y) & 0xffff0000u);
-    t.y = (__float_as_uint(v.z) >> 16) | (__float_as_uint(v.w) & 0xffff0000u);
-  }
   v.x = __fsub_rn(v.x, low(t.x));
   v.y = __fsub_rn(v.y, high(t.x));
   v.z = __fsub_rn(v.z, low(t.y));

@@ -211,6 +211,7 @@ def test_score_of_short_sequences_beside_long_ones(d, scale, causal):
 INF_KEYS = {
     "resident_r32": ("bf16", 1, 3, 3, 128, 2500, 32), "resident_r64": ("bf16", 1, 4, 2, 64, 1500, 32),
     "longer": ("bf16", 22, 1, 1, 64, 17003, 32), "two_passes": ("bf16", 1, 8, 2, 128, 900, 32),
+    "f32_split_before": ("f32", 1, 2, 1, 128, 700, 16), "f32_split_on_loading": ("f32", 30, 2, 1, 64, 700, 16),
 }
 
 
@@ -240,6 +241,28 @@ def test_score_with_infinite_keys(name):
     mk.madakv_score_lse(cfg, *args)
     assert psi_close(psi.cpu().numpy(), want, PSI_RTOL) < PSI_RTOL_SEEN
     assert mk.madakv_poll_status(ws) == 0
+
+
+# the largest fp32 keys (most of them round up to infinity as bf16) keep all their bits: one column of powers of two brings the logits
+# to +-16
+@pytest.mark.parametrize("L", [1, 40])
+def test_score_with_the_largest_finite_keys(L):
+    n, w, d = 600, 8, 64
+    cfg = mk.make_config(torch.float32, 1, L, 1, 1, d, n, w)
+    k = synth.hash_normal(3, 5, 0, L * n * d).view(1, L, 1, n, d).contiguous()
+    bits = torch.arange(L * n, dtype=torch.int32).mul(3).remainder(40000).neg().add(0x7F7FFFFF).view(1, L, 1, n)
+    k[..., 0] = bits.view(torch.float32) * (1 - 2 * (torch.arange(n) % 7 == 3).float())
+    q = torch.zeros((1, L, 1, w, d))
+    q[..., 0] = 2.0 ** -121
+    sl = np.array([n], np.int32)
+    psi = torch.full((1, L, 1, n), -1.0, device="cuda")
+    lse = torch.zeros((1, L, 1, w), device="cuda")
+    ws = mk.new_workspace(cfg)
+    mk.madakv_score(cfg, q.cuda(), k.cuda(), torch.from_numpy(sl).cuda(), lse, psi, ws)
+    assert mk.madakv_poll_status(ws) == 0
+    want, want_lse = oracle.score(0, to_np(q), to_np(k), sl, want_lse=True)
+    assert psi_close(psi.cpu().numpy(), want, PSI_RTOL) < PSI_RTOL_SEEN
+    np.testing.assert_allclose(lse.cpu().numpy(), want_lse, rtol=0, atol=2e-5)
 
 
 @pytest.mark.parametrize("lag", ["8", "9", "40", "1000"])
