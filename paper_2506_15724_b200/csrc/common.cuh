@@ -21,7 +21,7 @@ namespace madakv {
 //                            proxy tokens per sequence [B] int32
 //   [.., .. + score)         stage 1 scratch: finished-item counters [units * rows] int32, log2-domain row
 //                            log-sum-exp [units * rows] fp32 (rows = g * w padded to a multiple of 32), per-chunk
-//                            partial (max, sum) pairs (see ws_layout)
+//                            partial (max, sum) pairs, the bf16 terms of small fp32 calls (see ws_layout)
 //   [.., .. + decode)        stage 5 scratch: split partials [B * L * H_q * splits * (d + 2)] fp32
 // Stages 2-3 keep their scratch in shared memory.
 // ---------------------------------------------------------------------------------------------------------------
@@ -68,14 +68,24 @@ constexpr size_t kSplitBytes = 96u << 20;
 inline size_t split_unit_bytes(const madakv_config& c) {
   return ((size_t)c.max_seq_len + (size_t)(c.n_q_heads / c.n_kv_heads) * c.window) * c.head_dim * 6;
 }
-// The most units that such a call may have. The workspace of any fp32 config holds that many (or all of its own), so that it
-// serves calls on one of its layers too.
+// The most units that such a call may have.
 inline size_t split_units_max(const madakv_config& c) {
   const size_t tiles = ((size_t)c.max_seq_len + 127) / 128, by_tiles = (kSplitTiles - 1) / tiles, by_bytes = kSplitBytes / split_unit_bytes(c);
   return by_tiles < by_bytes ? by_tiles : by_bytes;
 }
 inline bool split_first(const madakv_config& c) {
   return c.dtype == MADAKV_F32 && (size_t)c.batch * c.n_layers * c.n_kv_heads <= split_units_max(c);
+}
+// Room for the terms of such a call, on this config or on one of fewer layers, sequences or tokens: x units of up to t tiles, x * t
+// below kSplitTiles, have no more keys than the config nor than kSplitTiles - 1 tiles hold. (What the config's own calls need is less
+// for long prompts than for short ones; a workspace for the longest prompt serves the shorter ones.)
+inline size_t split_area_bytes(const madakv_config& c) {
+  if (c.dtype != MADAKV_F32) return 0;
+  const size_t most = kSplitTiles - 1, units = (size_t)c.batch * c.n_layers * c.n_kv_heads;
+  const size_t keys = units * c.max_seq_len < most * 128 ? units * c.max_seq_len : most * 128;
+  const size_t rows = (units < most ? units : most) * (c.n_q_heads / c.n_kv_heads) * c.window;
+  const size_t bytes = (keys + rows) * c.head_dim * 6;
+  return bytes < kSplitBytes ? bytes : kSplitBytes;
 }
 
 inline WsLayout ws_layout(const madakv_config& c) {
@@ -107,7 +117,7 @@ inline WsLayout ws_layout(const madakv_config& c) {
   part = wide > part ? wide : part;
   off = align_up(off + part, 256);
   w.score_split_off = off;
-  if (c.dtype == MADAKV_F32) off = align_up(off + (units < split_units_max(c) ? units : split_units_max(c)) * split_unit_bytes(c), 256);
+  off = align_up(off + split_area_bytes(c), 256);
   w.decode_off = off;
   off = align_up(off + (size_t)c.batch * c.n_layers * c.n_q_heads * (size_t)w.decode_splits * (c.head_dim + 2) *
                            sizeof(float), 256);

@@ -122,3 +122,11 @@ def test_workspace_of_a_config_serves_its_layers(dtype, n, w, Hq):
     sizes = [mk.madakv_workspace_bytes(mk.make_config(dtype, B, L, Hq, 2, 128, n, w))
              for B, L in ((1, 1), (1, 2), (2, 5), (3, 32), (8, 64))]
     assert sizes == sorted(sizes)
+
+
+@pytest.mark.parametrize("dtype", [mk.MADAKV_F32, mk.MADAKV_BF16])
+@pytest.mark.parametrize("L,Hq,w,d", [(1, 2, 1, 64), (1, 8, 256, 128), (18, 14, 32, 128), (73, 2, 8, 64), (28, 16, 512, 128)])
+def test_workspace_of_the_longest_prompt_serves_shorter_ones(dtype, L, Hq, w, d):
+    sizes = [mk.madakv_workspace_bytes(mk.make_config(dtype, 1, L, Hq, 2, d, n, w))
+             for n in (1, 77, 128, 129, 500, 1000, 2048, 5000, 9408, 18816, 18817, 20000, 131072, 1 << 20)]
+    assert sizes == sorted(sizes)
