@@ -91,9 +91,10 @@ typedef struct madakv_strides {
 } madakv_strides;
 
 /* Bytes of caller-provided scratch every other call expects in `ws` (a device buffer, 256-byte aligned).
- * The first 256 bytes hold the device status word and counters; the caller zeroes the buffer once after
- * allocating it (cudaMemsetAsync) and may then reuse it across calls on one stream. Two calls that run
- * concurrently on different streams need separate workspaces.                                             */
+ * The first 256 bytes hold the device status word, the 64 KB behind them counters that are zero between calls; the
+ * caller zeroes the buffer once after allocating it (cudaMemsetAsync) and may then reuse it across calls on one
+ * stream. Two calls that run concurrently on different streams need separate workspaces: with a shared one they spoil
+ * each other's results, and may leave counters behind that spoil later calls until the buffer is zeroed again.   */
 int madakv_workspace_bytes(const madakv_config* cfg, size_t* bytes_out);
 
 /* Stage 1 (Eq. 7 with the softmax of Eq. 5). For unit (b,l,h) and key i < seq_len[b]:
@@ -222,9 +223,10 @@ int madakv_decode_attn(const madakv_config* cfg, int32_t layer, const void* q, c
  *     MADAKV_STATIC_SCRATCH_BYTES; a larger problem returns MADAKV_ESTATIC before anything is launched.
  *   - The first call on each device looks up the device address of the built-in array (a host-side query, no
  *     allocation) with that device current; make that first call outside any stream capture.
- *   - All calls on one device share the one array. Nothing in it has to start at zero (every partial that is read
- *     was written earlier in the same call), but two calls whose kernels overlap on the GPU (different streams, or
- *     different host threads) race on it: serialise them.                                                  */
+ *   - All calls on one device share the one array: two calls whose work overlaps on the GPU (different streams, or
+ *     different host threads) race on it and spoil each other's results, so serialise them. Calls after them are not
+ *     affected: every partial that is read was written earlier in the same call, and the counters that a call uses
+ *     are cleared on `stream` before its kernel.                                                            */
 #define MADAKV_STATIC_SCRATCH_BYTES (16u << 20)
 int madakv_decode_attn_static(const madakv_config* cfg, int32_t layer, const void* q, const void* k_c, const void* v_c,
                               const int64_t* seg_off, const int32_t* kept_len, int64_t capacity, void* out,

@@ -37,7 +37,7 @@ struct DecodeParams {
   float* lse_out;
   float* part;        // slots > 1: [B*L*Hq, slots, D] partial outputs, then [B*L*Hq, slots, 2] their (max, sum)
   float2* part_ml;
-  unsigned* counter;  // slots > 1: one per segment of the call, zero between calls
+  unsigned* counter;  // slots > 1: one per segment of the call, zero when it begins and when it ends
   void* ws;
   int L, Hq, Hkv, g, layer, slots, n_sel, min_rows;
   float scale2;
@@ -763,6 +763,8 @@ int run(DecodeParams p, const madakv_config& c, int splits, cudaStream_t st) {
   p.slots = s.slots;
   p.min_rows = s.min_rows;
   p.part_ml = reinterpret_cast<float2*>(p.part + (int64_t)c.batch * c.n_layers * c.n_q_heads * s.slots * D);
+  // Counters that no caller can reach are cleared by every call: two calls that overlapped may leave them anywhere.
+  if (!p.ws && p.slots > 1 && cudaMemsetAsync(p.counter, 0, (size_t)p.n_sel * sizeof(unsigned), st) != cudaSuccess) return MADAKV_ECUDA;
   const dim3 grid((unsigned)p.n_sel * p.slots);  // one dimension: no 65535 limit on the number of segments
   if constexpr (sizeof(T) == 2) {
     if (mma) {
@@ -830,7 +832,7 @@ int launch_decode(const madakv_config& c, int layer, const void* q, const void* 
 // ---------------------------------------------------------------------------------------------------------------
 
 // Split partials of the no-allocation entry point. One copy per GPU that loads the library, shared by all calls. The segment
-// counters of a split call lie behind them; they start at zero and every call leaves them at zero.
+// counters of a split call lie behind them; every call clears those it uses (see run()).
 struct StaticScratch {
   unsigned char part[MADAKV_STATIC_SCRATCH_BYTES];
   unsigned counter[madakv::kCounters];

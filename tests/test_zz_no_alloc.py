@@ -46,6 +46,35 @@ def test_static_scratch_decode_matches_workspace_decode(name):
         assert float(want.float().abs().max()) > 0
 
 
+def test_calls_that_overlapped_spoil_no_later_call():
+    # against the rule, calls of different splits on two streams: their own results are undefined, those of calls after them are not
+    wl = synth.scaled(TINY, dtype="bf16", B=1, L=8, Hq=4, Hkv=4, d=128, n=4096, w=16)
+    cfg = config_of(wl)
+    rows = [4000, 900]
+    calls = []
+    for r in rows:
+        k, v = (synth.hash_normal(2, t, 0, wl.units * r * wl.d).view(-1, wl.d).bfloat16().cuda() for t in (1, 2))
+        off = (torch.arange(wl.units + 1) * r).cuda()
+        calls.append((k, v, off, torch.full((wl.units,), r, dtype=torch.int32).cuda()))
+    q = synth.make_decode_step(wl, 0)[0].cuda()
+    ws = mk.new_workspace(cfg)
+    out = torch.zeros((1, wl.L, wl.Hq, wl.d), dtype=torch.bfloat16, device="cuda")
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    scrap = [torch.zeros_like(out), torch.zeros_like(out)]
+    for _ in range(20):
+        for st, call, o in zip(streams, calls, scrap):
+            with torch.cuda.stream(st):
+                mk.madakv_decode_attn_static(cfg, -1, q, *call, o, None)
+    torch.cuda.synchronize()
+    for call in calls:
+        want, got = torch.zeros_like(out), torch.zeros_like(out)
+        mk.madakv_decode_attn(cfg, -1, q, None, None, *call, want, None, ws)
+        mk.madakv_decode_attn_static(cfg, -1, q, *call, got, None)
+        torch.cuda.synchronize()
+        assert torch.equal(got, want) and float(want.float().abs().max()) > 0
+
+
 def test_static_scratch_limit_is_reported():
     # 64 layers * 64 query heads * 33 splits * 130 floats * 4 B > 16 MiB: refused on the host, nothing is launched
     wl = synth.scaled(TINY, dtype="bf16", L=64, Hq=64, Hkv=64, d=128, n=8192)
