@@ -255,7 +255,7 @@ __device__ __forceinline__ void finish_segment(const DecodeParams& p, const floa
 // four warps work on whole stages: 32 KB are on the wire per block whatever the compiler does with the loop (with 16-byte
 // loads to registers the kernel took 139 or 241 us on 1024 segments of 1638 rows depending on the code around them; this
 // one takes 135, merge included: 0.98 of the measured copy bandwidth. 12 segments of 53038 rows: 118 -> 72 us).
-// Stages: two keep seven blocks resident per SM, so that a block's start and end are covered by the others (four stages: 163 us
+// Stages: two keep six blocks resident per SM, so that a block's start and end are covered by the others (four stages: 163 us
 // instead of 135); in a call of at most two blocks per SM six hold most of a share (8 segments of 3020 fp32 rows, us with 2 / 3
 // / 4 / 6 stages: g = 1 14.1 / 13.6 / 13.6 / 13.5, g = 4 23.0 / 20.6 / 22.9 / 20.4; 4 of 11329 bf16 rows 15.9 / 15.6 / 15.8 / 15.2).
 // (The tensor-core kernel gains nothing by deeper buffers, 10.5 -> 10.9 us for 8 segments of 2952 rows, g = 4: with them the next
@@ -727,11 +727,15 @@ __global__ void __launch_bounds__(kMmaWarps * 32, 3) decode_mma_kernel(const __g
 //   fewer than 64 segments (one layer of a model): bound by the latency of the blocks, so shares of at least 128 rows
 //     (tensor-core kernel, two iterations of its warps; 256 where that would be more than a block per SM, because every
 //     block more makes the merge longer: 4 segments of 771 rows, g = 7, 9.7 us at 128, 10.8 at 256; 8 of 1777 8.6 and
-//     9.0; 8 of 2952 11.9 and 10.9; 20 of 2000 15.8 and 15.5), as many blocks as are resident at once, at most 32 (16 segments of 8725 rows, g = 4: 46 us with 16 blocks each, 56 with
-//     32, which no longer fit; 12 of 53038, g = 1: 72 with 32, 111 with 16)
-//   more: shares of 1024 rows where that gives two full waves of blocks, else 512 (896 segments of 2512 rows, g = 7:
+//     9.0; 8 of 2952 11.9 and 10.9; 20 of 2000 15.8 and 15.5), as many blocks as are resident at once, at most 32 (16
+//     segments of 8725 rows, g = 4: 46 us with 16 blocks each, 56 with 32, which no longer fit; 12 of 53038, g = 1: 72 with
+//     32, 111 with 16). Resident per SM: six of the scalar kernel by their shared memory, but three for fp32 with g > 4 (159
+//     registers); three of the tensor-core kernel. (The most that fit against one more per SM: 40 segments of 8000 rows,
+//     g = 1 36 and 40; 60 of 3000 21.2 and 23.3; fp32 40 of 5000, g = 4 52 and 58; with g = 8, three against seven, 20 of 5000
+//     50 and 64)
+//   more: shares of 1024 rows where that gives this many blocks, else 512 (896 segments of 2512 rows, g = 7:
 //     190 us at 1024, 197 at 512, 247 at 256; 10240 of 410, g = 1: 311 with one block each, 335 with two; 1024 of 1638,
-//     g = 1: 137 at 1024, 135 at 512; 112 of 3000, g = 1: 44 at 1024, 38 at 512)
+//     g = 1: 137 at 1024, 135 at 512; 900 of 1500 115 and 111; 640 of 2500 135 and 129; 112 of 3000 44 and 38)
 //   more than there are counters: one block each
 struct DecodeShape {
   int slots, min_rows;
@@ -740,13 +744,13 @@ DecodeShape decode_shape(const madakv_config& c, int n_sel, int64_t capacity, bo
   if (n_sel > kCounters) return {1, 1};
   const int64_t units = (int64_t)c.batch * c.n_layers * c.n_kv_heads, longest = c.max_seq_len + c.max_new_tokens;
   const int64_t rows = capacity / units < longest ? capacity / units : longest;
-  const int resident = 148 * (tensor_core_kernel ? 3 : 7);
+  const int resident = 148 * (tensor_core_kernel || c.n_q_heads / c.n_kv_heads > 4 ? 3 : 6);
   int share, most;
   if (n_sel < 64) {
     share = tensor_core_kernel && n_sel * ((rows + 127) / 128) > 148 ? 256 : 128;
     most = resident / n_sel < kDecodeSlots ? resident / n_sel : kDecodeSlots;
   } else {
-    share = n_sel * (rows / 1024 + 1) >= 2 * resident ? 1024 : 512;
+    share = n_sel * (rows / 1024 + 1) >= 148 * (tensor_core_kernel ? 6 : 14) ? 1024 : 512;
     most = 8;
   }
   const int64_t want = 3 * rows / (2 * share) + 1;  // (segments may be longer than the mean)

@@ -783,7 +783,7 @@ def test_decode_with_more_than_65535_segments():
 @pytest.mark.parametrize("dtype,d,g,units,rows", [
     ("bf16", 128, 1, 1, 6000), ("bf16", 64, 2, 9, 513), ("bf16", 128, 5, 3, 4100), ("bf16", 64, 16, 20, 257),
     ("bf16", 128, 1, 70, 1500), ("bf16", 128, 3, 70, 1025), ("bf16", 128, 2, 1100, 63), ("f32", 128, 1, 5, 1000),
-    ("f32", 64, 3, 66, 700), ("f32", 128, 7, 2, 300), ("f32", 64, 8, 64, 33)])
+    ("f32", 64, 3, 66, 700), ("f32", 128, 7, 2, 300), ("f32", 64, 8, 64, 33), ("bf16", 128, 1, 40, 2900), ("f32", 64, 7, 36, 2000)])
 def test_decode_over_blocks_per_segment(dtype, d, g, units, rows):
     """Every way the decode kernels share a segment out, against the oracle: two appending steps in a row on a workspace
     that a call of another shape has used, then a step without append. Tolerances as for the other decode tests."""
