@@ -198,7 +198,8 @@ int madakv_compact(const madakv_config* cfg, const void* k, const void* v, madak
  *                         (a full segment is left unchanged and sets MADAKV_ECAPACITY)              (Eq. 4)
  *   out[b,l,hq,:] = softmax( scale * q[b,l,hq,:] . K_seg^T ) V_seg for the g query heads of the group (Eq. 5)
  *   q, out [B,L,H_q,d] dtype contiguous; k_new, v_new [B,L,H_kv,d] dtype contiguous or both null;
- *   lse_out [B,L,H_q] fp32 or null. An empty segment gives out = 0, lse = -inf.
+ *   lse_out [B,L,H_q] fp32 or null. An empty segment gives out = 0, lse = -inf; a segment whose rows did not arrive within a
+ *   bounded wait (MADAKV_ETIMEOUT) gives NaN in both.
  * Accumulation is fp32; out is rounded to dtype once. With bf16 and 3 <= g <= 16 the products run on the tensor
  * cores and the softmax weights enter the P V product rounded to bf16 (the denominator stays fp32).
  * Supported: g <= 8 for fp32, g <= 16 for bf16; beyond that MADAKV_EUNSUPPORTED.                           */
@@ -219,6 +220,7 @@ int madakv_decode_attn(const madakv_config* cfg, int32_t layer, const void* q, c
  *
  * Arguments are those of madakv_decode_attn without k_new / v_new (no append, kept_len is only read), without the
  * workspace, and with read-only caches. Same layouts, same result bits as madakv_decode_attn on the same inputs.
+ *   - There is no status word: a bounded wait that ran out shows as NaN in the segment's out and lse_out only.
  *   - Limit: B * L * H_q * ceil((n_max + max_new_tokens) / 256) * (d + 2) * 4 bytes must not exceed
  *     MADAKV_STATIC_SCRATCH_BYTES; a larger problem returns MADAKV_ESTATIC before anything is launched.
  *   - The first call on each device looks up the device address of the built-in array (a host-side query, no

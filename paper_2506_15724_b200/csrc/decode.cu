@@ -41,6 +41,8 @@ struct DecodeParams {
   void* ws;
   int L, Hq, Hkv, g, layer, slots, n_sel, min_rows;
   float scale2;
+  int hold_copies;        // test of waits that run out: no row is copied
+  long long wait_clocks;  // bound of a wait for a copy
 };
 
 __device__ __forceinline__ float fast_ex2(float x) {
@@ -147,10 +149,12 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)
 // The weight of a partial with maximum m against the overall maximum M.
 __device__ __forceinline__ float part_weight(float m, float M) { return m == -INFINITY ? 0.f : exp2f(m - M); }
 
+constexpr float kLost = -1.f;  // in the place of a sum of weights: a wait for the rows ran out
 // Four results of one query head: `o` unnormalised, l their sum of weights.
 template <typename T, int D>
 __device__ __forceinline__ void store4(const DecodeParams& p, int64_t row, int c, float4 o, float l) {
-  const float r0 = l > 0.f ? o.x / l : 0.f, r1 = l > 0.f ? o.y / l : 0.f, r2 = l > 0.f ? o.z / l : 0.f, r3 = l > 0.f ? o.w / l : 0.f;
+  const float none = l < 0.f ? NAN : 0.f;
+  const float r0 = l > 0.f ? o.x / l : none, r1 = l > 0.f ? o.y / l : none, r2 = l > 0.f ? o.z / l : none, r3 = l > 0.f ? o.w / l : none;
   if constexpr (sizeof(T) == 4) {
     *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + row * D + c) = make_float4(r0, r1, r2, r3);
   } else {
@@ -160,7 +164,7 @@ __device__ __forceinline__ void store4(const DecodeParams& p, int64_t row, int c
   }
 }
 __device__ __forceinline__ void store_lse(const DecodeParams& p, int64_t row, float M, float l) {
-  if (p.lse_out) p.lse_out[row] = l > 0.f ? (M + log2f(l)) * kLn2 : -INFINITY;
+  if (p.lse_out) p.lse_out[row] = l > 0.f ? (M + log2f(l)) * kLn2 : (l < 0.f ? NAN : -INFINITY);
 }
 
 // The end of a block: its results lie in shared memory (bo [g][D] unnormalised, bm and bl [g], complete behind a barrier of
@@ -225,6 +229,7 @@ __device__ __forceinline__ void finish_segment(const DecodeParams& p, const floa
     if (s < nb) fac[i * kDecodeSlots + s] = f;
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+    if (__any_sync(0xffffffffu, ml[j].y < 0.f)) l = kLost;
     if (s == 0) {
       s_l[i] = l;
       store_lse(p, row0 + i, M, l);
@@ -262,6 +267,7 @@ __device__ __forceinline__ void finish_segment(const DecodeParams& p, const floa
 // call's blocks find no room beside these.)
 constexpr int kStageBytes = 16384;  // K, then V
 constexpr long long kCopyWait = 4000000000ll;  // ~2 s: bound of a wait for a copy
+constexpr long long kLandWait = 2000000ll;     // ~1 ms: what copies in flight get to land once a wait has run out
 
 __device__ __forceinline__ void bar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count));
@@ -281,15 +287,18 @@ __device__ __forceinline__ bool bar_try(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Bounded wait; a wait that runs out is reported (where there is a workspace) and the caller goes on with what is there.
-__device__ __forceinline__ void bar_wait(const DecodeParams& p, uint64_t* bar, uint32_t parity) {
-  if (bar_try(bar, parity)) return;
+// Bounded wait. False if it runs out, here or in another thread of the block; that is reported where there is a workspace.
+__device__ __forceinline__ bool bar_wait(const DecodeParams& p, uint64_t* bar, uint32_t parity, volatile int* gave_up) {
+  if (bar_try(bar, parity)) return true;
   const long long t0 = clock64();
-  while (!bar_try(bar, parity))
-    if (clock64() - t0 > kCopyWait) {
+  while (!bar_try(bar, parity)) {
+    if (*gave_up) return false;
+    if (clock64() - t0 > p.wait_clocks) {
+      *gave_up = 1;
       if (p.ws) set_status(p.ws, MADAKV_ETIMEOUT);
-      return;
     }
+  }
+  return true;
 }
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
@@ -309,8 +318,10 @@ __global__ void __launch_bounds__(NT) decode_kernel(const __grid_constant__ Deco
   static_assert(GROUPS * G * (D + 2) * 4 + G * (D + 2) * 4 <= kRingStages * kStageBytes, "the merge reuses the ring");
   extern __shared__ __align__(128) unsigned char dsmem[];
   __shared__ uint64_t full[kRingStages], empty[kRingStages];
+  __shared__ int gave_up;
 
   if (threadIdx.x == 0) {
+    gave_up = 0;
     for (int i = 0; i < kRingStages; ++i) {
       bar_init(&full[i], 1);
       bar_init(&empty[i], NT / 32);
@@ -348,6 +359,7 @@ __global__ void __launch_bounds__(NT) decode_kernel(const __grid_constant__ Deco
       const uint32_t bytes = (uint32_t)(rows - (fresh ? 1 : 0)) * ROW_BYTES;
       const uint32_t kd = smem_addr(dsmem) + st * kStageBytes, vd = kd + kStageBytes / 2;
       bar_expect(&full[st], (uint32_t)(2 * rows * ROW_BYTES));
+      if (p.hold_copies) return;
       if (bytes) {
         bulk_load(kd, (const char*)p.k_c + (off + r) * ROW_BYTES, bytes, &full[st]);
         bulk_load(vd, (const char*)p.v_c + (off + r) * ROW_BYTES, bytes, &full[st]);
@@ -381,10 +393,11 @@ __global__ void __launch_bounds__(NT) decode_kernel(const __grid_constant__ Deco
 #pragma unroll
       for (int c = 0; c < EPL; ++c) o[i][c] = 0.f;
     }
+    bool ok = true;  // (else the steps go on, on whatever the stages hold: a way out of the loop cost a fifth at G = 8)
     for (int it = 0; it < steps; ++it) {
       const int st = it % kRingStages;
       const uint32_t use = (uint32_t)(it / kRingStages) & 1u;
-      bar_wait(p, &full[st], use);
+      ok &= bar_wait(p, &full[st], use, &gave_up);
       const uint4* ks = reinterpret_cast<const uint4*>(dsmem + st * kStageBytes) + grp * LPR + lane;
       const uint4* vs = ks + kStageBytes / 32;
       const int left = row_end - row_begin - it * ROWS - grp;  // row j of this thread exists while GROUPS * j < left
@@ -443,11 +456,16 @@ __global__ void __launch_bounds__(NT) decode_kernel(const __grid_constant__ Deco
       __syncwarp();
       if (threadIdx.x % 32 == 0) bar_arrive(&empty[st]);
       if (threadIdx.x == 0 && it + kRingStages < steps) {  // refill the stage once all warps are done with it
-        bar_wait(p, &empty[st], use);
-        issue(it + kRingStages);
+        ok &= bar_wait(p, &empty[st], use, &gave_up);
+        if (ok) issue(it + kRingStages);
       }
     }
-    __syncthreads();
+    const bool lost = __syncthreads_or(!ok);
+    if (lost) {  // no copy may land in shared memory that the merge or another block uses
+      const long long t0 = clock64();
+      while (clock64() - t0 < kLandWait) __nanosleep(1000);
+      __syncthreads();
+    }
 #pragma unroll
     for (int i = 0; i < G; ++i) {
       if (lane == 0) {
@@ -475,7 +493,7 @@ __global__ void __launch_bounds__(NT) decode_kernel(const __grid_constant__ Deco
       b_o[i * D + c] = O;
       if (c == 0) {
         b_m[i] = M;
-        b_l[i] = Lsum;
+        b_l[i] = lost ? kLost : Lsum;
       }
     }
     __syncthreads();
@@ -729,7 +747,7 @@ __global__ void __launch_bounds__(kMmaWarps * 32, 3) decode_mma_kernel(const __g
 //     block more makes the merge longer: 4 segments of 771 rows, g = 7, 9.7 us at 128, 10.8 at 256; 8 of 1777 8.6 and
 //     9.0; 8 of 2952 11.9 and 10.9; 20 of 2000 15.8 and 15.5), as many blocks as are resident at once, at most 32 (16
 //     segments of 8725 rows, g = 4: 46 us with 16 blocks each, 56 with 32, which no longer fit; 12 of 53038, g = 1: 72 with
-//     32, 111 with 16). Resident per SM: six of the scalar kernel by their shared memory, but three for fp32 with g > 4 (159
+//     32, 111 with 16). Resident per SM: six of the scalar kernel by their shared memory, but three for fp32 with g > 4 (160
 //     registers); three of the tensor-core kernel. (The most that fit against one more per SM: 40 segments of 8000 rows,
 //     g = 1 36 and 40; 60 of 3000 21.2 and 23.3; fp32 40 of 5000, g = 4 52 and 58; with g = 8, three against seven, 20 of 5000
 //     50 and 64)
@@ -779,6 +797,15 @@ int run(DecodeParams p, const madakv_config& c, int splits, cudaStream_t st) {
       return launch_status();
     }
   }
+  // Failure-path test (no GPU fault involved): MADAKV_TEST_HOLD_COPIES withholds the copies of cache rows, so every wait for
+  // them runs out, after the given number of clock cycles (at least 100 000).
+  if (const char* e = getenv("MADAKV_TEST_HOLD_COPIES")) {
+    const long long v = atoll(e);
+    if (v >= 100000 && v < kCopyWait) {
+      p.hold_copies = 1;
+      p.wait_clocks = v;
+    }
+  }
   auto go = [&](auto heads) {
     constexpr int G = decltype(heads)::value;
     if (p.n_sel * p.slots <= 2 * 148) {
@@ -824,6 +851,8 @@ int launch_decode(const madakv_config& c, int layer, const void* q, const void* 
   p.n_sel = (layer < 0 ? c.batch * c.n_layers : c.batch) * c.n_kv_heads;
   const int splits = wl.decode_splits;
   p.scale2 = scale_of(c) * kLog2e;
+  p.hold_copies = 0;
+  p.wait_clocks = kCopyWait;
   if (c.dtype == MADAKV_F32) return c.head_dim == 64 ? run<float, 64>(p, c, splits, st) : run<float, 128>(p, c, splits, st);
   return c.head_dim == 64 ? run<__nv_bfloat16, 64>(p, c, splits, st) : run<__nv_bfloat16, 128>(p, c, splits, st);
 }
@@ -904,7 +933,7 @@ extern "C" int madakv_decode_attn_static(const madakv_config* cfg, int32_t layer
   p.lse_out = lse_out;
   p.part = reinterpret_cast<float*>(scratch);
   p.counter = counters;
-  p.ws = nullptr;  // only an appending call reports through the workspace
+  p.ws = nullptr;  // no status word: a wait that ran out shows as NaN in the segment's results
   p.L = c.n_layers;
   p.Hq = c.n_q_heads;
   p.Hkv = c.n_kv_heads;
@@ -912,6 +941,8 @@ extern "C" int madakv_decode_attn_static(const madakv_config* cfg, int32_t layer
   p.layer = layer;
   p.n_sel = (layer < 0 ? c.batch * c.n_layers : c.batch) * c.n_kv_heads;
   p.scale2 = scale_of(c) * kLog2e;
+  p.hold_copies = 0;
+  p.wait_clocks = kCopyWait;
   cudaStream_t st = (cudaStream_t)stream;
   if (c.dtype == MADAKV_F32) return c.head_dim == 64 ? run<float, 64>(p, c, splits, st) : run<float, 128>(p, c, splits, st);
   return c.head_dim == 64 ? run<__nv_bfloat16, 64>(p, c, splits, st) : run<__nv_bfloat16, 128>(p, c, splits, st);

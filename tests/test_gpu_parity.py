@@ -850,6 +850,42 @@ def test_bounded_wait_runs_out_and_the_library_recovers(monkeypatch):
     assert psi_close(buf.psi.cpu().numpy(), want, PSI_RTOL) < PSI_RTOL_SEEN
 
 
+@pytest.mark.parametrize("dtype,units,rows", [("bf16", 70, 200), ("bf16", 3, 3000), ("f32", 500, 900)])
+def test_decode_wait_for_rows_runs_out_and_the_library_recovers(dtype, units, rows, monkeypatch):
+    """The scalar decode kernel's waits for its copies of cache rows, with the copies withheld and the bound shortened to ~1 ms:
+    one block per segment, several, and more blocks than fit at once. The call reports MADAKV_ETIMEOUT, the results are NaN
+    (with the built-in scratch too, which has no status word), an empty segment's are not, and the next call on the same
+    scratch is right."""
+    wl = synth.scaled(TINY, dtype=dtype, B=1, L=units, Hq=2, Hkv=1, d=64, n=rows, w=4)
+    cfg = config_of(wl)
+    lens = np.full(units, rows, np.int32)
+    lens[0] = 0
+    seg_off = np.concatenate([[0], np.cumsum(lens.astype(np.int64) + wl.max_new_tokens)])
+    total = int(seg_off[-1])
+    k_c, v_c = (synth.hash_normal(1, t, 0, total * 64).view(total, 64).to(wl.torch_dtype) for t in (91, 92))
+    q = synth.make_decode_step(wl, 0)[0]
+    d_q, d_kc, d_vc, d_len, d_off = q.cuda(), k_c.cuda(), v_c.cuda(), torch.from_numpy(lens).cuda(), torch.from_numpy(seg_off).cuda()
+    out, lse = torch.zeros_like(d_q), torch.zeros((1, units, 2), device="cuda")
+    ws = mk.new_workspace(cfg)
+    regular = lambda: mk.madakv_decode_attn(cfg, -1, d_q, None, None, d_kc, d_vc, d_off, d_len, out, lse, ws)  # noqa: E731
+    static = lambda: mk.madakv_decode_attn_static(cfg, -1, d_q, d_kc, d_vc, d_off, d_len, out, lse)  # noqa: E731
+    monkeypatch.setenv("MADAKV_TEST_HOLD_COPIES", "2000000")
+    for call, status in ((regular, mk.ETIMEOUT), (static, 0)):
+        out.zero_()
+        lse.zero_()
+        call()
+        assert mk.madakv_poll_status(ws) == status
+        assert (out[:, 0] == 0).all() and torch.isneginf(lse[:, 0]).all()
+        assert torch.isnan(out[:, 1:]).all() and torch.isnan(lse[:, 1:]).all()
+    monkeypatch.delenv("MADAKV_TEST_HOLD_COPIES")
+    rc, want, want_lse = oracle.decode(dcode(wl), to_np(q), None, None, to_np(k_c), to_np(v_c), seg_off, lens, Hkv=1)
+    for call in (regular, static):
+        call()
+        assert mk.madakv_poll_status(ws) == 0
+        assert np.abs(out.float().cpu().numpy() - want).max() <= DEC_ATOL[dtype]
+        assert np.abs(lse[:, 1:].cpu().numpy() - want_lse[:, 1:]).max() <= 1e-5 * np.abs(want_lse[:, 1:]).max()
+
+
 def test_strided_kv_layout():
     # K/V stored per layer as [B, H, n, d] inside a larger allocation (token stride > d)
     wl = synth.scaled(TINY, dtype="bf16", L=2, Hq=4, Hkv=2, d=128, n=340, w=8, budget=50)
