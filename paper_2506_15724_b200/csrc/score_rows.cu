@@ -11,7 +11,7 @@
 // shared memory, so that both passes read K as it is (CV). What bounds them is that conversion, 2700-3500 clocks per 64 columns of
 // 128 keys and lately the operands' shared-memory traffic, 3072 + 768 clocks per tile of six products; the exponentials of 128 rows
 // need 1024, so four epilogue warps do. (us with the terms of all keys written to the workspace by a kernel before, in slices of
-// 96 MB -> now: 16 units of 73557 keys at most, 56 rows 1072 -> 329; 1024 of 1263, 64 rows 1064 -> 466; 8 of 82828, 224 rows 964 ->
+// 96 MB -> now, but for the second accumulator of the MMA issuer, which costs the first pass a fifth at head_dim 64: 16 units of 73557 keys at most, 56 rows 1072 -> 329; 1024 of 1263, 64 rows 1064 -> 466; 8 of 82828, 224 rows 964 ->
 // 450; 1280 of 2357, head_dim 64, 64 rows 1236 -> 600. Eight converting warps and eight or four for the epilogue: 379 and 359 on
 // the first. An issuer chosen by elect.sync, which spares a move to a uniform register per operand, took the MMA issue from 5000 to
 // 2900 clocks per tile.)
@@ -82,6 +82,10 @@ struct RowParams {
   int smax;          // runs (CTAs) a unit's tiles can be spread over at most: wide_max_runs()
   int grid;          // CTAs of the two passes (the merge kernel needs the partition)
   float scale2;
+  // 1 / scale2 as the sum of two. In 32 bits it is off by 2.8e-8 for head_dim 128 (64 rows, 20480 keys: 2-norm of the scores' error
+  // 3.6e-7 -> 1.8e-7). bf16 with given log-sum-exps does without the second (0), because the first one's error makes up for a part
+  // of what the accumulation of q.k cuts off the largest logits (3.3e-7, with the second 6.9e-7).
+  float inv, inv_more;
 };
 
 template <int D, int PASS, int NS, bool CV>  // NS: bf16 terms per operand (1, or 3 for fp32); CV: fp32 inputs are split here
@@ -571,7 +575,6 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
       if (PASS == 2) {
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (!ok) break;
-        const float inv = 1.0f / p.scale2;
 #pragma unroll
         for (int i = 0; i < SL::kQRows / 32; ++i) {
           const int r = lane + 32 * i;
@@ -579,10 +582,11 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
           if (p.given_lse) nl[i] = nl[i] > -INFINITY ? -nl[i] * kLog2e : kEmptyMax;
           if (r >= p.R) nl[i] = kEmptyMax;
           if (r < p.n16) {
-            const float v = nl[i] * inv;
-            const float hi = __bfloat162float(__float2bfloat16_rn(v));
-            const float mid = __bfloat162float(__float2bfloat16_rn(v - hi));
-            const float low = __bfloat162float(__float2bfloat16_rn((v - hi) - mid));
+            // (v + more is the quotient to some 40 bits, see RowParams)
+            const float v = nl[i] * p.inv, more = p.inv_more != 0.f ? fmaf(nl[i], p.inv, -v) + nl[i] * p.inv_more : 0.f;
+            const float hi = __bfloat162float(__float2bfloat16_rn(v)), rest = (v - hi) + more;
+            const float mid = __bfloat162float(__float2bfloat16_rn(rest));
+            const float low = __bfloat162float(__float2bfloat16_rn(rest - mid));
             const uint32_t w0 = (__float_as_uint(hi) >> 16) | (__float_as_uint(mid) & 0xffff0000u);
             *reinterpret_cast<uint4*>(shift_s + (buf * 128 + r) * 128 + (r & 7) * 16) = make_uint4(w0, __float_as_uint(low) >> 16, 0u, 0u);
           }
@@ -625,15 +629,22 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
           if (NS == 3) {
             // A stage is one term of 64 columns of the keys, in the order lo, mid, hi of the first 64, then of the others. The
             // accumulation truncates, so the small products come first (lo hi, mid hi, mid mid, hi lo, hi mid) and the 8 or 4
-            // steps of hi hi last, for which the stages of hi are held: the result is as exact as that of a plain bf16
-            // contraction. (hi hi first: log-sum-exps off by 7e-7 instead of 6e-8, relative.)
-            auto product = [&](uint32_t k_lo, int qt, int kb, uint32_t first) {
+            // steps of hi hi last, for which the stages of hi are held; the second half of those goes to an accumulator of its
+            // own, which the epilogue adds. With one accumulator large logits lost more than in the fp32 FMA kernels (8000 keys,
+            // 32 heads, head_dim 128: log-sum-exps off by 7.7e-7 rms and -4.8e-7 on average, scores with given ones by 4.9e-7
+            // in the 2-norm; FMA 5.1e-7, -1.0e-7 and 4.2e-7; now 4.5e-7, -2.9e-7 and 2.1e-7). us with one / two: 32 units of
+            // 8000 keys, head_dim 128 100.9 / 101.2; with given log-sum-exps 80.1 / 80.3; head_dim 64: 16 of 8000 46.2 / 49.2,
+            // 1024 of 2357 472 / 527, given 75.1 / 73.3.
+            const uint32_t d1 = tmem_base + buf * 256, d2 = d1 + 128;
+            auto product = [&](uint32_t k_lo, int qt, int kb, bool first, bool hi_hi) {
 #pragma unroll
               for (int kk = 0; kk < 4; ++kk) {
+                const int step = kb * 4 + kk, half = D / 32;  // of hi hi
                 const uint32_t q_op = q_lo0 + (((qt * kKBlocks + kb) * SL::kQRows * 128 + kk * 32) >> 4);
-                const uint32_t k_op = k_lo + ((kk * 32) >> 4), add = first && kk == 0 ? 0u : 1u;
-                if (PASS == 1) umma_bf16(tmem_base + buf * 256, q_op, k_op, kIdescRows, add);
-                else umma_bf16(tmem_base + buf * 256, k_op, q_op, idesc2, add);
+                const uint32_t k_op = k_lo + ((kk * 32) >> 4), add = (first && kk == 0) || (hi_hi && step == half) ? 0u : 1u;
+                const uint32_t d = hi_hi && step >= half ? d2 : d1;
+                if (PASS == 1) umma_bf16(d, q_op, k_op, kIdescRows, add);
+                else umma_bf16(d, k_op, q_op, idesc2, add);
               }
             };
             uint32_t hi_lo[kKBlocks];
@@ -646,10 +657,10 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
                 tc_fence_after();
                 const uint32_t k_lo = k_lo0 + (uint32_t)stage * (SL::kStageBytes >> 4);
                 if (term == 2) {
-                  product(k_lo, 0, kb, piece == 0);
+                  product(k_lo, 0, kb, piece == 0, false);
                 } else {
-                  product(k_lo, term == 1 ? 0 : 2, kb, 0);
-                  product(k_lo, 1, kb, 0);
+                  product(k_lo, term == 1 ? 0 : 2, kb, false, false);
+                  product(k_lo, 1, kb, false, false);
                 }
                 if (term == 0) {
                   hi_lo[kb] = k_lo;
@@ -666,10 +677,10 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
             if (!ok) break;
 #pragma unroll
             for (int kb = 0; kb < kKBlocks; ++kb) {
-              product(hi_lo[kb], 0, kb, 0);
+              product(hi_lo[kb], 0, kb, false, true);
               umma_commit(&empty[hi_stage[kb]]);
             }
-            if (PASS == 2) umma_bf16(tmem_base + buf * 256, ones_lo, shift_lo, idesc2, 1u);
+            if (PASS == 2) umma_bf16(d2, ones_lo, shift_lo, idesc2, 1u);
           } else {
           const uint32_t k_lo = k_lo0 + (uint32_t)stage * (SL::kStageBytes >> 4);
           ok = mbar_wait(&full[stage], stage_par, abort_flag, p.status, kSiteFull);
@@ -812,7 +823,19 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
             acc[0] = add2(acc[0], exp2_sum16(x));
           }
         };
-        if (plain) {  // all but the tiles at the window
+        if (NS == 3) {  // the two accumulators' sum, block by block (loads of the next block under the work on this one: the
+                        // registers do not suffice, 527 -> 675 us on 1024 units of 2357 keys, head_dim 64)
+#pragma unroll 1
+          for (int j = 0; j < nblk; ++j) {
+            tmem_ld16_issue(taddr + j * 16, ra);
+            tmem_ld16_issue(taddr + 128 + j * 16, rb);
+            tmem_ld_wait16(ra);
+            tmem_ld_tie16(rb);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) ra[i] = __float_as_uint(__uint_as_float(ra[i]) + __uint_as_float(rb[i]));
+            block(ra, j);
+          }
+        } else if (plain) {  // all but the tiles at the window
           if (PASS == 1) {
             if (SL::kShares == 1) stat_tile<8>(taddr, p.scale2, sc2, m, zacc, z_run);
             else if (nblk == 4) stat_tile<4>(taddr, p.scale2, sc2, m, zacc, z_run);
@@ -1076,12 +1099,15 @@ __global__ void __launch_bounds__(256) score_rows_merge_kernel(RowParams p, floa
   Z = 0.f;
 #pragma unroll
   for (int j = 0; j < 8; ++j) Z += s_z[j][lane] * exp2f(s_m[j][lane] - M);
-  const float l2 = Z > 0.f ? M + log2f(Z) : 0.f;
-  nlse2[x] = -l2;
+  // (the sum's exponent apart and the additions in 64 bits: M + log2f(Z) in 32 is off by up to 2^-20)
+  int e = 0;
+  const float f = Z > 0.f ? frexpf(Z, &e) : 1.f;
+  const double l2 = Z > 0.f ? (double)M + (double)e + (double)log2f(f) : 0.0;
+  nlse2[x] = (float)-l2;
   if (lse_out) {
     const int h = u % p.Hkv, bl = u / p.Hkv;
     const int hq = h * p.g + p.h0 + row / p.wc, wr = p.r0 + row % p.wc;
-    lse_out[((int64_t)bl * p.Hq + hq) * p.w + wr] = Z > 0.f ? l2 * 0.6931471805599453f : -INFINITY;
+    lse_out[((int64_t)bl * p.Hq + hq) * p.w + wr] = Z > 0.f ? (float)(l2 * 0.6931471805599453) : -INFINITY;
   }
 }
 
@@ -1162,6 +1188,8 @@ int score_rows(const madakv_config& c, const void* q, madakv_strides sq, const v
   p.causal = c.causal;
   p.smax = wide_max_runs(p.lh, c.max_seq_len);
   p.scale2 = scale_of(c) * kLog2e;
+  p.inv = 1.0f / p.scale2;
+  p.inv_more = f32 || !given_lse ? (float)(1.0 / (double)p.scale2 - (double)p.inv) : 0.f;
   p.by_hkv = FastDiv(c.n_kv_heads);
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||

@@ -265,6 +265,33 @@ def test_score_with_the_largest_finite_keys(L):
     np.testing.assert_allclose(lse.cpu().numpy(), want_lse, rtol=0, atol=2e-5)
 
 
+# fp32 against the FMA kernels, bf16 of up to 64 rows in two passes against the two-phase kernel: the faster path's error against
+# 64 bits is no larger (a tenth for the sampling: the errors are those of a few thousand rows and keys)
+@pytest.mark.parametrize("dtype,other,L,Hq,Hkv,d,n,w", [
+    ("f32", "generic", 2, 32, 8, 128, 2000, 16), ("f32", "generic", 8, 16, 16, 64, 1500, 32), ("f32", "generic", 1, 4, 4, 64, 512, 32),
+    ("f32", "generic", 1, 4, 4, 128, 1000, 32), ("bf16", "twophase", 1, 8, 4, 128, 20480, 32), ("bf16", "twophase", 4, 64, 32, 64, 3072, 32)])
+def test_score_is_as_exact_as_the_path_it_replaced(dtype, other, L, Hq, Hkv, d, n, w, monkeypatch):
+    wl = synth.scaled(TINY, dtype=dtype, L=L, Hq=Hq, Hkv=Hkv, d=d, n=n, w=w, budget=n // 5, n_needles=16)
+    inp = synth.make_inputs(wl)
+    cfg = config_of(wl)
+    g = dev(inp)
+    ws = mk.new_workspace(cfg)
+    want, want_lse = oracle.score(dcode(wl), to_np(inp["q_win"]), to_np(inp["k"]), to_np(inp["seq_len"]), want_lse=True)
+    err = {}
+    for path in ("auto", other):
+        if path != "auto":
+            monkeypatch.setenv("MADAKV_SCORE_PATH", path)
+        lse, psi = torch.zeros((1, L, Hq, w), device="cuda"), torch.zeros((1, L, Hkv, n), device="cuda")
+        mk.madakv_score(cfg, g["q_win"], g["k"], g["seq_len"], lse, psi, ws)
+        err[path] = [np.linalg.norm(lse.cpu().numpy() - want_lse), np.linalg.norm(psi.cpu().numpy() - want)]
+        if dtype == "f32":
+            given = torch.from_numpy(want_lse.astype(np.float32)).cuda()
+            mk.madakv_score_lse(cfg, g["q_win"], g["k"], g["seq_len"], given, psi, ws)
+            err[path].append(np.linalg.norm(psi.cpu().numpy() - want))
+    assert mk.madakv_poll_status(ws) == 0
+    assert all(a <= 1.1 * b for a, b in zip(err["auto"], err[other])), err
+
+
 @pytest.mark.parametrize("lag", ["8", "9", "40", "1000"])
 def test_tensor_core_score_item_interleaving(lag, monkeypatch):
     # many more work items than the phase-1 lead: exercises the interleaved phase-2 / phase-1 item order and the
