@@ -19,7 +19,6 @@ struct CompactParams {
   const int32_t* kept_idx;
   const int64_t* seg_off;
   const int32_t* kept_len;
-  const int32_t* seq_len;  // unused (bounds come from n_max); kept for symmetry
   int64_t capacity;
   int64_t stride_b, stride_l, stride_h, stride_t;  // bytes
   int L, Hkv, n_max, row_bytes, headroom;
@@ -97,7 +96,6 @@ int launch_compact(const madakv_config& c, const void* k, const void* v, madakv_
   p.kept_idx = kept_idx;
   p.seg_off = seg_off;
   p.kept_len = kept_len;
-  p.seq_len = nullptr;
   p.capacity = capacity;
   p.stride_b = s.batch * e;
   p.stride_l = s.layer * e;

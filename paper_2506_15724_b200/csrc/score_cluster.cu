@@ -124,6 +124,7 @@ struct ClSmem {
 template <int D, int NPAD, bool kLong>
 __global__ void __launch_bounds__(kClThreads, 1)
 score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_q, ClParams p) {
+  static_assert(!kLong || NPAD == 32, "longer sequences of more rows take two passes");
   using SL = ClSmem<D, NPAD>;
   constexpr int kStages = SL::kStages;
   constexpr int kKBlocks = SL::kKBlocks;
@@ -492,7 +493,6 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_co
         ok = sweep(0, my_tiles, [&](int x) { return wait_tile(x); },
                    [&](int j, uint32_t (&r)[16], int x) {
                      const int key0 = (tile0 + x) * kTileKeys;
-                     if (kLong && j == kBlocks - 1 && x < again) release_tile(x);  // all loads of the tile have completed
                      if (key0 + kTileKeys > all_bound) mask_block16(r, key0 + et, vis_s + j * 16);
                      if (x == grp || __any_sync(0xffffffffu, block_max_exponent(r, scale2x, shift2 + j * 8) > kMaxExponent)) {
                        float mine = kEmptyMax;  // lane c < 16: the warp's maximum of row c
@@ -628,8 +628,7 @@ int run_cluster(const CUtensorMap& mk, const CUtensorMap& mq, const ClParams& p,
   using SL = ClSmem<D, NPAD>;
   const int smem = SL::alloc_bytes(p.C);
   auto kern = score_cluster_kernel<D, NPAD, kLong>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-      (p.C > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
     cudaGetLastError();
     return MADAKV_EUNSUPPORTED;
   }
@@ -745,11 +744,8 @@ int launch_score_cluster(const madakv_config& c, const void* q, madakv_strides s
       !make_map(&mq, q, c.head_dim, c.window, c.n_q_heads, c.n_layers, c.batch, sq, c.window, g))
     return MADAKV_EUNSUPPORTED;
   const int npad = p.R <= 32 ? 32 : 64;
-  if (((c.max_seq_len + kTileKeys - 1) / kTileKeys + C - 1) / C > kTmemCols / npad) {
-    if (c.head_dim == 128)
-      return npad == 32 ? run_cluster<128, 32, true>(mk, mq, p, sms, st) : run_cluster<128, 64, true>(mk, mq, p, sms, st);
-    return npad == 32 ? run_cluster<64, 32, true>(mk, mq, p, sms, st) : run_cluster<64, 64, true>(mk, mq, p, sms, st);
-  }
+  if (((c.max_seq_len + kTileKeys - 1) / kTileKeys + C - 1) / C > kTmemCols / npad)  // (cluster_size_for: up to 32 rows)
+    return c.head_dim == 128 ? run_cluster<128, 32, true>(mk, mq, p, sms, st) : run_cluster<64, 32, true>(mk, mq, p, sms, st);
   if (c.head_dim == 128)
     return npad == 32 ? run_cluster<128, 32, false>(mk, mq, p, sms, st) : run_cluster<128, 64, false>(mk, mq, p, sms, st);
   return npad == 32 ? run_cluster<64, 32, false>(mk, mq, p, sms, st) : run_cluster<64, 64, false>(mk, mq, p, sms, st);

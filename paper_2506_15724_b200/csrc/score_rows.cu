@@ -54,8 +54,9 @@ constexpr int kConvertWarps = 16;  // CV: the last 16 warps
 constexpr int kMaxSeqScan = 1024; // batches up to this size get the exact (ragged-aware) tile partition
 constexpr int kFoldTiles = 16;    // pass 1 moves a row's sum to its second level every this many tiles
 
-// Division of numbers below 2^31 by a number known on the host: a multiplication instead of some forty instructions, of which
-// every warp of a CTA did several before its first tile.
+// Division of numbers below 2^31 by a number known on the host: a multiplication (Granlund and Montgomery, "Division by invariant
+// integers using multiplication", 1994, the multiplier rounded up) instead of some forty instructions, of which every warp of a
+// CTA did several before its first tile.
 struct FastDiv {
   uint32_t d, mul, shift;
   explicit FastDiv(int by = 1) : d((uint32_t)by), shift(0) {
@@ -363,7 +364,7 @@ __device__ __forceinline__ float4 load4(const float* p) {
 }
 
 template <int D, int PASS, int NS, bool CV>
-__global__ void __launch_bounds__((RowSmem<D, PASS, NS, CV>::kThreads), 1)  // 96 registers: warps are allocated four at a time (18 -> 20)
+__global__ void __launch_bounds__((RowSmem<D, PASS, NS, CV>::kThreads), 1)  // 96 registers: warps are allocated four at a time (18 -> 20); CV: 80 (22 -> 24)
 score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_q, RowParams p) {
   using SL = RowSmem<D, PASS, NS, CV>;
   constexpr int kStages = SL::kStages;
@@ -1253,7 +1254,7 @@ int launch_score_rows(const madakv_config& c, const void* q, madakv_strides sq, 
   return score_rows(c, q, sq, k, sk, seq_len, nullptr, lse, psi, ws, st);
 }
 
-// Single-pass scoring with the rows' log-sum-exps supplied by the caller: a conversion kernel, then pass 2 alone.
+// Single-pass scoring with the rows' log-sum-exps supplied by the caller: pass 2 alone.
 int launch_score_lse_rows(const madakv_config& c, const void* q, madakv_strides sq, const void* k, madakv_strides sk,
                           const int32_t* seq_len, const float* lse, float* psi, void* ws, cudaStream_t st) {
   return score_rows(c, q, sq, k, sk, seq_len, lse, nullptr, psi, ws, st);
