@@ -676,13 +676,34 @@ class Bench:
                     "ms_overlapped": None if s2 is None else s2["ms"],
                     "overlapped_is_a_cuda_graph": None if s2 is None else s2["cuda_graph"],
                     "ms_eager_one_stream": None if s1 is None else s1["ms"],
-                    "ratio_to_all_layer_pass": None if s2 is None else s2["ms"] / pass_ms, "launches": wl.L * 7,
+                    "ratio_to_all_layer_pass": None if s2 is None else s2["ms"] / pass_ms,
+                    "launches": wl.L * (5 if wl.B == 1 and wl.Hkv < 148 else 6),  # score, demand, allocate, select 1-2, compact
                     "note": "stages 1-4 layer by layer (madakv_score_lse, madakv_allocate_layer, select and compact "
                             "with one-layer configs). overlapped: eight layers in flight on their own streams (scoring; "
                             "madakv_demand_layer, then madakv_allocate_layer without scores once the layer before "
                             "has passed phi on, selection; compaction), replayed from one CUDA graph; not part of "
                             "the step"}
         return rec
+
+
+def summary_of(rec):
+    """What the JSON line says of a workload beside the headline; the whole record goes to stderr. (With all records the line
+    had 28 000 characters, and a reader that keeps the last few thousand lost it.)"""
+    dec, single, streamed = rec["decode"], rec.get("single_pass_score"), rec.get("streamed_pass")
+    return {"ms_per_step": rec.get("ms_per_step"), "stages_ms": rec["stages_ms"],
+            "roofline": {x: rec["roofline"][x] for x in ("bound", "frac")},
+            "decode_us": dec["us_per_step"], "decode_frac": dec["frac_of_measured_peak_alone"],
+            "single_pass_ms": single and single["ms"], "streamed_ms": streamed and streamed["ms_overlapped"],
+            "sm_mhz": (rec["clocks"] or {}).get("sm_mhz")}
+
+
+def rounded(x):
+    """The same with six significant digits in every number."""
+    if isinstance(x, dict):
+        return {k: rounded(v) for k, v in x.items()}
+    if isinstance(x, list):
+        return [rounded(v) for v in x]
+    return float(f"{x:.6g}") if isinstance(x, float) else x
 
 
 def main():
@@ -830,6 +851,9 @@ def main():
     cpu = None
     if world == 1 and not args.no_cpu_baseline:
         cpu, _ = cpu_oracle_leg(wl)
+    for name, rec in workloads.items():
+        print(json.dumps({"record": name, **rec}), file=sys.stderr)
+    dec = head["decode"]
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -841,14 +865,14 @@ def main():
         "roofline": head["roofline"],
         "stages_ms": head["stages_ms"],
         "eviction_pass": head["eviction_pass"],
-        "decode": head["decode"],
+        "decode": {x: dec[x] for x in dec if not isinstance(dec[x], dict) or x == "us_per_step"},
         "single_pass_score": head.get("single_pass_score"),
         "streamed_pass": head.get("streamed_pass"),
         "cpu_baseline": cpu,
         "exp2_roof_probe": None if exp2_roof is None else exp2_roof[2],
-        "workloads": workloads,
+        "workloads": {name: summary_of(rec) for name, rec in workloads.items() if name != wl.name},
     }
-    print(json.dumps(line))
+    print(json.dumps(rounded(line)))
     if world > 1:
         dist.destroy_process_group()
 

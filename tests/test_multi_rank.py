@@ -91,3 +91,19 @@ def test_two_gloo_ranks_shard_batches_and_reduce():
     for p in procs:
         p.join(timeout=60)
     assert results == {0: "ok", 1: "ok"}, results
+
+
+def test_bench_line_stays_short():
+    """The workloads' part of bench.py's JSON line: a summary of a few hundred characters each, six digits per number."""
+    import json
+
+    import bench
+
+    us = {"compressed": 123.456789012, "full": 1234.56789012}
+    rec = {"ms_per_step": 0.123456789, "stages_ms": {x: 1.0 / 3.0 for x in ("score", "allocate", "select", "compact", "decode")},
+           "roofline": {"bound": "hbm", "frac": 2.0 / 3.0, "peak_kind": "x" * 500}, "clocks": {"sm_mhz": 1965.0, "reasons": ["y" * 500]},
+           "decode": {"us_per_step": us, "frac_of_measured_peak_alone": 0.9876543210, "run_with_append": {"note": "z" * 500}},
+           "single_pass_score": {"ms": 0.32, "note": "n" * 500}, "streamed_pass": None}
+    short = bench.rounded(bench.summary_of(rec))
+    assert len(json.dumps(short)) < 500
+    assert short["decode_us"]["compressed"] == 123.457 and short["streamed_ms"] is None and short["sm_mhz"] == 1965.0
