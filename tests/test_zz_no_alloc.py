@@ -75,6 +75,26 @@ def test_calls_that_overlapped_spoil_no_later_call():
         assert torch.equal(got, want) and float(want.float().abs().max()) > 0
 
 
+def test_static_call_replayed_from_a_cuda_graph():
+    # the clearing of the counters is part of what is captured
+    wl = synth.scaled(TINY, dtype="bf16", B=1, L=2, Hq=8, Hkv=2, d=128, n=2048, w=16)
+    cfg = config_of(wl)
+    k, v = (synth.hash_normal(2, t, 0, wl.units * 2000 * wl.d).view(-1, wl.d).bfloat16().cuda() for t in (1, 2))
+    cache = k, v, (torch.arange(wl.units + 1) * 2000).cuda(), torch.full((wl.units,), 2000, dtype=torch.int32).cuda()
+    qs = [synth.make_decode_step(wl, step)[0].cuda() for step in range(3)]
+    q, got, want = qs[0].clone(), torch.zeros_like(qs[0]), torch.zeros_like(qs[0])
+    mk.madakv_decode_attn_static(cfg, -1, q, *cache, got, None)  # the first call on a device comes before any capture
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        mk.madakv_decode_attn_static(cfg, -1, q, *cache, got, None)
+    for x in qs:
+        q.copy_(x)
+        graph.replay()
+        mk.madakv_decode_attn_static(cfg, -1, x, *cache, want, None)
+        torch.cuda.synchronize()
+        assert torch.equal(got, want) and float(want.float().abs().max()) > 0
+
+
 def test_static_scratch_limit_is_reported():
     # 64 layers * 64 query heads * 33 splits * 130 floats * 4 B > 16 MiB: refused on the host, nothing is launched
     wl = synth.scaled(TINY, dtype="bf16", L=64, Hq=64, Hkv=64, d=128, n=8192)
