@@ -20,7 +20,7 @@ struct AllocParams {
   int32_t* demand;
   double* phi;
   int32_t* budgets;
-  int L, Hkv, n_max, mpa, hcc_mode, keep_window, window;
+  int L, Hkv, n_max, mpa, hcc_mode, keep_window, window, rows;  // rows: window rows per KV head
   u64 theta_fix;  // floor(theta * 2^32)
   unsigned* counter;  // one per sequence, zero between calls: the units that are done; null: masses and demands only
   int depth, layer;   // one layer of a pass over `depth` layers (the arrays hold that layer, L = 1), or layer = -1: all layers
@@ -32,6 +32,7 @@ __device__ __forceinline__ void count_visual(const uint8_t* mask, int n, int* s_
   int c = 0;
   if ((reinterpret_cast<uintptr_t>(mask) & 15) == 0) {  // 16 tokens per load
     const int n16 = n >> 4;
+#pragma unroll 4
     for (int i = threadIdx.x; i < n16; i += blockDim.x) {
       const uint4 v = __ldg(reinterpret_cast<const uint4*>(mask) + i);
       const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
@@ -40,21 +41,15 @@ __device__ __forceinline__ void count_visual(const uint8_t* mask, int n, int* s_
         c += __popc(((w4[k] | (w4[k] >> 1) | (w4[k] >> 2) | (w4[k] >> 3) | (w4[k] >> 4) | (w4[k] >> 5) | (w4[k] >> 6) |
                       (w4[k] >> 7)) & 0x01010101u));
     }
+#pragma unroll 1
     for (int i = (n16 << 4) + threadIdx.x; i < n; i += blockDim.x) c += mask[i] ? 1 : 0;
   } else {
+#pragma unroll 1
     for (int i = threadIdx.x; i < n; i += blockDim.x) c += mask[i] ? 1 : 0;
   }
 #pragma unroll
   for (int off = 16; off >= 1; off >>= 1) c += __shfl_xor_sync(0xffffffffu, c, off);
   if ((threadIdx.x & 31) == 0 && c) atomicAdd(s_nv, c);
-}
-// Eq. 10's sum over the heads of one layer (both modalities), by one warp; every lane returns it.
-__device__ __forceinline__ long long layer_demand(const int32_t* demand_layer, int Hkv) {
-  long long dem = 0;
-  for (int x = threadIdx.x & 31; x < 2 * Hkv; x += 32) dem += (long long)__ldcg(demand_layer + x);
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) dem += __shfl_xor_sync(0xffffffffu, dem, off);
-  return dem;
 }
 // The layer's integer budget Phi^l from phi^l, and phi^{l+1} (Eq. 10-11); l counts from 1, the update exists for l < L.
 __device__ __forceinline__ double rounded_budget(double ph, double lo, double hi) {
@@ -70,8 +65,8 @@ __device__ __forceinline__ double phi_divisor(int Hkv, int L, int l, int hcc_mod
 // place, and one correction by the exact remainder makes it the correctly rounded one (Markstein, "Computation of
 // elementary functions on the IBM RISC System/6000 processor", 1990). Three dependent operations instead of a division in
 // a chain that is one layer after the other (llava: 11.8 us for the 32 layers with divisions).
-__device__ __forceinline__ double next_phi(double ph, long long dem, int Hkv, double div, double rcp, double lo, double hi) {
-  const double K = __dsub_rn((double)dem, __dmul_rn((double)Hkv, ph));  // Eq. 10
+__device__ __forceinline__ double next_phi(double ph, double dem, int Hkv, double div, double rcp, double lo, double hi) {
+  const double K = __dsub_rn(dem, __dmul_rn((double)Hkv, ph));  // Eq. 10
   const double q = __dmul_rn(K, rcp);
   const double quot = __fma_rn(__fma_rn(-q, div, K), rcp, q);
   const double next = div > 0.0 ? __dsub_rn(ph, quot) : ph;  // Eq. 11
@@ -81,18 +76,17 @@ __device__ __forceinline__ double next_phi(double ph, long long dem, int Hkv, do
 // few tokens passed to the other. With `keep_demand` (mode DEMAND, every layer but the last) the head keeps what
 // Eq. 9 asked for instead. lo_v, lo_t: the proxy tokens of each modality when they are retained unconditionally
 // (cfg->keep_window), else 0: budgets are floored at them, the head's total at their sum.
-__device__ __forceinline__ void split_budget(const AllocParams& p, int64_t u, double Phi, int n, int n_v, int n_t,
+__device__ __forceinline__ void split_budget(const AllocParams& p, int64_t u, double pref_v, int2 dem, double Phi, int n, int n_v, int n_t,
                                              int lo_v, int lo_t, bool keep_demand) {
   if (keep_demand) {
-    const int dv = __ldcg(p.demand + u * 2), dt = __ldcg(p.demand + u * 2 + 1);
-    p.budgets[u * 2] = p.mpa ? max(dv, lo_v) : 0;
-    p.budgets[u * 2 + 1] = p.mpa ? max(dt, lo_t) : min(max(dv + dt, lo_v + lo_t), n);
+    p.budgets[u * 2] = p.mpa ? max(dem.x, lo_v) : 0;
+    p.budgets[u * 2 + 1] = p.mpa ? max(dem.y, lo_t) : min(max(dem.x + dem.y, lo_v + lo_t), n);
     return;
   }
   const int P = max((int)Phi, lo_v + lo_t);
   int bv, bt;
   if (p.mpa) {
-    bv = (int)floor(__dadd_rn(__dmul_rn(__ldcg(p.pref + u * 2), Phi), 0.5));  // Eq. 8, rounded half up
+    bv = (int)floor(__dadd_rn(__dmul_rn(pref_v, Phi), 0.5));  // Eq. 8, rounded half up
     bv = min(max(bv, lo_v), P - lo_t);
     bt = P - bv;
     if (bv > n_v) { bt += bv - n_v; bv = n_v; }
@@ -106,63 +100,120 @@ __device__ __forceinline__ void split_budget(const AllocParams& p, int64_t u, do
 }
 
 // What is left once all units of sequence b have their masses and demands, by one block: Eq. 10-11 as a scalar scan over the
-// layers (or one step of it), then Eq. 8 integerised for every (layer, head). n_v: the sequence's visual tokens.
-// s_phi, s_dem: kLayerChunk values each in shared memory.
-constexpr int kLayerChunk = 1024;
-__device__ __noinline__ void sequence_budgets(const AllocParams& p, int b, int n, int n_v, double* s_phi, long long* s_dem) {
+// layers (or one step of it), then Eq. 8 integerised for every (layer, head). n_v: the sequence's visual tokens; ph: phi of the
+// first layer. What bounds it is a chain of latencies, so demands and preferences are read together, before anything else,
+// and the scan finds its operands converted and a layer ahead. (Read where they were used, with the scan's conversions
+// in its chain, 11700 clocks for 2 layers of 4 heads, a whole all-layer call of 32 layers 10.7 us.)
+constexpr int kLayerChunk = 512;
+constexpr int kUnitChunk = 2048;  // units whose demands are summed from shared memory
+constexpr int kBudgetBytes = 4 * (kLayerChunk + 1) * 8 + kUnitChunk * 4;
+__device__ __forceinline__ double first_phi(const AllocParams& p, int b) {
+  return p.layer > 0 ? p.phi[(int64_t)b * p.depth + p.layer] : (double)p.budget[b];
+}
+__device__ __noinline__ void sequence_budgets(const AllocParams& p, int b, int n, int n_v, double ph, double* s_phi) {
   __shared__ int s_wv;
+  double *s_rcp = s_phi + kLayerChunk + 1, *s_div = s_rcp + kLayerChunk + 1, *s_dem = s_div + kLayerChunk + 1;
+  int* s_unit = reinterpret_cast<int*>(s_dem + kLayerChunk + 1);
+  constexpr int U = 2;  // units per thread whose demand and preference stay in registers
+  const int tid = threadIdx.x, nt = blockDim.x;
   const int wlen = p.keep_window ? min(p.window, n) : 0;  // proxy tokens retained unconditionally
-  if (threadIdx.x == 0) s_wv = 0;
-  __syncthreads();
-  if (wlen > 0) {
-    count_visual(p.mask + (int64_t)b * p.n_max + (n - wlen), wlen, &s_wv);
-    __syncthreads();
-  }
-  const int n_t = n - n_v;
-  const int lo_v = p.mpa ? s_wv : 0, lo_t = wlen - lo_v;
   const double lo = n >= 1 ? 1.0 : 0.0, hi = (double)n;
   const int depth = p.depth, first = max(p.layer, 0);  // the layers of the arrays: first .. first + L - 1 of depth
-  double ph = 0.0;
-  for (int l0 = 0; l0 < p.L; l0 += kLayerChunk) {
-    const int ln = min(kLayerChunk, p.L - l0);
-    for (int l = threadIdx.x; l < ln; l += blockDim.x) {
-      const double div = first + l0 + l + 1 < depth ? phi_divisor(p.Hkv, depth, first + l0 + l + 1, p.hcc_mode) : 0.0;
-      s_phi[l] = div > 0.0 ? __drcp_rn(div) : 0.0;
+  const int chunk = min(kLayerChunk, max(1, kUnitChunk / p.Hkv));
+  for (int l0 = 0; l0 < p.L; l0 += chunk) {
+    const int ln = min(chunk, p.L - l0), units = ln * p.Hkv;
+    const int64_t u0 = ((int64_t)b * p.L + l0) * p.Hkv;
+    auto unit_demand = [&](int x) { return __ldcg(reinterpret_cast<const int2*>(p.demand) + u0 + x); };
+    double pref[U];
+    int2 dem[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const int x = tid + j * nt;
+      pref[j] = 0.0;
+      dem[j] = make_int2(0, 0);
+      if (x < units) {
+        pref[j] = __ldcg(p.pref + (u0 + x) * 2);
+        dem[j] = unit_demand(x);
+      }
     }
-    // Eq. 10's sum over heads, one warp per layer (integers: any order gives the same sum)
-    for (int l = threadIdx.x >> 5; l < ln; l += blockDim.x >> 5) {
-      const long long dem = layer_demand(p.demand + ((int64_t)b * p.L + l0 + l) * p.Hkv * 2, p.Hkv);
-      if ((threadIdx.x & 31) == 0) s_dem[l] = dem;
+    if (l0 == 0 && tid == 0) s_wv = 0;
+#pragma unroll 1
+    for (int l = tid; l < ln; l += nt) {
+      const double div = first + l0 + l + 1 < depth ? phi_divisor(p.Hkv, depth, first + l0 + l + 1, p.hcc_mode) : 0.0;
+      s_div[l] = div;
+      s_rcp[l] = div > 0.0 ? __drcp_rn(div) : 0.0;
+    }
+    const bool in_shared = units <= kUnitChunk;
+    if (in_shared) {
+#pragma unroll
+      for (int j = 0; j < U; ++j)
+        if (tid + j * nt < units) s_unit[tid + j * nt] = dem[j].x + dem[j].y;
+#pragma unroll 1
+      for (int x = tid + U * nt; x < units; x += nt) {
+        const int2 d = unit_demand(x);
+        s_unit[x] = d.x + d.y;
+      }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      if (l0 == 0) ph = first == 0 ? (double)p.budget[b] : p.phi[(int64_t)b * depth + first];
+    if (l0 == 0 && wlen > 0) count_visual(p.mask + (int64_t)b * p.n_max + (n - wlen), wlen, &s_wv);
+    // Eq. 10's sum over heads (integers: any order gives the same sum)
+    if (in_shared) {
+#pragma unroll 1
+      for (int l = tid; l < ln; l += nt) {
+        long long sum = 0;
 #pragma unroll 4
+        for (int h = 0; h < p.Hkv; ++h) sum += s_unit[l * p.Hkv + h];
+        s_dem[l] = (double)sum;
+      }
+    } else if (tid < 32) {  // one layer of very many heads
+      long long sum = 0;
+#pragma unroll 1
+      for (int x = tid; x < units; x += 32) {
+        const int2 d = unit_demand(x);
+        sum += (long long)d.x + d.y;
+      }
+#pragma unroll
+      for (int off = 16; off >= 1; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+      if (tid == 0) s_dem[0] = (double)sum;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      double rcp = s_rcp[0], div = s_div[0], dm = s_dem[0];
+#pragma unroll 1
       for (int l = 0; l < ln; ++l) {
-        const double rcp = s_phi[l];
+        const double r1 = s_rcp[l + 1], d1 = s_div[l + 1], m1 = s_dem[l + 1];  // (the last ones are not used)
         s_phi[l] = ph;
-        const int at = first + l0 + l + 1;  // the paper counts layers from 1
-        if (at < depth) ph = next_phi(ph, s_dem[l], p.Hkv, phi_divisor(p.Hkv, depth, at, p.hcc_mode), rcp, lo, hi);
+        if (first + l0 + l + 1 < depth) ph = next_phi(ph, dm, p.Hkv, div, rcp, lo, hi);  // (the paper counts layers from 1)
+        rcp = r1;
+        div = d1;
+        dm = m1;
       }
       if (p.layer >= 0 && first + 1 < depth) p.phi[(int64_t)b * depth + first + 1] = ph;
     }
     __syncthreads();
-    for (int l = threadIdx.x; l < ln; l += blockDim.x)
+    const int n_t = n - n_v;
+    const int lo_v = p.mpa ? s_wv : 0, lo_t = wlen - lo_v;
+#pragma unroll 1
+    for (int l = tid; l < ln; l += nt)
       if (p.layer <= 0) p.phi[(int64_t)b * depth + l0 + l] = s_phi[l];
-    for (int x = threadIdx.x; x < ln * p.Hkv; x += blockDim.x) {
+#pragma unroll 1
+    for (int x = tid; x < units; x += nt) {  // (one copy of the code: it is run once)
+      const bool again = x >= U * nt;
+      const bool second = x >= nt;
+      const double pv = again ? __ldcg(p.pref + (u0 + x) * 2) : second ? pref[1] : pref[0];
+      const int2 d = again ? unit_demand(x) : second ? dem[1] : dem[0];
       const int l = x / p.Hkv;
-      split_budget(p, ((int64_t)b * p.L + l0) * p.Hkv + x, rounded_budget(s_phi[l], lo, hi), n, n_v, n_t, lo_v, lo_t,
+      split_budget(p, u0 + x, pv, d, rounded_budget(s_phi[l], lo, hi), n, n_v, n_t, lo_v, lo_t,
                    p.hcc_mode == MADAKV_HCC_DEMAND && first + l0 + l + 1 < depth);
     }
     __syncthreads();
   }
 }
 
-// The low 32 bits of floor(x * 2^32), plus kLowBias, by fp32 additions, for keys below kSmallKey (512.0): adding 512
+// The low 32 bits of floor(x * 2^32), plus kLowBias, by fp32 additions, for keys below 512.0: adding 512
 // rounded towards zero leaves floor(x * 2^14) in the low bits of the significand, the remainder (exact) added to 2^-9 the
 // other 18 bits; the constants of the first sum are shifted out. (The conversion to a 64-bit integer runs at a small
 // fraction of the rate of additions.)
-constexpr uint32_t kSmallKey = 0x44000000u, kLowBias = 0x3b000000u;
 __device__ __forceinline__ uint32_t low_mass(uint32_t key) {
   const float x = __uint_as_float(key);
   const float t = __fadd_rz(x, 512.0f);
@@ -170,14 +221,15 @@ __device__ __forceinline__ uint32_t low_mass(uint32_t key) {
 }
 
 // The ranges Eq. 9's two thresholds can lie in, with the exact masses before them, the masses to reach and the modalities' own.
+template <int CAP>  // candidates that fit the list
 struct MassRanges {
   RankRange r0, r1;
   u64 above0, above1, need0, need1, W0, W1;
   bool exact;
   uint32_t n_vis;  // visual tokens
-  __device__ __forceinline__ bool listed() const { return r0.in <= kListCap && r1.in <= kListCap; }
-  __device__ __forceinline__ bool crowded0() const { return r0.in > kListCap && r0.span > 0; }
-  __device__ __forceinline__ bool crowded1() const { return r1.in > kListCap && r1.span > 0; }
+  __device__ __forceinline__ bool listed() const { return r0.in <= CAP && r1.in <= CAP; }
+  __device__ __forceinline__ bool crowded0() const { return r0.in > CAP && r0.span > 0; }
+  __device__ __forceinline__ bool crowded1() const { return r1.in > CAP && r1.span > 0; }
 };
 // The mass to reach, Eq. 9: theta_fix * W has 96 bits; the prefix test  prefix * 2^32 >= theta_fix * W  is
 // prefix >= ceil(theta_fix * W / 2^32)
@@ -198,19 +250,19 @@ __device__ __forceinline__ void add_key(uint32_t* at, uint32_t t) {
   atomicAdd(at + 2 * RankShared<TEAM, 2>::kStride, low_mass(kTopKey - t));
 }
 template <int KPT, int TEAM>
-__device__ __forceinline__ void add_first(RankShared<TEAM, 2>& sh, const uint32_t (&t)[KPT], uint32_t vis, uint32_t valid) {
+__device__ __forceinline__ void add_first(RankShared<TEAM, 2>& sh, const BucketMap& map, const uint32_t (&t)[KPT], uint32_t vis, uint32_t valid) {
   constexpr int kStride = RankShared<TEAM, 2>::kStride;
   if (valid == valid_bits<KPT>(KPT, 0)) {
 #pragma unroll
-    for (int j = 0; j < KPT; ++j) add_key<TEAM>(sh.cnt + ((vis >> j) & 1u ? 0 : kStride) + map_bucket(t[j]), t[j]);
+    for (int j = 0; j < KPT; ++j) add_key<TEAM>(sh.cnt + ((vis >> j) & 1u ? 0 : kStride) + map_bucket(map, t[j]), t[j]);
   } else {
 #pragma unroll
     for (int j = 0; j < KPT; ++j)
-      if ((valid >> j) & 1u) add_key<TEAM>(sh.cnt + ((vis >> j) & 1u ? 0 : kStride) + map_bucket(t[j]), t[j]);
+      if ((valid >> j) & 1u) add_key<TEAM>(sh.cnt + ((vis >> j) & 1u ? 0 : kStride) + map_bucket(map, t[j]), t[j]);
   }
 }
 template <int KPT, int TEAM>
-__device__ __forceinline__ void add_again(RankShared<TEAM, 2>& sh, const MassRanges& g, const uint32_t (&t)[KPT], uint32_t vis, int shift0,
+__device__ __forceinline__ void add_again(RankShared<TEAM, 2>& sh, const MassRanges<RankShared<TEAM, 2>::kCap>& g, const uint32_t (&t)[KPT], uint32_t vis, int shift0,
                                           int shift1) {
 #pragma unroll
   for (int j = 0; j < KPT; ++j) {
@@ -220,122 +272,47 @@ __device__ __forceinline__ void add_again(RankShared<TEAM, 2>& sh, const MassRan
   }
 }
 
-// Walk of the buckets: block r of the team adds up its share of the buckets over all blocks, half of the threads per modality;
-// the ranges shrink to the buckets in which the masses are reached (if all sums are exact).
+// Walk of the buckets (of the first layout, `map`, or of one over the ranges): the ranges shrink to the buckets in which the
+// masses are reached (if all sums are exact).
 template <int TEAM>
-__device__ __forceinline__ void mass_walk(RankShared<TEAM, 2>& sh, uint32_t rank, bool first, u64 theta_fix, MassRanges& g, int shift0, int shift1) {
-  using SH = RankShared<TEAM, 2>;
-  constexpr int kPer = SH::kPer;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, m = tid / kHalf, i = tid % kHalf;
-  const uint32_t b0 = (rank * kHalf + i) * kPer;
-  const uint32_t lo = first ? (uint32_t)kMapFirst << kMapShift : (m ? g.r1.lo : g.r0.lo);
-  const int shift = first ? kMapShift : (m ? shift1 : shift0);
-  if (tid == 0) sh.inexact = 0;
-  team_sync<TEAM>();
-  uint32_t c[kPer], s[kPer], lc = 0;
-  u64 q[kPer], lq = 0;
-  bucket_counts<TEAM, 2>(sh, m * SH::kStride + b0, c);
-  bucket_counts<TEAM, 2>(sh, (2 + m) * SH::kStride + b0, s);
-  {
-    auto edge = [&](uint32_t bk) {  // mass of the largest value of bucket bk (the bucket of 512 and more counts as inexact)
-      const u64 t = (u64)lo + ((u64)bk << shift);
-      return t <= kTopKey && !(first && bk >= kBuckets) ? __float2ull_rz(__uint_as_float(kTopKey - (uint32_t)t) * 4294967296.0f) : 0ull;
-    };
-    u64 e = edge(b0);
-    bool bad = false;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-      const u64 e1 = edge(b0 + k + 1);
-      q[k] = c[k] * e1 + (u64)(s[k] - c[k] * (kLowBias + (uint32_t)e1));
-      bad = bad || c[k] * (e - e1) >> 32;
-      e = e1;
-      lc += c[k];
-      lq += q[k];
-    }
-    if (bad) {
-#pragma unroll
-      for (int r = 0; r < TEAM; ++r) peer_store<TEAM>(&sh.inexact, r, 1u);
-    }
-  }
-  uint32_t ic = warp_scan32(lc);
-  u64 iq = warp_scan64(lq);
-  if (lane == 31) {
-    sh.wscan_c[warp] = ic;
-    sh.wscan_q[warp] = iq;
-  }
-  __syncthreads();
-  {
-    const bool lower = lane >= m * (kRankWarps / 2) && lane < warp;
-    ic += __reduce_add_sync(kFull, lower ? sh.wscan_c[lane] : 0u);
-    iq += warp_sum64(lower ? sh.wscan_q[lane] : 0ull);
-  }
-  if (i >= kHalf - 32) {  // the last warp of the modality has the block's totals (in its last lane): to every block
-    const uint32_t tc = __shfl_sync(kFull, ic, 31);
-    const u64 tq = __shfl_sync(kFull, iq, 31);
-    if (lane < TEAM) {
-      peer_store<TEAM>(&sh.slice_c[m][rank], lane, tc);
-      peer_store<TEAM>(&sh.slice_q[m][rank], lane, tq);
-    }
-  }
-  team_sync<TEAM>();
-  if (TEAM > 1) {
-    const bool lower = lane < (int)rank;
-    ic += __reduce_add_sync(kFull, lower ? sh.slice_c[m][lane] : 0u);
-    iq += warp_sum64(lower ? sh.slice_q[m][lane] : 0ull);
-  }
-  g.exact = sh.inexact == 0;
-  if (first) {
-    g.n_vis = __reduce_add_sync(kFull, lane < TEAM ? sh.slice_c[0][lane] : 0u);
-    g.W0 = warp_sum64(lane < TEAM ? sh.slice_q[0][lane] : 0ull);
-    g.W1 = warp_sum64(lane < TEAM ? sh.slice_q[1][lane] : 0ull);
+__device__ __forceinline__ void mass_walk(RankShared<TEAM, 2>& sh, uint32_t rank, const BucketMap* map, u64 theta_fix,
+                                          MassRanges<RankShared<TEAM, 2>::kCap>& g, int shift0, int shift1) {
+  walk<TEAM, 2>(
+      sh, rank,
+      [&](int m, int b) {
+        const int shift = m ? shift1 : shift0;
+        return map ? bucket_start(*map, b) : BucketStart{(m ? g.r1.lo : g.r0.lo) + ((uint32_t)b << shift), shift};
+      },
+      [&](int m, u64 W) { return map ? mass_target(theta_fix, W) : (m ? g.need1 - g.above1 : g.need0 - g.above0); });
+  g.exact = !(sh.found[0].inexact | sh.found[1].inexact);
+  if (map) {
+    g.n_vis = sh.found[0].total;
+    g.W0 = sh.found[0].mass;
+    g.W1 = sh.found[1].mass;
     g.need0 = mass_target(theta_fix, g.W0);
     g.need1 = mass_target(theta_fix, g.W1);
   }
-  const u64 need = m ? g.need1 : g.need0;
-  ic += m ? g.r1.above : g.r0.above;
-  iq += m ? g.above1 : g.above0;
-  if (need && iq - lq < need && iq >= need) {  // the threshold lies in one of this thread's buckets
-    u64 run = iq - lq, at_q = 0;
-    uint32_t run_c = ic - lc, at = 0, at_c = 0, at_in = 0;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-      if (run < need) {
-        at = b0 + k;
-        at_c = run_c;
-        at_in = c[k];
-        at_q = run;
-      }
-      run += q[k];
-      run_c += c[k];
-    }
-#pragma unroll
-    for (int r = 0; r < TEAM; ++r) {
-      peer_store<TEAM>(&sh.first[m], r, ((u64)at_c << 32) | at);
-      peer_store<TEAM>(&sh.last[m], r, (u64)at_in);
-      peer_store<TEAM>(&sh.first_q[m], r, at_q);
-    }
-  }
-  team_sync<TEAM>();
-  auto narrow = [&](RankRange& r, u64& above, u64 need, int q2, int sft) {
+  auto narrow = [&](RankRange& r, u64& above, u64 need, const Found& f, int shift) {
     if (!need) {  // nothing to reach
       r = RankRange{kNowhere, 0u, 0u, 0u};
       return;
     }
-    bucket_range(r, first, (uint32_t)sh.first[q2], sft);
-    r.above = (uint32_t)(sh.first[q2] >> 32);
-    r.in = (uint32_t)sh.last[q2];
-    above = sh.first_q[q2];
+    bucket_range(r, map, f.at, shift);
+    r.above += f.above;
+    r.in = f.in;
+    above += f.above_q;
   };
   if (g.exact) {
-    narrow(g.r0, g.above0, g.need0, 0, shift0);
-    narrow(g.r1, g.above1, g.need1, 1, shift1);
+    narrow(g.r0, g.above0, g.need0, sh.found[0], shift0);
+    narrow(g.r1, g.above1, g.need1, sh.found[1], shift1);
   }
 }
 
 // (Rare) too many keys in a range, or sums that were not exact: halve it with exact sweeps until its keys fit the list or
 // are all alike. `sweep` calls its argument with the keys of the thread, some at a time.
 template <int TEAM, typename Sweep>
-__device__ __forceinline__ void mass_bisect(RankShared<TEAM, 2>& sh, uint32_t rank, u64 theta_fix, MassRanges& g, Sweep sweep) {
+__device__ __forceinline__ void mass_bisect(RankShared<TEAM, 2>& sh, uint32_t rank, u64 theta_fix,
+                                            MassRanges<RankShared<TEAM, 2>::kCap>& g, Sweep sweep) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // sums over the team, into every thread (of values that are already summed up over the warp)
   auto team_sums = [&](u64& a0, u64& a1) {
@@ -415,53 +392,56 @@ __device__ __forceinline__ void mass_bisect(RankShared<TEAM, 2>& sh, uint32_t ra
   }
 }
 
-// With the candidates of all blocks in their lists: block 0 finds the counts and writes the unit's results; the unit that is
-// done last goes on with its sequence.
+// With all candidates on their way to block 0's list: it finds the counts and writes the unit's results; the unit that is
+// done last goes on with its sequence (ph: phi of its first layer).
 template <int TEAM>
-__device__ __forceinline__ void mass_finish(RankShared<TEAM, 2>& sh, const AllocParams& p, uint32_t rank, int u, int b, int n, const MassRanges& g) {
+__device__ __forceinline__ void mass_finish(RankShared<TEAM, 2>& sh, const AllocParams& p, uint32_t rank, int u, int b, int n, double ph,
+                                            const MassRanges<RankShared<TEAM, 2>::kCap>& g) {
+  constexpr uint32_t kCap = RankShared<TEAM, 2>::kCap;
   const int tid = threadIdx.x;
-  if (rank == 0 && tid < 2) {
-    const u64 W = tid ? g.W1 : g.W0, tot = g.W0 + g.W1;
-    p.mass[(int64_t)u * 2 + tid] = __ull2double_rn(W) / 4294967296.0;
-    p.pref[(int64_t)u * 2 + tid] = tot ? __ddiv_rn(__ull2double_rn(W), __ull2double_rn(tot)) : 0.0;
-    if ((tid ? g.need1 : g.need0) == 0) p.demand[(int64_t)u * 2 + tid] = 0;
-  }
-  team_sync<TEAM>();
-  if (rank == 0) {
-    const uint32_t got = gather_lists<TEAM, 2>(sh);
-    const bool on0 = g.need0 && g.r0.in <= kListCap, on1 = g.need1 && g.r1.in <= kListCap;
-    finish_lists<TEAM, 2, true>(sh, g.r0, g.r1, got, on0, on1, g.need0, g.need1, g.above0, g.above1);
-    if (tid < 2 && (tid ? g.need1 : g.need0)) {
+  team_sync<TEAM>();  // (the last access to another block's shared memory)
+  if (rank != 0) return;
+  const bool on0 = g.need0 && g.r0.in <= kCap, on1 = g.need1 && g.r1.in <= kCap;
+  finish_lists<TEAM, 2, true>(sh, g.r0, g.r1, on0, on1, g.need0, g.need1, g.above0, g.above1);
+  if (tid < 2) {
+    const u64 need = tid ? g.need1 : g.need0;
+    uint32_t count = 0;
+    if (need) {
       // every key left has the value kTopKey - t: as few of them as reach the threshold
       const RankRange my = tid ? g.r1 : g.r0;
       const bool listed = tid ? on1 : on0;
       uint32_t take = listed ? sh.fin_in[tid] : my.in;
       if (take > 1) {
-        const u64 need = tid ? g.need1 : g.need0, above = listed ? sh.fin_m[tid] : (tid ? g.above1 : g.above0);
+        const u64 above = listed ? sh.fin_m[tid] : (tid ? g.above1 : g.above0);
         const u64 each = psi_fix(kTopKey - (listed ? sh.fin_lo[tid] : my.lo));
         if (each > 0) {
           const u64 k = (need - above + each - 1) / each;
           if (k < (u64)take) take = (uint32_t)k;
         }
       }
-      p.demand[(int64_t)u * 2 + tid] = (int32_t)((listed ? sh.fin_c[tid] : my.above) + take);
+      count = (listed ? sh.fin_c[tid] : my.above) + take;
     }
+    p.demand[(int64_t)u * 2 + tid] = (int32_t)count;
+  } else if (tid >= 32 && tid < 34) {
+    const int m = tid - 32;
+    const u64 W = m ? g.W1 : g.W0, tot = g.W0 + g.W1;
+    p.mass[(int64_t)u * 2 + m] = __ull2double_rn(W) / 4294967296.0;
+    p.pref[(int64_t)u * 2 + m] = tot ? __ddiv_rn(__ull2double_rn(W), __ull2double_rn(tot)) : 0.0;
   }
-  if (TEAM > 1) team_sync<TEAM>();  // no block leaves while block 0 still reads its shared memory
-  if (rank != 0 || !p.counter) return;
+  if (!p.counter) return;
   __shared__ unsigned s_last;
   __syncthreads();
   if (tid == 0) s_last = arrive_inc(p.counter + b, (unsigned)(p.L * p.Hkv) - 1u);  // (wraps to 0: ready for the next call)
   __syncthreads();
   if (s_last != (unsigned)(p.L * p.Hkv) - 1u) return;
-  static_assert(sizeof(sh.cnt) >= kLayerChunk * 16, "the scan reuses the buckets");
-  sequence_budgets(p, b, n, (int)g.n_vis, reinterpret_cast<double*>(sh.cnt), reinterpret_cast<long long*>(sh.cnt) + kLayerChunk);
+  static_assert(sizeof(sh.cnt) >= kBudgetBytes, "the scan reuses the buckets");
+  sequence_budgets(p, b, n, (int)g.n_vis, ph, reinterpret_cast<double*>(sh.cnt));
 }
 
 // t of KPT consecutive positions (kNoKey outside the sequence); returns those that are inside.
 template <int KPT>
-__device__ __forceinline__ uint32_t load_valid(const float* psi, int mis, int n_max, int n, int pos0, uint32_t (&t)[KPT]) {
-  load_scores<KPT>(psi, mis, n_max, pos0, t);
+__device__ __forceinline__ uint32_t take_valid(const RawScores<KPT>& raw, int mis, int n, int pos0, uint32_t (&t)[KPT]) {
+  take_scores<KPT>(raw, mis, t);
   const uint32_t valid = valid_bits<KPT>(n, pos0);
   if (valid != valid_bits<KPT>(KPT, 0)) {
 #pragma unroll
@@ -470,35 +450,60 @@ __device__ __forceinline__ uint32_t load_valid(const float* psi, int mis, int n_
   }
   return valid;
 }
+template <int KPT>
+__device__ __forceinline__ uint32_t load_valid(const float* psi, int mis, int n_max, int n, int pos0, uint32_t (&t)[KPT]) {
+  RawScores<KPT> raw;
+  issue_scores<KPT>(psi, mis, n_max, pos0, raw);
+  return take_valid<KPT>(raw, mis, n, pos0, t);
+}
 
-// Masses, preference and Eq. 9's counts of one unit whose keys fit the registers of its team (see rank_common.cuh).
+// Masses, preference and Eq. 9's counts of one unit whose keys fit the registers of its team (see rank_common.cuh). (A
+// team clears its buckets, and its blocks learn of one another, under the kernel before; blocks on their own, which may be
+// several rounds of them, while their loads are on the way.)
 template <int KPT, int TEAM>
 __global__ void __launch_bounds__(kRankThreads, 2) alloc_unit_kernel(const __grid_constant__ AllocParams p) {
+  constexpr uint32_t kCap = RankShared<TEAM, 2>::kCap;
   __shared__ RankShared<TEAM, 2> sh;
+  team_started<TEAM>();
+  if (TEAM > 1) zero_buckets<TEAM, 2>(sh);
   pdl_wait();
   pdl_go();
   const uint32_t rank = TEAM > 1 ? team_rank() : 0u;
   const int u = blockIdx.x / TEAM, b = u / (p.Hkv * p.L);
-  const int n = clamped_len(p.seq_len, b, p.n_max);
   const int pos0 = (int)rank * kRankThreads * KPT + threadIdx.x * KPT;  // a block owns consecutive positions
+  const int mis = (int)(((int64_t)u * p.n_max) & 3);
+  RawScores<KPT> raw;
+  RawMask<KPT> raw_mask;
+  issue_scores<KPT>(p.psi + (int64_t)u * p.n_max, mis, p.n_max, pos0, raw);
+  issue_mask<KPT>(p.mask + (int64_t)b * p.n_max, p.n_max, pos0, raw_mask);
+  if (TEAM == 1) zero_buckets<TEAM, 2>(sh);
+  const int n = clamped_len(p.seq_len, b, p.n_max);
+  const double ph = p.counter ? first_phi(p, b) : 0.0;
   uint32_t t[KPT];
-  const uint32_t valid = load_valid<KPT>(p.psi + (int64_t)u * p.n_max, (int)(((int64_t)u * p.n_max) & 3), p.n_max, n, pos0, t);
-  const uint32_t vis = load_mask<KPT>(p.mask + (int64_t)b * p.n_max, p.n_max, pos0);
-  zero_buckets<TEAM, 2>(sh);
-  add_first<KPT, TEAM>(sh, t, vis, valid);
-  MassRanges g = {};
-  mass_walk<TEAM>(sh, rank, true, p.theta_fix, g, 0, 0);
+  const uint32_t valid = take_valid<KPT>(raw, mis, n, pos0, t), vis = take_mask<KPT>(raw_mask);
+  const BucketMap map = bucket_map(p.rows, n);
+  __syncthreads();
+  add_first<KPT, TEAM>(sh, map, t, vis, valid);
+  MassRanges<kCap> g = {};
+  team_wait_started<TEAM>();
+  mass_walk<TEAM>(sh, rank, &map, p.theta_fix, g, 0, 0);
+  bool swept = false;
   if (!g.exact || !g.listed()) {
     if (g.exact) {
       const int shift0 = range_shift(g.r0.span, kDig), shift1 = range_shift(g.r1.span, kDig);
+      team_sync<TEAM>();
       zero_buckets<TEAM, 2>(sh);
+      __syncthreads();
       add_again<KPT, TEAM>(sh, g, t, vis, shift0, shift1);
-      mass_walk<TEAM>(sh, rank, false, p.theta_fix, g, shift0, shift1);
+      mass_walk<TEAM>(sh, rank, nullptr, p.theta_fix, g, shift0, shift1);
     }
-    mass_bisect<TEAM>(sh, rank, p.theta_fix, g, [&](auto each) {
+    if (!g.exact || g.crowded0() || g.crowded1()) {
+      mass_bisect<TEAM>(sh, rank, p.theta_fix, g, [&](auto each) {
 #pragma unroll
-      for (int j = 0; j < KPT; ++j) each(t[j], (vis >> j) & 1u);
-    });
+        for (int j = 0; j < KPT; ++j) each(t[j], (vis >> j) & 1u);
+      });
+      swept = true;
+    }
   }
   uint32_t in = 0;
 #pragma unroll
@@ -506,8 +511,10 @@ __global__ void __launch_bounds__(kRankThreads, 2) alloc_unit_kernel(const __gri
     const bool v = (vis >> j) & 1u;
     if (t[j] - (v ? g.r0.lo : g.r1.lo) <= (v ? g.r0.span : g.r1.span)) in |= 1u << j;
   }
-  append<TEAM, 2, KPT>(sh, g.r0.in <= kListCap ? in & vis : 0u, g.r1.in <= kListCap ? in & ~vis : 0u, t, g.r0.lo, g.r1.lo);
-  mass_finish<TEAM>(sh, p, rank, u, b, n, g);
+  const uint32_t in0 = g.r0.in <= kCap ? in & vis : 0u, in1 = g.r1.in <= kCap ? in & ~vis : 0u;
+  if (swept) find_places<TEAM, 2>(sh, rank, __popc(in0), __popc(in1));
+  append<TEAM, 2, KPT, false>(sh, rank, in0, in1, t, g.r0.lo, g.r1.lo);
+  mass_finish<TEAM>(sh, p, rank, u, b, n, ph, g);
 }
 
 // The same for a longer unit, which is read twice, for the buckets and for the candidates (listed as positions); the mask is
@@ -515,20 +522,25 @@ __global__ void __launch_bounds__(kRankThreads, 2) alloc_unit_kernel(const __gri
 template <int TEAM>
 __global__ void __launch_bounds__(kRankThreads, 2) alloc_long_kernel(const __grid_constant__ AllocParams p) {
   constexpr int KPT = 16, kRound = kRankThreads * KPT;
+  constexpr uint32_t kCap = RankShared<TEAM, 2>::kCap;
   __shared__ RankShared<TEAM, 2> sh;
   extern __shared__ __align__(16) uint32_t bits[];
+  team_started<TEAM>();
+  zero_buckets<TEAM, 2>(sh);
   pdl_wait();
   pdl_go();
   const uint32_t rank = TEAM > 1 ? team_rank() : 0u;
   const int tid = threadIdx.x, u = blockIdx.x / TEAM, b = u / (p.Hkv * p.L);
   const int n = clamped_len(p.seq_len, b, p.n_max);
+  const double ph = p.counter ? first_phi(p, b) : 0.0;
   const float* psi = p.psi + (int64_t)u * p.n_max;
   const int mis = (int)(((int64_t)u * p.n_max) & 3);
   const uint8_t* mask = p.mask + (int64_t)b * p.n_max;
   uint32_t *pos0 = bits, *pos1 = bits + kListCap, *vis_w = bits + 2 * kListCap;
   const int rounds = (n + kRound * TEAM - 1) / (kRound * TEAM);
   const int start = (int)rank * rounds * kRound;  // a block owns consecutive positions
-  zero_buckets<TEAM, 2>(sh);
+  const BucketMap map = bucket_map(p.rows, n);
+  __syncthreads();
 #pragma unroll 1
   for (int r = 0; r < rounds; ++r) {
     const int at = start + r * kRound + tid * KPT;
@@ -536,34 +548,41 @@ __global__ void __launch_bounds__(kRankThreads, 2) alloc_long_kernel(const __gri
     const uint32_t valid = load_valid<KPT>(psi, mis, p.n_max, n, at, t);
     const uint32_t vis = load_mask<KPT>(mask, p.n_max, at);
     bits_of_thread(vis_w, r) = (uint16_t)vis;
-    add_first<KPT, TEAM>(sh, t, vis, valid);
+    add_first<KPT, TEAM>(sh, map, t, vis, valid);
   }
-  MassRanges g = {};
-  mass_walk<TEAM>(sh, rank, true, p.theta_fix, g, 0, 0);
+  MassRanges<kCap> g = {};
+  team_wait_started<TEAM>();
+  mass_walk<TEAM>(sh, rank, &map, p.theta_fix, g, 0, 0);
+  bool swept = false;
   if (!g.exact || !g.listed()) {
     if (g.exact) {
       const int shift0 = range_shift(g.r0.span, kDig), shift1 = range_shift(g.r1.span, kDig);
+      team_sync<TEAM>();
       zero_buckets<TEAM, 2>(sh);
+      __syncthreads();
 #pragma unroll 1
       for (int r = 0; r < rounds; ++r) {
         uint32_t t[KPT];
         load_valid<KPT>(psi, mis, p.n_max, n, start + r * kRound + tid * KPT, t);
         add_again<KPT, TEAM>(sh, g, t, bits_of_thread(vis_w, r), shift0, shift1);
       }
-      mass_walk<TEAM>(sh, rank, false, p.theta_fix, g, shift0, shift1);
+      mass_walk<TEAM>(sh, rank, nullptr, p.theta_fix, g, shift0, shift1);
     }
-    mass_bisect<TEAM>(sh, rank, p.theta_fix, g, [&](auto each) {
+    if (!g.exact || g.crowded0() || g.crowded1()) {
+      mass_bisect<TEAM>(sh, rank, p.theta_fix, g, [&](auto each) {
 #pragma unroll 1
-      for (int r = 0; r < rounds; ++r) {
-        uint32_t t[KPT];
-        load_valid<KPT>(psi, mis, p.n_max, n, start + r * kRound + tid * KPT, t);
-        const uint32_t vis = bits_of_thread(vis_w, r);
+        for (int r = 0; r < rounds; ++r) {
+          uint32_t t[KPT];
+          load_valid<KPT>(psi, mis, p.n_max, n, start + r * kRound + tid * KPT, t);
+          const uint32_t vis = bits_of_thread(vis_w, r);
 #pragma unroll
-        for (int j = 0; j < KPT; ++j) each(t[j], (vis >> j) & 1u);
-      }
-    });
+          for (int j = 0; j < KPT; ++j) each(t[j], (vis >> j) & 1u);
+        }
+      });
+      swept = true;
+    }
   }
-  const bool on0 = g.r0.in <= kListCap, on1 = g.r1.in <= kListCap;
+  const bool on0 = g.r0.in <= kCap, on1 = g.r1.in <= kCap;
 #pragma unroll 1
   for (int r = 0; r < rounds; ++r) {
     const int at = r * kRound + tid * KPT;
@@ -579,10 +598,12 @@ __global__ void __launch_bounds__(kRankThreads, 2) alloc_long_kernel(const __gri
     append_positions<TEAM, 2>(sh, pos0, pos1, on0 ? in & vis : 0u, on1 ? in & ~vis : 0u, at);
   }
   __syncthreads();
-  const int m = tid / kHalf, mine_n = m ? sh.list_n >> 16 : sh.list_n & 0xffffu;
+  const uint32_t listed = sh.list_n;
+  if (swept) find_places<TEAM, 2>(sh, rank, tid == 0 ? listed & 0xffffu : 0u, tid == 0 ? listed >> 16 : 0u);
+  const int m = tid / kHalf, mine_n = m ? listed >> 16 : listed & 0xffffu;
   for (int i = tid % kHalf; i < mine_n; i += kHalf)
-    sh.list[m][i] = score_t(__ldg(psi + start + (m ? pos1 : pos0)[i])) - (m ? g.r1.lo : g.r0.lo);
-  mass_finish<TEAM>(sh, p, rank, u, b, n, g);
+    put<TEAM, 2, false>(sh, m, sh.found[m].seg[rank] + i, score_t(__ldg(psi + start + (m ? pos1 : pos0)[i])) - (m ? g.r1.lo : g.r0.lo));
+  mass_finish<TEAM>(sh, p, rank, u, b, n, ph, g);
 }
 
 // The same as a kernel of its own, one block per sequence: for the budgets of one layer whose masses and demands are given
@@ -590,18 +611,18 @@ __global__ void __launch_bounds__(kRankThreads, 2) alloc_long_kernel(const __gri
 // one, which has waited for all kernels before it, so the tokens can be counted before the wait for its results.
 __global__ void __launch_bounds__(1024) alloc_seq_kernel(const __grid_constant__ AllocParams p, int after_units) {
   __shared__ int s_nv;
-  __shared__ double s_phi[kLayerChunk];
-  __shared__ long long s_dem[kLayerChunk];
+  __shared__ __align__(16) double s_phi[kBudgetBytes / 8];
   if (!after_units) pdl_wait();
   const int b = blockIdx.x;
   const int n = clamped_len(p.seq_len, b, p.n_max);
+  const double ph = first_phi(p, b);
   if (threadIdx.x == 0) s_nv = 0;
   __syncthreads();
   count_visual(p.mask + (int64_t)b * p.n_max, n, &s_nv);
   __syncthreads();
   if (after_units) pdl_wait();
   pdl_go();
-  sequence_budgets(p, b, n, s_nv, s_phi, s_dem);
+  sequence_budgets(p, b, n, s_nv, ph, s_phi);
 }
 
 template <int TEAM>
@@ -657,6 +678,7 @@ AllocParams alloc_params(const madakv_config& c, int layers, const float* psi, c
   p.hcc_mode = c.hcc_mode;
   p.keep_window = c.keep_window;
   p.window = c.window;
+  p.rows = c.n_q_heads / c.n_kv_heads * c.window;
   p.theta_fix = (u64)((double)c.theta * 4294967296.0);
   p.depth = c.n_layers;
   p.layer = -1;

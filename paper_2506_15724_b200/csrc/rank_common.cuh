@@ -7,11 +7,16 @@
 // largest key, or the key at which a mass is reached) is found in few steps. Two things bound these kernels: the integer
 // instructions per key in calls with many units (an SM has some 230 000 keys of 256 units of 131072 keys to handle), and the
 // fixed latency of a step (barriers, walking the buckets) in calls with few.
-//   buckets  a count (and for Eq. 9 a mass, see allocate.cu) per key into 2048 buckets that are the same for all units, by
-//            shared atomics without a result; a walk of the buckets narrows the range that the threshold can lie in to one
-//            bucket, usually some tens of keys
-//   list     the keys of the narrowed range are collected in shared memory, where half of a block's threads per modality
-//            lay buckets over them once more; the few keys left are compared with one another
+//   buckets  a count (and for Eq. 9 a mass, see allocate.cu) per key into 2048 buckets by shared atomics without a result
+//            (bucket_map); a walk of the buckets narrows the range that the threshold can lie in to one bucket, usually
+//            some tens of keys
+//   list     the keys of the narrowed range are collected in shared memory and compared with one another (more than 256
+//            of them: after half of a block's threads per modality have laid buckets over them once more)
+// A team's blocks meet twice. Every block sums its buckets up to 32 coarse ones and pushes those to all; behind the first
+// barrier a warp per modality of every block finds the coarse bucket, reads its 64 buckets from all blocks and finds the
+// bucket, the same in every block, with the places of all blocks' keys in the list; the keys are pushed there before the
+// second barrier. (With a share of all buckets per block, read from all others, their totals and the bucket announced and
+// the lists gathered, five barriers in all, allocation and selection of 4 units of 32768 keys took 17 and 13 us; now 13 and 9.)
 // Buckets over the range of each unit's keys needed a sweep for that range before; without it, and with long units read
 // twice instead of three (allocation) or four times (selection), allocation + selection + compaction went from 602 to 483 us
 // on 256 units of 131072 keys, from 618 to 523 on 1600 of 13411, from 213 to 161 on 3360 of 471, from 31 to 26 on 200 of 772.
@@ -30,8 +35,8 @@ constexpr unsigned int kFull = 0xffffffffu;
 constexpr int kRankThreads = 512;
 constexpr int kRankWarps = kRankThreads / 32;
 constexpr int kHalf = kRankThreads / 2;        // threads per modality in the walks
-constexpr int kListCap = 1024;                 // candidates per modality
-constexpr int kFewCap = 32;                    // candidates compared with one another
+constexpr int kListCap = 1024;                 // candidates per modality at most
+constexpr int kFewCap = kHalf;                 // candidates compared with one another
 constexpr int kMaxTeam = 8;
 constexpr uint32_t kTopKey = 0x7f81ffffu;      // t = kTopKey - key: ascending t is descending importance
 constexpr uint32_t kNoKey = 0xffffffffu;       // t of a slot without a key
@@ -50,6 +55,15 @@ __device__ __forceinline__ void team_sync() {
     asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
   else
     __syncthreads();
+}
+// The two halves of a first barrier: no block of a cluster touches another's shared memory before that one has started.
+template <int TEAM>
+__device__ __forceinline__ void team_started() {
+  if (TEAM > 1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+}
+template <int TEAM>
+__device__ __forceinline__ void team_wait_started() {
+  if (TEAM > 1) asm volatile("barrier.cluster.wait;" ::: "memory");
 }
 __device__ __forceinline__ uint32_t peer_addr(const void* local, uint32_t rank) {
   uint32_t r;
@@ -79,6 +93,12 @@ template <int TEAM>
 __device__ __forceinline__ void peer_store(u64* local, uint32_t rank, u64 v) {
   if (TEAM == 1) *local = v;
   else asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(peer_addr(local, rank)), "l"(v) : "memory");
+}
+
+template <int TEAM>
+__device__ __forceinline__ void peer_store(uint4* local, uint32_t rank, uint4 v) {
+  if (TEAM == 1) *local = v;
+  else asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(peer_addr(local, rank)), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
 // ---- sums over a warp
@@ -114,76 +134,106 @@ __device__ __forceinline__ u64 warp_scan64(u64 v) {
 // element by element.
 // A score's order-preserving key is its bits where it is positive, else (NaN too) 0; kept is t, its distance from kTopKey.
 __device__ __forceinline__ uint32_t score_t(float x) { return kTopKey - __float_as_uint(fmaxf(x, 0.0f)); }
+// The loads are issued apart from their use, so that scores, mask, length and budgets are all on their way together (one after
+// the other, as the branches had them, they took two or three latencies of the memory: 5000 of a block's 16000 clocks).
 template <int KPT>
-__device__ __forceinline__ void load_scores(const float* row, int mis, int n_max, int pos0, uint32_t (&t)[KPT]) {
+struct RawScores {
+  float4 v[KPT / 4 + 1];
+  int down;  // elements to move down
+};
+template <int KPT>
+__device__ __forceinline__ void issue_scores(const float* row, int mis, int n_max, int pos0, RawScores<KPT>& raw) {
+  raw.down = 0;
+  raw.v[KPT / 4] = make_float4(0.f, 0.f, 0.f, 0.f);
   if (mis == 0 && pos0 + KPT <= n_max) {
 #pragma unroll
-    for (int j = 0; j < KPT; j += 4) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(row + pos0 + j));
-      t[j] = score_t(v.x);
-      t[j + 1] = score_t(v.y);
-      t[j + 2] = score_t(v.z);
-      t[j + 3] = score_t(v.w);
-    }
+    for (int j = 0; j < KPT / 4; ++j) raw.v[j] = __ldg(reinterpret_cast<const float4*>(row + pos0) + j);
   } else if (mis != 0 && pos0 + KPT + 4 <= n_max) {
     // (a misaligned row has a unit before it: the pieces start inside the array; they end inside the row)
-    float f[KPT + 4];
-    const float4* src = reinterpret_cast<const float4*>(row + pos0 - mis);
 #pragma unroll
-    for (int j = 0; j < KPT + 4; j += 4) {
-      const float4 v = __ldg(src + j / 4);
-      f[j] = v.x;
-      f[j + 1] = v.y;
-      f[j + 2] = v.z;
-      f[j + 3] = v.w;
-    }
-#pragma unroll
-    for (int j = 0; j < KPT + 3; ++j) f[j] = (mis & 1) ? f[j + 1] : f[j];
-#pragma unroll
-    for (int j = 0; j < KPT; ++j) t[j] = score_t((mis & 2) ? f[j + 2] : f[j]);
+    for (int j = 0; j < KPT / 4 + 1; ++j) raw.v[j] = __ldg(reinterpret_cast<const float4*>(row + pos0 - mis) + j);
+    raw.down = mis;
   } else {
+    auto one = [&](int x) { return pos0 + x < n_max ? __ldg(row + pos0 + x) : 0.f; };
 #pragma unroll
-    for (int j = 0; j < KPT; ++j) t[j] = pos0 + j < n_max ? score_t(__ldg(row + pos0 + j)) : kTopKey;
+    for (int j = 0; j < KPT / 4; ++j) raw.v[j] = make_float4(one(4 * j), one(4 * j + 1), one(4 * j + 2), one(4 * j + 3));
   }
 }
 template <int KPT>
-__device__ __forceinline__ uint32_t load_mask(const uint8_t* row, int n_max, int pos0) {  // bit j: position pos0 + j is visual
+__device__ __forceinline__ void take_scores(const RawScores<KPT>& raw, int mis, uint32_t (&t)[KPT]) {
+  float f[KPT + 4];
+#pragma unroll
+  for (int j = 0; j < KPT / 4 + 1; ++j) {
+    f[4 * j] = raw.v[j].x;
+    f[4 * j + 1] = raw.v[j].y;
+    f[4 * j + 2] = raw.v[j].z;
+    f[4 * j + 3] = raw.v[j].w;
+  }
+  if (mis) {  // (the same for the whole unit)
+#pragma unroll
+    for (int j = 0; j < KPT + 3; ++j) f[j] = (raw.down & 1) ? f[j + 1] : f[j];
+#pragma unroll
+    for (int j = 0; j < KPT; ++j) f[j] = (raw.down & 2) ? f[j + 2] : f[j];
+  }
+#pragma unroll
+  for (int j = 0; j < KPT; ++j) t[j] = score_t(f[j]);
+}
+template <int KPT>
+__device__ __forceinline__ void load_scores(const float* row, int mis, int n_max, int pos0, uint32_t (&t)[KPT]) {
+  RawScores<KPT> raw;
+  issue_scores<KPT>(row, mis, n_max, pos0, raw);
+  take_scores<KPT>(raw, mis, t);
+}
+template <int KPT>
+struct RawMask {
+  uint32_t w[KPT / 4 + 1];
+  uint32_t shift;  // bits to move down
+  uint32_t bits;   // of positions that were read one by one
+};
+template <int KPT>
+__device__ __forceinline__ void issue_mask(const uint8_t* row, int n_max, int pos0, RawMask<KPT>& raw) {
   const uintptr_t at = reinterpret_cast<uintptr_t>(row + pos0);
-  uint32_t vis = 0;
+  raw.shift = raw.bits = 0;
+#pragma unroll
+  for (int j = 0; j < KPT / 4 + 1; ++j) raw.w[j] = 0;
   if (pos0 + KPT <= n_max && (at & (KPT - 1)) == 0) {
-    uint32_t w[KPT / 4];
     if (KPT == 8) {
       const uint2 v = __ldg(reinterpret_cast<const uint2*>(row + pos0));
-      w[0] = v.x;
-      w[1] = v.y;
+      raw.w[0] = v.x;
+      raw.w[1] = v.y;
     } else {
 #pragma unroll
       for (int j = 0; j < KPT / 16; ++j) {
         const uint4 v = __ldg(reinterpret_cast<const uint4*>(row + pos0) + j);
-        w[4 * j] = v.x;
-        w[4 * j + 1] = v.y;
-        w[4 * j + 2] = v.z;
-        w[4 * j + 3] = v.w;
+        raw.w[4 * j] = v.x;
+        raw.w[4 * j + 1] = v.y;
+        raw.w[4 * j + 2] = v.z;
+        raw.w[4 * j + 3] = v.w;
       }
     }
-#pragma unroll
-    for (int j = 0; j < KPT / 4; ++j) vis |= nonzero_bytes(w[j]) << (4 * j);
   } else if (pos0 >= 4 && pos0 + KPT + 4 <= n_max) {
     const uint32_t* src = reinterpret_cast<const uint32_t*>(at & ~(uintptr_t)3);
-    const uint32_t sh = (uint32_t)(at & 3) * 8;
-    uint32_t w = __ldg(src);
+    raw.shift = (uint32_t)(at & 3) * 8;
 #pragma unroll
-    for (int j = 0; j < KPT / 4; ++j) {
-      const uint32_t nx = __ldg(src + j + 1);
-      vis |= nonzero_bytes(__funnelshift_r(w, nx, sh)) << (4 * j);
-      w = nx;
-    }
+    for (int j = 0; j < KPT / 4 + 1; ++j) raw.w[j] = __ldg(src + j);
   } else {
 #pragma unroll
     for (int j = 0; j < KPT; ++j)
-      if (pos0 + j < n_max && __ldg(row + pos0 + j)) vis |= 1u << j;
+      if (pos0 + j < n_max && __ldg(row + pos0 + j)) raw.bits |= 1u << j;
   }
+}
+template <int KPT>
+__device__ __forceinline__ uint32_t take_mask(const RawMask<KPT>& raw) {  // bit j: position pos0 + j is visual
+  uint32_t vis = raw.bits;
+#pragma unroll
+  for (int j = 0; j < KPT / 4; ++j) vis |= nonzero_bytes(__funnelshift_r(raw.w[j], raw.w[j + 1], raw.shift)) << (4 * j);
   return vis;
+}
+template <int KPT>
+__device__ __forceinline__ uint32_t load_mask(const uint8_t* row, int n_max, int pos0) {
+  RawMask<KPT> raw;
+  issue_mask<KPT>(row, n_max, pos0, raw);
+  return take_mask<KPT>(raw);
 }
 // Bits of a long unit in shared memory, one per position of the block: word w sits at w + w / 32, so that threads that walk
 // several consecutive words each hit different banks. A thread's 16 positions of round r are half a word.
@@ -198,38 +248,86 @@ __device__ __forceinline__ uint32_t valid_bits(int n, int pos0) {  // bit j: pos
   return k == 32 ? 0xffffffffu : (1u << k) - 1u;
 }
 
-// The first layout of the buckets is the same for all units, so that no sweep has to find the range of the keys before: 64
-// buckets per octave from 512 down to 2^-23, the first and the last one take what lies outside. It is as fine as a
-// layout over the range of importance values is (they spread over some twenty octaves).
-constexpr int kMapShift = 17, kMapFirst = 7616;  // t >> 17 of the values from 512 up
-constexpr int kDig = 11, kBuckets = 1 << kDig;
+// The first layout of the buckets depends on a sequence's length and the window only, so that no sweep has to find the range of
+// the keys before. The scores of a unit add up to its window rows, so their mean is known; sums of many rows crowd around
+// it or, where a few tokens hold much of the mass, somewhat below (half of the keys of a grouped-query unit lie within a
+// twelfth of an octave). 768 buckets cover 1.5 octaves there, for fewer than 128 rows three; 64 or, for small means, 32 per
+// octave lie above, up to 512.0, and 64 below; the first and the last one take what lies outside. (64 buckets per octave
+// throughout: 1000 candidates for 32768 keys of 224 rows and a sweep more for 131072 keys of 256 rows, 3400 in one
+// bucket; and atomics on few addresses. One octave: 64 units of 3688 keys, 256 rows, whose keys lie half an octave below
+// the mean, 60 us for the three steps after scoring instead of 50.)
+constexpr int kBuckets = 2048, kDig = 11, kMidBuckets = 768;
+constexpr int kMidRows = 128;              // from this many window rows on: 1.5 octaves
+constexpr uint32_t kMapTop = 0x3b800000u;  // t of 512.0, rounded down to where a bucket starts
+struct BucketMap {
+  uint32_t mid;              // where the fine buckets start
+  int mid_shift, high_shift; // values of t per bucket there and above, as shifts; below it is kLowShift
+  int c1, b0, c3;            // bucket of t above: (t >> high_shift) - c1; first fine bucket; below: (t >> kLowShift) + c3
+};
+constexpr int kLowShift = 17;
+__device__ __forceinline__ BucketMap bucket_map(int rows, int n) {
+  BucketMap g;
+  g.mid_shift = rows >= kMidRows ? 14 : 15;
+  // (aligned so that eight buckets from a multiple of eight on are equally wide)
+  const float top = __fdividef((float)rows, (float)max(n, 1)) * (rows >= kMidRows ? 1.23f : 2.2f);
+  g.mid = max((kTopKey - __float_as_uint(top)) & ~((8u << 18) - 1u), kMapTop + (8u << 18));
+  g.high_shift = (g.mid - kMapTop) >> 17 <= 832u ? 17 : 18;
+  g.c1 = (int)(kMapTop >> g.high_shift);
+  g.b0 = (int)(g.mid >> g.high_shift) - g.c1;
+  g.c3 = g.b0 + kMidBuckets - (int)((g.mid + ((uint32_t)kMidBuckets << g.mid_shift)) >> kLowShift);
+  return g;
+}
+// The fine buckets' line is steeper than the two others, so the three meet as a minimum of a maximum.
+__device__ __forceinline__ uint32_t map_bucket(const BucketMap& g, uint32_t t) {
+  const int high = (int)(t >> g.high_shift) - g.c1, fine = ((int)(t - g.mid) >> g.mid_shift) + g.b0, low = (int)(t >> kLowShift) + g.c3;
+  return (uint32_t)max(min(min(max(high, fine), low), kBuckets - 1), 0);
+}
+// Where bucket b starts (t; the first one: where it would) and, as a shift, the width of it and of its neighbours up to the next
+// multiple of eight.
+struct BucketStart {
+  uint32_t t;
+  int shift;
+};
+__device__ __forceinline__ BucketStart bucket_start(const BucketMap& g, int b) {
+  if (b < g.b0) return {(uint32_t)(b + g.c1) << g.high_shift, g.high_shift};
+  if (b < g.b0 + kMidBuckets) return {g.mid + ((uint32_t)(b - g.b0) << g.mid_shift), g.mid_shift};
+  return {(uint32_t)(b - g.c3) << kLowShift, kLowShift};
+}
 
 // ---- shared memory of a block
+// What a walk finds for a modality.
+struct Found {
+  u64 mass, above_q;                   // mass of all its keys (allocation); mass before the bucket
+  uint32_t total, hit, at, above, in;  // its keys; whether what is needed is reached; the bucket; keys before it and in it
+  uint32_t before;                     // of the keys before the bucket (of all, if it is not reached) those of the blocks before this one
+  uint32_t inexact;                    // masses are not known exactly
+  uint32_t seg[kMaxTeam + 1];          // places of each block's keys of the bucket
+};
+constexpr int kCoarse = kBuckets / 64;
 template <int TEAM, int WORDS>  // WORDS: count, or count and mass, per bucket
 struct RankShared {
-  static constexpr int kPer = kBuckets / (kHalf * TEAM);  // buckets per thread of the walk: 8, 4, 2, 1
   static constexpr int kStride = kBuckets;
-  // the buckets' counts; once they are walked, the candidates of the whole team and the buckets of the finish (count,
-  // mass low, mass high; one per thread and modality) take their place
-  static constexpr int kFinish = 2 * kListCap + 6 * kHalf;
-  static constexpr int kArea = 2 * WORDS * kStride > kFinish ? 2 * WORDS * kStride : kFinish;
-  alignas(16) uint32_t cnt[kArea];
-  uint32_t list[2][kListCap];                   // this block's candidates
+  static constexpr int kCap = TEAM > 1 ? kListCap / 2 : kListCap;
+  // the buckets' counts; once they are walked, the buckets of the finish (count, mass low, mass high; one per thread and
+  // modality) and the keys that are compared with one another, with their masses, take their place
+  alignas(16) uint32_t cnt[2 * WORDS * kStride];
+  uint4 coarse[2][TEAM][TEAM > 1 ? kCoarse : 1];  // every block's sums of 64 buckets: count, mass (low, high), inexact
+  uint32_t list[2][kCap];                       // candidates of the team (allocation: in block 0)
+  Found found[2];
   u64 wsum[2][kRankWarps];                      // per warp: masses (allocation)
   u64 slice_q[2][kMaxTeam];
-  u64 wscan_q[kRankWarps], wscan_r[kRankWarps];
-  u64 few_m[2][kFewCap];
-  u64 first[2], last[2], first_q[2];            // walk: (count before << 32) | bucket, its count, mass before
+  u64 wscan_q[kRankWarps];
+  u64 want[2];                                  // walk: what is to be reached
   u64 fin_m[2];                                 // finish: mass before the range
   uint32_t slice_c[2][kMaxTeam];
-  uint32_t wscan_c[kRankWarps], wcnt[2][kRankWarps], inexact;
-  uint32_t few[2][kFewCap], few_n[2];
+  uint32_t wscan_c[kRankWarps], wcnt[2][kRankWarps];
+  uint32_t few_n[2];
   uint32_t fin_c[2], fin_lo[2], fin_in[2], fin_more[2];
   uint32_t list_n;                              // candidates of this block: visual | text << 16
-  uint32_t res[2][2];                           // selection: threshold, ties still wanted
-  __device__ uint32_t* all(int m) { return cnt + m * kListCap; }  // the team's candidates
-  __device__ uint32_t* fin_bucket(int m, int k) { return cnt + 2 * kListCap + (m * 3 + k) * kHalf; }
-  __device__ uint32_t* candidates(int m) { return TEAM > 1 ? all(m) : list[m]; }
+  __device__ uint32_t* fin_bucket(int m, int k) { return cnt + (m * 3 + k) * kHalf; }
+  __device__ uint32_t* few(int m) { return cnt + (6 + m) * kHalf; }
+  __device__ u64* few_mass(int m) { return reinterpret_cast<u64*>(cnt + (8 + 2 * m) * kHalf); }
+  static_assert((WORDS == 2 ? 12 : 8) * kHalf <= 2 * WORDS * kStride, "room for the finish");
 };
 
 // What is known of modality m's threshold: t lies in [lo, lo + span], `in` keys of the modality do, `above` keys lie
@@ -239,73 +337,264 @@ struct RankRange {
 };
 __device__ __forceinline__ int range_shift(uint32_t span, int dig) { return max(32 - __clz((int)span) - dig, 0); }
 
-__device__ __forceinline__ uint32_t map_bucket(uint32_t t) {
-  return (uint32_t)max(min((int)(t >> kMapShift) - kMapFirst, kBuckets - 1), 0);
-}
 // The range of t of bucket `at`, of the first layout or of one over g with 2^shift values of t per bucket.
-__device__ __forceinline__ void bucket_range(RankRange& g, bool first, uint32_t at, int shift) {
-  if (first) {
-    g.lo = at ? (kMapFirst + at) << kMapShift : 0u;
-    g.span = (at < kBuckets - 1 ? ((kMapFirst + at + 1) << kMapShift) - 1u : kTopKey) - g.lo;
+__device__ __forceinline__ void bucket_range(RankRange& g, const BucketMap* map, uint32_t at, int shift) {
+  if (map) {
+    const BucketStart s = bucket_start(*map, (int)at);
+    g.lo = at ? s.t : 0u;
+    g.span = (at < kBuckets - 1 ? s.t + (1u << s.shift) - 1u : kTopKey) - g.lo;
   } else {
     const uint32_t cut = at << shift;
     g.span = min(g.span - cut, (1u << shift) - 1u);
     g.lo += cut;
   }
 }
+// (Without a barrier: the caller has one before the buckets are used.)
 template <int TEAM, int WORDS>
 __device__ __forceinline__ void zero_buckets(RankShared<TEAM, WORDS>& sh) {
   for (int x = threadIdx.x; x < 2 * WORDS * RankShared<TEAM, WORDS>::kStride / 4; x += kRankThreads)
     reinterpret_cast<uint4*>(sh.cnt)[x] = make_uint4(0, 0, 0, 0);
   if (threadIdx.x == 0) sh.list_n = 0;
+}
+
+constexpr uint32_t kLowBias = 0x3b000000u;  // added to every term of a bucket's mass (low_mass() of allocate.cu)
+// The edges of neighbouring buckets: the largest score that the bucket can hold that starts at t, and its mass.
+__device__ __forceinline__ float edge_score(uint32_t t) { return __uint_as_float(kTopKey - min(t, kTopKey)); }
+__device__ __forceinline__ u64 edge_mass(float x) { return __float2ull_rz(x * 4294967296.0f); }
+// Mass of a bucket's c keys, all of at least the mass e1, from their sum modulo 2^32: c * e1 and a remainder, which is known
+// exactly if it is below 2^32.
+__device__ __forceinline__ uint32_t mass_rest(uint32_t c, uint32_t sum, u64 e1) { return sum - c * (kLowBias + (uint32_t)e1); }
+// It is if c scores between x1 and x (a little is left for the rounding).
+__device__ __forceinline__ bool mass_known(uint32_t c, float x, float x1) { return (float)c * (x - x1) < 0.999f; }
+
+// Walk of the buckets, filled in by all threads of the block: start(m, b) tells where bucket b of modality m starts,
+// need(m, mass) what is to be reached, a mass (WORDS = 2) or a count; 0: nothing. Leaves `found`, the same in every block
+// (but for `before`). Ends with a barrier of the block.
+template <int TEAM, int WORDS, typename Start, typename Need>
+__device__ __forceinline__ void walk(RankShared<TEAM, WORDS>& sh, uint32_t rank, Start start, Need need) {
+  constexpr bool kMass = WORDS == 2;
+  constexpr int kStride = RankShared<TEAM, WORDS>::kStride;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  __syncthreads();
+  {  // eight buckets per thread
+    const int m = tid / kHalf, i = tid % kHalf, b0 = i * 8;
+    const uint4* w = reinterpret_cast<const uint4*>(sh.cnt + m * kStride + b0);
+    const uint4 v0 = w[0], v1 = w[1];
+    uint32_t lc = ((v0.x + v0.y) + (v0.z + v0.w)) + ((v1.x + v1.y) + (v1.z + v1.w));
+    const uint32_t c[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+    u64 q[8] = {}, lq = 0;
+    bool bad = false;
+    if (kMass && lc) {  // (the buckets of most threads are empty)
+      const uint4 s0 = w[2 * kStride / 4], s1 = w[2 * kStride / 4 + 1];
+      const uint32_t s[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+      const BucketStart at = start(m, b0);
+      float x = edge_score(at.t);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const float x1 = b0 + k + 1 < kBuckets ? edge_score(at.t + ((uint32_t)(k + 1) << at.shift)) : 0.f;
+        const u64 e1 = edge_mass(x1);
+        q[k] = c[k] * e1 + mass_rest(c[k], s[k], e1);
+        lq += q[k];
+        bad = bad || (c[k] && !mass_known(c[k], x, x1));
+        x = x1;
+      }
+    }
+    const uint32_t bads = kMass ? __ballot_sync(kFull, bad) : 0u;
+    if (TEAM == 1) {  // a block on its own: every thread learns what lies before its buckets
+      uint32_t ic = warp_scan32(lc);
+      u64 iq = kMass ? warp_scan64(lq) : 0ull;
+      Found& f = sh.found[m];
+      if (lane == 31) {
+        sh.wscan_c[warp] = ic;
+        if (kMass) {
+          sh.wscan_q[warp] = iq;
+          sh.wcnt[0][warp] = bads;
+        }
+      }
+      __syncthreads();
+      if (i < 32) {  // a warp per modality: what lies before each of its warps, and what is needed
+        const bool here = lane / (kRankWarps / 2) == m;
+        const uint32_t wc = here ? sh.wscan_c[lane] : 0u, before_c = warp_scan32(wc) - wc;
+        const u64 wq = kMass && here ? sh.wscan_q[lane] : 0ull, before_q = kMass ? warp_scan64(wq) - wq : 0ull;
+        const uint32_t inexact = kMass ? __any_sync(kFull, lane < kRankWarps && sh.wcnt[0][lane]) : 0u;
+        if (here) {
+          sh.wscan_c[lane] = before_c;
+          if (kMass) sh.wscan_q[lane] = before_q;
+        }
+        if (lane == (m + 1) * (kRankWarps / 2) - 1) {
+          const u64 all = before_q + wq;
+          f.total = before_c + wc;
+          f.mass = all;
+          f.inexact = inexact;
+          f.hit = 0;
+          f.seg[0] = 0;
+          sh.want[m] = need(m, all);
+        }
+      }
+      __syncthreads();
+      ic += sh.wscan_c[warp];
+      if (kMass) iq += sh.wscan_q[warp];
+      const u64 want = sh.want[m];
+      if (want && (kMass ? iq - lq < want && iq >= want : ic - lc < want && ic >= want)) {
+        uint32_t run = ic - lc, at = 0, at_c = 0, at_in = 0;
+        u64 run_q = iq - lq, at_q = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          if (kMass ? run_q < want : run < want) {
+            at = b0 + k;
+            at_c = run;
+            at_in = c[k];
+            at_q = run_q;
+          }
+          run += c[k];
+          run_q += q[k];
+        }
+        f.hit = 1;
+        f.at = at;
+        f.above = at_c;
+        f.in = at_in;
+        f.above_q = at_q;
+      }
+      __syncthreads();
+      return;
+    }
+    // eight threads per coarse bucket
+#pragma unroll
+    for (int off = 1; off < 8; off <<= 1) {
+      lc += __shfl_xor_sync(kFull, lc, off);
+      if (kMass) lq += __shfl_xor_sync(kFull, lq, off);
+    }
+    if ((lane & 7) < TEAM)
+      peer_store<TEAM>(&sh.coarse[m][rank][i >> 3], lane & 7, make_uint4(lc, (uint32_t)lq, (uint32_t)(lq >> 32), (bads >> (lane & 24)) & 0xffu));
+  }
+  team_sync<TEAM>();
+  if (warp < 2) {
+    const int m = warp;
+    uint32_t c = 0, mine = 0, bad = 0;  // mine: of the blocks before this one
+    u64 q = 0;
+#pragma unroll
+    for (int r = 0; r < TEAM; ++r) {
+      const uint4 e = sh.coarse[m][r][lane];
+      c += e.x;
+      if (r < (int)rank) mine += e.x;
+      q += ((u64)e.z << 32) | e.y;
+      bad |= e.w;
+    }
+    const uint32_t ic = warp_scan32(c);
+    const u64 iq = kMass ? warp_scan64(q) : 0ull;
+    const u64 all_q = kMass ? __shfl_sync(kFull, iq, 31) : 0ull, want = need(m, all_q);
+    const uint32_t at_coarse = __ballot_sync(kFull, want && (kMass ? iq - q < want && iq >= want : ic - c < want && ic >= want));
+    Found& f = sh.found[m];
+    bad = kMass ? __any_sync(kFull, bad) : 0u;
+    if (lane == 31) {
+      f.total = ic;
+      f.mass = iq;
+      f.hit = at_coarse ? 1u : 0u;
+      f.inexact = bad;
+    }
+    if (!at_coarse) {
+      if (!kMass) {
+        mine = __reduce_add_sync(kFull, mine);
+        if (lane == 0) f.before = want ? mine : 0u;
+      }
+    } else {
+      const int who = __ffs((int)at_coarse) - 1, b = who * 64 + 2 * lane;
+      u64 pair[TEAM], sums[TEAM];
+      const uint32_t* w = sh.cnt + m * kStride + b;
+#pragma unroll
+      for (int r = 0; r < TEAM; ++r) {
+        pair[r] = peer_load<TEAM>(reinterpret_cast<const u64*>(w), r);
+        if (kMass) sums[r] = peer_load<TEAM>(reinterpret_cast<const u64*>(w + 2 * kStride), r);
+      }
+      u64 e1 = 0, e2 = 0;
+      if (kMass) {
+        const BucketStart at = start(m, b);
+        e1 = edge_mass(edge_score(at.t + (1u << at.shift)));
+        e2 = b + 2 < kBuckets ? edge_mass(edge_score(at.t + (2u << at.shift))) : 0ull;
+      }
+      uint32_t c0 = 0, c1 = 0, m0 = 0, m1 = 0;
+      u64 q0 = 0, q1 = 0;
+#pragma unroll
+      for (int r = 0; r < TEAM; ++r) {
+        const uint32_t x = (uint32_t)pair[r], y = (uint32_t)(pair[r] >> 32);
+        c0 += x;
+        c1 += y;
+        if (r < (int)rank) m0 += x, m1 += y;
+        if (kMass) {
+          q0 += mass_rest(x, (uint32_t)sums[r], e1);
+          q1 += mass_rest(y, (uint32_t)(sums[r] >> 32), e2);
+        }
+      }
+      if (kMass) {
+        q0 += c0 * e1;
+        q1 += c1 * e2;
+      }
+      const uint32_t run_c = __shfl_sync(kFull, ic - c, who) + warp_scan32(c0 + c1) - (c0 + c1);
+      const u64 run_q = kMass ? __shfl_sync(kFull, iq - q, who) + warp_scan64(q0 + q1) - (q0 + q1) : 0ull;
+      const uint32_t here = __ballot_sync(kFull, kMass ? run_q < want && run_q + q0 + q1 >= want : run_c < want && run_c + c0 + c1 >= want);
+      const int at = here ? __ffs((int)here) - 1 : 31;  // (none only where the masses are not exact)
+      const bool second = kMass ? run_q + q0 < want : run_c + c0 < want;
+      uint32_t before = 0;
+      if (!kMass)
+        before = __reduce_add_sync(kFull, (lane < who ? mine : 0u) + (lane < at ? m0 + m1 : 0u) + (lane == at && second ? m0 : 0u));
+      if (lane == at) {
+        f.at = b + (second ? 1 : 0);
+        f.above = run_c + (second ? c0 : 0u);
+        f.in = second ? c1 : c0;
+        f.above_q = run_q + (second ? q0 : 0ull);
+        f.before = before;
+        uint32_t place = 0;
+#pragma unroll
+        for (int r = 0; r < TEAM; ++r) {
+          f.seg[r] = place;
+          place += second ? (uint32_t)(pair[r] >> 32) : (uint32_t)pair[r];
+        }
+        f.seg[TEAM] = place;
+      }
+    }
+  }
   __syncthreads();
 }
 
-// This thread's words of the buckets, from word `at` on, added up over all blocks (the loads from distributed shared memory are
-// in flight together).
+// The places of the blocks' candidates in the list where no walk has told them (after exact sweeps): c0 and c1 are the
+// numbers in this thread's hands. Barriers of the team.
 template <int TEAM, int WORDS>
-__device__ __forceinline__ void bucket_counts(const RankShared<TEAM, WORDS>& sh, uint32_t at,
-                                              uint32_t (&c)[RankShared<TEAM, WORDS>::kPer]) {
-  constexpr int kPer = RankShared<TEAM, WORDS>::kPer;
-  const uint32_t* w = sh.cnt + at;
-  if (TEAM == 1) {
-#pragma unroll
-    for (int k = 0; k < kPer; k += 4) {
-      const uint4 v = *reinterpret_cast<const uint4*>(w + k);
-      c[k] = v.x;
-      c[(k + 1) % kPer] = v.y;
-      c[(k + 2) % kPer] = v.z;
-      c[(k + 3) % kPer] = v.w;
-    }
-  } else if (kPer == 1) {
-    uint32_t v[TEAM];
-#pragma unroll
-    for (int r = 0; r < TEAM; ++r) v[r] = peer_load<TEAM>(w, r);
-    c[0] = 0;
-#pragma unroll
-    for (int r = 0; r < TEAM; ++r) c[0] += v[r];
-  } else {
-    u64 v[TEAM][kPer / 2 + (kPer == 1)];
-#pragma unroll
-    for (int r = 0; r < TEAM; ++r)
-#pragma unroll
-      for (int k = 0; k < kPer / 2; ++k) v[r][k] = peer_load<TEAM>(reinterpret_cast<const u64*>(w) + k, r);
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) c[k] = 0;
-#pragma unroll
-    for (int r = 0; r < TEAM; ++r)
-#pragma unroll
-      for (int k = 0; k < kPer / 2; ++k) {
-        c[2 * k] += (uint32_t)v[r][k];
-        c[(2 * k + 1) % kPer] += (uint32_t)(v[r][k] >> 32);
-      }
+__device__ __forceinline__ void find_places(RankShared<TEAM, WORDS>& sh, uint32_t rank, uint32_t c0, uint32_t c1) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  c0 = __reduce_add_sync(kFull, c0);
+  c1 = __reduce_add_sync(kFull, c1);
+  __syncthreads();
+  if (lane == 0) {
+    sh.wcnt[0][warp] = c0;
+    sh.wcnt[1][warp] = c1;
   }
+  __syncthreads();
+  if (warp < 2) {
+    const uint32_t n = __reduce_add_sync(kFull, lane < kRankWarps ? sh.wcnt[warp][lane] : 0u);
+    if (lane < TEAM) peer_store<TEAM>(&sh.slice_c[warp][rank], lane, n);
+  }
+  team_sync<TEAM>();
+  if (threadIdx.x < 2) {
+    uint32_t place = 0;
+    for (int r = 0; r < TEAM; ++r) {
+      sh.found[threadIdx.x].seg[r] = place;
+      place += sh.slice_c[threadIdx.x][r];
+    }
+  }
+  __syncthreads();
 }
 
-// A warp's candidates into the block's lists, as offsets from lo0 / lo1: bit j of in0 / in1 is set where the thread's j-th
-// key belongs to the list of modality 0 / 1. One atomic per warp; candidates are few, so a thread picks them one by one.
-template <int TEAM, int WORDS, int KPT>
-__device__ __forceinline__ void append(RankShared<TEAM, WORDS>& sh, uint32_t in0, uint32_t in1, const uint32_t (&key)[KPT],
+// A candidate of modality m into the list, at place x: of block 0, or (kAll) of all blocks.
+template <int TEAM, int WORDS, bool kAll>
+__device__ __forceinline__ void put(RankShared<TEAM, WORDS>& sh, int m, uint32_t x, uint32_t v) {
+  uint32_t* at = &sh.list[m][x];
+#pragma unroll
+  for (int r = 0; r < (kAll ? TEAM : 1); ++r) peer_store<TEAM>(at, r, v);
+}
+// A warp's candidates into the list, as offsets from lo0 / lo1: bit j of in0 / in1 is set where the thread's j-th key belongs to
+// the list of modality 0 / 1. One atomic per warp; candidates are few, so a thread picks them one by one.
+template <int TEAM, int WORDS, int KPT, bool kAll>
+__device__ __forceinline__ void append(RankShared<TEAM, WORDS>& sh, uint32_t rank, uint32_t in0, uint32_t in1, const uint32_t (&key)[KPT],
                                        uint32_t lo0, uint32_t lo1) {
   if (!__any_sync(kFull, (in0 | in1) != 0)) return;
   const int lane = threadIdx.x & 31;
@@ -313,18 +602,19 @@ __device__ __forceinline__ void append(RankShared<TEAM, WORDS>& sh, uint32_t in0
   uint32_t base = 0;
   if (lane == 31) base = atomicAdd(&sh.list_n, incl);
   base = __shfl_sync(kFull, base, 31) + incl - mine;
-  uint32_t o0 = base & 0xffffu, o1 = base >> 16;
+  uint32_t o0 = (base & 0xffffu) + sh.found[0].seg[rank], o1 = (base >> 16) + sh.found[1].seg[rank];
   for (uint32_t left = in0 | in1; left; left &= left - 1) {
     const int j = __ffs(left) - 1;
     uint32_t k = key[0];
 #pragma unroll
     for (int x = 1; x < KPT; ++x) k = x == j ? key[x] : k;
-    if ((in0 >> j) & 1u) sh.list[0][o0++] = k - lo0;
-    else sh.list[1][o1++] = k - lo1;
+    const bool first = (in0 >> j) & 1u;
+    put<TEAM, WORDS, kAll>(sh, first ? 0 : 1, first ? o0++ : o1++, k - (first ? lo0 : lo1));
   }
 }
 
-// The same for a unit that is not in registers: positions instead of keys (the keys are read again when the list is complete).
+// The same for a unit that is not in registers: positions instead of keys, into lists of the block's own (the keys are read
+// again when those are complete).
 template <int TEAM, int WORDS>
 __device__ __forceinline__ void append_positions(RankShared<TEAM, WORDS>& sh, uint32_t* pos0, uint32_t* pos1, uint32_t in0, uint32_t in1, int at) {
   if (!__any_sync(kFull, (in0 | in1) != 0)) return;
@@ -338,142 +628,128 @@ __device__ __forceinline__ void append_positions(RankShared<TEAM, WORDS>& sh, ui
   for (; in1; in1 &= in1 - 1) pos1[o1++] = (uint32_t)(at + __ffs(in1) - 1);
 }
 
-// All blocks' candidates into this block (warp r copies block r's); returns their number, visual | text << 16. A block on
-// its own has them already. Ends with a barrier of the block.
-template <int TEAM, int WORDS>
-__device__ __forceinline__ uint32_t gather_lists(RankShared<TEAM, WORDS>& sh) {
-  if (TEAM == 1) return sh.list_n;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t n = lane < TEAM ? peer_load<TEAM>(&sh.list_n, lane) : 0u;
-  const uint32_t incl = warp_scan32(n), total = __shfl_sync(kFull, incl, 31);
-  if (warp < TEAM) {
-    const uint32_t k = __shfl_sync(kFull, n, warp), to = __shfl_sync(kFull, incl, warp) - k;
-#pragma unroll
-    for (int m = 0; m < 2; ++m) {
-      const uint32_t km = m ? k >> 16 : k & 0xffffu, at = m ? to >> 16 : to & 0xffffu;
-      for (uint32_t x = lane; x < km; x += 32) sh.all(m)[at + x] = peer_load<TEAM>(&sh.list[m][x], warp);
-    }
-  }
-  __syncthreads();
-  return total;
-}
-
-// The whole block: where among the candidates (offsets into rg[m]) the thresholds lie, half of the threads per modality. need: a
-// mass (with kMass; `before` is the exact mass before the range) or a count. Leaves in shared memory, per modality: fin_lo
-// (the smallest t up to which the threshold is reached), fin_c and fin_m (count and mass before it), fin_in (candidates
-// that equal it). A modality that is not `on` is left out. Ends with a barrier of the block.
+// The whole block: where among the candidates (offsets into the ranges; r0.in and r1.in of them) the thresholds lie, half of
+// the threads per modality. need: a mass (with kMass; `before` is the exact mass before the range) or a count. Leaves in
+// shared memory, per modality: fin_lo (the smallest t up to which the threshold is reached), fin_c and fin_m (count and mass
+// before it), fin_in (candidates that equal it). A modality that is not `on` is left out. The lists are complete behind a
+// barrier; ends with a barrier of the block.
 template <int TEAM, int WORDS, bool kMass>
-__device__ __forceinline__ void finish_lists(RankShared<TEAM, WORDS>& sh, const RankRange& r0, const RankRange& r1, uint32_t got, bool on0,
-                                             bool on1, u64 need0, u64 need1, u64 before0, u64 before1) {
+__device__ __forceinline__ void finish_lists(RankShared<TEAM, WORDS>& sh, const RankRange& r0, const RankRange& r1, bool on0, bool on1,
+                                             u64 need0, u64 need1, u64 before0, u64 before1) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, m = tid / kHalf, i = tid % kHalf;
-  const uint32_t n = m ? got >> 16 : got & 0xffffu, base = m ? r1.lo : r0.lo;
+  const uint32_t n = m ? r1.in : r0.in, base = m ? r1.lo : r0.lo;
   const bool on = m ? on1 : on0;
   const u64 need = m ? need1 : need0;
-  const uint32_t* list = sh.candidates(m);
-  uint32_t lo = 0, span = m ? r1.span : r0.span, in = n, above_c = m ? r1.above : r0.above;
+  const uint32_t* list = sh.list[m];
+  uint32_t in = n, above_c = m ? r1.above : r0.above;
   u64 above = m ? before1 : before0;
-  uint32_t *fc = sh.fin_bucket(m, 0), *flo = sh.fin_bucket(m, 1), *fhi = sh.fin_bucket(m, 2);
   auto mass = [&](uint32_t x) { return psi_fix(kTopKey - (base + x)); };
-  for (;;) {
-    const bool more = on && in > kFewCap && span > 0;
-    if (i == 0) {
-      sh.fin_more[m] = more ? 1u : 0u;
-      sh.few_n[m] = 0;
-    }
-    fc[i] = 0;
-    if (kMass) flo[i] = fhi[i] = 0;
-    __syncthreads();
-    if (!(sh.fin_more[0] | sh.fin_more[1])) break;
-    const int shift = range_shift(span, 8);
-    if (more) {
-      for (uint32_t x = i; x < n; x += kHalf) {
-        const uint32_t d = list[x] - lo;
-        if (d <= span) {
-          const uint32_t b = d >> shift;
-          atomicAdd(&fc[b], 1u);
-          if (kMass) {
-            const u64 q = mass(list[x]);
-            const uint32_t add = (uint32_t)q, old = atomicAdd(&flo[b], add);
-            const uint32_t hi = (uint32_t)(q >> 32) + ((uint32_t)(old + add) < old ? 1u : 0u);
-            if (hi) atomicAdd(&fhi[b], hi);
+  const bool many0 = on0 && r0.in > kFewCap && r0.span > 0, many1 = on1 && r1.in > kFewCap && r1.span > 0;
+  if (many0 || many1) {  // (the same in all threads)
+    uint32_t lo = 0, span = m ? r1.span : r0.span;
+    uint32_t *fc = sh.fin_bucket(m, 0), *flo = sh.fin_bucket(m, 1), *fhi = sh.fin_bucket(m, 2);
+    for (;;) {
+      const bool more = on && in > kFewCap && span > 0;
+      if (i == 0) {
+        sh.fin_more[m] = more ? 1u : 0u;
+        sh.few_n[m] = 0;
+      }
+      fc[i] = 0;
+      if (kMass) flo[i] = fhi[i] = 0;
+      __syncthreads();
+      if (!(sh.fin_more[0] | sh.fin_more[1])) break;
+      const int shift = range_shift(span, 8);
+      if (more) {
+        for (uint32_t x = i; x < n; x += kHalf) {
+          const uint32_t d = list[x] - lo;
+          if (d <= span) {
+            const uint32_t b = d >> shift;
+            atomicAdd(&fc[b], 1u);
+            if (kMass) {
+              const u64 q = mass(list[x]);
+              const uint32_t add = (uint32_t)q, old = atomicAdd(&flo[b], add);
+              const uint32_t hi = (uint32_t)(q >> 32) + ((uint32_t)(old + add) < old ? 1u : 0u);
+              if (hi) atomicAdd(&fhi[b], hi);
+            }
           }
         }
       }
+      __syncthreads();
+      const uint32_t c = fc[i];
+      uint32_t ic = warp_scan32(c);
+      u64 q = 0, iq = 0;
+      if (kMass) {
+        q = ((u64)fhi[i] << 32) | flo[i];
+        iq = warp_scan64(q);
+      }
+      if (lane == 31) {
+        sh.wscan_c[warp] = ic;
+        if (kMass) sh.wscan_q[warp] = iq;
+      }
+      __syncthreads();
+      const bool lower = lane >= m * (kRankWarps / 2) && lane < warp;
+      ic += above_c + __reduce_add_sync(kFull, lower ? sh.wscan_c[lane] : 0u);
+      if (kMass) iq += above + warp_sum64(lower ? sh.wscan_q[lane] : 0ull);
+      if (more && (kMass ? iq - q < need && iq >= need : ic - c < need && ic >= need)) {
+        sh.fin_lo[m] = i;
+        sh.fin_in[m] = c;
+        sh.fin_c[m] = ic - c;
+        if (kMass) sh.fin_m[m] = iq - q;
+      }
+      __syncthreads();
+      if (more) {
+        const uint32_t cut = sh.fin_lo[m] << shift;
+        lo += cut;
+        span = min(span - cut, (1u << shift) - 1u);
+        in = sh.fin_in[m];
+        above_c = sh.fin_c[m];
+        if (kMass) above = sh.fin_m[m];
+      }
     }
+    if (on)
+      for (uint32_t x = i; x < n; x += kHalf) {
+        const uint32_t v = list[x];
+        if (v - lo <= span) {
+          const uint32_t s = atomicAdd(&sh.few_n[m], 1u);
+          if (s < kFewCap) sh.few(m)[s] = v;  // (more than kFewCap are left only if all are alike)
+        }
+      }
     __syncthreads();
-    const uint32_t c = fc[i];
-    uint32_t ic = warp_scan32(c);
-    u64 q = 0, iq = 0;
-    if (kMass) {
-      q = ((u64)fhi[i] << 32) | flo[i];
-      iq = warp_scan64(q);
-    }
-    if (lane == 31) {
-      sh.wscan_c[warp] = ic;
-      if (kMass) sh.wscan_q[warp] = iq;
-    }
-    __syncthreads();
-    const bool lower = lane >= m * (kRankWarps / 2) && lane < warp;
-    ic += above_c + __reduce_add_sync(kFull, lower ? sh.wscan_c[lane] : 0u);
-    if (kMass) iq += above + warp_sum64(lower ? sh.wscan_q[lane] : 0ull);
-    if (more && (kMass ? iq - q < need && iq >= need : ic - c < need && ic >= need)) {
-      sh.fin_lo[m] = i;
-      sh.fin_in[m] = c;
-      sh.fin_c[m] = ic - c;
-      if (kMass) sh.fin_m[m] = iq - q;
-    }
-    __syncthreads();
-    if (more) {
-      const uint32_t cut = sh.fin_lo[m] << shift;
-      lo += cut;
-      span = min(span - cut, (1u << shift) - 1u);
-      in = sh.fin_in[m];
-      above_c = sh.fin_c[m];
-      if (kMass) above = sh.fin_m[m];
-    }
+    list = sh.few(m);
   }
-  // the keys left, compared with one another by one warp per modality
-  if (on && span > 0)
-    for (uint32_t x = i; x < n; x += kHalf) {
-      const uint32_t v = list[x];
-      if (v - lo <= span) {
-        const uint32_t s = atomicAdd(&sh.few_n[m], 1u);
-        if (s < kFewCap) {
-          sh.few[m][s] = v;
-          if (kMass) sh.few_m[m][s] = mass(v);
-        }
-      }
-    }
-  __syncthreads();
-  if (on && i < 32) {
-    uint32_t at = lo, equal = in;
-    if (span > 0) {
-      const uint32_t v = lane < (int)in ? sh.few[m][lane] : kNoKey;
-      uint32_t lt_c = 0, eq_c = 0;
-      u64 lt = 0, eq = 0;
+  // The keys left, compared with one another, 2^log threads per key. The threshold's keys are those that what is needed is
+  // reached with, but not before. (Keys that crowd are all alike: one of them is enough.)
+  const uint32_t k = !on ? 0u : in > kFewCap ? 1u : in;
+  if (kMass) {
+    if ((uint32_t)i < k) sh.few_mass(m)[i] = mass(list[i]);
+    __syncthreads();
+  }
+  const int log = min(__clz((int)k - 1) - 24, 2);  // kHalf >> log >= k
+  if (((uint32_t)i & ~31u) >> log < k) {  // (the other warps have no key)
+    const uint32_t x = (uint32_t)i >> log, part = (uint32_t)i & ((1u << log) - 1u), v = list[min(x, k - 1u)];
+    uint32_t lt_c = 0, eq_c = 0;
+    u64 lt = 0;
 #pragma unroll 4
-      for (uint32_t j = 0; j < in; ++j) {
-        const uint32_t o = sh.few[m][j];
-        if (o < v) ++lt_c;
-        if (o == v) ++eq_c;
-        if (kMass) {
-          const u64 q = sh.few_m[m][j];
-          if (o < v) lt += q;
-          if (o == v) eq += q;
-        }
+    for (uint32_t j = part; j < k; j += 1u << log) {
+      const uint32_t o = list[j];
+      if (o < v) {
+        ++lt_c;
+        if (kMass) lt += sh.few_mass(m)[j];
       }
-      const bool ok = lane < (int)in && (kMass ? above + lt + eq >= need : above_c + lt_c + eq_c >= need);
-      at = __reduce_min_sync(kFull, ok ? v : kNoKey);
-      const int who = max(__ffs(__ballot_sync(kFull, ok && v == at)) - 1, 0);
-      equal = __shfl_sync(kFull, eq_c, who);
-      above_c += __shfl_sync(kFull, lt_c, who);
-      if (kMass) above += __shfl_sync(kFull, lt, who);
+      if (o == v) ++eq_c;
     }
-    if (lane == 0) {
-      sh.fin_lo[m] = base + at;
-      sh.fin_in[m] = equal;
-      sh.fin_c[m] = above_c;
-      if (kMass) sh.fin_m[m] = above;
+    for (int off = 1; off < 1 << log; off <<= 1) {
+      lt_c += __shfl_xor_sync(kFull, lt_c, off);
+      eq_c += __shfl_xor_sync(kFull, eq_c, off);
+      if (kMass) lt += __shfl_xor_sync(kFull, lt, off);
+    }
+    if (k < in) eq_c = in;
+    const bool here = kMass ? above + lt < need && above + lt + eq_c * mass(v) >= need : above_c + lt_c < need && above_c + lt_c + eq_c >= need;
+    if (x < k && part == 0 && here) {  // (all that write write the same)
+      sh.fin_lo[m] = base + v;
+      sh.fin_in[m] = eq_c;
+      sh.fin_c[m] = above_c + lt_c;
+      if (kMass) sh.fin_m[m] = above + lt;
     }
   }
   __syncthreads();

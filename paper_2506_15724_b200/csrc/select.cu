@@ -1,6 +1,6 @@
 // Stage 4a: per-head, per-modality top-budget selection (Section 3.3, the eviction step after Eq. 8).
 //
-//   seg_scan     (batches only) one block: visual-token count of every sequence, kept_len[u] = b_v + b_t and the exclusive
+//   seg_scan     (large calls only) one block: visual-token count of every sequence, kept_len[u] = b_v + b_t and the exclusive
 //                scan seg_off (rows, with headroom)
 //   select_unit  a team of blocks per unit (rank_common.cuh) finds, for both modalities at once, the budget-th largest
 //                value and how many of its ties are still needed; an ordered sweep then emits the kept positions in
@@ -29,9 +29,37 @@ struct SelParams {
   int32_t* seq_nv;  // ws: visual-token count of every sequence
   int32_t* seq_wv;  // ws: visual tokens among the proxy tokens of every sequence (forced retention)
   int units, B, L, Hkv, n_max, mpa, headroom, keep_window, window, pool_r;  // pool_r: (pool_kernel - 1) / 2
+  int rows;   // window rows per KV head
   int words;  // of bits, per kind of bit and block (long kernels)
   int alone;  // no seg_scan before: every unit adds up the segments before its own
 };
+
+// Segment of a unit with these budgets: its visual and text tokens, those of them that are kept anyway.
+__device__ __forceinline__ int segment_length(const SelParams& p, int2 bud, int n, int n_v, int lo_v, int lo_t) {
+  return (p.mpa ? min(max(bud.x, lo_v), n_v) : 0) + min(max(bud.y, lo_t), n - n_v);
+}
+
+// A warp's part (of `parts`) of the visual tokens among the first n of a sequence (c), and of those from wfrom on (cw); sums of
+// the warp.
+__device__ __forceinline__ void count_tokens(const uint8_t* mask, int n, int wfrom, int part, int parts, int& c, int& cw) {
+  const int lane = threadIdx.x & 31;
+  c = cw = 0;
+  // whole 16-byte pieces of the row by vector loads, its ends by bytes
+  const int lead = min(n, (int)((16 - (reinterpret_cast<uintptr_t>(mask) & 15)) & 15));
+  const int n16 = (n - lead) >> 4;
+  for (int i = part * 32 + lane; i < n16; i += parts * 32) {
+    const uint4 v = __ldg(reinterpret_cast<const uint4*>(mask + lead) + i);
+    c += __popc(nonzero_bytes(v.x) | (nonzero_bytes(v.y) << 4) | (nonzero_bytes(v.z) << 8) | (nonzero_bytes(v.w) << 12));
+  }
+  if (part == 0) {
+    if (lane < lead) c += mask[lane] ? 1 : 0;
+    const int i = lead + (n16 << 4) + lane;
+    if (i < n) c += mask[i] ? 1 : 0;
+  }
+  for (int i = wfrom + part * 32 + lane; i < n; i += parts * 32) cw += mask[i] ? 1 : 0;  // (no proxy tokens: wfrom = n)
+  c = __reduce_add_sync(kFull, c);
+  cw = __reduce_add_sync(kFull, cw);
+}
 
 // One block. The visual tokens are counted by warps that share the sequences (several warps per sequence when there are
 // fewer sequences than warps), then the segments are scanned, 1024 units at a time.
@@ -53,23 +81,7 @@ __global__ void __launch_bounds__(1024) seg_scan_kernel(SelParams p) {
       const uint8_t* mask = p.mask + (int64_t)b * p.n_max;
       const int wfrom = p.keep_window ? max(n - p.window, 0) : n;  // first proxy token retained unconditionally
       int c = 0, cw = 0;                                           // visual tokens, visual proxy tokens
-      if (p.mpa) {
-        // whole 16-byte pieces of the row by vector loads, its ends by bytes
-        const int lead = min(n, (int)((16 - (reinterpret_cast<uintptr_t>(mask) & 15)) & 15));
-        const int n16 = (n - lead) >> 4;
-        for (int i = part * 32 + lane; i < n16; i += share * 32) {
-          const uint4 v = __ldg(reinterpret_cast<const uint4*>(mask + lead) + i);
-          c += __popc(nonzero_bytes(v.x) | (nonzero_bytes(v.y) << 4) | (nonzero_bytes(v.z) << 8) | (nonzero_bytes(v.w) << 12));
-        }
-        if (part == 0) {
-          if (lane < lead) c += mask[lane] ? 1 : 0;
-          const int i = lead + (n16 << 4) + lane;
-          if (i < n) c += mask[i] ? 1 : 0;
-        }
-        for (int i = wfrom + part * 32 + lane; i < n; i += share * 32) cw += mask[i] ? 1 : 0;  // (no proxy tokens: wfrom = n)
-      }
-      c = __reduce_add_sync(kFull, c);
-      cw = __reduce_add_sync(kFull, cw);
+      if (p.mpa) count_tokens(mask, n, wfrom, part, share, c, cw);
       if (lane == 0 && c) atomicAdd(&s_cnt[slot], c);
       if (lane == 0 && cw) atomicAdd(&s_wcnt[slot], cw);
     }
@@ -90,7 +102,7 @@ __global__ void __launch_bounds__(1024) seg_scan_kernel(SelParams p) {
       const int n = clamped_len(p.seq_len, b, p.n_max);
       const int n_v = p.seq_nv[b];
       const int lo_v = p.seq_wv[b], lo_t = (p.keep_window ? min(p.window, n) : 0) - lo_v;  // proxy tokens kept anyway
-      const int len = (p.mpa ? min(max(p.budgets[2 * u], lo_v), n_v) : 0) + min(max(p.budgets[2 * u + 1], lo_t), n - n_v);
+      const int len = segment_length(p, make_int2(p.budgets[2 * u], p.budgets[2 * u + 1]), n, n_v, lo_v, lo_t);
       p.kept_len[u] = len;
       v = (long long)len + p.headroom;
     }
@@ -148,6 +160,12 @@ __device__ __forceinline__ void load_pooled(const float* row, int mis, int n, in
   }
 }
 
+// What a call without seg_scan knows of the sequences before a block's own: their visual tokens, all and among the proxy tokens.
+constexpr int kAloneSeqs = 64, kAloneTokens = 65536;
+struct SeqCounts {
+  int nv[kAloneSeqs], wv[kAloneSeqs];
+};
+
 // A unit of a block, and what is wanted of it.
 template <bool kPool>
 struct SelUnit {
@@ -155,12 +173,22 @@ struct SelUnit {
   const uint8_t* mask;
   int u, b, mis, n, wfrom, lo_v, lo_t;
   uint32_t want0, want1;
+  int2 bud;         // the unit's budgets
+  int2 before_bud;  // p.alone: budgets of unit threadIdx.x, if that comes before this one, its sequence and that one's length
+  int before_b, before_n;
   __device__ __forceinline__ SelUnit(const SelParams& p, int unit) {
     u = unit;
     b = u / (p.Hkv * p.L);
     psi = p.psi + (int64_t)u * p.n_max;
     mis = (int)(((int64_t)u * p.n_max) & 3);
     mask = p.mask + (int64_t)b * p.n_max;
+  }
+  __device__ __forceinline__ void set_up(const SelParams& p) {
+    if (p.alone && (int)threadIdx.x < u) {
+      before_b = threadIdx.x / (p.Hkv * p.L);
+      before_bud = __ldg(reinterpret_cast<const int2*>(p.budgets) + threadIdx.x);
+      before_n = clamped_len(p.seq_len, before_b, p.n_max);
+    }
     n = clamped_len(p.seq_len, b, p.n_max);
     // proxy tokens retained unconditionally (none without cfg->keep_window): they are emitted by the sweep and the
     // ranking only has to find the rest of each modality's budget
@@ -172,14 +200,35 @@ struct SelUnit {
       for (int x = wfrom; x < n; x += kRankThreads)
         lo_v += __syncthreads_count(x + (int)threadIdx.x < n && mask[x + threadIdx.x] != 0);
     lo_t = (n - wfrom) - lo_v;
-    want0 = (uint32_t)(p.mpa ? max(p.budgets[2 * u] - lo_v, 0) : 0);
-    want1 = (uint32_t)max(p.budgets[2 * u + 1] - lo_t, 0);
+    bud = __ldg(reinterpret_cast<const int2*>(p.budgets) + u);
+    want0 = (uint32_t)(p.mpa ? max(bud.x - lo_v, 0) : 0);
+    want1 = (uint32_t)max(bud.y - lo_t, 0);
+  }
+  // p.alone: the tokens of the sequences before this one (behind a barrier after the counts were cleared)
+  __device__ __forceinline__ void count_before(const SelParams& p, SeqCounts& s) const {
+    if (!p.mpa) return;
+    const int warp = threadIdx.x >> 5, parts = max(1, kRankWarps / b);
+    for (int x = warp; x < b * parts; x += kRankWarps) {
+      const int b2 = x / parts, n2 = clamped_len(p.seq_len, b2, p.n_max);
+      int c, cw;
+      count_tokens(p.mask + (int64_t)b2 * p.n_max, n2, p.keep_window ? max(n2 - p.window, 0) : n2, x % parts, parts, c, cw);
+      if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&s.nv[b2], c);
+        atomicAdd(&s.wv[b2], cw);
+      }
+    }
   }
   // t of KPT consecutive positions; returns those that are ranked, `forced`: those that are kept without
   template <int KPT>
   __device__ __forceinline__ uint32_t load(const SelParams& p, int pos0, uint32_t (&t)[KPT], uint32_t& forced) const {
+    RawScores<KPT> raw;
+    if (!kPool) issue_scores<KPT>(psi, mis, p.n_max, pos0, raw);
+    return take(p, raw, pos0, t, forced);
+  }
+  template <int KPT>  // (raw: not used with pooling, which does not know its neighbours' bounds before the length)
+  __device__ __forceinline__ uint32_t take(const SelParams& p, const RawScores<KPT>& raw, int pos0, uint32_t (&t)[KPT], uint32_t& forced) const {
     if (kPool) load_pooled<KPT>(psi, mis, n, pos0, p.pool_r, t);
-    else load_scores<KPT>(psi, mis, p.n_max, pos0, t);
+    else take_scores<KPT>(raw, mis, t);
     uint32_t valid = valid_bits<KPT>(n, pos0);
     forced = 0;
     if (kPool) {
@@ -202,28 +251,30 @@ struct SelUnit {
 };
 
 // The ranges the two thresholds can lie in. short: the modality has no more keys than are wanted, all of them are kept.
+template <int CAP>  // candidates that fit the list
 struct SelRanges {
   RankRange r0, r1;
   bool short0, short1;
-  uint32_t n_vis;  // visual tokens in the ranking
-  __device__ __forceinline__ bool crowded0() const { return r0.in > kListCap && r0.span > 0; }
-  __device__ __forceinline__ bool crowded1() const { return r1.in > kListCap && r1.span > 0; }
+  uint32_t n_vis;   // visual tokens in the ranking
+  uint32_t before;  // keys before their ranges in the blocks before this one
+  __device__ __forceinline__ bool crowded0() const { return r0.in > CAP && r0.span > 0; }
+  __device__ __forceinline__ bool crowded1() const { return r1.in > CAP && r1.span > 0; }
 };
 
 template <int KPT, int TEAM>
-__device__ __forceinline__ void count_first(RankShared<TEAM, 1>& sh, const uint32_t (&t)[KPT], uint32_t vis, uint32_t valid) {
+__device__ __forceinline__ void count_first(RankShared<TEAM, 1>& sh, const BucketMap& map, const uint32_t (&t)[KPT], uint32_t vis, uint32_t valid) {
   constexpr int kStride = RankShared<TEAM, 1>::kStride;
   if (valid == valid_bits<KPT>(KPT, 0)) {
 #pragma unroll
-    for (int j = 0; j < KPT; ++j) atomicAdd(sh.cnt + ((vis >> j) & 1u ? 0 : kStride) + map_bucket(t[j]), 1u);
+    for (int j = 0; j < KPT; ++j) atomicAdd(sh.cnt + ((vis >> j) & 1u ? 0 : kStride) + map_bucket(map, t[j]), 1u);
   } else {
 #pragma unroll
     for (int j = 0; j < KPT; ++j)
-      if ((valid >> j) & 1u) atomicAdd(sh.cnt + ((vis >> j) & 1u ? 0 : kStride) + map_bucket(t[j]), 1u);
+      if ((valid >> j) & 1u) atomicAdd(sh.cnt + ((vis >> j) & 1u ? 0 : kStride) + map_bucket(map, t[j]), 1u);
   }
 }
 template <int KPT, int TEAM>
-__device__ __forceinline__ void count_again(RankShared<TEAM, 1>& sh, const SelRanges& g, const uint32_t (&t)[KPT], uint32_t vis, int shift0, int shift1) {
+__device__ __forceinline__ void count_again(RankShared<TEAM, 1>& sh, const SelRanges<RankShared<TEAM, 1>::kCap>& g, const uint32_t (&t)[KPT], uint32_t vis, int shift0, int shift1) {
 #pragma unroll
   for (int j = 0; j < KPT; ++j) {
     const bool v = (vis >> j) & 1u;
@@ -232,72 +283,35 @@ __device__ __forceinline__ void count_again(RankShared<TEAM, 1>& sh, const SelRa
   }
 }
 
-// Walk of the buckets: block r of the team adds up its share of the buckets over all blocks, half of the threads per modality;
-// the ranges shrink to the buckets with the wanted keys.
+// Walk of the buckets (of the first layout, `map`, or of one over the ranges): the ranges shrink to the buckets with the wanted
+// keys.
 template <int TEAM>
-__device__ __forceinline__ void select_walk(RankShared<TEAM, 1>& sh, uint32_t rank, bool first, uint32_t want0, uint32_t want1, SelRanges& g,
-                                            int shift0, int shift1) {
-  using SH = RankShared<TEAM, 1>;
-  constexpr int kPer = SH::kPer;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, m = tid / kHalf, i = tid % kHalf;
-  const uint32_t b0 = (rank * kHalf + i) * kPer;
-  const uint32_t want = m ? want1 : want0;
-  if (i == 0) sh.first[m] = ~0ull;  // (stays if the modality has fewer keys than wanted)
-  team_sync<TEAM>();
-  uint32_t c[kPer], lc = 0;
-  bucket_counts<TEAM, 1>(sh, m * SH::kStride + b0, c);
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) lc += c[k];
-  uint32_t ic = warp_scan32(lc);
-  if (lane == 31) sh.wscan_c[warp] = ic;
-  __syncthreads();
-  ic += __reduce_add_sync(kFull, lane >= m * (kRankWarps / 2) && lane < warp ? sh.wscan_c[lane] : 0u);
-  if (i >= kHalf - 32) {  // the last warp of the modality has the block's total (in its last lane): to every block
-    const uint32_t tc = __shfl_sync(kFull, ic, 31);
-    if (lane < TEAM) peer_store<TEAM>(&sh.slice_c[m][rank], lane, tc);
-  }
-  if (TEAM > 1) {
-    team_sync<TEAM>();
-    ic += __reduce_add_sync(kFull, lane < (int)rank ? sh.slice_c[m][lane] : 0u);
-  }
-  ic += m ? g.r1.above : g.r0.above;
-  if (want && ic - lc < want && ic >= want) {
-    uint32_t run = ic - lc, at = 0, at_c = 0, at_in = 0;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-      if (run < want) {
-        at = b0 + k;
-        at_c = run;
-        at_in = c[k];
-      }
-      run += c[k];
-    }
-#pragma unroll
-    for (int r = 0; r < TEAM; ++r) {
-      peer_store<TEAM>(&sh.first[m], r, ((u64)at_c << 32) | at);
-      peer_store<TEAM>(&sh.last[m], r, (u64)at_in);
-    }
-  }
-  team_sync<TEAM>();
-  if (first) g.n_vis = __reduce_add_sync(kFull, lane < TEAM ? sh.slice_c[0][lane] : 0u);
-  auto narrow = [&](RankRange& r, bool& is_short, int q, int s) {
-    if (sh.first[q] == ~0ull) {
+__device__ __forceinline__ void select_walk(RankShared<TEAM, 1>& sh, uint32_t rank, const BucketMap* map, uint32_t want0, uint32_t want1,
+                                            SelRanges<RankShared<TEAM, 1>::kCap>& g, int shift0, int shift1) {
+  walk<TEAM, 1>(
+      sh, rank, [](int, int) { return BucketStart{0u, 0}; },
+      [&](int m, u64) -> u64 { return m ? (g.short1 || !want1 ? 0u : want1 - g.r1.above) : (g.short0 || !want0 ? 0u : want0 - g.r0.above); });
+  if (map) g.n_vis = sh.found[0].total;
+  auto narrow = [&](RankRange& r, bool& is_short, const Found& f, int shift) {
+    if (TEAM > 1) g.before += f.before;
+    if (!f.hit) {  // the modality has no more keys than wanted
       is_short = true;
       r = RankRange{kNowhere, 0u, 0u, 0u};
       return;
     }
-    bucket_range(r, first, (uint32_t)sh.first[q], s);
-    r.above = (uint32_t)(sh.first[q] >> 32);
-    r.in = (uint32_t)sh.last[q];
+    bucket_range(r, map, f.at, shift);
+    r.above += f.above;
+    r.in = f.in;
   };
-  if (want0 && !g.short0) narrow(g.r0, g.short0, 0, shift0);
-  if (want1 && !g.short1) narrow(g.r1, g.short1, 1, shift1);
+  if (want0 && !g.short0) narrow(g.r0, g.short0, sh.found[0], shift0);
+  if (want1 && !g.short1) narrow(g.r1, g.short1, sh.found[1], shift1);
 }
 
 // (Rare) too many keys in a range: halve it with exact sweeps until they fit the list or are all alike. `sweep` calls its
 // argument with the keys of the thread, some at a time.
 template <int TEAM, typename Sweep>
-__device__ __forceinline__ void select_bisect(RankShared<TEAM, 1>& sh, uint32_t want0, uint32_t want1, SelRanges& g, Sweep sweep) {
+__device__ __forceinline__ void select_bisect(RankShared<TEAM, 1>& sh, uint32_t want0, uint32_t want1,
+                                              SelRanges<RankShared<TEAM, 1>::kCap>& g, Sweep sweep) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   while (g.crowded0() || g.crowded1()) {
     const bool on0 = g.crowded0(), on1 = g.crowded1();
@@ -348,11 +362,12 @@ struct Thresholds {
   uint32_t thr0, thr1, ties0, ties1;
 };
 template <int TEAM>
-__device__ __forceinline__ Thresholds select_thresholds(RankShared<TEAM, 1>& sh, uint32_t want0, uint32_t want1, const SelRanges& g) {
-  team_sync<TEAM>();
-  const uint32_t got = gather_lists<TEAM, 1>(sh);
-  const bool on0 = want0 && !g.short0 && g.r0.in <= kListCap, on1 = want1 && !g.short1 && g.r1.in <= kListCap;
-  finish_lists<TEAM, 1, false>(sh, g.r0, g.r1, got, on0, on1, want0, want1, 0ull, 0ull);
+__device__ __forceinline__ Thresholds select_thresholds(RankShared<TEAM, 1>& sh, uint32_t want0, uint32_t want1,
+                                                        const SelRanges<RankShared<TEAM, 1>::kCap>& g) {
+  constexpr uint32_t kCap = RankShared<TEAM, 1>::kCap;
+  team_sync<TEAM>();  // (the last access to another block's shared memory)
+  const bool on0 = want0 && !g.short0 && g.r0.in <= kCap, on1 = want1 && !g.short1 && g.r1.in <= kCap;
+  finish_lists<TEAM, 1, false>(sh, g.r0, g.r1, on0, on1, want0, want1, 0ull, 0ull);
   Thresholds h;
   h.thr0 = !want0 ? 0u : (g.short0 ? kNowhere : (on0 ? sh.fin_lo[0] : g.r0.lo));
   h.thr1 = !want1 ? 0u : (g.short1 ? kNowhere : (on1 ? sh.fin_lo[1] : g.r1.lo));
@@ -366,19 +381,43 @@ __device__ __forceinline__ Thresholds select_thresholds(RankShared<TEAM, 1>& sh,
 __device__ __forceinline__ u64 emit_counts(uint32_t gt, uint32_t eq, uint32_t vis) {
   return (u64)__popc(eq & vis) | ((u64)__popc(eq & ~vis) << 21) | ((u64)__popc(gt) << 42);
 }
+// The blocks before this one: their keys before the ranges are known from the walk, those of them in the ranges from the list,
+// where every block's keys have places of their own. After exact sweeps (`swept`) the blocks exchange their totals instead.
 template <int TEAM>
-__device__ __forceinline__ u64 counts_before(RankShared<TEAM, 1>& sh, uint32_t rank, u64 mine) {
+__device__ __forceinline__ u64 counts_before(RankShared<TEAM, 1>& sh, uint32_t rank, u64 mine, const Thresholds& h, uint32_t want0, uint32_t want1,
+                                             const SelRanges<RankShared<TEAM, 1>::kCap>& g, uint32_t forced_before, bool swept) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const u64 incl = warp_scan64(mine);
   if (lane == 31) sh.wscan_q[warp] = incl;
-  __syncthreads();
   u64 before = 0;
-  if (TEAM > 1) {
+  if (TEAM > 1 && !swept) {
+    const int m = threadIdx.x / kHalf;
+    const RankRange r = m ? g.r1 : g.r0;
+    const bool ranked = m ? want1 && !g.short1 : want0 && !g.short0;
+    const uint32_t thr = m ? h.thr1 : h.thr0, mine_n = ranked ? sh.found[m].seg[rank] : 0u;
+    uint32_t lt = 0, eq = 0;
+    if (r.in <= RankShared<TEAM, 1>::kCap) {
+      for (uint32_t x = threadIdx.x % kHalf; x < mine_n; x += kHalf) {
+        const uint32_t v = r.lo + sh.list[m][x];
+        lt += v < thr ? 1u : 0u;
+        eq += v == thr ? 1u : 0u;
+      }
+    } else if (threadIdx.x % kHalf == 0) {  // all keys of the range are alike
+      eq = mine_n;
+    }
+    lt = __reduce_add_sync(kFull, lt);
+    eq = __reduce_add_sync(kFull, eq);
+    if (lane == 0) sh.wsum[0][warp] = ((u64)eq << (m ? 21 : 0)) | ((u64)lt << 42);
+  }
+  __syncthreads();
+  if (TEAM > 1 && !swept) {
+    before = warp_sum64(lane < kRankWarps ? sh.wsum[0][lane] : 0ull) + ((u64)(g.before + forced_before) << 42);
+  } else if (TEAM > 1) {
     if (warp == 0) {
       const u64 tot = warp_sum64(lane < kRankWarps ? sh.wscan_q[lane] : 0ull);
       if (lane < TEAM) peer_store<TEAM>(&sh.slice_q[0][rank], lane, tot);
     }
-    team_sync<TEAM>();  // (also the last access to a peer's shared memory)
+    team_sync<TEAM>();
     before = warp_sum64(lane < (int)rank ? sh.slice_q[0][lane] : 0ull);
   }
   return before + incl - mine + warp_sum64(lane < warp ? sh.wscan_q[lane] : 0ull);
@@ -386,24 +425,25 @@ __device__ __forceinline__ u64 counts_before(RankShared<TEAM, 1>& sh, uint32_t r
 
 // Where the unit's segment starts; -1: the cache is too small.
 template <int TEAM, bool kPool>
-__device__ __forceinline__ int64_t segment_start(RankShared<TEAM, 1>& sh, const SelParams& p, const SelUnit<kPool>& x, uint32_t rank, uint32_t n_vis) {
+__device__ __forceinline__ int64_t segment_start(RankShared<TEAM, 1>& sh, const SeqCounts& s, const SelParams& p, const SelUnit<kPool>& x,
+                                                 uint32_t rank, uint32_t n_vis) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (p.alone) {
-    // one sequence: the segments' lengths follow from the budgets and the modalities' token counts, which are at hand
-    pdl_go();
+    // the segments' lengths follow from the budgets and the modalities' token counts, which are at hand
     const int n_v = (int)n_vis + x.lo_v;
-    auto length = [&](int i) {
-      const int2 bud = __ldg(reinterpret_cast<const int2*>(p.budgets) + i);
-      return (p.mpa ? min(max(bud.x, x.lo_v), n_v) : 0) + min(max(bud.y, x.lo_t), x.n - n_v);
-    };
     u64 sum = 0;
-    for (int i = tid; i < x.u; i += kRankThreads) sum += (u64)(length(i) + p.headroom);
+    if (tid < x.u) {
+      const bool own = x.before_b == x.b;
+      const int nv = own ? n_v : s.nv[x.before_b], lv = own ? x.lo_v : s.wv[x.before_b];
+      const int lt = (kPool && p.keep_window ? min(p.window, x.before_n) : 0) - lv;
+      sum = (u64)(segment_length(p, x.before_bud, x.before_n, nv, lv, lt) + p.headroom);
+    }
     sum = warp_sum64(sum);
     __syncthreads();
-    if (lane == 0) sh.wsum[0][warp] = sum;
+    if (lane == 0) sh.wsum[1][warp] = sum;
     __syncthreads();
-    const int64_t off = (int64_t)warp_sum64(lane < kRankWarps ? sh.wsum[0][lane] : 0ull);
-    const int len = length(x.u);
+    const int64_t off = (int64_t)warp_sum64(lane < kRankWarps ? sh.wsum[1][lane] : 0ull);
+    const int len = segment_length(p, x.bud, x.n, n_v, x.lo_v, x.lo_t);
     const int64_t end = off + len + p.headroom;
     if (rank == 0 && tid == 0) {
       p.kept_len[x.u] = len;
@@ -445,30 +485,52 @@ __device__ __forceinline__ void emit(int32_t* seg, const Thresholds& h, int pos0
 
 // A unit whose keys fit the registers of its team.
 template <int KPT, int TEAM, bool kPool>
-__global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(SelParams p) {
+__global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(const __grid_constant__ SelParams p) {
+  constexpr uint32_t kCap = RankShared<TEAM, 1>::kCap;
   __shared__ RankShared<TEAM, 1> sh;
+  __shared__ SeqCounts s;
+  team_started<TEAM>();
+  if (TEAM > 1) zero_buckets<TEAM, 1>(sh);
+  if (threadIdx.x < kAloneSeqs) s.nv[threadIdx.x] = s.wv[threadIdx.x] = 0;
   // (no wait here after seg_scan: it has waited for everything before it, so the scores, the mask and the budgets are final;
   // what seg_scan itself writes is read after the wait of segment_start)
-  if (p.alone) pdl_wait();
+  if (p.alone) {
+    pdl_wait();
+    pdl_go();
+  }
   const uint32_t rank = TEAM > 1 ? team_rank() : 0u;
-  const SelUnit<kPool> x(p, blockIdx.x / TEAM);
+  SelUnit<kPool> x(p, blockIdx.x / TEAM);
   const int pos0 = (int)rank * kRankThreads * KPT + threadIdx.x * KPT;  // a block owns consecutive positions
+  RawScores<KPT> raw;
+  RawMask<KPT> raw_mask;
+  if (!kPool) issue_scores<KPT>(x.psi, x.mis, p.n_max, pos0, raw);
+  if (p.mpa) issue_mask<KPT>(x.mask, p.n_max, pos0, raw_mask);
+  if (TEAM == 1) zero_buckets<TEAM, 1>(sh);
+  x.set_up(p);
   uint32_t t[KPT], forced;
-  const uint32_t valid = x.template load<KPT>(p, pos0, t, forced);
-  const uint32_t vis = p.mpa ? load_mask<KPT>(x.mask, p.n_max, pos0) : 0u;
-  zero_buckets<TEAM, 1>(sh);
-  count_first<KPT, TEAM>(sh, t, vis, valid);
-  SelRanges g{{kNowhere, 0u, 0u, 0u}, {kNowhere, 0u, 0u, 0u}, false, false, 0u};
-  select_walk<TEAM>(sh, rank, true, x.want0, x.want1, g, 0, 0);
+  const uint32_t valid = x.template take<KPT>(p, raw, pos0, t, forced), vis = p.mpa ? take_mask<KPT>(raw_mask) : 0u;
+  const BucketMap map = bucket_map(p.rows, x.n);
+  __syncthreads();
+  if (p.alone && x.b > 0) x.count_before(p, s);
+  count_first<KPT, TEAM>(sh, map, t, vis, valid);
+  SelRanges<kCap> g{{kNowhere, 0u, 0u, 0u}, {kNowhere, 0u, 0u, 0u}, false, false, 0u, 0u};
+  team_wait_started<TEAM>();
+  select_walk<TEAM>(sh, rank, &map, x.want0, x.want1, g, 0, 0);
+  bool swept = false;
   if (g.crowded0() || g.crowded1()) {
     const int shift0 = range_shift(g.r0.span, kDig), shift1 = range_shift(g.r1.span, kDig);
+    team_sync<TEAM>();
     zero_buckets<TEAM, 1>(sh);
+    __syncthreads();
     count_again<KPT, TEAM>(sh, g, t, vis, shift0, shift1);
-    select_walk<TEAM>(sh, rank, false, x.want0, x.want1, g, shift0, shift1);
-    select_bisect<TEAM>(sh, x.want0, x.want1, g, [&](auto each) {
+    select_walk<TEAM>(sh, rank, nullptr, x.want0, x.want1, g, shift0, shift1);
+    if (g.crowded0() || g.crowded1()) {
+      select_bisect<TEAM>(sh, x.want0, x.want1, g, [&](auto each) {
 #pragma unroll
-      for (int j = 0; j < KPT; ++j) each(t[j], (vis >> j) & 1u);
-    });
+        for (int j = 0; j < KPT; ++j) each(t[j], (vis >> j) & 1u);
+      });
+      swept = true;
+    }
   }
   uint32_t in = 0;
 #pragma unroll
@@ -476,7 +538,9 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(SelParams 
     const bool v = (vis >> j) & 1u;
     if (t[j] - (v ? g.r0.lo : g.r1.lo) <= (v ? g.r0.span : g.r1.span)) in |= 1u << j;
   }
-  append<TEAM, 1, KPT>(sh, g.r0.in <= kListCap ? in & vis : 0u, g.r1.in <= kListCap ? in & ~vis : 0u, t, g.r0.lo, g.r1.lo);
+  const uint32_t in0 = g.r0.in <= kCap ? in & vis : 0u, in1 = g.r1.in <= kCap ? in & ~vis : 0u;
+  if (swept) find_places<TEAM, 1>(sh, rank, __popc(in0), __popc(in1));
+  append<TEAM, 1, KPT, true>(sh, rank, in0, in1, t, g.r0.lo, g.r1.lo);
   const Thresholds h = select_thresholds<TEAM>(sh, x.want0, x.want1, g);
   uint32_t eq = 0, gt = 0;
 #pragma unroll
@@ -486,8 +550,9 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(SelParams 
     if (t[j] < thr) gt |= 1u << j;
   }
   if (kPool) gt |= forced;
-  const u64 ahead = counts_before<TEAM>(sh, rank, emit_counts(gt, eq, vis));
-  const int64_t off = segment_start<TEAM, kPool>(sh, p, x, rank, g.n_vis);
+  const uint32_t forced_before = kPool ? (uint32_t)max(min((int)rank * kRankThreads * KPT, x.n) - x.wfrom, 0) : 0u;
+  const u64 ahead = counts_before<TEAM>(sh, rank, emit_counts(gt, eq, vis), h, x.want0, x.want1, g, forced_before, swept);
+  const int64_t off = segment_start<TEAM, kPool>(sh, s, p, x, rank, g.n_vis);
   if (off >= 0) emit(p.kept_idx + off, h, pos0, ahead, gt, eq, vis);
 }
 
@@ -496,14 +561,23 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(SelParams 
 // thresholds are known their bits are put right, so that the positions are emitted from the bits. (With every sweep over the
 // keys themselves, range, buckets, candidates and emission, 256 units of 131072 keys took 187 us instead of 110.)
 template <int TEAM, bool kPool>
-__global__ void __launch_bounds__(kRankThreads, 2) select_long_kernel(SelParams p) {
+__global__ void __launch_bounds__(kRankThreads, 2) select_long_kernel(const __grid_constant__ SelParams p) {
   constexpr int KPT = 16, kRound = kRankThreads * KPT;
+  constexpr uint32_t kCap = RankShared<TEAM, 1>::kCap;
   __shared__ RankShared<TEAM, 1> sh;
+  __shared__ SeqCounts s;
   extern __shared__ __align__(16) uint32_t bits[];
-  if (p.alone) pdl_wait();
+  team_started<TEAM>();
+  zero_buckets<TEAM, 1>(sh);
+  if (threadIdx.x < kAloneSeqs) s.nv[threadIdx.x] = s.wv[threadIdx.x] = 0;
+  if (p.alone) {
+    pdl_wait();
+    pdl_go();
+  }
   const uint32_t rank = TEAM > 1 ? team_rank() : 0u;
   const int tid = threadIdx.x;
-  const SelUnit<kPool> x(p, blockIdx.x / TEAM);
+  SelUnit<kPool> x(p, blockIdx.x / TEAM);
+  x.set_up(p);
   uint32_t* cand_pos[2] = {bits, bits + kListCap};
   uint32_t* vis_w = bits + 2 * kListCap;
   uint32_t* keep_w = vis_w + p.words;
@@ -511,7 +585,9 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_long_kernel(SelParams 
   const int rounds = (x.n + kRound * TEAM - 1) / (kRound * TEAM);
   const int start = (int)rank * rounds * kRound;  // a block owns consecutive positions
 
-  zero_buckets<TEAM, 1>(sh);
+  const BucketMap map = bucket_map(p.rows, x.n);
+  __syncthreads();
+  if (p.alone && x.b > 0) x.count_before(p, s);
 #pragma unroll 1
   for (int r = 0; r < rounds; ++r) {
     const int pos0 = start + r * kRound + tid * KPT;
@@ -519,36 +595,43 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_long_kernel(SelParams 
     const uint32_t valid = x.template load<KPT>(p, pos0, t, forced);
     const uint32_t vis = p.mpa ? load_mask<KPT>(x.mask, p.n_max, pos0) : 0u;
     bits_of_thread(vis_w, r) = (uint16_t)vis;
-    count_first<KPT, TEAM>(sh, t, vis, valid);
+    count_first<KPT, TEAM>(sh, map, t, vis, valid);
   }
-  SelRanges g{{kNowhere, 0u, 0u, 0u}, {kNowhere, 0u, 0u, 0u}, false, false, 0u};
-  select_walk<TEAM>(sh, rank, true, x.want0, x.want1, g, 0, 0);
+  SelRanges<kCap> g{{kNowhere, 0u, 0u, 0u}, {kNowhere, 0u, 0u, 0u}, false, false, 0u, 0u};
+  team_wait_started<TEAM>();
+  select_walk<TEAM>(sh, rank, &map, x.want0, x.want1, g, 0, 0);
+  bool swept = false;
   if (g.crowded0() || g.crowded1()) {
     const int shift0 = range_shift(g.r0.span, kDig), shift1 = range_shift(g.r1.span, kDig);
+    team_sync<TEAM>();
     zero_buckets<TEAM, 1>(sh);
+    __syncthreads();
 #pragma unroll 1
     for (int r = 0; r < rounds; ++r) {
       uint32_t t[KPT], forced;
       x.template load<KPT>(p, start + r * kRound + tid * KPT, t, forced);
       count_again<KPT, TEAM>(sh, g, t, bits_of_thread(vis_w, r), shift0, shift1);
     }
-    select_walk<TEAM>(sh, rank, false, x.want0, x.want1, g, shift0, shift1);
-    select_bisect<TEAM>(sh, x.want0, x.want1, g, [&](auto each) {
+    select_walk<TEAM>(sh, rank, nullptr, x.want0, x.want1, g, shift0, shift1);
+    if (g.crowded0() || g.crowded1()) {
+      select_bisect<TEAM>(sh, x.want0, x.want1, g, [&](auto each) {
 #pragma unroll 1
-      for (int r = 0; r < rounds; ++r) {
-        uint32_t t[KPT], forced;
-        x.template load<KPT>(p, start + r * kRound + tid * KPT, t, forced);
-        const uint32_t vis = bits_of_thread(vis_w, r);
+        for (int r = 0; r < rounds; ++r) {
+          uint32_t t[KPT], forced;
+          x.template load<KPT>(p, start + r * kRound + tid * KPT, t, forced);
+          const uint32_t vis = bits_of_thread(vis_w, r);
 #pragma unroll
-        for (int j = 0; j < KPT; ++j) each(t[j], (vis >> j) & 1u);
-      }
-    });
+          for (int j = 0; j < KPT; ++j) each(t[j], (vis >> j) & 1u);
+        }
+      });
+      swept = true;
+    }
   }
 
   // ---- kept and candidates. Nothing wanted: nothing lies before 0; all wanted: everything lies before kNowhere.
   const uint32_t lo0 = x.want0 ? g.r0.lo : 0u, lo1 = x.want1 ? g.r1.lo : 0u;
   const uint32_t wide0 = x.want0 && !g.short0 ? g.r0.span + 1u : 0u, wide1 = x.want1 && !g.short1 ? g.r1.span + 1u : 0u;
-  const bool on0 = g.r0.in <= kListCap, on1 = g.r1.in <= kListCap;
+  const bool on0 = g.r0.in <= kCap, on1 = g.r1.in <= kCap;
 #pragma unroll 1
   for (int r = 0; r < rounds; ++r) {
     const int at = r * kRound + tid * KPT;
@@ -568,13 +651,15 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_long_kernel(SelParams 
     append_positions<TEAM, 1>(sh, cand_pos[0], cand_pos[1], on0 ? in & vis : 0u, on1 ? in & ~vis : 0u, at);
   }
   __syncthreads();
-  const int m = tid / kHalf, mine_n = m ? sh.list_n >> 16 : sh.list_n & 0xffffu;
+  const uint32_t listed = sh.list_n;
+  if (swept) find_places<TEAM, 1>(sh, rank, tid == 0 ? listed & 0xffffu : 0u, tid == 0 ? listed >> 16 : 0u);
+  const int m = tid / kHalf, mine_n = m ? listed >> 16 : listed & 0xffffu, place = mine_n ? sh.found[m].seg[rank] : 0;
   for (int i = tid % kHalf; i < mine_n; i += kHalf)
-    sh.list[m][i] = x.load_one(p, start + (int)cand_pos[m][i]) - (m ? lo1 : lo0);
+    put<TEAM, 1, true>(sh, m, place + i, x.load_one(p, start + (int)cand_pos[m][i]) - (m ? lo1 : lo0));
   const Thresholds h = select_thresholds<TEAM>(sh, x.want0, x.want1, g);
   // ---- of the candidates, those before the threshold are kept and those at it stay candidates (ties)
   for (int i = tid % kHalf; i < mine_n; i += kHalf) {
-    const uint32_t t = sh.list[m][i] + (m ? lo1 : lo0), thr = m ? h.thr1 : h.thr0, at = cand_pos[m][i];
+    const uint32_t t = sh.list[m][place + i] + (m ? lo1 : lo0), thr = m ? h.thr1 : h.thr0, at = cand_pos[m][i];
     if (t < thr) atomicOr(keep_w + bits_slot(at >> 5), 1u << (at & 31));
     if (t != thr) atomicAnd(cand_w + bits_slot(at >> 5), ~(1u << (at & 31)));
   }
@@ -583,8 +668,9 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_long_kernel(SelParams 
   const int w0 = min(tid * share, words), w1 = min(w0 + share, words);
   u64 mine = 0;
   for (int w = w0; w < w1; ++w) mine += emit_counts(keep_w[bits_slot(w)], cand_w[bits_slot(w)], vis_w[bits_slot(w)]);
-  u64 ahead = counts_before<TEAM>(sh, rank, mine);
-  const int64_t off = segment_start<TEAM, kPool>(sh, p, x, rank, g.n_vis);
+  const uint32_t forced_before = kPool ? (uint32_t)max(min(start, x.n) - x.wfrom, 0) : 0u;
+  u64 ahead = counts_before<TEAM>(sh, rank, mine, h, x.want0, x.want1, g, forced_before, swept);
+  const int64_t off = segment_start<TEAM, kPool>(sh, s, p, x, rank, g.n_vis);
   if (off < 0) return;
   for (int w = w0; w < w1; ++w) {
     const uint32_t gt = keep_w[bits_slot(w)], eq = cand_w[bits_slot(w)], vis = vis_w[bits_slot(w)];
@@ -648,10 +734,11 @@ int launch_select(const madakv_config& c, const float* psi, const uint8_t* mask,
   p.keep_window = c.keep_window;
   p.window = c.window;
   p.pool_r = (c.pool_kernel - 1) / 2;
-  // One sequence, few units: no kernel of its own for the scan of the segments (2 us on the host, 3-5 on the GPU). Units of
-  // other sequences would need those sequences' visual-token counts, and a larger call is better off with a scan that runs
-  // beside the ranking.
-  p.alone = c.batch == 1 && p.units < 148;
+  p.rows = c.n_q_heads / c.n_kv_heads * c.window;
+  // Few units: no kernel of its own for the scan of the segments (2 us on the host, 3-5 on the GPU). A unit needs the visual-token
+  // counts of the sequences before its own, which it takes itself as long as they are a few loads per thread; a larger call is
+  // better off with a scan that runs beside the ranking.
+  p.alone = p.units < 148 && c.batch <= kAloneSeqs && (c.batch == 1 || (int64_t)c.batch * c.max_seq_len <= kAloneTokens);
   if (!p.alone) launch_pdl(seg_scan_kernel, dim3(1), dim3(1024), 0, st, p);
   if (c.pool_kernel > 1 || c.keep_window) launch_select_unit<true>(c, p, st);
   else launch_select_unit<false>(c, p, st);

@@ -565,6 +565,43 @@ def test_allocate_and_select_over_blocks_and_lengths(kind, units, n):
     assert_segments_equal(kept_len, seg_off, buf.kept_idx.cpu().numpy(), kept_idx, "kept_idx")
 
 
+@pytest.mark.parametrize("B,Hkv,n", [(2, 2, 32768), (2, 2, 32769), (64, 1, 131), (65, 1, 131), (7, 3, 4097), (16, 2, 4096), (36, 4, 33)])
+@pytest.mark.parametrize("kind", ["scale", "one_bucket", "octaves"])
+@pytest.mark.parametrize("w,g", [(8, 1), (64, 2), (64, 64)])
+def test_allocate_and_select_over_batches_and_score_ranges(B, Hkv, n, kind, w, g):
+    """Ragged batches on both sides of the size up to which selection needs no scan of its own, and scores at the edges of the
+    ranking kernels' buckets, whose layout follows the mean score g * w / n: scores around that mean, more than 256 and
+    more than 1024 of them in one bucket, and scores from 30 octaves; bit-exact against the oracle, with and without the
+    options outside the paper."""
+    rng = np.random.RandomState(B * n + w * g)
+    keep, pool = (1, 5) if kind == "octaves" else (0, 1)
+    cfg = mk.make_config(torch.float32, B, 1, Hkv * g, Hkv, 64, n, w, max_new_tokens=3, theta=0.4, keep_window=keep, pool_kernel=pool)
+    sl = np.maximum(n - rng.randint(0, n // 2 + 1, B), 1).astype(np.int32)
+    sl[0] = n
+    mean = g * w / n
+    psi = {"scale": lambda: mean * np.exp(0.4 * rng.randn(B, 1, Hkv, n)),
+           "one_bucket": lambda: mean * (1.0 + 3e-4 * rng.rand(B, 1, Hkv, n)),
+           "octaves": lambda: np.exp2(rng.uniform(-24, 6, (B, 1, Hkv, n)))}[kind]().astype(np.float32)
+    mask = (rng.rand(B, n) < rng.uniform(0, 1, (B, 1))).astype(np.uint8)
+    bud = rng.randint(1, n + 1, B).astype(np.int32)
+    want = oracle.allocate(psi, mask, sl, bud, float(np.float32(cfg.theta)), keep_window=keep, window=w)
+    cap = B * Hkv * (n + 3)
+    rc, kept_len, seg_off, kept_idx = oracle.select(psi, mask, sl, want["budgets"], headroom=3, capacity=cap, keep_window=keep, window=w,
+                                                    pool_kernel=pool)
+    assert rc == 0
+    buf = mk.EvictionBuffers(cfg, cap)
+    buf.psi.copy_(torch.from_numpy(psi))
+    d_mask, d_sl, d_bud = (torch.from_numpy(x).cuda() for x in (mask, sl, bud))
+    mk.madakv_allocate(cfg, buf.psi, d_mask, d_sl, d_bud, buf.mass, buf.pref, buf.demand, buf.phi, buf.budgets, buf.ws)
+    for key in ("mass", "pref", "demand", "phi", "budgets"):
+        assert np.array_equal(getattr(buf, key).cpu().numpy(), want[key]), key
+    mk.madakv_select(cfg, buf.psi, d_mask, d_sl, buf.budgets, buf.kept_len, buf.seg_off, buf.kept_idx, buf.ws)
+    assert mk.madakv_poll_status(buf.ws) == 0
+    assert np.array_equal(buf.kept_len.cpu().numpy(), kept_len)
+    assert np.array_equal(buf.seg_off.cpu().numpy(), seg_off)
+    assert_segments_equal(kept_len, seg_off, buf.kept_idx.cpu().numpy(), kept_idx, "kept_idx")
+
+
 @pytest.mark.parametrize("name", ["tiny_gqa_ragged", "bf16_d128", "bf16_gqa7", "tc_short_seqs"])
 @pytest.mark.parametrize("hcc", [mk.HCC_PAPER, mk.HCC_LITERAL, mk.HCC_DEMAND])
 @pytest.mark.parametrize("split", [False, True])
