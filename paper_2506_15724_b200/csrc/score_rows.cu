@@ -75,13 +75,14 @@ struct RowParams {
   int32_t* status;   // ws header
   int B, units, L, Hq, Hkv, g, w, R, n_max, causal, rs, mblocks, cparts, n16;  // n16: R rounded up to 16
   int lh;            // units per sequence
-  FastDiv by_hkv, by_wc;
+  FastDiv by_hkv, by_wc, by_grid, by_per;
   const float *qf, *kf;  // fp32 inputs
   madakv_strides sq, sk; // of fp32 inputs, in elements
   int h0, r0, wc;    // the launch's window rows: rows [r0, r0 + wc) of query heads h0 .. of the group, R = heads * wc
   int accumulate;    // psi += instead of =
   int smax;          // runs (CTAs) a unit's tiles can be spread over at most: wide_max_runs()
   int grid;          // CTAs of the two passes (the merge kernel needs the partition)
+  int per, slack;    // CTAs per unit (0: fewer CTAs than units), tiles a CTA may have more for it: see partition_of()
   float scale2;
   // 1 / scale2 as the sum of two. In 32 bits it is off by 2.8e-8 for head_dim 128 (64 rows, 20480 keys: 2-norm of the scores' error
   // 3.6e-7 -> 1.8e-7). bf16 with given log-sum-exps does without the second (0), because the first one's error makes up for a part
@@ -110,7 +111,8 @@ struct RowSmem {
   // full[kStages], empty[kStages], qfull[2], qempty[2], tfull[2], tempty[2], drain, xfull[8], xempty[8]
   static constexpr int kNumBars = 2 * kStages + 4 + 4 + 1 + 16;
   static constexpr int kMiscOff = (kBarOff + kNumBars * 8 + 15) / 16 * 16;
-  static constexpr int kColOff = kMiscOff + 48;            // window position (row % w) of every row [256]
+  static constexpr int kFirstOff = kMiscOff + 48;          // the CTA's first run and the cursor behind it
+  static constexpr int kColOff = kFirstOff + 64;           // window position (row % w) of every row [256]
   static constexpr int kOffOff = kColOff + 256 * 4;        // pass 2: place of every row in the group's log-sum-exps [256]
   static constexpr int kXchOff = kOffOff + 256 * 4;        // pass 2: partial psi of column shares 1-3 [2][3][128]
   static constexpr int kLenOff = kXchOff + 6 * 128 * 4;    // lengths of the sequences
@@ -298,10 +300,10 @@ __device__ __forceinline__ void cursor_settle(const RowParams& p, TileCursor& c,
 }
 __device__ __forceinline__ Run cursor_run(const RowParams& p, const TileCursor& c, const int* lens) {
   Run r;
-  int ub = 0;  // c.r / c.tb: by the reciprocal, then put right (it is off by one at most, there are few units per sequence)
+  int ub = 0;  // c.r / c.tb: by the reciprocal, then put right (it is off by one at most where there are fewer than 2^20 units)
   r.t0 = c.r;
   if (c.r >= c.tb) {
-    ub = (int)((float)c.r * __frcp_rn((float)c.tb));
+    ub = (int)__fdividef((float)c.r, (float)c.tb);
     r.t0 = c.r - ub * c.tb;
     while (r.t0 < 0) --ub, r.t0 += c.tb;
     while (r.t0 >= c.tb) ++ub, r.t0 -= c.tb;
@@ -323,8 +325,38 @@ __device__ __forceinline__ void cursor_advance(const RowParams& p, TileCursor& c
   cursor_settle(p, c, lens);
 }
 // The partition: of `total` tiles CTA c of `ctas` gets [first_tile(c), first_tile(c + 1)), the first ones one more each.
-// (The host refuses shapes with 2^30 tiles or more.)
-__device__ __forceinline__ int first_tile(int total, int ctas, int c) { return total / ctas * c + min(c, total % ctas); }
+// (The host refuses shapes with 2^30 tiles or more.) Units of equal length that are fewer than CTAs get `per` CTAs of their
+// own each, if that makes no CTA's share longer by more than p.slack tiles: a CTA that changes units waits for the new row
+// operands, 5000 clocks with one buffer for them, 2-3 tiles' time, and ends that much later than all others (4 units of 256
+// tiles, 224 rows: three of 148 CTAs did, and a layer took 17.1 us; with this, and a start under
+// the kernel before it (see score_rows_kernel), 14.8).
+struct Partition {
+  int total, ctas, per, tb;  // per: 0, or the CTAs of a unit, all of tb tiles
+};
+template <typename Tiles>
+__device__ __forceinline__ Partition partition_of(const RowParams& p, bool exact, Tiles tiles) {
+  Partition x{0, 0, 0, tiles(0)};
+  bool same = exact && x.tb > 0 && p.per > 0;
+  if (exact) {
+    for (int b = 0; b < p.B; ++b) {
+      const int tb = tiles(b);
+      x.total += p.lh * tb;
+      same = same && tb == x.tb;
+    }
+  } else {
+    x.total = p.units * x.tb;
+  }
+  // (a batch with fewer tiles than CTAs is spread over as many CTAs as it has tiles: no empty range lies between
+  // two CTAs that share a unit)
+  x.ctas = min(x.total, p.grid);
+  if (same && p.by_per.div(x.tb + p.per - 1) <= p.by_grid.div(x.total + p.grid - 1) + p.slack) x.per = p.per;
+  return x;
+}
+__device__ __forceinline__ int first_tile(const RowParams& p, const Partition& x, int c) {  // (without CTAs of a unit's own)
+  if (x.total < p.grid) return min(c, x.total);
+  const int q = p.by_grid.div(x.total);
+  return q * c + min(c, x.total - q * p.grid);
+}
 __device__ __forceinline__ int cta_of(int total, int ctas, int x) {
   const int q = total / ctas, more = total % ctas;
   return x < more * (q + 1) ? x / (q + 1) : more + (x - more * (q + 1)) / q;  // (x < total, so q > 0 in the second case)
@@ -387,7 +419,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
   uint64_t* xempty = xfull + 8;        // [2][4]    pass 2: share 0 -> shares 1-3
   uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(smem + SL::kMiscOff);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + SL::kMiscOff + 4);
-  int* range_s = reinterpret_cast<int*>(smem + SL::kMiscOff + 8);  // first sequence, tile in it, tiles, empty sequences, lo, total, CTAs in use
+  int* range_s = reinterpret_cast<int*>(smem + SL::kMiscOff + 8);  // are there empty sequences, first tile, total, CTAs in use, CTAs per unit or 0
   int* len_s = reinterpret_cast<int*>(smem + SL::kLenOff);
   int* rowpos = reinterpret_cast<int*>(smem + SL::kColOff);
   int* rowoff = reinterpret_cast<int*>(smem + SL::kOffOff);
@@ -396,30 +428,57 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(&full[s], CV ? kConvertWarps : 1);
-      mbar_init(&empty[s], 1);
+  // The lengths are read, the CTA's range is found and its first operands are asked for (into the L2) under the kernel before
+  // this one, on whose results none of that rests: the lengths are read again behind the wait, and should one have changed the
+  // range is found anew. Apart from that nothing before the wait touches more than this CTA's shared memory and TMEM. In a call
+  // of a few tiles per CTA the way to the first MMA counts as much as the tiles, and what it costs is instructions that
+  // are run once, by one warp: so all threads together write the first unit's shift rows, only what the MMAs read is
+  // cleared, and the roles find the first run in shared memory. (Range, loads and shift rows one after the other behind the
+  // wait, 112 KB cleared: first MMA 7000 clocks behind it; now 2700. One layer of 4 units of 256 tiles, 224 rows: 17.1 -> 14.8 us;
+  // 8 units of 33 tiles, 448 rows in two chunks 20.9 -> 19.3; an fp32 call of 4 units of 4 tiles 17.1 -> 16.3. Prefetching by one
+  // instruction per 128 bytes and thread, and the range by a warp of its own: slower where CTAs change units, 373 against 346 us
+  // for 32 layers of 40 units of 20 tiles.)
+  const int* lens = p.B <= kMaxSeqScan ? len_s : nullptr;
+  auto length_now = [&](int b) { return max(0, min(__ldcg(p.seq_len + b), p.n_max)); };
+  auto read_lengths = [&]() {  // (by the last threads first: the first warps have more to set up)
+    if (lens)
+      for (int b = SL::kThreads - 1 - (int)threadIdx.x; b < p.B; b += SL::kThreads) len_s[b] = length_now(b);
+  };
+  read_lengths();
+  if (warp == 0) {
+    for (int x = lane; x < SL::kNumBars; x += 32) {
+      const int y = x - 2 * kStages;  // qfull, qempty, tfull, tempty, drain, xfull, xempty from 0 on
+      uint32_t count = 1;
+      if (x < kStages) count = CV ? kConvertWarps : 1;
+      if (y >= 0 && y < 2) count = (CV ? kConvertWarps : 1) + (PASS == 2 ? 1 : 0);
+      if (y >= 6 && y < 8) count = 32 * SL::kEpiWarps;  // every epilogue thread
+      if (y >= 9 && y < 17) count = SL::kShares > 1 ? 32 * (SL::kShares - 1) : 1;
+      if (y >= 17) count = 32;
+      mbar_init(&bars[x], count);
     }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&qfull[i], (CV ? kConvertWarps : 1) + (PASS == 2 ? 1 : 0));
-      mbar_init(&qempty[i], 1);
-      mbar_init(&tfull[i], 1);
-      mbar_init(&tempty[i], 32 * SL::kEpiWarps);  // every epilogue thread
-    }
-    mbar_init(drain, 1);
-    for (int i = 0; i < 8; ++i) {
-      mbar_init(&xfull[i], SL::kShares > 1 ? 32 * (SL::kShares - 1) : 1);
-      mbar_init(&xempty[i], 32);
-    }
-    *abort_flag = 0;
+    if (lane == 0) *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // rows R..255 of the Q buffer are never written by TMA: keep them zero so their logits are 0. Pass 2: the operands
-  // of the extra contraction step start out as zeros, the key side gets its three ones per row (128-byte rows with
-  // the 128-byte swizzle: the 16-byte piece that holds columns 0-7 of row r sits at position r % 8).
-  for (int x = threadIdx.x; x < (SL::kBarOff - SL::kQOff) / 16; x += SL::kThreads)
-    reinterpret_cast<uint4*>(q_s)[x] = make_uint4(0, 0, 0, 0);
+  // Rows R.. of the Q buffers are never written by TMA: keep them zero so their logits are 0 (CV writes all rows; where
+  // the operands are fp32 terms or have two buffers all of them are cleared). Pass 2: of the operands of the extra contraction step an MMA reads
+  // columns 0-15 of every row, two 16-byte pieces (128-byte rows with the 128-byte swizzle: piece x of row r sits at position
+  // x ^ (r % 8)): the key side gets its three ones per row, the shift rows start as zeros.
+  {
+    const bool some = NS == 1 && p.R > 128;
+    const int rows = some ? SL::kQRows - p.R : SL::kQRows;
+#pragma unroll 1
+    for (int kb = 0; kb < (CV ? 0 : kKBlocks * NS); ++kb) {
+      uint4* at = reinterpret_cast<uint4*>(q_s + (kb * SL::kQRows + (some ? p.R : 0)) * 128);
+      for (int x = threadIdx.x; x < rows * 8; x += SL::kThreads) at[x] = make_uint4(0, 0, 0, 0);
+    }
+  }
+  if (PASS == 2) {
+    for (int x = threadIdx.x; x < 2 * (SL::kQRows + kTileKeys); x += SL::kThreads) {
+      const int piece = x & 1, r = x >> 1, rr = r < SL::kQRows ? r : r - SL::kQRows;
+      uint8_t* at = (r < SL::kQRows ? shift_s : ones_s) + rr * 128 + ((piece ^ (rr & 7)) * 16);
+      *reinterpret_cast<uint4*>(at) = r >= SL::kQRows && !piece ? make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u) : make_uint4(0, 0, 0, 0);
+    }
+  }
   if (threadIdx.x < 256) {
     const int x = threadIdx.x, hh = p.by_wc.div(x), pos = p.r0 + x - hh * p.wc;
     rowpos[x] = pos;
@@ -436,38 +495,43 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  if (PASS == 2) {
-    __syncthreads();  // (the zeros are written)
-    if (threadIdx.x < kTileKeys) {
-      const int r = threadIdx.x;
-      *reinterpret_cast<uint4*>(ones_s + r * 128 + (r & 7) * 16) = make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);
-    }
-  }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  // (everything above touches only this CTA's shared memory and TMEM: it overlaps the kernel before this one)
-  pdl_wait();
-  pdl_go();
-  const int* lens = p.B <= kMaxSeqScan ? len_s : nullptr;
-  if (lens)
-    for (int b = threadIdx.x; b < p.B; b += SL::kThreads) len_s[b] = clamped_len(p.seq_len, b, p.n_max);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    // this CTA's range of tiles
-    int total = 0, none = 0;
-    if (lens) {
-      for (int b = 0; b < p.B; ++b) {
-        const int tb = tiles_of(p, lens, b);
-        total += p.lh * tb;
-        none |= tb == 0 ? 1 : 0;
+  struct First {  // what the roles need of the CTA's first run
+    Run run;
+    TileCursor behind;
+  };
+  static_assert(sizeof(First) <= 64, "its place in shared memory");
+  First* first_s = reinterpret_cast<First*>(smem + SL::kFirstOff);
+  auto find_range = [&]() {  // one thread
+    const Partition x = partition_of(p, lens != nullptr, [&](int b) { return tiles_of(p, lens, b); });
+    int none = 0;
+    if (lens)
+      for (int b = 0; b < p.B; ++b) none |= lens[b] == 0 ? 1 : 0;
+    range_s[0] = none;
+    range_s[2] = x.total;
+    range_s[3] = x.ctas;
+    range_s[4] = x.per;
+    if (x.per) {  // a part of one unit
+      const int u = p.by_per.div(blockIdx.x), i = (int)blockIdx.x - u * x.per, q = p.by_per.div(x.tb), more = x.tb - q * x.per;
+      Run run = {};
+      if (u < p.units) {
+        run.u = u;
+        for (run.b = 0; u >= (run.b + 1) * p.lh;) ++run.b;
+        const int ub = u - run.b * p.lh;
+        run.n = lens[run.b];
+        run.l = p.by_hkv.div(ub);
+        run.h = ub - run.l * p.Hkv;
+        run.t0 = i * q + min(i, more);
+        run.cnt = run.tiles = q + (i < more ? 1 : 0);
       }
-    } else {
-      total = p.units * tiles_of(p, lens, 0);
+      range_s[1] = u * x.tb + run.t0;
+      first_s->run = run;
+      TileCursor none_left = {};
+      none_left.done = run.cnt;
+      first_s->behind = none_left;
+      return;
     }
-    // (a batch with fewer tiles than CTAs is spread over as many CTAs as it has tiles: no empty range lies between
-    // two CTAs that share a unit)
-    const int ctas = min(total, (int)gridDim.x);
-    const bool idle = (int)blockIdx.x >= ctas;
-    const int lo = idle ? total : first_tile(total, ctas, blockIdx.x), hi = idle ? total : first_tile(total, ctas, blockIdx.x + 1);
+    const int lo = first_tile(p, x, blockIdx.x), hi = first_tile(p, x, blockIdx.x + 1);
     int b0 = 0, r0 = lo;
     if (lens) {
       while (b0 < p.B) {
@@ -481,13 +545,109 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
       b0 = lo / per;
       r0 = lo - b0 * per;
     }
-    range_s[0] = b0;
-    range_s[1] = r0;
-    range_s[2] = hi - lo;
-    range_s[3] = none;
-    range_s[4] = lo;
-    range_s[5] = total;
-    range_s[6] = ctas;
+    range_s[1] = lo;
+    TileCursor c;
+    c.b = b0;
+    c.r = r0;
+    c.left = c.b < p.B ? hi - lo : 0;
+    c.done = 0;
+    c.tb = c.left > 0 ? tiles_of(p, lens, c.b) : 1;
+    c.per_b = p.lh * c.tb;
+    cursor_settle(p, c, lens);
+    Run run = {};
+    if (c.left > 0) {
+      run = cursor_run(p, c, lens);
+      cursor_advance(p, c, run, lens);
+    }
+    first_s->run = run;
+    first_s->behind = c;
+  };
+  // Where a role starts, and its next run: the first one from shared memory, the others from the cursor.
+  auto cursor_begin = [&]() {
+    TileCursor c = {};
+    c.left = first_s->run.cnt;
+    return c;
+  };
+  auto take_run = [&](TileCursor& c) {
+    Run run;
+    if (c.done == 0) {
+      run = first_s->run;
+      c = first_s->behind;
+    } else {
+      run = cursor_run(p, c, lens);
+      cursor_advance(p, c, run, lens);
+    }
+    return run;
+  };
+  __syncthreads();
+  if (warp == 0) {
+    if (lens && lane == 0) find_range();
+    __syncwarp();
+    if (NS == 1 && lens && first_s->run.tiles > 0) {
+      const Run run = first_s->run;
+      if (PASS == 2 && p.given_lse) {
+        const float* src = p.given_lse + (((int64_t)run.b * p.L + run.l) * p.Hq + run.h * p.g + p.h0) * p.w;
+        if (lane * 32 < p.R) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + rowoff[lane * 32]));
+      }
+      if (lane < 2 * kKBlocks) {  // the queries and the first tiles, half a row at a time
+        const bool is_q = lane < kKBlocks;
+        const int kb = lane % kKBlocks;
+        for (int t = 0; t < (is_q ? 1 : min(run.tiles, kStages)); ++t)
+          tma_prefetch_5d(is_q ? &tmap_q : &tmap_k, kb * 64, is_q ? p.r0 : (run.t0 + t) * kTileKeys, is_q ? run.h * p.g + p.h0 : run.h, run.l, run.b);
+      }
+    }
+  }
+  pdl_wait();
+  pdl_go();
+  bool moved = !lens;  // (very large batches: found behind the wait)
+  if (lens)
+    for (int b = SL::kThreads - 1 - (int)threadIdx.x; b < p.B; b += SL::kThreads) moved = moved || length_now(b) != len_s[b];
+  if (__syncthreads_or(moved)) {
+    read_lengths();
+    __syncthreads();
+    if (threadIdx.x == 0) find_range();
+    __syncthreads();
+  }
+  // Row r of the shift operand: -lse_r / scale as the sum of three bf16 numbers (24 bits) in columns 0-2. Multiplied by
+  // the key side's ones in the extra contraction step, the accumulator holds q.k - lse / scale and the epilogue needs no
+  // per-row operand at all.
+  auto load_lse = [&](const Run& run, int r) {
+    const float* src = p.given_lse ? p.given_lse + (((int64_t)run.b * p.L + run.l) * p.Hq + run.h * p.g + p.h0) * p.w : p.lse2 + (int64_t)run.u * p.rs;
+    return __ldcg(src + (p.given_lse ? rowoff[r] : min(r, p.rs - 1)));
+  };
+  auto store_shift = [&](int buf, int r, float nl) {
+    // a row that sees no key (-inf) and the padding rows get a shift that turns every weight into 0
+    if (p.given_lse) nl = nl > -INFINITY ? -nl * kLog2e : kEmptyMax;
+    if (r >= p.R) nl = kEmptyMax;
+    if (r < p.n16) {
+      // (v + more is the quotient to some 40 bits, see RowParams)
+      const float v = nl * p.inv, more = p.inv_more != 0.f ? fmaf(nl, p.inv, -v) + nl * p.inv_more : 0.f;
+      const float hi = __bfloat162float(__float2bfloat16_rn(v)), rest = (v - hi) + more;
+      const float mid = __bfloat162float(__float2bfloat16_rn(rest));
+      const float low = __bfloat162float(__float2bfloat16_rn(rest - mid));
+      const uint32_t w0 = (__float_as_uint(hi) >> 16) | (__float_as_uint(mid) & 0xffff0000u);
+      *reinterpret_cast<uint4*>(shift_s + (buf * 128 + r) * 128 + (r & 7) * 16) = make_uint4(w0, __float_as_uint(low) >> 16, 0u, 0u);
+    }
+  };
+  // The first unit's operands, before the roles begin: one thread asks for them, all write the shift rows.
+  const bool begun = first_s->run.tiles > 0;
+  const int ahead0 = NS == 1 ? min(kStages, first_s->run.tiles) : 0;
+  if (begun) {
+    const Run run = first_s->run;
+    if (NS == 1 && threadIdx.x == 0) {
+      const uint64_t pol_k = l2_policy_evict_first(), pol_q = l2_policy_evict_last();
+      for (int t = 0; t < ahead0; ++t) {
+        mbar_expect_tx(&full[t], (uint32_t)SL::kStageBytes);
+        for (int kb = 0; kb < kKBlocks; ++kb)
+          tma_load_5d(k_s + t * SL::kStageBytes + kb * kTileKeys * 128, &tmap_k, &full[t], kb * 64, (run.t0 + t) * kTileKeys, run.h, run.l, run.b, pol_k);
+        if (t) continue;
+        mbar_expect_tx(&qfull[0], (uint32_t)(p.R * 128 * kKBlocks));
+        for (int kb = 0; kb < kKBlocks; ++kb)
+          tma_load_5d(q_s + kb * SL::kQRows * 128, &tmap_q, &qfull[0], kb * 64, p.r0, run.h * p.g + p.h0, run.l, run.b, pol_q);
+      }
+    }
+    if (PASS == 2 && (int)threadIdx.x >= 32 && (int)threadIdx.x < 32 + SL::kQRows) store_shift(0, threadIdx.x - 32, load_lse(run, threadIdx.x - 32));
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
@@ -495,30 +655,18 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
   const uint32_t tmem_base = *tmem_base_s;
   const int nq = NS == 1 && p.R <= 128 ? 2 : 1;  // buffers of the row operands: buffer i starts at row 128 * i
 
-  auto cursor_begin = [&]() {
-    TileCursor c;
-    c.b = range_s[0];
-    c.r = range_s[1];
-    c.left = c.b < p.B ? range_s[2] : 0;
-    c.done = 0;
-    c.tb = c.left > 0 ? tiles_of(p, lens, c.b) : 1;
-    c.per_b = p.lh * c.tb;
-    cursor_settle(p, c, lens);
-    return c;
-  };
-
   if (warp == 0) {
     // ================================================================ TMA producer: lane 0 waits and issues the copies;
     // in pass 2 all lanes write the units' shift rows (with
     // CV all that this warp does)
     const uint64_t pol_k = NS == 3 ? l2_policy_evict_last() : l2_policy_evict_first();  // (split keys are read again)
     const uint64_t pol_q = l2_policy_evict_last();
-    int stage = 0, k = 0;  // k: units begun
-    uint32_t stage_par = 0;
+    int stage = ahead0 % kStages, k = 0;  // k: units begun
+    uint32_t stage_par = ahead0 == kStages ? 1u : 0u;
     bool ok = true;
+    if (PASS == 2 && begun && lane == 0) mbar_arrive(&qfull[0]);  // (its shift rows)
     for (TileCursor c = cursor_begin(); ok && c.left > 0;) {
-      const Run run = cursor_run(p, c, lens);
-      cursor_advance(p, c, run, lens);
+      const Run run = take_run(c);
       const int u = run.u, key_begin = run.t0 * kTileKeys, loads = run.tiles * SL::kPieces;
       if (loads == 0) continue;
       const int h = run.h, l = run.l, b = run.b;
@@ -526,17 +674,11 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
       const int th = NS == 3 ? u : h, tl = NS == 3 ? 0 : l, tb = NS == 3 ? 0 : b;
       const int buf = k % nq;
       const uint32_t q_par = (uint32_t)(k / nq) & 1u;
-      // Row r of the shift operand: -lse_r / scale as the sum of three bf16 numbers (24 bits) in columns 0-2. Multiplied by
-      // the key side's ones in the extra contraction step, the accumulator holds q.k - lse / scale and the epilogue needs no
-      // per-row operand at all. (All loads first; one after the other they took 5 us.)
-      float nl[SL::kQRows / 32];
-      if (PASS == 2) {
-        const float* src = p.given_lse ? p.given_lse + (((int64_t)b * p.L + l) * p.Hq + h * p.g + p.h0) * p.w : p.lse2 + (int64_t)u * p.rs;
+      const bool under_way = k == 0 && begun;  // the first unit's shift rows are written, and with NS = 1 its first loads issued
+      float nl[SL::kQRows / 32];  // (all loads first; one after the other they took 5 us)
+      if (PASS == 2 && !under_way) {
 #pragma unroll
-        for (int i = 0; i < SL::kQRows / 32; ++i) {
-          const int r = lane + 32 * i;
-          nl[i] = __ldcg(src + (p.given_lse ? rowoff[r] : min(r, p.rs - 1)));
-        }
+        for (int i = 0; i < SL::kQRows / 32; ++i) nl[i] = load_lse(run, lane + 32 * i);
       }
       // [from, to) of the unit's K loads, by lane 0
       auto load_keys = [&](int from, int to) {
@@ -562,9 +704,9 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
       // The unit's queries once the stages are full of its keys (those stages were the unit's before, whose tiles need
       // nothing that is still to come; from the next load on the stages wait for this unit's own tiles); the first
       // unit's at once.
-      const int ahead = k == 0 ? 1 : min(kStages, loads);
+      const int ahead = k == 0 ? (NS == 1 && begun ? ahead0 : 1) : min(kStages, loads);
       ++k;
-      if (lane == 0) {
+      if (lane == 0 && !(NS == 1 && under_way)) {
         if (!CV) load_keys(0, ahead);
         ok = ok && mbar_wait(&qempty[buf], q_par ^ 1, abort_flag, p.status, kSiteQEmpty);
         if (ok && !CV) {
@@ -573,28 +715,18 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
             tma_load_5d(q_s + (kb * SL::kQRows + buf * 128) * 128, &tmap_q, &qfull[buf], kb * 64, p.r0, th * p.g + p.h0, tl, tb, pol_q);
         }
       }
-      if (PASS == 2) {
+      if (PASS == 2 && !under_way) {
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (!ok) break;
 #pragma unroll
-        for (int i = 0; i < SL::kQRows / 32; ++i) {
-          const int r = lane + 32 * i;
-          // a row that sees no key (-inf) and the padding rows get a shift that turns every weight into 0
-          if (p.given_lse) nl[i] = nl[i] > -INFINITY ? -nl[i] * kLog2e : kEmptyMax;
-          if (r >= p.R) nl[i] = kEmptyMax;
-          if (r < p.n16) {
-            // (v + more is the quotient to some 40 bits, see RowParams)
-            const float v = nl[i] * p.inv, more = p.inv_more != 0.f ? fmaf(nl[i], p.inv, -v) + nl[i] * p.inv_more : 0.f;
-            const float hi = __bfloat162float(__float2bfloat16_rn(v)), rest = (v - hi) + more;
-            const float mid = __bfloat162float(__float2bfloat16_rn(rest));
-            const float low = __bfloat162float(__float2bfloat16_rn(rest - mid));
-            const uint32_t w0 = (__float_as_uint(hi) >> 16) | (__float_as_uint(mid) & 0xffff0000u);
-            *reinterpret_cast<uint4*>(shift_s + (buf * 128 + r) * 128 + (r & 7) * 16) = make_uint4(w0, __float_as_uint(low) >> 16, 0u, 0u);
-          }
-        }
+        for (int i = 0; i < SL::kQRows / 32; ++i) store_shift(buf, lane + 32 * i, nl[i]);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();  // every lane's rows are written (and fenced) before lane 0 signals them
         if (lane == 0) mbar_arrive(&qfull[buf]);
+      }
+      if (NS == 1 && nq == 1 && lane == 0 && c.left > 0) {  // the next unit's queries, to the L2: their place here is free only when this unit's MMAs are done
+        const Run next = cursor_run(p, c, lens);
+        for (int kb = 0; kb < kKBlocks; ++kb) tma_prefetch_5d(&tmap_q, kb * 64, p.r0, next.h * p.g + p.h0, next.l, next.b);
       }
       if (!CV && lane == 0) load_keys(ahead, loads);
       ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -613,8 +745,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
       uint32_t stage_par = 0;
       bool ok = true;
       for (TileCursor c = cursor_begin(); ok && c.left > 0;) {
-        const Run run = cursor_run(p, c, lens);
-        cursor_advance(p, c, run, lens);
+        const Run run = take_run(c);
         const int tiles = run.tiles;
         if (tiles == 0) continue;
         const int qb = k % nq;
@@ -753,7 +884,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
     float m = 4.f * kEmptyMax, z_run = 0.f;
     uint64_t zacc[4] = {0ull, 0ull, 0ull, 0ull};  // pass 1: the item's sum, as four packed partial sums
     float* xslot = xch + quarter * 32 + lane;  // pass 2: [buffer][share - 1][128 keys]
-    if (PASS == 2 && range_s[3] && !p.accumulate) {  // sequences without keys have no tiles
+    if (PASS == 2 && range_s[0] && !p.accumulate) {  // sequences without keys have no tiles
       for (int b = 0; b < p.B; ++b)
         if (len_s[b] == 0)
           for (int64_t x = ((int64_t)blockIdx.x * SL::kEpiWarps + ew) * 32 + lane; x < (int64_t)p.lh * p.n_max;
@@ -762,9 +893,8 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
     }
 
     for (TileCursor c = cursor_begin(); ok && c.left > 0;) {
-      const Run run = cursor_run(p, c, lens);
-      const int run_first = range_s[4] + c.done;  // the run's first tile in the global order
-      cursor_advance(p, c, run, lens);
+      const int run_first = range_s[1] + c.done;  // the run's first tile in the global order
+      const Run run = take_run(c);
       const int u = run.u, tiles = run.tiles, key_begin = run.t0 * kTileKeys, n = run.n;
       float* psi = p.psi + (int64_t)u * p.n_max;
       m = 4.f * kEmptyMax;  // pass 1: every run starts its own statistics
@@ -908,7 +1038,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
           // one pair per run: slot = this CTA's place among the CTAs that the unit's tiles are spread over (the merge
           // kernel walks the same partition). A row that saw no visible key only summed masked entries: it is
           // recorded as empty, and so is a run without keys (the uniform partition of very large batches has those).
-          const int k = run.t0 ? (int)blockIdx.x - cta_of(range_s[5], range_s[6], run_first - run.t0) : 0;
+          const int k = range_s[4] ? (int)blockIdx.x - p.by_per.div(blockIdx.x) * p.per : run.t0 ? (int)blockIdx.x - cta_of(range_s[2], range_s[3], run_first - run.t0) : 0;
           const bool none = tiles == 0 || m < 0.5f * kEmptyMax * p.scale2;
           if (k >= 0 && k < p.smax)
             p.part[(((int64_t)u * p.smax + k) * p.cparts + share) * p.rs + row] =
@@ -932,8 +1062,7 @@ score_rows_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
       uint32_t stage_par = 0;
       bool ok = true;
       for (TileCursor c = cursor_begin(); ok && c.left > 0;) {
-        const Run run = cursor_run(p, c, lens);
-        cursor_advance(p, c, run, lens);
+        const Run run = take_run(c);
         if (run.tiles == 0) continue;
         const int h = run.h, l = run.l, b = run.b, n = run.n;
         const float* kf = p.kf + b * p.sk.batch + l * p.sk.layer + h * p.sk.head;
@@ -1053,24 +1182,18 @@ __global__ void __launch_bounds__(256) score_rows_merge_kernel(RowParams p, floa
     const int b = u / p.lh;
     const bool exact = p.B <= kMaxSeqScan;
     auto seq_tiles = [&](int b2) { return ((exact ? clamped_len(p.seq_len, b2, p.n_max) : p.n_max) + kTileKeys - 1) / kTileKeys; };
-    int all_tiles = 0, first = 0;  // tiles of the batch; the unit's first tile in the global order
+    const Partition x = partition_of(p, exact, seq_tiles);
     const int tb = seq_tiles(b);
+    int first = 0;  // the unit's first tile in the global order
     if (exact) {
-      for (int b2 = 0; b2 < p.B; ++b2) {
-        const int per = p.lh * seq_tiles(b2);
-        if (b2 < b) first += per;
-        all_tiles += per;
-      }
+      for (int b2 = 0; b2 < b; ++b2) first += p.lh * seq_tiles(b2);
     } else {
-      all_tiles = p.units * tb;
       first = b * p.lh * tb;
     }
     first += (u - b * p.lh) * tb;
     s_entries = 0;
-    if (tb > 0) {
-      const int ctas = min(all_tiles, p.grid);
-      s_entries = p.cparts * min(p.smax, cta_of(all_tiles, ctas, first + tb - 1) - cta_of(all_tiles, ctas, first) + 1);
-    }
+    if (tb > 0)
+      s_entries = p.cparts * min(p.smax, x.per ? min(x.per, tb) : cta_of(x.total, x.ctas, first + tb - 1) - cta_of(x.total, x.ctas, first) + 1);
   }
   __syncthreads();
   const int entries = s_entries;
@@ -1201,6 +1324,9 @@ int score_rows(const madakv_config& c, const void* q, madakv_strides sq, const v
   if (sms > kWideMaxGrid) sms = kWideMaxGrid;
   const int grid = (int)(tiles < sms ? tiles : sms);
   p.grid = grid;
+  p.per = grid / p.units;
+  p.by_grid = FastDiv(grid);
+  p.by_per = FastDiv(p.per > 0 ? p.per : 1);
   const bool convert = f32 && (given_lse || !split_first(c));
   CUtensorMap mk = {}, mq = {};  // (convert: not used)
   const madakv_strides split_k{0, 0, (int64_t)c.max_seq_len * 3 * d, 3 * d}, split_q{0, 0, (int64_t)c.window * 3 * d, 3 * d};
@@ -1232,6 +1358,7 @@ int score_rows(const madakv_config& c, const void* q, madakv_strides sq, const v
       p.mblocks = p.R <= 128 ? 1 : 2;
       p.cparts = convert ? 1 : (p.R <= 128 ? 4 : 2);
       p.n16 = (p.R + 15) / 16 * 16;
+      p.slack = !f32 && p.R <= 128 ? 0 : 2;  // (two buffers for the row operands, or one)
       if (!convert && !(f32 ? make_map(&mq, q, 3 * d, c.window, p.units * g, 1, 1, split_q, p.wc, heads)
                             : make_map(&mq, q, d, c.window, c.n_q_heads, c.n_layers, c.batch, sq, p.wc, heads)))
         return MADAKV_EUNSUPPORTED;

@@ -160,6 +160,39 @@ def test_score_in_chunks(dtype, B, L, Hq, Hkv, d, n, w, causal):
 # sequences longer than a cluster's TMEM holds: a whole round of clusters, tiles that pass twice in one sequence of the batch
 # and not in the other, lengths that end inside a tile; with logits so far apart that references are raised; and the calls
 # next to the rule (too few units, too many rows), which take two passes
+@pytest.mark.parametrize("dtype,B,Hq,Hkv,w,n", [
+    ("bf16", 1, 28, 4, 32, 37 * 128 + 5), ("bf16", 1, 28, 4, 32, 36 * 128), ("bf16", 1, 28, 4, 32, 75 * 128), ("bf16", 2, 16, 4, 64, 2500),
+    ("bf16", 1, 32, 8, 20, 600), ("bf16", 3, 147, 49, 30, 400), ("f32", 1, 8, 4, 32, 36 * 128 + 1)])
+@pytest.mark.parametrize("given", [False, True])
+def test_score_partition_and_lengths_written_just_before(dtype, B, Hq, Hkv, w, n, given):
+    """Wide-window scoring where every unit gets thread blocks of its own (about as many tiles as blocks, one more or fewer, far
+    fewer; as many units as blocks), where it does not because the lengths differ, and with lengths that the kernel before
+    in the stream has just changed, since the range of a block is found before that kernel has ended. Against the oracle,
+    with the tolerance of the other score tests (1e-4 relative: fp32 sums of up to 10^4 terms)."""
+    wl = synth.scaled(TINY, B=B, L=1, Hq=Hq, Hkv=Hkv, n=n, w=w, d=64, dtype=dtype)
+    inp = synth.make_inputs(wl, device="cpu", want_v=False)
+    g = dev(inp)
+    cfg = config_of(wl)
+    psi, lse = torch.zeros((B, 1, Hkv, n), device="cuda"), torch.zeros((B, 1, Hq, w), device="cuda")
+    ws = mk.new_workspace(cfg)
+    short = np.full(B, n, np.int32)
+    short[0] = max(n - 2 * 128 - 1, w)
+    d_sl = torch.zeros(B, dtype=torch.int32, device="cuda")
+    for sl in (np.full(B, n, np.int32), short, np.full(B, n - 130, np.int32), np.full(B, n, np.int32)):
+        want = oracle.score(dcode(wl), to_np(inp["q_win"]), to_np(inp["k"]), sl)
+        if given:
+            mk.madakv_score(cfg, g["q_win"], g["k"], torch.from_numpy(sl).cuda(), lse, psi, ws)
+        new = torch.from_numpy(sl).cuda()
+        psi.fill_(7.0)
+        d_sl.copy_(new)
+        if given:
+            mk.madakv_score_lse(cfg, g["q_win"], g["k"], d_sl, lse, psi, ws)
+        else:
+            mk.madakv_score(cfg, g["q_win"], g["k"], d_sl, lse, psi, ws)
+        assert mk.madakv_poll_status(ws) == 0
+        psi_close(psi.cpu().numpy(), want, rtol=1e-4)
+
+
 @pytest.mark.parametrize("B,H,d,n,w", [(1, 22, 64, 16500, 32), (2, 11, 128, 17003, 20), (1, 2, 64, 17000, 32), (1, 24, 64, 5200, 64)])
 @pytest.mark.parametrize("spread", [False, True])
 def test_score_longer_than_tensor_memory(B, H, d, n, w, spread):
