@@ -764,7 +764,8 @@ struct RankShape {
 // allocation 156, 167, 174, 228 us, selection 219, 223, 240, 297 us), because every block pays for the fixed steps. With
 // fewer units a team of up to 8 blocks per unit brings the call to about a block per SM, and a call with a few units (one
 // layer), which is bound by the latency of its blocks, takes 8 keys per thread instead of 16 (4 units of 32768 keys: 12.8 +
-// 10.9 us with 8 blocks of 8 keys, 15.5 + 13.7 with 4 blocks of 16, 30 + 54 with one block per unit).
+// 10.9 us with 8 blocks of 8 keys, 15.5 + 13.7 with 4 blocks of 16, 30 + 54 with one block per unit, when a team met five
+// times).
 constexpr int kLongKeys = 262144;  // keys per block that a long kernel has bits for in shared memory
 inline RankShape rank_shape(long long units, int n_max) {
   const int cap16 = kRankThreads * 16, cap8 = kRankThreads * 8;

@@ -983,6 +983,26 @@ def test_decode_wait_for_rows_runs_out_and_the_library_recovers(dtype, units, ro
         assert np.abs(lse[:, 1:].cpu().numpy() - want_lse[:, 1:]).max() <= 1e-5 * np.abs(want_lse[:, 1:]).max()
 
 
+@pytest.mark.parametrize("dtype,d", [("bf16", 64), ("bf16", 128), ("f32", 128)])
+@pytest.mark.parametrize("lens", [[1, 2000, 3, 0], [700, 33, 32, 31], [17, 16, 15, 1], [0, 0, 0, 5]])
+def test_compact_segments_far_from_the_mean(dtype, d, lens):
+    """Compaction of few units launches blocks for half as much again as the cache's rows per segment: segments much longer than
+    that, and caches without a row to spare, are bit copies all the same (against indexing by torch)."""
+    n, td = 2048, torch.bfloat16 if dtype == "bf16" else torch.float32
+    cfg = mk.make_config(td, 1, 1, 4, 4, d, n, 8, max_new_tokens=0)
+    gen = torch.Generator().manual_seed(5)
+    k, v = (torch.randn(1, 1, 4, n, d, generator=gen).to(td).cuda() for _ in range(2))
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    idx = [torch.randperm(n, generator=gen)[:x].sort().values for x in lens]
+    kept = torch.cat(idx).to(torch.int32).cuda()
+    k_c, v_c = (torch.zeros(int(off[-1]), d, dtype=td, device="cuda") for _ in range(2))
+    ws = mk.new_workspace(cfg)
+    mk.madakv_compact(cfg, k, v, kept, torch.from_numpy(off).cuda(), torch.tensor(lens, dtype=torch.int32, device="cuda"), k_c, v_c, ws)
+    assert mk.madakv_poll_status(ws) == 0
+    for got, src in ((k_c, k), (v_c, v)):
+        assert torch.equal(got, torch.cat([src[0, 0, u, i.cuda()] for u, i in enumerate(idx)]))
+
+
 def test_strided_kv_layout():
     # K/V stored per layer as [B, H, n, d] inside a larger allocation (token stride > d)
     wl = synth.scaled(TINY, dtype="bf16", L=2, Hq=4, Hkv=2, d=128, n=340, w=8, budget=50)
