@@ -635,6 +635,52 @@ def test_allocate_and_select_over_batches_and_score_ranges(B, Hkv, n, kind, w, g
     assert_segments_equal(kept_len, seg_off, buf.kept_idx.cpu().numpy(), kept_idx, "kept_idx")
 
 
+# teams of 4 and 8 blocks with 8 keys per thread, a team and a single block that read their units twice, a block with 16 keys per thread
+@pytest.mark.parametrize("units,n,rows", [(3, 16384, 8), (4, 32768, 8), (2, 131072, 8), (2, 131072, 32), (150, 16391, 8), (150, 8192, 2),
+                                          (1, 1 << 20, 8), (1, 1 << 20, 32)])
+@pytest.mark.parametrize("kind", ["upper", "upper_crowd", "sink"])
+def test_allocate_and_select_large_scores_at_small_means(units, n, rows, kind):
+    """Scores far above the mean of long sequences, with the thresholds among them: a caller's up to 500 (the buckets end at 512), more
+    than the list of candidates holds in one bucket, and the library's own where one key holds most of the window's
+    attention. Bit-exact against the oracle, and nothing written outside the segments."""
+    rng = np.random.RandomState(units + n + rows)
+    psi = (rows / n * np.exp(0.5 * rng.randn(1, units, 1, n))).astype(np.float32)
+    if kind == "sink":
+        share = rng.uniform(0.7, 0.95, units)
+        psi *= (1.0 - share)[None, :, None, None].astype(np.float32)
+        psi[0, np.arange(units), 0, rng.randint(0, n // 2, units)] = (share * rows).astype(np.float32)
+    else:
+        lo, hi = (40.0, 500.0) if kind == "upper" else (300.0, 303.0)
+        for u in range(units):
+            psi[0, u, 0, rng.choice(n, min(3000, n // 3), replace=False)] = np.exp(rng.uniform(np.log(lo), np.log(hi), min(3000, n // 3)))
+    mask = (rng.rand(1, n) < 0.6).astype(np.uint8)
+    sl, bud = np.array([n - 1], np.int32), np.array([n // 7], np.int32)
+    d_psi, d_mask, d_sl, d_bud = (torch.from_numpy(x).cuda() for x in (psi, mask, sl, bud))
+    for theta in (0.3, 0.9):
+        cfg = mk.make_config(torch.float32, 1, units, 1, 1, 64, n, rows, max_new_tokens=3, theta=theta)
+        buf = mk.EvictionBuffers(cfg, 64)
+        mk.madakv_allocate(cfg, d_psi, d_mask, d_sl, d_bud, buf.mass, buf.pref, buf.demand, buf.phi, buf.budgets, buf.ws)
+        want = oracle.allocate(psi, mask, sl, bud, float(np.float32(theta)))
+        for key in ("mass", "pref", "demand", "phi", "budgets"):
+            assert np.array_equal(getattr(buf, key).cpu().numpy(), want[key]), (key, theta)
+    for keep, pool in ((0, 1), (1, 5)):
+        cfg = mk.make_config(torch.float32, 1, units, 1, 1, 64, n, rows, max_new_tokens=3, keep_window=keep, pool_kernel=pool)
+        for wanted in ((1, 1), (10, 500), (700, 10), (1000, 2000)):
+            budgets = np.broadcast_to(np.array(wanted, np.int32), (1, units, 1, 2)).copy()
+            cap = units * (sum(wanted) + rows + 3)
+            rc, kept_len, seg_off, kept_idx = oracle.select(psi, mask, sl, budgets, headroom=3, capacity=cap, keep_window=keep,
+                                                            window=rows, pool_kernel=pool)
+            assert rc == 0
+            got = torch.full((cap + 4096,), -1, dtype=torch.int32, device="cuda")
+            d_len, d_off = torch.zeros(units, dtype=torch.int32, device="cuda"), torch.zeros(units + 1, dtype=torch.int64, device="cuda")
+            mk.madakv_select(cfg, d_psi, d_mask, d_sl, torch.from_numpy(budgets).cuda(), d_len, d_off, got[:cap], buf.ws)
+            assert mk.madakv_poll_status(buf.ws) == 0
+            assert np.array_equal(d_len.cpu().numpy(), kept_len) and np.array_equal(d_off.cpu().numpy(), seg_off)
+            got = got.cpu().numpy()
+            assert np.array_equal(got[:cap], kept_idx), (wanted, keep, pool)  # (-1 between the segments on both sides)
+            assert (got[cap:] == -1).all()
+
+
 @pytest.mark.parametrize("name", ["tiny_gqa_ragged", "bf16_d128", "bf16_gqa7", "tc_short_seqs"])
 @pytest.mark.parametrize("hcc", [mk.HCC_PAPER, mk.HCC_LITERAL, mk.HCC_DEMAND])
 @pytest.mark.parametrize("split", [False, True])
