@@ -210,16 +210,6 @@ __device__ __noinline__ void sequence_budgets(const AllocParams& p, int b, int n
   }
 }
 
-// The low 32 bits of floor(x * 2^32), plus kLowBias, by fp32 additions, for keys below 512.0: adding 512
-// rounded towards zero leaves floor(x * 2^14) in the low bits of the significand, the remainder (exact) added to 2^-9 the
-// other 18 bits; the constants of the first sum are shifted out. (The conversion to a 64-bit integer runs at a small
-// fraction of the rate of additions.)
-__device__ __forceinline__ uint32_t low_mass(uint32_t key) {
-  const float x = __uint_as_float(key);
-  const float t = __fadd_rz(x, 512.0f);
-  return (__float_as_uint(t) << 18) + __float_as_uint(__fadd_rz(__fsub_rn(x, __fsub_rn(t, 512.0f)), 0x1p-9f));
-}
-
 // The ranges Eq. 9's two thresholds can lie in, with the exact masses before them, the masses to reach and the modalities' own.
 template <int CAP>  // candidates that fit the list
 struct MassRanges {
@@ -238,16 +228,14 @@ __device__ __forceinline__ u64 mass_target(u64 theta_fix, u64 W) {
   return (hi << 32) + (lo >> 32) + ((lo & 0xffffffffull) ? 1ull : 0ull);
 }
 
-// A bucket holds a count and the sum of its keys' masses modulo 2^32, two shared atomics without a result per key. That is
-// enough for the exact mass: all keys of a bucket lie between its two edges, so the mass is count * (mass of the lower
-// edge) plus a remainder below count * (distance of the edges), and the remainder is known exactly where that bound is
-// below 2^32 (it is by a wide margin for importance values: buckets are narrow where the keys are). A unit for which the
-// bound fails anywhere, or with scores of 512 and more, goes the slow way: exact sweeps that halve the range.
+// A bucket holds a count and the sum of a word per key, two shared atomics without a result, which is enough for the exact mass
+// (bucket_map.cuh). A unit with a bucket for which it is not (mass_known: ten thousands of nearly equal scores), or with scores of
+// 512 and more, goes the slow way: exact sweeps that halve the range.
 // (Exact 64-bit masses by atomics that return the old word, to detect carries: alloc 52 us on llava.)
 template <int TEAM>
 __device__ __forceinline__ void add_key(uint32_t* at, uint32_t t) {
   atomicAdd(at, 1u);
-  atomicAdd(at + 2 * RankShared<TEAM, 2>::kStride, low_mass(kTopKey - t));
+  atomicAdd(at + 2 * RankShared<TEAM, 2>::kStride, mass_word(t));
 }
 template <int KPT, int TEAM>
 __device__ __forceinline__ void add_first(RankShared<TEAM, 2>& sh, const BucketMap& map, const uint32_t (&t)[KPT], uint32_t vis, uint32_t valid) {
@@ -281,7 +269,7 @@ __device__ __forceinline__ void mass_walk(RankShared<TEAM, 2>& sh, uint32_t rank
       sh, rank,
       [&](int m, int b) {
         const int shift = m ? shift1 : shift0;
-        return map ? bucket_start(*map, b) : BucketStart{(m ? g.r1.lo : g.r0.lo) + ((uint32_t)b << shift), shift};
+        return map ? bucket_start(*map, b) : BucketStart{(m ? g.r1.lo : g.r0.lo) + ((uint32_t)b << shift), shift, false};
       },
       [&](int m, u64 W) { return map ? mass_target(theta_fix, W) : (m ? g.need1 - g.above1 : g.need0 - g.above0); });
   g.exact = !(sh.found[0].inexact | sh.found[1].inexact);

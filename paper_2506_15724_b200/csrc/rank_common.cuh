@@ -316,16 +316,6 @@ __device__ __forceinline__ void zero_buckets(RankShared<TEAM, WORDS>& sh) {
   if (threadIdx.x == 0) sh.list_n = 0;
 }
 
-constexpr uint32_t kLowBias = 0x3b000000u;  // added to every term of a bucket's mass (low_mass() of allocate.cu)
-// The edges of neighbouring buckets: the largest score that the bucket can hold that starts at t, and its mass.
-__device__ __forceinline__ float edge_score(uint32_t t) { return __uint_as_float(kTopKey - min(t, kTopKey)); }
-__device__ __forceinline__ u64 edge_mass(float x) { return __float2ull_rz(x * 4294967296.0f); }
-// Mass of a bucket's c keys, all of at least the mass e1, from their sum modulo 2^32: c * e1 and a remainder, which is known
-// exactly if it is below 2^32.
-__device__ __forceinline__ uint32_t mass_rest(uint32_t c, uint32_t sum, u64 e1) { return sum - c * (kLowBias + (uint32_t)e1); }
-// It is if c scores between x1 and x (a little is left for the rounding).
-__device__ __forceinline__ bool mass_known(uint32_t c, float x, float x1) { return (float)c * (x - x1) < 0.999f; }
-
 // Walk of the buckets, filled in by all threads of the block: start(m, b) tells where bucket b of modality m starts,
 // need(m, mass) what is to be reached, a mass (WORDS = 2) or a count; 0: nothing. Leaves `found`, the same in every block
 // (but for `before`). Ends with a barrier of the block.
@@ -341,22 +331,24 @@ __device__ __forceinline__ void walk(RankShared<TEAM, WORDS>& sh, uint32_t rank,
     const uint4 v0 = w[0], v1 = w[1];
     uint32_t lc = ((v0.x + v0.y) + (v0.z + v0.w)) + ((v1.x + v1.y) + (v1.z + v1.w));
     const uint32_t c[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-    u64 q[8] = {}, lq = 0;
+    u64 lq = 0;
     bool bad = false;
     if (kMass && lc) {  // (the buckets of most threads are empty)
       const uint4 s0 = w[2 * kStride / 4], s1 = w[2 * kStride / 4 + 1];
       const uint32_t s[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
       const BucketStart at = start(m, b0);
-      float x = edge_score(at.t);
+      const MassRule rule = mass_rule(at.t);
+      uint32_t most = 0;
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
-        const float x1 = b0 + k + 1 < kBuckets ? edge_score(at.t + ((uint32_t)(k + 1) << at.shift)) : 0.f;
-        const u64 e1 = edge_mass(x1);
-        q[k] = c[k] * e1 + mass_rest(c[k], s[k], e1);
-        lq += q[k];
-        bad = bad || (c[k] && !mass_known(c[k], x, x1));
-        x = x1;
+        lq += mass_sum(rule, c[k], s[k], bucket_last(at, k, b0 + k));
+        most = max(most, c[k]);
       }
+      lq <<= rule.up;
+      // (the eight are equally wide, but for what the first and the last one of a layout take besides)
+      bad = !mass_known(rule, most, at.t, bucket_last(at, 0, b0));
+      if (at.ends && b0 == 0) bad = bad || c[0];
+      if (at.ends && b0 == kBuckets - 8) bad = bad || !mass_known(rule, c[7], at.t + (7u << at.shift), kTopKey);
     }
     const uint32_t bads = kMass ? __ballot_sync(kFull, bad) : 0u;
     if (TEAM == 1) {  // a block on its own: every thread learns what lies before its buckets
@@ -397,6 +389,12 @@ __device__ __forceinline__ void walk(RankShared<TEAM, WORDS>& sh, uint32_t rank,
       if (want && (kMass ? iq - lq < want && iq >= want : ic - lc < want && ic >= want)) {
         uint32_t run = ic - lc, at = 0, at_c = 0, at_in = 0;
         u64 run_q = iq - lq, at_q = 0;
+        BucketStart first = {};
+        MassRule rule = {};
+        if (kMass) {
+          first = start(m, b0);
+          rule = mass_rule(first.t);
+        }
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           if (kMass ? run_q < want : run < want) {
@@ -406,7 +404,7 @@ __device__ __forceinline__ void walk(RankShared<TEAM, WORDS>& sh, uint32_t rank,
             at_q = run_q;
           }
           run += c[k];
-          run_q += q[k];
+          if (kMass) run_q += mass_sum(rule, c[k], sh.cnt[(2 + m) * kStride + b0 + k], bucket_last(first, k, b0 + k)) << rule.up;
         }
         f.hit = 1;
         f.at = at;
@@ -465,11 +463,13 @@ __device__ __forceinline__ void walk(RankShared<TEAM, WORDS>& sh, uint32_t rank,
         pair[r] = peer_load<TEAM>(reinterpret_cast<const u64*>(w), r);
         if (kMass) sums[r] = peer_load<TEAM>(reinterpret_cast<const u64*>(w + 2 * kStride), r);
       }
-      u64 e1 = 0, e2 = 0;
+      uint32_t last0 = 0, last1 = 0;
+      MassRule rule = {};
       if (kMass) {
         const BucketStart at = start(m, b);
-        e1 = edge_mass(edge_score(at.t + (1u << at.shift)));
-        e2 = b + 2 < kBuckets ? edge_mass(edge_score(at.t + (2u << at.shift))) : 0ull;
+        rule = mass_rule(at.t);
+        last0 = bucket_last(at, 0, b);
+        last1 = bucket_last(at, 1, b + 1);
       }
       uint32_t c0 = 0, c1 = 0, m0 = 0, m1 = 0;
       u64 q0 = 0, q1 = 0;
@@ -480,13 +480,13 @@ __device__ __forceinline__ void walk(RankShared<TEAM, WORDS>& sh, uint32_t rank,
         c1 += y;
         if (r < (int)rank) m0 += x, m1 += y;
         if (kMass) {
-          q0 += mass_rest(x, (uint32_t)sums[r], e1);
-          q1 += mass_rest(y, (uint32_t)(sums[r] >> 32), e2);
+          q0 += mass_sum(rule, x, (uint32_t)sums[r], last0);
+          q1 += mass_sum(rule, y, (uint32_t)(sums[r] >> 32), last1);
         }
       }
       if (kMass) {
-        q0 += c0 * e1;
-        q1 += c1 * e2;
+        q0 <<= rule.up;
+        q1 <<= rule.up;
       }
       const uint32_t run_c = __shfl_sync(kFull, ic - c, who) + warp_scan32(c0 + c1) - (c0 + c1);
       const u64 run_q = kMass ? __shfl_sync(kFull, iq - q, who) + warp_scan64(q0 + q1) - (q0 + q1) : 0ull;

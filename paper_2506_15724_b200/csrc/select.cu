@@ -289,7 +289,7 @@ template <int TEAM>
 __device__ __forceinline__ void select_walk(RankShared<TEAM, 1>& sh, uint32_t rank, const BucketMap* map, uint32_t want0, uint32_t want1,
                                             SelRanges<RankShared<TEAM, 1>::kCap>& g, int shift0, int shift1) {
   walk<TEAM, 1>(
-      sh, rank, [](int, int) { return BucketStart{0u, 0}; },
+      sh, rank, [](int, int) { return BucketStart{0u, 0, false}; },
       [&](int m, u64) -> u64 { return m ? (g.short1 || !want1 ? 0u : want1 - g.r1.above) : (g.short0 || !want0 ? 0u : want0 - g.r0.above); });
   if (map) g.n_vis = sh.found[0].total;
   auto narrow = [&](RankRange& r, bool& is_short, const Found& f, int shift) {

@@ -7,6 +7,7 @@ import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 SHIM = r"""
+#include <initializer_list>
 #include "bucket_map.cuh"
 using namespace madakv;
 // Buckets of the layout of `rows` window rows whose fine part begins at t0 that do not hold exactly the keys between their start
@@ -23,6 +24,48 @@ extern "C" int misplaced(uint32_t t0, int rows) {
     ok = ok && s.shift == first.shift && s.t == first.t + ((uint32_t)(b & 7) << s.shift);
     ok = ok && (b + 1 == kBuckets || end == s.t + (1u << s.shift));
     bad += !ok;
+  }
+  return bad;
+}
+// Buckets whose mass does not come out right from the words of its keys, for as many keys as mass_known() takes, or that take
+// fewer than they have to: one key of any score, and of scores from 2^-9 on as many as 2^32 over the bucket's width. Of a
+// layout over [t, t + 2^(11 + shift)) too.
+static int wrong(const BucketStart& s, int x, int b) {
+  const uint32_t first = s.t + ((uint32_t)x << s.shift), last = bucket_last(s, x, b), at[3] = {first, last, first + (last - first) / 3u};
+  const MassRule rule = mass_rule(s.t);
+  int bad = mass_rule(last).up != rule.up || mass_rule(last).linear != rule.linear || !mass_known(rule, 1, first, last);
+  uint32_t most = 1;
+  while (most < (1u << 20) && mass_known(rule, 2 * most, first, last)) most *= 2;
+  for (uint32_t step = most / 4; step > 0; step /= 2)
+    if (mass_known(rule, most + step, first, last)) most += step;
+  if (rule.linear && most < (1u << (31 - s.shift)) && most < (1u << 20)) ++bad;
+  for (uint32_t c : {1u, 2u, most}) {
+    if (!mass_known(rule, c, first, last)) continue;
+    for (int kind = 0; kind < 7; ++kind) {  // all alike, two values half and half, all three
+      uint32_t n[3] = {0, 0, 0}, sum = 0;
+      unsigned long long want = 0;
+      if (kind < 3) n[kind] = c;
+      else if (kind < 6) n[kind - 3] = c / 2, n[(kind - 2) % 3] = c - c / 2;
+      else n[0] = c / 3, n[1] = c / 3, n[2] = c - 2 * (c / 3);
+      for (int k = 0; k < 3; ++k) {
+        sum += n[k] * mass_word(at[k]);
+        want += n[k] * (unsigned long long)((double)score_of(at[k]) * 4294967296.0);
+      }
+      bad += mass_sum(rule, c, sum, last) << rule.up != want;
+    }
+  }
+  return bad;
+}
+extern "C" int wrong_masses(uint32_t t0, int rows) {
+  const BucketMap g = bucket_map_from(t0, rows);
+  int bad = 0;
+  for (int b = 1; b < kBuckets; ++b) bad += wrong(bucket_start(g, b & ~7), b & 7, b);
+  for (int b = 1; b < kBuckets - 1; b += 13) {
+    const BucketStart s = bucket_start(g, b);
+    for (int x : {0, 8, 1024, 2040}) {
+      const BucketStart in = {s.t + ((uint32_t)x << (s.shift - 11)), s.shift - 11, false};
+      for (int k = 0; k < 8; ++k) bad += wrong(in, k, x + k);
+    }
   }
   return bad;
 }
@@ -44,7 +87,7 @@ def shim(tmp_path_factory):
     lib = ctypes.CDLL(str(out))
     lib.t_of.restype, lib.t_of.argtypes = ctypes.c_uint32, [ctypes.c_float]
     lib.top_of.restype, lib.top_of.argtypes = ctypes.c_float, [ctypes.c_int]
-    lib.misplaced.argtypes = [ctypes.c_uint32, ctypes.c_int]
+    lib.misplaced.argtypes = lib.wrong_masses.argtypes = [ctypes.c_uint32, ctypes.c_int]
     return lib
 
 
@@ -59,3 +102,11 @@ def test_every_bucket_holds_the_keys_between_its_edges(shim, rows):
         assert shim.misplaced(t0, rows) == 0, (rows, hex(t0))
         layouts += 1
     assert layouts > 80
+
+
+@pytest.mark.parametrize("rows", [8, 127, 128, 4096])
+def test_masses_of_buckets_are_exact(shim, rows):
+    """The mass of a bucket follows exactly from the sum of its keys' words, for one key of any score below the last 512 and for as many
+    equal or spread ones as the layout says it does."""
+    for t0 in range(shim.t_of(rows * 3.0) & ~((1 << 21) - 1), shim.t_of(rows * 0.5 / (1 << 20)) + (1 << 21), 1 << 21):
+        assert shim.wrong_masses(t0, rows) == 0, (rows, hex(t0))
