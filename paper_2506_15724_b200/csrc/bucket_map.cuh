@@ -24,6 +24,10 @@ constexpr uint32_t kTopKey = 0x7fffffffu;  // t = kTopKey - key: ascending t is 
 // throughout: 1000 candidates for 32768 keys of 224 rows and a sweep more for 131072 keys of 256 rows, 3400 in one
 // bucket; and atomics on few addresses. One octave: 64 units of 3688 keys, 256 rows, whose keys lie half an octave below
 // the mean, 60 us for the three steps after scoring instead of 50.)
+// The last bucket has to begin so low that the mass of a unit's keys is known if all of them lie there (mass_known), as nearly all
+// do in a unit whose mass one token holds: n keys below 1 / n. 832 buckets above leave seven octaves below the fine ones,
+// enough for 256 rows, 576 leave eleven, enough for the most rows there can be (4096). (With 832 for any number, 4 units of
+// 8192 keys, 448 rows, all but a two-thousandth of the mass in one key: allocation 23.8 us, with 576 15.5.)
 constexpr int kBuckets = 2048, kDig = 11, kMidBuckets = 768;
 constexpr int kMidRows = 128;              // from this many window rows on: 1.5 octaves
 constexpr uint32_t kMapTop = 0x3c000000u;  // t of the largest score below 512.0
@@ -40,7 +44,7 @@ MADAKV_HD BucketMap bucket_map_from(uint32_t t0, int rows) {
   // (aligned so that eight buckets from a multiple of eight on are equally wide)
   const uint32_t first = kMapTop + (8u << 18), mid = t0 & ~((8u << 18) - 1u);
   g.mid = mid > first ? mid : first;
-  g.high_shift = (g.mid - kMapTop) >> 17 <= 832u ? 17 : 18;
+  g.high_shift = (g.mid - kMapTop) >> 17 <= (rows <= 256 ? 832u : 576u) ? 17 : 18;
   g.c1 = (int)(kMapTop >> g.high_shift);
   g.b0 = (int)(g.mid >> g.high_shift) - g.c1;
   g.c3 = g.b0 + kMidBuckets - (int)((g.mid + ((uint32_t)kMidBuckets << g.mid_shift)) >> kLowShift);

@@ -69,6 +69,18 @@ extern "C" int wrong_masses(uint32_t t0, int rows) {
   }
   return bad;
 }
+// Is the mass of n keys known if all of them lie in the last bucket?
+extern "C" int known_at_the_end(int rows, int n) {
+  const float top = (float)rows / (float)n * fine_top(rows);
+  uint32_t key;
+  memcpy(&key, &top, 4);
+  for (int x = -1; x <= 1; ++x) {  // (the quotient may be off by two places)
+    const BucketMap g = bucket_map_from(kTopKey - key + 2 * x, rows);
+    const BucketStart last = bucket_start(g, kBuckets - 1);
+    if (!mass_known(mass_rule(last.t), n, last.t, kTopKey)) return 0;
+  }
+  return 1;
+}
 extern "C" uint32_t t_of(float score) {
   union { float f; uint32_t u; } x = {score};
   return kTopKey - x.u;
@@ -110,3 +122,14 @@ def test_masses_of_buckets_are_exact(shim, rows):
     equal or spread ones as the layout says it does."""
     for t0 in range(shim.t_of(rows * 3.0) & ~((1 << 21) - 1), shim.t_of(rows * 0.5 / (1 << 20)) + (1 << 21), 1 << 21):
         assert shim.wrong_masses(t0, rows) == 0, (rows, hex(t0))
+
+
+def test_keys_that_all_lie_in_the_last_bucket(shim):
+    """However many window rows and tokens there are, the mass of keys that all lie below the layout is known without exact
+    sweeps (which 290 rows and more needed at four to sixteen tokens per row)."""
+    rows = sorted({int(1.17 ** x) for x in range(53)} | {127, 128, 255, 256, 257, 288, 289, 448, 2048, 4095, 4096})
+    lengths = sorted({int(1.07 ** x) for x in range(205)} | {(1 << x) + y for x in range(21) for y in (-1, 0, 1)} - {0, (1 << 20) + 1})
+    assert max(lengths) == 1 << 20
+    for r in rows:
+        for n in lengths:
+            assert shim.known_at_the_end(r, n), (r, n)
