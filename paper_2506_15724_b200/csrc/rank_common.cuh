@@ -10,7 +10,7 @@
 //   buckets  a count (and for Eq. 9 a mass, see allocate.cu) per key into 2048 buckets by shared atomics without a result
 //            (bucket_map); a walk of the buckets narrows the range that the threshold can lie in to one bucket, usually
 //            some tens of keys
-//   list     the keys of the narrowed range are collected in shared memory and compared with one another (more than 256
+//   list     the keys of the narrowed range are collected in shared memory and compared with one another (more than 64
 //            of them: after half of a block's threads per modality have laid buckets over them once more)
 // A team's blocks meet twice. Every block sums its buckets up to 32 coarse ones and pushes those to all; behind the first
 // barrier a warp per modality of every block finds the coarse bucket, reads its 64 buckets from all blocks and finds the
@@ -37,7 +37,11 @@ constexpr int kRankThreads = 512;
 constexpr int kRankWarps = kRankThreads / 32;
 constexpr int kHalf = kRankThreads / 2;        // threads per modality in the walks
 constexpr int kListCap = 1024;                 // candidates per modality at most
-constexpr int kFewCap = kHalf;                 // candidates compared with one another
+// Candidates that are compared with one another, which takes instructions in proportion to their square; more are sorted into
+// buckets once more before, some 1500 clocks. (With up to 256 compared, 8 x 4 units of 8192 keys, 224 rows, one key with nine
+// tenths of the mass or two heaps of scores, 110-280 candidates: allocation 20.4 and 22.5 us, selection 13.2 and 16.2; with 64,
+// 10.8, 11.3, 9.9, 10.0. With 96 and 128 the same within 3 %.)
+constexpr uint32_t kFewCap = 64;
 constexpr int kMaxTeam = 8;
 constexpr uint32_t kNoKey = 0xffffffffu;       // t of a slot without a key
 constexpr uint32_t kNowhere = 0xfffffffeu;     // start of a range that holds no t at all (t < 2^31)
@@ -271,7 +275,7 @@ struct RankShared {
   // modality) and the keys that are compared with one another, with their masses, take their place
   alignas(16) uint32_t cnt[2 * WORDS * kStride];
   uint4 coarse[2][TEAM][TEAM > 1 ? kCoarse : 1];  // every block's sums of 64 buckets: count, mass (low, high), inexact
-  uint32_t list[2][kCap];                       // candidates of the team (allocation: in block 0)
+  alignas(16) uint32_t list[2][kCap];           // candidates of the team (allocation: in block 0)
   Found found[2];
   u64 wsum[2][kRankWarps];                      // per warp: masses (allocation)
   u64 slice_q[2][kMaxTeam];
@@ -676,28 +680,33 @@ __device__ __forceinline__ void finish_lists(RankShared<TEAM, WORDS>& sh, const 
     __syncthreads();
     list = sh.few(m);
   }
-  // The keys left, compared with one another, 2^log threads per key. The threshold's keys are those that what is needed is
+  // The keys left, compared with one another, four threads per key. The threshold's keys are those that what is needed is
   // reached with, but not before. (Keys that crowd are all alike: one of them is enough.)
+  constexpr uint32_t kPer = kHalf / kFewCap;
   const uint32_t k = !on ? 0u : in > kFewCap ? 1u : in;
   if (kMass) {
     if ((uint32_t)i < k) sh.few_mass(m)[i] = mass(list[i]);
     __syncthreads();
   }
-  const int log = min(__clz((int)k - 1) - 24, 2);  // kHalf >> log >= k
-  if (((uint32_t)i & ~31u) >> log < k) {  // (the other warps have no key)
-    const uint32_t x = (uint32_t)i >> log, part = (uint32_t)i & ((1u << log) - 1u), v = list[min(x, k - 1u)];
+  if (((uint32_t)i & ~31u) / kPer < k) {  // (the other warps have no key)
+    const uint32_t x = (uint32_t)i / kPer, part = (uint32_t)i % kPer, v = list[min(x, k - 1u)];
     uint32_t lt_c = 0, eq_c = 0;
     u64 lt = 0;
-#pragma unroll 4
-    for (uint32_t j = part; j < k; j += 1u << log) {
-      const uint32_t o = list[j];
-      if (o < v) {
-        ++lt_c;
-        if (kMass) lt += sh.few_mass(m)[j];
+#pragma unroll 1
+    for (uint32_t j = 4 * part; j < k; j += 4 * kPer) {  // (four at a time; behind the last one none counts)
+      const uint4 o4 = *reinterpret_cast<const uint4*>(list + j);
+      const uint32_t o[4] = {o4.x, j + 1 < k ? o4.y : kNoKey, j + 2 < k ? o4.z : kNoKey, j + 3 < k ? o4.w : kNoKey};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (o[e] < v) {
+          ++lt_c;
+          if (kMass) lt += sh.few_mass(m)[j + e];
+        }
+        if (o[e] == v) ++eq_c;
       }
-      if (o == v) ++eq_c;
     }
-    for (int off = 1; off < 1 << log; off <<= 1) {
+#pragma unroll
+    for (int off = 1; off < (int)kPer; off <<= 1) {
       lt_c += __shfl_xor_sync(kFull, lt_c, off);
       eq_c += __shfl_xor_sync(kFull, eq_c, off);
       if (kMass) lt += __shfl_xor_sync(kFull, lt, off);

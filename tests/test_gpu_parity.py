@@ -598,6 +598,38 @@ def test_allocate_and_select_over_blocks_and_lengths(kind, units, n):
     assert_segments_equal(kept_len, seg_off, buf.kept_idx.cpu().numpy(), kept_idx, "kept_idx")
 
 
+@pytest.mark.parametrize("units,n", [(1, 2048), (2, 16384), (150, 8200)])
+@pytest.mark.parametrize("close", [1, 2, 3, 4, 5, 31, 33, 63, 64, 65, 67, 96, 130, 256, 257])
+def test_allocate_and_select_with_so_many_candidates(units, n, close):
+    """`close` scores of each modality in one bucket with the thresholds among them, on both sides of the number up to which candidates
+    are compared with one another at once, half of them in pairs of equal ones; all others far below. Bit-exact against
+    the oracle."""
+    rng = np.random.RandomState(close + n)
+    rows = 64
+    psi = np.exp(rng.uniform(-14.0, -12.0, (1, units, 1, n))).astype(np.float32)
+    mask = (np.arange(n) % 2).astype(np.uint8)[None]
+    for u in range(units):
+        for m in (0, 1):
+            few = np.float32(0.3) + rng.permutation(close)[: close - close // 4].astype(np.float32) * np.float32(2.0 ** -24)
+            psi[0, u, 0, rng.choice(n // 2, close, replace=False) * 2 + 1 - m] = np.concatenate([few, few[: close // 4]])
+    sl = np.array([n], np.int32)
+    d_psi, d_mask, d_sl = (torch.from_numpy(x).cuda() for x in (psi, mask, sl))
+    for theta in (0.02, 0.5, 0.9):
+        cfg = mk.make_config(torch.float32, 1, units, 1, 1, 64, n, rows, max_new_tokens=0, theta=theta)
+        buf = mk.EvictionBuffers(cfg, units * n)
+        bud = np.array([close], np.int32)
+        mk.madakv_allocate(cfg, d_psi, d_mask, d_sl, torch.from_numpy(bud).cuda(), buf.mass, buf.pref, buf.demand, buf.phi, buf.budgets, buf.ws)
+        want = oracle.allocate(psi, mask, sl, bud, float(np.float32(theta)))
+        for key in ("mass", "pref", "demand", "phi", "budgets"):
+            assert np.array_equal(getattr(buf, key).cpu().numpy(), want[key]), (key, theta)
+        budgets = np.maximum(want["demand"], 1).astype(np.int32)
+        rc, kept_len, seg_off, kept_idx = oracle.select(psi, mask, sl, budgets, capacity=units * n)
+        mk.madakv_select(cfg, d_psi, d_mask, d_sl, torch.from_numpy(budgets).cuda(), buf.kept_len, buf.seg_off, buf.kept_idx, buf.ws)
+        assert rc == 0 and mk.madakv_poll_status(buf.ws) == 0
+        assert np.array_equal(buf.kept_len.cpu().numpy(), kept_len)
+        assert_segments_equal(kept_len, seg_off, buf.kept_idx.cpu().numpy(), kept_idx, "kept_idx")
+
+
 @pytest.mark.parametrize("B,Hkv,n", [(2, 2, 32768), (2, 2, 32769), (64, 1, 131), (65, 1, 131), (7, 3, 4097), (16, 2, 4096), (36, 4, 33)])
 @pytest.mark.parametrize("kind", ["scale", "one_bucket", "octaves"])
 @pytest.mark.parametrize("w,g", [(8, 1), (64, 2), (64, 64)])
