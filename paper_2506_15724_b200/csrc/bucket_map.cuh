@@ -78,6 +78,14 @@ MADAKV_HD uint32_t bucket_last(const BucketStart& b, int x, int at) {
   return (b.ends && at == kBuckets - 1) || last > kTopKey ? kTopKey : last;
 }
 
+// The plain layout, the same for all sequences: 64 buckets per octave from 512 down to 2^-23, for half the instructions per key.
+struct PlainMap {};
+MADAKV_HD uint32_t map_bucket(const PlainMap&, uint32_t t) {
+  const int b = (int)(t >> 17) - (int)(kMapTop >> 17), last = b < kBuckets - 1 ? b : kBuckets - 1;
+  return (uint32_t)(last > 0 ? last : 0);
+}
+MADAKV_HD BucketStart bucket_start(const PlainMap&, int b) { return {kMapTop + ((uint32_t)b << 17), 17, true}; }
+
 // The mass of a bucket, exactly, from its keys' count and the sum modulo 2^32 of a word per key. Scores from 2^-9 on are multiples
 // of 2^-32 and those of a bucket lie in one octave, so that q = floor(x * 2^32) is linear in the key: their word is the key itself,
 // and what it tells is exact however large the scores are (as long as they are fewer than 2^32 / width: 16384 for the widest buckets).

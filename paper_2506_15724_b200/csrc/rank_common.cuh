@@ -270,7 +270,7 @@ constexpr int kCoarse = kBuckets / 64;
 template <int TEAM, int WORDS>  // WORDS: count, or count and mass, per bucket
 struct RankShared {
   static constexpr int kStride = kBuckets;
-  static constexpr int kCap = TEAM > 1 ? kListCap / 2 : kListCap;
+  static constexpr int kCap = TEAM > 1 && WORDS == 2 ? kListCap / 2 : kListCap;  // (allocation's teams have no room for more)
   // the buckets' counts; once they are walked, the buckets of the finish (count, mass low, mass high; one per thread and
   // modality) and the keys that are compared with one another, with their masses, take their place
   alignas(16) uint32_t cnt[2 * WORDS * kStride];
@@ -301,7 +301,8 @@ struct RankRange {
 __device__ __forceinline__ int range_shift(uint32_t span, int dig) { return max(32 - __clz((int)span) - dig, 0); }
 
 // The range of t of bucket `at`, of the first layout or of one over g with 2^shift values of t per bucket.
-__device__ __forceinline__ void bucket_range(RankRange& g, const BucketMap* map, uint32_t at, int shift) {
+template <typename Map>
+__device__ __forceinline__ void bucket_range(RankRange& g, const Map* map, uint32_t at, int shift) {
   if (map) {
     const BucketStart s = bucket_start(*map, (int)at);
     g.lo = at ? s.t : 0u;

@@ -261,8 +261,22 @@ struct SelRanges {
   __device__ __forceinline__ bool crowded1() const { return r1.in > CAP && r1.span > 0; }
 };
 
-template <int KPT, int TEAM>
-__device__ __forceinline__ void count_first(RankShared<TEAM, 1>& sh, const BucketMap& map, const uint32_t (&t)[KPT], uint32_t vis, uint32_t valid) {
+// Blocks on their own, whose calls are bound by instructions per key, take the plain layout of the buckets: of the finer one they
+// have fewer candidates but no shorter steps (1024 units of 8192 keys 33.0 us with it, 31.4 without; 896 of 16384, 224
+// rows, 47.1 and 44.9, and 50.4 and 47.5 with nine tenths of the mass in one key; 256 of 131072, 256 rows, 82.3 and 84.7,
+// 88.2 and 83.5). Teams, whose steps grow with the candidates, take the finer one.
+template <int TEAM>
+struct SelectMap {
+  using Map = BucketMap;
+  static __device__ __forceinline__ Map of(int rows, int n) { return bucket_map(rows, n); }
+};
+template <>
+struct SelectMap<1> {
+  using Map = PlainMap;
+  static __device__ __forceinline__ Map of(int, int) { return {}; }
+};
+template <int KPT, int TEAM, typename Map>
+__device__ __forceinline__ void count_first(RankShared<TEAM, 1>& sh, const Map& map, const uint32_t (&t)[KPT], uint32_t vis, uint32_t valid) {
   constexpr int kStride = RankShared<TEAM, 1>::kStride;
   if (valid == valid_bits<KPT>(KPT, 0)) {
 #pragma unroll
@@ -285,8 +299,8 @@ __device__ __forceinline__ void count_again(RankShared<TEAM, 1>& sh, const SelRa
 
 // Walk of the buckets (of the first layout, `map`, or of one over the ranges): the ranges shrink to the buckets with the wanted
 // keys.
-template <int TEAM>
-__device__ __forceinline__ void select_walk(RankShared<TEAM, 1>& sh, uint32_t rank, const BucketMap* map, uint32_t want0, uint32_t want1,
+template <int TEAM, typename Map>
+__device__ __forceinline__ void select_walk(RankShared<TEAM, 1>& sh, uint32_t rank, const Map* map, uint32_t want0, uint32_t want1,
                                             SelRanges<RankShared<TEAM, 1>::kCap>& g, int shift0, int shift1) {
   walk<TEAM, 1>(
       sh, rank, [](int, int) { return BucketStart{0u, 0, false}; },
@@ -486,6 +500,7 @@ __device__ __forceinline__ void emit(int32_t* seg, const Thresholds& h, int pos0
 // A unit whose keys fit the registers of its team.
 template <int KPT, int TEAM, bool kPool>
 __global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(const __grid_constant__ SelParams p) {
+  using Map = typename SelectMap<TEAM>::Map;
   constexpr uint32_t kCap = RankShared<TEAM, 1>::kCap;
   __shared__ RankShared<TEAM, 1> sh;
   __shared__ SeqCounts s;
@@ -509,13 +524,13 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(const __gr
   x.set_up(p);
   uint32_t t[KPT], forced;
   const uint32_t valid = x.template take<KPT>(p, raw, pos0, t, forced), vis = p.mpa ? take_mask<KPT>(raw_mask) : 0u;
-  const BucketMap map = bucket_map(p.rows, x.n);
+  const Map map = SelectMap<TEAM>::of(p.rows, x.n);
   __syncthreads();
   if (p.alone && x.b > 0) x.count_before(p, s);
   count_first<KPT, TEAM>(sh, map, t, vis, valid);
   SelRanges<kCap> g{{kNowhere, 0u, 0u, 0u}, {kNowhere, 0u, 0u, 0u}, false, false, 0u, 0u};
   team_wait_started<TEAM>();
-  select_walk<TEAM>(sh, rank, &map, x.want0, x.want1, g, 0, 0);
+  select_walk<TEAM, Map>(sh, rank, &map, x.want0, x.want1, g, 0, 0);
   bool swept = false;
   if (g.crowded0() || g.crowded1()) {
     const int shift0 = range_shift(g.r0.span, kDig), shift1 = range_shift(g.r1.span, kDig);
@@ -523,7 +538,7 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(const __gr
     zero_buckets<TEAM, 1>(sh);
     __syncthreads();
     count_again<KPT, TEAM>(sh, g, t, vis, shift0, shift1);
-    select_walk<TEAM>(sh, rank, nullptr, x.want0, x.want1, g, shift0, shift1);
+    select_walk<TEAM, Map>(sh, rank, nullptr, x.want0, x.want1, g, shift0, shift1);
     if (g.crowded0() || g.crowded1()) {
       select_bisect<TEAM>(sh, x.want0, x.want1, g, [&](auto each) {
 #pragma unroll
@@ -563,6 +578,7 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_unit_kernel(const __gr
 template <int TEAM, bool kPool>
 __global__ void __launch_bounds__(kRankThreads, 2) select_long_kernel(const __grid_constant__ SelParams p) {
   constexpr int KPT = 16, kRound = kRankThreads * KPT;
+  using Map = typename SelectMap<TEAM>::Map;
   constexpr uint32_t kCap = RankShared<TEAM, 1>::kCap;
   __shared__ RankShared<TEAM, 1> sh;
   __shared__ SeqCounts s;
@@ -585,7 +601,7 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_long_kernel(const __gr
   const int rounds = (x.n + kRound * TEAM - 1) / (kRound * TEAM);
   const int start = (int)rank * rounds * kRound;  // a block owns consecutive positions
 
-  const BucketMap map = bucket_map(p.rows, x.n);
+  const Map map = SelectMap<TEAM>::of(p.rows, x.n);
   __syncthreads();
   if (p.alone && x.b > 0) x.count_before(p, s);
 #pragma unroll 1
@@ -599,7 +615,7 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_long_kernel(const __gr
   }
   SelRanges<kCap> g{{kNowhere, 0u, 0u, 0u}, {kNowhere, 0u, 0u, 0u}, false, false, 0u, 0u};
   team_wait_started<TEAM>();
-  select_walk<TEAM>(sh, rank, &map, x.want0, x.want1, g, 0, 0);
+  select_walk<TEAM, Map>(sh, rank, &map, x.want0, x.want1, g, 0, 0);
   bool swept = false;
   if (g.crowded0() || g.crowded1()) {
     const int shift0 = range_shift(g.r0.span, kDig), shift1 = range_shift(g.r1.span, kDig);
@@ -612,7 +628,7 @@ __global__ void __launch_bounds__(kRankThreads, 2) select_long_kernel(const __gr
       x.template load<KPT>(p, start + r * kRound + tid * KPT, t, forced);
       count_again<KPT, TEAM>(sh, g, t, bits_of_thread(vis_w, r), shift0, shift1);
     }
-    select_walk<TEAM>(sh, rank, nullptr, x.want0, x.want1, g, shift0, shift1);
+    select_walk<TEAM, Map>(sh, rank, nullptr, x.want0, x.want1, g, shift0, shift1);
     if (g.crowded0() || g.crowded1()) {
       select_bisect<TEAM>(sh, x.want0, x.want1, g, [&](auto each) {
 #pragma unroll 1

@@ -11,9 +11,9 @@ SHIM = r"""
 #include "bucket_map.cuh"
 using namespace madakv;
 // Buckets of the layout of `rows` window rows whose fine part begins at t0 that do not hold exactly the keys between their start
-// and the next one's, or whose start does not follow from that of their group of eight.
-extern "C" int misplaced(uint32_t t0, int rows) {
-  const BucketMap g = bucket_map_from(t0, rows);
+// and the next one's, or whose start does not follow from that of their group of eight. (0 rows: of the plain layout.)
+template <typename Map>
+static int misplaced_in(const Map& g) {
   int bad = map_bucket(g, 0u) != 0u || map_bucket(g, kTopKey) != (uint32_t)kBuckets - 1u;
   for (int b = 0; b < kBuckets; ++b) {
     const BucketStart s = bucket_start(g, b), first = bucket_start(g, b & ~7);
@@ -27,6 +27,7 @@ extern "C" int misplaced(uint32_t t0, int rows) {
   }
   return bad;
 }
+extern "C" int misplaced(uint32_t t0, int rows) { return rows ? misplaced_in(bucket_map_from(t0, rows)) : misplaced_in(PlainMap()); }
 // Buckets whose mass does not come out right from the words of its keys, for as many keys as mass_known() takes, or that take
 // fewer than they have to: one key of any score, and of scores from 2^-9 on as many as 2^32 over the bucket's width. Of a
 // layout over [t, t + 2^(11 + shift)) too.
@@ -114,6 +115,10 @@ def test_every_bucket_holds_the_keys_between_its_edges(shim, rows):
         assert shim.misplaced(t0, rows) == 0, (rows, hex(t0))
         layouts += 1
     assert layouts > 80
+
+
+def test_every_bucket_of_the_plain_layout_holds_the_keys_between_its_edges(shim):
+    assert shim.misplaced(0, 0) == 0
 
 
 @pytest.mark.parametrize("rows", [8, 127, 128, 4096])
