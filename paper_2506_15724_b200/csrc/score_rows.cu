@@ -1358,7 +1358,10 @@ int score_rows(const madakv_config& c, const void* q, madakv_strides sq, const v
       p.mblocks = p.R <= 128 ? 1 : 2;
       p.cparts = convert ? 1 : (p.R <= 128 ? 4 : 2);
       p.n16 = (p.R + 15) / 16 * 16;
-      p.slack = !f32 && p.R <= 128 ? 0 : 2;  // (two buffers for the row operands, or one)
+      // (bf16 rows beyond 128 have one buffer, and a change of units costs two or three tiles' time; fp32 has one, too, but its tiles
+      // take several times as long: 60 units of 24 tiles, 32 rows, 84.0 us with CTAs of two tiles more, 77.1 without; 40 of
+      // 16 51.3 and 49.4; 20 of 71 78.9 and 77.1)
+      p.slack = !f32 && p.R > 128 ? 2 : 0;
       if (!convert && !(f32 ? make_map(&mq, q, 3 * d, c.window, p.units * g, 1, 1, split_q, p.wc, heads)
                             : make_map(&mq, q, d, c.window, c.n_q_heads, c.n_layers, c.batch, sq, p.wc, heads)))
         return MADAKV_EUNSUPPORTED;
