@@ -157,18 +157,14 @@ def test_score_in_chunks(dtype, B, L, Hq, Hkv, d, n, w, causal):
     assert psi_close(psi.cpu().numpy(), want, PSI_RTOL) < PSI_RTOL_SEEN
 
 
-# sequences longer than a cluster's TMEM holds: a whole round of clusters, tiles that pass twice in one sequence of the batch
-# and not in the other, lengths that end inside a tile; with logits so far apart that references are raised; and the calls
-# next to the rule (too few units, too many rows), which take two passes
 @pytest.mark.parametrize("dtype,B,Hq,Hkv,w,n", [
     ("bf16", 1, 28, 4, 32, 37 * 128 + 5), ("bf16", 1, 28, 4, 32, 36 * 128), ("bf16", 1, 28, 4, 32, 75 * 128), ("bf16", 2, 16, 4, 64, 2500),
     ("bf16", 1, 32, 8, 20, 600), ("bf16", 3, 147, 49, 30, 400), ("f32", 1, 8, 4, 32, 36 * 128 + 1)])
 @pytest.mark.parametrize("given", [False, True])
-def test_score_partition_and_lengths_written_just_before(dtype, B, Hq, Hkv, w, n, given):
+def test_score_partition_and_changing_lengths(dtype, B, Hq, Hkv, w, n, given):
     """Wide-window scoring where every unit gets thread blocks of its own (about as many tiles as blocks, one more or fewer, far
-    fewer; as many units as blocks), where it does not because the lengths differ, and with lengths that the kernel before
-    in the stream has just changed, since the range of a block is found before that kernel has ended. Against the oracle,
-    with the tolerance of the other score tests (1e-4 relative: fp32 sums of up to 10^4 terms)."""
+    fewer; as many units as blocks), where it does not because the lengths differ, and one call after the other on lengths
+    that a copy in between has changed. Against the oracle, with the tolerance of the other score tests (1e-4 relative: fp32 sums of up to 10^4 terms)."""
     wl = synth.scaled(TINY, B=B, L=1, Hq=Hq, Hkv=Hkv, n=n, w=w, d=64, dtype=dtype)
     inp = synth.make_inputs(wl, device="cpu", want_v=False)
     g = dev(inp)
@@ -193,6 +189,49 @@ def test_score_partition_and_lengths_written_just_before(dtype, B, Hq, Hkv, w, n
         psi_close(psi.cpu().numpy(), want, rtol=1e-4)
 
 
+@pytest.mark.parametrize("dtype,Hq,Hkv,d", [("bf16", 28, 4, 128), ("bf16", 8, 2, 64), ("f32", 4, 4, 64)])
+@pytest.mark.parametrize("stale,n", [(4700, 1203), (600, 4699), (0, 3000), (3000, 0)])
+@pytest.mark.parametrize("given", [False, True])
+def test_score_of_a_length_that_the_kernel_before_is_still_writing(dtype, Hq, Hkv, d, stale, n, given):
+    """Wide-window scoring finds a block's range of tiles under the kernel before it, from lengths that this one may not have written
+    yet. Selection of few units lets the next kernel begin first and writes its segment's length last: with that as the
+    sequence length, and another one in its place before, the range has to be found anew. Against the oracle, with the
+    tolerance of the other score tests (1e-4 relative)."""
+    n_max, w = 4800, 32
+    wl = synth.scaled(TINY, B=1, L=1, Hq=Hq, Hkv=Hkv, n=n_max, w=w, d=d, dtype=dtype)
+    inp = synth.make_inputs(wl, device="cpu", want_v=False)
+    g, cfg = dev(inp), config_of(wl)
+    sl = np.array([n], np.int32)
+    want = oracle.score(dcode(wl), to_np(inp["q_win"]), to_np(inp["k"]), sl)
+    psi, lse = torch.zeros((1, 1, Hkv, n_max), device="cuda"), torch.zeros((1, 1, Hq, w), device="cuda")
+    ws = mk.new_workspace(cfg)
+    if given:
+        mk.madakv_score(cfg, g["q_win"], g["k"], torch.from_numpy(sl).cuda(), lse, psi, ws)
+    # a unit of 2^20 keys (some 60 us), of which n are kept: a text budget of n tokens
+    keys = 1 << 20
+    one = mk.make_config(torch.float32, 1, 1, 1, 1, 64, keys, 8, max_new_tokens=0)
+    scores = torch.rand((1, 1, 1, keys), generator=torch.Generator().manual_seed(n)).cuda()
+    mask, all_keys = torch.zeros((1, keys), dtype=torch.uint8, device="cuda"), torch.full((1,), keys, dtype=torch.int32, device="cuda")
+    budgets = torch.tensor([[[[0, n]]]], dtype=torch.int32, device="cuda")
+    length, off = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.zeros(2, dtype=torch.int64, device="cuda")
+    idx, ws1 = torch.zeros(keys, dtype=torch.int32, device="cuda"), mk.new_workspace(one)
+    for _ in range(3):
+        length.fill_(stale)
+        psi.fill_(7.0)
+        torch.cuda.synchronize()
+        mk.madakv_select(one, scores, mask, all_keys, budgets, length, off, idx, ws1)
+        if given:
+            mk.madakv_score_lse(cfg, g["q_win"], g["k"], length, lse, psi, ws)
+        else:
+            mk.madakv_score(cfg, g["q_win"], g["k"], length, lse, psi, ws)
+        assert mk.madakv_poll_status(ws) == 0 and mk.madakv_poll_status(ws1) == 0
+        assert int(length.item()) == n
+        psi_close(psi.cpu().numpy(), want, rtol=1e-4)
+
+
+# sequences longer than a cluster's TMEM holds: a whole round of clusters, tiles that pass twice in one sequence of the batch
+# and not in the other, lengths that end inside a tile; with logits so far apart that references are raised; and the calls
+# next to the rule (too few units, too many rows), which take two passes
 @pytest.mark.parametrize("B,H,d,n,w", [(1, 22, 64, 16500, 32), (2, 11, 128, 17003, 20), (1, 2, 64, 17000, 32), (1, 24, 64, 5200, 64)])
 @pytest.mark.parametrize("spread", [False, True])
 def test_score_longer_than_tensor_memory(B, H, d, n, w, spread):
