@@ -173,8 +173,9 @@ inline int launch_status() {
 }
 
 // Launch with programmatic stream serialisation: the grid may be scheduled while the kernel before it in the stream is
-// still running, which hides its launch latency. A kernel launched this way calls pdl_wait() before it touches global
-// memory (the call returns once the kernels before it have completed and their writes are visible; it is a no-op in a
+// still running, which hides its launch latency. A kernel launched this way calls pdl_wait() before it uses what earlier
+// kernels write (score_rows_kernel reads the lengths and prefetches operands into the L2 before it, and reads the lengths again
+// behind it), and before it writes to global memory (the call returns once the kernels before it have completed and their writes are visible; it is a no-op in a
 // kernel launched the ordinary way) and pdl_go() to let the kernel after it be scheduled.
 // `team` > 1 launches thread-block clusters of that many blocks.
 template <typename... KArgs, typename... Args>

@@ -16,7 +16,8 @@
 // barrier a warp per modality of every block finds the coarse bucket, reads its 64 buckets from all blocks and finds the
 // bucket, the same in every block, with the places of all blocks' keys in the list; the keys are pushed there before the
 // second barrier. (With a share of all buckets per block, read from all others, their totals and the bucket announced and
-// the lists gathered, five barriers in all, allocation and selection of 4 units of 32768 keys took 17 and 13 us; now 13 and 9.)
+// the lists gathered, five barriers in all, allocation and selection of 4 units of 32768 keys, 224 rows, took 17.1 and 10.2 us;
+// now 11.9 and 7.6, one call after the other.)
 // Buckets over the range of each unit's keys needed a sweep for that range before; without it, and with long units read
 // twice instead of three (allocation) or four times (selection), allocation + selection + compaction went from 602 to 483 us
 // on 256 units of 131072 keys, from 618 to 523 on 1600 of 13411, from 213 to 161 on 3360 of 471, from 31 to 26 on 200 of 772.
@@ -732,9 +733,13 @@ struct RankShape {
 // "long" kernels): spread over 2, 4 and 8 blocks such a call was slower the more blocks there were (256 units of 131072 keys:
 // allocation 156, 167, 174, 228 us, selection 219, 223, 240, 297 us), because every block pays for the fixed steps. With
 // fewer units a team of up to 8 blocks per unit brings the call to about a block per SM, and a call with a few units (one
-// layer), which is bound by the latency of its blocks, takes 8 keys per thread instead of 16 (4 units of 32768 keys: 12.8 +
-// 10.9 us with 8 blocks of 8 keys, 15.5 + 13.7 with 4 blocks of 16, 30 + 54 with one block per unit, when a team met five
-// times).
+// layer), which is bound by the latency of its blocks, takes 8 keys per thread instead of 16. Measured, allocation + selection
+// in us: 4 units of 32768 keys 11.9 + 7.6 with 8 blocks of 8 keys, 12.8 + 8.2 with 4 of 16; 32 of 8192, batch of 8, 9.7 + 8.8 with
+// 2 of 8, 10.7 + 9.6 with one of 16; 4 of 8192, 448 rows, 9.7 + 6.6 and 10.8 + 7.6. Where 8 keys per thread make more than
+// two blocks per SM, 16 would be as good or better: 40 units of 16384 13.9 + 9.7 with 4 of 8, 13.0 + 8.5 with 2 of 16; 80 of
+// 5000 11.6 + 9.9 and 11.1 + 8.8; 16 of 20000 12.8 + 10.7 and 12.2 + 9.2. Teams that bring a call to half a block per SM instead
+// of one: 32 of 65536 19.5 + 15.4 instead of 21.7 + 13.9, 112 of 12000 17.8 + 11.2 and 19.2 + 10.8; to two: 112 of 12000 24.2 + 16.2,
+// 256 of 32768 42.8 + 33.3 instead of 35.0 + 24.5, 256 of 131072 122 + 85 instead of 101 + 85.
 constexpr int kLongKeys = 262144;  // keys per block that a long kernel has bits for in shared memory
 inline RankShape rank_shape(long long units, int n_max) {
   const int cap16 = kRankThreads * 16, cap8 = kRankThreads * 8;

@@ -379,7 +379,7 @@ template <int TEAM>
 __device__ __forceinline__ Thresholds select_thresholds(RankShared<TEAM, 1>& sh, uint32_t want0, uint32_t want1,
                                                         const SelRanges<RankShared<TEAM, 1>::kCap>& g) {
   constexpr uint32_t kCap = RankShared<TEAM, 1>::kCap;
-  team_sync<TEAM>();  // (the last access to another block's shared memory)
+  team_sync<TEAM>();  // (the last access to another block's shared memory, but for counts_before() after exact sweeps)
   const bool on0 = want0 && !g.short0 && g.r0.in <= kCap, on1 = want1 && !g.short1 && g.r1.in <= kCap;
   finish_lists<TEAM, 1, false>(sh, g.r0, g.r1, on0, on1, want0, want1, 0ull, 0ull);
   Thresholds h;
@@ -753,7 +753,11 @@ int launch_select(const madakv_config& c, const float* psi, const uint8_t* mask,
   p.rows = c.n_q_heads / c.n_kv_heads * c.window;
   // Few units: no kernel of its own for the scan of the segments (2 us on the host, 3-5 on the GPU). A unit needs the visual-token
   // counts of the sequences before its own, which it takes itself as long as they are a few loads per thread; a larger call is
-  // better off with a scan that runs beside the ranking.
+  // better off with a scan that runs beside the ranking. Layer by layer, where the host is the bound, a step of allocation,
+  // selection and compaction takes 28.4 us without the scan and 30.4 with it (8 x 4 units of 1000 or 4000 keys, 4 x 8 of 2000,
+  // 64 x 2 of 500), about the same near the limit (8 x 4 of 8000, 36.0 and 35.7); selections one after the other, which the GPU is
+  // the bound of, take 0.3-1.4 us more without it up to the limit (36 x 4 of 1024 7.6 and 7.0, 8 x 4 of 8192 8.8 and 7.5) and 2-9
+  // beyond (8 x 4 of 16384 10.8 and 7.7, 64 x 2 of 8192 24.2 and 15.3).
   p.alone = p.units < 148 && c.batch <= kAloneSeqs && (c.batch == 1 || (int64_t)c.batch * c.max_seq_len <= kAloneTokens);
   if (!p.alone) launch_pdl(seg_scan_kernel, dim3(1), dim3(1024), 0, st, p);
   if (c.pool_kernel > 1 || c.keep_window) launch_select_unit<true>(c, p, st);
